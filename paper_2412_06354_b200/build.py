@@ -1,4 +1,4 @@
-"""Builds libgnn_b200.so (nvcc, sm_100a only) and the input-generator library, in-tree.
+"""Builds libgnn_b200.so (nvcc, sm_100a only), the Python extension in front of it and the input-generator library, in-tree.
 
     python -m paper_2412_06354_b200.build [--force]
 """
@@ -19,6 +19,9 @@ NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std=c++17",
          "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include"), "-I" + CSRC,
          *os.environ.get("GNN_NVCC_FLAGS", "").split()]
+
+
+BINDING = os.path.join(HERE, "_binding.so")
 
 
 def _newest(paths):
@@ -46,9 +49,27 @@ def build(force: bool = False, verbose: bool = False) -> str:
                     raise RuntimeError("nvcc failed: " + " ".join(r.args))
     if jobs or not os.path.exists(LIB):
         subprocess.check_call([NVCC, "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", LIB, *objs])
+    build_binding(force)
     from . import synth
     synth.build(force)
     return LIB
+
+
+def build_binding(force: bool = False) -> str:
+    """The CPython extension (host code only) that gnn.py calls; linked against libgnn_b200.so beside it and torch."""
+    src = os.path.join(CSRC, "binding.cpp")
+    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= _newest([src, os.path.join(ROOT, "include", "gnn.h")]):
+        return BINDING
+    import sysconfig
+    import torch
+    tdir = os.path.dirname(torch.__file__)
+    inc = [os.path.join(ROOT, "include"), os.path.join(tdir, "include"), os.path.join(tdir, "include", "torch", "csrc", "api", "include"),
+           sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include")]
+    subprocess.check_call(["g++", "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden", *["-I" + d for d in inc],
+                           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", src, "-o", BINDING,
+                           "-L" + HERE, "-l:libgnn_b200.so", "-Wl,-rpath,$ORIGIN", "-L" + os.path.join(tdir, "lib"),
+                           "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python"])
+    return BINDING
 
 
 if __name__ == "__main__":

@@ -1,4 +1,7 @@
-"""ctypes binding of libgnn_b200.so: argument marshalling only.
+"""Binding of libgnn_b200.so: argument marshalling only.
+
+The calls go through the compiled extension ``_binding`` (csrc/binding.cpp), which unpacks tensors and allocates
+outputs and workspaces; the ctypes prototypes of the C ABI stay available through ``load()``.
 
 Every function here has the name of the C entry point without the ``gnn_`` prefix, takes torch
 CUDA tensors (torch is used for device memory and streams, nothing else), allocates outputs and
@@ -9,12 +12,24 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+from ctypes import addressof as _addr
 
 import torch
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libgnn_b200.so")
 _lib = None
+
+
+class _Unloaded:
+    """Stands for the extension until the first call loads the library."""
+
+    def __getattr__(self, name):
+        load()
+        return getattr(_b, name)
+
+
+_b = _Unloaded()
 
 SUM, MEAN, MAX, MIN = 0, 1, 2, 3
 COPY_XJ, E_MUL_XJ, GAT_LOGIT, XI_SUB_XJ, XI_DOT_XJ = 0, 1, 2, 3, 4
@@ -121,6 +136,9 @@ def load(path: str = LIB_PATH):
             fn = getattr(lib, name)
             fn.restype = res
             fn.argtypes = args
+        from . import _binding
+        _binding.attach(globals(), torch, GnnError)
+        globals()["_b"] = _binding
         _lib = lib
     return _lib
 
@@ -181,6 +199,9 @@ class Graph:
         self.rowptrT = torch.empty(N + 1, **i64)
         n = max(self.E, 1)
         self.col, self.eid, self.colT, self.eidT, self.t2f = (torch.empty(n, **i32) for _ in range(5))
+        self._describe()
+
+    def _describe(self):
         self.c = CsrStruct(self.N, self.E, *(t.data_ptr() for t in (self.rowptr, self.col, self.eid, self.rowptrT, self.colT, self.eidT, self.t2f)))
 
     @property
@@ -193,13 +214,10 @@ class Graph:
 
 # ------------------------------------------------------------------ graph set-up
 def coo_to_csr(N, src, dst, ws=None) -> Graph:
-    src, dst = _dev(src), _dev(dst)
-    E = src.numel()
-    g = Graph(N, E, src.device)
-    need = load().gnn_coo_to_csr_workspace(N, E)
-    if ws is None:
-        ws = torch.empty(need, dtype=torch.uint8, device=src.device)
-    _check(load().gnn_coo_to_csr(N, E, _pi(src, torch.int32, "src"), _pi(dst, torch.int32, "dst"), g.ref, _p(ws), ws.numel(), _stream()))
+    g = Graph.__new__(Graph)
+    g.rowptr, g.rowptrT, g.col, g.eid, g.colT, g.eidT, g.t2f = _b.coo_to_csr(N, src, dst, ws)
+    g.N, g.E = int(N), src.numel()
+    g._describe()
     return g
 
 
@@ -220,36 +238,20 @@ def csr_validate(g: Graph, ws=None):
 
 
 def degree(g: Graph, transposed=False, w=None):
-    out = torch.empty(g.N, dtype=torch.int32 if w is None else torch.float32, device=g.rowptr.device)
-    _check(load().gnn_degree(g.ref, int(transposed), _p(w), _p(out), _stream()))
-    return out
+    return _b.degree(_addr(g.c), transposed, w, g.rowptr)
 
 
 def add_self_loops(N, src, dst):
-    E = src.numel()
-    so = torch.empty(E + N, dtype=torch.int32, device=src.device)
-    do = torch.empty(E + N, dtype=torch.int32, device=src.device)
-    _check(load().gnn_add_self_loops(N, E, _pi(src, torch.int32, "src"), _pi(dst, torch.int32, "dst"), _p(so), _p(do), _stream()))
-    return so, do
+    return _b.add_self_loops(N, src, dst)
 
 
 def gcn_norm(g: Graph, w_csr=None, want_T=True):
-    dev = g.rowptr.device
-    deg = torch.empty(g.N, dtype=torch.float32, device=dev)
-    coef = torch.empty(max(g.E, 1), dtype=torch.float32, device=dev)
-    coefT = torch.empty(max(g.E, 1), dtype=torch.float32, device=dev) if want_T else None
-    _check(load().gnn_gcn_norm(g.ref, _pf32(w_csr, "w_csr"), _p(deg), _p(coef), _p(coefT), _stream()))
-    return deg, coef[:g.E], (coefT[:g.E] if want_T else None)
+    """-> (degrees, coefficients in CSR order, coefficients in transposed-CSR order or None)"""
+    return _b.gcn_norm(_addr(g.c), w_csr, want_T, g.rowptr)
 
 
 def permute_edge_data(perm, x, out=None):
-    x = _dev(x)
-    E = perm.numel()
-    width = x.numel() // max(E, 1) if E else 1
-    if out is None:
-        out = torch.empty_like(x)
-    _check(load().gnn_permute_edge_data(_pi(perm, torch.int32, "perm"), E, max(width, 1), x.element_size(), _p(x), _p(out), _stream()))
-    return out
+    return _b.permute_edge_data(perm, x, out)
 
 
 # ------------------------------------------------------------------ fused propagate
@@ -259,36 +261,13 @@ def propagate_fused_workspace(E, F, op="sum"):
 
 def propagate_fused(g: Graph, X, w_csr=None, op="sum", out=None, argmax=None, ws=None):
     """-> out, or (out, argmax) for max/min."""
-    X = _dev(X)
-    F = X.shape[1]
-    opc = _op(op)
-    if out is None:
-        out = torch.empty((g.N, F), dtype=X.dtype, device=X.device)
-    if opc in (MAX, MIN) and argmax is None:
-        argmax = torch.empty((g.N, F), dtype=torch.int32, device=X.device)
-    if ws is None:
-        ws = torch.empty(propagate_fused_workspace(g.E, F, opc), dtype=torch.uint8, device=X.device)
-    msg = COPY_XJ if w_csr is None else E_MUL_XJ
-    _check(load().gnn_propagate_fused(g.ref, msg, opc, _p(X), _pf32(w_csr, "w_csr"), F, _dtype(X), _p(out), _pi(argmax, torch.int32, "argmax"), _p(ws), ws.numel(), _stream()))
-    return (out, argmax) if opc in (MAX, MIN) else out
+    return _b.propagate_fused(_addr(g.c), X, w_csr, op, out, argmax, ws)
 
 
 def propagate_fused_backward(g: Graph, dOut, op="sum", X=None, w_csrT=None, argmax=None, want_dX=True, want_dW=False,
                              dX=None, dW=None, ws=None):
     """-> (dX or None, dW or None)."""
-    dOut = _dev(dOut)
-    F = dOut.shape[1]
-    opc = _op(op)
-    if want_dX and dX is None:
-        dX = torch.empty((g.N, F), dtype=dOut.dtype, device=dOut.device)
-    if want_dW and dW is None:
-        dW = torch.empty(max(g.E, 1), dtype=torch.float32, device=dOut.device)
-    if ws is None:
-        ws = torch.empty(propagate_fused_workspace(g.E, F, opc), dtype=torch.uint8, device=dOut.device)
-    msg = COPY_XJ if (w_csrT is None) else E_MUL_XJ
-    _check(load().gnn_propagate_fused_backward(g.ref, msg, opc, _p(dOut), _p(X), _pf32(w_csrT, "w_csrT"), _pi(argmax, torch.int32, "argmax"), F, _dtype(dOut),
-                                               _p(dX if want_dX else None), _p(dW if want_dW else None), _p(ws), ws.numel(), _stream()))
-    return (dX if want_dX else None), (dW[:g.E] if want_dW else None)
+    return _b.propagate_fused_backward(_addr(g.c), dOut, op, X, w_csrT, argmax, want_dX, want_dW, dX, dW, ws)
 
 
 def propagate_fused_host(g: Graph, h_X, w_csr, op, h_out, d_in, d_out, ws, argmax=None):
@@ -309,289 +288,116 @@ def propagate_fused_backward_host(g: Graph, h_dOut, op, w_csrT, h_dX, d_in, d_ou
 
 
 # ------------------------------------------------------------------ more (message, op) pairs, GIN, XI_DOT_XJ
-def _epi(epi):
-    """dict(Xself=, self_coef=, self_mode=, bias=, relu=) -> (struct or None, the tensors it points to)."""
-    if epi is None:
-        return None, ()
-    xs, b = epi.get("Xself"), epi.get("bias")
-    st = RowEpilogueStruct(xs.data_ptr() if xs is not None else None, float(epi.get("self_coef", 0.0)),
-                           int(epi.get("self_mode", SELF_ALWAYS)), _pf32(b, "bias").value if b is not None else None,
-                           int(bool(epi.get("relu", False))))
-    return C.byref(st), (st, xs, b)
-
-
 def propagate_msg(g: Graph, msg, Xj, Xi=None, e_csr=None, op="sum", epi=None, out=None, argmax=None, ws=None):
-    """gnn_propagate_msg -> out, or (out, argmax) for max/min.  e_csr: float32 [E] or [E,width] in CSR order."""
-    Xj = _dev(Xj)
-    F = Xj.shape[1]
-    opc = _op(op)
-    ew = 0 if e_csr is None else (1 if e_csr.dim() == 1 else e_csr.shape[1])
-    if out is None:
-        out = torch.empty((g.N, F), dtype=Xj.dtype, device=Xj.device)
-    if opc in (MAX, MIN) and argmax is None:
-        argmax = torch.empty((g.N, F), dtype=torch.int32, device=Xj.device)
-    ws = _ws(g.E, F, opc, Xj.device, ws)
-    ep, keep = _epi(epi)
-    _check(load().gnn_propagate_msg(g.ref, msg, opc, _p(Xj), _p(Xi), _pf32(e_csr, "e_csr"), ew, F, _dtype(Xj), ep, _p(out),
-                                    _pi(argmax, torch.int32, "argmax"), _p(ws), ws.numel(), _stream()))
-    del keep
-    return (out, argmax) if opc in (MAX, MIN) else out
+    """gnn_propagate_msg -> out, or (out, argmax) for max/min.  e_csr: float32 [E] or [E,width] in CSR order.
+    epi: dict(Xself=, self_coef=, self_mode=, bias=, relu=) or None."""
+    return _b.propagate_msg(_addr(g.c), msg, Xj, Xi, e_csr, op, epi, out, argmax, ws)
 
 
 def propagate_msg_backward(g: Graph, msg, dOut, op="sum", Xj=None, e_csrT=None, e_width=0, argmax=None, self_grad=None,
                            want_dXj=True, want_dXi=False, want_de=False, ws=None):
     """gnn_propagate_msg_backward -> dict(dXj, dXi, de) with None for the outputs not asked for."""
-    dOut = _dev(dOut)
-    F = dOut.shape[1]
-    opc = _op(op)
-    ew = e_width or (0 if e_csrT is None else (1 if e_csrT.dim() == 1 else e_csrT.shape[1]))
-    dev = dOut.device
-    dXj = torch.empty((g.N, F), dtype=dOut.dtype, device=dev) if want_dXj else None
-    dXi = torch.empty((g.N, F), dtype=dOut.dtype, device=dev) if want_dXi else None
-    de = torch.empty((max(g.E, 1), max(ew, 1)), dtype=torch.float32, device=dev) if want_de else None
-    ws = _ws(g.E, F, opc, dev, ws)
-    sg, keep = _epi(self_grad)
-    _check(load().gnn_propagate_msg_backward(g.ref, msg, opc, _p(dOut), _p(Xj), _pf32(e_csrT, "e_csrT"), ew, _pi(argmax, torch.int32, "argmax"),
-                                             F, _dtype(dOut), sg, _p(dXj), _p(dXi), _p(de), _p(ws), ws.numel(), _stream()))
-    del keep
-    return dict(dXj=dXj, dXi=dXi, de=None if de is None else de[:g.E])
+    dXj, dXi, de = _b.propagate_msg_backward(_addr(g.c), msg, dOut, op, Xj, e_csrT, e_width, argmax, self_grad, want_dXj, want_dXi, want_de, ws)
+    return dict(dXj=dXj, dXi=dXi, de=de)
 
 
 def row_epilogue_backward(Y, dY, relu=True, want_dbias=True, dZ=None, ws=None):
     """-> (dZ, dbias or None)"""
-    dY = _dev(dY)
-    N, F = dY.shape
-    if dZ is None:
-        dZ = torch.empty_like(dY)
-    dbias = torch.empty(F, dtype=torch.float32, device=dY.device) if want_dbias else None
-    if ws is None:
-        ws = torch.empty(load().gnn_row_epilogue_backward_workspace(N, F), dtype=torch.uint8, device=dY.device)
-    _check(load().gnn_row_epilogue_backward(_p(Y), _p(dY), N, F, _dtype(dY), int(bool(relu)), _p(dZ), _p(dbias), _p(ws), ws.numel(), _stream()))
-    return dZ, dbias
+    return _b.row_epilogue_backward(Y, dY, relu, want_dbias, dZ, ws)
 
 
 def gin(g: Graph, X, eps, out=None, ws=None):
-    X = _dev(X)
-    F = X.shape[1]
-    if out is None:
-        out = torch.empty((g.N, F), dtype=X.dtype, device=X.device)
-    if ws is None:
-        ws = torch.empty(load().gnn_gin_workspace(g.E, F), dtype=torch.uint8, device=X.device)
-    _check(load().gnn_gin(g.ref, _p(X), float(eps), F, _dtype(X), _p(out), _p(ws), ws.numel(), _stream()))
-    return out
+    return _b.gin(_addr(g.c), X, eps, out, ws)
 
 
 def gin_backward(g: Graph, dOut, eps, X=None, want_deps=False, ws=None):
     """-> (dX, deps as a float32 device tensor of one element, or None)"""
-    dOut = _dev(dOut)
-    F = dOut.shape[1]
-    dX = torch.empty((g.N, F), dtype=dOut.dtype, device=dOut.device)
-    deps = torch.empty(1, dtype=torch.float32, device=dOut.device) if want_deps else None
-    if ws is None:
-        ws = torch.empty(load().gnn_gin_workspace(g.E, F), dtype=torch.uint8, device=dOut.device)
-    _check(load().gnn_gin_backward(g.ref, _p(dOut), _p(X), float(eps), F, _dtype(dOut), _p(dX), _p(deps), _p(ws), ws.numel(), _stream()))
-    return dX, deps
+    return _b.gin_backward(_addr(g.c), dOut, eps, X, want_deps, ws)
 
 
 def edge_dot(g: Graph, Xj, Xi, H=1):
     """s[p,h] = <Xi[row(p),h,:], Xj[col[p],h,:]> -> float32 [E,H], CSR order."""
-    Xj, Xi = _dev(Xj), _dev(Xi)
-    F = Xj.shape[1]
-    s = torch.empty((max(g.E, 1), H), dtype=torch.float32, device=Xj.device)
-    _check(load().gnn_edge_dot(g.ref, _p(Xj), _p(Xi), H, F // H, _dtype(Xj), _p(s), _stream()))
-    return s[:g.E]
+    return _b.edge_dot(_addr(g.c), Xj, Xi, H)
 
 
 def edge_dot_backward(g: Graph, Xj, Xi, ds_csr, H=1, want_dXj=True, want_dXi=True, ws=None):
-    Xj, Xi = _dev(Xj), _dev(Xi)
-    N, F = Xj.shape
-    dXj = torch.empty_like(Xj) if want_dXj else None
-    dXi = torch.empty_like(Xi) if want_dXi else None
-    if ws is None:
-        ws = torch.empty(load().gnn_edge_dot_backward_workspace(g.E, H, F // H), dtype=torch.uint8, device=Xj.device)
-    _check(load().gnn_edge_dot_backward(g.ref, _p(Xj), _p(Xi), _pf32(ds_csr, "ds_csr"), H, F // H, _dtype(Xj), _p(dXj), _p(dXi), _p(ws), ws.numel(), _stream()))
-    return dXj, dXi
+    return _b.edge_dot_backward(_addr(g.c), Xj, Xi, ds_csr, H, want_dXj, want_dXi, ws)
 
 
 def gatv2_logits(g: Graph, Xl, Xr, a, H, slope=0.2):
     """s[p,h] = sum_c a[h,c] * LeakyReLU(Xl[col[p],h,c] + Xr[row(p),h,c]) -> float32 [E,H], CSR order."""
-    Xl, Xr = _dev(Xl), _dev(Xr)
-    F = Xl.shape[1]
-    s = torch.empty((max(g.E, 1), H), dtype=torch.float32, device=Xl.device)
-    _check(load().gnn_gatv2_logits(g.ref, _p(Xl), _p(Xr), _pf32(a, "a"), H, F // H, _dtype(Xl), float(slope), _p(s), _stream()))
-    return s[:g.E]
+    return _b.gatv2_logits(_addr(g.c), Xl, Xr, a, H, slope)
 
 
 def gatv2_logits_backward(g: Graph, Xl, Xr, a, ds_csr, H, slope=0.2, ws=None):
     """-> (dXl, dXr, da)"""
-    Xl, Xr = _dev(Xl), _dev(Xr)
-    N, F = Xl.shape
-    dXl, dXr = torch.empty_like(Xl), torch.empty_like(Xr)
-    da = torch.empty((H, F // H), dtype=torch.float32, device=Xl.device)
-    if ws is None:
-        ws = torch.empty(load().gnn_gatv2_logits_backward_workspace(N, H, F // H), dtype=torch.uint8, device=Xl.device)
-    _check(load().gnn_gatv2_logits_backward(g.ref, _p(Xl), _p(Xr), _pf32(a, "a"), _pf32(ds_csr, "ds_csr"), H, F // H, _dtype(Xl), float(slope),
-                                            _p(dXl), _p(dXr), _p(da), _p(ws), ws.numel(), _stream()))
-    return dXl, dXr, da
+    return _b.gatv2_logits_backward(_addr(g.c), Xl, Xr, a, ds_csr, H, slope, ws)
 
 
 # ------------------------------------------------------------------ heterogeneous / temporal graphs
 def merge_edge_lists(segments):
     """segments: list of (src, dst, src_offset, dst_offset) with int32 device tensors -> (src, dst, seg) of the merged list."""
-    S = len(segments)
-    arr = (EdgeSegmentStruct * S)()
-    total = 0
-    for k, (src, dst, so, do) in enumerate(segments):
-        arr[k] = EdgeSegmentStruct(src.numel(), _pi(src, torch.int32, "src").value if src.numel() else None,
-                                   _pi(dst, torch.int32, "dst").value if dst.numel() else None, int(so), int(do))
-        total += src.numel()
-    dev = segments[0][0].device
-    so_, do_, sg_ = (torch.empty(max(total, 1), dtype=torch.int32, device=dev) for _ in range(3))
-    _check(load().gnn_merge_edge_lists(arr, S, _p(so_), _p(do_), _p(sg_), _stream()))
-    return so_[:total], do_[:total], sg_[:total]
+    return _b.merge_edge_lists(segments)
 
 
 def segment_coef(g: Graph, seg_csr, seg_is_mean, w_csr=None, want_T=True):
     """-> (coef_csr, coef_csrT or None): per-position multipliers of a merged multi-relation / multi-snapshot form."""
-    dev = g.rowptr.device
-    coef = torch.empty(max(g.E, 1), dtype=torch.float32, device=dev)
-    coefT = torch.empty(max(g.E, 1), dtype=torch.float32, device=dev) if want_T else None
-    _check(load().gnn_segment_coef(g.ref, _pi(seg_csr, torch.int32, "seg_csr"), _pf32(w_csr, "w_csr"), _pi(seg_is_mean, torch.int32, "seg_is_mean"),
-                                   seg_is_mean.numel(), _p(coef), _p(coefT), _stream()))
-    return coef[:g.E], (coefT[:g.E] if want_T else None)
+    return _b.segment_coef(_addr(g.c), seg_csr, seg_is_mean, w_csr, want_T, g.rowptr)
 
 
 # ------------------------------------------------------------------ unfused primitives
-def _ws(E, F, op, device, ws):
-    if ws is None:
-        ws = torch.empty(propagate_fused_workspace(E, F, op), dtype=torch.uint8, device=device)
-    return ws
-
-
 def gather(idx, X, out=None):
-    X = _dev(X)
-    E, F = idx.numel(), X.shape[1]
-    if out is None:
-        out = torch.empty((E, F), dtype=X.dtype, device=X.device)
-    _check(load().gnn_gather(_pi(idx, torch.int32, "idx"), E, _p(X), X.shape[0], F, _dtype(X), _p(out), _stream()))
-    return out
+    return _b.gather(idx, X, out)
 
 
 def gather_backward(g: Graph, dOut_EF, by_src=False, ws=None):
-    dOut_EF = _dev(dOut_EF)
-    F = dOut_EF.shape[1]
-    dX = torch.empty((g.N, F), dtype=dOut_EF.dtype, device=dOut_EF.device)
-    ws = _ws(g.E, F, SUM, dOut_EF.device, ws)
-    _check(load().gnn_gather_backward(g.ref, int(by_src), _p(dOut_EF), F, _dtype(dOut_EF), _p(dX), _p(ws), ws.numel(), _stream()))
-    return dX
+    return _b.gather_backward(_addr(g.c), dOut_EF, by_src, ws)
 
 
 def apply_edges(g: Graph, msg, X, ar=None, e=None, slope=0.2):
     """COPY_XJ / E_MUL_XJ: X [N,F], e float32 [E] or [E,w] (CSR order) -> m [E,F] of X.dtype.
     GAT_LOGIT: X = al, ar float32 [N,H] -> float32 [E,H]."""
-    X = _dev(X)
-    F = X.shape[1]
-    ew = 0 if e is None else (1 if e.dim() == 1 else e.shape[1])
-    m = torch.empty((max(g.E, 1), F), dtype=X.dtype, device=X.device)
-    _check(load().gnn_apply_edges(g.ref, msg, _p(X), _p(ar), _p(e), ew, F, _dtype(X), float(slope), _p(m), _stream()))
-    return m[:g.E]
+    return _b.apply_edges(_addr(g.c), msg, X, ar, e, slope)
 
 
 def aggregate(g: Graph, m_EF, op="sum", ws=None):
-    m_EF = _dev(m_EF)
-    F = m_EF.shape[1]
-    opc = _op(op)
-    out = torch.empty((g.N, F), dtype=m_EF.dtype, device=m_EF.device)
-    argmax = torch.empty((g.N, F), dtype=torch.int32, device=m_EF.device) if opc in (MAX, MIN) else None
-    ws = _ws(g.E, F, opc, m_EF.device, ws)
-    _check(load().gnn_aggregate(g.ref, opc, _p(m_EF), F, _dtype(m_EF), _p(out), _pi(argmax, torch.int32, "argmax"), _p(ws), ws.numel(), _stream()))
-    return (out, argmax) if opc in (MAX, MIN) else out
+    return _b.aggregate(_addr(g.c), m_EF, op, ws)
 
 
 def aggregate_backward(g: Graph, dOut, op="sum", argmax=None):
-    dOut = _dev(dOut)
-    F = dOut.shape[1]
-    dm = torch.empty((max(g.E, 1), F), dtype=dOut.dtype, device=dOut.device)
-    _check(load().gnn_aggregate_backward(g.ref, _op(op), _p(dOut), _pi(argmax, torch.int32, "argmax"), F, _dtype(dOut), _p(dm), _stream()))
-    return dm[:g.E]
+    return _b.aggregate_backward(_addr(g.c), dOut, op, argmax)
 
 
 def edge_softmax(g: Graph, logits, want_stats=False):
-    logits = _dev(logits)
-    H = logits.shape[1]
-    alpha = torch.empty_like(logits)
-    rmax = torch.empty((g.N, H), dtype=torch.float32, device=logits.device) if want_stats else None
-    rsum = torch.empty((g.N, H), dtype=torch.float32, device=logits.device) if want_stats else None
-    _check(load().gnn_edge_softmax(g.ref, _p(logits), H, _dtype(logits), _p(alpha), _p(rmax), _p(rsum), _stream()))
-    return (alpha, rmax, rsum) if want_stats else alpha
+    return _b.edge_softmax(_addr(g.c), logits, want_stats)
 
 
 def edge_softmax_backward(g: Graph, alpha, dalpha):
-    alpha, dalpha = _dev(alpha), _dev(dalpha)
-    ds = torch.empty_like(alpha)
-    _check(load().gnn_edge_softmax_backward(g.ref, _p(alpha), _p(dalpha), alpha.shape[1], _dtype(alpha), _p(ds), _stream()))
-    return ds
+    return _b.edge_softmax_backward(_addr(g.c), alpha, dalpha)
 
 
 # ------------------------------------------------------------------ pooling
 def graph_ptr_from_ids(graph_id, G):
-    N = graph_id.numel()
-    gptr = torch.empty(G + 1, dtype=torch.int64, device=graph_id.device)
-    ws = torch.empty(256, dtype=torch.uint8, device=graph_id.device)
-    _check(load().gnn_graph_ptr_from_ids(_pi(graph_id, torch.int32, "graph_id"), N, G, _p(gptr), _p(ws), ws.numel(), _stream()))
-    return gptr
+    return _b.graph_ptr_from_ids(graph_id, G)
 
 
 def reduce_nodes(graph_ptr, X, op="mean", ws=None):
-    X = _dev(X)
-    G, (N, F) = graph_ptr.numel() - 1, X.shape
-    opc = _op(op)
-    out = torch.empty((G, F), dtype=X.dtype, device=X.device)
-    argmax = torch.empty((G, F), dtype=torch.int32, device=X.device) if opc in (MAX, MIN) else None
-    ws = _ws(N, F, opc, X.device, ws)
-    _check(load().gnn_reduce_nodes(_pi(graph_ptr, torch.int64, "graph_ptr"), G, N, opc, _p(X), F, _dtype(X), _p(out), _pi(argmax, torch.int32, "argmax"), _p(ws), ws.numel(), _stream()))
-    return (out, argmax) if opc in (MAX, MIN) else out
+    return _b.reduce_nodes(graph_ptr, X, op, ws)
 
 
 def reduce_nodes_backward(graph_ptr, dOut, N, op="mean", argmax=None):
-    dOut = _dev(dOut)
-    G, F = dOut.shape
-    dX = torch.empty((N, F), dtype=dOut.dtype, device=dOut.device)
-    _check(load().gnn_reduce_nodes_backward(_pi(graph_ptr, torch.int64, "graph_ptr"), G, N, _op(op), _p(dOut), _pi(argmax, torch.int32, "argmax"), F, _dtype(dOut), _p(dX), _stream()))
-    return dX
+    return _b.reduce_nodes_backward(graph_ptr, dOut, N, op, argmax)
 
 
 # ------------------------------------------------------------------ GAT
 def gat_fused(g: Graph, Wx, a_src, a_dst, H, slope=0.2, ws=None):
     """Wx [N, H*C] -> dict(out, alpha (float32 [E,H], CSR order), al, ar (float32 [N,H]))."""
-    Wx = _dev(Wx)
-    N, F = Wx.shape
-    Cw = F // H
-    dev = Wx.device
-    out = torch.empty_like(Wx)
-    alpha = torch.empty((max(g.E, 1), H), dtype=torch.float32, device=dev)
-    al = torch.empty((N, H), dtype=torch.float32, device=dev)
-    ar = torch.empty((N, H), dtype=torch.float32, device=dev)
-    if ws is None:
-        ws = torch.empty(load().gnn_gat_fused_workspace(N, g.E, H, Cw, 0), dtype=torch.uint8, device=dev)
-    _check(load().gnn_gat_fused(g.ref, _p(Wx), _p(a_src), _p(a_dst), H, Cw, _dtype(Wx), float(slope), _p(out), _p(alpha),
-                                _p(al), _p(ar), _p(ws), ws.numel(), _stream()))
-    return dict(out=out, alpha=alpha[:g.E], al=al, ar=ar)
+    out, alpha, al, ar = _b.gat_fused(_addr(g.c), Wx, a_src, a_dst, H, slope, ws)
+    return dict(out=out, alpha=alpha, al=al, ar=ar)
 
 
 def gat_fused_backward(g: Graph, Wx, a_src, a_dst, fwd, dOut, H, slope=0.2, ws=None):
-    Wx, dOut = _dev(Wx), _dev(dOut)
-    N, F = Wx.shape
-    Cw = F // H
-    dev = Wx.device
-    dWx = torch.empty_like(Wx)
-    da_src = torch.empty((H, Cw), dtype=torch.float32, device=dev)
-    da_dst = torch.empty((H, Cw), dtype=torch.float32, device=dev)
-    if ws is None:
-        ws = torch.empty(load().gnn_gat_fused_workspace(N, g.E, H, Cw, 1), dtype=torch.uint8, device=dev)
-    _check(load().gnn_gat_fused_backward(g.ref, _p(Wx), _p(a_src), _p(a_dst), _p(fwd["alpha"]), _p(fwd["al"]), _p(fwd["ar"]),
-                                         _p(dOut), H, Cw, _dtype(Wx), float(slope), _p(dWx), _p(da_src), _p(da_dst),
-                                         _p(ws), ws.numel(), _stream()))
+    dWx, da_src, da_dst = _b.gat_fused_backward(_addr(g.c), Wx, a_src, a_dst, fwd["alpha"], fwd["al"], fwd["ar"], dOut, H, slope, ws)
     return dict(dWx=dWx, da_src=da_src, da_dst=da_dst)
 
 
@@ -599,82 +405,32 @@ def propagate_fused_static(g: Graph, X, w_csr=None, op="sum", out=None, argmax=N
     """gnn_propagate_fused_static: the fused propagate with the library's built-in 8 MiB scratch, for
     embedders that may not allocate device memory.  The caller passes `out` (and `argmax` for max/min);
     nothing is allocated here when they are given."""
-    X = _dev(X)
-    F = X.shape[1]
-    opc = _op(op)
-    if out is None:
-        out = torch.empty((g.N, F), dtype=X.dtype, device=X.device)
-    if opc in (MAX, MIN) and argmax is None:
-        argmax = torch.empty((g.N, F), dtype=torch.int32, device=X.device)
-    msg = COPY_XJ if w_csr is None else E_MUL_XJ
-    _check(load().gnn_propagate_fused_static(g.ref, msg, opc, _p(X), _pf32(w_csr, "w_csr"), F, _dtype(X), _p(out), _pi(argmax, torch.int32, "argmax"), _stream()))
-    return (out, argmax) if opc in (MAX, MIN) else out
+    return _b.propagate_fused(_addr(g.c), X, w_csr, op, out, argmax, False)
 
 
 # ------------------------------------------------------------------ dense transform
 def linear(X, W, ws=None, return_ws=False):
-    X, W = _dev(X), _dev(W)
-    (N, K), M = X.shape, W.shape[1]
-    Y = torch.empty((N, M), dtype=X.dtype, device=X.device)
-    if ws is None:
-        ws = torch.empty(load().gnn_linear_workspace(N, K, M), dtype=torch.uint8, device=X.device)
-    _check(load().gnn_linear(_p(X), _p(W), N, K, M, _dtype(X), _p(Y), _p(ws), ws.numel(), _stream()))
-    return (Y, ws) if return_ws else Y
+    return _b.linear(X, W, None, False, ws, return_ws)
 
 
 def linear_bias_act(X, W, bias=None, relu=False, ws=None):
     """Y = act(X W + bias) with the tail inside the product kernel's epilogue."""
-    X, W = _dev(X), _dev(W)
-    (N, K), M = X.shape, W.shape[1]
-    Y = torch.empty((N, M), dtype=X.dtype, device=X.device)
-    if ws is None:
-        ws = torch.empty(load().gnn_linear_workspace(N, K, M), dtype=torch.uint8, device=X.device)
-    _check(load().gnn_linear_bias_act(_p(X), _p(W), N, K, M, _dtype(X), _pf32(bias, "bias"), int(bool(relu)), _p(Y), _p(ws), ws.numel(), _stream()))
-    return Y
+    return _b.linear(X, W, bias, relu, ws, False)
 
 
 def propagate_linear(g: Graph, X, W, w_csr=None, op="sum", bias=None, relu=False, ws=None, return_ws=False):
     """Y = act((op over incoming edges of w * X[source]) W + bias) in one kernel."""
-    X, W = _dev(X), _dev(W)
-    K, M = W.shape
-    Y = torch.empty((g.N, M), dtype=X.dtype, device=X.device)
-    if ws is None:
-        ws = torch.empty(load().gnn_propagate_linear_workspace(g.N, g.E, K, M), dtype=torch.uint8, device=X.device)
-    msg = COPY_XJ if w_csr is None else E_MUL_XJ
-    _check(load().gnn_propagate_linear(g.ref, msg, _op(op), _p(X), _pf32(w_csr, "w_csr"), _p(W), K, M, _dtype(X), _pf32(bias, "bias"),
-                                       int(bool(relu)), _p(Y), _p(ws), ws.numel(), _stream()))
-    return (Y, ws) if return_ws else Y
+    return _b.propagate_linear(_addr(g.c), X, W, w_csr, op, bias, relu, ws, return_ws)
 
 
 def propagate_linear_backward(g: Graph, dY, X, W, w_csrT=None, op="sum", want_dX=True, want_dW=True, ws=None):
     """-> (dX or None, dW or None)"""
-    dY, W = _dev(dY), _dev(W)
-    K, M = W.shape
-    dX = torch.empty((g.N, K), dtype=dY.dtype, device=dY.device) if want_dX else None
-    dW = torch.empty((K, M), dtype=dY.dtype, device=dY.device) if want_dW else None
-    if ws is None:
-        ws = torch.empty(load().gnn_propagate_linear_workspace(g.N, g.E, K, M), dtype=torch.uint8, device=dY.device)
-    msg = COPY_XJ if w_csrT is None else E_MUL_XJ
-    _check(load().gnn_propagate_linear_backward(g.ref, msg, _op(op), _p(dY), _p(X), _pf32(w_csrT, "w_csrT"), _p(W), K, M, _dtype(dY),
-                                                _p(dX), _p(dW), _p(ws), ws.numel(), _stream()))
-    return dX, dW
+    return _b.propagate_linear_backward(_addr(g.c), dY, X, W, w_csrT, op, want_dX, want_dW, ws)
 
 
 def linear_backward(X, W, dY, want_dX=True, want_dW=True, ws=None, return_ws=False):
-    dY = _dev(dY)
-    N, M = dY.shape
-    K = W.shape[0] if W is not None else X.shape[1]
-    dX = torch.empty((N, K), dtype=dY.dtype, device=dY.device) if want_dX else None
-    dW = torch.empty((K, M), dtype=dY.dtype, device=dY.device) if want_dW else None
-    if ws is None:
-        ws = torch.empty(load().gnn_linear_workspace(N, K, M), dtype=torch.uint8, device=dY.device)
-    _check(load().gnn_linear_backward(_p(X), _p(W), _p(dY), N, K, M, _dtype(dY), _p(dX), _p(dW), _p(ws), ws.numel(), _stream()))
-    return (dX, dW, ws) if return_ws else (dX, dW)
+    return _b.linear_backward(X, W, dY, want_dX, want_dW, ws, return_ws)
 
 
 def axpby(alpha, a, beta, b, out=None):
-    a, b = _dev(a), _dev(b)
-    if out is None:
-        out = torch.empty_like(a)
-    _check(load().gnn_axpby(float(alpha), _p(a), float(beta), _p(b), a.numel(), _dtype(a), _p(out), _stream()))
-    return out
+    return _b.axpby(a, b, alpha, beta, out)
