@@ -45,8 +45,32 @@ static inline int grid_for(int64_t n, int threads) {
     return (int)(b < cap ? b : cap);
 }
 
-// ---------------------------------------------------------------- device helpers
 #ifdef __CUDACC__
+// ---------------------------------------------------------------- launches
+// Launch whose blocks may be set up while the kernel before it in the stream drains.  The kernel's first statement is
+// pdl_wait(): nothing of it touches global memory before all earlier work of the stream is complete and visible, so the
+// order of the stream is kept; what overlaps is the launch latency (about 1 us of a 3-5 us kernel on a small graph).
+template <class... Params, class... Args>
+static inline void launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);  // errors: GNN_CHECK_LAUNCH of the caller
+}
+
+// ---------------------------------------------------------------- device helpers
+// every thread of a kernel started by launch_overlapped, before its first access to global memory
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the next kernel of the stream may be set up from here on
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 
 // 16-byte global loads/stores with L2 cache policies (createpolicy + .L2::cache_hint).
 //   feature rows that are gathered many times: keep in L2 (evict_last)
@@ -85,6 +109,16 @@ __device__ __forceinline__ int ld_hint_i32(const int* p, uint64_t pol) {
 __device__ __forceinline__ float ld_hint_f32(const float* p, uint64_t pol) {
     float v;
     asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
+    return v;
+}
+__device__ __forceinline__ int ld_stream_i32(const int* p) {
+    int v;
+    asm volatile("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_stream_f32(const float* p) {
+    float v;
+    asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 }
 __device__ __forceinline__ void st_stream16(void* p, uint4 v) {

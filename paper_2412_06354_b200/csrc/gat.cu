@@ -385,16 +385,7 @@ gnn_status gnn_gat_fused_backward(const gnn_csr* g, const void* Wx, const float*
         GNN_FAIL(GNN_ERR_CUDA, "%s: launch failed", who);
     }
     // dWx[j,h,:] = sum_q alpha[t2f[q],h]*dOut[colT[q],h,:] + dal[j,h]*a_src[h,:] + dar[j,h]*a_dst[h,:]
-    // the flat kernel reads alpha through t2f; the row-walking one wants it permuted to transposed order first
-    const bool indexed = chunked_is_flat(g->E, F, dtype);
-    if (g->E > 0 && !indexed) {
-        rc = gnn_permute_edge_data(g->t2f, g->E, H, 4, alpha_csr, w.alphaT, stream);
-        if (rc != GNN_OK) {
-            side_join(st, side);
-            return rc;
-        }
-    }
-    HeadExtra hx = {indexed ? alpha_csr : w.alphaT, indexed ? g->t2f : nullptr, H, w.dal, w.dar, a_src, a_dst};
+    HeadExtra hx = {alpha_csr, g->t2f, H, w.dal, w.dar, a_src, a_dst};
     rc = run_chunked(who, MODE_HEADSUM, g->N, g->E, g->rowptrT, g->colT, nullptr, dOut, dWx, nullptr, nullptr,
                      nullptr, nullptr, 0, F, dtype, w.chunk_ws, w.chunk_bytes, st, &hx);
     side_join(st, side);  // the call's work is complete in the caller's stream only once the side branch is

@@ -1,19 +1,19 @@
-// Declarations shared by the kernels that reduce gathered rows over fixed edge chunks.
+// Declarations shared by the calls that reduce gathered rows.
 #pragma once
 #include "common.cuh"
 
 namespace gnn {
 
-constexpr int PF_SLAB = 256;   // positions staged in shared memory at a time
+constexpr int PF_SLAB = 256;   // positions per warp of the edge-wise dot products
 constexpr int PF_WARPS = 8;    // warps per block
 
-enum { MODE_SUM = 0, MODE_MAX = 1, MODE_MIN = 2, MODE_ROUTE = 3, MODE_HEADSUM = 4, MODE_EFSUM = 5 };
+enum { MODE_SUM = 0, MODE_MAX = 1, MODE_MIN = 2, MODE_ROUTE = 3, MODE_HEADSUM = 4, MODE_EFSUM = 5, MODE_WSUM = 6 };
 
 // MODE_HEADSUM extras: multipliers per (position, head) and an optional rank-1 row epilogue
 //   out[r,f] += epi_l[r,h(f)] * epi_a[f] + epi_r[r,h(f)] * epi_b[f]
 struct HeadExtra {
     const float* wh;  // [E,H]
-    const int32_t* wh_index;  // nullptr: position p uses row p of wh; else row wh_index[p] (only where chunked_is_flat())
+    const int32_t* wh_index;  // nullptr: position p uses row p of wh; else row wh_index[p]
     int H;
     const float *epi_l, *epi_r;  // [rows,H] or nullptr
     const float *epi_a, *epi_b;  // [F]
@@ -39,10 +39,7 @@ bool pick_shape(int nvec, int* lpr, int* vpl);
 
 size_t chunked_workspace(int64_t E, int F, bool with_arg);
 
-// does run_chunked use the position-first (flat) kernel for this problem?  (It honours HeadExtra::wh_index.)
-bool chunked_is_flat(int64_t E, int F, gnn_dtype dtype);
-
-// out[r,:] = reduce over positions p of row r of  w[p] * X[col[p],:]   (see propagate.cu)
+// out[r,:] = reduce over positions p of row r of  w[p] * X[col[p],:]   (see reduce_rows.cuh)
 gnn_status run_chunked(const char* who, int mode, int32_t N, int64_t E, const int64_t* rowptr,
                        const int32_t* col, const float* w, const void* X, void* out,
                        int32_t* argmax, const int64_t* gscale_rowptr, const int32_t* route_arg,

@@ -1,0 +1,6 @@
+// Segmented reductions over f32 rows: max, min, the routing of their backward pass and per-feature factors.
+#include "reduce_rows.cuh"
+
+namespace gnn {
+template void launch_reduce_others<float>(const PropParams&, int, bool, cudaStream_t);
+}  // namespace gnn

@@ -1,0 +1,6 @@
+// Segmented reductions over f32 rows: sums (plain, one factor per position, one per position and head).
+#include "reduce_rows.cuh"
+
+namespace gnn {
+template void launch_reduce_sums<float>(const PropParams&, int, bool, cudaStream_t);
+}  // namespace gnn
