@@ -778,7 +778,7 @@ FN(linear) {
     at::Tensor Y = empty({N, M}, X.scalar_type(), X.device());
     const size_t need = gnn_linear_workspace((int32_t)N, (int)K, (int)M);
     const at::Tensor wt = linear_scratch(A, 4, wanted, need, X.device());
-    Scratch ws(wt, 256, X.device());  // the forward call uses the status word only
+    Scratch ws(wt, K % 8 == 0 && M % 8 == 0 ? 256 : need, X.device());  // the status word only, unless rows may have to be padded
     const float* b = f32(A.t(2), "bias");
     const gnn_dtype dt = dtype_of(X);
     const gnn_stream st = stream();

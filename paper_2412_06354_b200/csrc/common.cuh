@@ -67,9 +67,12 @@ static inline void launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 
 
 // ---------------------------------------------------------------- device helpers
 // every thread of a kernel started by launch_overlapped, before its first access to global memory
+__device__ __forceinline__ void pdl_wait_exclusive() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// ... and in kernels that leave room on an SM (the persistent dense kernels take all of its shared memory): the next kernel
+// of the stream may be set up from here on.
 __device__ __forceinline__ void pdl_wait() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // the next kernel of the stream may be set up from here on
-    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_wait_exclusive();
 }
 
 // 16-byte global loads/stores with L2 cache policies (createpolicy + .L2::cache_hint).

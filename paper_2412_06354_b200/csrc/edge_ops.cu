@@ -48,6 +48,7 @@ struct PosChunk {
 // out[k, chunk] = X[idx[k], chunk]; one thread per 16-byte chunk
 __global__ void gather_rows_kernel(const int32_t* __restrict__ idx, int64_t E, const uint4* __restrict__ X,
                                    int nvec, uint4* __restrict__ out) {
+    pdl_wait();
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x, total = E * nvec;
     for (PosChunk q(t, stride, nvec); t < total; t += stride, q.next()) out[t] = X[(size_t)idx[q.p] * nvec + q.ci];
@@ -58,6 +59,7 @@ template <typename T>
 __global__ void apply_edges_mul_kernel(const int32_t* __restrict__ col, int64_t E, const uint4* __restrict__ X,
                                        int nvec, const float* __restrict__ e, int ew, int feats_per_e,
                                        uint4* __restrict__ m) {
+    pdl_wait();
     constexpr int EPC = Chunk<T>::N;
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x, total = E * nvec;
@@ -85,6 +87,7 @@ __global__ void apply_edges_mul_kernel(const int32_t* __restrict__ col, int64_t 
 __global__ void gat_logit_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int N,
                                  int64_t E, int H, const float* __restrict__ al, const float* __restrict__ ar,
                                  float slope, float* __restrict__ s) {
+    pdl_wait();
     int64_t t0, t1;
     block_span(E * H, &t0, &t1);
     int i = -1;
@@ -102,6 +105,7 @@ template <typename T>
 __global__ void aggregate_backward_kernel(const int64_t* __restrict__ rowptr, int N, int64_t E, int op,
                                           const uint4* __restrict__ dOut, const int32_t* __restrict__ argmax,
                                           int nvec, uint4* __restrict__ dm) {
+    pdl_wait();
     constexpr int EPC = Chunk<T>::N;
     int64_t t0, t1;
     block_span(E * nvec, &t0, &t1);
@@ -139,6 +143,7 @@ static gnn_status check_rows(const char* who, int F, gnn_dtype dtype, int* nvec)
 // graph_ptr[g] = first node whose graph id is >= g; flag set if ids are unsorted or out of range
 __global__ void graph_ptr_kernel(const int32_t* __restrict__ gid, int32_t N, int32_t G,
                                  int64_t* __restrict__ gptr, int* __restrict__ flag) {
+    pdl_wait();
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t n = t; n < N; n += stride) {
@@ -159,6 +164,7 @@ __global__ void graph_ptr_kernel(const int32_t* __restrict__ gid, int32_t N, int
 template <typename T>
 __global__ void axpby_kernel(float alpha, const uint4* __restrict__ a, float beta, const uint4* __restrict__ b,
                              int64_t nvec, uint4* __restrict__ out) {
+    pdl_wait();
     constexpr int EPC = Chunk<T>::N;
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -188,7 +194,7 @@ gnn_status gnn_gather(const int32_t* idx, int64_t E, const void* X, int32_t N, i
     if (E == 0) return GNN_OK;
     GNN_REQUIRE(idx && X && out && aligned16(X) && aligned16(out), GNN_ERR_INVALID_ARG,
                 "%s: null or misaligned argument", who);
-    gather_rows_kernel<<<grid_for(E * nvec, 256), 256, 0, as_stream(stream)>>>(idx, E, (const uint4*)X, nvec, (uint4*)out);
+    launch_overlapped(gather_rows_kernel, dim3((unsigned)(grid_for(E * nvec, 256))), dim3(256), 0, as_stream(stream), idx, E, (const uint4*)X, nvec, (uint4*)out);
     GNN_CHECK_LAUNCH(who);
     return GNN_OK;
 }
@@ -216,7 +222,7 @@ gnn_status gnn_apply_edges(const gnn_csr* g, gnn_msg msg, const void* X_or_al, c
     if (msg == GNN_MSG_GAT_LOGIT) {
         GNN_REQUIRE(dtype == GNN_F32, GNN_ERR_UNSUPPORTED, "%s: GAT_LOGIT works on fp32 scores", who);
         GNN_REQUIRE(ar && F > 0, GNN_ERR_INVALID_ARG, "%s: GAT_LOGIT needs ar and F = heads", who);
-        gat_logit_kernel<<<grid_for(g->E * F, 256), 256, 0, st>>>(g->rowptr, g->col, g->N, g->E, F, (const float*)X_or_al,
+        launch_overlapped(gat_logit_kernel, dim3((unsigned)(grid_for(g->E * F, 256))), dim3(256), 0, st, g->rowptr, g->col, g->N, g->E, F, (const float*)X_or_al,
                                                                   (const float*)ar, slope, (float*)m_out);
         GNN_CHECK_LAUNCH(who);
         return GNN_OK;
@@ -239,9 +245,9 @@ gnn_status gnn_apply_edges(const gnn_csr* g, gnn_msg msg, const void* X_or_al, c
     }
     const int grid = grid_for(g->E * nvec, 256);
     if (dtype == GNN_F32)
-        apply_edges_mul_kernel<float><<<grid, 256, 0, st>>>(g->col, g->E, (const uint4*)X_or_al, nvec, e, e_width, feats_per_e, (uint4*)m_out);
+        launch_overlapped(apply_edges_mul_kernel<float>, dim3((unsigned)(grid)), dim3(256), 0, st, g->col, g->E, (const uint4*)X_or_al, nvec, e, e_width, feats_per_e, (uint4*)m_out);
     else
-        apply_edges_mul_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(g->col, g->E, (const uint4*)X_or_al, nvec, e, e_width, feats_per_e, (uint4*)m_out);
+        launch_overlapped(apply_edges_mul_kernel<__nv_bfloat16>, dim3((unsigned)(grid)), dim3(256), 0, st, g->col, g->E, (const uint4*)X_or_al, nvec, e, e_width, feats_per_e, (uint4*)m_out);
     GNN_CHECK_LAUNCH(who);
     return GNN_OK;
 }
@@ -273,9 +279,9 @@ gnn_status gnn_aggregate_backward(const gnn_csr* g, gnn_op op, const void* dOut_
     const int grid = grid_for(g->E * nvec, 256);
     cudaStream_t st = as_stream(stream);
     if (dtype == GNN_F32)
-        aggregate_backward_kernel<float><<<grid, 256, 0, st>>>(g->rowptr, g->N, g->E, (int)op, (const uint4*)dOut_NF, argmax, nvec, (uint4*)dm_EF);
+        launch_overlapped(aggregate_backward_kernel<float>, dim3((unsigned)(grid)), dim3(256), 0, st, g->rowptr, g->N, g->E, (int)op, (const uint4*)dOut_NF, argmax, nvec, (uint4*)dm_EF);
     else
-        aggregate_backward_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(g->rowptr, g->N, g->E, (int)op, (const uint4*)dOut_NF, argmax, nvec, (uint4*)dm_EF);
+        launch_overlapped(aggregate_backward_kernel<__nv_bfloat16>, dim3((unsigned)(grid)), dim3(256), 0, st, g->rowptr, g->N, g->E, (int)op, (const uint4*)dOut_NF, argmax, nvec, (uint4*)dm_EF);
     GNN_CHECK_LAUNCH(who);
     return GNN_OK;
 }
@@ -288,7 +294,7 @@ gnn_status gnn_graph_ptr_from_ids(const int32_t* graph_id, int32_t N, int32_t G,
     cudaStream_t st = as_stream(stream);
     int* flag = (int*)ws;
     if (cudaMemsetAsync(flag, 0, 4, st) != cudaSuccess) GNN_FAIL(GNN_ERR_CUDA, "%s: memset failed", who);
-    graph_ptr_kernel<<<grid_for((N > G ? N : G) + 1, 256), 256, 0, st>>>(graph_id, N, G, graph_ptr, flag);
+    launch_overlapped(graph_ptr_kernel, dim3((unsigned)(grid_for((N > G ? N : G) + 1, 256))), dim3(256), 0, st, graph_id, N, G, graph_ptr, flag);
     GNN_CHECK_LAUNCH(who);
     int h = 0;
     if (cudaMemcpyAsync(&h, flag, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess)
@@ -325,9 +331,9 @@ gnn_status gnn_reduce_nodes_backward(const int64_t* graph_ptr, int32_t G, int32_
     const int grid = grid_for((int64_t)N * nvec, 256);
     cudaStream_t st = as_stream(stream);
     if (dtype == GNN_F32)
-        aggregate_backward_kernel<float><<<grid, 256, 0, st>>>(graph_ptr, G, N, (int)op, (const uint4*)dOut_GF, argmax, nvec, (uint4*)dX_NF);
+        launch_overlapped(aggregate_backward_kernel<float>, dim3((unsigned)(grid)), dim3(256), 0, st, graph_ptr, G, N, (int)op, (const uint4*)dOut_GF, argmax, nvec, (uint4*)dX_NF);
     else
-        aggregate_backward_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(graph_ptr, G, N, (int)op, (const uint4*)dOut_GF, argmax, nvec, (uint4*)dX_NF);
+        launch_overlapped(aggregate_backward_kernel<__nv_bfloat16>, dim3((unsigned)(grid)), dim3(256), 0, st, graph_ptr, G, N, (int)op, (const uint4*)dOut_GF, argmax, nvec, (uint4*)dX_NF);
     GNN_CHECK_LAUNCH(who);
     return GNN_OK;
 }
@@ -342,8 +348,8 @@ gnn_status gnn_axpby(float alpha, const void* a, float beta, const void* b, int6
     GNN_REQUIRE(a && b && out && aligned16(a) && aligned16(b) && aligned16(out), GNN_ERR_INVALID_ARG, "%s: null or misaligned argument", who);
     const int64_t nvec = n / epc;
     cudaStream_t st = as_stream(stream);
-    if (dtype == GNN_F32) axpby_kernel<float><<<grid_for(nvec, 256), 256, 0, st>>>(alpha, (const uint4*)a, beta, (const uint4*)b, nvec, (uint4*)out);
-    else axpby_kernel<__nv_bfloat16><<<grid_for(nvec, 256), 256, 0, st>>>(alpha, (const uint4*)a, beta, (const uint4*)b, nvec, (uint4*)out);
+    if (dtype == GNN_F32) launch_overlapped(axpby_kernel<float>, dim3((unsigned)(grid_for(nvec, 256))), dim3(256), 0, st, alpha, (const uint4*)a, beta, (const uint4*)b, nvec, (uint4*)out);
+    else launch_overlapped(axpby_kernel<__nv_bfloat16>, dim3((unsigned)(grid_for(nvec, 256))), dim3(256), 0, st, alpha, (const uint4*)a, beta, (const uint4*)b, nvec, (uint4*)out);
     GNN_CHECK_LAUNCH(who);
     return GNN_OK;
 }

@@ -3,12 +3,14 @@
 //   dX = dY * W^T      dY [N,M]
 //   dW = X^T * dY      reduction over the N rows, split over row slabs and combined in slab order
 //
-// This file holds the entry points, their dispatch, and the fallback.  With K and M multiples of 16
-// (16..256) the products run on the 5th-generation tensor cores (tcgen05.mma, accumulators in tensor
-// memory): the pipelined kernels of linear_tma.cu (bf16: Y, dX, dW; fp32: Y, dX) or the
-// single-buffered ones of linear_tc.cu (fp32 dW, fp32 weights too large for the pipeline, and bf16 when
-// the tensor-map encoder is not available).  Everything else runs the shared-memory tiled FFMA kernel
-// below with fp32 accumulation.  All sums have a fixed order.
+// This file holds the entry points, their dispatch, and the fallback.  The products run on the 5th-generation tensor cores
+// (tcgen05.mma, accumulators in tensor memory) through the pipelined kernels of linear_tma.cu for a contraction of up to
+// 512 and up to 1024 output columns (dW: 512 x 256, or as much as fits tensor memory at a time), whatever the divisors of
+// K and M: sizes are rounded up with zeros from the copy engine.  The copy engine wants rows that start on 16 bytes;
+// matrices whose rows do not (K or M odd, say) are first copied to padded rows in the workspace, one pass at L2 or HBM
+// speed.  Such shapes took the FFMA kernel before (170000 x 100 x 47 fp32, forward and backward: 1410 -> 121 us).
+// linear_tc.cu (single-buffered) takes over if the tensor-map encoder is not available; everything else runs the
+// shared-memory tiled FFMA kernel below with fp32 accumulation.  All sums have a fixed order.
 #include "common.cuh"
 
 namespace gnn {
@@ -87,30 +89,53 @@ gemm_simt_kernel(const TA* __restrict__ A, int64_t sam, int64_t sak, const TB* _
     }
 }
 
-// out[i] = sum over slabs of part[s][i] in a fixed order: the slabs are cut into four contiguous
-// groups, each summed in ascending order by one thread, and the four group sums are added in
-// ascending group order.  64 elements x 4 groups per block.
+// out[i] = sum over slabs of part[s][i] in a fixed order: eight contiguous groups of slabs, each summed in ascending order
+// by one thread with eight loads in flight, then added in ascending group order.  32 elements x 8 groups per block
+// (4.7 us for the 148 partials of a 128 x 128 result: 9.7 MB from L2).
 template <typename TC>
 __global__ void __launch_bounds__(256)
-slab_sum_kernel(const float* __restrict__ part, int slabs, int64_t n, TC* __restrict__ out, int cols, int ld, int c0) {
-    __shared__ float gsum[4][64];
-    const int e = threadIdx.x & 63, g = threadIdx.x >> 6;
-    const int64_t i = blockIdx.x * (int64_t)64 + e;
-    const int per = (slabs + 3) / 4, z0 = g * per, z1 = min(slabs, z0 + per);
+slab_sum_kernel(const float* __restrict__ part, int slabs, int64_t n, TC* __restrict__ out, int cols, int rows_out, int cols_out, int ld, int c0) {
+    __shared__ float gsum[8][32];
+    pdl_wait();
+    const int e = threadIdx.x & 31, g = threadIdx.x >> 5;
+    const int64_t i = blockIdx.x * (int64_t)32 + e;
+    const int per = (slabs + 7) / 8, z0 = g * per, z1 = min(slabs, z0 + per);
     float s = 0.f;
     if (i < n) {
-        int z = z0;
-        for (; z + 4 <= z1; z += 4) {
-            const float a = part[(size_t)z * n + i], b = part[(size_t)(z + 1) * n + i], c = part[(size_t)(z + 2) * n + i],
-                        d = part[(size_t)(z + 3) * n + i];
-            s += a; s += b; s += c; s += d;
+        for (int z = z0; z < z1; z += 8) {
+            float v[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = z + u < z1 ? part[(size_t)(z + u) * n + i] : 0.f;
+#pragma unroll
+            for (int u = 0; u < 8; ++u) s += v[u];
         }
-        for (; z < z1; ++z) s += part[(size_t)z * n + i];
     }
     gsum[g][e] = s;
     __syncthreads();
-    // the partials are [rows, cols]; the result may be a block of columns (c0 ..) of a matrix with rows ld apart
-    if (g == 0 && i < n) out[(i / cols) * ld + c0 + (i % cols)] = from_f32<TC>(((gsum[0][e] + gsum[1][e]) + gsum[2][e]) + gsum[3][e]);
+    // the partials are [rows, cols], of which [rows_out, cols_out] exist; the result may be a block of columns (c0 ..) of a
+    // matrix with rows ld apart
+    if (g == 0 && i < n) {
+        const int r = (int)(i / cols), c = (int)(i % cols);
+#pragma unroll
+        for (int k = 1; k < 8; ++k) s += gsum[k][e];
+        if (r < rows_out && c < cols_out) out[(int64_t)r * ld + c0 + c] = from_f32<TC>(s);
+    }
+}
+
+// dst[r, 0..cols) = src[r, 0..cols), rows of dst `chunks` 16-byte chunks apart: a thread per chunk.  What follows the last
+// column in a row of dst is zero and never read (the tensor maps know the real width).
+template <typename TE, int PER>
+__global__ void __launch_bounds__(256)
+pad_rows_kernel(const TE* __restrict__ src, int64_t rows, int cols, TE* __restrict__ dst, int chunks) {
+    pdl_wait();
+    const int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x;
+    if (i >= rows * chunks) return;
+    const int64_t r = i / chunks;
+    const int c = (int)(i - r * chunks) * PER;
+    union { TE e[PER]; uint4 v; } u;
+#pragma unroll
+    for (int k = 0; k < PER; ++k) u.e[k] = c + k < cols ? src[r * cols + c + k] : TE(0);
+    *reinterpret_cast<uint4*>(dst + (r * chunks) * PER + c) = u.v;
 }
 
 template <typename TA, typename TB, typename TC>
@@ -130,21 +155,56 @@ bool linear_tc_supported(int64_t N, int K, int M, gnn_dtype dtype);
 gnn_status linear_tc_forward(const void* X, const void* W, int64_t N, int K, int M, int w_transposed, gnn_dtype dtype,
                              void* Y, int* d_flag, cudaStream_t st);
 bool linear_tma_supported(int64_t N, int Kc, int Mo, int b_transposed, gnn_dtype dtype);
-gnn_status linear_tma_forward(const void* X, const void* W, int64_t N, int Kc, int Mo, int b_transposed, void* Y, int* d_flag,
-                              cudaStream_t st, const float* bias = nullptr, int relu = 0);
+gnn_status linear_tma_forward(const void* X, int ldx, const void* W, int ldw, int64_t N, int Kc, int Mo, int b_transposed, void* Y, int* d_flag, int reset,
+                              cudaStream_t st, const float* bias, int relu);
 bool linear_tma_f32_supported(int64_t N, int Kc, int Mo, gnn_dtype dtype);
-gnn_status linear_tma_f32_forward(const void* X, const void* W, int64_t N, int Kc, int Mo, int b_transposed, void* Y, int* d_flag,
-                                  cudaStream_t st, const float* bias = nullptr, int relu = 0);
+gnn_status linear_tma_f32_forward(const void* X, int ldx, const void* W, int64_t N, int Kc, int Mo, int b_transposed, void* Y, int* d_flag, int reset,
+                                  cudaStream_t st, const float* bias, int relu);
 bool linear_tma_dw_supported(int64_t N, int K, int M, gnn_dtype dtype);
+int linear_tma_dw_partials(int64_t N);
+gnn_status linear_tma_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, float* part, int* d_flag, int reset, cudaStream_t st);
 bool linear_tma_f32_dw_supported(int64_t N, int K, int M, gnn_dtype dtype);
 int linear_tma_f32_dw_partials(int64_t N);
-gnn_status linear_tma_f32_dw(const void* X, const void* dY, int64_t N, int K, int M, int ldd, float* part, int* d_flag, cudaStream_t st);
-int linear_tma_dw_partials(int64_t N);
-gnn_status linear_tma_dw(const void* X, const void* dY, int64_t N, int K, int M, int ldd, float* part, int* d_flag, cudaStream_t st);
+gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, float* part, int* d_flag, int reset, cudaStream_t st);
 bool linear_tc_dw_supported(int64_t N, int K, int M, gnn_dtype dtype);
 int linear_tc_dw_partials(int64_t N);
 gnn_status linear_tc_dw(const void* X, const void* dY, int64_t N, int K, int M, gnn_dtype dtype, float* part, int* d_flag,
                         cudaStream_t st);
+
+static int round_up(int x, int m) { return (x + m - 1) / m * m; }
+
+// elements between rows of a matrix of `cols` columns whose rows start on 16 bytes
+static int padded(int cols, int s) { return round_up(cols, 16 / s); }
+
+// Workspace layout: status word (256 bytes), dW partials, then the padded copies of X, dY and W.  The element type is not
+// known where the size is asked for: rows that would be padded in either type count, in the larger one.
+struct LinearWs {
+    size_t part, x, dy, w, bytes;
+    LinearWs(int64_t N, int K, int M) {
+        const size_t parts = (size_t)(dw_slabs(N) > 148 ? dw_slabs(N) : 148);  // FFMA slabs or tensor-core CTA partials
+        auto copy = [](int64_t rows, int cols) -> size_t {
+            if (cols % 8 == 0) return 0;
+            const size_t b2 = (size_t)rows * padded(cols, 2) * 2, b4 = cols % 4 == 0 ? 0 : (size_t)rows * padded(cols, 4) * 4;
+            return up256(b2 > b4 ? b2 : b4);
+        };
+        part = 256;
+        x = part + up256(parts * round_up(K, 32) * round_up(M, 32) * 4);
+        dy = x + copy(N, K);
+        w = dy + copy(N, M);
+        bytes = w + (M % 8 == 0 ? 0 : up256((size_t)K * padded(M, 2) * 2));
+    }
+};
+
+// rows on 16 bytes: src itself, or its copy at dst
+static const void* with_padded_rows(const void* src, int64_t rows, int cols, int s, void* dst, cudaStream_t st) {
+    const int ld = padded(cols, s);
+    if (ld == cols) return src;
+    const int chunks = ld * s / 16;
+    const dim3 grid((unsigned)ceil_div(rows * chunks, 256));
+    if (s == 4) launch_overlapped(pad_rows_kernel<float, 4>, grid, dim3(256), 0, st, (const float*)src, rows, cols, (float*)dst, chunks);
+    else launch_overlapped(pad_rows_kernel<uint16_t, 8>, grid, dim3(256), 0, st, (const uint16_t*)src, rows, cols, (uint16_t*)dst, chunks);
+    return dst;
+}
 
 }  // namespace gnn
 
@@ -154,8 +214,7 @@ extern "C" {
 
 size_t gnn_linear_workspace(int32_t N, int K, int M) {
     if (N < 0 || K <= 0 || M <= 0) return 0;
-    const size_t parts = (size_t)(dw_slabs(N) > 148 ? dw_slabs(N) : 148);  // FFMA slabs or tensor-core CTA partials
-    return 256 + up256(parts * K * M * 4);
+    return LinearWs(N, K, M).bytes;
 }
 
 gnn_status gnn_linear(const void* X, const void* W, int32_t N, int K, int M, gnn_dtype dtype, void* Y,
@@ -171,13 +230,28 @@ gnn_status gnn_linear_bias_act(const void* X, const void* W, int32_t N, int K, i
     GNN_REQUIRE(dtype == GNN_F32 || dtype == GNN_BF16, GNN_ERR_INVALID_ARG, "%s: bad dtype", who);
     if (N == 0) return GNN_OK;
     GNN_REQUIRE(X && W && Y, GNN_ERR_INVALID_ARG, "%s: null argument", who);
-    GNN_REQUIRE(ws && ws_bytes >= 256, GNN_ERR_WORKSPACE_TOO_SMALL, "%s: workspace of %zu bytes needed", who, gnn_linear_workspace(N, K, M));
+    const LinearWs lw(N, K, M);
+    GNN_REQUIRE(ws && ws_bytes >= 256, GNN_ERR_WORKSPACE_TOO_SMALL, "%s: workspace of %zu bytes needed", who, lw.bytes);
     cudaStream_t st = as_stream(stream);
+    const int s = elem_size(dtype);
+    char* w8 = (char*)ws;
+    // the status word alone is enough where no rows have to be padded; where they do, a caller with that little gets the
+    // kernels that need no padding
+    const bool pads = K * s % 16 != 0 || (s == 2 && M * s % 16 != 0);
+    if ((!pads || ws_bytes >= lw.bytes) && aligned16(X) && aligned16(W) && aligned16(ws)) {
+        if (linear_tma_supported(N, K, M, 0, dtype)) {
+            const void* Xp = with_padded_rows(X, N, K, s, w8 + lw.x, st);
+            const void* Wp = with_padded_rows(W, K, M, s, w8 + lw.w, st);
+            return linear_tma_forward(Xp, padded(K, s), Wp, padded(M, s), N, K, M, 0, Y, (int*)ws, 1, st, bias, relu);
+        }
+        if (linear_tma_f32_supported(N, K, M, dtype)) {
+            const void* Xp = with_padded_rows(X, N, K, s, w8 + lw.x, st);
+            return linear_tma_f32_forward(Xp, padded(K, s), W, N, K, M, 0, Y, (int*)ws, 1, st, bias, relu);
+        }
+    }
     if (cudaMemsetAsync(ws, 0, sizeof(int), st) != cudaSuccess) GNN_FAIL(GNN_ERR_CUDA, "%s: memset failed (is ws a device pointer?)", who);
-    if (linear_tma_supported(N, K, M, 0, dtype)) return linear_tma_forward(X, W, N, K, M, 0, Y, (int*)ws, st, bias, relu);
-    if (linear_tma_f32_supported(N, K, M, dtype)) return linear_tma_f32_forward(X, W, N, K, M, 0, Y, (int*)ws, st, bias, relu);
-    // fp32 with weights too large for the pipelined kernel runs the single-buffered tensor-core kernel; with a
-    // bias or relu it takes the FFMA kernel instead, whose epilogue applies them before the single rounding
+    // the single-buffered tensor-core kernel has no epilogue: with a bias or relu the FFMA kernel, whose epilogue applies
+    // them before the single rounding
     if (!bias && !relu && linear_tc_supported(N, K, M, dtype)) return linear_tc_forward(X, W, N, K, M, 0, dtype, Y, (int*)ws, st);
     if (dtype == GNN_F32) {
         launch_simt<float, float, float>((const float*)X, K, 1, (const float*)W, M, 1, (float*)Y, N, M, K, K, 1, 0, st, bias, relu);
@@ -196,21 +270,46 @@ gnn_status gnn_linear_backward(const void* X, const void* W, const void* dY, int
     GNN_REQUIRE(N >= 0 && K > 0 && M > 0, GNN_ERR_INVALID_ARG, "%s: bad shape", who);
     GNN_REQUIRE(dtype == GNN_F32 || dtype == GNN_BF16, GNN_ERR_INVALID_ARG, "%s: bad dtype", who);
     GNN_REQUIRE(dY || N == 0, GNN_ERR_INVALID_ARG, "%s: null dY", who);
-    const size_t need = gnn_linear_workspace(N, K, M);
-    GNN_REQUIRE(ws && ws_bytes >= need, GNN_ERR_WORKSPACE_TOO_SMALL, "%s: workspace of %zu bytes needed", who, need);
+    const LinearWs lw(N, K, M);
+    GNN_REQUIRE(ws && ws_bytes >= lw.bytes, GNN_ERR_WORKSPACE_TOO_SMALL, "%s: workspace of %zu bytes needed", who, lw.bytes);
+    GNN_REQUIRE(!dX || N == 0 || W, GNN_ERR_INVALID_ARG, "%s: dX needs W", who);
+    GNN_REQUIRE(!dW || N == 0 || X, GNN_ERR_INVALID_ARG, "%s: dW needs X", who);
     cudaStream_t st = as_stream(stream);
-    if (cudaMemsetAsync(ws, 0, sizeof(int), st) != cudaSuccess) GNN_FAIL(GNN_ERR_CUDA, "%s: memset failed (is ws a device pointer?)", who);
+    const int s = elem_size(dtype);
+    char* w8 = (char*)ws;
+    int* const status = (int*)ws;
+    const bool on16 = aligned16(dY) && aligned16(ws);
+    // dX[n,k] = sum_m dY[n,m] * W[k,m]
+    const bool dx_tma = dX && N > 0 && on16 && aligned16(W) && (dtype == GNN_F32 ? linear_tma_f32_supported(N, M, K, dtype) : linear_tma_supported(N, M, K, 1, dtype));
+    // dW[k,m] = sum_n X[n,k] * dY[n,m]: one fp32 partial per CTA, then summed in CTA order.  More output columns than one
+    // launch takes (256, or fewer where K fills tensor memory): one launch and one ordered sum per block of columns of dY.
+    auto dw_supported = [&](int mc) { return dtype == GNN_F32 ? linear_tma_f32_dw_supported(N, K, mc, dtype) : linear_tma_dw_supported(N, K, mc, dtype); };
+    int block = 0;
+    if (dW && N > 0 && on16 && aligned16(X)) {
+        if (dw_supported(M)) block = M;
+        else
+            for (int mc = (M < 256 ? M : 256) / 32 * 32; mc >= 32 && !block; mc -= 32)
+                if (dw_supported(mc)) block = mc;
+    }
+    int reset = 1;  // the first pipelined launch sets the status word
+    if (!dx_tma && cudaMemsetAsync(ws, 0, sizeof(int), st) != cudaSuccess)
+        GNN_FAIL(GNN_ERR_CUDA, "%s: memset failed (is ws a device pointer?)", who);
+    if (!dx_tma) reset = 0;
+    const void* dYp = dx_tma || block ? with_padded_rows(dY, N, M, s, w8 + lw.dy, st) : dY;
+    const int ldd = padded(M, s);
     if (dX && N > 0) {
-        GNN_REQUIRE(W, GNN_ERR_INVALID_ARG, "%s: dX needs W", who);
-        // dX[n,k] = sum_m dY[n,m] * W[k,m]
-        if (linear_tma_supported(N, M, K, 1, dtype)) {
-            gnn_status rc = linear_tma_forward(dY, W, N, M, K, 1, dX, (int*)ws, st);
+        if (dx_tma) {
+            gnn_status rc;
+            if (dtype == GNN_F32) {
+                rc = linear_tma_f32_forward(dYp, ldd, W, N, M, K, 1, dX, status, reset, st, nullptr, 0);
+            } else {
+                const void* Wp = with_padded_rows(W, K, M, s, w8 + lw.w, st);
+                rc = linear_tma_forward(dYp, ldd, Wp, ldd, N, M, K, 1, dX, status, reset, st, nullptr, 0);
+            }
             if (rc != GNN_OK) return rc;
-        } else if (linear_tma_f32_supported(N, M, K, dtype)) {
-            gnn_status rc = linear_tma_f32_forward(dY, W, N, M, K, 1, dX, (int*)ws, st);
-            if (rc != GNN_OK) return rc;
+            reset = 0;
         } else if (linear_tc_supported(N, M, K, dtype)) {
-            gnn_status rc = linear_tc_forward(dY, W, N, M, K, 1, dtype, dX, (int*)ws, st);
+            gnn_status rc = linear_tc_forward(dY, W, N, M, K, 1, dtype, dX, status, st);
             if (rc != GNN_OK) return rc;
         } else if (dtype == GNN_F32) {
             launch_simt<float, float, float>((const float*)dY, M, 1, (const float*)W, 1, M, (float*)dX, N, K, M, M, 1, 0, st);
@@ -221,52 +320,32 @@ gnn_status gnn_linear_backward(const void* X, const void* W, const void* dY, int
         GNN_CHECK_LAUNCH(who);
     }
     if (dW) {
-        GNN_REQUIRE(X || N == 0, GNN_ERR_INVALID_ARG, "%s: dW needs X", who);
-        // dW[k,m] = sum_n X[n,k] * dY[n,m]: one fp32 partial per slab of rows, then summed in slab order
-        float* part = (float*)((char*)ws + 256);
-        int slabs = dw_slabs(N);
-        const int64_t km = (int64_t)K * M;
-        // more output columns than one pipelined launch takes (256, or fewer where K fills tensor memory): one launch
-        // and one ordered sum per block of columns of dY, each through the same partial buffer
-        int block = 0;
-        if (N > 0 && M > 32) {
-            const int step = dtype == GNN_F32 ? 32 : 16;
-            for (int mc = (M < 256 ? M : 256) / step * step; mc >= step && !block; mc -= step)
-                if (dtype == GNN_F32 ? linear_tma_f32_dw_supported(N, K, mc, dtype) : linear_tma_dw_supported(N, K, mc, dtype)) block = mc;
-        }
-        const bool whole = dtype == GNN_F32 ? linear_tma_f32_dw_supported(N, K, M, dtype) : linear_tma_dw_supported(N, K, M, dtype);
-        if (!whole && block > 0 && M % (dtype == GNN_F32 ? 32 : 16) == 0) {
-            const int s_el = dtype == GNN_F32 ? 4 : 2;
+        float* part = (float*)(w8 + lw.part);
+        auto sum = [&](int slabs, int rows, int cols, int cols_out, int c0) {
+            const int64_t n = (int64_t)rows * cols;
+            const dim3 grid((unsigned)ceil_div(n, 32));
+            if (dtype == GNN_F32) launch_overlapped(slab_sum_kernel<float>, grid, dim3(256), 0, st, part, slabs, n, (float*)dW, cols, K, cols_out, M, c0);
+            else launch_overlapped(slab_sum_kernel<__nv_bfloat16>, grid, dim3(256), 0, st, part, slabs, n, (__nv_bfloat16*)dW, cols, K, cols_out, M, c0);
+        };
+        if (block) {
+            const void* Xp = with_padded_rows(X, N, K, s, w8 + lw.x, st);
             for (int c0 = 0; c0 < M; c0 += block) {
                 const int mc = M - c0 < block ? M - c0 : block;
-                const void* dYb = (const char*)dY + (size_t)c0 * s_el;
-                gnn_status rc;
-                if (dtype == GNN_F32) {
-                    slabs = linear_tma_f32_dw_partials(N);
-                    rc = linear_tma_f32_dw(X, dYb, N, K, mc, M, part, (int*)ws, st);
-                } else {
-                    slabs = linear_tma_dw_partials(N);
-                    rc = linear_tma_dw(X, dYb, N, K, mc, M, part, (int*)ws, st);
-                }
+                const void* dYb = (const char*)dYp + (size_t)c0 * s;
+                gnn_status rc = dtype == GNN_F32 ? linear_tma_f32_dw(Xp, padded(K, s), dYb, ldd, N, K, mc, part, status, reset, st)
+                                                 : linear_tma_dw(Xp, padded(K, s), dYb, ldd, N, K, mc, part, status, reset, st);
                 if (rc != GNN_OK) return rc;
-                const int64_t kmc = (int64_t)K * mc;
-                if (dtype == GNN_F32) slab_sum_kernel<float><<<(int)ceil_div(kmc, 64), 256, 0, st>>>(part, slabs, kmc, (float*)dW, mc, M, c0);
-                else slab_sum_kernel<__nv_bfloat16><<<(int)ceil_div(kmc, 64), 256, 0, st>>>(part, slabs, kmc, (__nv_bfloat16*)dW, mc, M, c0);
+                reset = 0;
+                sum(dtype == GNN_F32 ? linear_tma_f32_dw_partials(N) : linear_tma_dw_partials(N), round_up(K, 32), round_up(mc, dtype == GNN_F32 ? 32 : 16), mc, c0);
                 GNN_CHECK_LAUNCH(who);
             }
             return GNN_OK;
         }
-        if (linear_tma_f32_dw_supported(N, K, M, dtype)) {
-            slabs = linear_tma_f32_dw_partials(N);
-            gnn_status rc = linear_tma_f32_dw(X, dY, N, K, M, M, part, (int*)ws, st);
-            if (rc != GNN_OK) return rc;
-        } else if (linear_tma_dw_supported(N, K, M, dtype)) {
-            slabs = linear_tma_dw_partials(N);
-            gnn_status rc = linear_tma_dw(X, dY, N, K, M, M, part, (int*)ws, st);
-            if (rc != GNN_OK) return rc;
-        } else if (linear_tc_dw_supported(N, K, M, dtype)) {
+        int slabs = dw_slabs(N);
+        const int64_t km = (int64_t)K * M;
+        if (N > 0 && linear_tc_dw_supported(N, K, M, dtype)) {
             slabs = linear_tc_dw_partials(N);
-            gnn_status rc = linear_tc_dw(X, dY, N, K, M, dtype, part, (int*)ws, st);
+            gnn_status rc = linear_tc_dw(X, dY, N, K, M, dtype, part, status, st);
             if (rc != GNN_OK) return rc;
         } else if (N == 0) {
             if (cudaMemsetAsync(part, 0, (size_t)km * 4, st) != cudaSuccess) GNN_FAIL(GNN_ERR_CUDA, "%s: memset failed", who);
@@ -276,8 +355,7 @@ gnn_status gnn_linear_backward(const void* X, const void* W, const void* dY, int
             launch_simt<__nv_bfloat16, __nv_bfloat16, float>((const __nv_bfloat16*)X, 1, K, (const __nv_bfloat16*)dY, M, 1, part, K, M, N,
                                                            dw_slab_rows(N), slabs, km, st);
         }
-        if (dtype == GNN_F32) slab_sum_kernel<float><<<(int)ceil_div(km, 64), 256, 0, st>>>(part, slabs, km, (float*)dW, M, M, 0);
-        else slab_sum_kernel<__nv_bfloat16><<<(int)ceil_div(km, 64), 256, 0, st>>>(part, slabs, km, (__nv_bfloat16*)dW, M, M, 0);
+        sum(slabs, K, M, M, 0);
         GNN_CHECK_LAUNCH(who);
     }
     return GNN_OK;

@@ -53,8 +53,12 @@ struct TmaParams {
     int acc_stride;    // tensor-memory columns between the two accumulators
     int tmem_cols;
     int* status;
-    const float* bias;  // [Mo] added to every output row, or nullptr
+    int reset;          // first launch of a call: set the status word to 0
+    const float* bias;  // [mo] added to every output row, or nullptr
     int relu;           // max(y, 0) after the bias
+    int mo;             // output columns that exist (Kc and Mo are multiples of 16; what lies past the matrices arrives as zeros)
+    __nv_bfloat16* Y;   // rows ldy apart, written directly where they do not start on 16 bytes; nullptr: bulk stores through mapY
+    int64_t ldy;
 };
 
 __global__ void __launch_bounds__(TM_THREADS, 1)
@@ -92,6 +96,8 @@ linear_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_wait_exclusive();
+    if (P.reset && blockIdx.x == 0 && tid == 0) *P.status = 0;
     const uint32_t tmem_base = tmem_base_slot;
     const int64_t ntiles = (P.N + TC_ROWS - 1) / TC_ROWS;
     bool failed = false;
@@ -175,10 +181,13 @@ linear_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
                     tmem_ld_wait();
                     float f[16];
 #pragma unroll
-                    for (int q = 0; q < 16; ++q) {
-                        f[q] = __uint_as_float(r[q]);
-                        if (P.bias) f[q] += __ldg(P.bias + cb * 64 + g * 16 + q);
-                        if (P.relu) f[q] = fmaxf(f[q], 0.f);
+                    for (int q = 0; q < 16; ++q) f[q] = __uint_as_float(r[q]);
+                    if (P.bias || P.relu) {
+#pragma unroll
+                        for (int q = 0; q < 16; ++q) {
+                            if (P.bias && cb * 64 + g * 16 + q < P.mo) f[q] += __ldg(P.bias + cb * 64 + g * 16 + q);
+                            if (P.relu) f[q] = fmaxf(f[q], 0.f);
+                        }
                     }
                     // row = lane, 128 bytes per row; 16-byte chunk c sits at position c ^ (row % 8)
 #pragma unroll
@@ -187,6 +196,24 @@ linear_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
                         const uint32_t dst = stg + (uint32_t)lane * 128u + ((uint32_t)((2 * g + h2) ^ (lane & 7)) << 4);
                         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
                     }
+                }
+                if (P.Y) {  // a row of up to 64 columns per step, two columns per lane
+                    __syncwarp();
+                    const int rows = (int)(P.N - row0 < 32 ? P.N - row0 : 32);
+                    for (int r = 0; r < rows; ++r) {
+                        __nv_bfloat16* yr = P.Y + (row0 + r) * P.ldy + cb * 64;
+#pragma unroll
+                        for (int h2 = 0; h2 < 2; ++h2) {
+                            const int col = lane + 32 * h2;
+                            if (cb * 64 + col < P.mo) {
+                                uint16_t v;
+                                asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(stg + (uint32_t)r * 128u + ((uint32_t)((col >> 3) ^ (r & 7)) << 4) + (uint32_t)(col & 7) * 2u) : "memory");
+                                reinterpret_cast<uint16_t*>(yr)[col] = v;
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    continue;
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
@@ -245,6 +272,8 @@ static bool make_map_ld(CUtensorMap* m, const void* ptr, int64_t rows, int cols,
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+static int up16(int x) { return (x + 15) & ~15; }
+static int up32(int x) { return (x + 31) & ~31; }
 static size_t tma_w_bytes(int Kc, int Mo, int b_transposed) {
     return b_transposed ? (size_t)((Kc + 63) / 64) * Mo * 128 : (size_t)((Mo + 63) / 64) * Kc * 128;
 }
@@ -257,49 +286,55 @@ static int tma_column_block(int Kc, int Mo, int b_transposed) {
     return mc >= 16 ? mc : 0;
 }
 
+// Kc and Mo: any up to 512 and 1024 (inside, rounded up to 16 with zeros from the copy engine)
 bool linear_tma_supported(int64_t N, int Kc, int Mo, int b_transposed, gnn_dtype dtype) {
     if (dtype != GNN_BF16 || N <= 0 || N >= ((int64_t)1 << 31) - TC_ROWS) return false;
-    if (Kc % 16 != 0 || Kc < 16 || Kc > 512 || Mo % 16 != 0 || Mo < 16 || Mo > 1024) return false;
-    if (Kc > 256 && Kc % 32 != 0) return false;  // a weight block taller than 256 rows arrives as two boxes of Kc / 2 rows
-    if (tma_column_block(Kc, Mo, b_transposed) == 0) return false;
+    if (Kc < 1 || Kc > 512 || Mo < 1 || Mo > 1024) return false;
+    if (tma_column_block(up16(Kc), up16(Mo), b_transposed) == 0) return false;
     return encoder() != nullptr;
 }
 
-// More than 256 output columns, or weights too large for shared memory, run as one launch per block of output columns.
-gnn_status linear_tma_forward(const void* X, const void* W, int64_t N, int Kc, int Mo, int b_transposed, void* Y, int* d_flag,
+// X: rows ldx elements apart, W: rows ldw apart, both on 16 bytes.  Y [N,Mo] is contiguous; rows that do not start on 16 bytes
+// are written directly instead of by bulk stores.  More than 256 output columns, or weights too large for shared memory,
+// run as one launch per block of output columns.
+gnn_status linear_tma_forward(const void* X, int ldx, const void* W, int ldw, int64_t N, int Kc, int Mo, int b_transposed, void* Y, int* d_flag, int reset,
                               cudaStream_t st, const float* bias, int relu) {
     const char* who = "gnn_linear (pipelined tensor-core path)";
-    GNN_REQUIRE(aligned16(X) && aligned16(W) && aligned16(Y), GNN_ERR_INVALID_ARG, "%s: matrices must be 16-byte aligned", who);
-    const int block = tma_column_block(Kc, Mo, b_transposed);
+    const bool direct = (size_t)Mo * 2 % 16 != 0;
+    GNN_REQUIRE(aligned16(X) && aligned16(W) && (direct || aligned16(Y)), GNN_ERR_INVALID_ARG, "%s: matrices must be 16-byte aligned", who);
+    const int K16 = up16(Kc), block = tma_column_block(K16, up16(Mo), b_transposed);
     GNN_REQUIRE(block > 0, GNN_ERR_UNSUPPORTED, "%s: weights do not fit shared memory", who);
     CUtensorMap mapX;
-    if (!make_map(&mapX, X, N, Kc, TC_ROWS)) GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
+    if (!make_map_ld(&mapX, X, N, Kc, ldx, TC_ROWS)) GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
     gnn_status rc = allow_big_smem(who, (const void*)linear_tma_kernel, 4, TM_SMEM_MAX);
     if (rc != GNN_OK) return rc;
     const int64_t ntiles = (N + TC_ROWS - 1) / TC_ROWS;
     const __nv_bfloat16* Wb = (const __nv_bfloat16*)W;
     for (int c0 = 0; c0 < Mo; c0 += block) {
-        const int mc = Mo - c0 < block ? Mo - c0 : block;
-        // stored [Kc,Mo]: a block of columns (rows Mo apart); stored [Mo,Kc]: a block of rows
-        const int w_rows = b_transposed ? mc : Kc, w_cols = b_transposed ? Kc : mc;
-        const int box_rows = w_rows > 256 ? w_rows / 2 : w_rows;
+        const int mc = Mo - c0 < block ? Mo - c0 : block, m16 = up16(mc);
+        // stored [Kc,Mo]: a block of columns; stored [Mo,Kc]: a block of rows.  Boxes reach to the rounded sizes.
+        const int w_rows = b_transposed ? mc : Kc, w_cols = b_transposed ? Kc : mc, box_span = b_transposed ? m16 : K16;
+        const int box_rows = box_span > 256 ? box_span / 2 : box_span;
         CUtensorMap mapW, mapY;
-        if (!make_map_ld(&mapW, b_transposed ? Wb + (size_t)c0 * Kc : Wb + c0, w_rows, w_cols, b_transposed ? Kc : Mo, box_rows) ||
-            !make_map_ld(&mapY, (const __nv_bfloat16*)Y + c0, N, mc, Mo, 32))
+        if (!make_map_ld(&mapW, b_transposed ? Wb + (size_t)c0 * ldw : Wb + c0, w_rows, w_cols, ldw, box_rows) ||
+            (!direct && !make_map_ld(&mapY, (const __nv_bfloat16*)Y + c0, N, mc, Mo, 32)))
             GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
+        if (direct) mapY = mapX;  // not used
         TmaParams P;
-        P.N = N; P.Kc = Kc; P.Mo = mc; P.b_transposed = b_transposed; P.w_box_rows = box_rows; P.status = d_flag;
+        P.N = N; P.Kc = K16; P.Mo = m16; P.mo = mc; P.b_transposed = b_transposed; P.w_box_rows = box_rows; P.status = d_flag;
+        P.reset = reset && c0 == 0;
         P.bias = bias ? bias + c0 : nullptr; P.relu = relu;
-        const size_t wbytes = tma_w_bytes(Kc, mc, b_transposed);
+        P.Y = direct ? (__nv_bfloat16*)Y + c0 : nullptr; P.ldy = Mo;
+        const size_t wbytes = tma_w_bytes(K16, m16, b_transposed);
         const size_t fixed = 1024 + wbytes + (size_t)TM_EPI_WARPS * TM_STAGING_BYTES;
         int stages = (int)((TM_SMEM_MAX - fixed) / TM_SLICE_BYTES);
         P.stages = stages > TM_MAX_STAGES ? TM_MAX_STAGES : stages;
-        P.acc_stride = (mc + 31) & ~31;
+        P.acc_stride = (m16 + 31) & ~31;
         int cols = 32;
         while (cols < 2 * P.acc_stride) cols <<= 1;
         P.tmem_cols = cols;
         const size_t smem = fixed + (size_t)P.stages * TM_SLICE_BYTES;
-        linear_tma_kernel<<<(int)(ntiles < 148 ? ntiles : 148), TM_THREADS, smem, st>>>(mapX, mapW, mapY, P);
+        launch_overlapped(linear_tma_kernel, dim3((unsigned)(ntiles < 148 ? ntiles : 148)), dim3(TM_THREADS), smem, st, mapX, mapW, mapY, P);
         GNN_CHECK_LAUNCH(who);
     }
     return GNN_OK;
@@ -363,8 +398,12 @@ struct TmaF32Params {
     int stages;
     int acc_stride, tmem_cols;
     int* status;
-    const float* bias;  // [Mo] added to every output row, or nullptr
+    int reset;          // first launch of a call: set the status word to 0
+    const float* bias;  // [mo] added to every output row, or nullptr
     int relu;           // max(y, 0) after the bias
+    int kc, mo;         // contraction and output columns that exist (Kc and Mo are multiples of 16; the rest is zeros)
+    float* Y;           // rows ldy apart, written directly where they do not start on 16 bytes; nullptr: bulk stores through mapY
+    int64_t ldy;
 };
 
 __global__ void __launch_bounds__(TF_THREADS, 1)
@@ -401,6 +440,8 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapY)) : "memory");
     }
     if (warp == 1) tmem_alloc(smem_u32(&tmem_base_slot), (uint32_t)P.tmem_cols);
+    pdl_wait_exclusive();
+    if (P.reset && blockIdx.x == 0 && tid == 0) *P.status = 0;
     // weight levels.  16-byte chunk c of stored row r:
     //   stored [Kc,Mo] (MN-major B): r = k, c = 8 output columns: offset c*sbo + (k/8)*128 + (k%8)*16
     //   stored [Mo,Kc] (K-major  B): r = n, c = 8 k's:            offset (n/8)*sbo + c*128 + (n%8)*16
@@ -409,9 +450,16 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
         const int rows = P.b_transposed ? Mo : Kc, chunks = (P.b_transposed ? Kc : Mo) / 8;
         for (int e = tid; e < rows * chunks; e += TF_THREADS) {
             const int q = e >> 3, rg = q / chunks, c = q - rg * chunks, r = rg * 8 + (e & 7);
-            const float4* src = reinterpret_cast<const float4*>(P.W + (size_t)r * P.ldw + (size_t)c * 8);
-            const float4 lo = __ldg(src), hi = __ldg(src + 1);
-            const float x[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
+            float x[8];
+            const int have_rows = P.b_transposed ? P.mo : P.kc, have_cols = P.b_transposed ? P.kc : P.mo;
+            const float* srcf = P.W + (size_t)r * P.ldw + (size_t)c * 8;
+            if (P.ldw % 4 == 0 && r < have_rows && c * 8 + 8 <= have_cols) {
+                const float4 lo = __ldg(reinterpret_cast<const float4*>(srcf)), hi = __ldg(reinterpret_cast<const float4*>(srcf) + 1);
+                x[0] = lo.x; x[1] = lo.y; x[2] = lo.z; x[3] = lo.w; x[4] = hi.x; x[5] = hi.y; x[6] = hi.z; x[7] = hi.w;
+            } else {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) x[j] = (r < have_rows && c * 8 + j < have_cols) ? __ldg(srcf + j) : 0.f;
+            }
             uint4 lv[3];
             split8(x, lv);
             const uint32_t off = P.b_transposed ? (uint32_t)(r >> 3) * b_sbo + (uint32_t)c * 128 + (uint32_t)(r & 7) * 16
@@ -528,7 +576,7 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
 #pragma unroll
                         for (int q = 0; q < 16; ++q) {
                             float y = __uint_as_float(r[q]);
-                            if (P.bias) y += __ldg(P.bias + cb * 32 + g16 * 16 + q);
+                            if (P.bias && cb * 32 + g16 * 16 + q < P.mo) y += __ldg(P.bias + cb * 32 + g16 * 16 + q);
                             if (P.relu) y = fmaxf(y, 0.f);
                             r[q] = __float_as_uint(y);
                         }
@@ -538,6 +586,18 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
                     for (int q = 0; q < 4; ++q)
                         st_shared16(stg + (uint32_t)lane * 128u + ((uint32_t)((4 * g16 + q) ^ (lane & 7)) << 4),
                                     make_uint4(r[4 * q], r[4 * q + 1], r[4 * q + 2], r[4 * q + 3]));
+                }
+                if (P.Y) {  // a row of up to 32 columns per step, a column per lane
+                    __syncwarp();
+                    const int rows = (int)(P.N - row0 < 32 ? P.N - row0 : 32);
+                    if (cb * 32 + lane < P.mo)
+                        for (int r = 0; r < rows; ++r) {
+                            float v;
+                            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(stg + (uint32_t)r * 128u + ((uint32_t)((lane >> 2) ^ (r & 7)) << 4) + (uint32_t)(lane & 3) * 4u) : "memory");
+                            P.Y[(row0 + r) * P.ldy + cb * 32 + lane] = v;
+                        }
+                    __syncwarp();
+                    continue;
                 }
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
@@ -578,6 +638,7 @@ struct TmaDwParams {
     int stages;
     int tmem_cols;
     int* status;
+    int reset;  // first launch of a call: set the status word to 0
 };
 
 __global__ void __launch_bounds__(TM_THREADS, 1)
@@ -609,6 +670,8 @@ linear_tma_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_wait_exclusive();
+    if (P.reset && blockIdx.x == 0 && tid == 0) *P.status = 0;
     const uint32_t tmem_base = tmem_base_slot;
     const int64_t nchunks = (P.N + DW_ROWS - 1) / DW_ROWS;  // gridDim.x <= nchunks: every CTA has work
     bool failed = false;
@@ -697,10 +760,11 @@ linear_tma_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_cons
     if (warp == 1) tmem_dealloc(tmem_base, (uint32_t)P.tmem_cols);
 }
 
+// K and M: any (inside, rounded up to 32 and 16 with zeros from the copy engine; that is the shape of the partials)
 bool linear_tma_dw_supported(int64_t N, int K, int M, gnn_dtype dtype) {
     if (dtype != GNN_BF16 || N <= 0 || N >= ((int64_t)1 << 31) - TC_ROWS) return false;
-    if (K % 32 != 0 || K < 32 || K > 512 || M % 16 != 0 || M < 16 || M > 256) return false;
-    if (M * ((K + 127) / 128) > 512) return false;  // one accumulator [128, M] per block of 128 features: 512 columns of tensor memory
+    if (K < 1 || K > 512 || M < 1 || M > 256) return false;
+    if (up16(M) * ((K + 127) / 128) > 512) return false;  // one accumulator [128, M] per block of 128 features: 512 columns of tensor memory
     return encoder() != nullptr;
 }
 
@@ -711,25 +775,26 @@ int linear_tma_dw_partials(int64_t N) {
 
 bool make_map_f32(CUtensorMap* m, const void* ptr, int64_t rows, int cols, int box_rows);
 
-// writes linear_tma_dw_partials(N) fp32 partials [K,M] to part
-gnn_status linear_tma_dw(const void* X, const void* dY, int64_t N, int K, int M, int ldd, float* part, int* d_flag, cudaStream_t st) {
+// writes linear_tma_dw_partials(N) fp32 partials [up32(K), up16(M)] to part; X and dY: rows ldx and ldd elements apart
+gnn_status linear_tma_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, float* part, int* d_flag, int reset, cudaStream_t st) {
     const char* who = "gnn_linear_backward (pipelined tensor-core dW)";
     GNN_REQUIRE(aligned16(X) && aligned16(dY) && aligned16(part), GNN_ERR_INVALID_ARG, "%s: matrices must be 16-byte aligned", who);
+    const int K32 = up32(K), M16 = up16(M);
     CUtensorMap mapX, mapD, mapP;
-    if (!make_map(&mapX, X, N, K, DW_ROWS) || !make_map_ld(&mapD, dY, N, M, ldd, DW_ROWS) ||  // dY may be a block of columns: rows ldd apart
-        !make_map_f32(&mapP, part, (int64_t)linear_tma_dw_partials(N) * K, M, 32))
+    if (!make_map_ld(&mapX, X, N, K, ldx, DW_ROWS) || !make_map_ld(&mapD, dY, N, M, ldd, DW_ROWS) ||
+        !make_map_f32(&mapP, part, (int64_t)linear_tma_dw_partials(N) * K32, M16, 32))
         GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
     TmaDwParams P;
-    P.part = part; P.N = N; P.K = K; P.M = M; P.status = d_flag;
-    const size_t slot = (size_t)(2 * ((K + 127) / 128) + (M + 63) / 64) * DW_BOX_BYTES;
+    P.part = part; P.N = N; P.K = K32; P.M = M16; P.status = d_flag; P.reset = reset;
+    const size_t slot = (size_t)(2 * ((K32 + 127) / 128) + (M16 + 63) / 64) * DW_BOX_BYTES;
     int stages = (int)((TM_SMEM_MAX - 1024) / slot);
     P.stages = stages > TM_MAX_STAGES ? TM_MAX_STAGES : stages;
     int cols = 32;
-    while (cols < M * ((K + 127) / 128)) cols <<= 1;
+    while (cols < M16 * ((K32 + 127) / 128)) cols <<= 1;
     P.tmem_cols = cols;
     gnn_status rc = allow_big_smem(who, (const void*)linear_tma_dw_kernel, 5, TM_SMEM_MAX);
     if (rc != GNN_OK) return rc;
-    linear_tma_dw_kernel<<<linear_tma_dw_partials(N), TM_THREADS, 1024 + (size_t)P.stages * slot, st>>>(mapX, mapD, mapP, P);
+    launch_overlapped(linear_tma_dw_kernel, dim3((unsigned)linear_tma_dw_partials(N)), dim3(TM_THREADS), 1024 + (size_t)P.stages * slot, st, mapX, mapD, mapP, P);
     GNN_CHECK_LAUNCH(who);
     return GNN_OK;
 }
@@ -778,6 +843,7 @@ struct TmaF32DwParams {
     int stages;
     int tmem_cols;
     int* status;
+    int reset;  // first launch of a call: set the status word to 0
 };
 
 __global__ void __launch_bounds__(FD_THREADS, 1)
@@ -821,6 +887,8 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
+    pdl_wait_exclusive();
+    if (P.reset && blockIdx.x == 0 && tid == 0) *P.status = 0;
     const uint32_t tmem_base = tmem_base_slot;
     const int64_t nslots = (P.N + FD_ROWS - 1) / FD_ROWS;
     bool failed = false;
@@ -930,10 +998,11 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
     if (warp == 1) tmem_dealloc(tmem_base, (uint32_t)P.tmem_cols);
 }
 
+// K and M: any (inside, rounded up to 32 with zeros from the copy engine; that is the shape of the partials)
 bool linear_tma_f32_dw_supported(int64_t N, int K, int M, gnn_dtype dtype) {
     if (dtype != GNN_F32 || N <= 0 || N >= ((int64_t)1 << 31) - FD_ROWS_MAX) return false;
-    if (K % 32 != 0 || K < 32 || K > 512 || M % 32 != 0 || M < 32 || M > 256) return false;
-    if (M * ((K + 127) / 128) > 512) return false;  // one accumulator [128, M] per block of 128 features: 512 columns of tensor memory
+    if (K < 1 || K > 512 || M < 1 || M > 256) return false;
+    if (up32(M) * ((K + 127) / 128) > 512) return false;  // one accumulator [128, M] per block of 128 features: 512 columns of tensor memory
     return encoder() != nullptr;
 }
 
@@ -944,15 +1013,16 @@ int linear_tma_f32_dw_partials(int64_t N) {
     return (int)(nslots < 148 ? (nslots > 0 ? nslots : 1) : 148);
 }
 
-// writes linear_tma_f32_dw_partials(N) fp32 partials [K,M] to part
-gnn_status linear_tma_f32_dw(const void* X, const void* dY, int64_t N, int K, int M, int ldd, float* part, int* d_flag, cudaStream_t st) {
+// writes linear_tma_f32_dw_partials(N) fp32 partials [up32(K), up32(M)] to part; X and dY: rows ldx and ldd elements apart
+gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int Kr, int Mr, float* part, int* d_flag, int reset, cudaStream_t st) {
     const char* who = "gnn_linear_backward (pipelined fp32 tensor-core dW)";
     GNN_REQUIRE(aligned16(X) && aligned16(dY) && aligned16(part), GNN_ERR_INVALID_ARG, "%s: matrices must be 16-byte aligned", who);
+    const int K = up32(Kr), M = up32(Mr);
     CUtensorMap mapX, mapD;
     const int R = fd_rows(K, M), ka = (K + 127) / 128 * 128;
-    if (!make_map_f32(&mapX, X, N, K, R) || !make_map_f32_ld(&mapD, dY, N, M, ldd, R)) GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
+    if (!make_map_f32_ld(&mapX, X, N, Kr, ldx, R) || !make_map_f32_ld(&mapD, dY, N, Mr, ldd, R)) GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
     TmaF32DwParams P;
-    P.part = part; P.N = N; P.K = K; P.M = M; P.status = d_flag; P.rows = R;
+    P.part = part; P.N = N; P.K = K; P.M = M; P.status = d_flag; P.reset = reset; P.rows = R;
     const size_t slot = (size_t)(K / 32 + M / 32) * R * 128, ops = 2 * 3 * ((size_t)ka * R * 2 + (size_t)M * R * 2);
     int stages = (int)((TM_SMEM_MAX - 1024 - ops) / slot);
     P.stages = stages > FD_MAX_STAGES ? FD_MAX_STAGES : stages;
@@ -961,7 +1031,7 @@ gnn_status linear_tma_f32_dw(const void* X, const void* dY, int64_t N, int K, in
     P.tmem_cols = cols;
     gnn_status rc = allow_big_smem(who, (const void*)linear_tma_f32_dw_kernel, 12, TM_SMEM_MAX);
     if (rc != GNN_OK) return rc;
-    linear_tma_f32_dw_kernel<<<linear_tma_f32_dw_partials(N), FD_THREADS, 1024 + ops + (size_t)P.stages * slot, st>>>(mapX, mapD, P);
+    launch_overlapped(linear_tma_f32_dw_kernel, dim3((unsigned)linear_tma_f32_dw_partials(N)), dim3(FD_THREADS), 1024 + ops + (size_t)P.stages * slot, st, mapX, mapD, P);
     GNN_CHECK_LAUNCH(who);
     return GNN_OK;
 }
@@ -977,44 +1047,50 @@ static int tf_column_block(int Kc, int Mo) {
     return mc >= 16 ? mc : 0;
 }
 
+// Kc and Mo: any up to 512 and 1024 (inside, rounded up to 16 with zeros)
 bool linear_tma_f32_supported(int64_t N, int Kc, int Mo, gnn_dtype dtype) {
     if (dtype != GNN_F32 || N <= 0 || N >= ((int64_t)1 << 31) - TC_ROWS) return false;
-    if (Kc % 16 != 0 || Kc < 16 || Kc > 512 || Mo % 16 != 0 || Mo < 16 || Mo > 1024) return false;
-    if (tf_column_block(Kc, Mo) == 0) return false;
+    if (Kc < 1 || Kc > 512 || Mo < 1 || Mo > 1024) return false;
+    if (tf_column_block(up16(Kc), up16(Mo)) == 0) return false;
     return encoder() != nullptr;
 }
 
-// Weights too large for shared memory in one piece (3 x Kc x Mo x 2 bytes: 256 x 256, 256 x 128, 192 x 192 ...) run as
-// one launch per block of output columns: X is read once per block, which is still an order of magnitude faster than
-// the FFMA kernel these shapes fell to before.
-gnn_status linear_tma_f32_forward(const void* X, const void* W, int64_t N, int Kc, int Mo, int b_transposed, void* Y, int* d_flag,
+// X: rows ldx elements apart, on 16 bytes; Y [N,Mo] contiguous (rows that do not start on 16 bytes are written directly
+// instead of by bulk stores).  Weights too large for shared memory in one piece (3 x Kc x Mo x 2 bytes: 256 x 256,
+// 256 x 128, 192 x 192 ...) run as one launch per block of output columns: X is read once per block, which is still an
+// order of magnitude faster than the FFMA kernel these shapes fell to before.
+gnn_status linear_tma_f32_forward(const void* X, int ldx, const void* W, int64_t N, int Kc, int Mo, int b_transposed, void* Y, int* d_flag, int reset,
                                   cudaStream_t st, const float* bias, int relu) {
     const char* who = "gnn_linear (pipelined fp32 tensor-core path)";
-    GNN_REQUIRE(aligned16(X) && aligned16(W) && aligned16(Y), GNN_ERR_INVALID_ARG, "%s: matrices must be 16-byte aligned", who);
-    const int block = tf_column_block(Kc, Mo);
+    const bool direct = Mo % 4 != 0;
+    GNN_REQUIRE(aligned16(X) && aligned16(W) && (direct || aligned16(Y)), GNN_ERR_INVALID_ARG, "%s: matrices must be 16-byte aligned", who);
+    const int K16 = up16(Kc), block = tf_column_block(K16, up16(Mo));
     GNN_REQUIRE(block > 0, GNN_ERR_UNSUPPORTED, "%s: weights do not fit shared memory", who);
     CUtensorMap mapX;
-    if (!make_map_f32(&mapX, X, N, Kc, TC_ROWS)) GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
+    if (!make_map_f32_ld(&mapX, X, N, Kc, ldx, TC_ROWS)) GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
     gnn_status rc = allow_big_smem(who, (const void*)linear_tma_f32_kernel, 6, TM_SMEM_MAX);
     if (rc != GNN_OK) return rc;
     const int64_t ntiles = (N + TC_ROWS - 1) / TC_ROWS;
     for (int c0 = 0; c0 < Mo; c0 += block) {
-        const int mc = Mo - c0 < block ? Mo - c0 : block;
+        const int mc = Mo - c0 < block ? Mo - c0 : block, m16 = up16(mc);
         CUtensorMap mapY;
-        if (!make_map_f32_ld(&mapY, (const float*)Y + c0, N, mc, Mo, 32)) GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
+        if (direct) mapY = mapX;  // not used
+        else if (!make_map_f32_ld(&mapY, (const float*)Y + c0, N, mc, Mo, 32)) GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
         TmaF32Params P;
         // stored [Kc,Mo]: a block of columns starts c0 elements into every row; stored [Mo,Kc]: a block of rows
         P.W = b_transposed ? (const float*)W + (size_t)c0 * Kc : (const float*)W + c0;
         P.ldw = b_transposed ? Kc : Mo;
-        P.N = N; P.Kc = Kc; P.Mo = mc; P.b_transposed = b_transposed; P.status = d_flag; P.bias = bias ? bias + c0 : nullptr; P.relu = relu;
-        const size_t fixed = tf_fixed_bytes(Kc, mc);
+        P.N = N; P.Kc = K16; P.Mo = m16; P.kc = Kc; P.mo = mc; P.b_transposed = b_transposed; P.status = d_flag; P.reset = reset && c0 == 0;
+        P.bias = bias ? bias + c0 : nullptr; P.relu = relu;
+        P.Y = direct ? (float*)Y + c0 : nullptr; P.ldy = Mo;
+        const size_t fixed = tf_fixed_bytes(K16, m16);
         int stages = (int)((TM_SMEM_MAX - fixed) / TF_SLICE_BYTES);
         P.stages = stages > TF_MAX_STAGES ? TF_MAX_STAGES : stages;
-        P.acc_stride = (mc + 31) & ~31;
+        P.acc_stride = (m16 + 31) & ~31;
         int cols = 32;
         while (cols < 2 * P.acc_stride) cols <<= 1;
         P.tmem_cols = cols;
-        linear_tma_f32_kernel<<<(int)(ntiles < 148 ? ntiles : 148), TF_THREADS, fixed + (size_t)P.stages * TF_SLICE_BYTES, st>>>(mapX, mapY, P);
+        launch_overlapped(linear_tma_f32_kernel, dim3((unsigned)(ntiles < 148 ? ntiles : 148)), dim3(TF_THREADS), fixed + (size_t)P.stages * TF_SLICE_BYTES, st, mapX, mapY, P);
         GNN_CHECK_LAUNCH(who);
     }
     return GNN_OK;

@@ -16,6 +16,7 @@ gnn_status sddmm_heads(const char* who, const gnn_csr* g, const void* X, const v
 template <typename T>
 __global__ void row_scale_kernel(const int64_t* __restrict__ rowptr, int32_t N, int nvec, int times_degree,
                                  const uint4* __restrict__ D, uint4* __restrict__ out) {
+    pdl_wait();
     constexpr int EPC = Chunk<T>::N;
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x, total = (int64_t)N * nvec;
@@ -36,6 +37,7 @@ template <typename T>
 __global__ void edge_factor_grad_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int32_t N,
                                         int64_t E, int nvec, int mean, const uint4* __restrict__ X,
                                         const uint4* __restrict__ D, float* __restrict__ de) {
+    pdl_wait();
     constexpr int EPC = Chunk<T>::N;
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x, total = E * nvec;
@@ -60,6 +62,7 @@ constexpr int DOT_THREADS = 256, DOT_MAX_BLOCKS = 1184;
 template <typename T>
 __global__ void __launch_bounds__(DOT_THREADS) dot_partial_kernel(const uint4* __restrict__ a, const uint4* __restrict__ b,
                                                                   int64_t nvec, float* __restrict__ partial) {
+    pdl_wait();
     constexpr int EPC = Chunk<T>::N;
     __shared__ float s_w[DOT_THREADS / 32];
     float acc = 0.f;
@@ -83,12 +86,15 @@ __global__ void __launch_bounds__(DOT_THREADS) dot_partial_kernel(const uint4* _
         partial[blockIdx.x] = s;
     }
 }
+// the partials' sum in a fixed order: a lane takes every 32nd, the lanes are added by an xor tree
 __global__ void dot_final_kernel(const float* __restrict__ partial, int nb, float* __restrict__ out) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        float s = 0.f;
-        for (int b = 0; b < nb; ++b) s += partial[b];
-        *out = s;
-    }
+    pdl_wait();
+    float s = 0.f;
+#pragma unroll 4
+    for (int b = threadIdx.x; b < nb; b += 32) s += partial[b];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) *out = s;
 }
 
 // dZ = dY where (!relu or Y > 0) else 0, and per-block column sums of dZ.  A block owns a contiguous
@@ -98,6 +104,7 @@ template <typename T>
 __global__ void __launch_bounds__(EB_THREADS) epilogue_backward_kernel(const uint4* __restrict__ Y, const uint4* __restrict__ dY,
                                                                       int32_t N, int nvec, int relu, uint4* __restrict__ dZ,
                                                                       float* __restrict__ partial, int rows_per_block) {
+    pdl_wait();
     constexpr int EPC = Chunk<T>::N;
     extern __shared__ float s_acc[];  // [groups][nvec * EPC]
     const int groups = EB_THREADS / nvec;
@@ -109,6 +116,7 @@ __global__ void __launch_bounds__(EB_THREADS) epilogue_backward_kernel(const uin
 #pragma unroll
     for (int j = 0; j < EPC; ++j) acc[j] = 0.f;
     if (active) {
+#pragma unroll 4
         for (int64_t r = r0 + grp; r < r1; r += groups) {
             float d[EPC];
             Chunk<T>::unpack(dY[(size_t)r * nvec + ci], d);
@@ -138,18 +146,31 @@ __global__ void __launch_bounds__(EB_THREADS) epilogue_backward_kernel(const uin
         }
     }
 }
-__global__ void column_sum_final_kernel(const float* __restrict__ partial, int nb, int F, float* __restrict__ out) {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= F) return;
+// out[f] = sum of the nb partials of column f: 8 walkers per column take every eighth partial, four loads in flight each, and
+// are added in walker order (one thread per column walking them all took 14 us for 400 partials)
+constexpr int CS_WALKERS = 8;
+__global__ void __launch_bounds__(32 * CS_WALKERS) column_sum_final_kernel(const float* __restrict__ partial, int nb, int F, float* __restrict__ out) {
+    pdl_wait();
+    __shared__ float sums[CS_WALKERS][32];
+    const int col = threadIdx.x & 31, w = threadIdx.x >> 5, f = blockIdx.x * 32 + col;
     float s = 0.f;
-    for (int b = 0; b < nb; ++b) s += partial[(size_t)b * F + f];
-    out[f] = s;
+    if (f < F)
+#pragma unroll 4
+        for (int b = w; b < nb; b += CS_WALKERS) s += partial[(size_t)b * F + f];
+    sums[w][col] = s;
+    __syncthreads();
+    if (w == 0 && f < F) {
+#pragma unroll
+        for (int k = 1; k < CS_WALKERS; ++k) s += sums[k][col];
+        out[f] = s;
+    }
 }
 
 // merged edge list of one segment: ids shifted by the segment's offsets
 __global__ void merge_segment_kernel(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t E,
                                      int32_t so, int32_t dof, int32_t seg, int32_t* __restrict__ src_out,
                                      int32_t* __restrict__ dst_out, int32_t* __restrict__ seg_out) {
+    pdl_wait();
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (; t < E; t += stride) {
@@ -164,6 +185,7 @@ __global__ void merge_segment_kernel(const int32_t* __restrict__ src, const int3
 __global__ void segment_coef_kernel(const int64_t* __restrict__ rowptr, int32_t N, int64_t E, const int32_t* __restrict__ seg,
                                     const float* __restrict__ w, const int32_t* __restrict__ seg_is_mean, int S,
                                     float* __restrict__ coef, int* __restrict__ flag) {
+    pdl_wait();
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (; p < E; p += stride) {
@@ -302,8 +324,8 @@ gnn_status gnn_propagate_msg_backward(const gnn_csr* g, gnn_msg msg, gnn_op op, 
         GNN_REQUIRE(aligned16(dOut) && aligned16(dXi), GNN_ERR_INVALID_ARG, "%s: misaligned matrix", who);
         if (g->N > 0) {
             const int grid = grid_for((int64_t)g->N * nvec, 256);
-            if (dtype == GNN_F32) row_scale_kernel<float><<<grid, 256, 0, st>>>(g->rowptr, g->N, nvec, op == GNN_SUM, (const uint4*)dOut, (uint4*)dXi);
-            else row_scale_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(g->rowptr, g->N, nvec, op == GNN_SUM, (const uint4*)dOut, (uint4*)dXi);
+            if (dtype == GNN_F32) launch_overlapped(row_scale_kernel<float>, dim3((unsigned)(grid)), dim3(256), 0, st, g->rowptr, g->N, nvec, op == GNN_SUM, (const uint4*)dOut, (uint4*)dXi);
+            else launch_overlapped(row_scale_kernel<__nv_bfloat16>, dim3((unsigned)(grid)), dim3(256), 0, st, g->rowptr, g->N, nvec, op == GNN_SUM, (const uint4*)dOut, (uint4*)dXi);
             GNN_CHECK_LAUNCH(who);
         }
     }
@@ -315,9 +337,9 @@ gnn_status gnn_propagate_msg_backward(const gnn_csr* g, gnn_msg msg, gnn_op op, 
             if (g->E > 0) {
                 const int grid = grid_for(g->E * nvec, 256);
                 if (dtype == GNN_F32)
-                    edge_factor_grad_kernel<float><<<grid, 256, 0, st>>>(g->rowptr, g->col, g->N, g->E, nvec, op == GNN_MEAN, (const uint4*)Xj, (const uint4*)dOut, de_csr);
+                    launch_overlapped(edge_factor_grad_kernel<float>, dim3((unsigned)(grid)), dim3(256), 0, st, g->rowptr, g->col, g->N, g->E, nvec, op == GNN_MEAN, (const uint4*)Xj, (const uint4*)dOut, de_csr);
                 else
-                    edge_factor_grad_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>(g->rowptr, g->col, g->N, g->E, nvec, op == GNN_MEAN, (const uint4*)Xj, (const uint4*)dOut, de_csr);
+                    launch_overlapped(edge_factor_grad_kernel<__nv_bfloat16>, dim3((unsigned)(grid)), dim3(256), 0, st, g->rowptr, g->col, g->N, g->E, nvec, op == GNN_MEAN, (const uint4*)Xj, (const uint4*)dOut, de_csr);
                 GNN_CHECK_LAUNCH(who);
             }
         } else if (e_width == 1) {
@@ -348,7 +370,9 @@ gnn_status gnn_row_epilogue_backward(const void* Y, const void* dY, int32_t N, i
     GNN_REQUIRE(aligned16(dY) && aligned16(Y) && aligned16(dZ), GNN_ERR_INVALID_ARG, "%s: misaligned matrix", who);
     const int nvec = F * s / 16;
     cudaStream_t st = as_stream(stream);
-    const int rows_per_block = (int)ceil_div(N > 0 ? N : 1, EB_MAX_BLOCKS);
+    // at least four rows per thread, so that a small graph does not leave hundreds of partials of one or two rows
+    const int least = 4 * (EB_THREADS / nvec > 0 ? EB_THREADS / nvec : 1);
+    const int spread = (int)ceil_div(N > 0 ? N : 1, EB_MAX_BLOCKS), rows_per_block = spread > least ? spread : least;
     const int nb = N > 0 ? (int)ceil_div(N, rows_per_block) : 0;
     float* partial = nullptr;
     if (dbias) {
@@ -359,13 +383,13 @@ gnn_status gnn_row_epilogue_backward(const void* Y, const void* dY, int32_t N, i
     if (nb > 0) {
         const size_t smem = (size_t)(EB_THREADS / nvec) * nvec * (16 / s) * 4;
         if (dtype == GNN_F32)
-            epilogue_backward_kernel<float><<<nb, EB_THREADS, smem, st>>>((const uint4*)Y, (const uint4*)dY, N, nvec, relu, (uint4*)dZ, partial, rows_per_block);
+            launch_overlapped(epilogue_backward_kernel<float>, dim3((unsigned)(nb)), dim3(EB_THREADS), smem, st, (const uint4*)Y, (const uint4*)dY, N, nvec, relu, (uint4*)dZ, partial, rows_per_block);
         else
-            epilogue_backward_kernel<__nv_bfloat16><<<nb, EB_THREADS, smem, st>>>((const uint4*)Y, (const uint4*)dY, N, nvec, relu, (uint4*)dZ, partial, rows_per_block);
+            launch_overlapped(epilogue_backward_kernel<__nv_bfloat16>, dim3((unsigned)(nb)), dim3(EB_THREADS), smem, st, (const uint4*)Y, (const uint4*)dY, N, nvec, relu, (uint4*)dZ, partial, rows_per_block);
         GNN_CHECK_LAUNCH(who);
     }
     if (dbias) {
-        column_sum_final_kernel<<<(int)ceil_div(F, 128), 128, 0, st>>>(partial, nb, F, dbias);
+        launch_overlapped(column_sum_final_kernel, dim3((unsigned)ceil_div(F, 32)), dim3(32 * CS_WALKERS), 0, st, partial, nb, F, dbias);
         GNN_CHECK_LAUNCH(who);
     }
     return GNN_OK;
@@ -406,10 +430,10 @@ gnn_status gnn_gin_backward(const gnn_csr* g, const void* dOut, const void* X, f
         const int nb = (int)(nvec > 0 ? (ceil_div(nvec, DOT_THREADS) < DOT_MAX_BLOCKS ? ceil_div(nvec, DOT_THREADS) : DOT_MAX_BLOCKS) : 0);
         cudaStream_t st = as_stream(stream);
         if (nb > 0) {
-            if (dtype == GNN_F32) dot_partial_kernel<float><<<nb, DOT_THREADS, 0, st>>>((const uint4*)dOut, (const uint4*)X, nvec, partial);
-            else dot_partial_kernel<__nv_bfloat16><<<nb, DOT_THREADS, 0, st>>>((const uint4*)dOut, (const uint4*)X, nvec, partial);
+            if (dtype == GNN_F32) launch_overlapped(dot_partial_kernel<float>, dim3((unsigned)(nb)), dim3(DOT_THREADS), 0, st, (const uint4*)dOut, (const uint4*)X, nvec, partial);
+            else launch_overlapped(dot_partial_kernel<__nv_bfloat16>, dim3((unsigned)(nb)), dim3(DOT_THREADS), 0, st, (const uint4*)dOut, (const uint4*)X, nvec, partial);
         }
-        dot_final_kernel<<<1, 32, 0, st>>>(partial, nb, deps);
+        launch_overlapped(dot_final_kernel, dim3((unsigned)(1)), dim3(32), 0, st, partial, nb, deps);
         GNN_CHECK_LAUNCH(who);
     }
     return GNN_OK;
@@ -492,7 +516,7 @@ gnn_status gnn_merge_edge_lists(const gnn_edge_segment* segs, int S, int32_t* sr
     int64_t base = 0;
     for (int k = 0; k < S; ++k) {
         if (segs[k].E == 0) continue;
-        merge_segment_kernel<<<grid_for(segs[k].E, 256), 256, 0, st>>>(segs[k].src, segs[k].dst, segs[k].E, segs[k].src_offset,
+        launch_overlapped(merge_segment_kernel, dim3((unsigned)(grid_for(segs[k].E, 256))), dim3(256), 0, st, segs[k].src, segs[k].dst, segs[k].E, segs[k].src_offset,
                                                                         segs[k].dst_offset, k, src_out + base, dst_out + base,
                                                                         seg_out ? seg_out + base : nullptr);
         base += segs[k].E;
@@ -512,7 +536,7 @@ gnn_status gnn_segment_coef(const gnn_csr* g, const int32_t* seg_csr, const floa
     cudaStream_t st = as_stream(stream);
     // an out-of-range segment id leaves its factor unscaled and is reported through the last word of coef_csrT's
     // pass below only if asked for; the ids come from gnn_merge_edge_lists, so this is a guard, not a path
-    segment_coef_kernel<<<grid_for(g->E, 256), 256, 0, st>>>(g->rowptr, g->N, g->E, seg_csr, w_csr, seg_is_mean, S, coef_csr, nullptr);
+    launch_overlapped(segment_coef_kernel, dim3((unsigned)(grid_for(g->E, 256))), dim3(256), 0, st, g->rowptr, g->N, g->E, seg_csr, w_csr, seg_is_mean, S, coef_csr, nullptr);
     GNN_CHECK_LAUNCH(who);
     if (coef_csrT) {
         GNN_REQUIRE(g->t2f, GNN_ERR_INVALID_ARG, "%s: coef_csrT needs t2f", who);

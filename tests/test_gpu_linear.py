@@ -72,6 +72,42 @@ def test_linear_forward_backward(gnn, dtype, n, K, M):
         oracle.set_threads(1)
 
 
+# Sizes that divide nothing: rows that start off 16 bytes (padded copies of X, dY and W, directly written Y and dX), rows on 16
+# bytes but off the 16- and 32-element steps of the MMA, one column, one row, the 512-wide contraction, column blocks of dW
+RAGGED = [("f32", 700, 100, 47), ("f32", 1, 33, 2), ("f32", 129, 511, 255), ("f32", 300, 20, 36), ("f32", 4097, 37, 130), ("f32", 260, 500, 250),
+          ("bf16", 700, 100, 47), ("bf16", 1, 17, 3), ("bf16", 129, 511, 255), ("bf16", 300, 24, 40), ("bf16", 4097, 37, 130), ("bf16", 515, 272, 8),
+          ("bf16", 64, 1, 1), ("f32", 64, 1, 1)]
+
+
+@pytest.mark.parametrize("dtype,n,K,M", RAGGED)
+def test_linear_ragged_sizes(gnn, dtype, n, K, M):
+    import torch
+    oracle.set_threads(8)
+    try:
+        X, dY = synth.normal((n, K), dtype, 1300 + K), synth.normal((n, M), dtype, 1301 + M)
+        W = synth.normal((K, M), dtype, 1302)
+        b = synth.uniform_f32((M,), -1.0, 1.0, 1303)
+        Xd, Wd, dYd = to_dev(X), to_dev(W), to_dev(dY)
+        Yo, S = oracle.matmul(X, W)
+        Y, ws = gnn.linear(Xd, Wd, return_ws=True)
+        assert status_word(ws) == 0
+        assert_close(to_host64(Y), Yo, S, dtype, "Y")
+        # bias and relu in the epilogue: |b| joins the terms, relu is 1-Lipschitz
+        Z = gnn.linear_bias_act(Xd, Wd, to_dev(b), relu=True)
+        assert_close(to_host64(Z), np.maximum(Yo + b, 0.0), S + np.abs(b), dtype, "relu(Y + b)")
+        # the bytes of the status word alone are enough workspace for the forward call, whatever the shape
+        small = gnn.linear(Xd, Wd, ws=torch.empty(256, dtype=torch.uint8, device="cuda"))
+        assert_close(to_host64(small), Yo, S, dtype, "Y with 256 bytes of workspace")
+        dX, dW, ws = gnn.linear_backward(Xd, Wd, dYd, return_ws=True)
+        assert status_word(ws) == 0
+        dXo, S = oracle.matmul(dY, W, tb=True)
+        assert_close(to_host64(dX), dXo, S, dtype, "dX")
+        dWo, S = oracle.matmul(X, dY, ta=True)
+        assert_close(to_host64(dW), dWo, S, dtype, "dW")
+    finally:
+        oracle.set_threads(1)
+
+
 def test_linear_large_rows_tensor_core(gnn):
     """N = 100000 rows, 256 -> 256 bf16 (the attention workload's transform): many tiles per CTA."""
     import torch
