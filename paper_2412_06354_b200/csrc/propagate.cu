@@ -339,28 +339,26 @@ static ReduceWs carve(void* ws, int64_t pieces, int F, bool with_arg) {
 }
 
 
-// Positions per piece (see reduce_rows.cuh): a function of the shape alone, so that results are reproducible.
-//  - From 4 Mi positions on 256, the most a warp stages.  Below that a piece of 256 leaves the machine with one wave of
-//    warps and a nearly empty second: rows over 128 bytes then take 128 (1.36 M edges, 512-byte rows: 82 -> 75 us), narrower
-//    ones below 1 M (557k edges, 128-byte rows: 26 -> 18 us; above, the set-up of twice as many pieces costs more than it
-//    gives).  Where the mean row spans pieces (pooling over a few large graphs), 256: every cut is one more partial row.
-//  - Small graphs are bound by the longest chain of loads of a warp, so their pieces shrink with them (80k edges with hubs,
-//    512-byte rows: 15.8 us at 64, 11.8 us at 32), as long as the partial rows stay within SMALL_WS.
-constexpr size_t SMALL_WS = (size_t)8 << 20;
-static int piece_positions(int32_t N, int64_t E, int F, int row_bytes, bool with_arg) {
+// Positions per warp (see reduce_rows.cuh): a function of the shape alone, so that results are reproducible.
+//  - From 2.5 M positions on 256, the most a warp stages.  Below that 256 leaves the machine with one wave of warps and a
+//    nearly empty second: rows over 128 bytes then take 128 (1.36 M edges, 512-byte rows: 82 -> 75 us), narrower ones below
+//    1 M (557k edges, 128-byte rows: 26 -> 18 us; above, the set-up of twice as many warps costs more than it gives).
+//  - Where the mean row spans several pieces (pooling over a few large graphs), 256: every cut is one more partial row.
+//  - Small graphs are bound by the longest chain of loads of a warp, so their shares shrink with them (80k edges with hubs,
+//    512-byte rows: 15.8 us at 64, 11.8 us at 32; 64-byte rows have eight groups per warp and gain nothing below 64).
+static int warp_positions(int32_t N, int64_t E, int row_bytes, bool stream) {
     if (E >= (int64_t)4 * 1024 * 1024) return 256;
     if (E >= 512 * 1024) return E > 64 * (int64_t)N || E >= 2500 * 1000 || (row_bytes <= 128 && E >= 1000 * 1000) ? 256 : 128;
-    const int coarse = E >= 128 * 1024 ? 128 : 64, fine = E >= 256 * 1024 ? 128 : E >= 128 * 1024 || row_bytes <= 64 ? 64 : 32;
-    return carve(nullptr, ceil_div(E, (int64_t)fine), F < 256 ? F : 256, with_arg).bytes <= SMALL_WS ? fine : coarse;
+    if (!stream) return 64;
+    return E >= 256 * 1024 ? 128 : E >= 128 * 1024 || row_bytes <= 64 ? 64 : 32;
 }
 
+// Room for a partial row per 64 to 256 positions.  The streaming kernel needs an eighth of that; the size is what callers
+// have been told since the first version, and what decides which problems the built-in scratch takes.
 size_t chunked_workspace(int64_t E, int F, bool with_arg) {
     if (E <= 0) return carve(nullptr, 1, F, with_arg).bytes;
-    auto bytes = [&](bool arg) {  // rows over 512 bytes are reduced in slabs of at most 256 features
-        return carve(nullptr, ceil_div(E, (int64_t)piece_positions(INT32_MAX, E, F, 512, arg)), F < 256 ? F : 256, arg).bytes;
-    };
-    // the backward pass of max / min needs no winners but may take finer pieces
-    return with_arg && bytes(false) > bytes(true) ? bytes(false) : bytes(with_arg);
+    const int per = E >= (int64_t)4 * 1024 * 1024 ? 1024 : E >= 512 * 1024 ? 128 : 64;
+    return carve(nullptr, ceil_div(E, (int64_t)per), F < 256 ? F : 256, with_arg).bytes;
 }
 
 gnn_status run_chunked(const char* who, int mode, int32_t N, int64_t E, const int64_t* rowptr,
@@ -414,15 +412,17 @@ gnn_status run_chunked(const char* who, int mode, int32_t N, int64_t E, const in
     // Rows over 512 bytes run one 512-byte column slab at a time: every pass re-reads the index stream but gathers from a
     // narrower matrix, of which more rows stay in L2 (2048-byte fp32 rows on 123 M edges: 141 -> 77 GB of DRAM traffic).
     const int slab_vec = nvec < 32 ? nvec : 32, slab_f = slab_vec * epc;
-    P.piece = piece_positions(N, E, F, nvec * 16, with_arg);
-    P.npieces = E > 0 ? ceil_div(E, (int64_t)P.piece) : 1;
-    const ReduceWs wsv = carve(ws, P.npieces, slab_f, with_arg);
-    P.tail_row = wsv.tail_row; P.part_val = wsv.part_val; P.part_arg = wsv.part_arg;
     // Graphs of up to 128 Ki edges and a handful per row are bound by latency and take a row per lane group (13k nodes,
     // 69k edges, 512-byte rows: 8.7 us against 11.6 us positions first); higher mean degrees say that long rows carry the
     // edges (10k nodes, 80k edges with hubs: 13.4 against 11.8 us).
     // The routing mode fetches two rows per position and has fewer in flight per lane: always positions first (17 / 14 us).
     const bool stream = E >= 128 * 1024 || E > 6 * (int64_t)N || (mode == MODE_ROUTE && E > 0);
+    P.sub = warp_positions(N, E, nvec * 16, stream);
+    P.piece = stream ? P.sub * RR_WARPS : P.sub;
+    P.npieces = E > 0 ? ceil_div(E, (int64_t)P.piece) : 1;
+    const ReduceWs wsv = carve(ws, P.npieces, slab_f, with_arg);
+    GNN_REQUIRE(wsv.bytes <= ws_bytes, GNN_ERR_WORKSPACE_TOO_SMALL, "%s: partial rows of %zu bytes exceed the workspace", who, wsv.bytes);
+    P.tail_row = wsv.tail_row; P.part_val = wsv.part_val; P.part_arg = wsv.part_arg;
     for (int v0 = 0; v0 < nvec; v0 += 32) {
         P.vec0 = v0;
         P.nvec = nvec - v0 < 32 ? nvec - v0 : 32;

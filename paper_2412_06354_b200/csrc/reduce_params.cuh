@@ -26,7 +26,7 @@ struct PropParams {
     int F;                  // features of the slab
     int arg_ld;             // features between rows of argmax / route_arg
     int mean;               // divide the finished row by max(1, row length)
-    int piece;              // positions per piece of the long rows
+    int sub, piece;         // positions per warp, and per piece (the unit of partial rows): sub, or RR_WARPS * sub
     int64_t npieces;
     int32_t* tail_row;  // [npieces] row whose partial lives in slot 1, or -1
     float* part_val;    // [npieces][2][F]

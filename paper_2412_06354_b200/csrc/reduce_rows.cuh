@@ -274,7 +274,7 @@ struct RowReducer {
 
 template <typename T, int MODE>
 __host__ __device__ constexpr int rr_min_blocks() {
-    return (MODE == MODE_SUM || MODE == MODE_WSUM) ? 5 : 4;
+    return (MODE == MODE_SUM || MODE == MODE_WSUM) ? 4 : 3;
 }
 
 template <typename T, int LPR, int MODE, bool EPI>
@@ -339,29 +339,35 @@ reduce_rows_kernel(const __grid_constant__ PropParams P, int long_blocks) {
 }
 
 // ------------------------------------------------------------------ positions first
-// One warp per piece of P.piece consecutive positions.  The gathers do not depend on the rows: every lane group streams a
-// run of piece/NG positions with four to eight gathers always in flight (two register buffers of H, each refilled as soon
+// One warp per run of P.sub consecutive positions, a block per piece of RR_WARPS such runs.  The gathers do not depend on the rows: every lane group streams
+// sub/NG of them with four to eight gathers always in flight (two register buffers of H, each refilled as soon
 // as it has been added), and a row's end, marked in the sign bit of the staged index of its last position, only makes the
-// accumulator go out.  Rows cut between runs are stitched inside the warp in run order; rows cut by the piece leave the
-// partials that the second kernel adds.  Rows without edges are written by a scan that is spread over all warps.
+// accumulator go out.  Rows cut between lane groups are stitched inside the warp, rows cut between warps inside the block
+// (through shared memory, by the warp in which they begin), both in position order; rows cut by the piece leave the
+// partials that the second kernel adds (a piece per warp: that kernel took 313 us of 4.9 ms on 123 M edges).  Rows without edges are written by a scan that is spread over all warps.
 //
 // What made the difference (170k nodes, 1.36 M edges, before -> after): a staging of 4 to 12 bytes per position (it was
 // 10 KB per warp, and shared memory is taken from the L1 that holds gathers in flight), 64 registers without spills (32
 // warps per SM), buffers refilled in turn instead of one batch after the other, an epilogue-free row end: fp32 sums over
 // 512-byte rows 113 -> 75 us, bf16 256-byte 74 -> 60 us, 64-byte 54 -> 32 us, max fp32 157 -> 117 us; on 123 M edges the
 // 128-byte rows of a weighted sum 2.45 -> 2.26 ms, max over 256-byte rows 8.1 -> 6.6 ms.
-constexpr int RS_PIECE = 256;  // most positions per piece
+constexpr int RS_SUB = 256;  // most positions per warp
 
-template <int EPC, bool HAS_W, bool HAS_T, bool ARG, bool STITCH>
+template <int EPC, bool HAS_W, bool HAS_T, bool ARG>
 struct StreamStage {
-    int col[RS_PIECE];                       // gathered row; sign bit: last position of a row
-    float w[HAS_W ? RS_PIECE : 1];           // multiplier
-    int t[HAS_T ? RS_PIECE : 1];             // ROUTE: forward position; HEAD: row of the multiplier matrix
-    int row[RS_PIECE + 1];                   // [q] the q-th row with positions in the piece
-    uint16_t start[RS_PIECE + 2];            // [q] its first position in the piece; [count]: end of the last, or n + 1 if it is cut
-    float head[STITCH ? 32 * EPC : 1];       // per lane: sum of the run's first row, which began before the run and ends in it
-    int32_t head_a[STITCH && ARG ? 32 * EPC : 1];
+    int col[RS_SUB];                       // gathered row; sign bit: last position of a row
+    float w[HAS_W ? RS_SUB : 1];           // multiplier
+    int t[HAS_T ? RS_SUB : 1];             // ROUTE: forward position; HEAD: row of the multiplier matrix
+    int row[RS_SUB + 1];                   // [q] the q-th row with positions in the warp's share
+    uint16_t start[RS_SUB + 2];            // [q] its first position in the warp's share; [count]: end of the last, or n + 1 if it is cut
+    float head[32 * EPC];                  // per lane: sum of a group's (then the warp's) first row, which began before it
+    int32_t head_a[ARG ? 32 * EPC : 1];
+    // the warp's last row, if it goes on past the warp: over col and w, which are done with by then
+    __device__ __forceinline__ float* tail() { return reinterpret_cast<float*>(col); }
+    __device__ __forceinline__ int32_t* tail_a() { return reinterpret_cast<int32_t*>(w); }
 };
+// what a warp leaves to the block: its first row began in an earlier warp and ends here (CLOSED) or does not (THROUGH)
+enum { HEAD_NONE = 0, HEAD_CLOSED = 1, HEAD_THROUGH = 2 };
 
 template <int MODE>
 __host__ __device__ constexpr int rs_min_blocks() {
@@ -376,15 +382,16 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     constexpr bool PLAIN = MODE == MODE_SUM;
     constexpr int H = (ROUTE || EF) ? 2 : 4;  // positions per register buffer
     constexpr int MW = EF ? EPC : 1;
-    using Stage = StreamStage<EPC, !PLAIN, ROUTE || HEAD, ARG, (NG > 1)>;
+    using Stage = StreamStage<EPC, !PLAIN, ROUTE || HEAD, ARG>;
+    static_assert(32 * EPC <= RS_SUB, "a row's sums fit over the staged indices");
     extern __shared__ __align__(16) unsigned char rs_smem[];
     pdl_wait();
     const int lane = threadIdx.x & 31, g = lane / LPR, li = lane % LPR;
-    const int c = (int)blockIdx.x * RR_WARPS + (threadIdx.x >> 5);
-    if (c >= P.npieces) return;
-    Stage& S = reinterpret_cast<Stage*>(rs_smem)[threadIdx.x >> 5];
-    const int cs = c * P.piece;
-    const int n = (int)min((int64_t)P.piece, P.E - cs);
+    const int wib = threadIdx.x >> 5, c = (int)blockIdx.x * RR_WARPS + wib;
+    __shared__ int s_head[RR_WARPS], s_tail_row[RR_WARPS];
+    Stage& S = reinterpret_cast<Stage*>(rs_smem)[wib];
+    const int cs = (int)min((int64_t)c * P.sub, P.E);
+    const int n = (int)min((int64_t)P.sub, P.E - cs);  // 0 in the last block's idle warps
     const bool col_lane = li < P.nvec;
     const int ci = col_lane ? li : 0;
 
@@ -406,11 +413,12 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
             }
         }
     }
-    // ---- rows with positions in the piece
-    const int r0 = row_of_position(P.rowptr, P.N, P.E, cs, lane);
-    int m = 1;
-    bool began_before;  // row r0 has positions in an earlier piece
-    {
+    // ---- rows with positions in the warp's share
+    int m = 0;
+    bool began_before = false;  // the first of them has positions in an earlier warp's
+    if (n > 0) {
+        const int r0 = row_of_position(P.rowptr, P.N, P.E, cs, lane);
+        m = 1;
         int64_t last_end = P.rowptr[r0 + 1];
         began_before = P.rowptr[r0] < cs;
         if (lane == 0) { S.row[0] = r0; S.start[0] = 0; }
@@ -456,7 +464,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     __syncwarp();
 
     // ---- this group's run
-    const int L = P.piece / NG, a = g * L, b = min(a + L, n);
+    const int L = P.sub / NG, a = g * L, b = min(a + L, n);
     const uint64_t pol_keep = policy_evict_last();
     const char* const Xl = reinterpret_cast<const char*>(P.X) + (size_t)ci * 16;
     const float* const wh_l = HEAD ? P.wh + ((P.vec0 + ci) * EPC) / P.fph : nullptr;
@@ -471,7 +479,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     };
     auto write_partial = [&](int which, const float* v, const int32_t* va) {
         if (lane >= LPR || !col_lane) return;
-        const size_t off = ((size_t)c * 2 + which) * P.F + (size_t)ci * EPC;
+        const size_t off = ((size_t)blockIdx.x * 2 + which) * P.F + (size_t)ci * EPC;
 #pragma unroll
         for (int j = 0; j < EPC; j += 4) {
             *reinterpret_cast<float4*>(P.part_val + off + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
@@ -493,15 +501,11 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     auto flush = [&]() {  // row q ends here
         if (open) {
             open = false;
-            if (NG == 1) {
-                write_partial(0, acc, arg);
-            } else {
-                head_q = q;
+            head_q = q;
 #pragma unroll
-                for (int j = 0; j < EPC; ++j) {
-                    S.head[lane * EPC + j] = acc[j];
-                    if (ARG) S.head_a[ARG ? lane * EPC + j : 0] = arg[ARG ? j : 0];
-                }
+            for (int j = 0; j < EPC; ++j) {
+                S.head[lane * EPC + j] = acc[j];
+                if (ARG) S.head_a[ARG ? lane * EPC + j : 0] = arg[ARG ? j : 0];
             }
         } else if (col_lane) {
             finish_row<T, MODE, EPI>(P, S.row[q], S.start[q + 1] - S.start[q], ci, acc, arg);
@@ -624,41 +628,59 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
             if (end) flush();
         }
     }
-    // ---- what the runs leave: a closed head (parked), and the sum of a row that goes on past the run (in acc)
+    // ---- what the groups leave: a closed head (parked), and the sum of a row that goes on past the group (in acc)
     const bool rest = a < b && S.col[b - 1] >= 0;
-    int tail_row = -1;
-    if (NG == 1) {
-        if (rest) {
-            write_partial(open ? 0 : 1, acc, arg);
-            if (!open) tail_row = S.row[q];
-        }
-    } else {
-        __syncwarp();
-        float carry[EPC];
-        int32_t carg[ARG ? EPC : 1];
-        bool have = false, before = false;
-        int ck = 0;
-        // values v of a later run join the carry, which wins ties
-        auto join = [&](const float* v, const int32_t* va) {
+    int head_state = HEAD_NONE, tail_row = -1;
+    __syncwarp();
+    // the warp's first or last row, as far as it lies here, for the block (lanes below LPR)
+    auto leave = [&](float* to, int32_t* to_a, const float* v, const int32_t* va) {
+        if (lane < LPR) {
 #pragma unroll
             for (int j = 0; j < EPC; ++j) {
-                if (ARG) {
-                    if (!have || beats<MODE>(v[j], va[ARG ? j : 0], carry[j], carg[ARG ? j : 0])) { carry[j] = v[j]; carg[ARG ? j : 0] = va[ARG ? j : 0]; }
-                } else {
-                    carry[j] = have ? carry[j] + v[j] : v[j];
-                }
+                to[li * EPC + j] = v[j];
+                if (ARG) to_a[li * EPC + j] = va[ARG ? j : 0];
             }
-            if (!have) before = true;  // only the first run can go on from before without a carry
-            have = true;
-        };
+        }
+    };
+    float carry[EPC];
+    int32_t carg[ARG ? EPC : 1];
+    // values v of later positions join the carry, which wins ties
+    auto join = [&](bool have, const float* v, const int32_t* va) {
+#pragma unroll
+        for (int j = 0; j < EPC; ++j) {
+            if (ARG) {
+                if (!have || beats<MODE>(v[j], va[ARG ? j : 0], carry[j], carg[ARG ? j : 0])) { carry[j] = v[j]; carg[ARG ? j : 0] = va[ARG ? j : 0]; }
+            } else {
+                carry[j] = have ? carry[j] + v[j] : v[j];
+            }
+        }
+    };
+    if (NG == 1) {
+        if (head_q >= 0) head_state = HEAD_CLOSED;
+        if (rest && open) {
+            head_state = HEAD_THROUGH;
+            leave(S.head, S.head_a, acc, arg);
+        } else if (rest) {
+            tail_row = S.row[q];
+            leave(S.tail(), S.tail_a(), acc, arg);
+        }
+    } else {
+        bool have = false, before = false;
+        int ck = 0;
 #pragma unroll 1
         for (int gg = 0; gg < NG; ++gg) {
             const int hq = __shfl_sync(0xffffffffu, head_q, gg * LPR), tq = __shfl_sync(0xffffffffu, q, gg * LPR);
             const bool left = __shfl_sync(0xffffffffu, (int)rest, gg * LPR), through = __shfl_sync(0xffffffffu, (int)open, gg * LPR);
             if (hq >= 0) {
-                join(S.head + (gg * LPR + li) * EPC, S.head_a + (ARG ? (gg * LPR + li) * EPC : 0));
-                if (before) write_partial(0, carry, carg);
-                else if (lane < LPR && col_lane) finish_row<T, MODE, EPI>(P, S.row[hq], S.start[hq + 1] - S.start[hq], ci, carry, carg);
+                if (!have) before = true;  // only the first group can go on from before without a carry
+                join(have, S.head + (gg * LPR + li) * EPC, S.head_a + (ARG ? (gg * LPR + li) * EPC : 0));
+                __syncwarp();
+                if (before) {
+                    head_state = HEAD_CLOSED;
+                    leave(S.head, S.head_a, carry, carg);
+                } else if (lane < LPR && col_lane) {
+                    finish_row<T, MODE, EPI>(P, S.row[hq], S.start[hq + 1] - S.start[hq], ci, carry, carg);
+                }
                 have = before = false;
             }
             if (left) {
@@ -669,21 +691,28 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
                     v[j] = __shfl_sync(0xffffffffu, acc[j], gg * LPR + li);
                     if (ARG) va[ARG ? j : 0] = __shfl_sync(0xffffffffu, arg[ARG ? j : 0], gg * LPR + li);
                 }
-                if (!through) have = false;
-                join(v, va);
-                if (!through) before = false;
+                if (!through) have = before = false;
+                else if (!have) before = true;
+                join(have, v, va);
+                have = true;
                 ck = tq;
             }
         }
-        if (have) {  // the row goes on in the next piece
-            write_partial(before ? 0 : 1, carry, carg);
-            if (!before) tail_row = S.row[ck];
+        if (have) {  // the row goes on past the warp
+            __syncwarp();
+            if (before) {
+                head_state = HEAD_THROUGH;
+                leave(S.head, S.head_a, carry, carg);
+            } else {
+                tail_row = S.row[ck];
+                leave(S.tail(), S.tail_a(), carry, carg);
+            }
         }
     }
-    if (lane == 0) P.tail_row[c] = tail_row;
+    if (lane == 0) { s_head[wib] = head_state; s_tail_row[wib] = tail_row; }
     // ---- rows without edges: warp c takes its share of all rows
     {
-        const int64_t per = (P.N + P.npieces - 1) / P.npieces;
+        const int64_t warps = P.npieces * RR_WARPS, per = (P.N + warps - 1) / warps;
         const int64_t b0 = c * per;
         const int e0 = (int)min(b0, (int64_t)P.N), e1 = (int)min(b0 + per, (int64_t)P.N);
         for (int rb = e0; rb < e1; rb += 32) {
@@ -697,6 +726,40 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
                 if (col_lane) finish_row<T, MODE, EPI>(P, rb + bit, 0, ci, acc, arg);
             }
         }
+    }
+    // ---- rows cut between the warps of the block
+    __syncthreads();
+    if (lane < LPR && col_lane) {
+        const Stage* const all = reinterpret_cast<const Stage*>(rs_smem);
+        auto chain = [&](int row) {  // carry goes on into the next warps; row < 0: it began before the block
+#pragma unroll 1
+            for (int k = wib + 1; k < RR_WARPS && s_head[k] != HEAD_NONE; ++k) {
+                join(true, all[k].head + li * EPC, all[k].head_a + (ARG ? li * EPC : 0));
+                if (s_head[k] == HEAD_CLOSED) {
+                    if (row >= 0) finish_row<T, MODE, EPI>(P, row, P.mean ? P.rowptr[row + 1] - P.rowptr[row] : 0, ci, carry, carg);
+                    else write_partial(0, carry, carg);
+                    return;
+                }
+            }
+            write_partial(row >= 0 ? 1 : 0, carry, carg);
+        };
+        if (wib == 0 && head_state != HEAD_NONE) {
+            join(false, S.head + li * EPC, S.head_a + (ARG ? li * EPC : 0));
+            if (head_state == HEAD_CLOSED) write_partial(0, carry, carg);
+            else chain(-1);
+        }
+        if (tail_row >= 0) {
+            join(false, S.tail() + li * EPC, S.tail_a() + (ARG ? li * EPC : 0));
+            chain(tail_row);
+        }
+    }
+    if (threadIdx.x == 0) {  // the row that begins in the block and reaches past it
+        int t = -1;
+        for (int k = 0; k < RR_WARPS; ++k) {
+            if (s_head[k] != HEAD_THROUGH) t = -1;
+            if (s_tail_row[k] >= 0) t = s_tail_row[k];
+        }
+        P.tail_row[blockIdx.x] = t;
     }
 }
 
@@ -874,14 +937,13 @@ fixup_rows_kernel(const __grid_constant__ PropParams P, int nsimple) {
 // ------------------------------------------------------------------ launches
 template <typename T, int MODE, bool EPI, int L>
 static void launch_width(const PropParams& P, bool stream, cudaStream_t st) {
-    const int pieces = (int)ceil_div(P.npieces, RR_WARPS);
     if (stream) {
         constexpr size_t smem = RR_WARPS * sizeof(StreamStage<Chunk<T>::N, MODE != MODE_SUM, MODE == MODE_ROUTE || MODE == MODE_HEADSUM,
-                                                             MODE == MODE_MAX || MODE == MODE_MIN, (L < 32)>);
+                                                             MODE == MODE_MAX || MODE == MODE_MIN>);
         static_assert(smem <= 48 * 1024, "staging fits the default shared memory");
-        launch_overlapped(stream_rows_kernel<T, L, MODE, EPI>, dim3(pieces), dim3(RR_WARPS * 32), smem, st, P);
+        launch_overlapped(stream_rows_kernel<T, L, MODE, EPI>, dim3((unsigned)P.npieces), dim3(RR_WARPS * 32), smem, st, P);
     } else {
-        const int long_blocks = P.E > RR_SHORT ? pieces : 0;
+        const int long_blocks = P.E > RR_SHORT ? (int)ceil_div(P.npieces, RR_WARPS) : 0;
         launch_overlapped(reduce_rows_kernel<T, L, MODE, EPI>, dim3((unsigned)(long_blocks + ceil_div(P.N, RR_WARPS * (32 / L)))), dim3(RR_WARPS * 32), 0, st, P,
                           long_blocks);
     }
