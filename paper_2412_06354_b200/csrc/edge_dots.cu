@@ -1,0 +1,326 @@
+// One value per edge (and head) from the two rows that meet there:
+//   dot      dW[p,h] = scale(i) * <X[col[p],h,:], D[i,h,:]>                      (edge-weight gradients, XI_DOT_XJ, attention)
+//   GATv2    s[p,h]  = sum_c a[h,c] * LeakyReLU(X[col[p],h,c] + D[i,h,c])         for p in row i
+// Every edge is independent, so there are no partials and no second pass.
+#include "reduce_params.cuh"
+
+namespace gnn {
+
+struct EdgeParams {
+    const int64_t* rowptr;
+    const int32_t* col;
+    const void* X;  // gathered rows
+    const void* D;  // rows of the sparse form
+    const float* a;  // GATv2: [F]
+    float* out;
+    int32_t N;
+    int64_t E;
+    int nvec, sub;  // 16-byte chunks per row; positions per warp
+    int H, lph;     // lph > 0: one result per (edge, head), a head = lph adjacent 16-byte chunks
+    float slope;
+};
+
+enum { EDGE_DOT = 0, EDGE_DOT_MEAN = 1, EDGE_GATV2 = 2 };
+
+// ------------------------------------------------------------------ rows of up to 512 bytes
+// Positions first, as in the segmented reduction: a warp stages the gathered rows' indices of its share of positions and
+// the rows they lie in; each of its lane groups streams a run of them with four to eight gathers in flight (two register
+// buffers, each refilled as soon as it is used).  The row's own chunk stays in registers while the row lasts (its end is
+// marked in the sign bit of the staged index), the next row's is fetched meanwhile.  The lanes' shares of four positions
+// are folded together: two levels halve the values a lane carries, the rest reduce the one left (32 lanes: 6 shuffles per
+// four positions instead of 20).
+// Bound by instruction issue for narrow rows and by the gathers (L2 -> SM) for rows of 512 bytes.  Before (4 positions per
+// batch, one batch after the other, 8-byte entries, the row's chunk loaded when it changes) -> now:
+//   100k nodes / 1.6 M edges, 512-byte rows, 8 heads bf16 150 -> 118 us; 123 M edges, 128-byte bf16 rows 2.86 -> 2.54 ms;
+//   GATv2 logits of 100k nodes / 1.6 M edges, 512-byte fp32 rows (a gather per index load, four at a time) 358 -> 130 us.
+constexpr int ED_SUB = 256;  // most positions per warp
+constexpr int ED_H = 4;      // positions per register buffer
+
+template <bool MEAN>
+struct EdgeStage {
+    int col[ED_SUB];           // gathered row; sign bit: last position of a row
+    int row[ED_SUB + 1];       // [q] the q-th row with positions in the warp's share
+    uint16_t start[ED_SUB + 2];
+    float inv[MEAN ? ED_SUB + 1 : 1];  // [q] 1 / length of that row
+};
+
+template <typename T, int LPR, int KIND>
+__global__ void __launch_bounds__(RR_WARPS * 32, sizeof(T) == 4 ? 4 : 3)
+edge_rows_kernel(const __grid_constant__ EdgeParams P) {
+    constexpr int EPC = Chunk<T>::N, NG = 32 / LPR, H = ED_H;
+    constexpr bool MEAN = KIND == EDGE_DOT_MEAN, V2 = KIND == EDGE_GATV2;
+    __shared__ EdgeStage<MEAN> s_all[RR_WARPS];
+    pdl_wait();
+    const int lane = threadIdx.x & 31, g = lane / LPR, li = lane % LPR;
+    const int c = (int)blockIdx.x * RR_WARPS + (threadIdx.x >> 5);
+    EdgeStage<MEAN>& S = s_all[threadIdx.x >> 5];
+    if ((int64_t)c * P.sub >= P.E) return;
+    const int cs = c * P.sub, n = (int)min((int64_t)P.sub, P.E - cs);
+    const bool col_lane = li < P.nvec;
+    const int ci = col_lane ? li : 0;
+    for (int i = lane; i < n; i += 32)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(S.col + i)), "l"(P.col + cs + i) : "memory");
+    bool began_before;
+    const int m = stage_rows(P.rowptr, P.N, P.E, cs, n, lane, S.row, S.start, began_before);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+    for (int q = lane; q < m; q += 32) {
+        const int e = S.start[q + 1];
+        if (e <= n) S.col[e - 1] |= (int)0x80000000;
+        if (MEAN) S.inv[MEAN ? q : 0] = 1.0f / (float)(P.rowptr[S.row[q] + 1] - P.rowptr[S.row[q]]);
+    }
+    __syncwarp();
+
+    const int L = P.sub / NG, a = g * L, b = min(a + L, n);
+    const uint64_t pol_keep = policy_evict_last();
+    const uint32_t row_bytes = (uint32_t)P.nvec * 16;
+    const char* const Xl = reinterpret_cast<const char*>(P.X) + (size_t)ci * 16;
+    const char* const Dl = reinterpret_cast<const char*>(P.D) + (size_t)ci * 16;
+    const int span = P.lph == 0 ? LPR : P.lph;  // lanes per result: the whole row, or one head
+    const int head = P.lph == 0 ? 0 : li / P.lph, wstride = P.lph == 0 ? 1 : P.H;
+    float av[V2 ? EPC : 1];
+#pragma unroll
+    for (int j = 0; j < (V2 ? EPC : 1); ++j) av[j] = V2 ? P.a[ci * EPC + j] : 0.f;
+    int q = 0;  // row of the next position
+    if (NG > 1 && a < b) {
+        int lo = 0, hi = m;  // start[lo] <= a < start[hi]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (S.start[mid] <= a) lo = mid; else hi = mid;
+        }
+        q = lo;
+    }
+    auto own = [&](int qq) { return __ldg(reinterpret_cast<const uint4*>(Dl + (size_t)(uint32_t)S.row[qq] * row_bytes)); };
+    float d[EPC], sc = 1.0f;
+    uint4 own_next = make_uint4(0u, 0u, 0u, 0u);
+    if (a < b) {
+        Chunk<T>::unpack(own(q), d);
+        if (MEAN) sc = S.inv[MEAN ? q : 0];
+        if (q + 1 < m) own_next = own(q + 1);
+    }
+    auto next_row = [&]() {
+        ++q;
+        Chunk<T>::unpack(own_next, d);
+        if (MEAN && q < m) sc = S.inv[MEAN ? q : 0];
+        if (q + 1 < m) own_next = own(q + 1);
+    };
+    auto issue = [&](uint4* x, int i) -> unsigned {  // positions past the group's last gather that one again
+        unsigned ends = 0;
+#pragma unroll
+        for (int u = 0; u < H; ++u) {
+            const int cc = S.col[max(min(i + u, b - 1), 0)];
+            ends |= ((unsigned)cc >> 31) << u;
+            x[u] = ld_hint16(Xl + (size_t)(uint32_t)(cc & 0x7fffffff) * row_bytes, pol_keep);
+        }
+        return ends;
+    };
+    auto use = [&](const uint4* xr, unsigned ends, int i) {
+        float dot[H], scale[MEAN ? H : 1];
+#pragma unroll
+        for (int u = 0; u < H; ++u) {
+            float x[EPC], t = 0.f;
+            Chunk<T>::unpack(xr[u], x);
+#pragma unroll
+            for (int j = 0; j < EPC; ++j) {
+                if (V2) {
+                    const float z = x[j] + d[j];
+                    t = fmaf(av[V2 ? j : 0], z > 0.f ? z : P.slope * z, t);
+                } else {
+                    t = fmaf(x[j], d[j], t);
+                }
+            }
+            dot[u] = col_lane ? t : 0.f;
+            if (MEAN) scale[MEAN ? u : 0] = sc;
+            if ((ends >> u & 1u) && i + u < b) next_row();
+        }
+        __syncwarp();
+        if (span >= 4) {
+            const int h1 = span >> 1, h2 = span >> 2;
+            const bool up1 = (li & h1) != 0, up2 = (li & h2) != 0;
+            const float s0 = up1 ? dot[0] : dot[2], s1 = up1 ? dot[1] : dot[3];
+            const float r0 = (up1 ? dot[2] : dot[0]) + __shfl_xor_sync(0xffffffffu, s0, h1);
+            const float r1 = (up1 ? dot[3] : dot[1]) + __shfl_xor_sync(0xffffffffu, s1, h1);
+            float v = (up2 ? r1 : r0) + __shfl_xor_sync(0xffffffffu, up2 ? r0 : r1, h2);
+            for (int o = span >> 3; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+            const int mine = (up1 ? 2 : 0) + (up2 ? 1 : 0);  // the position of the batch this lane holds
+            if (MEAN) v *= up1 ? (up2 ? scale[MEAN ? 3 : 0] : scale[MEAN ? 2 : 0]) : (up2 ? scale[MEAN ? 1 : 0] : scale[0]);
+            // any lane of the span may end up holding a result (with whole-row results also a lane past a narrow row)
+            if ((P.lph == 0 || col_lane) && (li & (h2 - 1)) == 0 && i + mine < b) P.out[(int64_t)(cs + i + mine) * wstride + head] = v;
+        } else {  // heads of one or two 16-byte chunks
+#pragma unroll
+            for (int u = 0; u < H; ++u) {
+                float v = dot[u];
+                for (int o = span >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (MEAN) v *= scale[MEAN ? u : 0];
+                if (col_lane && (li % span) == 0 && i + u < b) P.out[(int64_t)(cs + i + u) * wstride + head] = v;
+            }
+        }
+    };
+    // same trip count in every group (the shuffles are warp-wide); L is a multiple of 2 H
+    uint4 A[H], B[H];
+    unsigned ea = issue(A, a), eb = issue(B, a + H);
+#pragma unroll 1
+    for (int i = a; i < a + L; i += 2 * H) {
+        const bool more = i + 2 * H < a + L;
+        use(A, ea, i);
+        if (more) ea = issue(A, i + 2 * H);
+        use(B, eb, i + H);
+        if (more) eb = issue(B, i + 3 * H);
+    }
+}
+
+// ------------------------------------------------------------------ rows of up to 2048 bytes
+// A warp per 256 positions walks the rows, the own row's chunks held in registers along the row.
+constexpr int EC_POSITIONS = 256;
+
+template <typename T, int VPL, bool MEAN>
+__global__ void __launch_bounds__(RR_WARPS * 32)
+edge_wide_rows_kernel(const __grid_constant__ EdgeParams P) {
+    constexpr int LPR = 32;
+    pdl_wait();
+    constexpr int EPC = Chunk<T>::N;
+    constexpr int NG = 32 / LPR;
+    constexpr int U = (LPR >= 16) ? (8 / VPL) : 4;
+    const int lane = threadIdx.x & 31, g = lane / LPR, li = lane % LPR;
+    const int64_t c = (int64_t)blockIdx.x * RR_WARPS + (threadIdx.x >> 5);
+        const int64_t cs = c * EC_POSITIONS;
+    const int64_t ce = (cs + EC_POSITIONS < P.E) ? cs + EC_POSITIONS : P.E;
+    if (cs >= ce) return;
+    const uint64_t pol_keep = policy_evict_last(), pol_stream = policy_evict_first();
+    const size_t row_bytes = (size_t)P.nvec * 16;
+    const char* Xb = reinterpret_cast<const char*>(P.X);
+    const char* Db = reinterpret_cast<const char*>(P.D);
+    // row containing position cs: last row with rowptr[r] <= cs
+    int r = lower_bound_i64(P.rowptr, P.N + 1, cs + 1) - 1;
+    int64_t pos = cs;
+    while (pos < ce) {
+        r = first_row_ending_after(P.rowptr, r, P.N, pos, lane);  // skip rows that end at or before pos
+        const int64_t rs = P.rowptr[r], re = P.rowptr[r + 1];
+        const int64_t b = re < ce ? re : ce;
+        float d[VPL][EPC];
+#pragma unroll
+        for (int v = 0; v < VPL; ++v) {
+            const int ci = v * LPR + li;
+            if (ci < P.nvec) {
+                Chunk<T>::unpack(ld_hint16(Db + (size_t)r * row_bytes + (size_t)ci * 16, pol_stream), d[v]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < EPC; ++j) d[v][j] = 0.f;
+            }
+        }
+        const float scale = MEAN ? 1.0f / (float)(re - rs) : 1.0f;
+        for (int64_t base = pos; base < b; base += 32) {
+            const int n = (int)((b - base) < 32 ? (b - base) : 32);
+            int myc = lane < n ? ld_hint_i32(P.col + base + lane, pol_stream) : 0;
+            const int rounds = (n + NG - 1) / NG;
+            for (int r0 = 0; r0 < rounds; r0 += U) {
+                uint4 buf[U][VPL];
+                bool ok[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int e = (r0 + u) * NG + g;
+                    ok[u] = e < n;
+                    int cv = __shfl_sync(0xffffffffu, myc, e & 31);
+                    if (ok[u]) {
+#pragma unroll
+                        for (int v = 0; v < VPL; ++v) {
+                            const int ci = v * LPR + li;
+                            if (ci < P.nvec) buf[u][v] = ld_hint16(Xb + (size_t)cv * row_bytes + (size_t)ci * 16, pol_keep);
+                        }
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    float dotv[VPL];
+#pragma unroll
+                    for (int v = 0; v < VPL; ++v) {
+                        dotv[v] = 0.f;
+                        const int ci = v * LPR + li;
+                        if (ok[u] && ci < P.nvec) {
+                            float x[EPC];
+                            Chunk<T>::unpack(buf[u][v], x);
+#pragma unroll
+                            for (int j = 0; j < EPC; ++j) dotv[v] = fmaf(x[j], d[v][j], dotv[v]);
+                        }
+                    }
+                    const int64_t p = base + (r0 + u) * NG + g;
+                    if (P.lph == 0) {  // one dot product per edge over the whole row
+                        float dot = dotv[0];
+#pragma unroll
+                        for (int v = 1; v < VPL; ++v) dot += dotv[v];
+#pragma unroll
+                        for (int o = LPR / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+                        if (ok[u] && li == 0) P.out[p] = scale * dot;
+                    } else {  // one per (edge, head): a head covers lph adjacent lanes
+#pragma unroll
+                        for (int v = 0; v < VPL; ++v) {
+                            float dot = dotv[v];
+                            for (int o = P.lph >> 1; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
+                            const int ci = v * LPR + li;
+                            if (ok[u] && ci < P.nvec && (li % P.lph) == 0) P.out[p * P.H + ci / P.lph] = scale * dot;
+                        }
+                    }
+                }
+            }
+        }
+        pos = b;
+    }
+}
+
+template <typename T>
+static void launch_edge_rows(EdgeParams& P, int kind, cudaStream_t st) {
+    if (P.nvec > 32) {
+        const dim3 grid((unsigned)ceil_div(P.E, (int64_t)EC_POSITIONS * RR_WARPS)), block(RR_WARPS * 32);
+#define GNN_WIDE(V) \
+    kind == EDGE_DOT_MEAN ? launch_overlapped(edge_wide_rows_kernel<T, V, true>, grid, block, 0, st, P) : launch_overlapped(edge_wide_rows_kernel<T, V, false>, grid, block, 0, st, P)
+        if (P.nvec <= 64) GNN_WIDE(2);
+        else GNN_WIDE(4);
+#undef GNN_WIDE
+        return;
+    }
+    // positions per warp: fewer on small graphs, so that all SMs have warps
+    P.sub = P.E >= 2500 * 1000 ? 256 : P.E >= 512 * 1024 ? 128 : 64;
+    const dim3 grid((unsigned)ceil_div(P.E, (int64_t)P.sub * RR_WARPS)), block(RR_WARPS * 32);
+#define GNN_EDGE(L)                                                                                             \
+    kind == EDGE_DOT ? launch_overlapped(edge_rows_kernel<T, L, EDGE_DOT>, grid, block, 0, st, P)               \
+    : kind == EDGE_DOT_MEAN ? launch_overlapped(edge_rows_kernel<T, L, EDGE_DOT_MEAN>, grid, block, 0, st, P)   \
+                            : launch_overlapped(edge_rows_kernel<T, L, EDGE_GATV2>, grid, block, 0, st, P)
+    if (P.nvec <= 4) GNN_EDGE(4);
+    else if (P.nvec <= 8) GNN_EDGE(8);
+    else if (P.nvec <= 16) GNN_EDGE(16);
+    else GNN_EDGE(32);
+#undef GNN_EDGE
+}
+
+static gnn_status run_edges(const char* who, const gnn_csr* g, const void* X, const void* D, const float* a, int H, int C, int kind, float slope,
+                            gnn_dtype dtype, float* out, cudaStream_t st) {
+    const int s = elem_size(dtype), F = H * C;
+    GNN_REQUIRE(C > 0 && ((size_t)C * s) % 16 == 0, GNN_ERR_UNSUPPORTED, "%s: a head must be a multiple of 16 bytes wide", who);
+    const int nvec = F * s / 16, lph = C * s / 16;
+    GNN_REQUIRE(nvec <= 128, GNN_ERR_UNSUPPORTED, "%s: feature rows wider than 2048 bytes", who);
+    GNN_REQUIRE(H == 1 || (lph <= 32 && (lph & (lph - 1)) == 0), GNN_ERR_UNSUPPORTED,
+                "%s: a head must span a power-of-two number (<= 32) of 16-byte chunks (C=%d)", who, C);
+    GNN_REQUIRE(aligned16(X) && aligned16(D), GNN_ERR_INVALID_ARG, "%s: feature matrices must be 16-byte aligned", who);
+    GNN_REQUIRE(g->E < ((int64_t)1 << 31) - 4096, GNN_ERR_UNSUPPORTED, "%s: positions must fit 32 bits (E < 2^31)", who);
+    if (g->E == 0) return GNN_OK;
+    EdgeParams P = {};
+    P.rowptr = g->rowptr; P.col = g->col; P.X = X; P.D = D; P.a = a; P.out = out;
+    P.N = g->N; P.E = g->E; P.nvec = nvec; P.H = H; P.lph = H > 1 ? lph : 0; P.slope = slope;
+    if (dtype == GNN_F32) launch_edge_rows<float>(P, kind, st);
+    else launch_edge_rows<__nv_bfloat16>(P, kind, st);
+    GNN_CHECK_LAUNCH(who);
+    return GNN_OK;
+}
+
+// one dot product per edge (H == 1) or per edge and head, scaled by 1 / row length if mean
+gnn_status run_sddmm(const char* who, const gnn_csr* g, const void* X, const void* D, int H, int C, int mean,
+                     gnn_dtype dtype, float* dW, cudaStream_t st) {
+    return run_edges(who, g, X, D, nullptr, H, C, mean ? EDGE_DOT_MEAN : EDGE_DOT, 0.f, dtype, dW, st);
+}
+
+gnn_status run_gatv2_logits(const char* who, const gnn_csr* g, const void* X, const void* D, const float* a, int H, int C, float slope, gnn_dtype dtype,
+                            float* s, cudaStream_t st) {
+    return run_edges(who, g, X, D, a, H, C, EDGE_GATV2, slope, dtype, s, st);
+}
+
+}  // namespace gnn

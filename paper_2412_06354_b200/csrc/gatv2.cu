@@ -4,19 +4,20 @@
 // The nonlinearity sits between the sum of the two transformed endpoints and the attention vector, so the
 // logit is not a sum of a source term and a target term as in gnn_gat_fused: both rows meet at every edge.
 //
-// Forward: every position is independent.  A warp takes 256 consecutive positions, keeps the target row's chunk
-// in registers while the row lasts, gathers four source rows at a time and reduces over the lanes of a head.
+// Forward: one value per edge and head, the edge-wise kernel of edge_dots.cu.
 // Backward: dXr[i] sums over the positions of row i, dXl[j] over the transposed row of j, each term
-// ds * a * LeakyReLU'(z) needing both rows again.  A warp walks a row (four gathers in flight), rows over 256
-// positions get a block whose warps take contiguous shares that are added in warp order; da is the column sum
-// of per-row partials.  Every order is fixed: results are bit-reproducible.  Gathered rows stay in registers as
-// loaded and are unpacked where they are used (bf16: 14-16 registers fewer, one more block per SM).
-#include "common.cuh"
+// ds * a * LeakyReLU'(z) needing both rows again; da sums ds * LeakyReLU(z) over all positions.  Both are the segmented
+// reduction of reduce_rows.cuh with the own row's chunk in registers; da falls out of the first as one partial per block.
+// Its scratch (partial rows) has to fit the caller's workspace, whose size knows N only, and a call without da may come
+// without a workspace: then (below, mean degrees of several hundred) a warp walks a row, rows over 256 positions get a
+// block whose warps take contiguous shares that are added in warp order, and da is the column sum of per-row partials.
+// Every order is fixed: results are bit-reproducible.
+// 100k nodes / 1.6 M edges with hubs, 4 heads x 32 fp32: 1010 us by row and block, 265 us as segmented reductions.
+#include "propagate.cuh"
 
 namespace gnn {
 
 constexpr int V2_U = 4;           // gathers in flight per warp
-constexpr int V2_CHUNK = 256;     // positions per warp in the forward kernel
 constexpr int V2_LONG = 256;      // rows above this many positions get a block in the backward kernels
 constexpr int V2_BLOCK = 512;     // threads of that block
 constexpr int V2_SUM_BLOCKS = 592;
@@ -29,9 +30,8 @@ struct V2Params {
     const void* Xother;        // gathered rows
     const float* a;            // [F]
     const float* ds;           // [E,H]
-    float* s_out;              // forward: [E,H]
-    void* dX;                  // backward: [N,F]
-    float* da_part;            // backward: [N,F] per-row partial of da, or nullptr
+    void* dX;                  // [N,F]
+    float* da_part;            // [N,F] per-row partial of da, or nullptr
     int32_t N;
     int64_t E;
     int nvec, H, lph;          // 16-byte chunks per row (<= 32), heads, chunks per head
@@ -52,51 +52,6 @@ __device__ __forceinline__ void v2_load(const void* base, int64_t row, int nvec,
 // the same chunk as it lies in memory: unpacked where it is used, so that a gather in flight holds four registers
 __device__ __forceinline__ uint4 v2_load_raw(const void* base, int64_t row, int nvec, int li, bool on) {
     return on ? __ldg(reinterpret_cast<const uint4*>(base) + (size_t)row * nvec + li) : make_uint4(0u, 0u, 0u, 0u);
-}
-
-// ------------------------------------------------------------------ forward
-template <typename T>
-__global__ void __launch_bounds__(256) gatv2_logits_kernel(const V2Params P) {
-    constexpr int EPC = Chunk<T>::N;
-    const int lane = threadIdx.x & 31;
-    const int64_t c = (int64_t)blockIdx.x * 8 + (threadIdx.x >> 5);
-    const int64_t cs = c * V2_CHUNK;
-    if (cs >= P.E) return;
-    const int64_t ce = cs + V2_CHUNK < P.E ? cs + V2_CHUNK : P.E;
-    const bool on = lane < P.nvec;
-    const int span = P.H > 1 ? P.lph : 32;  // lanes that share one result
-    float av[EPC];
-#pragma unroll
-    for (int j = 0; j < EPC; ++j) av[j] = on ? P.a[lane * EPC + j] : 0.f;
-    int r = lower_bound_i64(P.rowptr, P.N + 1, cs + 1) - 1;  // row holding position cs
-    int64_t rend = P.rowptr[r + 1];
-    float xs[EPC];
-    v2_load<T>(P.Xself, r, P.nvec, lane, on, xs);
-    for (int64_t p0 = cs; p0 < ce; p0 += V2_U) {
-        uint4 raw[V2_U];
-#pragma unroll
-        for (int u = 0; u < V2_U; ++u)
-            if (p0 + u < ce) raw[u] = v2_load_raw(P.Xother, P.col[p0 + u], P.nvec, lane, on);
-#pragma unroll
-        for (int u = 0; u < V2_U; ++u) {
-            const int64_t p = p0 + u;
-            if (p >= ce) break;
-            if (p >= rend) {  // the row changed (rows without edges are passed over)
-                do { ++r; rend = P.rowptr[r + 1]; } while (p >= rend);
-                v2_load<T>(P.Xself, r, P.nvec, lane, on, xs);
-            }
-            float xo[EPC];
-            Chunk<T>::unpack(raw[u], xo);
-            float t = 0.f;
-#pragma unroll
-            for (int j = 0; j < EPC; ++j) {
-                const float z = xo[j] + xs[j];
-                t = fmaf(av[j], z > 0.f ? z : P.slope * z, t);
-            }
-            for (int o = span >> 1; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-            if (on && (lane % span) == 0) P.s_out[p * P.H + (P.H > 1 ? lane / P.lph : 0)] = t;
-        }
-    }
 }
 
 // ------------------------------------------------------------------ backward
@@ -225,12 +180,22 @@ __global__ void __launch_bounds__(256) v2_colsum_partial_kernel(const float* __r
         bsum[(size_t)blockIdx.x * F + f] = s;
     }
 }
-__global__ void v2_colsum_final_kernel(const float* __restrict__ bsum, int nb, int F, float* __restrict__ out) {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= F) return;
+// out[f] = sum of the nb partials of column f: 32 walkers per column, four loads in flight each, added in walker order
+__global__ void __launch_bounds__(1024) v2_colsum_final_kernel(const float* __restrict__ bsum, int nb, int F, float* __restrict__ out) {
+    pdl_wait();
+    __shared__ float sums[32][33];
+    const int col = threadIdx.x & 31, w = threadIdx.x >> 5, f = blockIdx.x * 32 + col;
     float s = 0.f;
-    for (int b = 0; b < nb; ++b) s += bsum[(size_t)b * F + f];
-    out[f] = s;
+    if (f < F)
+#pragma unroll 4
+        for (int b = w; b < nb; b += 32) s += bsum[(size_t)b * F + f];
+    sums[w][col] = s;
+    __syncthreads();
+    if (w == 0 && f < F) {
+#pragma unroll
+        for (int k = 1; k < 32; ++k) s += sums[k][col];
+        out[f] = s;
+    }
 }
 
 static gnn_status v2_check(const char* who, const gnn_csr* g, int H, int C, gnn_dtype dtype, int* nvec, int* lph) {
@@ -263,14 +228,7 @@ gnn_status gnn_gatv2_logits(const gnn_csr* g, const void* Xl, const void* Xr, co
     if (g->E == 0) return GNN_OK;
     GNN_REQUIRE(Xl && Xr && a && s_csr && g->col, GNN_ERR_INVALID_ARG, "%s: null argument", who);
     GNN_REQUIRE(aligned16(Xl) && aligned16(Xr), GNN_ERR_INVALID_ARG, "%s: feature matrices must be 16-byte aligned", who);
-    V2Params P = {};
-    P.rowptr = g->rowptr; P.col = g->col; P.Xself = Xr; P.Xother = Xl; P.a = a; P.s_out = s_csr;
-    P.N = g->N; P.E = g->E; P.nvec = nvec; P.H = H; P.lph = lph; P.slope = slope;
-    const int grid = (int)ceil_div(ceil_div(g->E, V2_CHUNK), 8);
-    if (dtype == GNN_F32) gatv2_logits_kernel<float><<<grid, 256, 0, as_stream(stream)>>>(P);
-    else gatv2_logits_kernel<__nv_bfloat16><<<grid, 256, 0, as_stream(stream)>>>(P);
-    GNN_CHECK_LAUNCH(who);
-    return GNN_OK;
+    return run_gatv2_logits(who, g, Xl, Xr, a, H, C, slope, dtype, s_csr, as_stream(stream));
 }
 
 size_t gnn_gatv2_logits_backward_workspace(int32_t N, int H, int C) {
@@ -296,6 +254,22 @@ gnn_status gnn_gatv2_logits_backward(const gnn_csr* g, const void* Xl, const voi
                 "%s: workspace of %zu bytes needed for da, %zu given", who, need, ws_bytes);
     if (g->N == 0) return GNN_OK;
     cudaStream_t st = as_stream(stream);
+    GNN_REQUIRE(dXr || !da, GNN_ERR_INVALID_ARG, "%s: da is computed with dXr; pass dXr as well", who);
+    const int row_bytes = F * elem_size(dtype);
+    const int64_t pieces = gatv2_rows_pieces(g->N, g->E, row_bytes);
+    const size_t rows_ws = gatv2_rows_workspace(g->N, g->E, F, row_bytes);
+    if (ws && aligned16(ws) && ws_bytes >= rows_ws + up256((size_t)pieces * F * 4)) {
+        float* const da_part = da ? (float*)((char*)ws + rows_ws) : nullptr;
+        if (dXr) {
+            rc = run_gatv2_rows(who, g->N, g->E, g->rowptr, g->col, nullptr, ds_csr, H, Xr, Xl, a, slope, F, dtype, dXr, da_part, ws, st);
+            if (rc != GNN_OK) return rc;
+        }
+        if (da) {
+            launch_overlapped(v2_colsum_final_kernel, dim3((unsigned)ceil_div(F, 32)), dim3(1024), 0, st, da_part, (int)pieces, F, da);
+            GNN_CHECK_LAUNCH(who);
+        }
+        return dXl ? run_gatv2_rows(who, g->N, g->E, g->rowptrT, g->colT, g->t2f, ds_csr, H, Xl, Xr, a, slope, F, dtype, dXl, nullptr, ws, st) : GNN_OK;
+    }
     V2Params P = {};
     P.a = a; P.ds = ds_csr; P.N = g->N; P.E = g->E; P.nvec = nvec; P.H = H; P.lph = lph; P.slope = slope;
     const int wgrid = (int)(ceil_div(g->N, 8) < 148 * 16 ? ceil_div(g->N, 8) : 148 * 16);
@@ -306,7 +280,6 @@ gnn_status gnn_gatv2_logits_backward(const gnn_csr* g, const void* Xl, const voi
     gatv2_backward_rows_kernel<TYPE, DAFLAG><<<wgrid, 256, 0, st>>>(P); \
     gatv2_backward_long_kernel<TYPE, DAFLAG><<<lgrid, V2_BLOCK, 0, st>>>(P);
     if (dXr || da) {  // rows = targets: self = Xr, gathered = Xl, factors at the positions themselves
-        GNN_REQUIRE(dXr, GNN_ERR_INVALID_ARG, "%s: da is computed with dXr; pass dXr as well", who);
         P.rowptr = g->rowptr; P.col = g->col; P.pos_index = nullptr; P.Xself = Xr; P.Xother = Xl; P.dX = dXr; P.da_part = part;
         if (dtype == GNN_F32) { if (da) { GNN_V2_BWD(float, true) } else { GNN_V2_BWD(float, false) } }
         else { if (da) { GNN_V2_BWD(__nv_bfloat16, true) } else { GNN_V2_BWD(__nv_bfloat16, false) } }
@@ -321,7 +294,7 @@ gnn_status gnn_gatv2_logits_backward(const gnn_csr* g, const void* Xl, const voi
     if (da) {
         const int rpb = (int)ceil_div(g->N, V2_SUM_BLOCKS), nb = (int)ceil_div(g->N, rpb);
         v2_colsum_partial_kernel<<<nb, 256, 0, st>>>(part, g->N, F, rpb, bsum);
-        v2_colsum_final_kernel<<<(int)ceil_div(F, 128), 128, 0, st>>>(bsum, nb, F, da);
+        launch_overlapped(v2_colsum_final_kernel, dim3((unsigned)ceil_div(F, 32)), dim3(1024), 0, st, bsum, nb, F, da);
         GNN_CHECK_LAUNCH(who);
     }
     return GNN_OK;

@@ -8,8 +8,6 @@
 
 namespace gnn {
 
-gnn_status sddmm_heads(const char* who, const gnn_csr* g, const void* X, const void* dOut, int H, int C,
-                       gnn_dtype dtype, float* dW_EH, cudaStream_t st, int mean);
 
 // ------------------------------------------------------------------ element-wise kernels
 // out[i, chunk] = c(i) * D[i, chunk], c(i) = row length (times_degree) or [row length > 0]
@@ -346,7 +344,7 @@ gnn_status gnn_propagate_msg_backward(const gnn_csr* g, gnn_msg msg, gnn_op op, 
             rc = run_sddmm(who, g, Xj, dOut, 1, F, op == GNN_MEAN, dtype, de_csr, st);
             if (rc != GNN_OK) return rc;
         } else {
-            rc = sddmm_heads(who, g, Xj, dOut, e_width, F / e_width, dtype, de_csr, st, op == GNN_MEAN);
+            rc = run_sddmm(who, g, Xj, dOut, e_width, F / e_width, op == GNN_MEAN, dtype, de_csr, st);
             if (rc != GNN_OK) return rc;
         }
     }
@@ -447,7 +445,7 @@ gnn_status gnn_edge_dot(const gnn_csr* g, const void* Xj, const void* Xi, int H,
     GNN_REQUIRE(dtype == GNN_F32 || dtype == GNN_BF16, GNN_ERR_INVALID_ARG, "%s: bad dtype", who);
     GNN_REQUIRE(H >= 1 && C >= 1, GNN_ERR_INVALID_ARG, "%s: bad H or C", who);
     if (H == 1) return run_sddmm(who, g, Xj, Xi, 1, C, 0, dtype, s_csr, as_stream(stream));
-    return sddmm_heads(who, g, Xj, Xi, H, C, dtype, s_csr, as_stream(stream), 0);
+    return run_sddmm(who, g, Xj, Xi, H, C, 0, dtype, s_csr, as_stream(stream));
 }
 
 size_t gnn_edge_dot_backward_workspace(int64_t E, int H, int C) {

@@ -1,278 +1,12 @@
 // Fused propagate (Sec. 3 "Message Passing": apply_edges + aggregate_neighbors combined into a
 // generalised sparse x dense product) and its backward passes: host side of the segmented reduction
-// (reduce_rows.cuh) and the edge-wise dot products of the weight gradients.
+// (reduce_rows.cuh); the edge-wise dot products of the weight gradients are in edge_dots.cu.
 #include <mutex>
 
 #include "reduce_params.cuh"
 
 namespace gnn {
 
-// ------------------------------------------------------------------ edge-weight gradient (SDDMM)
-// dW[p] = scale(i) * <X[col[p],:], dOut[i,:]> for p in row i.  Same chunking; every edge is
-// independent, so no partials.  The dOut row stays in registers along the row.
-struct SddmmParams {
-    const int64_t* rowptr;
-    const int32_t* col;
-    const void* X;
-    const void* dOut;
-    float* dW;
-    int32_t N;
-    int64_t E;
-    int nvec;
-    int mean;
-    int64_t nchunks;
-    int H, lph;  // lph > 0: one result per (edge, head), a head = lph adjacent 16-byte chunks
-};
-
-template <typename T, int LPR, int VPL>
-__global__ void __launch_bounds__(PF_WARPS * 32)
-sddmm_chunk_kernel(const SddmmParams P) {
-    constexpr int EPC = Chunk<T>::N;
-    constexpr int NG = 32 / LPR;
-    constexpr int U = (LPR >= 16) ? (8 / VPL) : 4;
-    const int lane = threadIdx.x & 31, g = lane / LPR, li = lane % LPR;
-    const int64_t c = (int64_t)blockIdx.x * PF_WARPS + (threadIdx.x >> 5);
-    if (c >= P.nchunks) return;
-    const int64_t cs = c * PF_SLAB;
-    const int64_t ce = (cs + PF_SLAB < P.E) ? cs + PF_SLAB : P.E;
-    if (cs >= ce) return;
-    const uint64_t pol_keep = policy_evict_last(), pol_stream = policy_evict_first();
-    const size_t row_bytes = (size_t)P.nvec * 16;
-    const char* Xb = reinterpret_cast<const char*>(P.X);
-    const char* Db = reinterpret_cast<const char*>(P.dOut);
-    // row containing position cs: last row with rowptr[r] <= cs
-    int r = lower_bound_i64(P.rowptr, P.N + 1, cs + 1) - 1;
-    int64_t pos = cs;
-    while (pos < ce) {
-        r = first_row_ending_after(P.rowptr, r, P.N, pos, lane);  // skip rows that end at or before pos
-        const int64_t rs = P.rowptr[r], re = P.rowptr[r + 1];
-        const int64_t b = re < ce ? re : ce;
-        float d[VPL][EPC];
-#pragma unroll
-        for (int v = 0; v < VPL; ++v) {
-            const int ci = v * LPR + li;
-            if (ci < P.nvec) {
-                Chunk<T>::unpack(ld_hint16(Db + (size_t)r * row_bytes + (size_t)ci * 16, pol_stream), d[v]);
-            } else {
-#pragma unroll
-                for (int j = 0; j < EPC; ++j) d[v][j] = 0.f;
-            }
-        }
-        const float scale = P.mean ? 1.0f / (float)(re - rs) : 1.0f;
-        for (int64_t base = pos; base < b; base += 32) {
-            const int n = (int)((b - base) < 32 ? (b - base) : 32);
-            int myc = lane < n ? ld_hint_i32(P.col + base + lane, pol_stream) : 0;
-            const int rounds = (n + NG - 1) / NG;
-            for (int r0 = 0; r0 < rounds; r0 += U) {
-                uint4 buf[U][VPL];
-                bool ok[U];
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const int e = (r0 + u) * NG + g;
-                    ok[u] = e < n;
-                    int cv = __shfl_sync(0xffffffffu, myc, e & 31);
-                    if (ok[u]) {
-#pragma unroll
-                        for (int v = 0; v < VPL; ++v) {
-                            const int ci = v * LPR + li;
-                            if (ci < P.nvec) buf[u][v] = ld_hint16(Xb + (size_t)cv * row_bytes + (size_t)ci * 16, pol_keep);
-                        }
-                    }
-                }
-#pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    float dotv[VPL];
-#pragma unroll
-                    for (int v = 0; v < VPL; ++v) {
-                        dotv[v] = 0.f;
-                        const int ci = v * LPR + li;
-                        if (ok[u] && ci < P.nvec) {
-                            float x[EPC];
-                            Chunk<T>::unpack(buf[u][v], x);
-#pragma unroll
-                            for (int j = 0; j < EPC; ++j) dotv[v] = fmaf(x[j], d[v][j], dotv[v]);
-                        }
-                    }
-                    const int64_t p = base + (r0 + u) * NG + g;
-                    if (P.lph == 0) {  // one dot product per edge over the whole row
-                        float dot = dotv[0];
-#pragma unroll
-                        for (int v = 1; v < VPL; ++v) dot += dotv[v];
-#pragma unroll
-                        for (int o = LPR / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-                        if (ok[u] && li == 0) P.dW[p] = scale * dot;
-                    } else {  // one per (edge, head): a head covers lph adjacent lanes
-#pragma unroll
-                        for (int v = 0; v < VPL; ++v) {
-                            float dot = dotv[v];
-                            for (int o = P.lph >> 1; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-                            const int ci = v * LPR + li;
-                            if (ok[u] && ci < P.nvec && (li % P.lph) == 0) P.dW[p * P.H + ci / P.lph] = scale * dot;
-                        }
-                    }
-                }
-            }
-        }
-        pos = b;
-    }
-}
-
-// ------------------------------------------------------------------ flat SDDMM for short rows
-// Same idea as propagate_flat_kernel: positions first, rows second.  The warp stages the gathered
-// rows of its 256 positions and finds, by marking row starts and a prefix maximum, the row of every
-// position; each lane group then takes a contiguous run and issues, per batch of 4 positions, the
-// independent loads of X[col[p]] and, where the row changes, dOut[row(p)].  Every position is independent, so there are no partials and no second pass.
-constexpr int SF_U = 4;
-constexpr int FL_WARPS = 4;
-
-struct SddmmFlatSmem {
-    int2 e[PF_SLAB];        // x: gathered row of X, y: start entry of the position's row
-    int32_t srow[PF_SLAB];  // [k] row starting at position k of the chunk ([0]: the row holding position 0)
-    float sinv[PF_SLAB];    // [k] 1, or 1 / row length for the mean
-};
-
-template <typename T, int LPR>
-__global__ void __launch_bounds__(FL_WARPS * 32, 8)
-sddmm_flat_kernel(const SddmmParams P) {
-    constexpr int EPC = Chunk<T>::N, NG = 32 / LPR, U = SF_U, L = PF_SLAB / NG;
-    __shared__ SddmmFlatSmem s_all[FL_WARPS];
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int64_t c = (int64_t)blockIdx.x * FL_WARPS + wib;
-    if (c >= P.nchunks) return;
-    SddmmFlatSmem& S = s_all[wib];
-    const uint64_t pol_keep = policy_evict_last(), pol_stream = policy_evict_first();
-    const int64_t cs = c * PF_SLAB;
-    const int n = (int)((cs + PF_SLAB < P.E ? cs + PF_SLAB : P.E) - cs);
-    const int g = lane / LPR, li = lane % LPR;
-    const bool col_lane = li < P.nvec;
-
-    // the row holding position cs: largest r with rowptr[r] <= cs (32-way search)
-    int lo = 0, hi = P.N;
-    while (hi - lo > 1) {
-        const int step = (hi - lo + 31) / 32;
-        const int idx = min(lo + (lane + 1) * step, hi);
-        const bool le = idx < hi && P.rowptr[idx] <= cs;
-        const int k = __popc(__ballot_sync(0xffffffffu, le));
-        const int nlo = lo + k * step;
-        hi = min(nlo + step, hi);
-        lo = nlo;
-    }
-    const int cur0 = lo;
-    auto row_factor = [&](int64_t len) { return P.mean ? 1.0f / (float)(len > 1 ? len : 1) : 1.0f; };
-    for (int i = lane; i < n; i += 32) S.e[i] = make_int2(ld_hint_i32(P.col + cs + i, pol_stream), 0);
-    if (lane == 0) { S.srow[0] = cur0; S.sinv[0] = row_factor(P.rowptr[cur0 + 1] - P.rowptr[cur0]); }
-    __syncwarp();
-    for (int rb = cur0 + 1; rb < P.N;) {  // non-empty rows starting inside the chunk
-        const int r = rb + lane;
-        int64_t rs = 0, re = 0;
-        bool live = false;
-        if (r < P.N) {
-            rs = P.rowptr[r];
-            live = rs < cs + n;
-            if (live) re = P.rowptr[r + 1];
-        }
-        if (live && re > rs) {
-            const int k = (int)(rs - cs);
-            S.srow[k] = r;
-            S.sinv[k] = row_factor(re - rs);
-            S.e[k].y = k;
-        }
-        if (!__all_sync(0xffffffffu, live)) break;
-        // 32 rows without edges: jump over the rest of the run
-        if (__all_sync(0xffffffffu, re == rs)) rb = first_row_ending_after(P.rowptr, rb + 32, P.N, __shfl_sync(0xffffffffu, rs, 0), lane);
-        else rb += 32;
-    }
-    __syncwarp();
-    {  // prefix maximum of the start marks: lane owns positions 8*lane .. 8*lane+7
-        int m[8];
-        int run = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int i = lane * 8 + q;
-            run = max(run, i < n ? S.e[i].y : 0);
-            m[q] = run;
-        }
-        int incl = run;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl = max(incl, t);
-        }
-        int before = __shfl_up_sync(0xffffffffu, incl, 1);
-        if (lane == 0) before = 0;
-#pragma unroll
-        for (int q = 0; q < 8; ++q) {
-            const int i = lane * 8 + q;
-            if (i < n) S.e[i].y = max(before, m[q]);
-        }
-    }
-    __syncwarp();
-
-    const int a = g * L, b = min(a + L, n);
-    const size_t row_bytes = (size_t)P.nvec * 16;
-    const char* Xl = reinterpret_cast<const char*>(P.X) + (size_t)(col_lane ? li : 0) * 16;
-    const char* Dl = reinterpret_cast<const char*>(P.dOut) + (size_t)(col_lane ? li : 0) * 16;
-    const int span = P.lph == 0 ? LPR : P.lph;  // lanes per result: the whole row, or one head
-    const bool writer = col_lane && (li % span) == 0;
-    const int head = P.lph == 0 ? 0 : li / P.lph, wstride = P.lph == 0 ? 1 : P.H;
-    const uint32_t row_bytes32 = (uint32_t)row_bytes;
-    int kprev = -1;   // start entry of the position before this batch
-    uint4 dcur = make_uint4(0, 0, 0, 0);  // this lane's chunk of the current row of dOut: reloaded only when the row changes
-    for (int i = a; i < a + L; i += U) {  // same trip count in every lane: the shuffles below are warp-wide
-        uint4 xb[U], db[U];
-        int k[U];
-        bool fresh[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const bool ok = i + u < b;
-            const int2 e = S.e[ok ? i + u : 0];
-            k[u] = ok ? e.y : -1;
-            fresh[u] = ok && k[u] != (u == 0 ? kprev : k[u - 1]);
-            if (ok) xb[u] = ld_hint16(Xl + (size_t)((uint32_t)e.x) * row_bytes32, pol_keep);
-            if (fresh[u]) db[u] = __ldg(reinterpret_cast<const uint4*>(Dl + (size_t)((uint32_t)S.srow[e.y]) * row_bytes32));
-        }
-        kprev = k[U - 1];
-        static_assert(SF_U == 4, "the reductions below fold four positions at a time");
-        float dot[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (fresh[u]) dcur = db[u];
-            dot[u] = 0.f;
-            if (k[u] >= 0 && col_lane) {
-                float x[EPC], d[EPC];
-                Chunk<T>::unpack(xb[u], x);
-                Chunk<T>::unpack(dcur, d);
-#pragma unroll
-                for (int j = 0; j < EPC; ++j) dot[u] = fmaf(x[j], d[j], dot[u]);
-            }
-        }
-        if (span >= 4) {
-            // fold the four positions while reducing over the span lanes: the first two levels halve the values
-            // a lane carries (2 + 1 shuffles), the rest reduce the one left; the quarter of the span a lane
-            // sits in decides which position it ends up with: 6 shuffles for 32 lanes instead of 20
-            const int h1 = span >> 1, h2 = span >> 2;
-            const bool up1 = (li & h1) != 0, up2 = (li & h2) != 0;
-            const float s0 = up1 ? dot[0] : dot[2], s1 = up1 ? dot[1] : dot[3];
-            const float r0 = (up1 ? dot[2] : dot[0]) + __shfl_xor_sync(0xffffffffu, s0, h1);
-            const float r1 = (up1 ? dot[3] : dot[1]) + __shfl_xor_sync(0xffffffffu, s1, h1);
-            float v = (up2 ? r1 : r0) + __shfl_xor_sync(0xffffffffu, up2 ? r0 : r1, h2);
-            for (int o = span >> 3; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-            const int mine = (up1 ? 2 : 0) + (up2 ? 1 : 0);  // the position of the batch this lane holds
-            const int km = mine == 0 ? k[0] : mine == 1 ? k[1] : mine == 2 ? k[2] : k[3];
-            // any lane of the span may end up holding a result (with whole-row results also a lane past a narrow row)
-            if ((P.lph == 0 || col_lane) && (li & (h2 - 1)) == 0 && km >= 0) P.dW[(cs + i + mine) * wstride + head] = S.sinv[km] * v;
-        } else {  // heads of one or two 16-byte chunks
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                float v = dot[u];
-                for (int o = span >> 1; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                if (k[u] >= 0 && writer) P.dW[(cs + i + u) * wstride + head] = S.sinv[k[u]] * v;
-            }
-        }
-    }
-}
-
-// ------------------------------------------------------------------ host dispatch
 bool pick_shape(int nvec, int* lpr, int* vpl) {
     if (nvec < 1 || nvec > 128) return false;
     if (nvec <= 4) { *lpr = 4; *vpl = 1; }
@@ -298,28 +32,6 @@ static void launch_mode(const PropParams& P, int mode, bool stream, cudaStream_t
     if (mode == MODE_SUM || mode == MODE_WSUM || mode == MODE_HEADSUM) launch_reduce_sums<T>(P, mode, stream, st);
     else launch_reduce_others<T>(P, mode, stream, st);
 }
-
-template <typename T>
-static void launch_sddmm(const SddmmParams& P, int lpr, int vpl, cudaStream_t st) {
-    if (vpl == 1) {  // positions first
-        const int grid = (int)ceil_div(P.nchunks, FL_WARPS);
-        switch (lpr) {
-            case 4: sddmm_flat_kernel<T, 4><<<grid, FL_WARPS * 32, 0, st>>>(P); break;
-            case 8: sddmm_flat_kernel<T, 8><<<grid, FL_WARPS * 32, 0, st>>>(P); break;
-            case 16: sddmm_flat_kernel<T, 16><<<grid, FL_WARPS * 32, 0, st>>>(P); break;
-            default: sddmm_flat_kernel<T, 32><<<grid, FL_WARPS * 32, 0, st>>>(P); break;
-        }
-        return;
-    }
-    const int grid = (int)ceil_div(P.nchunks, PF_WARPS);
-    const int thr = PF_WARPS * 32;
-#define GNN_SD_CASE(L, V) \
-    if (lpr == L && vpl == V) { sddmm_chunk_kernel<T, L, V><<<grid, thr, 0, st>>>(P); }
-    GNN_SD_CASE(4, 1) GNN_SD_CASE(8, 1) GNN_SD_CASE(16, 1) GNN_SD_CASE(32, 1) GNN_SD_CASE(32, 2) GNN_SD_CASE(32, 4)
-#undef GNN_SD_CASE
-}
-
-static int64_t num_slabs(int64_t E) { return E > 0 ? ceil_div(E, PF_SLAB) : 1; }
 
 struct ReduceWs {
     int32_t* tail_row;
@@ -361,6 +73,36 @@ size_t chunked_workspace(int64_t E, int F, bool with_arg) {
     return carve(nullptr, ceil_div(E, (int64_t)per), F < 256 ? F : 256, with_arg).bytes;
 }
 
+int64_t gatv2_rows_pieces(int32_t N, int64_t E, int row_bytes) {
+    return E > 0 ? ceil_div(E, (int64_t)warp_positions(N, E, row_bytes, true) * RR_WARPS) : 1;
+}
+
+size_t gatv2_rows_workspace(int32_t N, int64_t E, int F, int row_bytes) { return carve(nullptr, gatv2_rows_pieces(N, E, row_bytes), F, false).bytes; }
+
+template <typename T> void launch_gatv2_rows(const PropParams& P, cudaStream_t st);  // reduce_gatv2.cu
+extern template void launch_gatv2_rows<float>(const PropParams&, cudaStream_t);
+extern template void launch_gatv2_rows<__nv_bfloat16>(const PropParams&, cudaStream_t);
+
+gnn_status run_gatv2_rows(const char* who, int32_t N, int64_t E, const int64_t* rowptr, const int32_t* col, const int32_t* ds_index, const float* ds, int H,
+                          const void* Xself, const void* Xother, const float* a, float slope, int F, gnn_dtype dtype, void* out, float* da_part, void* ws,
+                          cudaStream_t st) {
+    PropParams P = {};
+    const int row_bytes = F * elem_size(dtype);
+    P.rowptr = rowptr; P.col = col; P.X = Xother; P.out = out;
+    P.N = N; P.E = E; P.nvec = row_bytes / 16; P.x_ld = P.out_ld = (uint32_t)row_bytes; P.F = P.arg_ld = F;
+    P.sub = warp_positions(N, E, row_bytes, true);
+    P.piece = P.sub * RR_WARPS;
+    P.npieces = gatv2_rows_pieces(N, E, row_bytes);
+    const ReduceWs w = carve(ws, P.npieces, F, false);
+    P.tail_row = w.tail_row; P.part_val = w.part_val;
+    P.wh = ds; P.wh_index = ds_index; P.H = H; P.fph = F / H; P.epi_a = a;
+    P.v2_self = Xself; P.slope = slope; P.da_part = da_part;
+    if (dtype == GNN_F32) launch_gatv2_rows<float>(P, st);
+    else launch_gatv2_rows<__nv_bfloat16>(P, st);
+    GNN_CHECK_LAUNCH(who);
+    return GNN_OK;
+}
+
 gnn_status run_chunked(const char* who, int mode, int32_t N, int64_t E, const int64_t* rowptr,
                        const int32_t* col, const float* w, const void* X, void* out,
                        int32_t* argmax, const int64_t* gscale_rowptr, const int32_t* route_arg,
@@ -382,6 +124,7 @@ gnn_status run_chunked(const char* who, int mode, int32_t N, int64_t E, const in
     P.rowptr = rowptr; P.col = col; P.w = w; P.argmax = argmax;
     P.gscale_rowptr = gscale_rowptr; P.route_arg = route_arg; P.route_pos = route_pos;
     P.N = N; P.E = E; P.mean = mean; P.arg_ld = F;
+    P.v2_self = nullptr; P.slope = 0.f; P.da_part = nullptr;
     P.wh = nullptr; P.wh_index = nullptr; P.H = 1; P.fph = F; P.epi_l = P.epi_r = P.epi_a = P.epi_b = nullptr;
     if (hx) {
         GNN_REQUIRE(mode == MODE_HEADSUM && (hx->wh || E == 0) && hx->H >= 1 && F % hx->H == 0 && (F / hx->H) % epc == 0, GNN_ERR_UNSUPPORTED,
@@ -439,50 +182,6 @@ gnn_status run_chunked(const char* who, int mode, int32_t N, int64_t E, const in
         if (dtype == GNN_F32) launch_mode<float>(P, mode, stream, st);
         else launch_mode<__nv_bfloat16>(P, mode, stream, st);
     }
-    GNN_CHECK_LAUNCH(who);
-    return GNN_OK;
-}
-
-// dW[p,h] = <X[col[p],h,:], dOut[i,h,:]> for p in row i: the per-head edge dot products of the
-// attention backward pass
-gnn_status sddmm_heads(const char* who, const gnn_csr* g, const void* X, const void* dOut, int H, int C,
-                       gnn_dtype dtype, float* dW_EH, cudaStream_t st, int mean) {
-    const int s = elem_size(dtype), F = H * C;
-    GNN_REQUIRE(((size_t)C * s) % 16 == 0, GNN_ERR_UNSUPPORTED, "%s: a head must be a multiple of 16 bytes wide", who);
-    const int lph = C * s / 16;
-    GNN_REQUIRE(lph <= 32 && (lph & (lph - 1)) == 0, GNN_ERR_UNSUPPORTED,
-                "%s: a head must span a power-of-two number (<= 32) of 16-byte chunks (C=%d)", who, C);
-    int lpr, vpl;
-    GNN_REQUIRE(pick_shape(F * s / 16, &lpr, &vpl), GNN_ERR_UNSUPPORTED, "%s: feature rows wider than 2048 bytes", who);
-    GNN_REQUIRE(lph <= lpr, GNN_ERR_UNSUPPORTED, "%s: head wider than the row layout", who);
-    GNN_REQUIRE(aligned16(X) && aligned16(dOut), GNN_ERR_INVALID_ARG, "%s: feature matrices must be 16-byte aligned", who);
-    if (g->E == 0) return GNN_OK;
-    SddmmParams S;
-    S.rowptr = g->rowptr; S.col = g->col; S.X = X; S.dOut = dOut; S.dW = dW_EH;
-    S.N = g->N; S.E = g->E; S.nvec = F * s / 16; S.mean = mean; S.nchunks = num_slabs(g->E); S.H = H; S.lph = lph;
-    if (dtype == GNN_F32) launch_sddmm<float>(S, lpr, vpl, st);
-    else launch_sddmm<__nv_bfloat16>(S, lpr, vpl, st);
-    GNN_CHECK_LAUNCH(who);
-    return GNN_OK;
-}
-
-// one dot product per edge (H == 1; scaled by 1 / row length if mean) or per edge and head
-gnn_status run_sddmm(const char* who, const gnn_csr* g, const void* X, const void* D, int H, int C, int mean,
-                     gnn_dtype dtype, float* dW, cudaStream_t st) {
-    if (H > 1) {
-        return sddmm_heads(who, g, X, D, H, C, dtype, dW, st, mean);
-    }
-    const int s = elem_size(dtype), F = C;
-    GNN_REQUIRE(F > 0 && ((size_t)F * s) % 16 == 0, GNN_ERR_UNSUPPORTED, "%s: F*sizeof(element) must be a multiple of 16 bytes", who);
-    int lpr, vpl;
-    GNN_REQUIRE(pick_shape(F * s / 16, &lpr, &vpl), GNN_ERR_UNSUPPORTED, "%s: feature rows wider than 2048 bytes", who);
-    GNN_REQUIRE(aligned16(X) && aligned16(D), GNN_ERR_INVALID_ARG, "%s: feature matrices must be 16-byte aligned", who);
-    if (g->E == 0) return GNN_OK;
-    SddmmParams S;
-    S.rowptr = g->rowptr; S.col = g->col; S.X = X; S.dOut = D; S.dW = dW;
-    S.N = g->N; S.E = g->E; S.nvec = F * s / 16; S.mean = mean; S.nchunks = num_slabs(g->E); S.H = 1; S.lph = 0;
-    if (dtype == GNN_F32) launch_sddmm<float>(S, lpr, vpl, st);
-    else launch_sddmm<__nv_bfloat16>(S, lpr, vpl, st);
     GNN_CHECK_LAUNCH(who);
     return GNN_OK;
 }

@@ -7,7 +7,7 @@ namespace gnn {
 constexpr int PF_SLAB = 256;   // positions per warp of the edge-wise dot products
 constexpr int PF_WARPS = 8;    // warps per block
 
-enum { MODE_SUM = 0, MODE_MAX = 1, MODE_MIN = 2, MODE_ROUTE = 3, MODE_HEADSUM = 4, MODE_EFSUM = 5, MODE_WSUM = 6 };
+enum { MODE_SUM = 0, MODE_MAX = 1, MODE_MIN = 2, MODE_ROUTE = 3, MODE_HEADSUM = 4, MODE_EFSUM = 5, MODE_WSUM = 6, MODE_V2 = 7 };
 
 // MODE_HEADSUM extras: multipliers per (position, head) and an optional rank-1 row epilogue
 //   out[r,f] += epi_l[r,h(f)] * epi_a[f] + epi_r[r,h(f)] * epi_b[f]
@@ -45,6 +45,18 @@ gnn_status run_chunked(const char* who, int mode, int32_t N, int64_t E, const in
                        int32_t* argmax, const int64_t* gscale_rowptr, const int32_t* route_arg,
                        const int32_t* route_pos, int mean, int F, gnn_dtype dtype, void* ws,
                        size_t ws_bytes, cudaStream_t st, const HeadExtra* hx = nullptr, const RowExtra* rx = nullptr);
+
+// Gradient of the GATv2 logits with respect to the rows of one sparse form (see PropParams): out [N,F], and with da_part one
+// partial of da per piece.  gatv2_rows_pieces: how many pieces; ws: gatv2_rows_workspace bytes.
+int64_t gatv2_rows_pieces(int32_t N, int64_t E, int row_bytes);
+size_t gatv2_rows_workspace(int32_t N, int64_t E, int F, int row_bytes);
+gnn_status run_gatv2_rows(const char* who, int32_t N, int64_t E, const int64_t* rowptr, const int32_t* col, const int32_t* ds_index, const float* ds, int H,
+                          const void* Xself, const void* Xother, const float* a, float slope, int F, gnn_dtype dtype, void* out, float* da_part, void* ws,
+                          cudaStream_t st);
+
+// s[p,h] = sum over the features f of head h of a[f] * LeakyReLU(X[col[p],f] + D[i,f]) for p in row i
+gnn_status run_gatv2_logits(const char* who, const gnn_csr* g, const void* X, const void* D, const float* a, int H, int C, float slope, gnn_dtype dtype,
+                            float* s, cudaStream_t st);
 
 // dW[p,h] = <X[col[p],h,:], D[i,h,:]> for p in row i (H = 1, lph = 0: one dot product per edge, times 1/row length if mean)
 gnn_status run_sddmm(const char* who, const gnn_csr* g, const void* X, const void* D, int H, int C, int mean,

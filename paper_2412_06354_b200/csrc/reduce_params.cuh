@@ -51,6 +51,10 @@ struct PropParams {
     uint32_t self_ld;  // bytes between rows of self_X
     const int64_t* self_rowptr;
     const float* bias;  // [F] or nullptr
+    // MODE_V2 (gradient of GATv2 logits): out[r,f] = epi_a[f] * sum over p of wh[p,h(f)] * LeakyReLU'(X[col[p],f] + v2_self[r,f])
+    const void* v2_self;
+    float slope;
+    float* da_part;  // [npieces][F]: per piece, sum over p of wh[p,h(f)] * LeakyReLU(X[col[p],f] + v2_self[r,f]); or nullptr
 };
 
 // Smallest row r in [lo, N) with rowptr[r + 1] > v, or N: the first row at or after lo that has a
@@ -75,6 +79,66 @@ __device__ __forceinline__ int first_row_ending_after(const int64_t* __restrict_
         lo = nlo;
     }
     return lo;
+}
+
+// Position holding `pos`: the last row r with rowptr[r] <= pos (0 <= pos < E).  Warp-cooperative.  The first look is at 32
+// rows spaced 64 apart around the row that even degrees would give, then 32-way steps, then 64 rows at once.
+__device__ __forceinline__ int row_of_position(const int64_t* __restrict__ rowptr, int N, int64_t E, int64_t pos, int lane) {
+    int lo = 0, hi = N;  // rowptr[lo] <= pos < rowptr[hi]
+    if (N > 1024) {
+        const int guess = (int)((double)pos * ((double)N / (double)E));
+        const int idx = guess + (lane - 16) * 64;
+        const bool le = idx <= 0 || (idx < N && rowptr[idx] <= pos);
+        const int c = __popc(__ballot_sync(0xffffffffu, le));
+        if (c > 0) lo = max(lo, guess + (c - 1 - 16) * 64);
+        if (c < 32) hi = min(hi, guess + (c - 16) * 64);
+    }
+    while (hi - lo > 64) {
+        const int step = (hi - lo + 31) / 32;
+        const int idx = lo + lane * step;
+        const bool le = idx < hi && rowptr[idx] <= pos;  // true for a prefix of the lanes, lane 0 among them
+        const int c = __popc(__ballot_sync(0xffffffffu, le));
+        lo = lo + (c - 1) * step;
+        hi = min(lo + step, hi);
+    }
+    const int a = lo + 1 + lane, b = a + 32;
+    const bool la = a < hi && rowptr[a] <= pos, lb = b < hi && rowptr[b] <= pos;
+    return lo + __popc(__ballot_sync(0xffffffffu, la)) + __popc(__ballot_sync(0xffffffffu, lb));
+}
+
+// The rows with positions in [cs, cs + n), n > 0: their ids to row[], their first positions relative to cs to start[] (0 for a
+// row that began before), start[count] = the last one's end, or n + 1 if it goes on.  Returns the count.  Warp-cooperative.
+__device__ __forceinline__ int stage_rows(const int64_t* __restrict__ rowptr, int N, int64_t E, int cs, int n, int lane, int* row, uint16_t* start,
+                                          bool& began_before) {
+    const int r0 = row_of_position(rowptr, N, E, cs, lane);
+    int m = 1;
+    int64_t last_end = rowptr[r0 + 1];
+    began_before = rowptr[r0] < cs;
+    if (lane == 0) { row[0] = r0; start[0] = 0; }
+    for (int rb = r0 + 1; rb < N;) {
+        const int r = rb + lane;
+        int64_t s = 0, e = 0;
+        bool in = false;
+        if (r < N) {
+            s = rowptr[r];
+            in = s < cs + n;
+            if (in) e = rowptr[r + 1];
+        }
+        const bool live = in && e > s;
+        const unsigned lm = __ballot_sync(0xffffffffu, live);
+        if (live) {
+            const int q = m + __popc(lm & ((1u << lane) - 1u));
+            row[q] = r;
+            start[q] = (uint16_t)(s - cs);
+        }
+        m += __popc(lm);
+        if (lm) last_end = __shfl_sync(0xffffffffu, e, 31 - __clz(lm));
+        if (!__all_sync(0xffffffffu, in)) break;
+        if (lm == 0) rb = first_row_ending_after(rowptr, rb + 32, N, __shfl_sync(0xffffffffu, s, 0), lane);  // over a run of empty rows
+        else rb += 32;
+    }
+    if (lane == 0) start[m] = (uint16_t)min(last_end - cs, (int64_t)n + 1);
+    return m;
 }
 
 }  // namespace gnn

@@ -52,6 +52,10 @@ __device__ __forceinline__ void finish_row(const PropParams& P, int row, int64_t
 #pragma unroll
         for (int j = 0; j < EPC; ++j) v[j] *= f;
     }
+    if (MODE == MODE_V2) {
+#pragma unroll
+        for (int j = 0; j < EPC; ++j) v[j] *= P.epi_a[ci * EPC + j];
+    }
     if (EPI && MODE == MODE_HEADSUM && P.epi_l) {
         const int f0 = (P.vec0 + ci) * EPC, h = f0 / P.fph;  // a 16-byte chunk lies inside one head
         const float el = P.epi_l[(size_t)row * P.H + h], er = P.epi_r[(size_t)row * P.H + h];
@@ -91,31 +95,6 @@ __device__ __forceinline__ void finish_row(const PropParams& P, int row, int64_t
     }
 }
 
-
-// Position holding `pos`: the last row r with rowptr[r] <= pos (0 <= pos < E).  Warp-cooperative.  The first look is at 32
-// rows spaced 64 apart around the row that even degrees would give, then 32-way steps, then 64 rows at once.
-__device__ __forceinline__ int row_of_position(const int64_t* __restrict__ rowptr, int N, int64_t E, int64_t pos, int lane) {
-    int lo = 0, hi = N;  // rowptr[lo] <= pos < rowptr[hi]
-    if (N > 1024) {
-        const int guess = (int)((double)pos * ((double)N / (double)E));
-        const int idx = guess + (lane - 16) * 64;
-        const bool le = idx <= 0 || (idx < N && rowptr[idx] <= pos);
-        const int c = __popc(__ballot_sync(0xffffffffu, le));
-        if (c > 0) lo = max(lo, guess + (c - 1 - 16) * 64);
-        if (c < 32) hi = min(hi, guess + (c - 16) * 64);
-    }
-    while (hi - lo > 64) {
-        const int step = (hi - lo + 31) / 32;
-        const int idx = lo + lane * step;
-        const bool le = idx < hi && rowptr[idx] <= pos;  // true for a prefix of the lanes, lane 0 among them
-        const int c = __popc(__ballot_sync(0xffffffffu, le));
-        lo = lo + (c - 1) * step;
-        hi = min(lo + step, hi);
-    }
-    const int a = lo + 1 + lane, b = a + 32;
-    const bool la = a < hi && rowptr[a] <= pos, lb = b < hi && rowptr[b] <= pos;
-    return lo + __popc(__ballot_sync(0xffffffffu, la)) + __popc(__ballot_sync(0xffffffffu, lb));
-}
 
 template <typename T, int LPR, int MODE>
 struct RowReducer {
@@ -378,11 +357,12 @@ template <typename T, int LPR, int MODE, bool EPI>
 __global__ void __launch_bounds__(RR_WARPS * 32, (rs_min_blocks<MODE>()))
 stream_rows_kernel(const __grid_constant__ PropParams P) {
     constexpr int EPC = Chunk<T>::N, NG = 32 / LPR;
-    constexpr bool ARG = MODE == MODE_MAX || MODE == MODE_MIN, EF = MODE == MODE_EFSUM, HEAD = MODE == MODE_HEADSUM, ROUTE = MODE == MODE_ROUTE;
-    constexpr bool PLAIN = MODE == MODE_SUM;
+    constexpr bool ARG = MODE == MODE_MAX || MODE == MODE_MIN, EF = MODE == MODE_EFSUM, HEAD = MODE == MODE_HEADSUM || MODE == MODE_V2, ROUTE = MODE == MODE_ROUTE;
+    constexpr bool PLAIN = MODE == MODE_SUM, V2 = MODE == MODE_V2, DA = V2 && EPI;
     constexpr int H = (ROUTE || EF) ? 2 : 4;  // positions per register buffer
     constexpr int MW = EF ? EPC : 1;
-    using Stage = StreamStage<EPC, !PLAIN, ROUTE || HEAD, ARG>;
+    constexpr bool HAS_W = !PLAIN && !V2;  // a multiplier per position
+    using Stage = StreamStage<EPC, HAS_W, ROUTE || HEAD, ARG>;
     static_assert(32 * EPC <= RS_SUB, "a row's sums fit over the staged indices");
     extern __shared__ __align__(16) unsigned char rs_smem[];
     pdl_wait();
@@ -402,7 +382,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
         for (int i = lane; i < n; i += 32) {
             if (P.col) copy(S.col + i, P.col + cs + i);
             else S.col[i] = cs + i;
-            if (!PLAIN) {
+            if (HAS_W) {
                 if (P.w) copy(S.w + i, P.w + cs + i);
                 else S.w[i] = 1.0f;
             }
@@ -416,39 +396,10 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     // ---- rows with positions in the warp's share
     int m = 0;
     bool began_before = false;  // the first of them has positions in an earlier warp's
-    if (n > 0) {
-        const int r0 = row_of_position(P.rowptr, P.N, P.E, cs, lane);
-        m = 1;
-        int64_t last_end = P.rowptr[r0 + 1];
-        began_before = P.rowptr[r0] < cs;
-        if (lane == 0) { S.row[0] = r0; S.start[0] = 0; }
-        for (int rb = r0 + 1; rb < P.N;) {
-            const int r = rb + lane;
-            int64_t s = 0, e = 0;
-            bool in = false;
-            if (r < P.N) {
-                s = P.rowptr[r];
-                in = s < cs + n;
-                if (in) e = P.rowptr[r + 1];
-            }
-            const bool live = in && e > s;
-            const unsigned lm = __ballot_sync(0xffffffffu, live);
-            if (live) {
-                const int q = m + __popc(lm & ((1u << lane) - 1u));
-                S.row[q] = r;
-                S.start[q] = (uint16_t)(s - cs);
-            }
-            m += __popc(lm);
-            if (lm) last_end = __shfl_sync(0xffffffffu, e, 31 - __clz(lm));
-            if (!__all_sync(0xffffffffu, in)) break;
-            if (lm == 0) rb = first_row_ending_after(P.rowptr, rb + 32, P.N, __shfl_sync(0xffffffffu, s, 0), lane);  // over a run of empty rows
-            else rb += 32;
-        }
-        if (lane == 0) S.start[m] = (uint16_t)min(last_end - cs, (int64_t)n + 1);
-    }
+    if (n > 0) m = stage_rows(P.rowptr, P.N, P.E, cs, n, lane, S.row, S.start, began_before);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncwarp();
-    if (!PLAIN && P.gscale_rowptr) {
+    if (HAS_W && P.gscale_rowptr) {
 #pragma unroll 4
         for (int i = lane; i < n; i += 32) {
             const int cc = S.col[i];
@@ -498,6 +449,18 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     }
     bool open = a < b && (S.start[q] < a || (a == 0 && began_before));  // the run's first row began before the run
     int head_q = -1;
+    // MODE_V2: this row's own features, the next row's on their way, and the share of da (all rows of the group together)
+    float xs[V2 ? EPC : 1], da[DA ? EPC : 1];
+    uint4 own_next = make_uint4(0u, 0u, 0u, 0u);
+    auto own = [&](int qq) { return __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(P.v2_self) + (size_t)S.row[qq] * P.x_ld) + ci); };
+    if (V2) {
+        if (a < b) {
+            Chunk<T>::unpack(own(q), xs);
+            if (q + 1 < m) own_next = own(q + 1);
+        }
+#pragma unroll
+        for (int j = 0; j < (DA ? EPC : 1); ++j) da[j] = 0.f;
+    }
     auto flush = [&]() {  // row q ends here
         if (open) {
             open = false;
@@ -512,6 +475,10 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
         }
         clear();
         ++q;
+        if (V2) {
+            Chunk<T>::unpack(own_next, xs);
+            if (q + 1 < m) own_next = own(q + 1);
+        }
     };
     struct Buf {
         uint4 x[H];
@@ -548,7 +515,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     auto use = [&](const Buf& B, int u, int i) {  // entry u of the buffer, position i of the piece
         float x[EPC];
         Chunk<T>::unpack(B.x[u], x);
-        const float w = PLAIN ? 1.0f : S.w[PLAIN ? 0 : i];
+        const float w = HAS_W ? S.w[HAS_W ? i : 0] : 1.0f;
         if (ARG) {
 #pragma unroll
             for (int k = 0; k < EPC; ++k) {
@@ -574,6 +541,15 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
         } else if (PLAIN) {
 #pragma unroll
             for (int k = 0; k < EPC; k += 2) add2(acc[k], acc[k + 1], x[k], x[k + 1]);
+        } else if (V2) {  // ds * LeakyReLU'(z), times a when the row is complete; da: ds * LeakyReLU(z)
+            const float f = B.hw[HEAD ? u : 0][0], fs = f * P.slope;
+#pragma unroll
+            for (int k = 0; k < EPC; ++k) {
+                const float z = x[k] + xs[V2 ? k : 0];
+                const float d = z > 0.f ? f : fs;
+                acc[k] += d;
+                if (DA) da[DA ? k : 0] = fmaf(d, z, da[DA ? k : 0]);
+            }
         } else {
             // w = 1 in the per-head mode unless the gathered rows are rescaled (backward of the mean)
             const float f = HEAD ? B.hw[HEAD ? u : 0][0] * w : w;
@@ -751,6 +727,24 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
         if (tail_row >= 0) {
             join(false, S.tail() + li * EPC, S.tail_a() + (ARG ? li * EPC : 0));
             chain(tail_row);
+        }
+    }
+    if (DA) {  // the block's share of da: lane groups by an xor tree, then the warps in order
+#pragma unroll
+        for (int o = LPR; o < 32; o <<= 1)
+#pragma unroll
+            for (int j = 0; j < EPC; ++j) da[DA ? j : 0] += __shfl_xor_sync(0xffffffffu, da[DA ? j : 0], o);
+        __syncthreads();  // the stages are done with
+        float* const sums = reinterpret_cast<float*>(rs_smem);  // [RR_WARPS][LPR * EPC]
+        if (lane < LPR)
+#pragma unroll
+            for (int j = 0; j < EPC; ++j) sums[(wib * LPR + li) * EPC + j] = da[DA ? j : 0];
+        __syncthreads();
+        for (int f = threadIdx.x; f < P.F; f += RR_WARPS * 32) {
+            float v = 0.f;
+#pragma unroll
+            for (int k = 0; k < RR_WARPS; ++k) v += sums[k * LPR * EPC + f];
+            P.da_part[(size_t)blockIdx.x * P.F + f] = v;
         }
     }
     if (threadIdx.x == 0) {  // the row that begins in the block and reaches past it
@@ -938,11 +932,11 @@ fixup_rows_kernel(const __grid_constant__ PropParams P, int nsimple) {
 template <typename T, int MODE, bool EPI, int L>
 static void launch_width(const PropParams& P, bool stream, cudaStream_t st) {
     if (stream) {
-        constexpr size_t smem = RR_WARPS * sizeof(StreamStage<Chunk<T>::N, MODE != MODE_SUM, MODE == MODE_ROUTE || MODE == MODE_HEADSUM,
-                                                             MODE == MODE_MAX || MODE == MODE_MIN>);
+        constexpr size_t smem = RR_WARPS * sizeof(StreamStage<Chunk<T>::N, MODE != MODE_SUM && MODE != MODE_V2,
+                                                             MODE == MODE_ROUTE || MODE == MODE_HEADSUM || MODE == MODE_V2, MODE == MODE_MAX || MODE == MODE_MIN>);
         static_assert(smem <= 48 * 1024, "staging fits the default shared memory");
         launch_overlapped(stream_rows_kernel<T, L, MODE, EPI>, dim3((unsigned)P.npieces), dim3(RR_WARPS * 32), smem, st, P);
-    } else {
+    } else if constexpr (MODE != MODE_V2) {
         const int long_blocks = P.E > RR_SHORT ? (int)ceil_div(P.npieces, RR_WARPS) : 0;
         launch_overlapped(reduce_rows_kernel<T, L, MODE, EPI>, dim3((unsigned)(long_blocks + ceil_div(P.N, RR_WARPS * (32 / L)))), dim3(RR_WARPS * 32), 0, st, P,
                           long_blocks);
@@ -951,7 +945,7 @@ static void launch_width(const PropParams& P, bool stream, cudaStream_t st) {
 
 template <typename T, int MODE>
 static void launch_reduce(const PropParams& P, bool stream, cudaStream_t st) {
-    const bool epi = P.has_epi || P.epi_l;
+    const bool epi = MODE == MODE_V2 ? P.da_part != nullptr : P.has_epi || P.epi_l;
 #define GNN_WIDTH(L) epi ? launch_width<T, MODE, true, L>(P, stream, st) : launch_width<T, MODE, false, L>(P, stream, st)
     if (P.nvec <= 4) GNN_WIDTH(4);
     else if (P.nvec <= 8) GNN_WIDTH(8);

@@ -265,3 +265,24 @@ def test_gatv2_backward_hub_rows_of_both_orientations(gnn, dtype, H, C):
     assert_close(to_host64(da), rb["da"], rb["Sda"], "f32", "GATv2 da")
     again = gnn.gatv2_logits_backward(g, to_dev(Xl), to_dev(Xr), to_dev(a), to_dev(ds[ref["eid"]]), H)
     assert all(np.array_equal(bits(x), bits(y)) for x, y in zip((dXl, dXr, da), again)), "not bit-reproducible"
+
+
+@pytest.mark.parametrize("dtype,H,C", [("f32", 4, 16), ("bf16", 8, 32)])
+def test_gatv2_backward_without_workspace(gnn, dtype, H, C):
+    """A call without da may come without a workspace: rows are then walked one by one (and hubs by a block)."""
+    import torch
+    n, src, dst = ragged_graph(150 + H)
+    g = build_graph(gnn, n, src, dst)
+    ref = host_csr(n, src, dst)
+    F = H * C
+    Xl, Xr = feats((n, F), dtype, 1700 + F), feats((n, F), dtype, 1701 + F, stream=1)
+    a, ds = synth.uniform_f32((H, C), -1.0, 1.0, 30), synth.normal_f32((len(src), H), 31)
+    t = [to_dev(x) for x in (Xl, Xr, a, ds[ref["eid"]])]
+    dXl, dXr = torch.empty_like(t[0]), torch.empty_like(t[1])
+    lib = gnn.load()
+    st = torch.cuda.current_stream().cuda_stream
+    assert lib.gnn_gatv2_logits_backward(g.ref, *(x.data_ptr() for x in t), H, C, 0 if dtype == "f32" else 1, 0.2, dXl.data_ptr(), dXr.data_ptr(),
+                                         None, None, 0, st) == 0
+    rb = oracle.gatv2_logits_backward(n, src, dst, Xl, Xr, a, H, ds)
+    assert_close(to_host64(dXl), rb["dXl"], rb["SXl"], dtype, "GATv2 dXl")
+    assert_close(to_host64(dXr), rb["dXr"], rb["SXr"], dtype, "GATv2 dXr")
