@@ -2,7 +2,10 @@
 // self-loops, edge-data permutation.  Integer results are unique and bit-exact.
 #include <stdarg.h>
 
-#include "common.cuh"
+#include <mutex>
+#include <vector>
+
+#include "reduce_params.cuh"
 
 namespace gnn {
 
@@ -12,19 +15,6 @@ void set_error(const char* fmt, ...) {
     va_start(ap, fmt);
     vsnprintf(g_err, sizeof(g_err), fmt, ap);
     va_end(ap);
-}
-
-// ------------------------------------------------------------------ validation
-__global__ void validate_coo_kernel(int32_t N, int64_t E, const int32_t* __restrict__ src,
-                                    const int32_t* __restrict__ dst, int* __restrict__ flag) {
-    int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    bool bad = false;
-    for (; k < E; k += stride) {
-        int s = src[k], d = dst[k];
-        bad |= (s < 0) | (s >= N) | (d < 0) | (d >= N);
-    }
-    if (bad) *flag = 1;  // benign race: every writer stores the same value
 }
 
 // ------------------------------------------------------------------ validation of a caller-built sparse form
@@ -89,11 +79,7 @@ __global__ void csr_validate_positions_kernel(int32_t N, int64_t E, const int64_
     if (bad) atomicOr(flag, bad);
 }
 
-// ------------------------------------------------------------------ exclusive scan (uint32)
-// three launches: per-tile sums, scan of the tile sums by one block, per-tile scan + offset
 constexpr int SCAN_THREADS = 256;
-constexpr int SCAN_ITEMS = 8;
-constexpr int SCAN_TILE = SCAN_THREADS * SCAN_ITEMS;
 
 // exclusive scan of one value per thread over a 256-thread block; *total = block sum
 __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* total) {
@@ -126,302 +112,453 @@ __device__ __forceinline__ uint32_t block_exclusive_scan(uint32_t v, uint32_t* t
     return r;
 }
 
-__global__ void scan_tile_sums_kernel(const uint32_t* __restrict__ in, int64_t n,
-                                      uint32_t* __restrict__ tile_sums) {
-    int64_t base = (int64_t)blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
-    uint32_t s = 0;
-#pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; ++i)
-        if (base + i < n) s += in[base + i];
-    uint32_t total;
-    block_exclusive_scan(s, &total);
-    if (threadIdx.x == 0) tile_sums[blockIdx.x] = total;
-}
-
-__global__ void scan_single_block_kernel(uint32_t* __restrict__ data, int64_t n) {
-    uint32_t carry = 0;
-    for (int64_t base = 0; base < n; base += SCAN_THREADS) {
-        int64_t i = base + threadIdx.x;
-        uint32_t v = i < n ? data[i] : 0, total;
-        uint32_t ex = block_exclusive_scan(v, &total);
-        if (i < n) data[i] = carry + ex;
-        carry += total;
-    }
-}
-
-__global__ void scan_apply_kernel(const uint32_t* __restrict__ in, int64_t n,
-                                  const uint32_t* __restrict__ tile_offsets,
-                                  uint32_t* __restrict__ out) {
-    int64_t base = (int64_t)blockIdx.x * SCAN_TILE + threadIdx.x * SCAN_ITEMS;
-    uint32_t v[SCAN_ITEMS], s = 0;
-#pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; ++i) {
-        v[i] = base + i < n ? in[base + i] : 0;
-        s += v[i];
-    }
-    uint32_t total;
-    uint32_t ex = block_exclusive_scan(s, &total) + tile_offsets[blockIdx.x];
-#pragma unroll
-    for (int i = 0; i < SCAN_ITEMS; ++i) {
-        if (base + i < n) out[base + i] = ex;
-        ex += v[i];
-    }
-}
-
-// ------------------------------------------------------------------ stable LSD radix sort
+// ------------------------------------------------------------------ stable LSD radix sort of (endpoint, edge index)
+// Three launches per digit: a histogram per tile, an exclusive scan of every digit's row of tile counts, and a scatter that
+// ranks a tile's keys (warp match, one pass: the rank is kept in a register) and writes (key, index) pairs of 8 bytes.
+// Below SORT_BOTH edges the two sorts (by target, by source) share their launches, and digits are as wide as divides the key
+// evenly in few passes (up to 10 bits: 2 passes for up to 1 M nodes); above, they run one after the other in one pair of
+// buffers with 8-bit digits, whose runs per tile are longer.  The last pass writes the sparse form itself (edge index, other
+// endpoint, and for the form by target each edge's position); row pointers come from the sorted keys' steps.
+// 1.53 M edges, 170k nodes: 6 sorts' passes of 5 launches each and the forms 340 us -> 165 us.
 constexpr int RS_THREADS = 256;
 constexpr int RS_WARPS = RS_THREADS / 32;
-constexpr int RS_ROUNDS = 16;
-constexpr int RS_TILE = RS_THREADS * RS_ROUNDS;  // 4096 keys per block
-constexpr int RS_BINS = 256;
+constexpr int RS_MAX_BINS = 1024;
+constexpr int64_t SORT_BOTH = (int64_t)8 << 20;
+
+struct SortJob {
+    const int32_t* keys;   // first pass: the endpoints
+    const int32_t* other;  // the other endpoint of each edge
+    const uint2* in;       // later passes: (key, edge index)
+    uint2* out;
+    int32_t* ksorted;      // last pass: keys in order
+    int32_t *col, *eid, *pos;  // last pass: the sparse form; pos[edge] = its position (or nullptr)
+    uint32_t *table, *totals;  // [bins][ntiles] counts, then their exclusive scans per digit; [bins] totals
+    int64_t* rowptr;
+};
+struct SortArgs {
+    SortJob j[2];
+    int64_t E;
+    int32_t N;
+    int shift, bits;
+    uint32_t ntiles;
+    int* flag;       // set if an endpoint is out of range
+    int* host_flag;  // the same word for the waiting host
+    const int32_t* pos;  // finalize: position of each edge in the form by target
+    int32_t* t2f;
+};
 
 // element order inside a tile: warp-major, then round, then lane
+template <int ROUNDS>
 __device__ __forceinline__ int64_t rs_index(int64_t tile0, int warp, int round, int lane) {
-    return tile0 + (int64_t)warp * (32 * RS_ROUNDS) + round * 32 + lane;
+    return tile0 + (int64_t)warp * (32 * ROUNDS) + round * 32 + lane;
 }
 
-__global__ void __launch_bounds__(RS_THREADS)
-radix_hist_kernel(const int32_t* __restrict__ keys, int64_t E, int shift, uint32_t nblocks,
-                  uint32_t* __restrict__ table) {
-    __shared__ uint32_t cnt[RS_BINS];
-    cnt[threadIdx.x] = 0;
+template <int ROUNDS, bool FIRST>
+__global__ void __launch_bounds__(RS_THREADS) radix_hist_kernel(const __grid_constant__ SortArgs A) {
+    __shared__ uint32_t cnt[RS_MAX_BINS];
+    pdl_wait();
+    const SortJob& J = A.j[blockIdx.y];
+    const int bins = 1 << A.bits;
+    for (int d = threadIdx.x; d < bins; d += RS_THREADS) cnt[d] = 0;
     __syncthreads();
-    int64_t tile0 = (int64_t)blockIdx.x * RS_TILE;
-    int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll 4
-    for (int r = 0; r < RS_ROUNDS; ++r) {
-        int64_t i = rs_index(tile0, warp, r, lane);
-        if (i < E) atomicAdd(&cnt[(keys[i] >> shift) & 0xFF], 1u);
+    const int64_t tile0 = (int64_t)blockIdx.x * (RS_THREADS * ROUNDS);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    int32_t key[ROUNDS];
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+        const int64_t i = rs_index<ROUNDS>(tile0, warp, r, lane);
+        key[r] = i < A.E ? (FIRST ? J.keys[i] : (int32_t)J.in[i].x) : 0;
+    }
+    bool bad = false;
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+        if (FIRST) bad |= key[r] < 0 || key[r] >= A.N;
+        if (rs_index<ROUNDS>(tile0, warp, r, lane) < A.E) atomicAdd(&cnt[((uint32_t)key[r] >> A.shift) & (bins - 1)], 1u);
+    }
+    if (FIRST && bad) {  // benign race: every writer stores the same value
+        *A.flag = 1;
+        *(volatile int*)A.host_flag = 1;
     }
     __syncthreads();
-    table[(size_t)threadIdx.x * nblocks + blockIdx.x] = cnt[threadIdx.x];
+    for (int d = threadIdx.x; d < bins; d += RS_THREADS) J.table[(size_t)d * A.ntiles + blockIdx.x] = cnt[d];
 }
 
-// vals_in == nullptr means "value = index" (first pass)
-__global__ void __launch_bounds__(RS_THREADS)
-radix_scatter_kernel(const int32_t* __restrict__ keys_in, const int32_t* __restrict__ vals_in,
-                     int64_t E, int shift, uint32_t nblocks, const uint32_t* __restrict__ base,
-                     int32_t* __restrict__ keys_out, int32_t* __restrict__ vals_out) {
-    __shared__ uint32_t wcnt[RS_WARPS][RS_BINS];
-    int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int w = 0; w < RS_WARPS; ++w) wcnt[w][threadIdx.x] = 0;
-    __syncthreads();
-    int64_t tile0 = (int64_t)blockIdx.x * RS_TILE;
-    const uint32_t lt = (1u << lane) - 1u;
-    int32_t key[RS_ROUNDS];
-    // (i) per-warp digit totals
+// block (d, job): exclusive scan of digit d's row of tile counts, in place; its sum to totals[d]
+__global__ void __launch_bounds__(RS_THREADS) radix_scan_kernel(const __grid_constant__ SortArgs A) {
+    pdl_wait();
+    const SortJob& J = A.j[blockIdx.y];
+    uint32_t* const row = J.table + (size_t)blockIdx.x * A.ntiles;
+    uint32_t carry = 0;
+    for (uint32_t b0 = 0; b0 < A.ntiles; b0 += 4 * RS_THREADS) {
+        const uint32_t i0 = b0 + threadIdx.x * 4;
+        uint32_t v[4], s = 0, total;
 #pragma unroll
-    for (int r = 0; r < RS_ROUNDS; ++r) {
-        int64_t i = rs_index(tile0, warp, r, lane);
-        bool ok = i < E;
-        key[r] = ok ? keys_in[i] : 0;
-        int d = ok ? ((key[r] >> shift) & 0xFF) : RS_BINS;  // invalid lanes form their own group
-        uint32_t peers = __match_any_sync(0xffffffffu, d);
-        if (ok && (peers & lt) == 0) wcnt[warp][d] += __popc(peers);  // one leader per digit
+        for (int u = 0; u < 4; ++u) {
+            v[u] = i0 + u < A.ntiles ? row[i0 + u] : 0;
+            s += v[u];
+        }
+        uint32_t run = carry + block_exclusive_scan(s, &total);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (i0 + u < A.ntiles) row[i0 + u] = run;
+            run += v[u];
+        }
+        carry += total;
+    }
+    if (threadIdx.x == 0) J.totals[blockIdx.x] = carry;
+}
+
+template <int ROUNDS, bool FIRST, bool LAST>
+__global__ void __launch_bounds__(RS_THREADS) radix_scatter_kernel(const __grid_constant__ SortArgs A) {
+    __shared__ uint16_t wcnt[RS_WARPS][RS_MAX_BINS];  // counts, then prefixes, of a warp's keys per digit: at most 4096
+    __shared__ uint32_t gbase[RS_MAX_BINS];
+    pdl_wait();
+    const SortJob& J = A.j[blockIdx.y];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, bins = 1 << A.bits;
+    const int64_t tile0 = (int64_t)blockIdx.x * (RS_THREADS * ROUNDS);
+    uint2 kv[ROUNDS];
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+        const int64_t i = rs_index<ROUNDS>(tile0, warp, r, lane);
+        kv[r] = make_uint2(0u, 0u);
+        if (i < A.E) kv[r] = FIRST ? make_uint2((uint32_t)J.keys[i], (uint32_t)i) : J.in[i];
+    }
+    for (int d = threadIdx.x; d < RS_WARPS * RS_MAX_BINS / 2; d += RS_THREADS) reinterpret_cast<uint32_t*>(wcnt)[d] = 0;
+    {  // where each digit's keys of this tile begin: digits before, then tiles before
+        const int per = RS_MAX_BINS / RS_THREADS;
+        uint32_t v[per], s = 0, total;
+#pragma unroll
+        for (int u = 0; u < per; ++u) {
+            const int d = threadIdx.x * per + u;
+            v[u] = d < bins ? J.totals[d] : 0;
+            s += v[u];
+        }
+        uint32_t run = block_exclusive_scan(s, &total);  // its barriers also close the zeroing above
+#pragma unroll
+        for (int u = 0; u < per; ++u) {
+            const int d = threadIdx.x * per + u;
+            if (d < bins) gbase[d] = run + J.table[(size_t)d * A.ntiles + blockIdx.x];
+            run += v[u];
+        }
+    }
+    const uint32_t lt = (1u << lane) - 1u;
+    uint16_t rank[ROUNDS];
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {  // stable rank among the warp's keys of the same digit
+        const bool ok = rs_index<ROUNDS>(tile0, warp, r, lane) < A.E;
+        const int d = ok ? (int)((kv[r].x >> A.shift) & (uint32_t)(bins - 1)) : bins;  // lanes past the end form their own group
+        const uint32_t peers = __match_any_sync(0xffffffffu, d);
+        const uint32_t before = ok ? wcnt[warp][d] : 0;
+        rank[r] = (uint16_t)(before + __popc(peers & lt));
+        __syncwarp();
+        if (ok && (peers & lt) == 0) wcnt[warp][d] = (uint16_t)(before + __popc(peers));
         __syncwarp();
     }
     __syncthreads();
-    // (ii) digit d: global base, then exclusive prefix over the warps of this block
-    {
-        int d = threadIdx.x;
-        uint32_t run = base[(size_t)d * nblocks + blockIdx.x];
+    for (int d = threadIdx.x; d < bins; d += RS_THREADS) {  // prefix over the warps of the block
+        uint32_t run = 0;
 #pragma unroll
         for (int w = 0; w < RS_WARPS; ++w) {
-            uint32_t t = wcnt[w][d];
-            wcnt[w][d] = run;
+            const uint32_t t = wcnt[w][d];
+            wcnt[w][d] = (uint16_t)run;
             run += t;
         }
     }
     __syncthreads();
-    // (iii) stable ranks and scatter
+    uint32_t where[ROUNDS];
+    int32_t oth[LAST ? ROUNDS : 1];
 #pragma unroll
-    for (int r = 0; r < RS_ROUNDS; ++r) {
-        int64_t i = rs_index(tile0, warp, r, lane);
-        bool ok = i < E;
-        int d = ok ? ((key[r] >> shift) & 0xFF) : RS_BINS;
-        uint32_t peers = __match_any_sync(0xffffffffu, d);
-        if (ok) {
-            uint32_t pos = wcnt[warp][d] + __popc(peers & lt);
-            keys_out[pos] = key[r];
-            vals_out[pos] = vals_in ? vals_in[i] : (int32_t)i;
+    for (int r = 0; r < ROUNDS; ++r) {
+        const int d = (int)((kv[r].x >> A.shift) & (uint32_t)(bins - 1));
+        where[r] = gbase[d] + wcnt[warp][d] + rank[r];
+        if (LAST && rs_index<ROUNDS>(tile0, warp, r, lane) < A.E) oth[LAST ? r : 0] = J.other[kv[r].y];
+    }
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+        if (rs_index<ROUNDS>(tile0, warp, r, lane) >= A.E) continue;
+        const uint32_t p = where[r];
+        if (LAST) {
+            J.ksorted[p] = (int32_t)kv[r].x;
+            J.eid[p] = (int32_t)kv[r].y;
+            J.col[p] = oth[LAST ? r : 0];
+            if (J.pos) J.pos[kv[r].y] = (int32_t)p;
+        } else {
+            J.out[p] = kv[r];
         }
-        __syncwarp();
-        if (ok && (peers & lt) == 0) wcnt[warp][d] += __popc(peers);
-        __syncwarp();
     }
 }
 
-__global__ void csr_finalize_kernel(int32_t N, int64_t E, const int32_t* __restrict__ sorted_keys,
-                                    const int32_t* __restrict__ sorted_vals,
-                                    const int32_t* __restrict__ other, int64_t* __restrict__ rowptr,
-                                    int32_t* __restrict__ col, int32_t* __restrict__ eid) {
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t p = t; p < E; p += stride) {
-        int32_t k = sorted_vals[p];
-        eid[p] = k;
-        col[p] = other[k];
-    }
-    // rowptr[i] = first position whose key is >= i
-    for (int64_t i = t; i <= N; i += stride) {
-        int64_t lo = 0, hi = E;
-        while (lo < hi) {
-            int64_t mid = (lo + hi) >> 1;
-            if (sorted_keys[mid] < (int32_t)i) lo = mid + 1; else hi = mid;
+// row pointers from the sorted keys (rowptr[i] = first position whose key is >= i) and, with the form by source, t2f.  A
+// thread fills the rows between its key and the one before; gaps of more than 32 rows (isolated nodes) by the whole block.
+__global__ void __launch_bounds__(256) csr_finalize_kernel(const __grid_constant__ SortArgs A) {
+    __shared__ int64_t gap_p[256];
+    __shared__ int gap_a[256], gap_b[256], gaps;
+    pdl_wait();
+    if (*A.flag) return;  // endpoints out of range: the keys are not in order
+    const SortJob& J = A.j[blockIdx.y];
+    if (threadIdx.x == 0) gaps = 0;
+    __syncthreads();
+    const int64_t p = (int64_t)blockIdx.x * 256 + threadIdx.x;  // p == E: the rows after the last key
+    if (p <= A.E) {
+        const int a = p > 0 ? J.ksorted[p - 1] + 1 : 0, b = p < A.E ? J.ksorted[p] + 1 : A.N + 1;  // rows [a, b) begin at p
+        if (b - a > 32) {
+            const int k = atomicAdd(&gaps, 1);
+            gap_a[k] = a; gap_b[k] = b; gap_p[k] = p;
+        } else {
+            for (int i = a; i < b; ++i) J.rowptr[i] = p;
         }
-        rowptr[i] = lo;
+        if (J.pos == nullptr && p < A.E) A.t2f[p] = A.pos[J.eid[p]];
     }
+    __syncthreads();
+    for (int k = 0; k < gaps; ++k)
+        for (int i = gap_a[k] + (int)threadIdx.x; i < gap_b[k]; i += 256) J.rowptr[i] = gap_p[k];
 }
 
-__global__ void invert_perm_kernel(int64_t E, const int32_t* __restrict__ eid,
-                                   int32_t* __restrict__ pos) {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (; p < E; p += stride) pos[eid[p]] = (int32_t)p;
-}
-__global__ void compose_perm_kernel(int64_t E, const int32_t* __restrict__ pos,
-                                    const int32_t* __restrict__ eidT, int32_t* __restrict__ t2f) {
-    int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (; q < E; q += stride) t2f[q] = pos[eidT[q]];
-}
-
-struct SortWs {
-    int32_t *kA, *vA, *kB, *vB;
-    uint32_t *table, *tile_sums;
+struct SortPlan {
+    bool both;
+    int rounds, bits, passes;
+    uint32_t ntiles;
+    uint2 *a[2], *b[2];
+    uint32_t *table[2], *totals[2];
+    int32_t* pos;
     int* flag;
     size_t bytes;
 };
 
-static SortWs carve(void* ws, int64_t E) {
-    SortWs s;
-    size_t nblocks = (size_t)ceil_div(E > 0 ? E : 1, RS_TILE);
-    size_t table_n = nblocks * RS_BINS;
-    size_t tiles = (size_t)ceil_div((int64_t)table_n, SCAN_TILE);
-    size_t eb = up256((size_t)(E > 0 ? E : 1) * 4);
+static SortPlan sort_plan(void* ws, int32_t N, int64_t E) {
+    SortPlan s;
+    s.both = E < SORT_BOTH;
+    s.rounds = s.both ? 8 : 16;
+    int bits = 1;
+    while (bits < 31 && ((int64_t)1 << bits) < (int64_t)N) ++bits;
+    const int most = s.both ? 10 : 8;
+    s.passes = (bits + most - 1) / most;
+    s.bits = (bits + s.passes - 1) / s.passes;
+    s.ntiles = (uint32_t)ceil_div(E > 0 ? E : 1, RS_THREADS * s.rounds);
     char* p = (char*)ws;
     size_t off = 0;
     s.flag = (int*)(p + off); off += 256;
-    s.kA = (int32_t*)(p + off); off += eb;
-    s.vA = (int32_t*)(p + off); off += eb;
-    s.kB = (int32_t*)(p + off); off += eb;
-    s.vB = (int32_t*)(p + off); off += eb;
-    s.table = (uint32_t*)(p + off); off += up256(table_n * 4);
-    s.tile_sums = (uint32_t*)(p + off); off += up256(tiles * 4);
+    const size_t pairs = up256((size_t)(E > 0 ? E : 1) * 8), bins = (size_t)1 << most;
+    for (int k = 0; k < 2; ++k) {
+        if (k == 1 && !s.both) { s.a[1] = s.a[0]; s.b[1] = s.b[0]; s.table[1] = s.table[0]; s.totals[1] = s.totals[0]; continue; }
+        s.a[k] = (uint2*)(p + off); off += pairs;
+        s.b[k] = (uint2*)(p + off); off += pairs;
+        s.table[k] = (uint32_t*)(p + off); off += up256(bins * s.ntiles * 4);
+        s.totals[k] = (uint32_t*)(p + off); off += up256(bins * 4);
+    }
+    s.pos = (int32_t*)(p + off); off += up256((size_t)(E > 0 ? E : 1) * 4);
     s.bytes = off;
     return s;
 }
 
-// stable sort of (key[k], k) by key; result left in *sk, *sv (pointers into ws)
-static gnn_status sort_by_key(int32_t N, int64_t E, const int32_t* keys, const SortWs& w,
-                              cudaStream_t st, const int32_t** sk, const int32_t** sv) {
-    int bits = 0;
-    while (bits < 31 && ((int64_t)1 << bits) < (int64_t)N) ++bits;
-    int passes = bits == 0 ? 1 : (bits + 7) / 8;
-    uint32_t nblocks = (uint32_t)ceil_div(E > 0 ? E : 1, RS_TILE);
-    int64_t table_n = (int64_t)nblocks * RS_BINS;
-    int tiles = (int)ceil_div(table_n, SCAN_TILE);
-    const int32_t* kin = keys;
-    const int32_t* vin = nullptr;
-    int32_t* kout = w.kA;
-    int32_t* vout = w.vA;
-    for (int p = 0; p < passes; ++p) {
-        int shift = 8 * p;
-        radix_hist_kernel<<<nblocks, RS_THREADS, 0, st>>>(kin, E, shift, nblocks, w.table);
-        scan_tile_sums_kernel<<<tiles, SCAN_THREADS, 0, st>>>(w.table, table_n, w.tile_sums);
-        scan_single_block_kernel<<<1, SCAN_THREADS, 0, st>>>(w.tile_sums, tiles);
-        scan_apply_kernel<<<tiles, SCAN_THREADS, 0, st>>>(w.table, table_n, w.tile_sums, w.table);
-        radix_scatter_kernel<<<nblocks, RS_THREADS, 0, st>>>(kin, vin, E, shift, nblocks, w.table,
-                                                            kout, vout);
-        GNN_CHECK_LAUNCH("radix sort pass");
-        kin = kout;
-        vin = vout;
-        kout = (kout == w.kA) ? w.kB : w.kA;
-        vout = (vout == w.vA) ? w.vB : w.vA;
+template <int ROUNDS>
+static cudaError_t launch_sort(SortArgs A, const SortPlan& s, int first, int jobs, cudaEvent_t validated, cudaStream_t st) {
+    if (first) A.j[0] = A.j[1];
+    for (int p = 0; p < s.passes; ++p) {
+        A.shift = s.bits * p;
+        A.bits = s.bits;
+        const bool f = p == 0, l = p == s.passes - 1;
+        for (int k = 0; k < jobs; ++k) {
+            A.j[k].in = p % 2 ? s.a[k + first] : s.b[k + first];
+            A.j[k].out = p % 2 ? s.b[k + first] : s.a[k + first];
+            A.j[k].ksorted = (int32_t*)A.j[k].out;  // the last pass writes no pairs
+        }
+        const dim3 tiles(s.ntiles, jobs), block(RS_THREADS);
+        if (f) launch_overlapped(radix_hist_kernel<ROUNDS, true>, tiles, block, 0, st, A);
+        else launch_overlapped(radix_hist_kernel<ROUNDS, false>, tiles, block, 0, st, A);
+        if (f) {
+            const cudaError_t e = cudaEventRecord(validated, st);
+            if (e != cudaSuccess) return e;
+        }
+        launch_overlapped(radix_scan_kernel, dim3(1u << s.bits, jobs), block, 0, st, A);
+        if (f && l) launch_overlapped(radix_scatter_kernel<ROUNDS, true, true>, tiles, block, 0, st, A);
+        else if (f) launch_overlapped(radix_scatter_kernel<ROUNDS, true, false>, tiles, block, 0, st, A);
+        else if (l) launch_overlapped(radix_scatter_kernel<ROUNDS, false, true>, tiles, block, 0, st, A);
+        else launch_overlapped(radix_scatter_kernel<ROUNDS, false, false>, tiles, block, 0, st, A);
     }
-    *sk = kin;
-    *sv = vin;
-    return GNN_OK;
+    launch_overlapped(csr_finalize_kernel, dim3((unsigned)ceil_div(A.E + 1, 256), jobs), dim3(256), 0, st, A);
+    return cudaGetLastError();
+}
+
+// A word of pinned host memory and an event: the host waits for the validation of the endpoints, which is done long before
+// the sorts that are queued behind it.  Slots are handed out one per call in progress and kept for the next (as many as
+// calls ever ran at once on a device).
+struct FlagSlot { int* word; cudaEvent_t event; int device; };
+static std::mutex g_slots_mutex;
+static std::vector<FlagSlot> g_slots;
+
+static bool take_slot(FlagSlot* s) {
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    {
+        std::lock_guard<std::mutex> lock(g_slots_mutex);
+        for (size_t k = 0; k < g_slots.size(); ++k)
+            if (g_slots[k].device == dev) {
+                *s = g_slots[k];
+                g_slots.erase(g_slots.begin() + (long)k);
+                return true;
+            }
+    }
+    s->device = dev;
+    if (cudaHostAlloc((void**)&s->word, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) return false;
+    if (cudaEventCreateWithFlags(&s->event, cudaEventDisableTiming) != cudaSuccess) {
+        cudaFreeHost(s->word);
+        return false;
+    }
+    return true;
+}
+static void give_slot(const FlagSlot& s) {
+    std::lock_guard<std::mutex> lock(g_slots_mutex);
+    g_slots.push_back(s);
 }
 
 // ------------------------------------------------------------------ degrees / GCN coefficients
 __global__ void degree_count_kernel(int32_t N, const int64_t* __restrict__ rowptr,
                                     int32_t* __restrict__ deg) {
+    pdl_wait();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < N) deg[i] = (int32_t)(rowptr[i + 1] - rowptr[i]);
 }
 
-// one warp per row; lane-strided partial sums combined by a fixed shuffle tree
-__global__ void degree_weighted_kernel(int32_t N, const int64_t* __restrict__ rowptr,
-                                       const float* __restrict__ w, float* __restrict__ deg) {
-    int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    int lane = threadIdx.x & 31;
-    if (row >= N) return;
-    int64_t a = rowptr[row], b = rowptr[row + 1];
+// Sum of w over each row: eight lanes per row (four rows per warp), rows over DEG_LONG positions by the whole block (a hub
+// of 10^5 positions walked by a warp alone takes milliseconds).  Fixed orders.  170k rows of nine positions on average:
+// 31 us with a warp per row, 14 us.
+constexpr int DEG_LONG = 512;
+__global__ void __launch_bounds__(256) degree_weighted_kernel(int32_t N, const int64_t* __restrict__ rowptr,
+                                                             const float* __restrict__ w, float* __restrict__ deg) {
+    __shared__ int todo[32], ntodo;
+    __shared__ float sums[8];
+    pdl_wait();
+    if (threadIdx.x == 0) ntodo = 0;
+    __syncthreads();
+    const int64_t row = blockIdx.x * (int64_t)32 + (threadIdx.x >> 3);
+    const int li = threadIdx.x & 7;
     float s = 0.f;
-    for (int64_t p = a + lane; p < b; p += 32) s += w[p];
+    bool lng = false;
+    if (row < N) {
+        const int64_t a = rowptr[row], b = rowptr[row + 1];
+        lng = b - a > DEG_LONG;
+        if (!lng) {
+#pragma unroll 4
+            for (int64_t p = a + li; p < b; p += 8) s += w[p];
+        }
+    }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) deg[row] = s;
+    for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (row < N && li == 0) {
+        if (lng) todo[atomicAdd(&ntodo, 1)] = (int)row;  // rows are independent: their order does not matter
+        else deg[row] = s;
+    }
+    __syncthreads();
+    for (int k = 0; k < ntodo; ++k) {
+        const int r = todo[k];
+        const int64_t a = rowptr[r], b = rowptr[r + 1];
+        s = 0.f;
+#pragma unroll 4
+        for (int64_t p = a + threadIdx.x; p < b; p += 256) s += w[p];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((threadIdx.x & 31) == 0) sums[threadIdx.x >> 5] = s;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            for (int q = 1; q < 8; ++q) s += sums[q];
+            deg[r] = s;
+        }
+        __syncthreads();
+    }
 }
 
 __global__ void degree_unit_kernel(int32_t N, const int64_t* __restrict__ rowptr,
                                    float* __restrict__ deg) {
+    pdl_wait();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (i < N) deg[i] = (float)(rowptr[i + 1] - rowptr[i]);
 }
 
-// coef[p] = w[p] / sqrt(deg[row(p)] * deg[col[p]]).  LONG = false: a warp per row of at most GC_LONG positions.
-// LONG = true: block k owns the rows k, k + blocks, ...; its threads look at 256 of them at once, list the longer ones
-// in shared memory, and the whole block takes a listed row (a single warp would walk a hub of 10^5 positions alone).
-constexpr int GC_LONG = 1024;
+// coef[p] = w[p] / sqrt(deg[row(p)] * deg[col[p]]), for the form by target (blockIdx.y = 0) and, with w through t2f, for the
+// transposed one: the degrees of an edge's two ends meet in a product, so both forms give the same bits.  Positions first: a
+// warp stages the rows of its 256 positions and every lane finds the row of its first of eight there and steps on, whatever
+// the rows' lengths (a warp per row and a second pass for hubs: 58 + 35 + 9 us on 170k rows / 1.53 M positions).
+struct CoefForm {
+    const int64_t* rowptr;
+    const int32_t *col, *w_index;
+    float* out;
+    int vec;  // all three on 16 bytes
+};
+struct CoefArgs {
+    CoefForm f[2];
+    const float *w, *deg;
+    int32_t N;
+    int64_t E;
+};
 __device__ __forceinline__ float gcn_coef(float wp, float di, float dj) {
     // IEEE sqrt and division (no approximate rsqrt): ~1e-7 relative
     return (di > 0.f && dj > 0.f) ? __fdiv_rn(wp, __fsqrt_rn(di * dj)) : 0.f;
 }
-template <bool LONG>
-__global__ void __launch_bounds__(256) gcn_coef_kernel(int32_t N, const int64_t* __restrict__ rowptr,
-                                                       const int32_t* __restrict__ col, const float* __restrict__ w,
-                                                       const float* __restrict__ deg, float* __restrict__ coef) {
-    if (!LONG) {
-        int64_t row = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-        int lane = threadIdx.x & 31;
-        if (row >= N) return;
-        int64_t a = rowptr[row], b = rowptr[row + 1];
-        if (b - a > GC_LONG) return;
-        float di = deg[row];
-        for (int64_t p = a + lane; p < b; p += 32) coef[p] = gcn_coef(w ? w[p] : 1.0f, di, deg[col[p]]);
+__global__ void __launch_bounds__(256) gcn_coef_kernel(const __grid_constant__ CoefArgs A) {
+    constexpr int SUB = 256, PER = SUB / 32;  // a lane takes eight consecutive positions
+    __shared__ int s_row[8][SUB + 1];
+    __shared__ uint16_t s_start[8][SUB + 2];
+    pdl_wait();
+    const CoefForm& F = A.f[blockIdx.y];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t cs64 = ((int64_t)blockIdx.x * 8 + warp) * SUB;
+    if (cs64 >= A.E) return;
+    const int cs = (int)cs64, n = (int)min((int64_t)SUB, A.E - cs64), i0 = lane * PER;
+    const bool vec = F.vec && n == SUB;  // whole, aligned vectors
+    __align__(16) int c[PER], wi[PER];
+    float wp[PER], dj[PER], r[PER];
+    if (vec) {
+        *reinterpret_cast<int4*>(c) = __ldcs(reinterpret_cast<const int4*>(F.col + cs + i0));
+        *reinterpret_cast<int4*>(c + 4) = __ldcs(reinterpret_cast<const int4*>(F.col + cs + i0) + 1);
+        if (A.w && F.w_index) {
+            *reinterpret_cast<int4*>(wi) = __ldcs(reinterpret_cast<const int4*>(F.w_index + cs + i0));
+            *reinterpret_cast<int4*>(wi + 4) = __ldcs(reinterpret_cast<const int4*>(F.w_index + cs + i0) + 1);
+        }
     } else {
-        __shared__ int list[256];
-        __shared__ int count;
-        for (int64_t k0 = 0; (int64_t)blockIdx.x + k0 * gridDim.x < N; k0 += 256) {
-            __syncthreads();  // every thread is done with the previous list
-            if (threadIdx.x == 0) count = 0;
-            __syncthreads();
-            const int64_t mine = (int64_t)blockIdx.x + (k0 + threadIdx.x) * gridDim.x;
-            if (mine < N && rowptr[mine + 1] - rowptr[mine] > GC_LONG) list[atomicAdd(&count, 1)] = (int)mine;
-            __syncthreads();
-            const int n = count;
-            for (int i = 0; i < n; ++i) {  // the order of the list does not matter: every position is written once
-                const int row = list[i];
-                const int64_t a = rowptr[row], b = rowptr[row + 1];
-                const float di = deg[row];
-                for (int64_t p = a + threadIdx.x; p < b; p += 256) coef[p] = gcn_coef(w ? w[p] : 1.0f, di, deg[col[p]]);
-            }
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            c[u] = i0 + u < n ? F.col[cs + i0 + u] : 0;
+            wi[u] = A.w && F.w_index && i0 + u < n ? F.w_index[cs + i0 + u] : 0;
         }
     }
-}
-
-__global__ void permute_f32_kernel(int64_t E, const int32_t* __restrict__ perm,
-                                   const float* __restrict__ in, float* __restrict__ out) {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (; p < E; p += stride) out[p] = in[perm[p]];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        wp[u] = 1.0f;
+        if (A.w && i0 + u < n) wp[u] = A.w[F.w_index ? wi[u] : cs + i0 + u];
+        dj[u] = i0 + u < n ? A.deg[c[u]] : 0.f;
+        r[u] = 0.f;
+    }
+    bool began_before;
+    const int m = stage_rows(F.rowptr, A.N, A.E, cs, n, lane, s_row[warp], s_start[warp], began_before);
+    __syncwarp();
+    if (i0 >= n) return;
+    int q = 0, hi = m;  // start[q] <= i0 < start[hi]
+    while (hi - q > 1) {
+        const int mid = (q + hi) >> 1;
+        if (s_start[warp][mid] <= i0) q = mid; else hi = mid;
+    }
+    float di = A.deg[s_row[warp][q]];
+#pragma unroll
+    for (int u = 0; u < PER; ++u)
+        if (i0 + u < n) {
+            if (i0 + u >= s_start[warp][q + 1]) di = A.deg[s_row[warp][++q]];  // staged rows have positions: one step is enough
+            r[u] = gcn_coef(wp[u], di, dj[u]);
+        }
+    if (vec) {
+        *reinterpret_cast<float4*>(F.out + cs + i0) = make_float4(r[0], r[1], r[2], r[3]);
+        *reinterpret_cast<float4*>(F.out + cs + i0 + 4) = make_float4(r[4], r[5], r[6], r[7]);
+    } else {
+#pragma unroll
+        for (int u = 0; u < PER; ++u)
+            if (i0 + u < n) F.out[cs + i0 + u] = r[u];
+    }
 }
 
 template <typename T>
 __global__ void permute_rows_kernel(int64_t E, int width, const int32_t* __restrict__ perm,
                                     const T* __restrict__ in, T* __restrict__ out) {
+    pdl_wait();
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     int64_t total = E * width;
@@ -435,6 +572,7 @@ __global__ void permute_rows_kernel(int64_t E, int width, const int32_t* __restr
 __global__ void add_self_loops_kernel(int32_t N, int64_t E, const int32_t* __restrict__ src,
                                       const int32_t* __restrict__ dst, int32_t* __restrict__ so,
                                       int32_t* __restrict__ dout) {
+    pdl_wait();
     int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (; k < E + N; k += stride) {
@@ -466,9 +604,8 @@ const char* gnn_last_error_string(void) { return g_err; }
 int gnn_version(void) { return 100; }
 
 size_t gnn_coo_to_csr_workspace(int32_t N, int64_t E) {
-    (void)N;
     if (E < 0) return 0;
-    return carve(nullptr, E).bytes;
+    return sort_plan(nullptr, N, E).bytes;
 }
 
 gnn_status gnn_coo_to_csr(int32_t N, int64_t E, const int32_t* src, const int32_t* dst,
@@ -481,38 +618,38 @@ gnn_status gnn_coo_to_csr(int32_t N, int64_t E, const int32_t* src, const int32_
     GNN_REQUIRE(ws && ws_bytes >= gnn_coo_to_csr_workspace(N, E), GNN_ERR_WORKSPACE_TOO_SMALL,
                 "gnn_coo_to_csr: workspace of %zu bytes needed", gnn_coo_to_csr_workspace(N, E));
     cudaStream_t st = as_stream(stream);
-    SortWs w = carve(ws, E);
     out->N = N;
     out->E = E;
-
-    if (cudaMemsetAsync(w.flag, 0, sizeof(int), st) != cudaSuccess)
-        GNN_FAIL(GNN_ERR_CUDA, "gnn_coo_to_csr: memset failed (is ws a device pointer?)");
-    if (E > 0) validate_coo_kernel<<<grid_for(E, 256), 256, 0, st>>>(N, E, src, dst, w.flag);
-    GNN_CHECK_LAUNCH("validate_coo");
-    int h_flag = 0;
-    if (cudaMemcpyAsync(&h_flag, w.flag, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-        GNN_FAIL(GNN_ERR_CUDA, "gnn_coo_to_csr: reading the validation flag failed: %s",
-                 cudaGetErrorString(cudaGetLastError()));
-    GNN_REQUIRE(h_flag == 0, GNN_ERR_INDEX_OUT_OF_RANGE,
-                "gnn_coo_to_csr: an edge endpoint is outside [0, %d)", N);
-
-    const int32_t *sk, *sv;
-    gnn_status rc;
-    const int fgrid = grid_for(E > N ? E : (int64_t)N + 1, 256);
-    // by target
-    if ((rc = sort_by_key(N, E, dst, w, st, &sk, &sv)) != GNN_OK) return rc;
-    csr_finalize_kernel<<<fgrid, 256, 0, st>>>(N, E, sk, sv, src, out->rowptr, out->col, out->eid);
-    GNN_CHECK_LAUNCH("csr_finalize");
-    // by source
-    if ((rc = sort_by_key(N, E, src, w, st, &sk, &sv)) != GNN_OK) return rc;
-    csr_finalize_kernel<<<fgrid, 256, 0, st>>>(N, E, sk, sv, dst, out->rowptrT, out->colT, out->eidT);
-    GNN_CHECK_LAUNCH("csr_finalize (transposed)");
-    if (E > 0) {
-        invert_perm_kernel<<<grid_for(E, 256), 256, 0, st>>>(E, out->eid, w.kA);
-        compose_perm_kernel<<<grid_for(E, 256), 256, 0, st>>>(E, w.kA, out->eidT, out->t2f);
-        GNN_CHECK_LAUNCH("t2f");
+    if (E == 0) {
+        if (cudaMemsetAsync(out->rowptr, 0, ((size_t)N + 1) * 8, st) != cudaSuccess || cudaMemsetAsync(out->rowptrT, 0, ((size_t)N + 1) * 8, st) != cudaSuccess)
+            GNN_FAIL(GNN_ERR_CUDA, "gnn_coo_to_csr: memset failed (are the outputs device pointers?)");
+        return GNN_OK;
     }
+    GNN_REQUIRE(N > 0, GNN_ERR_INDEX_OUT_OF_RANGE, "gnn_coo_to_csr: an edge endpoint is outside [0, %d)", N);
+    const SortPlan s = sort_plan(ws, N, E);
+    FlagSlot slot;
+    if (!take_slot(&slot)) GNN_FAIL(GNN_ERR_CUDA, "gnn_coo_to_csr: no pinned memory for the validation word: %s", cudaGetErrorString(cudaGetLastError()));
+    *(volatile int*)slot.word = 0;
+    SortArgs A = {};
+    A.E = E; A.N = N; A.ntiles = s.ntiles; A.flag = s.flag; A.host_flag = slot.word; A.pos = s.pos; A.t2f = out->t2f;
+    A.j[0].keys = dst; A.j[0].other = src; A.j[0].col = out->col; A.j[0].eid = out->eid; A.j[0].pos = s.pos; A.j[0].rowptr = out->rowptr;
+    A.j[1].keys = src; A.j[1].other = dst; A.j[1].col = out->colT; A.j[1].eid = out->eidT; A.j[1].pos = nullptr; A.j[1].rowptr = out->rowptrT;
+    for (int k = 0; k < 2; ++k) { A.j[k].table = s.table[k]; A.j[k].totals = s.totals[k]; }
+    cudaError_t e = cudaMemsetAsync(s.flag, 0, sizeof(int), st);
+    if (e == cudaSuccess) {
+        if (s.both) {
+            e = launch_sort<8>(A, s, 0, 2, slot.event, st);
+        } else {
+            e = launch_sort<16>(A, s, 0, 1, slot.event, st);
+            if (e == cudaSuccess) e = launch_sort<16>(A, s, 1, 1, slot.event, st);
+        }
+    }
+    if (e == cudaSuccess) e = cudaEventSynchronize(slot.event);
+    const int bad = *(volatile int*)slot.word;
+    give_slot(slot);
+    if (e != cudaSuccess) GNN_FAIL(GNN_ERR_CUDA, "gnn_coo_to_csr: %s", cudaGetErrorString(e));
+    GNN_REQUIRE(bad == 0, GNN_ERR_INDEX_OUT_OF_RANGE,
+                "gnn_coo_to_csr: an edge endpoint is outside [0, %d)", N);
     return GNN_OK;
 }
 
@@ -561,9 +698,9 @@ gnn_status gnn_degree(const gnn_csr* g, int transposed, const float* w, void* de
     if (g->N == 0) return GNN_OK;
     cudaStream_t st = as_stream(stream);
     if (!w)
-        degree_count_kernel<<<(int)ceil_div(g->N, 256), 256, 0, st>>>(g->N, rp, (int32_t*)deg_out);
+        launch_overlapped(degree_count_kernel, dim3((unsigned)ceil_div(g->N, 256)), dim3(256), 0, st, g->N, rp, (int32_t*)deg_out);
     else
-        degree_weighted_kernel<<<(int)ceil_div((int64_t)g->N * 32, 256), 256, 0, st>>>(g->N, rp, w, (float*)deg_out);
+        launch_overlapped(degree_weighted_kernel, dim3((unsigned)ceil_div(g->N, 32)), dim3(256), 0, st, g->N, rp, w, (float*)deg_out);
     GNN_CHECK_LAUNCH("gnn_degree");
     return GNN_OK;
 }
@@ -575,7 +712,7 @@ gnn_status gnn_add_self_loops(int32_t N, int64_t E, const int32_t* src, const in
     if (E + N == 0) return GNN_OK;
     GNN_REQUIRE(src_out && dst_out && (E == 0 || (src && dst)), GNN_ERR_INVALID_ARG,
                 "gnn_add_self_loops: null argument");
-    add_self_loops_kernel<<<grid_for(E + N, 256), 256, 0, as_stream(stream)>>>(N, E, src, dst, src_out, dst_out);
+    launch_overlapped(add_self_loops_kernel, dim3((unsigned)(grid_for(E + N, 256))), dim3(256), 0, as_stream(stream), N, E, src, dst, src_out, dst_out);
     GNN_CHECK_LAUNCH("gnn_add_self_loops");
     return GNN_OK;
 }
@@ -588,17 +725,17 @@ gnn_status gnn_gcn_norm(const gnn_csr* g, const float* w_csr, float* deg_out, fl
     if (g->N == 0) return GNN_OK;
     cudaStream_t st = as_stream(stream);
     if (w_csr)
-        degree_weighted_kernel<<<(int)ceil_div((int64_t)g->N * 32, 256), 256, 0, st>>>(g->N, g->rowptr, w_csr, deg_out);
+        launch_overlapped(degree_weighted_kernel, dim3((unsigned)ceil_div(g->N, 32)), dim3(256), 0, st, g->N, g->rowptr, w_csr, deg_out);
     else
-        degree_unit_kernel<<<(int)ceil_div(g->N, 256), 256, 0, st>>>(g->N, g->rowptr, deg_out);
+        launch_overlapped(degree_unit_kernel, dim3((unsigned)ceil_div(g->N, 256)), dim3(256), 0, st, g->N, g->rowptr, deg_out);
     if (coef_csr && g->E > 0) {
         GNN_REQUIRE(g->col, GNN_ERR_INVALID_ARG, "gnn_gcn_norm: null col");
-        gcn_coef_kernel<false><<<(int)ceil_div((int64_t)g->N * 32, 256), 256, 0, st>>>(g->N, g->rowptr, g->col, w_csr, deg_out, coef_csr);
-        gcn_coef_kernel<true><<<g->N < 148 * 8 ? g->N : 148 * 8, 256, 0, st>>>(g->N, g->rowptr, g->col, w_csr, deg_out, coef_csr);
-        if (coef_csrT) {
-            GNN_REQUIRE(g->t2f, GNN_ERR_INVALID_ARG, "gnn_gcn_norm: null t2f");
-            permute_f32_kernel<<<grid_for(g->E, 256), 256, 0, st>>>(g->E, g->t2f, coef_csr, coef_csrT);
-        }
+        GNN_REQUIRE(!coef_csrT || (g->t2f && g->rowptrT && g->colT), GNN_ERR_INVALID_ARG, "gnn_gcn_norm: null t2f");
+        CoefArgs A = {};
+        A.f[0] = {g->rowptr, g->col, nullptr, coef_csr, aligned16(g->col) && aligned16(coef_csr)};
+        A.f[1] = {g->rowptrT, g->colT, g->t2f, coef_csrT, aligned16(g->colT) && aligned16(g->t2f) && aligned16(coef_csrT)};
+        A.w = w_csr; A.deg = deg_out; A.N = g->N; A.E = g->E;
+        launch_overlapped(gcn_coef_kernel, dim3((unsigned)ceil_div(g->E, 256 * 8), coef_csrT ? 2 : 1), dim3(256), 0, st, A);
     }
     GNN_CHECK_LAUNCH("gnn_gcn_norm");
     return GNN_OK;
@@ -612,10 +749,10 @@ gnn_status gnn_permute_edge_data(const int32_t* perm, int64_t E, int width, int 
     cudaStream_t st = as_stream(stream);
     int grid = grid_for(E * width, 256);
     switch (elem_bytes) {
-        case 1: permute_rows_kernel<uint8_t><<<grid, 256, 0, st>>>(E, width, perm, (const uint8_t*)in, (uint8_t*)out); break;
-        case 2: permute_rows_kernel<uint16_t><<<grid, 256, 0, st>>>(E, width, perm, (const uint16_t*)in, (uint16_t*)out); break;
-        case 4: permute_rows_kernel<uint32_t><<<grid, 256, 0, st>>>(E, width, perm, (const uint32_t*)in, (uint32_t*)out); break;
-        case 8: permute_rows_kernel<uint64_t><<<grid, 256, 0, st>>>(E, width, perm, (const uint64_t*)in, (uint64_t*)out); break;
+        case 1: launch_overlapped(permute_rows_kernel<uint8_t>, dim3((unsigned)(grid)), dim3(256), 0, st, E, width, perm, (const uint8_t*)in, (uint8_t*)out); break;
+        case 2: launch_overlapped(permute_rows_kernel<uint16_t>, dim3((unsigned)(grid)), dim3(256), 0, st, E, width, perm, (const uint16_t*)in, (uint16_t*)out); break;
+        case 4: launch_overlapped(permute_rows_kernel<uint32_t>, dim3((unsigned)(grid)), dim3(256), 0, st, E, width, perm, (const uint32_t*)in, (uint32_t*)out); break;
+        case 8: launch_overlapped(permute_rows_kernel<uint64_t>, dim3((unsigned)(grid)), dim3(256), 0, st, E, width, perm, (const uint64_t*)in, (uint64_t*)out); break;
         default: GNN_FAIL(GNN_ERR_UNSUPPORTED, "gnn_permute_edge_data: elem_bytes must be 1, 2, 4 or 8");
     }
     GNN_CHECK_LAUNCH("gnn_permute_edge_data");
