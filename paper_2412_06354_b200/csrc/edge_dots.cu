@@ -31,8 +31,8 @@ enum { EDGE_DOT = 0, EDGE_DOT_MEAN = 1, EDGE_GATV2 = 2 };
 // four positions instead of 20).
 // Bound by instruction issue for narrow rows and by the gathers (L2 -> SM) for rows of 512 bytes.  Before (4 positions per
 // batch, one batch after the other, 8-byte entries, the row's chunk loaded when it changes) -> now:
-//   100k nodes / 1.6 M edges, 512-byte rows, 8 heads bf16 150 -> 118 us; 123 M edges, 128-byte bf16 rows 2.86 -> 2.54 ms;
-//   GATv2 logits of 100k nodes / 1.6 M edges, 512-byte fp32 rows (a gather per index load, four at a time) 358 -> 130 us.
+//   100k nodes / 1.6 M edges, 512-byte rows, 8 heads bf16 150 -> 116 us; 123 M edges, 128-byte bf16 rows 2.86 -> 2.49 ms;
+//   GATv2 logits of 100k nodes / 1.6 M edges, 512-byte fp32 rows (a gather per index load, four at a time) 358 -> 119 us.
 constexpr int ED_SUB = 256;  // most positions per warp
 constexpr int ED_H = 4;      // positions per register buffer
 
@@ -104,11 +104,13 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
         if (MEAN && q < m) sc = S.inv[MEAN ? q : 0];
         if (q + 1 < m) own_next = own(q + 1);
     };
-    auto issue = [&](uint4* x, int i) -> unsigned {  // positions past the group's last gather that one again
+    for (int i = n + lane; i < P.sub; i += 32) S.col[i] = 0;  // the last warp: positions past the end gather row 0
+    __syncwarp();
+    auto issue = [&](uint4* x, int i) -> unsigned {
         unsigned ends = 0;
 #pragma unroll
         for (int u = 0; u < H; ++u) {
-            const int cc = S.col[max(min(i + u, b - 1), 0)];
+            const int cc = S.col[i + u];
             ends |= ((unsigned)cc >> 31) << u;
             x[u] = ld_hint16(Xl + (size_t)(uint32_t)(cc & 0x7fffffff) * row_bytes, pol_keep);
         }
@@ -118,20 +120,21 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
         float dot[H], scale[MEAN ? H : 1];
 #pragma unroll
         for (int u = 0; u < H; ++u) {
-            float x[EPC], t = 0.f;
+            float x[EPC], t = 0.f, t1 = 0.f;
             Chunk<T>::unpack(xr[u], x);
 #pragma unroll
-            for (int j = 0; j < EPC; ++j) {
-                if (V2) {
-                    const float z = x[j] + d[j];
+            for (int j = 0; j < EPC; j += 2) {
+                if (V2) {  // single FMAs: packed ones measured 126 us instead of 119 (register pairs)
+                    const float z = x[j] + d[j], z1 = x[j + 1] + d[j + 1];
                     t = fmaf(av[V2 ? j : 0], z > 0.f ? z : P.slope * z, t);
+                    t = fmaf(av[V2 ? j + 1 : 0], z1 > 0.f ? z1 : P.slope * z1, t);
                 } else {
-                    t = fmaf(x[j], d[j], t);
+                    fma2(t, t1, x[j], x[j + 1], d[j], d[j + 1]);
                 }
             }
-            dot[u] = col_lane ? t : 0.f;
+            dot[u] = col_lane ? t + t1 : 0.f;
             if (MEAN) scale[MEAN ? u : 0] = sc;
-            if ((ends >> u & 1u) && i + u < b) next_row();
+            if (ends >> u & 1u) next_row();
         }
         __syncwarp();
         if (span >= 4) {

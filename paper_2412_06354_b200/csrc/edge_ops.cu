@@ -2,7 +2,7 @@
 // aggregate_neighbors and their backward passes, on explicit E x F message tensors.  These are
 // the building blocks custom layers are written with; the fused propagate avoids their E x F
 // traffic.  Edge tensors are in CSR order unless stated.
-#include "propagate.cuh"
+#include "reduce_params.cuh"
 
 namespace gnn {
 
@@ -31,55 +31,97 @@ __device__ __forceinline__ void block_span(int64_t total, int64_t* t0, int64_t* 
     *t1 = *t0 + per < total ? *t0 + per : total;
 }
 
-// Grid-stride walk over (position, 16-byte chunk) pairs t = p*nvec + ci without a division per step:
-// one 64-bit division when the thread starts, then p and ci advance by the quotient and remainder of
-// the stride.
-struct PosChunk {
-    int64_t p, dp;
-    int ci, dci, nvec;
-    __device__ __forceinline__ PosChunk(int64_t t0, int64_t stride, int nv) : p(t0 / nv), dp(stride / nv), ci((int)(t0 % nv)), dci((int)(stride % nv)), nvec(nv) {}
-    __device__ __forceinline__ void next() {
-        p += dp;
-        ci += dci;
-        if (ci >= nvec) { ci -= nvec; ++p; }
+// (position, 16-byte chunk) pairs t = p * nvec + ci, EO_U * 256 consecutive ones per block and EO_U per thread, so that a
+// thread has as many dependent index -> row loads in flight.  One 64-bit division per thread for the block's first pair;
+// the rest divide a number below nvec + EO_U * 256 by a multiplication (see over_nvec).  A thread that walked the grid's stride with one pair at a
+// time took 86 us to gather 1.36 M rows of 256 bytes; floor for writing them 54 us.
+constexpr int EO_U = 4;
+// x / nvec; magic = 2^32 / nvec rounded up, which is exact while x * nvec < 2^32: the callers' x is below 128 * nvec, so
+// rows of up to 4096 chunks have one and the others, and rows of one chunk, divide.
+__device__ __forceinline__ uint32_t over_nvec(uint32_t x, uint32_t nvec, uint32_t magic) { return magic ? __umulhi(x, magic) : x / nvec; }
+static uint32_t pair_magic(int nvec) { return nvec > 1 && nvec <= 4096 ? (uint32_t)((((uint64_t)1 << 32) + nvec - 1) / nvec) : 0; }
+struct PairTile {
+    int64_t p0, left;  // position of the block's first pair; pairs from it to the last of all
+    uint32_t r0, nvec, magic;
+    __device__ __forceinline__ PairTile(int64_t total, int nv, uint32_t mg) : nvec((uint32_t)nv), magic(mg) {
+        const int64_t t0 = (int64_t)blockIdx.x * (EO_U * 256);
+        p0 = t0 / nv;
+        r0 = (uint32_t)(t0 - p0 * nv);
+        left = total - t0;
+    }
+    __device__ __forceinline__ bool get(int u, int64_t* p, int* ci) const {  // this thread's u-th pair
+        const uint32_t k = threadIdx.x + u * 256, x = r0 + k, q = over_nvec(x, nvec, magic);
+        *p = p0 + q;
+        *ci = (int)(x - q * nvec);
+        return k < left;
     }
 };
+static dim3 pair_grid(int64_t total) { return dim3((unsigned)ceil_div(total, (int64_t)EO_U * 256)); }
 
-// out[k, chunk] = X[idx[k], chunk]; one thread per 16-byte chunk
-__global__ void gather_rows_kernel(const int32_t* __restrict__ idx, int64_t E, const uint4* __restrict__ X,
-                                   int nvec, uint4* __restrict__ out) {
+// out[k, chunk] = X[idx[k], chunk]
+__global__ void __launch_bounds__(256) gather_rows_kernel(const int32_t* __restrict__ idx, int64_t E, const uint4* __restrict__ X,
+                                                          int nvec, uint32_t magic, uint4* __restrict__ out) {
     pdl_wait();
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x, total = E * nvec;
-    for (PosChunk q(t, stride, nvec); t < total; t += stride, q.next()) out[t] = X[(size_t)idx[q.p] * nvec + q.ci];
+    const PairTile tile(E * nvec, nvec, magic);
+    const uint64_t pol_keep = policy_evict_last();
+    uint4* const o = out + (int64_t)blockIdx.x * (EO_U * 256) + threadIdx.x;
+    size_t at[EO_U];
+    bool ok[EO_U];
+#pragma unroll
+    for (int u = 0; u < EO_U; ++u) {
+        int64_t p;
+        int ci;
+        ok[u] = tile.get(u, &p, &ci);
+        at[u] = (size_t)(ok[u] ? idx[p] : 0) * nvec + ci;
+    }
+    uint4 v[EO_U];
+#pragma unroll
+    for (int u = 0; u < EO_U; ++u)
+        if (ok[u]) v[u] = ld_hint16(reinterpret_cast<const char*>(X + at[u]), pol_keep);
+#pragma unroll
+    for (int u = 0; u < EO_U; ++u)
+        if (ok[u]) o[u * 256] = v[u];
 }
 
 // m[p, f] = e[p, g(f)] * X[col[p], f]   (e == nullptr: plain copy of the source row)
 template <typename T>
-__global__ void apply_edges_mul_kernel(const int32_t* __restrict__ col, int64_t E, const uint4* __restrict__ X,
-                                       int nvec, const float* __restrict__ e, int ew, int feats_per_e,
-                                       uint4* __restrict__ m) {
+__global__ void __launch_bounds__(256) apply_edges_mul_kernel(const int32_t* __restrict__ col, int64_t E, const uint4* __restrict__ X,
+                                                              int nvec, uint32_t magic, const float* __restrict__ e, int ew, int feats_per_e,
+                                                              uint4* __restrict__ m) {
     pdl_wait();
     constexpr int EPC = Chunk<T>::N;
-    int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x, total = E * nvec;
+    const PairTile tile(E * nvec, nvec, magic);
+    const uint64_t pol_keep = policy_evict_last();
+    uint4* const o = m + (int64_t)blockIdx.x * (EO_U * 256) + threadIdx.x;
     const bool chunk_in_one = feats_per_e % EPC == 0;  // every 16-byte chunk lies under one multiplier
-    for (PosChunk q(t, stride, nvec); t < total; t += stride, q.next()) {
-        const int64_t p = q.p;
-        const int ci = q.ci;
-        float x[EPC];
-        Chunk<T>::unpack(X[(size_t)col[p] * nvec + ci], x);
+    int64_t p[EO_U];
+    int ci[EO_U], from[EO_U];
+    bool ok[EO_U];
+#pragma unroll
+    for (int u = 0; u < EO_U; ++u) {
+        ok[u] = tile.get(u, &p[u], &ci[u]);
+        from[u] = ok[u] ? col[p[u]] : 0;
+    }
+    uint4 v[EO_U];
+    float f[EO_U];
+#pragma unroll
+    for (int u = 0; u < EO_U; ++u) {
+        f[u] = 1.0f;
+        if (!ok[u]) continue;
+        v[u] = ld_hint16(reinterpret_cast<const char*>(X + (size_t)from[u] * nvec + ci[u]), pol_keep);
+        if (e && chunk_in_one) f[u] = e[p[u] * ew + (ew == 1 ? 0 : (ci[u] * EPC) / feats_per_e)];
+    }
+#pragma unroll
+    for (int u = 0; u < EO_U; ++u) {
+        if (!ok[u]) continue;
         if (e) {
-            if (chunk_in_one) {
-                const float f = e[p * ew + (ci * EPC) / feats_per_e];
+            float x[EPC];
+            Chunk<T>::unpack(v[u], x);
 #pragma unroll
-                for (int j = 0; j < EPC; ++j) x[j] *= f;
-            } else {
-#pragma unroll
-                for (int j = 0; j < EPC; ++j) x[j] *= e[p * ew + (ci * EPC + j) / feats_per_e];
-            }
+            for (int j = 0; j < EPC; ++j) x[j] *= chunk_in_one ? f[u] : e[p[u] * ew + (ci[u] * EPC + j) / feats_per_e];
+            v[u] = Chunk<T>::pack(x);
         }
-        m[t] = Chunk<T>::pack(x);
+        o[u * 256] = v[u];
     }
 }
 
@@ -100,35 +142,96 @@ __global__ void gat_logit_kernel(const int64_t* __restrict__ rowptr, const int32
     }
 }
 
-// backward of aggregate w.r.t. the messages: dm[p, :] from dOut[row(p), :]
+// backward of aggregate w.r.t. the messages: dm[p, :] from dOut[row(p), :].  A warp looks up the rows of its share of
+// positions once, notes each position's row in shared memory and then writes (position, chunk) pairs, four per lane in
+// flight.  Bound by the writes; looking the row up per pair, one pair at a time, took 160 us for 1.36 M rows of 256 bytes.
+constexpr int AB_SUB = 128;  // most positions per warp
 template <typename T>
-__global__ void aggregate_backward_kernel(const int64_t* __restrict__ rowptr, int N, int64_t E, int op,
-                                          const uint4* __restrict__ dOut, const int32_t* __restrict__ argmax,
-                                          int nvec, uint4* __restrict__ dm) {
+__global__ void __launch_bounds__(256) aggregate_backward_kernel(const int64_t* __restrict__ rowptr, int N, int64_t E, int op, int sub, bool wide,
+                                                                 const uint4* __restrict__ dOut, const int32_t* __restrict__ argmax,
+                                                                 int nvec, uint32_t magic, uint4* __restrict__ dm) {
+    constexpr int EPC = Chunk<T>::N, U = 4;
+    __shared__ int s_rows[8][AB_SUB + 1], s_row[8][AB_SUB];
+    __shared__ uint16_t s_start[8][AB_SUB + 2];
     pdl_wait();
-    constexpr int EPC = Chunk<T>::N;
-    int64_t t0, t1;
-    block_span(E * nvec, &t0, &t1);
-    int i = -1;
-    for (int64_t t = t0 + threadIdx.x; t < t1; t += blockDim.x) {
-        const int64_t p = t / nvec;
-        const int ci = (int)(t - p * nvec);
-        i = advance_row(rowptr, N, i, p);
-        uint4 raw = dOut[(size_t)i * nvec + ci];
-        if (op == GNN_SUM) { dm[t] = raw; continue; }
-        float x[EPC];
-        Chunk<T>::unpack(raw, x);
-        if (op == GNN_MEAN) {
-            const float d = (float)(rowptr[i + 1] - rowptr[i]);
-#pragma unroll
-            for (int j = 0; j < EPC; ++j) x[j] = x[j] / d;
-        } else {
-            const int32_t* a = argmax + ((size_t)i * nvec + ci) * EPC;
-#pragma unroll
-            for (int j = 0; j < EPC; ++j) x[j] = (a[j] == (int32_t)p) ? x[j] : 0.f;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int64_t c = (int64_t)blockIdx.x * 8 + wib;
+    if (c * sub >= E) return;
+    const int cs = (int)(c * sub), n = (int)min((int64_t)sub, E - cs);
+    int* const row_of = s_row[wib];
+    bool began_before;
+    const int m = stage_rows(rowptr, N, E, cs, n, lane, s_rows[wib], s_start[wib], began_before);
+    __syncwarp();
+    for (int i = lane; i < n; i += 32) {
+        int lo = 0, hi = m;  // start[lo] <= i < start[hi]
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (s_start[wib][mid] <= i) lo = mid; else hi = mid;
         }
-        dm[t] = Chunk<T>::pack(x);
+        row_of[i] = s_rows[wib][lo];
     }
+    __syncwarp();
+    const uint32_t pairs = (uint32_t)n * (uint32_t)nvec;
+    uint4* const o = dm + (size_t)cs * nvec;
+    for (uint32_t k0 = lane; k0 < pairs; k0 += 32 * U) {
+        uint4 raw[U], win[U][EPC / 4];
+        int at[U];
+        float deg[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t k = k0 + u * 32, i = over_nvec(k, nvec, magic);
+            at[u] = cs + (int)i;
+            if (k >= pairs) continue;
+            const int r = row_of[i];
+            const size_t from = (size_t)r * nvec + (k - i * nvec);
+            raw[u] = __ldg(dOut + from);
+            if (op == GNN_MEAN) deg[u] = (float)(rowptr[r + 1] - rowptr[r]);
+            if (op == GNN_MAX || op == GNN_MIN) {
+#pragma unroll
+                for (int j = 0; j < EPC / 4; ++j) {
+                    const int32_t* a = argmax + from * EPC + 4 * j;  // wide: 16-byte aligned
+                    if (wide) win[u][j] = __ldg(reinterpret_cast<const uint4*>(a));
+                    else win[u][j] = make_uint4(a[0], a[1], a[2], a[3]);
+                }
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const uint32_t k = k0 + u * 32;
+            if (k >= pairs) continue;
+            if (op != GNN_SUM) {
+                float x[EPC];
+                Chunk<T>::unpack(raw[u], x);
+                if (op == GNN_MEAN) {
+#pragma unroll
+                    for (int j = 0; j < EPC; ++j) x[j] = x[j] / deg[u];
+                } else {
+#pragma unroll
+                    for (int j = 0; j < EPC / 4; ++j) {
+                        x[4 * j] = (int)win[u][j].x == at[u] ? x[4 * j] : 0.f;
+                        x[4 * j + 1] = (int)win[u][j].y == at[u] ? x[4 * j + 1] : 0.f;
+                        x[4 * j + 2] = (int)win[u][j].z == at[u] ? x[4 * j + 2] : 0.f;
+                        x[4 * j + 3] = (int)win[u][j].w == at[u] ? x[4 * j + 3] : 0.f;
+                    }
+                }
+                raw[u] = Chunk<T>::pack(x);
+            }
+            o[k] = raw[u];
+        }
+    }
+}
+// Share of positions: 128 once they fill the machine, fewer below so that every SM has warps; rows of the output are whole.
+static gnn_status launch_aggregate_backward(const char* who, const int64_t* rowptr, int32_t N, int64_t E, gnn_op op, const void* dOut,
+                                            const int32_t* argmax, int nvec, gnn_dtype dtype, void* dm, cudaStream_t st) {
+    const int sub = E >= 512 * 1024 ? AB_SUB : E >= 128 * 1024 ? 64 : 32;
+    const dim3 grid((unsigned)ceil_div(E, (int64_t)sub * 8));
+    auto launch = [&](auto kernel) {
+        launch_overlapped(kernel, grid, dim3(256), 0, st, rowptr, N, E, (int)op, sub, aligned16(argmax), (const uint4*)dOut, argmax, nvec, pair_magic(nvec), (uint4*)dm);
+    };
+    if (dtype == GNN_F32) launch(aggregate_backward_kernel<float>);
+    else launch(aggregate_backward_kernel<__nv_bfloat16>);
+    GNN_CHECK_LAUNCH(who);
+    return GNN_OK;
 }
 
 static gnn_status check_rows(const char* who, int F, gnn_dtype dtype, int* nvec) {
@@ -194,7 +297,7 @@ gnn_status gnn_gather(const int32_t* idx, int64_t E, const void* X, int32_t N, i
     if (E == 0) return GNN_OK;
     GNN_REQUIRE(idx && X && out && aligned16(X) && aligned16(out), GNN_ERR_INVALID_ARG,
                 "%s: null or misaligned argument", who);
-    launch_overlapped(gather_rows_kernel, dim3((unsigned)(grid_for(E * nvec, 256))), dim3(256), 0, as_stream(stream), idx, E, (const uint4*)X, nvec, (uint4*)out);
+    launch_overlapped(gather_rows_kernel, pair_grid(E * nvec), dim3(256), 0, as_stream(stream), idx, E, (const uint4*)X, nvec, pair_magic(nvec), (uint4*)out);
     GNN_CHECK_LAUNCH(who);
     return GNN_OK;
 }
@@ -232,22 +335,20 @@ gnn_status gnn_apply_edges(const gnn_csr* g, gnn_msg msg, const void* X_or_al, c
     gnn_status rc = check_rows(who, F, dtype, &nvec);
     if (rc != GNN_OK) return rc;
     GNN_REQUIRE(aligned16(X_or_al) && aligned16(m_out), GNN_ERR_INVALID_ARG, "%s: misaligned matrix", who);
-    const int epc = dtype == GNN_F32 ? 4 : 8;
     int feats_per_e = 1;
     if (msg == GNN_MSG_E_MUL_XJ) {
         GNN_REQUIRE(e && e_width >= 1 && F % e_width == 0, GNN_ERR_INVALID_ARG,
                     "%s: E_MUL_XJ needs e of width 1, H (dividing F) or F", who);
         feats_per_e = F / e_width;
-        (void)epc;
     } else {
         e = nullptr;
         e_width = 1;
     }
-    const int grid = grid_for(g->E * nvec, 256);
-    if (dtype == GNN_F32)
-        launch_overlapped(apply_edges_mul_kernel<float>, dim3((unsigned)(grid)), dim3(256), 0, st, g->col, g->E, (const uint4*)X_or_al, nvec, e, e_width, feats_per_e, (uint4*)m_out);
-    else
-        launch_overlapped(apply_edges_mul_kernel<__nv_bfloat16>, dim3((unsigned)(grid)), dim3(256), 0, st, g->col, g->E, (const uint4*)X_or_al, nvec, e, e_width, feats_per_e, (uint4*)m_out);
+    auto launch = [&](auto kernel) {
+        launch_overlapped(kernel, pair_grid(g->E * nvec), dim3(256), 0, st, g->col, g->E, (const uint4*)X_or_al, nvec, pair_magic(nvec), e, e_width, feats_per_e, (uint4*)m_out);
+    };
+    if (dtype == GNN_F32) launch(apply_edges_mul_kernel<float>);
+    else launch(apply_edges_mul_kernel<__nv_bfloat16>);
     GNN_CHECK_LAUNCH(who);
     return GNN_OK;
 }
@@ -276,14 +377,7 @@ gnn_status gnn_aggregate_backward(const gnn_csr* g, gnn_op op, const void* dOut_
     if (rc != GNN_OK) return rc;
     if (g->E == 0) return GNN_OK;
     GNN_REQUIRE(aligned16(dOut_NF) && aligned16(dm_EF), GNN_ERR_INVALID_ARG, "%s: misaligned matrix", who);
-    const int grid = grid_for(g->E * nvec, 256);
-    cudaStream_t st = as_stream(stream);
-    if (dtype == GNN_F32)
-        launch_overlapped(aggregate_backward_kernel<float>, dim3((unsigned)(grid)), dim3(256), 0, st, g->rowptr, g->N, g->E, (int)op, (const uint4*)dOut_NF, argmax, nvec, (uint4*)dm_EF);
-    else
-        launch_overlapped(aggregate_backward_kernel<__nv_bfloat16>, dim3((unsigned)(grid)), dim3(256), 0, st, g->rowptr, g->N, g->E, (int)op, (const uint4*)dOut_NF, argmax, nvec, (uint4*)dm_EF);
-    GNN_CHECK_LAUNCH(who);
-    return GNN_OK;
+    return launch_aggregate_backward(who, g->rowptr, g->N, g->E, op, dOut_NF, argmax, nvec, dtype, dm_EF, as_stream(stream));
 }
 
 gnn_status gnn_graph_ptr_from_ids(const int32_t* graph_id, int32_t N, int32_t G, int64_t* graph_ptr,
@@ -328,14 +422,7 @@ gnn_status gnn_reduce_nodes_backward(const int64_t* graph_ptr, int32_t G, int32_
     if (rc != GNN_OK) return rc;
     if (N == 0) return GNN_OK;
     GNN_REQUIRE(aligned16(dOut_GF) && aligned16(dX_NF), GNN_ERR_INVALID_ARG, "%s: misaligned matrix", who);
-    const int grid = grid_for((int64_t)N * nvec, 256);
-    cudaStream_t st = as_stream(stream);
-    if (dtype == GNN_F32)
-        launch_overlapped(aggregate_backward_kernel<float>, dim3((unsigned)(grid)), dim3(256), 0, st, graph_ptr, G, N, (int)op, (const uint4*)dOut_GF, argmax, nvec, (uint4*)dX_NF);
-    else
-        launch_overlapped(aggregate_backward_kernel<__nv_bfloat16>, dim3((unsigned)(grid)), dim3(256), 0, st, graph_ptr, G, N, (int)op, (const uint4*)dOut_GF, argmax, nvec, (uint4*)dX_NF);
-    GNN_CHECK_LAUNCH(who);
-    return GNN_OK;
+    return launch_aggregate_backward(who, graph_ptr, G, N, op, dOut_GF, argmax, nvec, dtype, dX_NF, as_stream(stream));
 }
 
 gnn_status gnn_axpby(float alpha, const void* a, float beta, const void* b, int64_t n, gnn_dtype dtype,

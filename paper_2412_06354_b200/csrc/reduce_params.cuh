@@ -57,6 +57,21 @@ struct PropParams {
     float* da_part;  // [npieces][F]: per piece, sum over p of wh[p,h(f)] * LeakyReLU(X[col[p],f] + v2_self[r,f]); or nullptr
 };
 
+// d.xy += w.xy * x.xy as one packed fp32x2 FMA (each half is an IEEE fused multiply-add)
+__device__ __forceinline__ void fma2(float& a0, float& a1, float x0, float x1, float w0, float w1) {
+    asm("{\n\t.reg .b64 ra, rb, rc;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
+        "mov.b64 rc, {%0, %1};\n\tfma.rn.f32x2 rc, ra, rb, rc;\n\tmov.b64 {%0, %1}, rc;\n\t}"
+        : "+f"(a0), "+f"(a1)
+        : "f"(x0), "f"(x1), "f"(w0), "f"(w1));
+}
+
+// d.xy += x.xy
+__device__ __forceinline__ void add2(float& a0, float& a1, float x0, float x1) {
+    asm("{\n\t.reg .b64 ra, rc;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rc, {%0, %1};\n\tadd.rn.f32x2 rc, ra, rc;\n\tmov.b64 {%0, %1}, rc;\n\t}"
+        : "+f"(a0), "+f"(a1)
+        : "f"(x0), "f"(x1));
+}
+
 // Smallest row r in [lo, N) with rowptr[r + 1] > v, or N: the first row at or after lo that has a
 // position beyond v.  Warp-cooperative (every lane must call it with the same arguments): a look at the
 // next 32 rows, then a 32-way search.

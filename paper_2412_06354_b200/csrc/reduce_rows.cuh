@@ -26,21 +26,6 @@ __device__ __forceinline__ bool beats(float cv, int32_t ca, float v, int32_t a) 
     return better || (cv == v && ca < a);
 }
 
-// d.xy += w.xy * x.xy as one packed fp32x2 FMA (each half is an IEEE fused multiply-add)
-__device__ __forceinline__ void fma2(float& a0, float& a1, float x0, float x1, float w0, float w1) {
-    asm("{\n\t.reg .b64 ra, rb, rc;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rb, {%4, %5};\n\t"
-        "mov.b64 rc, {%0, %1};\n\tfma.rn.f32x2 rc, ra, rb, rc;\n\tmov.b64 {%0, %1}, rc;\n\t}"
-        : "+f"(a0), "+f"(a1)
-        : "f"(x0), "f"(x1), "f"(w0), "f"(w1));
-}
-
-// d.xy += x.xy
-__device__ __forceinline__ void add2(float& a0, float& a1, float x0, float x1) {
-    asm("{\n\t.reg .b64 ra, rc;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rc, {%0, %1};\n\tadd.rn.f32x2 rc, ra, rc;\n\tmov.b64 {%0, %1}, rc;\n\t}"
-        : "+f"(a0), "+f"(a1)
-        : "f"(x0), "f"(x1));
-}
-
 // Everything between the reduced values of a row and its stored 16-byte column ci (of the slab): division of the mean,
 // rank-1 epilogue of the per-head mode and row epilogue (only with EPI), rounding, winners.
 template <typename T, int MODE, bool EPI>
