@@ -44,6 +44,13 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar, uint64_t policy) {
+    asm volatile(
+        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3, %4}], [%5], %6;"
+        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar), "l"(policy)
+        : "memory");
+}
+
 struct TmaParams {
     int64_t N;
     int Kc, Mo;        // contraction length, output columns
@@ -346,20 +353,33 @@ gnn_status linear_tma_forward(const void* X, int ldx, const void* W, int ldw, in
 // the fp32 tolerance.  Roles of the persistent CTA:
 //   warp 0      loader: X arrives as fp32 slices of 128 rows x 32 columns (128-byte rows, 128-byte swizzle)
 //               in a ring of shared-memory slots;
-//   warps 2..9  converters: read a slice, split it, and write the three bf16 levels into one of two operand
-//               buffers in the tensor core's canonical no-swizzle layout (8 rows x 16 bytes per core matrix);
+//   converters  G groups of warps, slice i to group i mod G: read a slice, a row per lane, split it, and write the three
+//               bf16 levels into one of G operand buffers in tensor memory (48 columns each), which the MMA reads as A;
 //   warp 1      MMA issuer: 2 k-steps x 6 level pairs per slice into one of two accumulators;
-//   warps 10..17 epilogue: accumulator -> swizzled staging blocks of 32 rows x 32 columns -> bulk tensor stores to Y.
+//   epilogue    accumulator -> swizzled staging blocks of 32 rows x 32 columns -> bulk tensor stores to Y.
 // The weight matrix is split once per CTA by all warps before the roles start.
-constexpr int TF_CONV_WARPS = 8, TF_EPI_WARPS = 8;
+// What bounds it: the chain of a slice (wait, read, split, write, fence, arrive), about 1 us however few its columns.  With
+// all converter warps on one slice after the other that chain was the rate; now G slices are in it at a time.  Slots and
+// operand buffers are multiples of G, so that each belongs to one group, which sees all its phases (a parity wait only
+// tells the last two apart).  170k x 128 x 128: 46 us with one group, levels in shared memory and the tables below looked up
+// per MMA; 36 us now; reading X and writing Y takes 27 us.  200k x 256 -> 256: 346 -> 233 us.
+// G is 4 where tensor memory has room for four operand buffers (up to 160 output columns) and shared memory for four
+// slots.  More than 192 columns leave no room for two beside the accumulators: A_TMEM = false keeps the levels in two
+// buffers of shared memory, in the canonical no-swizzle layout (8 rows x 16 bytes per core matrix).
+constexpr int TF_CONV_WARPS = 16, TF_EPI_WARPS = 8;
 constexpr int TF_THREADS = 32 * (2 + TF_CONV_WARPS + TF_EPI_WARPS);
 constexpr int TF_KB = 32;                                  // contraction elements per slice
 constexpr uint32_t TF_SLICE_BYTES = TC_ROWS * TF_KB * 4;   // 16 KB of fp32
 constexpr uint32_t TF_LEVEL_BYTES = TC_ROWS * TF_KB * 2;   // 8 KB: one bf16 level of a slice
-constexpr int TF_MAX_STAGES = 6;
+constexpr int TF_MAX_STAGES = 8;
+constexpr int TF_MAX_OPS = 4;        // operand buffers, one per group
+constexpr int TF_OP_COLS = 3 * TF_KB / 2;  // tensor memory columns of one: three levels of 32 bf16
 
-__device__ __constant__ unsigned char kPairA3[6] = {2, 0, 1, 1, 0, 0};  // levels of A and B per product, small terms first
-__device__ __constant__ unsigned char kPairB3[6] = {0, 2, 1, 0, 1, 0};
+// Levels of A and B of product q, small terms first: (2,0) (0,2) (1,1) (1,0) (0,1) (0,0).  Functions of an unrolled index, so
+// that the issuing thread adds constants to a descriptor: with tables in constant memory and a descriptor built per MMA the
+// issue alone took 150 cycles an MMA, five times what the tensor core takes for 128 x 128 x 16.
+__device__ __forceinline__ constexpr uint32_t pair_a(int q) { return q == 0 ? 2u : q == 2 || q == 3 ? 1u : 0u; }
+__device__ __forceinline__ constexpr uint32_t pair_b(int q) { return q == 1 ? 2u : q == 2 || q == 4 ? 1u : 0u; }
 
 // 8 fp32 values -> three 16-byte chunks of bf16 (x = x1 + x2 + x3 exactly)
 __device__ __forceinline__ void split8(const float* xin, uint4* lv) {
@@ -406,11 +426,12 @@ struct TmaF32Params {
     int64_t ldy;
 };
 
+template <bool A_TMEM, int G>
 __global__ void __launch_bounds__(TF_THREADS, 1)
 linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY, const TmaF32Params P) {
     extern __shared__ unsigned char smem_raw[];
-    // f_full[S], f_empty[S], o_full[2], o_empty[2], acc_full[2], acc_empty[2]
-    __shared__ __align__(8) uint64_t bars[2 * TF_MAX_STAGES + 8];
+    // f_full[S], f_empty[S], o_full[G], o_empty[G], acc_full[2], acc_empty[2]
+    __shared__ __align__(8) uint64_t bars[2 * TF_MAX_STAGES + 2 * TF_MAX_OPS + 4];
     __shared__ uint32_t tmem_base_slot;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int Kc = P.Kc, Mo = P.Mo, S = P.stages;
@@ -419,22 +440,21 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
     const uint32_t b_sbo = (uint32_t)kchunks * 128;  // weight levels: same layout as a whole-K operand
     const uint32_t b_level = (uint32_t)Mo * Kc * 2;
     const uint32_t w0 = base, ring0 = base + ((3 * b_level + 1023u) & ~1023u), op0 = ring0 + (uint32_t)S * TF_SLICE_BYTES;
-    const uint32_t stage0 = op0 + 2u * 3u * TF_LEVEL_BYTES;  // per epilogue warp: 32 rows x 32 fp32 columns of Y
+    const uint32_t stage0 = op0 + (A_TMEM ? 0u : 2u * 3u * TF_LEVEL_BYTES);  // per epilogue warp: 32 rows x 32 fp32 columns of Y
     const int nslices = (Kc + TF_KB - 1) / TF_KB;
     const uint32_t bar0 = smem_u32(bars);
     auto f_full = [&](int s) { return bar0 + 8u * (uint32_t)s; };
     auto f_empty = [&](int s) { return bar0 + 8u * (uint32_t)(TF_MAX_STAGES + s); };
     auto o_full = [&](int o) { return bar0 + 8u * (uint32_t)(2 * TF_MAX_STAGES + o); };
-    auto o_empty = [&](int o) { return bar0 + 8u * (uint32_t)(2 * TF_MAX_STAGES + 2 + o); };
-    auto acc_full = [&](int a) { return bar0 + 8u * (uint32_t)(2 * TF_MAX_STAGES + 4 + a); };
-    auto acc_empty = [&](int a) { return bar0 + 8u * (uint32_t)(2 * TF_MAX_STAGES + 6 + a); };
+    auto o_empty = [&](int o) { return bar0 + 8u * (uint32_t)(2 * TF_MAX_STAGES + TF_MAX_OPS + o); };
+    auto acc_full = [&](int a) { return bar0 + 8u * (uint32_t)(2 * TF_MAX_STAGES + 2 * TF_MAX_OPS + a); };
+    auto acc_empty = [&](int a) { return bar0 + 8u * (uint32_t)(2 * TF_MAX_STAGES + 2 * TF_MAX_OPS + 2 + a); };
+    constexpr int GW = TF_CONV_WARPS / G;  // warps per group
 
     if (tid == 0) {
-        for (int s = 0; s < S; ++s) { mbar_init(f_full(s), 1); mbar_init(f_empty(s), TF_CONV_WARPS); }
-        for (int o = 0; o < 2; ++o) {
-            mbar_init(o_full(o), TF_CONV_WARPS); mbar_init(o_empty(o), 1);
-            mbar_init(acc_full(o), 1); mbar_init(acc_empty(o), TF_EPI_WARPS);
-        }
+        for (int s = 0; s < S; ++s) { mbar_init(f_full(s), 1); mbar_init(f_empty(s), GW); }
+        for (int o = 0; o < G; ++o) { mbar_init(o_full(o), GW); mbar_init(o_empty(o), 1); }
+        for (int a = 0; a < 2; ++a) { mbar_init(acc_full(a), 1); mbar_init(acc_empty(a), TF_EPI_WARPS); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapX)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapY)) : "memory");
@@ -494,7 +514,7 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
         }
     } else if (warp == 1) {
         if (lane == 0) {
-            const uint32_t idesc = make_idesc(Mo, P.b_transposed ? 0 : 1);
+            const uint32_t idesc = make_idesc(Mo, P.b_transposed ? 0 : 1), b_level16 = b_level / 16;
             uint32_t it = 0, lt = 0;
             for (int64_t t = blockIdx.x; t < ntiles && !failed; t += gridDim.x, ++lt) {
                 const uint32_t a = lt & 1u;
@@ -502,18 +522,25 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
                 tc_fence_after();
                 const uint32_t dacc = tmem_base + a * (uint32_t)P.acc_stride;
                 for (int j = 0; j < nslices; ++j, ++it) {
-                    const uint32_t o = it & 1u;
-                    if (!mbar_wait_bounded(o_full((int)o), (it >> 1) & 1u)) { failed = true; break; }
+                    const uint32_t o = it % G;
+                    if (!mbar_wait_bounded(o_full((int)o), (it / G) & 1u)) { failed = true; break; }
                     tc_fence_after();
-                    const uint32_t abuf = op0 + o * 3u * TF_LEVEL_BYTES;
-                    const int ksteps = (Kc - j * TF_KB) >= TF_KB ? TF_KB / 16 : (Kc - j * TF_KB) / 16;
-                    for (int kk = 0; kk < ksteps; ++kk)
-                        for (int q = 0; q < 6; ++q) {
-                            // A slice: 4 chunks along k, core matrices 128 bytes apart, groups of 8 rows 512 bytes apart
-                            const uint64_t adesc = make_smem_desc(abuf + (uint32_t)kPairA3[q] * TF_LEVEL_BYTES + (uint32_t)kk * 256u, 128, 512);
-                            const uint64_t bdesc = make_smem_desc(w0 + (uint32_t)kPairB3[q] * b_level + (uint32_t)(j * (TF_KB / 16) + kk) * 256u, 128, b_sbo);
-                            mma_bf16_ss(dacc, adesc, bdesc, idesc, (j > 0 || kk > 0 || q > 0) ? 1u : 0u);
+                    const uint32_t at = tmem_base + 2u * (uint32_t)P.acc_stride + o * (uint32_t)TF_OP_COLS;
+                    // A slice: 4 chunks along k, core matrices 128 bytes apart, groups of 8 rows 512 bytes apart
+                    const uint64_t adesc = make_smem_desc(op0 + o * 3u * TF_LEVEL_BYTES, 128, 512);
+                    const uint64_t bdesc = make_smem_desc(w0 + (uint32_t)j * (TF_KB / 16) * 256u, 128, b_sbo);
+                    const bool both = Kc - j * TF_KB >= TF_KB;  // else a last slice of 16
+#pragma unroll
+                    for (int kk = 0; kk < TF_KB / 16; ++kk) {
+                        if (kk > 0 && !both) break;
+#pragma unroll
+                        for (int q = 0; q < 6; ++q) {  // offsets add to the descriptors' address field, in units of 16 bytes
+                            const uint64_t bd = bdesc + (uint64_t)(pair_b(q) * b_level16 + (uint32_t)kk * 16u);
+                            const uint32_t more = (j > 0 || kk > 0 || q > 0) ? 1u : 0u;
+                            if (A_TMEM) mma_bf16_ts(dacc, at + pair_a(q) * (TF_KB / 2) + (uint32_t)kk * 8u, bd, idesc, more);
+                            else mma_bf16_ss(dacc, adesc + (uint64_t)(pair_a(q) * (TF_LEVEL_BYTES / 16) + (uint32_t)kk * 16u), bd, idesc, more);
                         }
+                    }
                     mma_commit(o_empty((int)o));
                 }
                 if (failed) break;
@@ -521,38 +548,52 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
             }
         }
     } else if (warp < 2 + TF_CONV_WARPS) {
-        // Every converter warp works on every slice, in order: a waiter that skipped uses of a slot would
-        // find the parity of an older completed phase and run ahead of the copy (parity waits only tell
-        // the last two phases apart), so the slices are not divided among groups of warps.
-        constexpr int GT = 32 * TF_CONV_WARPS;
-        const int ct = tid - 64;
+        const int grp = (warp - 2) / GW, wl = (warp - 2) % GW;
         uint32_t it = 0;
         for (int64_t t = blockIdx.x; t < ntiles && !failed; t += gridDim.x)
             for (int j = 0; j < nslices; ++j, ++it) {
+                if (it % G != (uint32_t)grp) continue;
                 const int s = (int)(it % (uint32_t)S);
-                const uint32_t o = it & 1u;
                 if (!mbar_wait_bounded(f_full(s), (it / (uint32_t)S) & 1u)) { failed = true; break; }
-                if (!mbar_wait_bounded(o_empty((int)o), ((it >> 1) & 1u) ^ 1u)) { failed = true; break; }
+                if (!mbar_wait_bounded(o_empty(grp), ((it / G) & 1u) ^ 1u)) { failed = true; break; }
                 tc_fence_after();
-                const uint32_t src = ring0 + (uint32_t)s * TF_SLICE_BYTES, dst = op0 + o * 3u * TF_LEVEL_BYTES;
-#pragma unroll
-                for (int rep = 0; rep < (TC_ROWS * (TF_KB / 8)) / GT; ++rep) {
-                    const int e = ct + rep * GT;
-                    const int q = e >> 3, rg = q >> 2, kc = q & 3, r = rg * 8 + (e & 7);
-                    // fp32 row r: 128 bytes, 16-byte chunk c at position c ^ (r % 8)
+                const uint32_t src = ring0 + (uint32_t)s * TF_SLICE_BYTES;
+                // 8 values of row r: fp32 row of 128 bytes, 16-byte chunk c at position c ^ (r % 8)
+                auto split_chunk = [&](int r, int kc, uint4* lv) {
                     const uint4 c0 = ld_shared16(src + (uint32_t)r * 128u + (uint32_t)(((2 * kc) ^ (r & 7)) << 4));
                     const uint4 c1 = ld_shared16(src + (uint32_t)r * 128u + (uint32_t)(((2 * kc + 1) ^ (r & 7)) << 4));
                     const float x[8] = {__uint_as_float(c0.x), __uint_as_float(c0.y), __uint_as_float(c0.z), __uint_as_float(c0.w),
                                         __uint_as_float(c1.x), __uint_as_float(c1.y), __uint_as_float(c1.z), __uint_as_float(c1.w)};
-                    uint4 lv[3];
                     split8(x, lv);
-                    const uint32_t off = (uint32_t)(r >> 3) * 512u + (uint32_t)kc * 128u + (uint32_t)(r & 7) * 16u;
+                };
+                if (A_TMEM) {  // a warp reaches the 32 lanes of tensor memory of its number modulo 4
+                    const uint32_t to = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + 2u * (uint32_t)P.acc_stride + (uint32_t)(grp * TF_OP_COLS);
 #pragma unroll
-                    for (int l = 0; l < 3; ++l) st_shared16(dst + (uint32_t)l * TF_LEVEL_BYTES + off, lv[l]);
+                    for (int rep = 0; rep < 16 / GW; ++rep) {
+                        const int kc = (wl >> 2) + rep * (GW / 4);
+                        uint4 lv[3];
+                        split_chunk((warp & 3) * 32 + lane, kc, lv);
+#pragma unroll
+                        for (int l = 0; l < 3; ++l) tmem_st4(to + (uint32_t)(l * (TF_KB / 2) + kc * 4), lv[l]);
+                    }
+                    tmem_st_wait();
+                    tc_fence_before();
+                } else {
+                    const uint32_t dst = op0 + (uint32_t)grp * 3u * TF_LEVEL_BYTES;
+#pragma unroll
+                    for (int rep = 0; rep < 16 / GW; ++rep) {
+                        const int e = wl * 32 + lane + rep * GW * 32;
+                        const int q = e >> 3, rg = q >> 2, kc = q & 3, r = rg * 8 + (e & 7);
+                        uint4 lv[3];
+                        split_chunk(r, kc, lv);
+                        const uint32_t off = (uint32_t)(r >> 3) * 512u + (uint32_t)kc * 128u + (uint32_t)(r & 7) * 16u;
+#pragma unroll
+                        for (int l = 0; l < 3; ++l) st_shared16(dst + (uint32_t)l * TF_LEVEL_BYTES + off, lv[l]);
+                    }
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the tensor core
                 }
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // generic-proxy writes -> visible to the tensor core
                 __syncwarp();
-                if (lane == 0) { mbar_arrive(f_empty(s)); mbar_arrive(o_full((int)o)); }
+                if (lane == 0) { mbar_arrive(f_empty(s)); mbar_arrive(o_full(grp)); }
             }
     } else {
         const int ew = warp - (2 + TF_CONV_WARPS), quarter = warp & 3, half = ew >> 2;
@@ -816,45 +857,64 @@ static bool make_map_f32_ld(CUtensorMap* m, const void* ptr, int64_t rows, int c
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The same with all columns in one box, stored as the boxes of 32 columns one after the other: dimensions (32 columns, rows,
+// blocks of 32 columns).  Whole blocks only: the copy engine would read a partial one past the row.
+static bool make_map_f32_blocks(CUtensorMap* m, const void* ptr, int64_t rows, int cols, int ld, int box_rows) {
+    EncodeTiledFn enc = encoder();
+    if (!enc) return false;
+    const cuuint64_t dims[3] = {32, (cuuint64_t)rows, (cuuint64_t)(cols / 32)};
+    const cuuint64_t strides[2] = {(cuuint64_t)ld * 4, 128};
+    const cuuint32_t box[3] = {32, (cuuint32_t)box_rows, (cuuint32_t)(cols / 32)};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    return enc(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<void*>(ptr), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+               CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 // ------------------------------------------------------------------ fp32: dW = X^T * dY on the bf16 tensor cores, pipelined
-// Contraction over the N rows, 32 rows per pipeline slot (16 where K or M is 256, so that two operand buffers and a
+// Contraction over the N rows, 32 rows per pipeline slot (16 where K or M is over 128, so that two operand buffers and a
 // ring still fit shared memory).  Roles of the persistent CTA:
 //   warp 0      loader: a slot is K/32 + M/32 boxes of 32 rows x 32 fp32 columns (128-byte rows, 128-byte swizzle)
 //               of X and dY, in a ring of shared-memory slots;
-//   warps 2..9  converters: split every value exactly into three bf16 terms and write the levels of both operands
-//               into one of two operand buffers in the canonical no-swizzle layout, MN-major (16-byte chunk c = 8
+//   warps 2..17 converters, P.groups groups of them, slot i to group i mod groups (see the kernel above): split every
+//               value exactly into three bf16 terms and write the levels of both operands
+//               into the group's operand buffer in the canonical no-swizzle layout, MN-major (16-byte chunk c = 8
 //               features or columns of row n at c*512 + (n/8)*128 + (n%8)*16);
 //   warp 1      MMA issuer: 2 k-steps of 16 rows x 6 level pairs per slot, all into one accumulator [128 features x M]
 //               that stays in tensor memory for the whole kernel;
-//   at the end the converter warps write the accumulator as this CTA's fp32 partial [K,M]; the caller sums the
+//   at the end the first eight converter warps write the accumulator as this CTA's fp32 partial [K,M]; the caller sums the
 //   partials in CTA order (fixed order: deterministic).
 // K a multiple of 32 up to 128 features (the MMA has 128 rows; those past K are zeros), M a multiple of 32 up to 128.
 // Every wait is bounded.
-constexpr int FD_ROWS_MAX = 32;
-constexpr int FD_CONV_WARPS = 8;
+// Two groups on slots of 32 rows, on slots of 16 four where four buffers and slots fit.  170k x 128 x 128: 50 us with 8 warps
+// on one slot after the other, 47 us with 16, 58 us in four groups on slots of 16 rows, 42 us so; reading X and dY takes 27 us.
+constexpr int FD_CONV_WARPS = 16;
 constexpr int FD_THREADS = 32 * (2 + FD_CONV_WARPS);
-constexpr int FD_MAX_STAGES = 4;
+constexpr int FD_MAX_STAGES = 8;
+constexpr int FD_MAX_GROUPS = 4;
 
 struct TmaF32DwParams {
     float* part;  // [gridDim.x][K][M]
     int64_t N;
     int K, M;
-    int rows;  // rows of X / dY per slot: 32 or 16
-    int stages;
+    int x_whole, d_whole;  // the slot's boxes of X or dY arrive in one copy
+    int groups;  // 4 or 2
+    int stages;  // a multiple of groups
     int tmem_cols;
     int* status;
     int reset;  // first launch of a call: set the status word to 0
 };
 
+template <int FD_ROWS>
 __global__ void __launch_bounds__(FD_THREADS, 1)
 linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapD, const TmaF32DwParams P) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t bars[2 * FD_MAX_STAGES + 5];  // f_full[S], f_empty[S], o_full[2], o_empty[2], acc_full
+    __shared__ __align__(8) uint64_t bars[2 * FD_MAX_STAGES + 2 * FD_MAX_GROUPS + 1];  // f_full[S], f_empty[S], o_full[G], o_empty[G], acc_full
     __shared__ uint32_t tmem_base_slot;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int K = P.K, M = P.M, S = P.stages, FD_ROWS = P.rows, halves = (K + 127) / 128;
-    const uint32_t FD_BOX_BYTES = (uint32_t)FD_ROWS * 128u;   // one box: FD_ROWS rows x 32 fp32 columns
-    const uint32_t FD_SBO = (uint32_t)(FD_ROWS / 8) * 128u;   // next chunk of 8 features / columns in an operand level
+    const int K = P.K, M = P.M, S = P.stages, halves = (K + 127) / 128;
+    const uint32_t G = (uint32_t)P.groups;
+    constexpr uint32_t FD_BOX_BYTES = (uint32_t)FD_ROWS * 128u;   // one box: FD_ROWS rows x 32 fp32 columns
+    constexpr uint32_t FD_SBO = (uint32_t)(FD_ROWS / 8) * 128u;   // next chunk of 8 features / columns in an operand level
     const int xboxes = K / 32, dboxes = M / 32;
     const uint32_t slot_bytes = (uint32_t)(xboxes + dboxes) * FD_BOX_BYTES;
     // the A operand always has whole blocks of the MMA's 128 feature rows; with K < 128 the rows past K stay zero
@@ -866,20 +926,20 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
     auto f_full = [&](int s) { return bar0 + 8u * (uint32_t)s; };
     auto f_empty = [&](int s) { return bar0 + 8u * (uint32_t)(FD_MAX_STAGES + s); };
     auto o_full = [&](int o) { return bar0 + 8u * (uint32_t)(2 * FD_MAX_STAGES + o); };
-    auto o_empty = [&](int o) { return bar0 + 8u * (uint32_t)(2 * FD_MAX_STAGES + 2 + o); };
-    const uint32_t acc_full = bar0 + 8u * (uint32_t)(2 * FD_MAX_STAGES + 4);
+    auto o_empty = [&](int o) { return bar0 + 8u * (uint32_t)(2 * FD_MAX_STAGES + FD_MAX_GROUPS + o); };
+    const uint32_t acc_full = bar0 + 8u * (uint32_t)(2 * FD_MAX_STAGES + 2 * FD_MAX_GROUPS);
 
     if (tid == 0) {
-        for (int s = 0; s < S; ++s) { mbar_init(f_full(s), 1); mbar_init(f_empty(s), FD_CONV_WARPS); }
-        for (int o = 0; o < 2; ++o) { mbar_init(o_full(o), FD_CONV_WARPS); mbar_init(o_empty(o), 1); }
+        for (int s = 0; s < S; ++s) { mbar_init(f_full(s), 1); mbar_init(f_empty(s), FD_CONV_WARPS / G); }
+        for (int o = 0; o < (int)G; ++o) { mbar_init(o_full(o), FD_CONV_WARPS / G); mbar_init(o_empty(o), 1); }
         mbar_init(acc_full, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapX)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapD)) : "memory");
     }
     if (warp == 1) tmem_alloc(smem_u32(&tmem_base_slot), (uint32_t)P.tmem_cols);
-    if (K % 128 != 0) {  // the converters never write the feature rows past K: zero both buffers' A levels once
-        for (int o = 0; o < 2; ++o)
+    if (K % 128 != 0) {  // the converters never write the feature rows past K: zero the buffers' A levels once
+        for (int o = 0; o < (int)G; ++o)
             for (uint32_t off = (uint32_t)tid * 16u; off < 3u * a_level; off += FD_THREADS * 16u)
                 st_shared16(op0 + (uint32_t)o * op_bytes + off, make_uint4(0u, 0u, 0u, 0u));
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -903,8 +963,13 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
                 if (!mbar_wait_bounded(f_empty(s), ((it / (uint32_t)S) & 1u) ^ 1u)) { failed = true; break; }
                 mbar_arrive_expect_tx(f_full(s), slot_bytes);  // rows past N arrive as zeros and count all the same
                 const uint32_t dst = ring0 + (uint32_t)s * slot_bytes;
-                for (int b = 0; b < xboxes; ++b) tma_load_2d(dst + (uint32_t)b * FD_BOX_BYTES, &mapX, b * 32, (int)(t * FD_ROWS), f_full(s), stream);
-                for (int b = 0; b < dboxes; ++b) tma_load_2d(dst + (uint32_t)(xboxes + b) * FD_BOX_BYTES, &mapD, b * 32, (int)(t * FD_ROWS), f_full(s), stream);
+                const int row = (int)(t * FD_ROWS);
+                if (P.x_whole) tma_load_3d(dst, &mapX, 0, row, 0, f_full(s), stream);
+                else
+                    for (int b = 0; b < xboxes; ++b) tma_load_2d(dst + (uint32_t)b * FD_BOX_BYTES, &mapX, b * 32, row, f_full(s), stream);
+                if (P.d_whole) tma_load_3d(dst + (uint32_t)xboxes * FD_BOX_BYTES, &mapD, 0, row, 0, f_full(s), stream);
+                else
+                    for (int b = 0; b < dboxes; ++b) tma_load_2d(dst + (uint32_t)(xboxes + b) * FD_BOX_BYTES, &mapD, b * 32, row, f_full(s), stream);
             }
             if (failed) {  // let the copies in flight land before the CTA goes away
                 const uint32_t first = it > (uint32_t)S ? it - (uint32_t)S : 0u;
@@ -917,53 +982,54 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
             const uint32_t idesc = make_idesc(M, 1) | (1u << 15);  // A and B both MN-major
             uint32_t it = 0;
             for (int64_t t = blockIdx.x; t < nslots; t += gridDim.x, ++it) {
-                const uint32_t o = it & 1u;
-                if (!mbar_wait_bounded(o_full((int)o), (it >> 1) & 1u)) { failed = true; break; }
+                const uint32_t o = it % G;
+                if (!mbar_wait_bounded(o_full((int)o), (it / G) & 1u)) { failed = true; break; }
                 tc_fence_after();
                 const uint32_t abuf = op0 + o * op_bytes, bbuf = abuf + 3u * a_level;
-                for (int h = 0; h < halves; ++h)  // features [128h, 128h + 128): chunks 16h.., accumulator columns h*M..
+                const uint64_t adesc = make_smem_desc(abuf, 128, FD_SBO), bdesc = make_smem_desc(bbuf, 128, FD_SBO);
+                for (int h = 0; h < halves; ++h) {  // features [128h, 128h + 128): chunks 16h.., accumulator columns h*M..
+#pragma unroll
                     for (int kk = 0; kk < FD_ROWS / 16; ++kk)
-                        for (int q = 0; q < 6; ++q) {
-                            const uint64_t adesc = make_smem_desc(abuf + (uint32_t)kPairA3[q] * a_level + (uint32_t)h * 16u * FD_SBO + (uint32_t)kk * 256u, 128, FD_SBO);
-                            const uint64_t bdesc = make_smem_desc(bbuf + (uint32_t)kPairB3[q] * b_level + (uint32_t)kk * 256u, 128, FD_SBO);
-                            mma_bf16_ss(tmem_base + (uint32_t)h * (uint32_t)M, adesc, bdesc, idesc, (it > 0 || kk > 0 || q > 0) ? 1u : 0u);
-                        }
+#pragma unroll
+                        for (int q = 0; q < 6; ++q)  // offsets add to the descriptors' address field, in units of 16 bytes
+                            mma_bf16_ss(tmem_base + (uint32_t)h * (uint32_t)M, adesc + (uint64_t)(pair_a(q) * (a_level / 16) + (uint32_t)h * FD_SBO + (uint32_t)kk * 16u),
+                                        bdesc + (uint64_t)(pair_b(q) * (b_level / 16) + (uint32_t)kk * 16u), idesc, (it > 0 || kk > 0 || q > 0) ? 1u : 0u);
+                }
                 mma_commit(o_empty((int)o));
             }
             if (!failed) mma_commit(acc_full);
         }
     } else {
-        // ------------------------------------------------------------ converters (every warp works on every slot, in order)
-        constexpr int GT = 32 * FD_CONV_WARPS;
-        const int ct = tid - 64;
-        const int xchunks = K / 8, dchunks = M / 8;
-        const int xops = FD_ROWS * xchunks, ops = xops + FD_ROWS * dchunks;
+        // ------------------------------------------------------------ converters
+        // A unit of 32 lanes: 8 rows of a box x its 4 chunks of 8 columns, so that every address is a sum of the lane's part
+        // and the unit's; eight lanes read eight rows (swizzled: no conflict) and write one core matrix.
+        constexpr int BU = FD_ROWS / 8;  // units per box
+        const int GW = FD_CONV_WARPS / (int)G;  // warps per group
+        const uint32_t o = (uint32_t)((warp - 2) / GW);
+        const int units = (xboxes + dboxes) * BU, r7 = lane & 7, kc = lane >> 3;
+        const uint32_t from0 = (uint32_t)r7 * 128u + (uint32_t)(((2 * kc) ^ r7) << 4), from1 = (uint32_t)r7 * 128u + (uint32_t)(((2 * kc + 1) ^ r7) << 4);
+        const uint32_t to_l = (uint32_t)kc * FD_SBO + (uint32_t)r7 * 16u;
         uint32_t it = 0;
         for (int64_t t = blockIdx.x; t < nslots && !failed; t += gridDim.x, ++it) {
+            if (it % G != o) continue;
             const int s = (int)(it % (uint32_t)S);
-            const uint32_t o = it & 1u;
             if (!mbar_wait_bounded(f_full(s), (it / (uint32_t)S) & 1u)) { failed = true; break; }
-            if (!mbar_wait_bounded(o_empty((int)o), ((it >> 1) & 1u) ^ 1u)) { failed = true; break; }
+            if (!mbar_wait_bounded(o_empty((int)o), ((it / G) & 1u) ^ 1u)) { failed = true; break; }
             tc_fence_after();
             const uint32_t src0 = ring0 + (uint32_t)s * slot_bytes;
             const uint32_t abuf = op0 + o * op_bytes, bbuf = abuf + 3u * a_level;
-#pragma unroll 4
-            for (int e = ct; e < ops; e += GT) {
-                // eight consecutive threads take the eight rows of one core matrix: contiguous 16-byte stores
-                const bool isx = e < xops;
-                const int ee = isx ? e : e - xops, chunks = isx ? xchunks : dchunks;
-                const int q = ee >> 3, rg = q / chunks, c8 = q - rg * chunks, r = rg * 8 + (ee & 7);
-                const int bx = (isx ? 0 : xboxes) + (c8 >> 2), kc = c8 & 3;
-                // fp32 row r of the box: 128 bytes, 16-byte chunk c at position c ^ (r % 8)
-                const uint32_t rowa = src0 + (uint32_t)bx * FD_BOX_BYTES + (uint32_t)r * 128u;
-                const uint4 c0 = ld_shared16(rowa + (uint32_t)(((2 * kc) ^ (r & 7)) << 4));
-                const uint4 c1 = ld_shared16(rowa + (uint32_t)(((2 * kc + 1) ^ (r & 7)) << 4));
+#pragma unroll 2
+            for (int u = (warp - 2) % GW; u < units; u += GW) {
+                const int box = u / BU, rg = u % BU;
+                const uint32_t rows8 = src0 + (uint32_t)box * FD_BOX_BYTES + (uint32_t)rg * 1024u;
+                const uint4 c0 = ld_shared16(rows8 + from0), c1 = ld_shared16(rows8 + from1);
                 const float x[8] = {__uint_as_float(c0.x), __uint_as_float(c0.y), __uint_as_float(c0.z), __uint_as_float(c0.w),
                                     __uint_as_float(c1.x), __uint_as_float(c1.y), __uint_as_float(c1.z), __uint_as_float(c1.w)};
                 uint4 lv[3];
                 split8(x, lv);
+                const bool isx = box < xboxes;
                 const uint32_t level = isx ? a_level : b_level;
-                const uint32_t dst = (isx ? abuf : bbuf) + (uint32_t)c8 * FD_SBO + (uint32_t)(r >> 3) * 128u + (uint32_t)(r & 7) * 16u;
+                const uint32_t dst = (isx ? abuf + (uint32_t)box * 4u * FD_SBO : bbuf + (uint32_t)(box - xboxes) * 4u * FD_SBO) + (uint32_t)rg * 128u + to_l;
 #pragma unroll
                 for (int l = 0; l < 3; ++l) st_shared16(dst + (uint32_t)l * level, lv[l]);
             }
@@ -975,7 +1041,7 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
         if (!failed && !mbar_wait_bounded(acc_full, 0u)) failed = true;
         tc_fence_after();
         const int quarter = warp & 3, half = (warp - 2) >> 2;
-        for (int h = 0; h < halves && !failed; ++h) {
+        for (int h = 0; h < halves && !failed && half < 2; ++h) {
             const int krow = h * 128 + quarter * 32 + lane;
             if (h * 128 + quarter * 32 >= K) break;  // tcgen05.ld is warp-wide: a warp whose 32 feature rows all lie past K skips it as one
             float* prow = P.part + ((size_t)blockIdx.x * K + krow) * M;
@@ -1000,17 +1066,16 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
 
 // K and M: any (inside, rounded up to 32 with zeros from the copy engine; that is the shape of the partials)
 bool linear_tma_f32_dw_supported(int64_t N, int K, int M, gnn_dtype dtype) {
-    if (dtype != GNN_F32 || N <= 0 || N >= ((int64_t)1 << 31) - FD_ROWS_MAX) return false;
+    if (dtype != GNN_F32 || N <= 0 || N >= ((int64_t)1 << 31) - 32) return false;
     if (K < 1 || K > 512 || M < 1 || M > 256) return false;
     if (up32(M) * ((K + 127) / 128) > 512) return false;  // one accumulator [128, M] per block of 128 features: 512 columns of tensor memory
     return encoder() != nullptr;
 }
 
-// every CTA has at least one slot, so every partial is written
-static int fd_rows(int K, int M) { return (K > 128 || M > 128) ? 16 : 32; }
+// every CTA has at least one slot of 32 rows, so every partial is written
 int linear_tma_f32_dw_partials(int64_t N) {
-    const int64_t nslots = (N + FD_ROWS_MAX - 1) / FD_ROWS_MAX;  // never more CTAs than slots, whichever the slot height
-    return (int)(nslots < 148 ? (nslots > 0 ? nslots : 1) : 148);
+    const int64_t n = (N + 31) / 32;
+    return (int)(n < 148 ? (n > 0 ? n : 1) : 148);
 }
 
 // writes linear_tma_f32_dw_partials(N) fp32 partials [up32(K), up32(M)] to part; X and dY: rows ldx and ldd elements apart
@@ -1019,25 +1084,34 @@ gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, in
     GNN_REQUIRE(aligned16(X) && aligned16(dY) && aligned16(part), GNN_ERR_INVALID_ARG, "%s: matrices must be 16-byte aligned", who);
     const int K = up32(Kr), M = up32(Mr);
     CUtensorMap mapX, mapD;
-    const int R = fd_rows(K, M), ka = (K + 127) / 128 * 128;
-    if (!make_map_f32_ld(&mapX, X, N, Kr, ldx, R) || !make_map_f32_ld(&mapD, dY, N, Mr, ldd, R)) GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
+    const int R = K > 128 || M > 128 ? 16 : 32, ka = (K + 127) / 128 * 128;
     TmaF32DwParams P;
-    P.part = part; P.N = N; P.K = K; P.M = M; P.status = d_flag; P.reset = reset; P.rows = R;
-    const size_t slot = (size_t)(K / 32 + M / 32) * R * 128, ops = 2 * 3 * ((size_t)ka * R * 2 + (size_t)M * R * 2);
+    P.x_whole = Kr % 32 == 0; P.d_whole = Mr % 32 == 0;
+    if (!(P.x_whole ? make_map_f32_blocks : make_map_f32_ld)(&mapX, X, N, Kr, ldx, R) || !(P.d_whole ? make_map_f32_blocks : make_map_f32_ld)(&mapD, dY, N, Mr, ldd, R))
+        GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
+    P.part = part; P.N = N; P.K = K; P.M = M; P.status = d_flag; P.reset = reset;
+    const size_t slot = (size_t)(K / 32 + M / 32) * R * 128, op = 3 * ((size_t)ka * R * 2 + (size_t)M * R * 2);
+    P.groups = R == 16 && 1024 + FD_MAX_GROUPS * (op + slot) <= TM_SMEM_MAX ? FD_MAX_GROUPS : 2;
+    const size_t ops = (size_t)P.groups * op;
     int stages = (int)((TM_SMEM_MAX - 1024 - ops) / slot);
-    P.stages = stages > FD_MAX_STAGES ? FD_MAX_STAGES : stages;
+    if (stages > FD_MAX_STAGES) stages = FD_MAX_STAGES;
+    P.stages = stages / P.groups * P.groups;
     int cols = 32;
     while (cols < M * (ka / 128)) cols <<= 1;
     P.tmem_cols = cols;
-    gnn_status rc = allow_big_smem(who, (const void*)linear_tma_f32_dw_kernel, 12, TM_SMEM_MAX);
+    gnn_status rc = allow_big_smem(who, (const void*)linear_tma_f32_dw_kernel<32>, 12, TM_SMEM_MAX);
+    if (rc == GNN_OK) rc = allow_big_smem(who, (const void*)linear_tma_f32_dw_kernel<16>, 15, TM_SMEM_MAX);
     if (rc != GNN_OK) return rc;
-    launch_overlapped(linear_tma_f32_dw_kernel, dim3((unsigned)linear_tma_f32_dw_partials(N)), dim3(FD_THREADS), 1024 + ops + (size_t)P.stages * slot, st, mapX, mapD, P);
+    launch_overlapped(R == 32 ? linear_tma_f32_dw_kernel<32> : linear_tma_f32_dw_kernel<16>, dim3((unsigned)linear_tma_f32_dw_partials(N)), dim3(FD_THREADS), 1024 + ops + (size_t)P.stages * slot, st, mapX, mapD, P);
     GNN_CHECK_LAUNCH(who);
     return GNN_OK;
 }
 
+// two accumulators and two operand buffers fit the 512 columns of tensor memory
+static bool tf_a_in_tmem(int Mo) { return 2 * ((Mo + 31) & ~31) + 2 * TF_OP_COLS <= 512; }
+
 static size_t tf_fixed_bytes(int Kc, int Mo) {
-    return 1024 + (((size_t)3 * Mo * Kc * 2 + 1023) & ~(size_t)1023) + 2 * 3 * (size_t)TF_LEVEL_BYTES + (size_t)TF_EPI_WARPS * 4096;
+    return 1024 + (((size_t)3 * Mo * Kc * 2 + 1023) & ~(size_t)1023) + (tf_a_in_tmem(Mo) ? 0 : 2 * 3 * (size_t)TF_LEVEL_BYTES) + (size_t)TF_EPI_WARPS * 4096;
 }
 
 // widest block of output columns (a multiple of 16) whose three weight levels fit shared memory beside two slices
@@ -1068,7 +1142,9 @@ gnn_status linear_tma_f32_forward(const void* X, int ldx, const void* W, int64_t
     GNN_REQUIRE(block > 0, GNN_ERR_UNSUPPORTED, "%s: weights do not fit shared memory", who);
     CUtensorMap mapX;
     if (!make_map_f32_ld(&mapX, X, N, Kc, ldx, TC_ROWS)) GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
-    gnn_status rc = allow_big_smem(who, (const void*)linear_tma_f32_kernel, 6, TM_SMEM_MAX);
+    gnn_status rc = allow_big_smem(who, (const void*)linear_tma_f32_kernel<true, 4>, 6, TM_SMEM_MAX);
+    if (rc == GNN_OK) rc = allow_big_smem(who, (const void*)linear_tma_f32_kernel<true, 2>, 13, TM_SMEM_MAX);
+    if (rc == GNN_OK) rc = allow_big_smem(who, (const void*)linear_tma_f32_kernel<false, 2>, 14, TM_SMEM_MAX);
     if (rc != GNN_OK) return rc;
     const int64_t ntiles = (N + TC_ROWS - 1) / TC_ROWS;
     for (int c0 = 0; c0 < Mo; c0 += block) {
@@ -1084,13 +1160,17 @@ gnn_status linear_tma_f32_forward(const void* X, int ldx, const void* W, int64_t
         P.bias = bias ? bias + c0 : nullptr; P.relu = relu;
         P.Y = direct ? (float*)Y + c0 : nullptr; P.ldy = Mo;
         const size_t fixed = tf_fixed_bytes(K16, m16);
-        int stages = (int)((TM_SMEM_MAX - fixed) / TF_SLICE_BYTES);
-        P.stages = stages > TF_MAX_STAGES ? TF_MAX_STAGES : stages;
         P.acc_stride = (m16 + 31) & ~31;
+        const bool a_tmem = tf_a_in_tmem(m16);
+        int stages = (int)((TM_SMEM_MAX - fixed) / TF_SLICE_BYTES);  // at least two
+        if (stages > TF_MAX_STAGES) stages = TF_MAX_STAGES;
+        const int groups = a_tmem && stages >= 4 && 2 * P.acc_stride + 4 * TF_OP_COLS <= 512 ? 4 : 2;
+        P.stages = stages / groups * groups;
         int cols = 32;
-        while (cols < 2 * P.acc_stride) cols <<= 1;
+        while (cols < 2 * P.acc_stride + (a_tmem ? groups * TF_OP_COLS : 0)) cols <<= 1;
         P.tmem_cols = cols;
-        launch_overlapped(linear_tma_f32_kernel, dim3((unsigned)(ntiles < 148 ? ntiles : 148)), dim3(TF_THREADS), fixed + (size_t)P.stages * TF_SLICE_BYTES, st, mapX, mapY, P);
+        launch_overlapped(!a_tmem ? linear_tma_f32_kernel<false, 2> : groups == 4 ? linear_tma_f32_kernel<true, 4> : linear_tma_f32_kernel<true, 2>,
+                          dim3((unsigned)(ntiles < 148 ? ntiles : 148)), dim3(TF_THREADS), fixed + (size_t)P.stages * TF_SLICE_BYTES, st, mapX, mapY, P);
         GNN_CHECK_LAUNCH(who);
     }
     return GNN_OK;

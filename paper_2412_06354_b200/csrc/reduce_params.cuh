@@ -65,6 +65,13 @@ __device__ __forceinline__ void fma2(float& a0, float& a1, float x0, float x1, f
         : "f"(x0), "f"(x1), "f"(w0), "f"(w1));
 }
 
+// d.xy *= w.xy
+__device__ __forceinline__ void mul2(float& a0, float& a1, float w0, float w1) {
+    asm("{\n\t.reg .b64 ra, rc;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rc, {%0, %1};\n\tmul.rn.f32x2 rc, ra, rc;\n\tmov.b64 {%0, %1}, rc;\n\t}"
+        : "+f"(a0), "+f"(a1)
+        : "f"(w0), "f"(w1));
+}
+
 // d.xy += x.xy
 __device__ __forceinline__ void add2(float& a0, float& a1, float x0, float x1) {
     asm("{\n\t.reg .b64 ra, rc;\n\tmov.b64 ra, {%2, %3};\n\tmov.b64 rc, {%0, %1};\n\tadd.rn.f32x2 rc, ra, rc;\n\tmov.b64 {%0, %1}, rc;\n\t}"

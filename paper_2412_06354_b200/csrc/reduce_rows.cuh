@@ -406,7 +406,9 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     const float* const wh_l = HEAD ? P.wh + ((P.vec0 + ci) * EPC) / P.fph : nullptr;
     float acc[EPC];
     int32_t arg[ARG ? EPC : 1];
+    bool fresh = true;  // ARG: the next position is the row's first in this run and is taken whatever its value
     auto clear = [&]() {
+        fresh = true;
 #pragma unroll
         for (int j = 0; j < EPC; ++j) {
             acc[j] = 0.f;
@@ -503,12 +505,14 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
         const float w = HAS_W ? S.w[HAS_W ? i : 0] : 1.0f;
         if (ARG) {
 #pragma unroll
+            for (int k = 0; k < EPC; k += 2) mul2(x[k], x[k + 1], w, w);  // w = 1 where there are no multipliers: exact
+#pragma unroll
             for (int k = 0; k < EPC; ++k) {
-                const float v = w * x[k];  // w = 1 where there are no multipliers: exact
                 // positions ascend within a run: a strict comparison keeps the first of equal values
-                const bool take = arg[ARG ? k : 0] < 0 || (MODE == MODE_MAX ? v > acc[k] : v < acc[k]);
-                if (take) { acc[k] = v; arg[ARG ? k : 0] = cs + i; }
+                const bool take = fresh || (MODE == MODE_MAX ? x[k] > acc[k] : x[k] < acc[k]);
+                if (take) { acc[k] = x[k]; arg[ARG ? k : 0] = cs + i; }
             }
+            fresh = false;
         } else if (ROUTE) {  // keep dOut only where this edge was the winner
             const int t = S.t[ROUTE ? i : 0];
 #pragma unroll
