@@ -16,7 +16,7 @@ namespace cg = cooperative_groups;
 
 namespace gnn {
 
-constexpr int SM_LONG_ROW = 512;  // positions (12 M-edge power-law graph, 8 heads: 2048 is 2 % / 16 % slower forward / backward)
+constexpr int SM_LONG_ROW = 256;  // positions (R-MAT graphs of 5 k to 200 k nodes, 4 and 8 heads: 512 is up to 5 % slower, 128 up to 4 %)
 constexpr int SM_BLOCK = 256;
 
 template <typename T> __device__ __forceinline__ float ld_as_f32(const T* p, size_t i);
@@ -677,7 +677,8 @@ __device__ __forceinline__ void reduce_heads(float (&v)[4 * HV], float* red) {
 }
 
 constexpr int PL_BLOCK = 512;     // threads per long row
-constexpr int PL_LONG_ROW = 1024;  // rows above this many positions get a block instead of a warp (256: +2 % on the attention workload, 2048: +13 %)
+constexpr int PL_LONG_ROW = 512;  // rows above this many positions get a block instead of a warp (R-MAT graphs of 2 k to 200 k nodes, a step of GAT:
+                                   // 1024 is up to 15 % slower, on 20 k nodes and 8 heads 208 against 184 us; 256 up to 5 %)
 // positions per thread and batch (their loads are all in flight together): 32 head values per thread
 __host__ __device__ constexpr int pl_unroll(int HV) { return HV <= 2 ? 4 : (HV == 4 ? 2 : 1); }
 
