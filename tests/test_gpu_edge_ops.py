@@ -261,3 +261,33 @@ def test_pooling_edge_cases(gnn):
     with pytest.raises(gnn.GnnError) as e:
         gnn.graph_ptr_from_ids(to_dev(np.array([0, 1, 5], np.int32)), 3)
     assert e.value.status == 3
+
+
+# Four 256-thread tiles of (edge, 16-byte chunk) pairs per block; the backward pass takes 8 to 128 positions per warp: rows of
+# one chunk, of a number of chunks that divides nothing, and of more than 4096 chunks (64 KB), which divide instead of multiplying
+@pytest.mark.parametrize("e,dtype,F", [(1, "f32", 4), (65, "bf16", 8), (1025, "f32", 4), (700, "bf16", 56), (70_001, "f32", 12), (131_200, "bf16", 24), (525_000, "f32", 4), (67, "f32", 16_420)])
+def test_edge_tensor_tiles(gnn, e, dtype, F):
+    import torch
+    rng = np.random.default_rng(e)
+    n = 50
+    src, dst = rng.integers(0, n, e).astype(np.int32), np.sort(rng.integers(0, n - 3, e)).astype(np.int32)  # edge order = CSR order
+    g = build_graph(gnn, n, src, dst)
+    X, R = feats((n, F), dtype, 900 + F), feats((n, F), dtype, 901 + F)
+    assert np.array_equal(bits(gnn.gather(to_dev(src), to_dev(X))), host_bits(X[src]))
+    f = np.float32(2.0) ** rng.integers(-3, 4, (e, 1)).astype(np.float32)  # powers of two: products are exact
+    m = gnn.apply_edges(g, gnn.E_MUL_XJ, to_dev(X), e=to_dev(f))
+    assert np.array_equal(to_host64(m), to_host64(to_dev(X))[src] * f)
+    assert np.array_equal(bits(gnn.aggregate_backward(g, to_dev(R), "sum")), host_bits(R[dst]))
+    mean = gnn.aggregate_backward(g, to_dev(R), "mean")
+    ref = to_host64(to_dev(R))[dst] / np.bincount(dst, minlength=n)[dst][:, None]
+    assert_close(to_host64(mean), ref, np.abs(ref), dtype, "mean")
+    first = np.searchsorted(dst, np.arange(n))
+    count = np.bincount(dst, minlength=n)
+    win = np.where(count > 0, first + rng.integers(0, 1 << 30, n) % np.maximum(count, 1), -1)
+    arg = np.repeat(win[:, None], F, 1).astype(np.int32)
+    arg[:, ::3] = np.where(count > 0, first, -1)[:, None]
+    want = np.where(arg[dst] == np.arange(e)[:, None], to_host64(to_dev(R))[dst], 0.0)
+    off = torch.empty(n * F + 1, dtype=torch.int32, device="cuda")[1:].view(n, F)  # winners that start off 16 bytes
+    off.copy_(to_dev(arg))
+    for a in (to_dev(arg), off):
+        assert np.array_equal(to_host64(gnn.aggregate_backward(g, to_dev(R), "max", argmax=a)), want)

@@ -159,3 +159,11 @@ def test_linear_back_to_back_launches_are_bitwise_identical(gnn, dtype):
     assert status_word(ws) == 0
     assert torch.equal(Y.view(torch.int16 if dtype == "bf16" else torch.int32), Y0.view(torch.int16 if dtype == "bf16" else torch.int32))
     assert torch.equal(dX.float(), dX0.float()) and torch.equal(dW.float(), dW0.float())
+
+
+# Blocks of output columns side by side (width a multiple of 16 that is not one of 32, a last block that is narrower), blocks of
+# 32 columns for few rows, four and two converter groups, dW in slots of 16 and 32 rows with four and two groups
+@pytest.mark.parametrize("dtype,n,K,M", [("f32", 9700, 256, 256), ("f32", 19100, 64, 224), ("f32", 9601, 480, 140), ("f32", 2000, 128, 128),
+                                         ("f32", 5000, 160, 160), ("f32", 257, 128, 192), ("f32", 700, 512, 128), ("bf16", 515, 64, 64)])
+def test_linear_column_blocks(gnn, dtype, n, K, M):
+    test_linear_ragged_sizes(gnn, dtype, n, K, M)

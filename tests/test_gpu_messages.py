@@ -286,3 +286,10 @@ def test_gatv2_backward_without_workspace(gnn, dtype, H, C):
     rb = oracle.gatv2_logits_backward(n, src, dst, Xl, Xr, a, H, ds)
     assert_close(to_host64(dXl), rb["dXl"], rb["SXl"], dtype, "GATv2 dXl")
     assert_close(to_host64(dXr), rb["dXr"], rb["SXr"], dtype, "GATv2 dXr")
+
+
+@pytest.mark.parametrize("dtype,H,C", [("bf16", 8, 8), ("f32", 8, 4), ("f32", 4, 8), ("bf16", 16, 16)])
+def test_edge_values_of_heads_of_one_and_two_chunks(gnn, dtype, H, C):
+    """Fewer lanes per result than positions in a register buffer: the fold over a head's lanes takes its other form."""
+    test_xi_dot_xj(gnn, dtype, H, C)
+    test_gatv2_logits_forward_backward(gnn, dtype, H, C)

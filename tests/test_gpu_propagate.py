@@ -434,3 +434,60 @@ def test_low_mean_degree_above_8mi_edges_takes_positions_first(gnn, dtype, F):
         assert_close(to_host64(dX[torch.from_numpy(srows).cuda()]), bw["dX"], bw["SdX"], dtype, "backward of the mean")
     finally:
         oracle.set_threads(1)
+
+
+# Positions first: a warp takes 32 to 256 positions and a block eight times as many.  Edge counts at and beside a warp's and a
+# block's share, every lane layout (rows of 16 to 512 bytes), rows of two and three 512-byte column slabs
+@pytest.mark.parametrize("e,dtype,F", [(1, "f32", 64), (256, "f32", 128), (257, "bf16", 128), (511, "bf16", 8), (513, "f32", 4), (2047, "f32", 32),
+                                       (4127, "bf16", 24), (1023, "f32", 200), (777, "bf16", 264), (131072 + 513, "bf16", 16), (525_000, "f32", 8)])
+def test_rows_cut_at_every_kind_of_boundary(gnn, e, dtype, F):
+    """Rows that end exactly at a warp's share, one position later, one row that holds everything, and short rows of every
+    length up to 33 with few edges per node (a lane group per row): forward, backward and the edge-weight gradient."""
+    rng = np.random.default_rng(e)
+    for lens in (np.full(e // 32 + 1, 32), np.full(e // 33 + 1, 33), np.array([0, e, 0]), np.resize(np.r_[np.arange(34), np.zeros(120, int)], 9000)):
+        dst = np.repeat(np.arange(len(lens)), lens)[:e].astype(np.int32)
+        m, n = len(dst), len(lens)
+        src = rng.integers(0, n, m).astype(np.int32)
+        g = build_graph(gnn, n, src, dst)
+        ref = host_csr(n, src, dst)
+        eid = ref["eid"]
+        X, R = feats((n, F), dtype, 500 + F), feats((n, F), dtype, 501 + F)
+        w = synth.uniform_f32((m,), 0.0, 1.0, 502)
+        Xd, Rd = to_dev(X), to_dev(R)
+        o, S, _ = oracle.propagate("sum", n, src, dst, X, w)
+        assert_close(to_host64(gnn.propagate_fused(g, Xd, to_dev(w[eid]), "sum")), o, S, dtype, "sum")
+        o, S, _ = oracle.propagate("mean", n, src, dst, X)
+        assert_close(to_host64(gnn.propagate_fused(g, Xd, None, "mean")), o, S, dtype, "mean")
+        out, arg = gnn.propagate_fused(g, Xd, None, "max")
+        o, _, a = oracle.propagate("max", n, src, dst, X)
+        ga = arg.cpu().numpy()
+        assert np.array_equal(bits(out), f64_to_dtype_bits(o, dtype)) and np.array_equal(np.where(ga >= 0, eid[np.maximum(ga, 0)], -1), a)
+        dX, dW = gnn.propagate_fused_backward(g, Rd, "mean", X=Xd, w_csrT=to_dev(w[ref["eidT"]]), want_dW=True)
+        bw = oracle.propagate_backward("mean", n, src, dst, X, w, R, want_dw=True)
+        assert_close(to_host64(dX), bw["dX"], bw["SdX"], dtype, "dX of the mean")
+        assert_close(to_host64(dW), bw["dw"][eid], bw["Sdw"][eid], "f32", "dW of the mean")
+        dX, _ = gnn.propagate_fused_backward(g, Rd, "max", argmax=arg)
+        bw = oracle.propagate_backward("max", n, src, dst, X, None, R, arg=a)
+        assert_close(to_host64(dX), bw["dX"], bw["SdX"], dtype, "dX of max")
+
+
+# Sort digits of 10 bits (ids at 2^10 and 2^20), tiles of 2048 edges, rows over 512 positions for the degrees, edge counts
+# that are no multiple of a vector
+@pytest.mark.parametrize("n,e", [(1023, 2047), (1024, 2048), (1025, 2049), (1 << 20, 4097), ((1 << 20) + 1, 6143), (3, 5001)])
+def test_setup_at_digit_and_tile_boundaries(gnn, n, e):
+    rng = np.random.default_rng(n + e)
+    src, dst = rng.integers(0, n, e).astype(np.int32), rng.integers(0, n, e).astype(np.int32)
+    src[:2], dst[:2] = (0, n - 1), (n - 1, 0)
+    dst[e // 2: e // 2 + 700] = n // 2
+    g = build_graph(gnn, n, src, dst)
+    ref = host_csr(n, src, dst)
+    for k, v in ref.items():
+        got = getattr(g, k).cpu().numpy()
+        assert np.array_equal(got if k.startswith("rowptr") else got[:e], v), k
+    w = synth.uniform_f32((e,), 0.5, 1.0, 31)
+    deg, coef, coefT = gnn.gcn_norm(g, to_dev(w[ref["eid"]]))
+    d = np.bincount(dst, weights=w.astype(np.float64), minlength=n)
+    assert_close(to_host64(deg), d, d, "f32", "weighted degrees")
+    c = np.where((d[src] > 0) & (d[dst] > 0), w / np.sqrt(np.maximum(d[src], 1e-300) * np.maximum(d[dst], 1e-300)), 0.0)
+    assert_close(to_host64(coef), c[ref["eid"]], c[ref["eid"]], "f32", "coefficients")
+    assert_close(to_host64(coefT), c[ref["eidT"]], c[ref["eidT"]], "f32", "transposed coefficients")
