@@ -34,7 +34,7 @@ UNIT = "edges*feat/s"
 ALL_CASES = [(F, dt) for dt in ("bf16", "f32") for F in (32, 64, 128, 256, 512)]
 FMAX = 512
 
-# DRAM bytes (read + write, GB) of one gnn_propagate_fused / _backward call (all its propagate_chunk_kernel and
+# DRAM bytes (read + write, GB) of one gnn_propagate_fused / _backward call (all its reduction and
 # fix-up launches: wide rows run as 512-byte column slabs), taken with the hardware counters
 # dram__bytes_read.sum + dram__bytes_write.sum on a REDUCED graph of the same generator (--graph-scale 20:
 # N = 600,000, E = 30,750,000, a quarter of the workload) so that the capture stays small.  The line reports
@@ -43,11 +43,11 @@ FMAX = 512
 # its gathers hits (a full-size capture of an earlier build of the same loop gave 79.6 GB where this gives 32.8).
 # The numbers belong to the kernel sources whose digest is TRAFFIC_KERNEL_SHA256; with other sources the line
 # reports traffic = null.
-TRAFFIC_SOURCE = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none -k regex:propagate_ over one step of "
+TRAFFIC_SOURCE = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none -k regex:rows_kernel over one step of "
                   "`bench.py --graph-scale 20` (N=600000, E=30.75M), scaled by 4.0 = ratio of edges*features; lower bound of the "
                   "full-size traffic (better L2 reuse on the reduced matrix); summary under profiles/")
 TRAFFIC_SCALE = 4.0
-TRAFFIC_KERNEL_FILES = ("propagate.cu", "propagate.cuh", "common.cuh")
+TRAFFIC_KERNEL_FILES = ("propagate.cu", "propagate.cuh", "reduce_params.cuh", "reduce_rows.cuh", "common.cuh")
 TRAFFIC_KERNEL_SHA256 = "62facf4d2c659f955d3468cd3144d3ed4b685ffbeb12d73cf41affba107fcf9c"
 TRAFFIC_GB_REDUCED = {
     "32:bf16:copy_xj:fwd": 0.192,
@@ -449,7 +449,7 @@ def main():
     traffic = TRAFFIC_GB.get(tkey) if traffic_valid else None
     achieved = comp / dom["fwd_ms"] / 1e6
     nslab = max(1, dom["F"] * sdom // 512)
-    roofline = {"bound": "hbm", "kernel": "propagate_chunk_kernel, forward call of F=%d %s %s = %d column-slab launch(es) + fix-up (largest share of the step: %.1f %%); bytes, time and traffic are per call"
+    roofline = {"bound": "hbm", "kernel": "stream_rows_kernel, forward call of F=%d %s %s = %d column-slab launch(es) + fix-up (largest share of the step: %.1f %%); bytes, time and traffic are per call"
                 % (dom["F"], dom["dtype"], dom["msg"], nslab, 100 * (dom["fwd_ms"] + dom["bwd_ms"]) / tot_ms),
                 "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
                 "traffic": None if traffic is None else traffic * 1e9,
@@ -500,10 +500,8 @@ def main():
 
 
 def launches_per_pass(E):
-    """Kernels one column-slab pass of a sum launches: the chunk kernel, the fix-up of cut rows and, on graphs of
-    16384 chunks and more, the fix-up of hub rows (chunks are 1024 positions from 8 Mi edges on, 256 below)."""
-    chunk = 1024 if E >= 8 * 1024 * 1024 else 256
-    return 3 if -(-E // chunk) >= 16384 else 2
+    """Kernels one column-slab pass of a sum launches: the reduction and the fix-up of rows cut between its blocks."""
+    return 2
 
 
 def run_e2e(args, torch, gnn, g, plan, hX, hR, w_csr, w_csrT, ws, N, E, fmax, dev, world, barrier):
