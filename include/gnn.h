@@ -147,11 +147,11 @@ gnn_status gnn_permute_edge_data(const int32_t* perm, int64_t E, int width, int 
  * MAX / MIN (element-wise; argmax int32 [N,F] receives the CSR position of the winner, the
  * smallest position among equal values; may be NULL).  A node with no incoming edge gets 0 and
  * argmax -1.  X, out: [N,F] of dtype.  ws: at least gnn_propagate_fused_workspace bytes, asked for the E and
- * the F of this very call: the edges-per-chunk of the reduction steps with the graph size and the row width,
+ * the F of this very call: the positions per partial row step with the graph size and the row width,
  * so the size is monotone neither in E nor in F (a workspace sized for a larger graph, or for wider rows, can
  * be too small; take the maximum over the calls that share it).
- * Which of the two reduction kernels runs (rows walked one by one, or positions first) is a fixed function of
- * N, E, F, dtype and op (small graphs and, for sums, large graphs of low mean degree take positions first);
+ * Which of the two reduction kernels runs (positions first, or a row per lane group on small graphs of short
+ * rows) is a fixed function of N, E, F, dtype and op;
  * results are bit-reproducible for a given graph and shape.
  * Bytes moved per call: at least 4E (+4E with weights) + 8N + 2*N*F*s, at most
  * 4E (+4E) + 8N + (E+N)*F*s when no source row is found in L2. */

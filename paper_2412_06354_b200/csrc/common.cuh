@@ -88,18 +88,9 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
     return p;
 }
-#ifndef PF_L1_POLICY
-#define PF_L1_POLICY 0
-#endif
 __device__ __forceinline__ uint4 ld_hint16(const void* p, uint64_t pol) {
     uint4 v;
-#if PF_L1_POLICY == 0
     asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
-#elif PF_L1_POLICY == 1
-    asm volatile("ld.global.nc.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
-#else
-    asm volatile("ld.global.nc.L1::evict_last.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
-#endif
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                  : "l"(p), "l"(pol));
     return v;
@@ -107,11 +98,6 @@ __device__ __forceinline__ uint4 ld_hint16(const void* p, uint64_t pol) {
 __device__ __forceinline__ int ld_hint_i32(const int* p, uint64_t pol) {
     int v;
     asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.s32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
-    return v;
-}
-__device__ __forceinline__ float ld_hint_f32(const float* p, uint64_t pol) {
-    float v;
-    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.f32 %0, [%1], %2;" : "=f"(v) : "l"(p), "l"(pol));
     return v;
 }
 __device__ __forceinline__ int ld_stream_i32(const int* p) {

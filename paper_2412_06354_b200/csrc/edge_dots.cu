@@ -38,7 +38,7 @@ constexpr int ED_H = 4;      // positions per register buffer
 
 template <bool MEAN>
 struct EdgeStage {
-    int col[ED_SUB];           // gathered row; sign bit: last position of a row
+    alignas(16) int col[ED_SUB + 32];  // gathered row; sign bit: last position of a row; four words further for every lane group before it
     int row[ED_SUB + 1];       // [q] the q-th row with positions in the warp's share
     uint16_t start[ED_SUB + 2];
     float inv[MEAN ? ED_SUB + 1 : 1];  // [q] 1 / length of that row
@@ -58,20 +58,24 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
     const int cs = c * P.sub, n = (int)min((int64_t)P.sub, P.E - cs);
     const bool col_lane = li < P.nvec;
     const int ci = col_lane ? li : 0;
+    // skewed as in the segmented reduction: the groups' runs are in different banks, and four entries are one load
+    const int L = P.sub / NG, lsh = 31 - __clz(L);
+    auto sk = [&](int i) { return i + ((i >> lsh) << 2); };
     for (int i = lane; i < n; i += 32)
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(S.col + i)), "l"(P.col + cs + i) : "memory");
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(S.col + sk(i))), "l"(P.col + cs + i) : "memory");
     bool began_before;
     const int m = stage_rows(P.rowptr, P.N, P.E, cs, n, lane, S.row, S.start, began_before);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncwarp();
     for (int q = lane; q < m; q += 32) {
         const int e = S.start[q + 1];
-        if (e <= n) S.col[e - 1] |= (int)0x80000000;
+        if (e <= n) S.col[sk(e - 1)] |= (int)0x80000000;
         if (MEAN) S.inv[MEAN ? q : 0] = 1.0f / (float)(P.rowptr[S.row[q] + 1] - P.rowptr[S.row[q]]);
     }
     __syncwarp();
 
-    const int L = P.sub / NG, a = g * L, b = min(a + L, n);
+    const int a = g * L, b = min(a + L, n);
+    const int* const Sc = S.col + 4 * g;
     const uint64_t pol_keep = policy_evict_last();
     const uint32_t row_bytes = (uint32_t)P.nvec * 16;
     const char* const Xl = reinterpret_cast<const char*>(P.X) + (size_t)ci * 16;
@@ -104,13 +108,15 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
         if (MEAN && q < m) sc = S.inv[MEAN ? q : 0];
         if (q + 1 < m) own_next = own(q + 1);
     };
-    for (int i = n + lane; i < P.sub; i += 32) S.col[i] = 0;  // the last warp: positions past the end gather row 0
+    for (int i = n + lane; i < P.sub; i += 32) S.col[sk(i)] = 0;  // the last warp: positions past the end gather row 0
     __syncwarp();
     auto issue = [&](uint4* x, int i) -> unsigned {
         unsigned ends = 0;
+        const int4 c4 = V2 ? make_int4(Sc[i], Sc[i + 1], Sc[i + 2], Sc[i + 3]) : *reinterpret_cast<const int4*>(Sc + i);
+        const int ccs[H] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
         for (int u = 0; u < H; ++u) {
-            const int cc = S.col[i + u];
+            const int cc = ccs[u];
             ends |= ((unsigned)cc >> 31) << u;
             x[u] = ld_hint16(Xl + (size_t)(uint32_t)(cc & 0x7fffffff) * row_bytes, pol_keep);
         }

@@ -114,7 +114,7 @@ gnn_status run_chunked(const char* who, int mode, int32_t N, int64_t E, const in
     const int nvec = F * s / 16;
     GNN_REQUIRE(nvec <= 128, GNN_ERR_UNSUPPORTED, "%s: feature rows wider than 2048 bytes are not supported (F=%d)", who, F);
     GNN_REQUIRE(aligned16(X) && aligned16(out), GNN_ERR_INVALID_ARG, "%s: feature matrices must be 16-byte aligned", who);
-    GNN_REQUIRE(E >= 0 && E < ((int64_t)1 << 31) - 4 * PF_SLAB, GNN_ERR_UNSUPPORTED, "%s: positions must fit 32 bits (E < 2^31)", who);
+    GNN_REQUIRE(E >= 0 && E < ((int64_t)1 << 31) - 1024, GNN_ERR_UNSUPPORTED, "%s: positions must fit 32 bits (E < 2^31)", who);
     const bool with_arg = (mode == MODE_MAX || mode == MODE_MIN);
     const size_t need = chunked_workspace(E, F, with_arg);
     GNN_REQUIRE(ws && ws_bytes >= need && aligned16(ws), GNN_ERR_WORKSPACE_TOO_SMALL,

@@ -4,9 +4,6 @@
 
 namespace gnn {
 
-constexpr int PF_SLAB = 256;   // positions per warp of the edge-wise dot products
-constexpr int PF_WARPS = 8;    // warps per block
-
 enum { MODE_SUM = 0, MODE_MAX = 1, MODE_MIN = 2, MODE_ROUTE = 3, MODE_HEADSUM = 4, MODE_EFSUM = 5, MODE_WSUM = 6, MODE_V2 = 7 };
 
 // MODE_HEADSUM extras: multipliers per (position, head) and an optional rank-1 row epilogue

@@ -316,12 +316,14 @@ reduce_rows_kernel(const __grid_constant__ PropParams P, int long_blocks) {
 // 512-byte rows 113 -> 75 us, bf16 256-byte 74 -> 60 us, 64-byte 54 -> 32 us, max fp32 157 -> 117 us; on 123 M edges the
 // 128-byte rows of a weighted sum 2.45 -> 2.26 ms, max over 256-byte rows 8.1 -> 6.6 ms.
 constexpr int RS_SUB = 256;  // most positions per warp
+constexpr int RS_SKEW = 32;
 
 template <int EPC, bool HAS_W, bool HAS_T, bool ARG>
-struct StreamStage {
-    int col[RS_SUB];                       // gathered row; sign bit: last position of a row
-    float w[HAS_W ? RS_SUB : 1];           // multiplier
-    int t[HAS_T ? RS_SUB : 1];             // ROUTE: forward position; HEAD: row of the multiplier matrix
+struct alignas(16) StreamStage {
+    // per position; four words further for every lane group before the position's (see sk)
+    int col[RS_SUB + RS_SKEW];                         // gathered row; sign bit: last position of a row
+    alignas(16) float w[HAS_W ? RS_SUB + RS_SKEW : 1]; // multiplier
+    alignas(16) int t[HAS_T ? RS_SUB + RS_SKEW : 1];   // ROUTE: forward position; HEAD: row of the multiplier matrix
     int row[RS_SUB + 1];                   // [q] the q-th row with positions in the warp's share
     uint16_t start[RS_SUB + 2];            // [q] its first position in the warp's share; [count]: end of the last, or n + 1 if it is cut
     float head[32 * EPC];                  // per lane: sum of a group's (then the warp's) first row, which began before it
@@ -360,21 +362,27 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     const bool col_lane = li < P.nvec;
     const int ci = col_lane ? li : 0;
 
+    // The groups' runs start sub / NG positions apart: at a multiple of 32 words they would read the same bank at the same
+    // time (eight-way conflicts with 64-byte rows, four-way with 128-byte rows: 90 % of the shared-memory path's cycles).  Four
+    // words of skew per group keep the runs apart and on 16 bytes, so that a register buffer's entries are one load.
+    const int L = P.sub / NG, lsh = 31 - __clz(L);
+    auto sk = [&](int i) { return i + ((i >> lsh) << 2); };
     {  // ---- indices and multipliers, asynchronously while the rows are looked up
         auto copy = [&](void* dst, const void* src) {
             asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
         };
         for (int i = lane; i < n; i += 32) {
-            if (P.col) copy(S.col + i, P.col + cs + i);
-            else S.col[i] = cs + i;
+            const int k = sk(i);
+            if (P.col) copy(S.col + k, P.col + cs + i);
+            else S.col[k] = cs + i;
             if (HAS_W) {
-                if (P.w) copy(S.w + i, P.w + cs + i);
-                else S.w[i] = 1.0f;
+                if (P.w) copy(S.w + k, P.w + cs + i);
+                else S.w[k] = 1.0f;
             }
-            if (ROUTE) copy(S.t + i, P.route_pos + cs + i);
+            if (ROUTE) copy(S.t + k, P.route_pos + cs + i);
             if (HEAD) {
-                if (P.wh_index) copy(S.t + i, P.wh_index + cs + i);
-                else S.t[i] = cs + i;
+                if (P.wh_index) copy(S.t + k, P.wh_index + cs + i);
+                else S.t[k] = cs + i;
             }
         }
     }
@@ -387,20 +395,27 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     if (HAS_W && P.gscale_rowptr) {
 #pragma unroll 4
         for (int i = lane; i < n; i += 32) {
-            const int cc = S.col[i];
+            const int k = sk(i), cc = S.col[k];
             const int64_t d = P.gscale_rowptr[cc + 1] - P.gscale_rowptr[cc];
-            S.w[i] = S.w[i] / (float)(d > 1 ? d : 1);
+            S.w[k] = S.w[k] / (float)(d > 1 ? d : 1);
         }
         __syncwarp();
     }
     for (int q = lane; q < m; q += 32) {
         const int e = S.start[q + 1];
-        if (e <= n) S.col[e - 1] |= (int)0x80000000;
+        if (e <= n) S.col[sk(e - 1)] |= (int)0x80000000;
     }
     __syncwarp();
 
     // ---- this group's run
-    const int L = P.sub / NG, a = g * L, b = min(a + L, n);
+    const int a = g * L, b = min(a + L, n);
+    const int* const Sc = S.col + 4 * g;
+    const float* const Sw = S.w + (HAS_W ? 4 * g : 0);
+    const int* const St = S.t + (ROUTE || HEAD ? 4 * g : 0);
+    auto words = [&](int* to, const void* from) {  // H staged words, on their own size
+        if (H == 4) *reinterpret_cast<int4*>(to) = *reinterpret_cast<const int4*>(from);
+        else *reinterpret_cast<int2*>(to) = *reinterpret_cast<const int2*>(from);
+    };
     const uint64_t pol_keep = policy_evict_last();
     const char* const Xl = reinterpret_cast<const char*>(P.X) + (size_t)ci * 16;
     const float* const wh_l = HEAD ? P.wh + ((P.vec0 + ci) * EPC) / P.fph : nullptr;
@@ -475,13 +490,21 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     // the gathers of positions i .. i + H - 1; a bit per row end
     auto issue = [&](Buf& B, int i) -> unsigned {
         unsigned ends = 0;
+        alignas(16) int ccs[H], ts[H];
+        if (PLAIN && EPC == 8) {  // one by one: four at a time cost these the registers they have left (59 -> 61 us on 1.36 M 256-byte rows)
+#pragma unroll
+            for (int u = 0; u < H; ++u) ccs[u] = Sc[i + u];
+        } else {
+            words(ccs, Sc + i);
+        }
+        if (HEAD) words(ts, St + (HEAD ? i : 0));
 #pragma unroll
         for (int u = 0; u < H; ++u) {
-            int cc = S.col[i + u];
+            int cc = ccs[u];
             ends |= ((unsigned)cc >> 31) << u;
             cc &= 0x7fffffff;
             B.x[u] = ld_hint16(Xl + (size_t)(uint32_t)cc * P.x_ld, pol_keep);
-            if (HEAD) B.hw[HEAD ? u : 0][0] = __ldg(wh_l + (size_t)(uint32_t)S.t[HEAD ? i + u : 0] * P.H);
+            if (HEAD) B.hw[HEAD ? u : 0][0] = __ldg(wh_l + (size_t)(uint32_t)ts[u] * P.H);
             if (EF) {
                 const float4* f = reinterpret_cast<const float4*>(P.ef + (size_t)(cs + i + u) * P.ef_ld + (size_t)ci * EPC);
 #pragma unroll
@@ -499,10 +522,9 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
         }
         return ends;
     };
-    auto use = [&](const Buf& B, int u, int i) {  // entry u of the buffer, position i of the piece
+    auto use = [&](const Buf& B, int u, int i, float w, int t) {  // entry u of the buffer, position i of the piece
         float x[EPC];
         Chunk<T>::unpack(B.x[u], x);
-        const float w = HAS_W ? S.w[HAS_W ? i : 0] : 1.0f;
         if (ARG) {
 #pragma unroll
             for (int k = 0; k < EPC; k += 2) mul2(x[k], x[k + 1], w, w);  // w = 1 where there are no multipliers: exact
@@ -514,7 +536,6 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
             }
             fresh = false;
         } else if (ROUTE) {  // keep dOut only where this edge was the winner
-            const int t = S.t[ROUTE ? i : 0];
 #pragma unroll
             for (int k = 0; k < EPC / 4; ++k) {
                 const int4 z = B.win[ROUTE ? u : 0][ROUTE ? k : 0];
@@ -546,6 +567,17 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
             for (int k = 0; k < EPC; k += 2) fma2(acc[k], acc[k + 1], x[k], x[k + 1], f, f);
         }
     };
+    auto use_all = [&](const Buf& B, unsigned ends, int i) {
+        alignas(16) float ws[H];
+        alignas(16) int ts[H];
+        if (HAS_W) words(reinterpret_cast<int*>(ws), Sw + (HAS_W ? i : 0));
+        if (ROUTE) words(ts, St + (ROUTE ? i : 0));
+#pragma unroll
+        for (int u = 0; u < H; ++u) {
+            use(B, u, i + u, HAS_W ? ws[u] : 1.0f, ROUTE ? ts[u] : 0);
+            if (ends >> u & 1u) flush();
+        }
+    };
     if (a < b) {
         Buf A, B;
         // L is a multiple of 2 H: only the last piece of the graph has a remainder
@@ -558,28 +590,20 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
 #pragma unroll 1
         for (; i + 2 * H <= b; i += 2 * H) {
             const bool more = i + 4 * H <= b;
-#pragma unroll
-            for (int u = 0; u < H; ++u) {
-                use(A, u, i + u);
-                if (ea >> u & 1u) flush();
-            }
+            use_all(A, ea, i);
             if (more) ea = issue(A, i + 2 * H);
-#pragma unroll
-            for (int u = 0; u < H; ++u) {
-                use(B, u, i + H + u);
-                if (eb >> u & 1u) flush();
-            }
+            use_all(B, eb, i + H);
             if (more) eb = issue(B, i + 3 * H);
         }
 #pragma unroll 1
         for (; i < b; ++i) {
             // one at a time: entry 0 of a buffer whose other entries repeat it
             Buf R;
-            int cc = S.col[i];
+            int cc = Sc[i];
             const bool end = cc < 0;
             cc &= 0x7fffffff;
             R.x[0] = ld_hint16(Xl + (size_t)(uint32_t)cc * P.x_ld, pol_keep);
-            if (HEAD) R.hw[0][0] = __ldg(wh_l + (size_t)(uint32_t)S.t[HEAD ? i : 0] * P.H);
+            if (HEAD) R.hw[0][0] = __ldg(wh_l + (size_t)(uint32_t)St[HEAD ? i : 0] * P.H);
             if (EF) {
 #pragma unroll
                 for (int k = 0; k < MW; ++k) R.hw[0][k] = P.ef[(size_t)(cs + i) * P.ef_ld + (size_t)ci * EPC + k];
@@ -589,12 +613,12 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
                 for (int k = 0; k < EPC / 4; ++k)
                     R.win[0][ROUTE ? k : 0] = __ldg(reinterpret_cast<const int4*>(P.route_arg + (size_t)(uint32_t)cc * P.arg_ld + (size_t)ci * EPC) + k);
             }
-            use(R, 0, i);
+            use(R, 0, i, HAS_W ? Sw[HAS_W ? i : 0] : 1.0f, ROUTE ? St[ROUTE ? i : 0] : 0);
             if (end) flush();
         }
     }
     // ---- what the groups leave: a closed head (parked), and the sum of a row that goes on past the group (in acc)
-    const bool rest = a < b && S.col[b - 1] >= 0;
+    const bool rest = a < b && Sc[b - 1] >= 0;
     int head_state = HEAD_NONE, tail_row = -1;
     __syncwarp();
     // the warp's first or last row, as far as it lies here, for the block (lanes below LPR)

@@ -899,13 +899,16 @@ static int row_grid_sub(int N) {
 }
 
 // The three row tiers (8 threads, a warp, a block per row) touch disjoint rows and none of them fills the
-// machine alone (the block tier runs two blocks per SM and is as long as its longest row).  They run side by
-// side: the block tier on the caller's stream, the other two on two helper streams that are forked from the
+// machine alone (the block tier runs one or two blocks per SM and is as long as its longest row).  They run side by
+// side: the warp tier on the caller's stream, the other two on two helper streams that are forked from the
 // caller's stream and joined back into it with events, so the call keeps its place in the caller's stream order.
+// The block tier's stream has the higher priority: its blocks need a whole SM's registers and, where the small blocks
+// of the other tiers came first (which it was differed from process to process), started when those were done (a GAT
+// step on 100k nodes and 8 heads: 752 or 835 us).
 // The helper streams and events are created on the first call on a device (make that call outside any stream
 // capture); if they cannot be had, the tiers run one after the other.
 struct TierStreams {
-    cudaStream_t s[2];
+    cudaStream_t s[2], first;
     cudaEvent_t fork, join[2];
     int state;  // 0: not tried, 1: ready, -1: unavailable
 };
@@ -919,8 +922,11 @@ static TierStreams* tier_streams() {
     if (cudaGetDevice(&dev) == cudaSuccess && dev >= 0 && dev < 64) {
         t = &g_tier[dev];
         if (t->state == 0) {
-            bool ok = cudaStreamCreateWithFlags(&t->s[0], cudaStreamNonBlocking) == cudaSuccess &&
+            int low = 0, high = 0;
+            bool ok = cudaDeviceGetStreamPriorityRange(&low, &high) == cudaSuccess &&
+                      cudaStreamCreateWithFlags(&t->s[0], cudaStreamNonBlocking) == cudaSuccess &&
                       cudaStreamCreateWithFlags(&t->s[1], cudaStreamNonBlocking) == cudaSuccess &&
+                      cudaStreamCreateWithPriority(&t->first, cudaStreamNonBlocking, high) == cudaSuccess &&
                       cudaEventCreateWithFlags(&t->fork, cudaEventDisableTiming) == cudaSuccess &&
                       cudaEventCreateWithFlags(&t->join[0], cudaEventDisableTiming) == cudaSuccess &&
                       cudaEventCreateWithFlags(&t->join[1], cudaEventDisableTiming) == cudaSuccess;
@@ -956,16 +962,16 @@ template <class Long, class Warp, class Sub>
 static void run_row_tiers(cudaStream_t st, Long run_long, Warp run_warp, Sub run_sub) {
     std::lock_guard<std::mutex> lock(g_tier_mutex);  // one host thread at a time forks and joins through the shared events
     TierStreams* t = tier_streams();
-    if (!t || cudaEventRecord(t->fork, st) != cudaSuccess || cudaStreamWaitEvent(t->s[0], t->fork, 0) != cudaSuccess ||
+    if (!t || cudaEventRecord(t->fork, st) != cudaSuccess || cudaStreamWaitEvent(t->first, t->fork, 0) != cudaSuccess ||
         cudaStreamWaitEvent(t->s[1], t->fork, 0) != cudaSuccess) {
         (void)cudaGetLastError();
         run_long(st); run_warp(st); run_sub(st);
         return;
     }
-    run_long(st);
-    run_warp(t->s[0]);
+    run_long(t->first);
+    run_warp(st);
     run_sub(t->s[1]);
-    cudaEventRecord(t->join[0], t->s[0]);
+    cudaEventRecord(t->join[0], t->first);
     cudaEventRecord(t->join[1], t->s[1]);
     cudaStreamWaitEvent(st, t->join[0], 0);
     cudaStreamWaitEvent(st, t->join[1], 0);
