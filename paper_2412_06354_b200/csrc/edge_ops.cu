@@ -36,7 +36,7 @@ __device__ __forceinline__ void block_span(int64_t total, int64_t* t0, int64_t* 
 // the rest divide a number below nvec + EO_U * 256 by a multiplication (see over_nvec).  A thread that walked the grid's stride with one pair at a
 // time took 86 us to gather 1.36 M rows of 256 bytes; floor for writing them 54 us.
 constexpr int EO_U = 4;
-// x / nvec; magic = 2^32 / nvec rounded up, which is exact while x * nvec < 2^32: the callers' x is below 128 * nvec, so
+// x / nvec; magic = 2^32 / nvec rounded up, which is exact while x * nvec < 2^32: the callers' x is below nvec + 1024, so
 // rows of up to 4096 chunks have one and the others, and rows of one chunk, divide.
 __device__ __forceinline__ uint32_t over_nvec(uint32_t x, uint32_t nvec, uint32_t magic) { return magic ? __umulhi(x, magic) : x / nvec; }
 static uint32_t pair_magic(int nvec) { return nvec > 1 && nvec <= 4096 ? (uint32_t)((((uint64_t)1 << 32) + nvec - 1) / nvec) : 0; }
@@ -143,80 +143,80 @@ __global__ void gat_logit_kernel(const int64_t* __restrict__ rowptr, const int32
 }
 
 // backward of aggregate w.r.t. the messages: dm[p, :] from dOut[row(p), :].  A warp looks up the rows of its share of
-// positions once, notes each position's row in shared memory and then writes (position, chunk) pairs, four per lane in
-// flight.  Bound by the writes; looking the row up per pair, one pair at a time, took 160 us for 1.36 M rows of 256 bytes.
+// positions once; lpr lanes cover a row (of more than 32 chunks: 32 of them at a time) and its lane groups take equal runs
+// of the share, each row's dOut and winners held in registers while its positions are written, the next row's on their way.
+// Bound by the writes.  1.36 M rows of 256 bytes, max: 160 us with a search per chunk, 119 us with a load of dOut and
+// winners per position and chunk (the L1 path was busy 77 % of the time), 86 us now; writing them takes 54 us.
 constexpr int AB_SUB = 128;  // most positions per warp
 template <typename T>
-__global__ void __launch_bounds__(256) aggregate_backward_kernel(const int64_t* __restrict__ rowptr, int N, int64_t E, int op, int sub, bool wide,
+__global__ void __launch_bounds__(256) aggregate_backward_kernel(const int64_t* __restrict__ rowptr, int N, int64_t E, int op, int sub, int lpr, bool wide,
                                                                  const uint4* __restrict__ dOut, const int32_t* __restrict__ argmax,
-                                                                 int nvec, uint32_t magic, uint4* __restrict__ dm) {
-    constexpr int EPC = Chunk<T>::N, U = 4;
-    __shared__ int s_rows[8][AB_SUB + 1], s_row[8][AB_SUB];
+                                                                 int nvec, uint4* __restrict__ dm) {
+    constexpr int EPC = Chunk<T>::N;
+    __shared__ int s_rows[8][AB_SUB + 1];
     __shared__ uint16_t s_start[8][AB_SUB + 2];
     pdl_wait();
-    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, g = lane / lpr;
     const int64_t c = (int64_t)blockIdx.x * 8 + wib;
     if (c * sub >= E) return;
     const int cs = (int)(c * sub), n = (int)min((int64_t)sub, E - cs);
-    int* const row_of = s_row[wib];
+    const int* const row = s_rows[wib];
+    const uint16_t* const start = s_start[wib];
     bool began_before;
     const int m = stage_rows(rowptr, N, E, cs, n, lane, s_rows[wib], s_start[wib], began_before);
     __syncwarp();
-    for (int i = lane; i < n; i += 32) {
-        int lo = 0, hi = m;  // start[lo] <= i < start[hi]
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (s_start[wib][mid] <= i) lo = mid; else hi = mid;
-        }
-        row_of[i] = s_rows[wib][lo];
+    const int L = sub * lpr / 32, a = g * L, b = min(a + L, n);
+    if (a >= b) return;
+    int q0 = 0, hi = m;  // start[q0] <= a < start[hi]
+    while (hi - q0 > 1) {
+        const int mid = (q0 + hi) >> 1;
+        if (start[mid] <= a) q0 = mid; else hi = mid;
     }
-    __syncwarp();
-    const uint32_t pairs = (uint32_t)n * (uint32_t)nvec;
-    uint4* const o = dm + (size_t)cs * nvec;
-    for (uint32_t k0 = lane; k0 < pairs; k0 += 32 * U) {
-        uint4 raw[U], win[U][EPC / 4];
-        int at[U];
-        float deg[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint32_t k = k0 + u * 32, i = over_nvec(k, nvec, magic);
-            at[u] = cs + (int)i;
-            if (k >= pairs) continue;
-            const int r = row_of[i];
-            const size_t from = (size_t)r * nvec + (k - i * nvec);
-            raw[u] = __ldg(dOut + from);
-            if (op == GNN_MEAN) deg[u] = (float)(rowptr[r + 1] - rowptr[r]);
-            if (op == GNN_MAX || op == GNN_MIN) {
+    const bool route = op == GNN_MAX || op == GNN_MIN;
+    struct Row { uint4 v, win[EPC / 4]; float deg; };
+    for (int ci = lane % lpr; ci < nvec; ci += lpr) {
+        auto load = [&](int q, Row& R) {
+            const size_t from = (size_t)row[q] * nvec + ci;
+            R.v = __ldg(dOut + from);
+            if (op == GNN_MEAN) R.deg = (float)(rowptr[row[q] + 1] - rowptr[row[q]]);
+            if (route) {
 #pragma unroll
                 for (int j = 0; j < EPC / 4; ++j) {
-                    const int32_t* a = argmax + from * EPC + 4 * j;  // wide: 16-byte aligned
-                    if (wide) win[u][j] = __ldg(reinterpret_cast<const uint4*>(a));
-                    else win[u][j] = make_uint4(a[0], a[1], a[2], a[3]);
+                    const int32_t* w = argmax + from * EPC + 4 * j;  // wide: 16-byte aligned
+                    if (wide) R.win[j] = __ldg(reinterpret_cast<const uint4*>(w));
+                    else R.win[j] = make_uint4(w[0], w[1], w[2], w[3]);
                 }
             }
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const uint32_t k = k0 + u * 32;
-            if (k >= pairs) continue;
-            if (op != GNN_SUM) {
+        };
+        Row R, next;
+        load(q0, R);
+        uint4* const o = dm + (size_t)cs * nvec + ci;
+        for (int q = q0, p = a;; ++q) {
+            const int e = min((int)start[q + 1], b);
+            if (e < b) load(q + 1, next);
+            if (op == GNN_MEAN) {
                 float x[EPC];
-                Chunk<T>::unpack(raw[u], x);
-                if (op == GNN_MEAN) {
+                Chunk<T>::unpack(R.v, x);
 #pragma unroll
-                    for (int j = 0; j < EPC; ++j) x[j] = x[j] / deg[u];
-                } else {
-#pragma unroll
-                    for (int j = 0; j < EPC / 4; ++j) {
-                        x[4 * j] = (int)win[u][j].x == at[u] ? x[4 * j] : 0.f;
-                        x[4 * j + 1] = (int)win[u][j].y == at[u] ? x[4 * j + 1] : 0.f;
-                        x[4 * j + 2] = (int)win[u][j].z == at[u] ? x[4 * j + 2] : 0.f;
-                        x[4 * j + 3] = (int)win[u][j].w == at[u] ? x[4 * j + 3] : 0.f;
+                for (int j = 0; j < EPC; ++j) x[j] = x[j] / R.deg;
+                R.v = Chunk<T>::pack(x);
+            }
+            for (; p < e; ++p) {
+                uint4 v = R.v;
+                if (route) {  // zero where another position won
+                    const uint32_t at = (uint32_t)(cs + p);
+                    if (EPC == 4) {
+                        v.x = R.win[0].x == at ? v.x : 0u; v.y = R.win[0].y == at ? v.y : 0u; v.z = R.win[0].z == at ? v.z : 0u; v.w = R.win[0].w == at ? v.w : 0u;
+                    } else {
+                        const uint4 &lo = R.win[0], &up = R.win[EPC / 4 - 1];
+                        v.x &= (lo.x == at ? 0xffffu : 0u) | (lo.y == at ? 0xffff0000u : 0u); v.y &= (lo.z == at ? 0xffffu : 0u) | (lo.w == at ? 0xffff0000u : 0u);
+                        v.z &= (up.x == at ? 0xffffu : 0u) | (up.y == at ? 0xffff0000u : 0u); v.w &= (up.z == at ? 0xffffu : 0u) | (up.w == at ? 0xffff0000u : 0u);
                     }
                 }
-                raw[u] = Chunk<T>::pack(x);
+                o[(size_t)p * nvec] = v;
             }
-            o[k] = raw[u];
+            if (e >= b) break;
+            R = next;
         }
     }
 }
@@ -225,9 +225,10 @@ __global__ void __launch_bounds__(256) aggregate_backward_kernel(const int64_t* 
 static gnn_status launch_aggregate_backward(const char* who, const int64_t* rowptr, int32_t N, int64_t E, gnn_op op, const void* dOut,
                                             const int32_t* argmax, int nvec, gnn_dtype dtype, void* dm, cudaStream_t st) {
     const int sub = E >= 512 * 1024 ? AB_SUB : E >= 128 * 1024 ? 64 : E >= 64 * 1024 ? 32 : 8;
+    const int lpr = nvec <= 4 ? 4 : nvec <= 8 ? 8 : nvec <= 16 ? 16 : 32;
     const dim3 grid((unsigned)ceil_div(E, (int64_t)sub * 8));
     auto launch = [&](auto kernel) {
-        launch_overlapped(kernel, grid, dim3(256), 0, st, rowptr, N, E, (int)op, sub, aligned16(argmax), (const uint4*)dOut, argmax, nvec, pair_magic(nvec), (uint4*)dm);
+        launch_overlapped(kernel, grid, dim3(256), 0, st, rowptr, N, E, (int)op, sub, lpr, aligned16(argmax), (const uint4*)dOut, argmax, nvec, (uint4*)dm);
     };
     if (dtype == GNN_F32) launch(aggregate_backward_kernel<float>);
     else launch(aggregate_backward_kernel<__nv_bfloat16>);
