@@ -412,6 +412,9 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     const int* const Sc = S.col + 4 * g;
     const float* const Sw = S.w + (HAS_W ? 4 * g : 0);
     const int* const St = S.t + (ROUTE || HEAD ? 4 * g : 0);
+    // four entries at a time cost some kernels the registers they have left: plain bf16 sums (59 -> 61 us on 1.36 M 256-byte
+    // rows), and all bf16 rows of 512 bytes, which have one lane group and no bank conflict
+    constexpr bool ONE_BY_ONE = EPC == 8 && (PLAIN || LPR == 32);
     auto words = [&](int* to, const void* from) {  // H staged words, on their own size
         if (H == 4) *reinterpret_cast<int4*>(to) = *reinterpret_cast<const int4*>(from);
         else *reinterpret_cast<int2*>(to) = *reinterpret_cast<const int2*>(from);
@@ -491,7 +494,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     auto issue = [&](Buf& B, int i) -> unsigned {
         unsigned ends = 0;
         alignas(16) int ccs[H], ts[H];
-        if (PLAIN && EPC == 8) {  // one by one: four at a time cost these the registers they have left (59 -> 61 us on 1.36 M 256-byte rows)
+        if (ONE_BY_ONE) {
 #pragma unroll
             for (int u = 0; u < H; ++u) ccs[u] = Sc[i + u];
         } else {
@@ -570,11 +573,11 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     auto use_all = [&](const Buf& B, unsigned ends, int i) {
         alignas(16) float ws[H];
         alignas(16) int ts[H];
-        if (HAS_W) words(reinterpret_cast<int*>(ws), Sw + (HAS_W ? i : 0));
+        if (HAS_W && !ONE_BY_ONE) words(reinterpret_cast<int*>(ws), Sw + (HAS_W ? i : 0));
         if (ROUTE) words(ts, St + (ROUTE ? i : 0));
 #pragma unroll
         for (int u = 0; u < H; ++u) {
-            use(B, u, i + u, HAS_W ? ws[u] : 1.0f, ROUTE ? ts[u] : 0);
+            use(B, u, i + u, !HAS_W ? 1.0f : ONE_BY_ONE ? Sw[HAS_W ? i + u : 0] : ws[u], ROUTE ? ts[u] : 0);
             if (ends >> u & 1u) flush();
         }
     };
