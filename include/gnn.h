@@ -444,12 +444,14 @@ gnn_status gnn_graph_ptr_from_ids(const int32_t* graph_id, int32_t N, int32_t G,
 
 /* Global pooling (GlobalPool in the training example): out[g,:] = op over the nodes of graph g
  * of X[n,:]; an empty graph gives 0; MAX/MIN: argmax int32 [G,F] = winning node id (first node
- * among equals), -1 if none.  ws: gnn_propagate_fused_workspace(N, F, op) bytes. */
+ * among equals), -1 if none.  graph_ptr: non-decreasing, 0 <= graph_ptr[0], graph_ptr[G] <= N; nodes before graph_ptr[0]
+ * and from graph_ptr[G] on (rows that pad X) belong to no graph.  ws: gnn_propagate_fused_workspace(N, F, op) bytes. */
 gnn_status gnn_reduce_nodes(const int64_t* graph_ptr, int32_t G, int32_t N, gnn_op op, const void* X,
                             int F, gnn_dtype dtype, void* out_GF, int32_t* argmax, void* ws,
                             size_t ws_bytes, gnn_stream stream);
 
-/* dX[n,:] = dOut[g(n),:] (SUM), / n_g (MEAN), or routed to the argmax node only (MAX/MIN) */
+/* dX[n,:] = dOut[g(n),:] (SUM), / n_g (MEAN), or routed to the argmax node only (MAX/MIN);
+ * 0 for a node of no graph */
 gnn_status gnn_reduce_nodes_backward(const int64_t* graph_ptr, int32_t G, int32_t N, gnn_op op,
                                      const void* dOut_GF, const int32_t* argmax, int F,
                                      gnn_dtype dtype, void* dX_NF, gnn_stream stream);

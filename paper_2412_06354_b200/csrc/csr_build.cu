@@ -538,11 +538,11 @@ __global__ void __launch_bounds__(256) gcn_coef_kernel(const __grid_constant__ C
         const int mid = (q + hi) >> 1;
         if (s_start[warp][mid] <= i0) q = mid; else hi = mid;
     }
-    float di = A.deg[s_row[warp][q]];
+    float di = A.deg[max(s_row[warp][q], 0)];
 #pragma unroll
     for (int u = 0; u < PER; ++u)
         if (i0 + u < n) {
-            if (i0 + u >= s_start[warp][q + 1]) di = A.deg[s_row[warp][++q]];  // staged rows have positions: one step is enough
+            if (i0 + u >= s_start[warp][q + 1]) di = A.deg[max(s_row[warp][++q], 0)];  // staged rows have positions: one step is enough
             r[u] = gcn_coef(wp[u], di, dj[u]);
         }
     if (vec) {

@@ -70,7 +70,10 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
     for (int q = lane; q < m; q += 32) {
         const int e = S.start[q + 1];
         if (e <= n) S.col[sk(e - 1)] |= (int)0x80000000;
-        if (MEAN) S.inv[MEAN ? q : 0] = 1.0f / (float)(P.rowptr[S.row[q] + 1] - P.rowptr[S.row[q]]);
+        if (MEAN) {
+            const int r = max(S.row[q], 0);
+            S.inv[MEAN ? q : 0] = 1.0f / (float)(P.rowptr[r + 1] - P.rowptr[r]);
+        }
     }
     __syncwarp();
 
@@ -94,7 +97,7 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
         }
         q = lo;
     }
-    auto own = [&](int qq) { return __ldg(reinterpret_cast<const uint4*>(Dl + (size_t)(uint32_t)S.row[qq] * row_bytes)); };
+    auto own = [&](int qq) { return __ldg(reinterpret_cast<const uint4*>(Dl + (size_t)(uint32_t)max(S.row[qq], 0) * row_bytes)); };
     float d[EPC], sc = 1.0f;
     uint4 own_next = make_uint4(0u, 0u, 0u, 0u);
     if (a < b) {

@@ -176,6 +176,13 @@ __global__ void __launch_bounds__(256) aggregate_backward_kernel(const int64_t* 
     struct Row { uint4 v, win[EPC / 4]; float deg; };
     for (int ci = lane % lpr; ci < nvec; ci += lpr) {
         auto load = [&](int q, Row& R) {
+            if (row[q] < 0) {  // positions of no row: zero
+                R.v = make_uint4(0u, 0u, 0u, 0u);
+                R.deg = 1.f;
+#pragma unroll
+                for (int j = 0; j < EPC / 4; ++j) R.win[j] = make_uint4(~0u, ~0u, ~0u, ~0u);
+                return;
+            }
             const size_t from = (size_t)row[q] * nvec + ci;
             R.v = __ldg(dOut + from);
             if (op == GNN_MEAN) R.deg = (float)(rowptr[row[q] + 1] - rowptr[row[q]]);
@@ -424,6 +431,10 @@ gnn_status gnn_reduce_nodes_backward(const int64_t* graph_ptr, int32_t G, int32_
     if (rc != GNN_OK) return rc;
     if (N == 0) return GNN_OK;
     GNN_REQUIRE(aligned16(dOut_GF) && aligned16(dX_NF), GNN_ERR_INVALID_ARG, "%s: misaligned matrix", who);
+    if (G == 0) {
+        if (cudaMemsetAsync(dX_NF, 0, (size_t)N * F * elem_size(dtype), as_stream(stream)) != cudaSuccess) GNN_FAIL(GNN_ERR_CUDA, "%s: memset failed", who);
+        return GNN_OK;
+    }
     return launch_aggregate_backward(who, graph_ptr, G, N, op, dOut_GF, argmax, nvec, dtype, dX_NF, as_stream(stream));
 }
 

@@ -103,8 +103,8 @@ __device__ __forceinline__ int first_row_ending_after(const int64_t* __restrict_
     return lo;
 }
 
-// Position holding `pos`: the last row r with rowptr[r] <= pos (0 <= pos < E).  Warp-cooperative.  The first look is at 32
-// rows spaced 64 apart around the row that even degrees would give, then 32-way steps, then 64 rows at once.
+// Position holding `pos`: the last row r with rowptr[r] <= pos (0 <= pos < E), or row 0 if there is none.  Warp-cooperative.  The
+// first look is at 32 rows spaced 64 apart around the row that even degrees would give, then 32-way steps, then 64 rows at once.
 __device__ __forceinline__ int row_of_position(const int64_t* __restrict__ rowptr, int N, int64_t E, int64_t pos, int lane) {
     int lo = 0, hi = N;  // rowptr[lo] <= pos < rowptr[hi]
     if (N > 1024) {
@@ -118,9 +118,9 @@ __device__ __forceinline__ int row_of_position(const int64_t* __restrict__ rowpt
     while (hi - lo > 64) {
         const int step = (hi - lo + 31) / 32;
         const int idx = lo + lane * step;
-        const bool le = idx < hi && rowptr[idx] <= pos;  // true for a prefix of the lanes, lane 0 among them
+        const bool le = idx < hi && rowptr[idx] <= pos;  // true for a prefix of the lanes; for none if pos lies before the first row
         const int c = __popc(__ballot_sync(0xffffffffu, le));
-        lo = lo + (c - 1) * step;
+        lo = lo + max(c - 1, 0) * step;
         hi = min(lo + step, hi);
     }
     const int a = lo + 1 + lane, b = a + 32;
@@ -129,15 +129,19 @@ __device__ __forceinline__ int row_of_position(const int64_t* __restrict__ rowpt
 }
 
 // The rows with positions in [cs, cs + n), n > 0: their ids to row[], their first positions relative to cs to start[] (0 for a
-// row that began before), start[count] = the last one's end, or n + 1 if it goes on.  Returns the count.  Warp-cooperative.
+// row that began before), start[count] = the last one's end, or n + 1 if it goes on.  Positions before the first row or after the
+// last (row pointers of a caller that leave some uncovered, as nodes outside graph_ptr) are staged as a row of id -1, whose
+// sums the callers drop.  Returns the count, at most n.  Warp-cooperative.
 __device__ __forceinline__ int stage_rows(const int64_t* __restrict__ rowptr, int N, int64_t E, int cs, int n, int lane, int* row, uint16_t* start,
                                           bool& began_before) {
     const int r0 = row_of_position(rowptr, N, E, cs, lane);
     int m = 1;
-    int64_t last_end = rowptr[r0 + 1];
-    began_before = rowptr[r0] < cs;
-    if (lane == 0) { row[0] = r0; start[0] = 0; }
-    for (int rb = r0 + 1; rb < N;) {
+    const int64_t s0 = rowptr[r0], e0 = rowptr[r0 + 1];
+    const bool none = s0 > cs || e0 <= cs;  // the first position is in no row
+    int64_t last_end = none ? (int64_t)cs + n + 1 : e0;
+    began_before = !none && s0 < cs;
+    if (lane == 0) { row[0] = none ? -1 : r0; start[0] = 0; }
+    for (int rb = s0 > cs ? r0 : r0 + 1; rb < N;) {
         const int r = rb + lane;
         int64_t s = 0, e = 0;
         bool in = false;
@@ -158,6 +162,11 @@ __device__ __forceinline__ int stage_rows(const int64_t* __restrict__ rowptr, in
         if (!__all_sync(0xffffffffu, in)) break;
         if (lm == 0) rb = first_row_ending_after(rowptr, rb + 32, N, __shfl_sync(0xffffffffu, s, 0), lane);  // over a run of empty rows
         else rb += 32;
+    }
+    if (last_end < (int64_t)cs + n) {  // no row holds the rest
+        if (lane == 0) { row[m] = -1; start[m] = (uint16_t)(last_end - cs); }
+        ++m;
+        last_end = (int64_t)cs + n + 1;
     }
     if (lane == 0) start[m] = (uint16_t)min(last_end - cs, (int64_t)n + 1);
     return m;

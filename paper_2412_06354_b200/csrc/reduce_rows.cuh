@@ -457,7 +457,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     // MODE_V2: this row's own features, the next row's on their way, and the share of da (all rows of the group together)
     float xs[V2 ? EPC : 1], da[DA ? EPC : 1];
     uint4 own_next = make_uint4(0u, 0u, 0u, 0u);
-    auto own = [&](int qq) { return __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(P.v2_self) + (size_t)S.row[qq] * P.x_ld) + ci); };
+    auto own = [&](int qq) { return __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(P.v2_self) + (size_t)max(S.row[qq], 0) * P.x_ld) + ci); };
     if (V2) {
         if (a < b) {
             Chunk<T>::unpack(own(q), xs);
@@ -475,7 +475,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
                 S.head[lane * EPC + j] = acc[j];
                 if (ARG) S.head_a[ARG ? lane * EPC + j : 0] = arg[ARG ? j : 0];
             }
-        } else if (col_lane) {
+        } else if (col_lane && S.row[q] >= 0) {
             finish_row<T, MODE, EPI>(P, S.row[q], S.start[q + 1] - S.start[q], ci, acc, arg);
         }
         clear();
@@ -670,7 +670,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
                 if (before) {
                     head_state = HEAD_CLOSED;
                     leave(S.head, S.head_a, carry, carg);
-                } else if (lane < LPR && col_lane) {
+                } else if (lane < LPR && col_lane && S.row[hq] >= 0) {
                     finish_row<T, MODE, EPI>(P, S.row[hq], S.start[hq + 1] - S.start[hq], ci, carry, carg);
                 }
                 have = before = false;

@@ -263,6 +263,34 @@ def test_pooling_edge_cases(gnn):
     assert e.value.status == 3
 
 
+# Nodes before graph_ptr[0] and from graph_ptr[G] on (a padded X) belong to no graph: inside a warp's share, whole shares and whole
+# blocks of them, for every number of lane groups, positions first and (last two) a row per lane group.
+@pytest.mark.parametrize("gp,n,dtype,F", [
+    ([0, 10, 20], 64, "f32", 128), ([0, 10, 20], 64, "f32", 4), ([37, 45], 400, "bf16", 8), ([300, 300, 301, 333], 5000, "f32", 32),
+    ([5, 9, 64], 64, "f32", 64), ([0, 64, 128], 1000, "bf16", 64), ([9000, 150_000, 290_000], 300_000, "f32", 16),
+    ([0, 1, 270_001], 600_000, "bf16", 256), ([3, 3, 5, 9, 9, 12, 13, 14, 15, 16, 17, 20], 40, "f32", 12), ([40] * 8, 40, "f32", 4)])
+def test_pooling_leaves_nodes_of_no_graph_out(gnn, gp, n, dtype, F):
+    import torch
+    gp = np.array(gp, np.int64)
+    G, lo, hi = len(gp) - 1, int(gp[0]), int(gp[-1])
+    X, R = feats((n, F), dtype, 40), feats((G, F), dtype, 41)
+    inner = gp - lo
+    for op in ("sum", "mean", "max", "min"):
+        got = gnn.reduce_nodes(to_dev(gp), to_dev(X), op)
+        o, S, a = oracle.reduce_nodes(op, inner, X[lo:hi])
+        arg = None
+        if op in ("max", "min"):
+            got, arg = got
+            a = np.where(a >= 0, a + lo, a)
+            assert np.array_equal(bits(got), f64_to_dtype_bits(o, dtype)) and np.array_equal(arg.cpu().numpy(), a)
+        else:
+            assert_close(to_host64(got), o, S, dtype, op)
+        dX = gnn.reduce_nodes_backward(to_dev(gp), to_dev(R), n, op, argmax=arg)
+        assert torch.count_nonzero(dX[:lo]) == 0 and torch.count_nonzero(dX[hi:]) == 0
+        ref = oracle.reduce_nodes_backward(op, inner, R, None if arg is None else np.where(a >= 0, a - lo, a))
+        assert_close(to_host64(dX[lo:hi]), ref, np.abs(ref), dtype, f"backward {op}")
+
+
 # Four 256-thread tiles of (edge, 16-byte chunk) pairs per block; the backward pass takes 8 to 128 positions per warp: rows of
 # one chunk, of a number of chunks that divides nothing, and of more than 4096 chunks (64 KB), which divide instead of multiplying
 @pytest.mark.parametrize("e,dtype,F", [(1, "f32", 4), (65, "bf16", 8), (1025, "f32", 4), (700, "bf16", 56), (70_001, "f32", 12), (131_200, "bf16", 24), (525_000, "f32", 4), (67, "f32", 16_420)])
