@@ -163,9 +163,9 @@ gnn_status linear_tma_f32_forward(const void* X, int ldx, const void* W, int64_t
 bool linear_tma_dw_supported(int64_t N, int K, int M, gnn_dtype dtype);
 int linear_tma_dw_partials(int64_t N);
 gnn_status linear_tma_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, float* part, int* d_flag, int reset, cudaStream_t st);
-bool linear_tma_f32_dw_supported(int64_t N, int K, int M, gnn_dtype dtype);
+bool linear_tma_f32_dw_supported(int64_t N, int K, int M, int Mo, gnn_dtype dtype);
 int linear_tma_f32_dw_partials(int64_t N);
-gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, float* part, int* d_flag, int reset, cudaStream_t st);
+gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, int Mo, float* part, int* d_flag, int reset, cudaStream_t st);
 bool linear_tc_dw_supported(int64_t N, int K, int M, gnn_dtype dtype);
 int linear_tc_dw_partials(int64_t N);
 gnn_status linear_tc_dw(const void* X, const void* dY, int64_t N, int K, int M, gnn_dtype dtype, float* part, int* d_flag,
@@ -283,7 +283,7 @@ gnn_status gnn_linear_backward(const void* X, const void* W, const void* dY, int
     const bool dx_tma = dX && N > 0 && on16 && aligned16(W) && (dtype == GNN_F32 ? linear_tma_f32_supported(N, M, K, dtype) : linear_tma_supported(N, M, K, 1, dtype));
     // dW[k,m] = sum_n X[n,k] * dY[n,m]: one fp32 partial per CTA, then summed in CTA order.  More output columns than one
     // launch takes (256, or fewer where K fills tensor memory): one launch and one ordered sum per block of columns of dY.
-    auto dw_supported = [&](int mc) { return dtype == GNN_F32 ? linear_tma_f32_dw_supported(N, K, mc, dtype) : linear_tma_dw_supported(N, K, mc, dtype); };
+    auto dw_supported = [&](int mc) { return dtype == GNN_F32 ? linear_tma_f32_dw_supported(N, K, mc, M, dtype) : linear_tma_dw_supported(N, K, mc, dtype); };
     int block = 0;
     if (dW && N > 0 && on16 && aligned16(X)) {
         if (dw_supported(M)) block = M;
@@ -332,7 +332,7 @@ gnn_status gnn_linear_backward(const void* X, const void* W, const void* dY, int
             for (int c0 = 0; c0 < M; c0 += block) {
                 const int mc = M - c0 < block ? M - c0 : block;
                 const void* dYb = (const char*)dYp + (size_t)c0 * s;
-                gnn_status rc = dtype == GNN_F32 ? linear_tma_f32_dw(Xp, padded(K, s), dYb, ldd, N, K, mc, part, status, reset, st)
+                gnn_status rc = dtype == GNN_F32 ? linear_tma_f32_dw(Xp, padded(K, s), dYb, ldd, N, K, mc, M, part, status, reset, st)
                                                  : linear_tma_dw(Xp, padded(K, s), dYb, ldd, N, K, mc, part, status, reset, st);
                 if (rc != GNN_OK) return rc;
                 reset = 0;

@@ -432,7 +432,9 @@ struct TmaF32Params {
     int Kc, Mo;         // multiples of 16: the contraction, the output columns of a block
     int b_transposed;
     int stages;         // a multiple of the groups
-    int acc_stride, tmem_cols;
+    int acc_bufs;       // 2: the next tile's products run beside this one's epilogue
+    int acc_stride, tmem_cols;  // tensor memory columns of an accumulator buffer, and of all
+    int split, half, corr;      // exact kernels: first k-step of the second main sum; columns of that sum and of the corrections in a buffer
     int* status;
     int reset;          // set the status word to 0
     const float* bias;  // [cols] added to every output row, or nullptr
@@ -443,7 +445,7 @@ struct TmaF32Params {
     int64_t ldy;
 };
 
-template <int G>
+template <int G, bool EXACT>
 __global__ void __launch_bounds__(TF_THREADS, 1)
 linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapY, const TmaF32Params P) {
     extern __shared__ unsigned char smem_raw[];
@@ -535,7 +537,7 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = tmem_base_slot;
+    const uint32_t tmem_base = tmem_base_slot, nbuf = EXACT ? (uint32_t)P.acc_bufs : 2u;
     bool failed = false;
 
     if (warp == 0) {
@@ -557,15 +559,15 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
             const uint32_t idesc = make_idesc(Mo, P.b_transposed ? 0 : 1), b_level16 = b_level / 16;
             uint32_t it = 0, lt = 0;
             for (int64_t t = blockIdx.x; t < ntiles && !failed; t += gridDim.x, ++lt) {
-                const uint32_t a = lt & 1u;
-                if (!mbar_wait_bounded(acc_empty((int)a), ((lt >> 1) & 1u) ^ 1u)) { failed = true; break; }
+                const uint32_t a = lt % nbuf;
+                if (!mbar_wait_bounded(acc_empty((int)a), ((lt / nbuf) & 1u) ^ 1u)) { failed = true; break; }
                 tc_fence_after();
                 const uint32_t dacc = tmem_base + a * (uint32_t)P.acc_stride;
                 for (int j = 0; j < nslices; ++j, ++it) {
                     const uint32_t o = it % G;
                     if (!mbar_wait_bounded(o_full((int)o), (it / G) & 1u)) { failed = true; break; }
                     tc_fence_after();
-                    const uint32_t at = tmem_base + 2u * (uint32_t)P.acc_stride + o * (uint32_t)TF_OP_COLS;
+                    const uint32_t at = tmem_base + nbuf * (uint32_t)P.acc_stride + o * (uint32_t)TF_OP_COLS;
                     const uint64_t bdesc = make_smem_desc(w0 + (uint32_t)j * (TF_KB / 16) * 256u, 128, b_sbo);
                     const bool both = Kc - j * TF_KB >= TF_KB;  // else a last slice of 16
 #pragma unroll
@@ -574,8 +576,16 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
 #pragma unroll
                         for (int q = 0; q < 6; ++q) {  // offsets add to the descriptors' address field, in units of 16 bytes
                             const uint64_t bd = bdesc + (uint64_t)(pair_b(q) * b_level16 + (uint32_t)kk * 16u);
-                            const uint32_t more = (j > 0 || kk > 0 || q > 0) ? 1u : 0u;
-                            mma_bf16_ts(dacc, at + pair_a(q) * (TF_KB / 2) + (uint32_t)kk * 8u, bd, idesc, more);
+                            uint32_t to = dacc, more = (j > 0 || kk > 0 || q > 0) ? 1u : 0u;
+                            if (EXACT) {
+                                const int ks = j * (TF_KB / 16) + kk;
+                                if (q < 5) to += (uint32_t)P.corr;
+                                else {
+                                    more = ks != 0 && ks != P.split;
+                                    if (ks >= P.split) to += (uint32_t)P.half;
+                                }
+                            }
+                            mma_bf16_ts(to, at + pair_a(q) * (TF_KB / 2) + (uint32_t)kk * 8u, bd, idesc, more);
                         }
                     }
                     mma_commit(o_empty((int)o));
@@ -597,7 +607,7 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
                 const uint32_t src = ring0 + (uint32_t)s * TF_SLICE_BYTES;
                 // a warp reaches the 32 lanes of tensor memory of its number modulo 4
                 const int r = (warp & 3) * 32 + lane;
-                const uint32_t to = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + 2u * (uint32_t)P.acc_stride + (uint32_t)(grp * TF_OP_COLS);
+                const uint32_t to = tmem_base + ((uint32_t)((warp & 3) * 32) << 16) + nbuf * (uint32_t)P.acc_stride + (uint32_t)(grp * TF_OP_COLS);
 #pragma unroll
                 for (int rep = 0; rep < 16 / GW; ++rep) {
                     const int kc = (wl >> 2) + rep * (GW / 4);
@@ -622,8 +632,8 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
         stage_bias(s_bias, P.bias ? P.bias + c0 : nullptr, mo, 32 * (2 + TF_CONV_WARPS));
         uint32_t lt = 0;
         for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x, ++lt) {
-            const uint32_t a = lt & 1u;
-            if (!mbar_wait_bounded(acc_full((int)a), (lt >> 1) & 1u)) { failed = true; break; }
+            const uint32_t a = lt % nbuf;
+            if (!mbar_wait_bounded(acc_full((int)a), (lt / nbuf) & 1u)) { failed = true; break; }
             tc_fence_after();
             const int64_t row0 = t * TC_ROWS + quarter * 32;  // first of this warp's 32 rows
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + a * (uint32_t)P.acc_stride;
@@ -635,6 +645,15 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
                     uint32_t r[16];
                     tmem_ld16(taddr + (uint32_t)(cb * 32 + g16 * 16), r);
                     tmem_ld_wait();
+                    if (EXACT) {  // main + second main + corrections
+                        for (int w = P.half > 0 ? 0 : 1; w < 2; ++w) {
+                            uint32_t more[16];
+                            tmem_ld16(taddr + (uint32_t)((w == 0 ? P.half : P.corr) + cb * 32 + g16 * 16), more);
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int q = 0; q < 16; ++q) r[q] = __float_as_uint(__uint_as_float(r[q]) + __uint_as_float(more[q]));
+                        }
+                    }
                     if (P.bias || P.relu) {
                         float f[16];
 #pragma unroll
@@ -909,8 +928,15 @@ static bool make_map_f32_blocks(CUtensorMap* m, const void* ptr, int64_t rows, i
 // Every wait is bounded.
 // Two groups on slots of 32 rows, on slots of 16 four where four buffers and slots fit.  170k x 128 x 128: 50 us with 8 warps
 // on one slot after the other, 47 us with 16, 58 us in four groups on slots of 16 rows, 42 us so; reading X and dY takes 27 us.
-constexpr int FD_CONV_WARPS = 16;
+// Exact form (K or M no multiple of 32): the accumulator truncates at every MMA, 1.8e-8 of the result each and one way, so that
+// a CTA's hundreds of rows in one sum cost 7.8e-6 norm-wise at 170k rows and 2.3e-5 at 500k, where the FFMA kernel that these
+// sizes took before has 1.1e-6.  There the five small products go to an accumulator of corrections, and after every FD_FLUSH
+// rows (32 main MMAs) four warps of their own add the main accumulator to the partial in fp32 while the MMAs go on in a second
+// one (where tensor memory has room: up to 160 accumulator columns): 4.7e-7 at either size.  170k x 100 x 47: 52 -> 60 us
+// (FFMA 1149 us); 500k x 500 x 250, where half as many columns fit a launch: 0.90 -> 1.79 ms (FFMA 6.4 ms).
+constexpr int FD_CONV_WARPS = 16, FD_FLUSH_WARPS = 4;
 constexpr int FD_THREADS = 32 * (2 + FD_CONV_WARPS);
+constexpr int FD_FLUSH = 512;
 constexpr int FD_MAX_STAGES = 8;
 constexpr int FD_MAX_GROUPS = 4;
 
@@ -921,16 +947,18 @@ struct TmaF32DwParams {
     int x_whole, d_whole;  // the slot's boxes of X or dY arrive in one copy
     int groups;  // 4 or 2
     int stages;  // a multiple of groups
+    int mains;   // exact: main accumulators, 2 or 1; the corrections' columns follow them
     int tmem_cols;
     int* status;
     int reset;  // first launch of a call: set the status word to 0
 };
 
-template <int FD_ROWS>
-__global__ void __launch_bounds__(FD_THREADS, 1)
+template <int FD_ROWS, bool EXACT>
+__global__ void __launch_bounds__(FD_THREADS + (EXACT ? 32 * FD_FLUSH_WARPS : 0), 1)
 linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapD, const TmaF32DwParams P) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t bars[2 * FD_MAX_STAGES + 2 * FD_MAX_GROUPS + 1];  // f_full[S], f_empty[S], o_full[G], o_empty[G], acc_full
+    // f_full[S], f_empty[S], o_full[G], o_empty[G], acc_full[2], acc_empty[2]
+    __shared__ __align__(8) uint64_t bars[2 * FD_MAX_STAGES + 2 * FD_MAX_GROUPS + 4];
     __shared__ uint32_t tmem_base_slot;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int K = P.K, M = P.M, S = P.stages, halves = (K + 127) / 128;
@@ -949,12 +977,15 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
     auto f_empty = [&](int s) { return bar0 + 8u * (uint32_t)(FD_MAX_STAGES + s); };
     auto o_full = [&](int o) { return bar0 + 8u * (uint32_t)(2 * FD_MAX_STAGES + o); };
     auto o_empty = [&](int o) { return bar0 + 8u * (uint32_t)(2 * FD_MAX_STAGES + FD_MAX_GROUPS + o); };
-    const uint32_t acc_full = bar0 + 8u * (uint32_t)(2 * FD_MAX_STAGES + 2 * FD_MAX_GROUPS);
+    auto acc_full = [&](uint32_t b) { return bar0 + 8u * ((uint32_t)(2 * FD_MAX_STAGES + 2 * FD_MAX_GROUPS) + b); };
+    auto acc_empty = [&](uint32_t b) { return bar0 + 8u * ((uint32_t)(2 * FD_MAX_STAGES + 2 * FD_MAX_GROUPS + 2) + b); };
+    constexpr uint32_t FLUSH = FD_FLUSH / FD_ROWS;  // slots per main sum
+    const uint32_t mains = EXACT ? (uint32_t)P.mains : 1u, acc_cols = (uint32_t)(halves * M);
 
     if (tid == 0) {
         for (int s = 0; s < S; ++s) { mbar_init(f_full(s), 1); mbar_init(f_empty(s), FD_CONV_WARPS / G); }
         for (int o = 0; o < (int)G; ++o) { mbar_init(o_full(o), FD_CONV_WARPS / G); mbar_init(o_empty(o), 1); }
-        mbar_init(acc_full, 1);
+        for (uint32_t b = 0; b < 2; ++b) { mbar_init(acc_full(b), 1); mbar_init(acc_empty(b), FD_FLUSH_WARPS); }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapX)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapD)) : "memory");
@@ -962,7 +993,7 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
     if (warp == 1) tmem_alloc(smem_u32(&tmem_base_slot), (uint32_t)P.tmem_cols);
     if (K % 128 != 0) {  // the converters never write the feature rows past K: zero the buffers' A levels once
         for (int o = 0; o < (int)G; ++o)
-            for (uint32_t off = (uint32_t)tid * 16u; off < 3u * a_level; off += FD_THREADS * 16u)
+            for (uint32_t off = (uint32_t)tid * 16u; off < 3u * a_level; off += blockDim.x * 16u)
                 st_shared16(op0 + (uint32_t)o * op_bytes + off, make_uint4(0u, 0u, 0u, 0u));
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     }
@@ -1002,9 +1033,13 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
             const uint32_t idesc = make_idesc(M, 1) | (1u << 15);  // A and B both MN-major
-            uint32_t it = 0;
+            uint32_t it = 0, acc = tmem_base, fresh = 1, v = 0;  // fresh: the main sum begins with this slot; v: how many began before
             for (int64_t t = blockIdx.x; t < nslots; t += gridDim.x, ++it) {
                 const uint32_t o = it % G;
+                if (EXACT && fresh) {
+                    if (!mbar_wait_bounded(acc_empty(v % mains), ((v / mains) & 1u) ^ 1u)) { failed = true; break; }
+                    acc = tmem_base + v % mains * acc_cols;
+                }
                 if (!mbar_wait_bounded(o_full((int)o), (it / G) & 1u)) { failed = true; break; }
                 tc_fence_after();
                 const uint32_t abuf = op0 + o * op_bytes, bbuf = abuf + 3u * a_level;
@@ -1013,13 +1048,61 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
 #pragma unroll
                     for (int kk = 0; kk < FD_ROWS / 16; ++kk)
 #pragma unroll
-                        for (int q = 0; q < 6; ++q)  // offsets add to the descriptors' address field, in units of 16 bytes
-                            mma_bf16_ss(tmem_base + (uint32_t)h * (uint32_t)M, adesc + (uint64_t)(pair_a(q) * (a_level / 16) + (uint32_t)h * FD_SBO + (uint32_t)kk * 16u),
-                                        bdesc + (uint64_t)(pair_b(q) * (b_level / 16) + (uint32_t)kk * 16u), idesc, (it > 0 || kk > 0 || q > 0) ? 1u : 0u);
+                        for (int q = 0; q < 6; ++q) {  // offsets add to the descriptors' address field, in units of 16 bytes
+                            uint32_t to = acc, more = (it > 0 || kk > 0 || q > 0) ? 1u : 0u;
+                            if (EXACT) {
+                                if (q < 5) to = tmem_base + mains * acc_cols;
+                                else more = (!fresh || kk > 0) ? 1u : 0u;
+                            }
+                            mma_bf16_ss(to + (uint32_t)h * (uint32_t)M, adesc + (uint64_t)(pair_a(q) * (a_level / 16) + (uint32_t)h * FD_SBO + (uint32_t)kk * 16u),
+                                        bdesc + (uint64_t)(pair_b(q) * (b_level / 16) + (uint32_t)kk * 16u), idesc, more);
+                        }
                 }
                 mma_commit(o_empty((int)o));
+                fresh = 0;
+                if (EXACT && (it % FLUSH == FLUSH - 1 || t + gridDim.x >= nslots)) {  // (commits cover everything issued so far)
+                    mma_commit(acc_full(v % mains));
+                    fresh = 1;
+                    ++v;
+                }
             }
-            if (!failed) mma_commit(acc_full);
+            if (!EXACT && !failed) mma_commit(acc_full(0));
+        }
+    } else if (EXACT && warp >= 2 + FD_CONV_WARPS) {
+        // ------------------------------------------------------------ flush: main sums, and at last the corrections, to this CTA's partial
+        const int quarter = warp & 3;  // a warp reaches the 32 lanes of tensor memory of its number modulo 4
+        const uint32_t slots = (uint32_t)((nslots - blockIdx.x + gridDim.x - 1) / gridDim.x), sums = (slots + FLUSH - 1) / FLUSH;
+        for (uint32_t v = 0; v < sums; ++v) {
+            if (!mbar_wait_bounded(acc_full(v % mains), (v / mains) & 1u)) { failed = true; break; }
+            tc_fence_after();
+            for (int h = 0; h < halves; ++h) {
+                if (h * 128 + quarter * 32 >= K) break;  // feature rows past K
+                float* prow = P.part + ((size_t)blockIdx.x * K + h * 128 + quarter * 32 + lane) * M;
+                const uint32_t lanes = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)h * (uint32_t)M;
+                for (int c0 = 0; c0 < M; c0 += 16) {
+                    uint32_t r[16], c[16];
+                    tmem_ld16(lanes + v % mains * acc_cols + (uint32_t)c0, r);
+                    if (v + 1 == sums) tmem_ld16(lanes + mains * acc_cols + (uint32_t)c0, c);
+                    tmem_ld_wait();
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        float4* const to = reinterpret_cast<float4*>(prow + c0) + q;
+                        float4 s = make_float4(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1]), __uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3]));
+                        if (v > 0) {
+                            const float4 b = *to;
+                            s.x += b.x; s.y += b.y; s.z += b.z; s.w += b.w;
+                        }
+                        if (v + 1 == sums) {
+                            s.x += __uint_as_float(c[4 * q]); s.y += __uint_as_float(c[4 * q + 1]);
+                            s.z += __uint_as_float(c[4 * q + 2]); s.w += __uint_as_float(c[4 * q + 3]);
+                        }
+                        *to = s;
+                    }
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(acc_empty(v % mains));
         }
     } else {
         // ------------------------------------------------------------ converters
@@ -1060,10 +1143,10 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
             if (lane == 0) { mbar_arrive(f_empty(s)); mbar_arrive(o_full((int)o)); }
         }
         // accumulator -> this CTA's partial.  Lane = feature row; warps 2..5 take the lower half of the columns, 6..9 the upper
-        if (!failed && !mbar_wait_bounded(acc_full, 0u)) failed = true;
+        if (!EXACT && !failed && !mbar_wait_bounded(acc_full(0), 0u)) failed = true;
         tc_fence_after();
         const int quarter = warp & 3, half = (warp - 2) >> 2;
-        for (int h = 0; h < halves && !failed && half < 2; ++h) {
+        for (int h = 0; h < halves && !failed && !EXACT && half < 2; ++h) {
             const int krow = h * 128 + quarter * 32 + lane;
             if (h * 128 + quarter * 32 >= K) break;  // tcgen05.ld is warp-wide: a warp whose 32 feature rows all lie past K skips it as one
             float* prow = P.part + ((size_t)blockIdx.x * K + krow) * M;
@@ -1086,11 +1169,15 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
     if (warp == 1) tmem_dealloc(tmem_base, (uint32_t)P.tmem_cols);
 }
 
+// The exact form where the whole product (K features, Mo columns, of which a launch may take a block of M) is no multiple of 32
+static bool fd_exact(int K, int Mo) { return K % 32 != 0 || Mo % 32 != 0; }
+
 // K and M: any (inside, rounded up to 32 with zeros from the copy engine; that is the shape of the partials)
-bool linear_tma_f32_dw_supported(int64_t N, int K, int M, gnn_dtype dtype) {
+bool linear_tma_f32_dw_supported(int64_t N, int K, int M, int Mo, gnn_dtype dtype) {
     if (dtype != GNN_F32 || N <= 0 || N >= ((int64_t)1 << 31) - 32) return false;
     if (K < 1 || K > 512 || M < 1 || M > 256) return false;
-    if (up32(M) * ((K + 127) / 128) > 512) return false;  // one accumulator [128, M] per block of 128 features: 512 columns of tensor memory
+    // accumulators [128, M] per block of 128 features, the exact form's main and corrections: 512 columns of tensor memory
+    if (up32(M) * ((K + 127) / 128) * (fd_exact(K, Mo) ? 2 : 1) > 512) return false;
     return encoder() != nullptr;
 }
 
@@ -1101,7 +1188,8 @@ int linear_tma_f32_dw_partials(int64_t N) {
 }
 
 // writes linear_tma_f32_dw_partials(N) fp32 partials [up32(K), up32(M)] to part; X and dY: rows ldx and ldd elements apart
-gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int Kr, int Mr, float* part, int* d_flag, int reset, cudaStream_t st) {
+// (a block of Mr of the Mo columns of dY)
+gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int Kr, int Mr, int Mo, float* part, int* d_flag, int reset, cudaStream_t st) {
     const char* who = "gnn_linear_backward (pipelined fp32 tensor-core dW)";
     GNN_REQUIRE(aligned16(X) && aligned16(dY) && aligned16(part), GNN_ERR_INVALID_ARG, "%s: matrices must be 16-byte aligned", who);
     const int K = up32(Kr), M = up32(Mr);
@@ -1118,34 +1206,54 @@ gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, in
     int stages = (int)((TM_SMEM_MAX - 1024 - ops) / slot);
     if (stages > FD_MAX_STAGES) stages = FD_MAX_STAGES;
     P.stages = stages / P.groups * P.groups;
+    const bool exact = fd_exact(Kr, Mo);
+    const int acc_cols = M * (ka / 128);
+    P.mains = exact && 3 * acc_cols <= 512 ? 2 : 1;
     int cols = 32;
-    while (cols < M * (ka / 128)) cols <<= 1;
+    while (cols < (exact ? P.mains + 1 : 1) * acc_cols) cols <<= 1;
     P.tmem_cols = cols;
-    gnn_status rc = allow_big_smem(who, (const void*)linear_tma_f32_dw_kernel<32>, 12, TM_SMEM_MAX);
-    if (rc == GNN_OK) rc = allow_big_smem(who, (const void*)linear_tma_f32_dw_kernel<16>, 15, TM_SMEM_MAX);
-    if (rc != GNN_OK) return rc;
-    launch_overlapped(R == 32 ? linear_tma_f32_dw_kernel<32> : linear_tma_f32_dw_kernel<16>, dim3((unsigned)linear_tma_f32_dw_partials(N)), dim3(FD_THREADS), 1024 + ops + (size_t)P.stages * slot, st, mapX, mapD, P);
-    GNN_CHECK_LAUNCH(who);
-    return GNN_OK;
+    auto launch = [&](auto kernel, int which, int threads) {
+        gnn_status rc = allow_big_smem(who, (const void*)kernel, which, TM_SMEM_MAX);
+        if (rc != GNN_OK) return rc;
+        launch_overlapped(kernel, dim3((unsigned)linear_tma_f32_dw_partials(N)), dim3((unsigned)threads), 1024 + ops + (size_t)P.stages * slot, st, mapX, mapD, P);
+        GNN_CHECK_LAUNCH(who);
+        return GNN_OK;
+    };
+    constexpr int more = FD_THREADS + 32 * FD_FLUSH_WARPS;
+    if (exact) return R == 32 ? launch(linear_tma_f32_dw_kernel<32, true>, 18, more) : launch(linear_tma_f32_dw_kernel<16, true>, 19, more);
+    return R == 32 ? launch(linear_tma_f32_dw_kernel<32, false>, 12, FD_THREADS) : launch(linear_tma_f32_dw_kernel<16, false>, 15, FD_THREADS);
 }
 
 static size_t tf_fixed_bytes(int Kc, int Mo) {
     return 1024 + (((size_t)3 * Mo * Kc * 2 + 1023) & ~(size_t)1023) + (size_t)TF_EPI_WARPS * 4096;
 }
 
-// widest block of output columns (a multiple of 16): two accumulators and two operand buffers fit the 512 columns of tensor
-// memory, the three weight levels shared memory beside two slices
-static int tf_column_block(int Kc, int Mo) {
+// Sizes that are no multiples of 16 take the exact form: their callers were given FFMA precision before they came to the
+// tensor cores, whose accumulator truncates at every MMA (1.8e-8 of the result each, norm-wise, one way).  There the five
+// small products of a k-step go to an accumulator of their own (2^-8 of the size, so are its truncations), and above ten
+// k-steps the main products to two, added in fp32.  Distance to 64 bits, norm-wise, one sum -> separate sums (FFMA): contraction
+// of 100 7.3e-7 -> 9.2e-8 (1.8e-7), of 512 3.4e-6 -> 2.1e-7 (4.1e-7), of 47 2.9e-7 -> 5.4e-8 (1.2e-7).  170k x 100 x 47 takes
+// 32 us forward either way, 43 instead of 33 us for dX, which has one accumulator buffer only (FFMA 127 and 112 us).
+static bool tf_exact(int Kc, int Mo) { return Kc % 16 != 0 || Mo % 16 != 0; }
+static int tf_sums(int Kc, bool exact) { return !exact ? 1 : up16(Kc) / 16 > 10 ? 3 : 2; }
+
+// do `bufs` buffers of `sums` accumulators and `groups` operand buffers fit the 512 columns of tensor memory?
+static bool tf_tmem_fits(int width, int sums, int bufs, int groups) { return bufs * sums * up32(width) + groups * TF_OP_COLS <= 512; }
+
+// widest block of output columns (a multiple of 16): two accumulator buffers (exact: at least one) and two operand buffers fit
+// tensor memory, the three weight levels shared memory beside two slices
+static int tf_column_block(int Kc, int Mo, bool exact) {
     int mc = Mo < 192 ? Mo : 192;
-    while (mc >= 16 && tf_fixed_bytes(Kc, mc) + 2 * TF_SLICE_BYTES > TM_SMEM_MAX) mc -= 16;
+    while (mc >= 16 && (tf_fixed_bytes(Kc, mc) + 2 * TF_SLICE_BYTES > TM_SMEM_MAX || !tf_tmem_fits(mc, tf_sums(Kc, exact), exact ? 1 : 2, 2))) mc -= 16;
     return mc >= 16 ? mc : 0;
 }
 
-// Kc and Mo: any up to 512 and 1024 (inside, rounded up to 16 with zeros)
+// Kc and Mo: any up to 512 and 1024 (inside, rounded up to 16 with zeros); a contraction of one is a single rounded product,
+// which FFMA has exactly
 bool linear_tma_f32_supported(int64_t N, int Kc, int Mo, gnn_dtype dtype) {
     if (dtype != GNN_F32 || N <= 0 || N >= ((int64_t)1 << 31) - TC_ROWS) return false;
-    if (Kc < 1 || Kc > 512 || Mo < 1 || Mo > 1024) return false;
-    if (tf_column_block(up16(Kc), up16(Mo)) == 0) return false;
+    if (Kc < 2 || Kc > 512 || Mo < 1 || Mo > 1024) return false;
+    if (tf_column_block(up16(Kc), up16(Mo), tf_exact(Kc, Mo)) == 0) return false;
     return encoder() != nullptr;
 }
 
@@ -1159,15 +1267,13 @@ gnn_status linear_tma_f32_forward(const void* X, int ldx, const void* W, int64_t
     const char* who = "gnn_linear (pipelined fp32 tensor-core path)";
     const bool direct = Mo % 4 != 0;
     GNN_REQUIRE(aligned16(X) && aligned16(W) && (direct || aligned16(Y)), GNN_ERR_INVALID_ARG, "%s: matrices must be 16-byte aligned", who);
-    const int K16 = up16(Kc), widest = tf_column_block(K16, up16(Mo));
+    const bool exact = tf_exact(Kc, Mo);
+    const int K16 = up16(Kc), sums = tf_sums(K16, exact), widest = tf_column_block(K16, up16(Mo), exact);
     GNN_REQUIRE(widest > 0, GNN_ERR_UNSUPPORTED, "%s: weights do not fit shared memory", who);
     CUtensorMap mapX, mapY;
     if (!make_map_f32_ld(&mapX, X, N, Kc, ldx, TC_ROWS) || (!direct && !make_map_f32_ld(&mapY, Y, N, Mo, Mo, 32)))
         GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
     if (direct) mapY = mapX;  // not used
-    gnn_status rc = allow_big_smem(who, (const void*)linear_tma_f32_kernel<4>, 6, TM_SMEM_MAX);
-    if (rc == GNN_OK) rc = allow_big_smem(who, (const void*)linear_tma_f32_kernel<2>, 13, TM_SMEM_MAX);
-    if (rc != GNN_OK) return rc;
     const int64_t ntiles = (N + TC_ROWS - 1) / TC_ROWS;
     int blocks = (int)ceil_div(Mo, widest), width = up16((int)ceil_div(Mo, blocks));
     if (ntiles * 2 * blocks <= 148 && width > 32) {
@@ -1181,19 +1287,37 @@ gnn_status linear_tma_f32_forward(const void* X, int ldx, const void* W, int64_t
     P.bias = bias; P.relu = relu;
     P.direct = direct; P.Y = (float*)Y; P.ldy = Mo;
     const size_t fixed = tf_fixed_bytes(K16, width);
-    P.acc_stride = up32(width);
     int stages = (int)((TM_SMEM_MAX - fixed) / TF_SLICE_BYTES);  // at least two
     if (stages > TF_MAX_STAGES) stages = TF_MAX_STAGES;
-    const int groups = stages >= 4 && 2 * P.acc_stride + 4 * TF_OP_COLS <= 512 ? 4 : 2;
+    // four groups before a second accumulator buffer: only the exact form may be short of room for both
+    const int most = stages >= 4 ? 4 : 2;
+    P.acc_bufs = 2;
+    int groups = most;
+    if (!tf_tmem_fits(width, sums, 2, groups)) {
+        if (tf_tmem_fits(width, sums, 1, groups) && exact) P.acc_bufs = 1;
+        else {
+            groups = 2;
+            if (!tf_tmem_fits(width, sums, 2, 2)) P.acc_bufs = 1;
+        }
+    }
+    P.acc_stride = sums * up32(width);
+    P.half = sums == 3 ? up32(width) : 0; P.corr = (sums - 1) * up32(width);
+    P.split = sums == 3 ? K16 / 32 : K16 / 16;
     P.stages = stages / groups * groups;
     int cols = 32;
-    while (cols < 2 * P.acc_stride + groups * TF_OP_COLS) cols <<= 1;
+    while (cols < P.acc_bufs * P.acc_stride + groups * TF_OP_COLS) cols <<= 1;
     P.tmem_cols = cols;
-    const int64_t per_block = blocks < 148 ? 148 / blocks : 1;
-    launch_overlapped(groups == 4 ? linear_tma_f32_kernel<4> : linear_tma_f32_kernel<2>, dim3((unsigned)(ntiles < per_block ? ntiles : per_block), (unsigned)blocks),
-                      dim3(TF_THREADS), fixed + (size_t)P.stages * TF_SLICE_BYTES, st, mapX, mapY, P);
-    GNN_CHECK_LAUNCH(who);
-    return GNN_OK;
+    auto launch = [&](auto kernel, int which) {
+        gnn_status rc = allow_big_smem(who, (const void*)kernel, which, TM_SMEM_MAX);
+        if (rc != GNN_OK) return rc;
+        const int64_t per_block = blocks < 148 ? 148 / blocks : 1;
+        launch_overlapped(kernel, dim3((unsigned)(ntiles < per_block ? ntiles : per_block), (unsigned)blocks), dim3(TF_THREADS),
+                          fixed + (size_t)P.stages * TF_SLICE_BYTES, st, mapX, mapY, P);
+        GNN_CHECK_LAUNCH(who);
+        return GNN_OK;
+    };
+    if (exact) return groups == 4 ? launch(linear_tma_f32_kernel<4, true>, 16) : launch(linear_tma_f32_kernel<2, true>, 17);
+    return groups == 4 ? launch(linear_tma_f32_kernel<4, false>, 6) : launch(linear_tma_f32_kernel<2, false>, 13);
 }
 
 }  // namespace gnn

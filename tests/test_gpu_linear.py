@@ -108,6 +108,34 @@ def test_linear_ragged_sizes(gnn, dtype, n, K, M):
         oracle.set_threads(1)
 
 
+# fp32 sums of sizes that divide nothing: no further from 64 bits than plain fp32 FMAs.  The tensor core truncates its accumulator at
+# every MMA of 16 terms, half a unit in the last place (2^-23 of the running sum) on average and one way; at most 10 main MMAs of
+# a forward sum follow one another (16 in each of two sums above that), 32 in dW, and the sums are then added with rounding:
+# norm-wise n * 2^-24 + 2^-23 for n in a row.  One sum for all products of all levels was 7.3e-7 / 3.4e-6 for contractions of 100
+# / 511 and 7.8e-6 / 2.3e-5 for dW over 170k / 500k rows.
+@pytest.mark.parametrize("n,K,M", [(170_000, 100, 47), (500_000, 33, 9), (20_000, 511, 255), (30_000, 161, 40), (9_000, 47, 100), (2_000, 300, 1)])
+def test_linear_ragged_fp32_is_as_exact_as_plain_fp32(gnn, n, K, M):
+    oracle.set_threads(8)
+    try:
+        X, W, dY = synth.normal((n, K), "f32", 1400 + K), synth.normal((K, M), "f32", 1401), synth.normal((n, M), "f32", 1402 + M)
+        Xd, Wd, dYd = to_dev(X), to_dev(W), to_dev(dY)
+
+        def check(got, ref, in_a_row, what):
+            err = np.linalg.norm(to_host64(got) - ref) / np.linalg.norm(ref)
+            assert err <= in_a_row * 2.0**-24 + 2.0**-23, f"{what}: {err:.2e}"
+
+        def steps(k):
+            s = -(-k // 16)
+            return s if s <= 10 else -(-s // 2)
+
+        check(gnn.linear(Xd, Wd), oracle.matmul(X, W)[0], steps(K), "Y")
+        dX, dW = gnn.linear_backward(Xd, Wd, dYd)
+        check(dX, oracle.matmul(dY, W, tb=True)[0], steps(M), "dX")
+        check(dW, oracle.matmul(X, dY, ta=True)[0], min(32, -(-n // (148 * 16)) + 1), "dW")
+    finally:
+        oracle.set_threads(1)
+
+
 def test_linear_large_rows_tensor_core(gnn):
     """N = 100000 rows, 256 -> 256 bf16 (the attention workload's transform): many tiles per CTA."""
     import torch
