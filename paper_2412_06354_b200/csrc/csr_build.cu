@@ -141,6 +141,7 @@ struct SortArgs {
     int32_t N;
     int shift, bits;
     uint32_t ntiles;
+    int both;        // the first histogram of this launch sees the keys of both forms; otherwise it also checks the other endpoints
     int* flag;       // set if an endpoint is out of range
     int* host_flag;  // the same word for the waiting host
     const int32_t* pos;  // finalize: position of each edge in the form by target
@@ -170,6 +171,16 @@ __global__ void __launch_bounds__(RS_THREADS) radix_hist_kernel(const __grid_con
         key[r] = i < A.E ? (FIRST ? J.keys[i] : (int32_t)J.in[i].x) : 0;
     }
     bool bad = false;
+    if (FIRST && !A.both) {
+        int32_t oth[ROUNDS];
+#pragma unroll
+        for (int r = 0; r < ROUNDS; ++r) {
+            const int64_t i = rs_index<ROUNDS>(tile0, warp, r, lane);
+            oth[r] = i < A.E ? J.other[i] : 0;
+        }
+#pragma unroll
+        for (int r = 0; r < ROUNDS; ++r) bad |= oth[r] < 0 || oth[r] >= A.N;
+    }
 #pragma unroll
     for (int r = 0; r < ROUNDS; ++r) {
         if (FIRST) bad |= key[r] < 0 || key[r] >= A.N;
@@ -354,6 +365,7 @@ static SortPlan sort_plan(void* ws, int32_t N, int64_t E) {
 template <int ROUNDS>
 static cudaError_t launch_sort(SortArgs A, const SortPlan& s, int first, int jobs, cudaEvent_t validated, cudaStream_t st) {
     if (first) A.j[0] = A.j[1];
+    A.both = jobs == 2 || first;  // (the sort by target has checked all endpoints by then)
     for (int p = 0; p < s.passes; ++p) {
         A.shift = s.bits * p;
         A.bits = s.bits;
@@ -366,7 +378,7 @@ static cudaError_t launch_sort(SortArgs A, const SortPlan& s, int first, int job
         const dim3 tiles(s.ntiles, jobs), block(RS_THREADS);
         if (f) launch_overlapped(radix_hist_kernel<ROUNDS, true>, tiles, block, 0, st, A);
         else launch_overlapped(radix_hist_kernel<ROUNDS, false>, tiles, block, 0, st, A);
-        if (f) {
+        if (f && !first) {
             const cudaError_t e = cudaEventRecord(validated, st);
             if (e != cudaSuccess) return e;
         }

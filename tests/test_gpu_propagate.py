@@ -90,6 +90,34 @@ def test_coo_to_csr_rejects_out_of_range(gnn):
     assert e.value.status == 4
 
 
+def test_coo_to_csr_waits_for_the_validation_alone(gnn):
+    """From 8 Mi edges on the two sorts run one after the other; the host waits for the check of all endpoints, which is the
+    first pass over them, and not for a sort (a sort is nearly half of the time on the device)."""
+    import time
+    import torch
+    n, e = 1 << 20, 100_000_000
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    src, dst = (torch.randint(n, (e,), dtype=torch.int32, device="cuda", generator=gen) for _ in range(2))
+    ws = torch.empty(gnn.load().gnn_coo_to_csr_workspace(n, e), dtype=torch.uint8, device="cuda")
+    share = []
+    for _ in range(4):
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        g = gnn.coo_to_csr(n, src, dst, ws=ws)
+        t1 = time.perf_counter()
+        torch.cuda.synchronize()
+        share.append((t1 - t0) / (time.perf_counter() - t0))
+        del g
+    assert min(share) < 0.3, share
+    for bad in (src, dst):  # either endpoint is caught by that first pass
+        was = bad[e - 1].item()
+        bad[e - 1] = n
+        with pytest.raises(gnn.GnnError) as err:
+            gnn.coo_to_csr(n, src, dst, ws=ws)
+        assert err.value.status == 2
+        bad[e - 1] = was
+
+
 def test_self_loops_gcn_norm_permute_weighted_degree(gnn):
     import torch
     n, src, dst = ragged_graph(2, n=800, e=9000, hub=900, empty_from=800)
