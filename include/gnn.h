@@ -15,8 +15,8 @@
  *    host.  gnn_csr itself is a host struct holding device pointers.
  *  - The caller owns every buffer, including workspaces; the library never allocates or
  *    frees device memory.  Calls enqueue work on the given stream and return without
- *    synchronising, except gnn_coo_to_csr, which synchronises the stream once to read its
- *    4-byte validation word, and the *_host calls, which are documented where declared.
+ *    synchronising, except gnn_coo_to_csr, which waits once for its validation of the
+ *    endpoints (and, if that fails, for the stream), and the *_host calls, which are documented where declared.
  *  - Feature matrices are row-major with the feature index contiguous ([N,F], [E,F], [G,F]),
  *    base address 16-byte aligned, and F*sizeof(element) a multiple of 16 bytes and at most
  *    2048 bytes for the row-gathering calls (GNN_ERR_UNSUPPORTED otherwise).
@@ -93,8 +93,9 @@ int gnn_version(void);
 /* COO (the default topology format, Sec. 3 "Graph Data Structures") -> both sparse forms.
  * src, dst: int32 [E].  out: host struct whose seven array pointers the caller has set to
  * device buffers of sizes rowptr,rowptrT [N+1] int64 and col,eid,colT,eidT,t2f [E] int32; N and
- * E are filled in.  Validates 0 <= src,dst < N first (GNN_ERR_INDEX_OUT_OF_RANGE; one stream
- * synchronisation to read the flag).  ws: scratch of at least gnn_coo_to_csr_workspace bytes.
+ * E are filled in.  Validates 0 <= src,dst < N first: the host waits for that check (one event), not for the sorts queued
+ * behind it.  GNN_ERR_INDEX_OUT_OF_RANGE leaves the output arrays as they were, and after any error nothing of the call is
+ * left running.  ws: scratch of at least gnn_coo_to_csr_workspace bytes.
  * The result is unique, so it can be compared bit for bit. */
 size_t gnn_coo_to_csr_workspace(int32_t N, int64_t E);
 gnn_status gnn_coo_to_csr(int32_t N, int64_t E, const int32_t* src, const int32_t* dst,

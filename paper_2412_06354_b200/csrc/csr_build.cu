@@ -227,6 +227,7 @@ __global__ void __launch_bounds__(RS_THREADS) radix_scatter_kernel(const __grid_
     const SortJob& J = A.j[blockIdx.y];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, bins = 1 << A.bits;
     const int64_t tile0 = (int64_t)blockIdx.x * (RS_THREADS * ROUNDS);
+    const int refused = LAST ? *(const volatile int*)A.flag : 0;  // an endpoint out of range: the outputs stay as they are
     uint2 kv[ROUNDS];
 #pragma unroll
     for (int r = 0; r < ROUNDS; ++r) {
@@ -234,6 +235,7 @@ __global__ void __launch_bounds__(RS_THREADS) radix_scatter_kernel(const __grid_
         kv[r] = make_uint2(0u, 0u);
         if (i < A.E) kv[r] = FIRST ? make_uint2((uint32_t)J.keys[i], (uint32_t)i) : J.in[i];
     }
+    if (refused) return;
     for (int d = threadIdx.x; d < RS_WARPS * RS_MAX_BINS / 2; d += RS_THREADS) reinterpret_cast<uint32_t*>(wcnt)[d] = 0;
     {  // where each digit's keys of this tile begin: digits before, then tiles before
         const int per = RS_MAX_BINS / RS_THREADS;
@@ -658,6 +660,11 @@ gnn_status gnn_coo_to_csr(int32_t N, int64_t E, const int32_t* src, const int32_
     }
     if (e == cudaSuccess) e = cudaEventSynchronize(slot.event);
     const int bad = *(volatile int*)slot.word;
+    // on any error nothing of the call is left running on the caller's buffers when it returns
+    if (e != cudaSuccess || bad) {
+        const cudaError_t quiet = cudaStreamSynchronize(st);
+        if (e == cudaSuccess) e = quiet;
+    }
     give_slot(slot);
     if (e != cudaSuccess) GNN_FAIL(GNN_ERR_CUDA, "gnn_coo_to_csr: %s", cudaGetErrorString(e));
     GNN_REQUIRE(bad == 0, GNN_ERR_INDEX_OUT_OF_RANGE,

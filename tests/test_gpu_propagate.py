@@ -90,6 +90,27 @@ def test_coo_to_csr_rejects_out_of_range(gnn):
     assert e.value.status == 4
 
 
+@pytest.mark.parametrize("n,e", [(50, 700), (3000, 300_000), (3_000_000, 9_000_000)])  # one and two passes at once, three one after the other
+def test_coo_to_csr_refuses_before_it_writes(gnn, n, e):
+    import torch
+    lib = gnn.load()
+    rng = np.random.default_rng(e)
+    good = [rng.integers(0, n, e).astype(np.int32) for _ in range(2)]
+    for which, at, value in ((0, e - 1, n), (1, 0, -1), (0, e // 2, 2**31 - 1), (1, e - 1, -2**31)):
+        ends = [a.copy() for a in good]
+        ends[which][at] = value
+        src, dst = (to_dev(a) for a in ends)
+        g = gnn.Graph(n, e, "cuda")
+        arrays = (g.rowptr, g.rowptrT, g.col, g.eid, g.colT, g.eidT, g.t2f)
+        for t in arrays:
+            t.fill_(-7)
+        ws = torch.empty(lib.gnn_coo_to_csr_workspace(n, e), dtype=torch.uint8, device="cuda")
+        rc = lib.gnn_coo_to_csr(n, e, src.data_ptr(), dst.data_ptr(), g.ref, ws.data_ptr(), ws.numel(), torch.cuda.current_stream().cuda_stream)
+        assert rc == 2 and torch.cuda.current_stream().query(), "work left in the stream"
+        for t in arrays:
+            assert bool((t == -7).all())
+
+
 def test_coo_to_csr_waits_for_the_validation_alone(gnn):
     """From 8 Mi edges on the two sorts run one after the other; the host waits for the check of all endpoints, which is the
     first pass over them, and not for a sort (a sort is nearly half of the time on the device)."""
