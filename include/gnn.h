@@ -14,7 +14,9 @@
  *  - Every pointer is a DEVICE pointer unless its name starts with h_ or the comment says
  *    host.  gnn_csr itself is a host struct holding device pointers.
  *  - The caller owns every buffer, including workspaces; the library never allocates or
- *    frees device memory.  Calls enqueue work on the given stream and return without
+ *    frees device memory.  What it keeps itself: gnn_coo_to_csr a word of pinned host memory and an event per
+ *    call in progress, of which at most eight stay for later calls, and the attention calls the streams
+ *    and events named there.  Calls enqueue work on the given stream and return without
  *    synchronising, except gnn_coo_to_csr, which waits once for its validation of the
  *    endpoints (and, if that fails, for the stream), and the *_host calls, which are documented where declared.
  *  - Feature matrices are row-major with the feature index contiguous ([N,F], [E,F], [G,F]),

@@ -2,9 +2,7 @@
 // self-loops, edge-data permutation.  Integer results are unique and bit-exact.
 #include <stdarg.h>
 
-#include <mutex>
-#include <vector>
-
+#include "flag_slots.h"
 #include "reduce_params.cuh"
 
 namespace gnn {
@@ -394,37 +392,15 @@ static cudaError_t launch_sort(SortArgs A, const SortPlan& s, int first, int job
     return cudaGetLastError();
 }
 
-// A word of pinned host memory and an event: the host waits for the validation of the endpoints, which is done long before
-// the sorts that are queued behind it.  Slots are handed out one per call in progress and kept for the next (as many as
-// calls ever ran at once on a device).
-struct FlagSlot { int* word; cudaEvent_t event; int device; };
-static std::mutex g_slots_mutex;
-static std::vector<FlagSlot> g_slots;
-
-static bool take_slot(FlagSlot* s) {
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess) return false;
-    {
-        std::lock_guard<std::mutex> lock(g_slots_mutex);
-        for (size_t k = 0; k < g_slots.size(); ++k)
-            if (g_slots[k].device == dev) {
-                *s = g_slots[k];
-                g_slots.erase(g_slots.begin() + (long)k);
-                return true;
-            }
-    }
-    s->device = dev;
-    if (cudaHostAlloc((void**)&s->word, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) return false;
-    if (cudaEventCreateWithFlags(&s->event, cudaEventDisableTiming) != cudaSuccess) {
-        cudaFreeHost(s->word);
-        return false;
-    }
-    return true;
-}
-static void give_slot(const FlagSlot& s) {
-    std::lock_guard<std::mutex> lock(g_slots_mutex);
-    g_slots.push_back(s);
-}
+// The host waits for the validation of the endpoints, which is done long before the sorts that are queued behind it.
+struct CudaSlots {
+    using Event = cudaEvent_t;
+    static bool make_word(int** w) { return cudaHostAlloc((void**)w, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) == cudaSuccess; }
+    static void free_word(int* w) { cudaFreeHost(w); }
+    static bool make_event(Event* e) { return cudaEventCreateWithFlags(e, cudaEventDisableTiming) == cudaSuccess; }
+    static void free_event(Event e) { cudaEventDestroy(e); }
+};
+static FlagSlots<CudaSlots> g_slots;
 
 // ------------------------------------------------------------------ degrees / GCN coefficients
 __global__ void degree_count_kernel(int32_t N, const int64_t* __restrict__ rowptr,
@@ -641,8 +617,9 @@ gnn_status gnn_coo_to_csr(int32_t N, int64_t E, const int32_t* src, const int32_
     }
     GNN_REQUIRE(N > 0, GNN_ERR_INDEX_OUT_OF_RANGE, "gnn_coo_to_csr: an edge endpoint is outside [0, %d)", N);
     const SortPlan s = sort_plan(ws, N, E);
-    FlagSlot slot;
-    if (!take_slot(&slot)) GNN_FAIL(GNN_ERR_CUDA, "gnn_coo_to_csr: no pinned memory for the validation word: %s", cudaGetErrorString(cudaGetLastError()));
+    FlagSlots<CudaSlots>::Slot slot;
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || !g_slots.take(dev, &slot)) GNN_FAIL(GNN_ERR_CUDA, "gnn_coo_to_csr: no pinned memory for the validation word: %s", cudaGetErrorString(cudaGetLastError()));
     *(volatile int*)slot.word = 0;
     SortArgs A = {};
     A.E = E; A.N = N; A.ntiles = s.ntiles; A.flag = s.flag; A.host_flag = slot.word; A.pos = s.pos; A.t2f = out->t2f;
@@ -660,12 +637,11 @@ gnn_status gnn_coo_to_csr(int32_t N, int64_t E, const int32_t* src, const int32_
     }
     if (e == cudaSuccess) e = cudaEventSynchronize(slot.event);
     const int bad = *(volatile int*)slot.word;
-    // on any error nothing of the call is left running on the caller's buffers when it returns
-    if (e != cudaSuccess || bad) {
-        const cudaError_t quiet = cudaStreamSynchronize(st);
-        if (e == cudaSuccess) e = quiet;
-    }
-    give_slot(slot);
+    // on any error nothing of the call is left running on the caller's buffers, or on the slot, when it returns
+    cudaError_t quiet = cudaSuccess;
+    if (e != cudaSuccess || bad) quiet = cudaStreamSynchronize(st);
+    g_slots.give(slot, quiet == cudaSuccess);
+    if (e == cudaSuccess) e = quiet;
     if (e != cudaSuccess) GNN_FAIL(GNN_ERR_CUDA, "gnn_coo_to_csr: %s", cudaGetErrorString(e));
     GNN_REQUIRE(bad == 0, GNN_ERR_INDEX_OUT_OF_RANGE,
                 "gnn_coo_to_csr: an edge endpoint is outside [0, %d)", N);
