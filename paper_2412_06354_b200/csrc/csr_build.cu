@@ -347,8 +347,9 @@ static SortPlan sort_plan(void* ws, int32_t N, int64_t E) {
     s.bits = (bits + s.passes - 1) / s.passes;
     s.ntiles = (uint32_t)ceil_div(E > 0 ? E : 1, RS_THREADS * s.rounds);
     char* p = (char*)ws;
-    size_t off = 0;
-    s.flag = (int*)(p + off); off += 256;
+    // the flag, then everything else: pairs are read and written as 8 bytes, also in a workspace that begins between two of them
+    s.flag = (int*)p;
+    size_t off = 256 - reinterpret_cast<uintptr_t>(ws) % 8;
     const size_t pairs = up256((size_t)(E > 0 ? E : 1) * 8), bins = (size_t)1 << most;
     for (int k = 0; k < 2; ++k) {
         if (k == 1 && !s.both) { s.a[1] = s.a[0]; s.b[1] = s.b[0]; s.table[1] = s.table[0]; s.totals[1] = s.totals[0]; continue; }

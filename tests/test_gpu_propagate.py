@@ -111,6 +111,22 @@ def test_coo_to_csr_refuses_before_it_writes(gnn, n, e):
             assert bool((t == -7).all())
 
 
+def test_coo_to_csr_workspace_on_four_bytes(gnn):
+    """A workspace carved from a buffer of 4-byte words, which need not begin on 8."""
+    import torch
+    n, src, dst = ragged_graph(4, n=70_000, e=90_000, hub=3000, empty_from=69_000)  # two passes per sort: pairs in between
+    need = gnn.load().gnn_coo_to_csr_workspace(n, len(src))
+    ref = build_graph(gnn, n, src, dst)
+    for off in (4, 12):
+        room = torch.full((need + off + 64,), 0xA5, dtype=torch.uint8, device="cuda")
+        ws = room[off:off + need]
+        assert ws.data_ptr() % 8 == 4
+        g = gnn.coo_to_csr(n, to_dev(src), to_dev(dst), ws=ws)
+        for k in ("rowptr", "rowptrT", "col", "eid", "colT", "eidT", "t2f"):
+            assert torch.equal(getattr(g, k), getattr(ref, k)), k
+        assert bool((room[:off] == 0xA5).all()) and bool((room[off + need:] == 0xA5).all())
+
+
 def test_coo_to_csr_waits_for_the_validation_alone(gnn):
     """From 8 Mi edges on the two sorts run one after the other; the host waits for the check of all endpoints, which is the
     first pass over them, and not for a sort (a sort is nearly half of the time on the device)."""
