@@ -97,7 +97,7 @@ int gnn_version(void);
  * device buffers of sizes rowptr,rowptrT [N+1] int64 and col,eid,colT,eidT,t2f [E] int32; N and
  * E are filled in.  Validates 0 <= src,dst < N first: the host waits for that check (one event), not for the sorts queued
  * behind it.  GNN_ERR_INDEX_OUT_OF_RANGE leaves the output arrays as they were, and after any error nothing of the call is
- * left running.  ws: scratch of at least gnn_coo_to_csr_workspace bytes.
+ * left running.  ws: scratch of at least gnn_coo_to_csr_workspace bytes, asked for this E or a larger one.
  * The result is unique, so it can be compared bit for bit. */
 size_t gnn_coo_to_csr_workspace(int32_t N, int64_t E);
 gnn_status gnn_coo_to_csr(int32_t N, int64_t E, const int32_t* src, const int32_t* dst,

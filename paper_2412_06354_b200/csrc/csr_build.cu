@@ -336,9 +336,11 @@ struct SortPlan {
     size_t bytes;
 };
 
-static SortPlan sort_plan(void* ws, int32_t N, int64_t E) {
+// Both sorts at once need twice the buffers.  A workspace that was sized for a graph of more edges, whose sorts run one after
+// the other, may lack them: then a smaller graph's do so too (`both` is a wish).  So a size that serves E serves fewer edges.
+static SortPlan sort_plan(void* ws, int32_t N, int64_t E, bool both = true) {
     SortPlan s;
-    s.both = E < SORT_BOTH;
+    s.both = both && E < SORT_BOTH;
     s.rounds = s.both ? 8 : 16;
     int bits = 1;
     while (bits < 31 && ((int64_t)1 << bits) < (int64_t)N) ++bits;
@@ -606,7 +608,8 @@ gnn_status gnn_coo_to_csr(int32_t N, int64_t E, const int32_t* src, const int32_
     GNN_REQUIRE(out && out->rowptr && out->rowptrT, GNN_ERR_INVALID_ARG, "gnn_coo_to_csr: null output");
     GNN_REQUIRE(E == 0 || (src && dst && out->col && out->eid && out->colT && out->eidT && out->t2f),
                 GNN_ERR_INVALID_ARG, "gnn_coo_to_csr: null edge array");
-    GNN_REQUIRE(ws && ws_bytes >= gnn_coo_to_csr_workspace(N, E), GNN_ERR_WORKSPACE_TOO_SMALL,
+    const bool both = ws_bytes >= gnn_coo_to_csr_workspace(N, E);
+    GNN_REQUIRE(ws && ws_bytes >= sort_plan(nullptr, N, E, both).bytes, GNN_ERR_WORKSPACE_TOO_SMALL,
                 "gnn_coo_to_csr: workspace of %zu bytes needed", gnn_coo_to_csr_workspace(N, E));
     cudaStream_t st = as_stream(stream);
     out->N = N;
@@ -617,7 +620,7 @@ gnn_status gnn_coo_to_csr(int32_t N, int64_t E, const int32_t* src, const int32_
         return GNN_OK;
     }
     GNN_REQUIRE(N > 0, GNN_ERR_INDEX_OUT_OF_RANGE, "gnn_coo_to_csr: an edge endpoint is outside [0, %d)", N);
-    const SortPlan s = sort_plan(ws, N, E);
+    const SortPlan s = sort_plan(ws, N, E, both);
     FlagSlots<CudaSlots>::Slot slot;
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || !g_slots.take(dev, &slot)) GNN_FAIL(GNN_ERR_CUDA, "gnn_coo_to_csr: no pinned memory for the validation word: %s", cudaGetErrorString(cudaGetLastError()));

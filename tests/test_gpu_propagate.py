@@ -127,6 +127,20 @@ def test_coo_to_csr_workspace_on_four_bytes(gnn):
         assert bool((room[:off] == 0xA5).all()) and bool((room[off + need:] == 0xA5).all())
 
 
+def test_coo_to_csr_workspace_of_a_larger_graph(gnn):
+    """A workspace sized for the largest graph serves the smaller ones: from 8 Mi edges on less of it is asked for than just below."""
+    import torch
+    lib = gnn.load()
+    ws = torch.empty(lib.gnn_coo_to_csr_workspace(1 << 20, 8 << 20), dtype=torch.uint8, device="cuda")
+    for n, e in ((1 << 20, (8 << 20) - 1), (900, (8 << 20) - 4097), (70_001, 7_000_000)):
+        assert ws.numel() < lib.gnn_coo_to_csr_workspace(n, e)
+        gen = torch.Generator(device="cuda").manual_seed(e)
+        src, dst = (torch.randint(n, (e,), dtype=torch.int32, device="cuda", generator=gen) for _ in range(2))
+        g, ref = gnn.coo_to_csr(n, src, dst, ws=ws), gnn.coo_to_csr(n, src, dst)
+        for k in ("rowptr", "rowptrT", "col", "eid", "colT", "eidT", "t2f"):
+            assert torch.equal(getattr(g, k), getattr(ref, k)), k
+
+
 def test_coo_to_csr_waits_for_the_validation_alone(gnn):
     """From 8 Mi edges on the two sorts run one after the other; the host waits for the check of all endpoints, which is the
     first pass over them, and not for a sort (a sort is nearly half of the time on the device)."""
