@@ -729,12 +729,18 @@ gnn_status gnn_gcn_norm(const gnn_csr* g, const float* w_csr, float* deg_out, fl
         launch_overlapped(degree_unit_kernel, dim3((unsigned)ceil_div(g->N, 256)), dim3(256), 0, st, g->N, g->rowptr, deg_out);
     if (coef_csr && g->E > 0) {
         GNN_REQUIRE(g->col, GNN_ERR_INVALID_ARG, "gnn_gcn_norm: null col");
-        GNN_REQUIRE(!coef_csrT || (g->t2f && g->rowptrT && g->colT), GNN_ERR_INVALID_ARG, "gnn_gcn_norm: null t2f");
+        GNN_REQUIRE(!coef_csrT || g->t2f, GNN_ERR_INVALID_ARG, "gnn_gcn_norm: null t2f");
+        // both forms in one launch need the transposed form's rows, and weights that neither output overwrites; else the
+        // second is the first, reordered
+        auto apart = [&](const float* out) { return !w_csr || w_csr + g->E <= out || out + g->E <= w_csr; };
+        const bool both = coef_csrT && g->rowptrT && g->colT && apart(coef_csr) && apart(coef_csrT);
         CoefArgs A = {};
         A.f[0] = {g->rowptr, g->col, nullptr, coef_csr, aligned16(g->col) && aligned16(coef_csr)};
         A.f[1] = {g->rowptrT, g->colT, g->t2f, coef_csrT, aligned16(g->colT) && aligned16(g->t2f) && aligned16(coef_csrT)};
         A.w = w_csr; A.deg = deg_out; A.N = g->N; A.E = g->E;
-        launch_overlapped(gcn_coef_kernel, dim3((unsigned)ceil_div(g->E, 256 * 8), coef_csrT ? 2 : 1), dim3(256), 0, st, A);
+        launch_overlapped(gcn_coef_kernel, dim3((unsigned)ceil_div(g->E, 256 * 8), both ? 2 : 1), dim3(256), 0, st, A);
+        if (coef_csrT && !both)
+            launch_overlapped(permute_rows_kernel<uint32_t>, dim3((unsigned)grid_for(g->E, 256)), dim3(256), 0, st, g->E, 1, g->t2f, (const uint32_t*)coef_csr, (uint32_t*)coef_csrT);
     }
     GNN_CHECK_LAUNCH("gnn_gcn_norm");
     return GNN_OK;

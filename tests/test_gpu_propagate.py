@@ -199,6 +199,31 @@ def test_self_loops_gcn_norm_permute_weighted_degree(gnn):
     assert np.array_equal(bits(got), host_bits(e2[ref["eidT"]]))
 
 
+def test_gcn_norm_without_the_transposed_rows_and_in_place(gnn):
+    """Of the transposed form the coefficients need t2f alone; weights may be overwritten by either output."""
+    import torch
+    n, src, dst = ragged_graph(12, n=900, e=9001, hub=700, empty_from=850)
+    g = build_graph(gnn, n, src, dst)
+    w = to_dev(synth.uniform_f32((g.E,), 0.1, 1.0, 7))
+    deg, coef, coefT = gnn.gcn_norm(g, w)
+    lib, st = gnn.load(), torch.cuda.current_stream().cuda_stream
+    part = gnn.CsrStruct(n, g.E, g.rowptr.data_ptr(), g.col.data_ptr(), None, None, None, None, g.t2f.data_ptr())
+
+    def call(struct, weights, out, outT):
+        d = torch.empty(n, device="cuda")
+        gnn._check(lib.gnn_gcn_norm(struct, weights.data_ptr(), d.data_ptr(), out.data_ptr(), outT.data_ptr(), st))
+        assert torch.equal(d, deg) and torch.equal(out, coef) and torch.equal(outT, coefT)
+
+    call(part, w, torch.empty_like(w), torch.empty_like(w))
+    for _ in range(20):
+        inplace = w.clone()
+        call(g.c, inplace, inplace, torch.empty_like(w))
+        inplace = w.clone()
+        d, out = torch.empty(n, device="cuda"), torch.empty_like(w)
+        gnn._check(lib.gnn_gcn_norm(g.ref, inplace.data_ptr(), d.data_ptr(), out.data_ptr(), inplace.data_ptr(), st))
+        assert torch.equal(out, coef) and torch.equal(inplace, coefT)
+
+
 # ---------------------------------------------------------------- forward
 SHAPES = [("f32", 4), ("f32", 32), ("f32", 64), ("f32", 100), ("f32", 128), ("f32", 256), ("f32", 512),
           ("bf16", 8), ("bf16", 32), ("bf16", 64), ("bf16", 128), ("bf16", 200), ("bf16", 256), ("bf16", 512), ("bf16", 1024)]
