@@ -466,9 +466,10 @@ gnn_status gnn_reduce_nodes_backward(const int64_t* graph_ptr, int32_t G, int32_
  * to 1024 the products run on the tensor cores with fp32 accumulation: bf16 directly, fp32 by an exact
  * three-term bf16 split of every value, which keeps fp32 accuracy (weights that do not fit shared memory
  * three times, e.g. 256x256, run as one launch per block of output columns).  Rows that do not start on 16 bytes
- * (K or M not a multiple of 16 bytes worth of elements) are first copied to padded rows in the workspace; a
- * forward call given less than gnn_linear_workspace bytes (256 are the least) then uses an fp32 FFMA kernel,
- * several times slower, as larger K and M do.  The first call on a device looks up the driver's tensor-map encoder;
+ * (K or M not a multiple of 16 bytes worth of elements) are first copied to padded rows in the workspace.  A
+ * call given less than gnn_linear_workspace bytes (say, sized for a wider layer without such rows; the least are
+ * 256 bytes forward, 512 + 4 K M max(148, ceil(N / 4096)) backward) then uses an fp32 FFMA kernel, several times
+ * slower, as larger K and M do.  The first call on a device looks up the driver's tensor-map encoder;
  * the calls themselves allocate nothing.
  * ws: gnn_linear_workspace(N, K, M) bytes; its first 4 bytes are a device status word that the
  * tensor-core path sets to GNN_ERR_TIMEOUT if one of its bounded waits expired (0 otherwise);

@@ -178,8 +178,10 @@ static int padded(int cols, int s) { return round_up(cols, 16 / s); }
 
 // Workspace layout: status word (256 bytes), dW partials, then the padded copies of X, dY and W.  The element type is not
 // known where the size is asked for: rows that would be padded in either type count, in the larger one.
+// least: what a backward call needs without the copies and the rounded partials (the FFMA kernel, and shapes without either).
+// It grows with K and M, so that a workspace sized for the widest layer serves the others; `bytes` does not.
 struct LinearWs {
-    size_t part, x, dy, w, bytes;
+    size_t part, x, dy, w, bytes, least;
     LinearWs(int64_t N, int K, int M) {
         const size_t parts = (size_t)(dw_slabs(N) > 148 ? dw_slabs(N) : 148);  // FFMA slabs or tensor-core CTA partials
         auto copy = [](int64_t rows, int cols) -> size_t {
@@ -188,6 +190,7 @@ struct LinearWs {
             return up256(b2 > b4 ? b2 : b4);
         };
         part = 256;
+        least = part + up256(parts * K * M * 4);
         x = part + up256(parts * round_up(K, 32) * round_up(M, 32) * 4);
         dy = x + copy(N, K);
         w = dy + copy(N, M);
@@ -271,7 +274,7 @@ gnn_status gnn_linear_backward(const void* X, const void* W, const void* dY, int
     GNN_REQUIRE(dtype == GNN_F32 || dtype == GNN_BF16, GNN_ERR_INVALID_ARG, "%s: bad dtype", who);
     GNN_REQUIRE(dY || N == 0, GNN_ERR_INVALID_ARG, "%s: null dY", who);
     const LinearWs lw(N, K, M);
-    GNN_REQUIRE(ws && ws_bytes >= lw.bytes, GNN_ERR_WORKSPACE_TOO_SMALL, "%s: workspace of %zu bytes needed", who, lw.bytes);
+    GNN_REQUIRE(ws && ws_bytes >= lw.least, GNN_ERR_WORKSPACE_TOO_SMALL, "%s: workspace of %zu bytes needed", who, lw.bytes);
     GNN_REQUIRE(!dX || N == 0 || W, GNN_ERR_INVALID_ARG, "%s: dX needs W", who);
     GNN_REQUIRE(!dW || N == 0 || X, GNN_ERR_INVALID_ARG, "%s: dW needs X", who);
     cudaStream_t st = as_stream(stream);
@@ -279,13 +282,14 @@ gnn_status gnn_linear_backward(const void* X, const void* W, const void* dY, int
     char* w8 = (char*)ws;
     int* const status = (int*)ws;
     const bool on16 = aligned16(dY) && aligned16(ws);
+    const bool room = ws_bytes >= lw.bytes;
     // dX[n,k] = sum_m dY[n,m] * W[k,m]
-    const bool dx_tma = dX && N > 0 && on16 && aligned16(W) && (dtype == GNN_F32 ? linear_tma_f32_supported(N, M, K, dtype) : linear_tma_supported(N, M, K, 1, dtype));
+    const bool dx_tma = dX && N > 0 && on16 && (room || M * s % 16 == 0) && aligned16(W) && (dtype == GNN_F32 ? linear_tma_f32_supported(N, M, K, dtype) : linear_tma_supported(N, M, K, 1, dtype));
     // dW[k,m] = sum_n X[n,k] * dY[n,m]: one fp32 partial per CTA, then summed in CTA order.  More output columns than one
     // launch takes (256, or fewer where K fills tensor memory): one launch and one ordered sum per block of columns of dY.
     auto dw_supported = [&](int mc) { return dtype == GNN_F32 ? linear_tma_f32_dw_supported(N, K, mc, M, dtype) : linear_tma_dw_supported(N, K, mc, dtype); };
     int block = 0;
-    if (dW && N > 0 && on16 && aligned16(X)) {
+    if (dW && N > 0 && on16 && aligned16(X) && (room || (K % 32 == 0 && M % (dtype == GNN_F32 ? 32 : 16) == 0))) {
         if (dw_supported(M)) block = M;
         else
             for (int mc = (M < 256 ? M : 256) / 32 * 32; mc >= 32 && !block; mc -= 32)

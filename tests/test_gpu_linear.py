@@ -108,6 +108,30 @@ def test_linear_ragged_sizes(gnn, dtype, n, K, M):
         oracle.set_threads(1)
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("K,M", [(100, 47), (104, 40), (48, 16), (96, 20), (128, 128), (36, 128)])
+def test_linear_backward_workspace_of_a_wider_layer(gnn, dtype, K, M):
+    """A workspace sized for 128 x 128 serves every layer up to that, with rows to be padded or partials to be rounded up or not."""
+    import torch
+    n = 3000
+    lib = gnn.load()
+    wide = lib.gnn_linear_workspace(n, 128, 128)
+    X, W, dY = synth.normal((n, K), dtype, 1500 + K), synth.normal((K, M), dtype, 1501), synth.normal((n, M), dtype, 1502 + M)
+    dXo, Sx = oracle.matmul(dY, W, tb=True)
+    dWo, Sw = oracle.matmul(X, dY, ta=True)
+    least = 512 + 4 * K * M * 148
+    for size in (wide, least):
+        room = torch.full((max(size, 256) + 64,), 0xA5, dtype=torch.uint8, device="cuda")
+        ws = room[:size]
+        dX, dW = gnn.linear_backward(to_dev(X), to_dev(W), to_dev(dY), ws=ws)
+        assert status_word(ws) == 0 and bool((room[size:] == 0xA5).all())
+        assert_close(to_host64(dX), dXo, Sx, dtype, "dX")
+        assert_close(to_host64(dW), dWo, Sw, dtype, "dW")
+    with pytest.raises(gnn.GnnError) as e:
+        gnn.linear_backward(to_dev(X), to_dev(W), to_dev(dY), ws=room[:4 * K * M * 148])
+    assert e.value.status == 4
+
+
 # fp32 sums of sizes that divide nothing: no further from 64 bits than plain fp32 FMAs.  The tensor core truncates its accumulator at
 # every MMA of 16 terms, half a unit in the last place (2^-23 of the running sum) on average and one way; at most 10 main MMAs of
 # a forward sum follow one another (16 in each of two sums above that), 32 in dW, and the sums are then added with rounding:
