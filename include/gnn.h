@@ -469,7 +469,8 @@ gnn_status gnn_reduce_nodes_backward(const int64_t* graph_ptr, int32_t G, int32_
  * (K or M not a multiple of 16 bytes worth of elements) are first copied to padded rows in the workspace.  A
  * call given less than gnn_linear_workspace bytes (say, sized for a wider layer without such rows; the least are
  * 256 bytes forward, 512 + 4 K M max(148, ceil(N / 4096)) backward) then uses an fp32 FFMA kernel, several times
- * slower, as larger K and M do.  The first call on a device looks up the driver's tensor-map encoder;
+ * slower, as larger K and M do.  So do sizes that are no multiples of 16 if a matrix is not on 16 bytes; multiples of
+ * 16 return GNN_ERR_INVALID_ARG then.  The first call on a device looks up the driver's tensor-map encoder;
  * the calls themselves allocate nothing.
  * ws: gnn_linear_workspace(N, K, M) bytes; its first 4 bytes are a device status word that the
  * tensor-core path sets to GNN_ERR_TIMEOUT if one of its bounded waits expired (0 otherwise);

@@ -198,6 +198,9 @@ struct LinearWs {
     }
 };
 
+// contraction and columns that the copy engine took before others were padded for it
+static bool sixteens(int Kc, int Mo, int s) { return Kc % 16 == 0 && Mo % 16 == 0 && (Kc <= 256 || Kc % 32 == 0 || s == 4); }
+
 // rows on 16 bytes: src itself, or its copy at dst
 static const void* with_padded_rows(const void* src, int64_t rows, int cols, int s, void* dst, cudaStream_t st) {
     const int ld = padded(cols, s);
@@ -241,7 +244,10 @@ gnn_status gnn_linear_bias_act(const void* X, const void* W, int32_t N, int K, i
     // the status word alone is enough where no rows have to be padded; where they do, a caller with that little gets the
     // kernels that need no padding
     const bool pads = K * s % 16 != 0 || (s == 2 && M * s % 16 != 0);
-    if ((!pads || ws_bytes >= lw.bytes) && aligned16(X) && aligned16(W) && aligned16(ws)) {
+    // Multiples of 16 have always asked for matrices on 16 bytes (the launches below refuse others); any other size takes
+    // matrices on whole elements, and the FFMA kernel if one of them is off 16 bytes.
+    const bool on16 = aligned16(X) && aligned16(W) && (aligned16(Y) || M * s % 16 != 0);
+    if (sixteens(K, M, s) || ((!pads || (ws_bytes >= lw.bytes && aligned16(ws))) && on16)) {
         if (linear_tma_supported(N, K, M, 0, dtype)) {
             const void* Xp = with_padded_rows(X, N, K, s, w8 + lw.x, st);
             const void* Wp = with_padded_rows(W, K, M, s, w8 + lw.w, st);
@@ -281,15 +287,15 @@ gnn_status gnn_linear_backward(const void* X, const void* W, const void* dY, int
     const int s = elem_size(dtype);
     char* w8 = (char*)ws;
     int* const status = (int*)ws;
-    const bool on16 = aligned16(dY) && aligned16(ws);
-    const bool room = ws_bytes >= lw.bytes;
+    const bool room = ws_bytes >= lw.bytes && aligned16(ws);
     // dX[n,k] = sum_m dY[n,m] * W[k,m]
-    const bool dx_tma = dX && N > 0 && on16 && (room || M * s % 16 == 0) && aligned16(W) && (dtype == GNN_F32 ? linear_tma_f32_supported(N, M, K, dtype) : linear_tma_supported(N, M, K, 1, dtype));
+    const bool dx_on16 = aligned16(dY) && aligned16(W) && (aligned16(dX) || K * s % 16 != 0);
+    const bool dx_tma = dX && N > 0 && (sixteens(M, K, s) || (dx_on16 && (room || M * s % 16 == 0))) && (dtype == GNN_F32 ? linear_tma_f32_supported(N, M, K, dtype) : linear_tma_supported(N, M, K, 1, dtype));
     // dW[k,m] = sum_n X[n,k] * dY[n,m]: one fp32 partial per CTA, then summed in CTA order.  More output columns than one
     // launch takes (256, or fewer where K fills tensor memory): one launch and one ordered sum per block of columns of dY.
     auto dw_supported = [&](int mc) { return dtype == GNN_F32 ? linear_tma_f32_dw_supported(N, K, mc, M, dtype) : linear_tma_dw_supported(N, K, mc, dtype); };
     int block = 0;
-    if (dW && N > 0 && on16 && aligned16(X) && (room || (K % 32 == 0 && M % (dtype == GNN_F32 ? 32 : 16) == 0))) {
+    if (dW && N > 0 && ((K % 32 == 0 && M % (dtype == GNN_F32 ? 32 : 16) == 0) || (room && aligned16(X) && aligned16(dY)))) {
         if (dw_supported(M)) block = M;
         else
             for (int mc = (M < 256 ? M : 256) / 32 * 32; mc >= 32 && !block; mc -= 32)

@@ -132,6 +132,41 @@ def test_linear_backward_workspace_of_a_wider_layer(gnn, dtype, K, M):
     assert e.value.status == 4
 
 
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("K,M", [(100, 48), (20, 40), (47, 33), (64, 64), (64, 24)])
+def test_linear_matrices_off_16_bytes(gnn, dtype, K, M):
+    """Sizes that are no multiples of 16 take matrices that begin at any element, multiples of 16 refuse them."""
+    import torch
+    n, s = 700, 4 if dtype == "f32" else 2
+    lib, st = gnn.load(), torch.cuda.current_stream().cuda_stream
+    X, W, dY = synth.normal((n, K), dtype, 1600 + K), synth.normal((K, M), dtype, 1601), synth.normal((n, M), dtype, 1602 + M)
+    want = [oracle.matmul(X, W), oracle.matmul(dY, W, tb=True), oracle.matmul(X, dY, ta=True)]
+
+    def at(a, off):  # the matrix, one element past a 16-byte boundary if off
+        room = torch.zeros(a.numel() + 8, dtype=a.dtype, device="cuda")
+        v = room[off:off + a.numel()].view(a.shape)
+        v.copy_(a)
+        return v
+
+    ws = torch.empty(lib.gnn_linear_workspace(n, K, M), dtype=torch.uint8, device="cuda")
+    d = [to_dev(a) for a in (X, W, dY)]
+    outs = [torch.zeros(sh, dtype=d[0].dtype, device="cuda") for sh in ((n, M), (n, K), (K, M))]
+    code = {"f32": gnn.F32, "bf16": gnn.BF16}[dtype]
+    for odd in range(5):  # X, W, dY, Y, dX
+        x, w, dy, y, dx = (at(a, k == odd) for k, a in enumerate((*d, outs[0], outs[1])))
+        dw = outs[2]
+        rc = [lib.gnn_linear(x.data_ptr(), w.data_ptr(), n, K, M, code, y.data_ptr(), ws.data_ptr(), ws.numel(), st),
+              lib.gnn_linear_backward(None, w.data_ptr(), dy.data_ptr(), n, K, M, code, dx.data_ptr(), None, ws.data_ptr(), ws.numel(), st),
+              lib.gnn_linear_backward(x.data_ptr(), None, dy.data_ptr(), n, K, M, code, None, dw.data_ptr(), ws.data_ptr(), ws.numel(), st)]
+        touches = [odd in (0, 1, 3), odd in (1, 2, 4), odd in (0, 2)]
+        for k, (got, what) in enumerate(((y, "Y"), (dx, "dX"), (dw, "dW"))):
+            if (K, M) == (64, 64) and touches[k]:
+                assert rc[k] == 1, (odd, what)
+            else:
+                assert rc[k] == 0, (odd, what)
+                assert_close(to_host64(got), *want[k], dtype, f"{what}, matrix {odd} off 16 bytes")
+
+
 # fp32 sums of sizes that divide nothing: no further from 64 bits than plain fp32 FMAs.  The tensor core truncates its accumulator at
 # every MMA of 16 terms, half a unit in the last place (2^-23 of the running sum) on average and one way; at most 10 main MMAs of
 # a forward sum follow one another (16 in each of two sums above that), 32 in dW, and the sums are then added with rounding:
