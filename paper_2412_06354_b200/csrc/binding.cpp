@@ -120,6 +120,14 @@ struct Args {
         }
         return (gnn_op)i(k);
     }
+    // heads of a row of F features: their number, and the features of one
+    int heads(int k, int64_t F, int* C) const {
+        const int64_t H = i(k);
+        if (H == 0) raise(PyExc_ZeroDivisionError, "the number of heads is zero");
+        const int64_t q = F / H;
+        *C = (int)(F % H != 0 && (F < 0) != (H < 0) ? q - 1 : q);
+        return (int)H;
+    }
     const gnn_csr* g(int k) const { return reinterpret_cast<const gnn_csr*>((intptr_t)i(k)); }
 };
 
@@ -531,11 +539,12 @@ FN(gin_backward) {
 FN(edge_dot) {
     const gnn_csr* g = A.g(0);
     const at::Tensor &Xj = A.dev(1), &Xi = A.dev(2);
-    const int H = (int)A.i(3), F = (int)Xj.size(1);
+    int C;
+    const int H = A.heads(3, Xj.size(1), &C);
     at::Tensor s = empty({at_least_one(g->E), H}, at::kFloat, Xj.device());
     const gnn_dtype dt = dtype_of(Xj);
     const gnn_stream st = stream();
-    CALL(gnn_edge_dot(g, ptr(Xj), ptr(Xi), H, F / H, dt, (float*)ptr(s), st));
+    CALL(gnn_edge_dot(g, ptr(Xj), ptr(Xi), H, C, dt, (float*)ptr(s), st));
     return wrap(first(s, g->E));
 }
 
@@ -543,15 +552,16 @@ FN(edge_dot) {
 FN(edge_dot_backward) {
     const gnn_csr* g = A.g(0);
     const at::Tensor &Xj = A.dev(1), &Xi = A.dev(2);
-    const int H = (int)A.i(4), F = (int)Xj.size(1);
+    int C;
+    const int H = A.heads(4, Xj.size(1), &C);
     at::Tensor dXj, dXi;
     if (A.flag(5)) dXj = empty_like(Xj);
     if (A.flag(6)) dXi = empty_like(Xi);
-    Scratch ws(A.t(7), gnn_edge_dot_backward_workspace(g->E, H, F / H), Xj.device());
+    Scratch ws(A.t(7), gnn_edge_dot_backward_workspace(g->E, H, C), Xj.device());
     const float* ds = f32(A.t(3), "ds_csr");
     const gnn_dtype dt = dtype_of(Xj);
     const gnn_stream st = stream();
-    CALL(gnn_edge_dot_backward(g, ptr(Xj), ptr(Xi), ds, H, F / H, dt, ptr(dXj), ptr(dXi), ws.p, ws.n, st));
+    CALL(gnn_edge_dot_backward(g, ptr(Xj), ptr(Xi), ds, H, C, dt, ptr(dXj), ptr(dXi), ws.p, ws.n, st));
     return wrap_all(dXj, dXi);
 }
 
@@ -560,12 +570,13 @@ FN(gatv2_logits) {
     const gnn_csr* g = A.g(0);
     const at::Tensor &Xl = A.dev(1), &Xr = A.dev(2);
     const float* a = f32(A.t(3), "a");
-    const int H = (int)A.i(4), F = (int)Xl.size(1);
+    int C;
+    const int H = A.heads(4, Xl.size(1), &C);
     const float slope = A.f(5);
     at::Tensor s = empty({at_least_one(g->E), H}, at::kFloat, Xl.device());
     const gnn_dtype dt = dtype_of(Xl);
     const gnn_stream st = stream();
-    CALL(gnn_gatv2_logits(g, ptr(Xl), ptr(Xr), a, H, F / H, dt, slope, (float*)ptr(s), st));
+    CALL(gnn_gatv2_logits(g, ptr(Xl), ptr(Xr), a, H, C, dt, slope, (float*)ptr(s), st));
     return wrap(first(s, g->E));
 }
 
@@ -574,13 +585,14 @@ FN(gatv2_logits_backward) {
     const gnn_csr* g = A.g(0);
     const at::Tensor &Xl = A.dev(1), &Xr = A.dev(2);
     const float *a = f32(A.t(3), "a"), *ds = f32(A.t(4), "ds_csr");
-    const int H = (int)A.i(5), F = (int)Xl.size(1), N = (int)Xl.size(0);
+    int C;
+    const int H = A.heads(5, Xl.size(1), &C), N = (int)Xl.size(0);
     const float slope = A.f(6);
-    at::Tensor dXl = empty_like(Xl), dXr = empty_like(Xr), da = empty({H, F / H}, at::kFloat, Xl.device());
-    Scratch ws(A.t(7), gnn_gatv2_logits_backward_workspace(N, H, F / H), Xl.device());
+    at::Tensor dXl = empty_like(Xl), dXr = empty_like(Xr), da = empty({H, C}, at::kFloat, Xl.device());
+    Scratch ws(A.t(7), gnn_gatv2_logits_backward_workspace(N, H, C), Xl.device());
     const gnn_dtype dt = dtype_of(Xl);
     const gnn_stream st = stream();
-    CALL(gnn_gatv2_logits_backward(g, ptr(Xl), ptr(Xr), a, ds, H, F / H, dt, slope, ptr(dXl), ptr(dXr), (float*)ptr(da), ws.p, ws.n, st));
+    CALL(gnn_gatv2_logits_backward(g, ptr(Xl), ptr(Xr), a, ds, H, C, dt, slope, ptr(dXl), ptr(dXr), (float*)ptr(da), ws.p, ws.n, st));
     return wrap_all(dXl, dXr, da);
 }
 
@@ -730,17 +742,18 @@ FN(reduce_nodes_backward) {
 FN(gat_fused) {
     const gnn_csr* g = A.g(0);
     const at::Tensor& Wx = A.dev(1);
-    const int64_t N = Wx.size(0), F = Wx.size(1), H = A.i(4);
-    const int C = (int)(F / H);
+    const int64_t N = Wx.size(0);
+    int C;
+    const int H = A.heads(4, Wx.size(1), &C);
     const float slope = A.f(5);
     const auto dev = Wx.device();
     at::Tensor out = empty_like(Wx), alpha = empty({at_least_one(g->E), H}, at::kFloat, dev), al = empty({N, H}, at::kFloat, dev),
                ar = empty({N, H}, at::kFloat, dev);
-    Scratch ws(A.t(6), gnn_gat_fused_workspace((int32_t)N, g->E, (int)H, C, 0), dev);
+    Scratch ws(A.t(6), gnn_gat_fused_workspace((int32_t)N, g->E, H, C, 0), dev);
     const float *as = (const float*)ptr(A.t(2)), *ad = (const float*)ptr(A.t(3));
     const gnn_dtype dt = dtype_of(Wx);
     const gnn_stream st = stream();
-    CALL(gnn_gat_fused(g, ptr(Wx), as, ad, (int)H, C, dt, slope, ptr(out), (float*)ptr(alpha), (float*)ptr(al), (float*)ptr(ar), ws.p, ws.n, st));
+    CALL(gnn_gat_fused(g, ptr(Wx), as, ad, H, C, dt, slope, ptr(out), (float*)ptr(alpha), (float*)ptr(al), (float*)ptr(ar), ws.p, ws.n, st));
     return wrap_all(out, first(alpha, g->E), al, ar);
 }
 
@@ -748,17 +761,18 @@ FN(gat_fused) {
 FN(gat_fused_backward) {
     const gnn_csr* g = A.g(0);
     const at::Tensor &Wx = A.dev(1), &dO = A.dev(7);
-    const int64_t N = Wx.size(0), F = Wx.size(1), H = A.i(8);
-    const int C = (int)(F / H);
+    const int64_t N = Wx.size(0);
+    int C;
+    const int H = A.heads(8, Wx.size(1), &C);
     const float slope = A.f(9);
     const auto dev = Wx.device();
     at::Tensor dWx = empty_like(Wx), das = empty({H, C}, at::kFloat, dev), dad = empty({H, C}, at::kFloat, dev);
-    Scratch ws(A.t(10), gnn_gat_fused_workspace((int32_t)N, g->E, (int)H, C, 1), dev);
+    Scratch ws(A.t(10), gnn_gat_fused_workspace((int32_t)N, g->E, H, C, 1), dev);
     const float *as = (const float*)ptr(A.t(2)), *ad = (const float*)ptr(A.t(3)), *alpha = (const float*)ptr(A.t(4)), *al = (const float*)ptr(A.t(5)),
                 *ar = (const float*)ptr(A.t(6));
     const gnn_dtype dt = dtype_of(Wx);
     const gnn_stream st = stream();
-    CALL(gnn_gat_fused_backward(g, ptr(Wx), as, ad, alpha, al, ar, ptr(dO), (int)H, C, dt, slope, ptr(dWx), (float*)ptr(das), (float*)ptr(dad), ws.p, ws.n, st));
+    CALL(gnn_gat_fused_backward(g, ptr(Wx), as, ad, alpha, al, ar, ptr(dO), H, C, dt, slope, ptr(dWx), (float*)ptr(das), (float*)ptr(dad), ws.p, ws.n, st));
     return wrap_all(dWx, das, dad);
 }
 

@@ -1,0 +1,37 @@
+"""What the compiled binding does with arguments before the library sees them: errors are Python errors."""
+import numpy as np
+import pytest
+
+from util import to_dev
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def gnn():
+    from paper_2412_06354_b200 import gnn as g
+    g.load()
+    return g
+
+
+@pytest.fixture(scope="module")
+def small(gnn):
+    """A graph of 6 nodes and 7 edges and features of 16 fp32 columns."""
+    import torch
+    src, dst = (to_dev(np.array(a, np.int32)) for a in ([0, 1, 2, 3, 4, 5, 0], [1, 2, 3, 4, 5, 0, 3]))
+    return gnn.coo_to_csr(6, src, dst), torch.randn((6, 16), device="cuda")
+
+
+def test_zero_heads_are_an_error_and_not_the_end_of_the_process(gnn, small):
+    import torch
+    g, X = small
+    a, s = torch.zeros((4, 4), device="cuda"), torch.zeros((g.E, 4), device="cuda")
+    fwd = gnn.gat_fused(g, X, a, a, 4)
+    for call in (lambda H: gnn.edge_dot(g, X, X, H), lambda H: gnn.edge_dot_backward(g, X, X, s, H), lambda H: gnn.gatv2_logits(g, X, X, a, H),
+                 lambda H: gnn.gatv2_logits_backward(g, X, X, a, s, H), lambda H: gnn.gat_fused(g, X, a, a, H),
+                 lambda H: gnn.gat_fused_backward(g, X, a, a, fwd, X, H)):
+        with pytest.raises(ZeroDivisionError):
+            call(0)
+        with pytest.raises((RuntimeError, ValueError)):  # (GnnError is a RuntimeError)
+            call(-1)
+        call(4)
