@@ -82,6 +82,11 @@ struct Args {
         if (!THPVariable_Check(o)) raise(PyExc_TypeError, std::string("expected a tensor or None, got ") + Py_TYPE(o)->tp_name);
         return THPVariable_Unpack(o);
     }
+    // a tensor that the call cannot do without
+    const at::Tensor& must(int i) const {
+        if (none(i)) raise(PyExc_AttributeError, "a tensor is needed, got None");
+        return t(i);
+    }
     // a contiguous tensor on the device
     const at::Tensor& dev(int i) const {
         const at::Tensor& x = t(i);
@@ -271,7 +276,7 @@ FN(degree) {
 // (N, src, dst) -> (src, dst)
 FN(add_self_loops) {
     const int64_t N = A.i(0);
-    const at::Tensor &src = A.t(1), &dst = A.t(2);
+    const at::Tensor &src = A.must(1), &dst = A.t(2);
     const int64_t E = src.numel();
     at::Tensor so = empty({E + N}, at::kInt, src.device()), d_o = empty({E + N}, at::kInt, src.device());
     const int32_t *s = i32(src, "src"), *d = i32(dst, "dst");
@@ -294,7 +299,7 @@ FN(gcn_norm) {
 
 // (perm, x, out)
 FN(permute_edge_data) {
-    const at::Tensor &perm = A.t(0), &x = A.dev(1);
+    const at::Tensor &perm = A.must(0), &x = A.dev(1);
     at::Tensor out = A.t(2);
     const int64_t E = perm.numel(), width = E ? x.numel() / E : 1;
     if (!out.defined()) out = empty_like(x);
@@ -312,7 +317,7 @@ FN(segment_coef) {
     if (A.flag(4)) coefT = empty({at_least_one(g->E)}, at::kFloat, dev);
     const int32_t *seg = i32(A.t(1), "seg_csr"), *mean = i32(A.t(2), "seg_is_mean");
     const float* w = f32(A.t(3), "w_csr");
-    const int S = (int)A.t(2).numel();
+    const int S = (int)A.must(2).numel();
     const gnn_stream st = stream();
     CALL(gnn_segment_coef(g, seg, w, mean, S, (float*)ptr(coef), (float*)ptr(coefT), st));
     return wrap_all(first(coef, g->E), first(coefT, g->E));
@@ -332,7 +337,7 @@ FN(merge_edge_lists) {
             if (!item) { python_error e; e.persist(); throw e; }
             const Args B{PySequence_Fast_ITEMS(item), PySequence_Fast_GET_SIZE(item)};
             try {
-                const at::Tensor &src = B.t(0), &dst = B.t(1);
+                const at::Tensor &src = B.must(0), &dst = B.must(1);
                 segs[(size_t)k] = gnn_edge_segment{src.numel(), src.numel() ? i32(src, "src") : nullptr, dst.numel() ? i32(dst, "dst") : nullptr,
                                                    (int32_t)B.i(2), (int32_t)B.i(3)};
                 if (k == 0) dev = src.device();
@@ -352,7 +357,7 @@ FN(merge_edge_lists) {
 
 // (graph_id, G) -> graph_ptr
 FN(graph_ptr_from_ids) {
-    const at::Tensor& id = A.t(0);
+    const at::Tensor& id = A.must(0);
     const int64_t G = A.i(1);
     at::Tensor out = empty({G + 1}, at::kLong, id.device());
     Scratch ws(at::Tensor(), 256, id.device());
@@ -599,7 +604,7 @@ FN(gatv2_logits_backward) {
 // ---------------------------------------------------------------- unfused primitives
 // (idx, X, out)
 FN(gather) {
-    const at::Tensor &idx = A.t(0), &X = A.dev(1);
+    const at::Tensor &idx = A.must(0), &X = A.dev(1);
     at::Tensor out = A.t(2);
     const int64_t E = idx.numel(), F = X.size(1);
     if (!out.defined()) out = empty({E, F}, X.scalar_type(), X.device());
@@ -710,7 +715,7 @@ FN(axpby) {
 // ---------------------------------------------------------------- pooling
 // (graph_ptr, X, op, ws) -> out or (out, argmax)
 FN(reduce_nodes) {
-    const at::Tensor &gp = A.t(0), &X = A.dev(1);
+    const at::Tensor &gp = A.must(0), &X = A.dev(1);
     const gnn_op op = A.op(2);
     const int64_t G = gp.numel() - 1, N = X.size(0), F = X.size(1);
     at::Tensor out = empty({G, F}, X.scalar_type(), X.device()), arg;
@@ -803,7 +808,7 @@ FN(linear) {
 // (X, W, dY, want_dX, want_dW, ws, return_ws) -> (dX, dW) or (dX, dW, ws)
 FN(linear_backward) {
     const at::Tensor &X = A.t(0), &W = A.t(1), &dY = A.dev(2);
-    const int64_t N = dY.size(0), M = dY.size(1), K = W.defined() ? W.size(0) : X.size(1);
+    const int64_t N = dY.size(0), M = dY.size(1), K = W.defined() ? W.size(0) : A.must(0).size(1);
     const bool wanted = A.flag(6);
     at::Tensor dX, dW;
     if (A.flag(3)) dX = empty({N, K}, dY.scalar_type(), dY.device());

@@ -35,3 +35,15 @@ def test_zero_heads_are_an_error_and_not_the_end_of_the_process(gnn, small):
         with pytest.raises((RuntimeError, ValueError)):  # (GnnError is a RuntimeError)
             call(-1)
         call(4)
+
+
+def test_none_is_not_an_empty_index(gnn, small):
+    import torch
+    g, X = small
+    i = torch.zeros(3, dtype=torch.int32, device="cuda")
+    for call in (lambda: gnn.gather(None, X), lambda: gnn.permute_edge_data(None, X), lambda: gnn.add_self_loops(3, None, i),
+                 lambda: gnn.merge_edge_lists([(i, None, 0, 0)]), lambda: gnn.merge_edge_lists([(None, i, 0, 0)]),
+                 lambda: gnn.graph_ptr_from_ids(None, 2), lambda: gnn.reduce_nodes(None, X), lambda: gnn.segment_coef(g, i, None),
+                 lambda: gnn.linear_backward(None, None, X)):
+        with pytest.raises(AttributeError):
+            call()
