@@ -18,6 +18,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/DynamicTypes.h>
 #include <torch/csrc/autograd/python_variable.h>
+#include <torch/csrc/utils/object_ptr.h>
 
 #include "gnn.h"
 
@@ -29,11 +30,37 @@ PyObject* g_s_torch = nullptr;
 PyObject* g_s_empty = nullptr;
 PyObject* g_error = nullptr;
 
-[[noreturn]] void raise(PyObject* type, const std::string& text) {
-    PyErr_SetString(type, text.c_str());
+// the Python error that is set, as an exception
+[[noreturn]] void rethrow() {
     python_error e;
     e.persist();
     throw e;
+}
+
+[[noreturn]] void raise(PyObject* type, const std::string& text) {
+    PyErr_SetString(type, text.c_str());
+    rethrow();
+}
+
+// int(o), float(o) and bool(o)
+int64_t as_int(PyObject* o) {
+    PyObject* n = PyNumber_Long(o);
+    const int64_t v = n ? PyLong_AsLongLong(n) : -1;
+    Py_XDECREF(n);
+    if (v == -1 && PyErr_Occurred()) rethrow();
+    return v;
+}
+double as_float(PyObject* o) {
+    PyObject* n = PyNumber_Float(o);
+    const double v = n ? PyFloat_AS_DOUBLE(n) : -1.0;
+    Py_XDECREF(n);
+    if (!n) rethrow();
+    return v;
+}
+bool as_bool(PyObject* o) {
+    const int v = PyObject_IsTrue(o);
+    if (v < 0) rethrow();
+    return v == 1;
 }
 
 // status of a C-ABI call -> GnnError(status, text)
@@ -48,9 +75,7 @@ void check(gnn_status rc) {
             Py_DECREF(exc);
         }
     }
-    python_error e;
-    e.persist();
-    throw e;
+    rethrow();
 }
 
 // a launch can block (a full queue, a synchronising call): other Python threads keep running meanwhile
@@ -95,23 +120,11 @@ struct Args {
     }
     int64_t i(int k) const {
         const int64_t v = PyLong_AsLongLong(at(k));
-        if (v == -1 && PyErr_Occurred()) {
-            python_error e;
-            e.persist();
-            throw e;
-        }
+        if (v == -1 && PyErr_Occurred()) rethrow();
         return v;
     }
-    bool flag(int k) const { return PyObject_IsTrue(at(k)) == 1; }
-    float f(int k) const {
-        const double v = PyFloat_AsDouble(at(k));
-        if (v == -1.0 && PyErr_Occurred()) {
-            python_error e;
-            e.persist();
-            throw e;
-        }
-        return (float)v;
-    }
+    bool flag(int k) const { return as_bool(at(k)); }
+    float f(int k) const { return (float)as_float(at(k)); }
     gnn_op op(int k) const {
         PyObject* o = at(k);
         if (PyUnicode_Check(o)) {
@@ -119,11 +132,9 @@ struct Args {
             for (int q = 0; q < 4; ++q)
                 if (PyUnicode_CompareWithASCIIString(o, names[q]) == 0) return (gnn_op)q;
             PyErr_SetObject(PyExc_KeyError, o);
-            python_error e;
-            e.persist();
-            throw e;
+            rethrow();
         }
-        return (gnn_op)i(k);
+        return (gnn_op)as_int(o);
     }
     // heads of a row of F features: their number, and the features of one
     int heads(int k, int64_t F, int* C) const {
@@ -178,9 +189,7 @@ at::Tensor empty(at::IntArrayRef shape, at::ScalarType type, c10::Device device)
     if (!r || !THPVariable_Check(r)) {
         if (!PyErr_Occurred()) PyErr_SetString(PyExc_RuntimeError, "empty() gave no tensor");
         Py_XDECREF(r);
-        python_error e;
-        e.persist();
-        throw e;
+        rethrow();
     }
     at::Tensor t = THPVariable_Unpack(r);
     Py_DECREF(r);
@@ -267,7 +276,7 @@ FN(degree) {
     const gnn_csr* g = A.g(0);
     const at::Tensor& w = A.t(2);
     at::Tensor out = empty({g->N}, w.defined() ? at::kFloat : at::kInt, A.t(3).device());
-    const int tr = (int)A.i(1);
+    const int tr = (int)as_int(A.at(1));
     const gnn_stream st = stream();
     CALL(gnn_degree(g, tr, (const float*)ptr(w), ptr(out), st));
     return wrap(out);
@@ -326,7 +335,7 @@ FN(segment_coef) {
 // ([(src, dst, src_offset, dst_offset), ...]) -> (src, dst, seg)
 FN(merge_edge_lists) {
     PyObject* seq = PySequence_Fast(A.at(0), "segments must be a sequence");
-    if (!seq) throw python_error();
+    if (!seq) rethrow();
     const Py_ssize_t S = PySequence_Fast_GET_SIZE(seq);
     std::vector<gnn_edge_segment> segs((size_t)S);
     int64_t total = 0;
@@ -334,12 +343,13 @@ FN(merge_edge_lists) {
     try {
         for (Py_ssize_t k = 0; k < S; ++k) {
             PyObject* item = PySequence_Fast(PySequence_Fast_GET_ITEM(seq, k), "a segment is (src, dst, src_offset, dst_offset)");
-            if (!item) { python_error e; e.persist(); throw e; }
+            if (!item) rethrow();
             const Args B{PySequence_Fast_ITEMS(item), PySequence_Fast_GET_SIZE(item)};
             try {
+                if (B.n != 4) raise(PyExc_ValueError, "a segment is (src, dst, src_offset, dst_offset)");
                 const at::Tensor &src = B.must(0), &dst = B.must(1);
                 segs[(size_t)k] = gnn_edge_segment{src.numel(), src.numel() ? i32(src, "src") : nullptr, dst.numel() ? i32(dst, "dst") : nullptr,
-                                                   (int32_t)B.i(2), (int32_t)B.i(3)};
+                                                   (int32_t)as_int(B.at(2)), (int32_t)as_int(B.at(3))};
                 if (k == 0) dev = src.device();
                 total += src.numel();
             } catch (...) { Py_DECREF(item); throw; }
@@ -370,7 +380,7 @@ FN(graph_ptr_from_ids) {
 // ---------------------------------------------------------------- fused propagate
 static bool has_winners(gnn_op op) { return op == GNN_MAX || op == GNN_MIN; }
 
-// (g, X, w_csr, op, out, argmax, ws) -> out or (out, argmax); ws false: the call without a workspace argument
+// (g, X, w_csr, op, out, argmax, ws, built_in) -> out or (out, argmax); built_in: the call without a workspace argument
 FN(propagate_fused) {
     const gnn_csr* g = A.g(0);
     const at::Tensor& X = A.dev(1);
@@ -385,7 +395,7 @@ FN(propagate_fused) {
     int32_t* ap = i32(arg, "argmax");
     const gnn_dtype dt = dtype_of(X);
     const gnn_stream st = stream();
-    if (A.at(6) == Py_False) {
+    if (A.flag(7)) {
         CALL(gnn_propagate_fused_static(g, msg, op, ptr(X), wp, (int)F, dt, ptr(out), ap, st));
     } else {
         Scratch ws(A.t(6), gnn_propagate_fused_workspace(g->E, (int)F, op), X.device());
@@ -425,23 +435,35 @@ FN(propagate_fused_backward) {
 struct Epilogue {
     gnn_row_epilogue e{};
     const gnn_row_epilogue* p = nullptr;
+    THPObjectPtr held[5];  // the values stay alive for the call, whatever becomes of the mapping meanwhile
     Epilogue(const Args& A, int k) {
         PyObject* o = A.at(k);
         if (o == Py_None) return;
-        if (!PyDict_Check(o)) raise(PyExc_AttributeError, "an epilogue is a dict(Xself=, self_coef=, self_mode=, bias=, relu=)");
-        e.Xself = ptr(tensor(o, "Xself"));
-        PyObject* v = PyDict_GetItemString(o, "self_coef");
-        e.self_coef = v ? (float)PyFloat_AsDouble(v) : 0.f;
-        v = PyDict_GetItemString(o, "self_mode");
-        e.self_mode = v ? (int)PyLong_AsLong(v) : GNN_SELF_ALWAYS;
-        if (PyErr_Occurred()) { python_error err; err.persist(); throw err; }
-        e.bias = f32(tensor(o, "bias"), "bias");
-        v = PyDict_GetItemString(o, "relu");
-        e.relu = v && PyObject_IsTrue(v) == 1;
+        static const char* const names[5] = {"Xself", "self_coef", "self_mode", "bias", "relu"};
+        for (int q = 0; q < 5; ++q) held[q] = value(o, names[q]);
+        e.Xself = ptr(tensor(0, "Xself"));
+        e.self_coef = held[1].get() ? (float)as_float(held[1].get()) : 0.f;
+        e.self_mode = held[2].get() ? (int)as_int(held[2].get()) : GNN_SELF_ALWAYS;
+        e.bias = f32(tensor(3, "bias"), "bias");
+        e.relu = held[4].get() && as_bool(held[4].get());
         p = &e;
     }
-    static at::Tensor tensor(PyObject* o, const char* name) {
-        PyObject* v = PyDict_GetItemString(o, name);
+    // a new reference, or null if the mapping (a dict, or anything with a get) has no such key
+    static PyObject* value(PyObject* o, const char* name) {
+        if (PyDict_Check(o)) {
+            PyObject* v = PyDict_GetItemString(o, name);
+            Py_XINCREF(v);
+            return v;
+        }
+        static PyObject* const absent = PyList_New(0);
+        PyObject* v = PyObject_CallMethod(o, "get", "sO", name, absent);
+        if (!v) rethrow();
+        if (v != absent) return v;
+        Py_DECREF(v);
+        return nullptr;
+    }
+    at::Tensor tensor(int q, const char* name) {
+        PyObject* v = held[q].get();
         if (!v || v == Py_None) return at::Tensor();
         if (!THPVariable_Check(v)) raise(PyExc_TypeError, std::string(name) + " must be a tensor");
         return THPVariable_Unpack(v);
@@ -477,7 +499,7 @@ FN(propagate_msg_backward) {
     const at::Tensor& dO = A.dev(2);
     const gnn_op op = A.op(3);
     const at::Tensor &Xj = A.t(4), &ef = A.t(5), &arg = A.t(7);
-    const int given = (int)A.i(6), ew = given ? given : factor_width(ef);
+    const int ew = A.flag(6) ? (int)A.i(6) : factor_width(ef);
     const Epilogue sg(A, 8);
     const int64_t F = dO.size(1);
     const auto dev = dO.device();
@@ -619,7 +641,7 @@ FN(gather) {
 FN(gather_backward) {
     const gnn_csr* g = A.g(0);
     const at::Tensor& dO = A.dev(1);
-    const int by_src = A.flag(2);
+    const int by_src = (int)as_int(A.at(2));
     const int64_t F = dO.size(1);
     at::Tensor dX = empty({g->N, F}, dO.scalar_type(), dO.device());
     Scratch ws(A.t(3), gnn_propagate_fused_workspace(g->E, (int)F, GNN_SUM), dO.device());

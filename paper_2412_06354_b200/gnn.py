@@ -261,7 +261,7 @@ def propagate_fused_workspace(E, F, op="sum"):
 
 def propagate_fused(g: Graph, X, w_csr=None, op="sum", out=None, argmax=None, ws=None):
     """-> out, or (out, argmax) for max/min."""
-    return _b.propagate_fused(_addr(g.c), X, w_csr, op, out, argmax, ws)
+    return _b.propagate_fused(_addr(g.c), X, w_csr, op, out, argmax, ws, False)
 
 
 def propagate_fused_backward(g: Graph, dOut, op="sum", X=None, w_csrT=None, argmax=None, want_dX=True, want_dW=False,
@@ -405,7 +405,7 @@ def propagate_fused_static(g: Graph, X, w_csr=None, op="sum", out=None, argmax=N
     """gnn_propagate_fused_static: the fused propagate with the library's built-in 8 MiB scratch, for
     embedders that may not allocate device memory.  The caller passes `out` (and `argmax` for max/min);
     nothing is allocated here when they are given."""
-    return _b.propagate_fused(_addr(g.c), X, w_csr, op, out, argmax, False)
+    return _b.propagate_fused(_addr(g.c), X, w_csr, op, out, argmax, None, True)
 
 
 # ------------------------------------------------------------------ dense transform

@@ -47,3 +47,36 @@ def test_none_is_not_an_empty_index(gnn, small):
                  lambda: gnn.linear_backward(None, None, X)):
         with pytest.raises(AttributeError):
             call()
+
+
+def test_arguments_convert_as_python_would(gnn, small):
+    import types
+    import torch
+    g, X = small
+    i = torch.zeros(3, dtype=torch.int32, device="cuda")
+    assert torch.equal(gnn.degree(g, transposed=np.bool_(True)), gnn.degree(g, transposed=True))
+    assert torch.equal(gnn.propagate_fused(g, X, None, np.float64(gnn.MEAN)), gnn.propagate_fused(g, X, None, "mean"))
+    b = torch.ones(16, device="cuda")
+    want = gnn.propagate_msg(g, gnn.COPY_XJ, X, epi=dict(Xself=X, self_coef=0.5, bias=b, relu=True))
+    for epi in (types.MappingProxyType(dict(Xself=X, self_coef="0.5", bias=b, relu=1)), dict(Xself=X, self_coef=torch.tensor(0.5), self_mode=np.float32(0), bias=b, relu=np.True_)):
+        assert torch.equal(gnn.propagate_msg(g, gnn.COPY_XJ, X, epi=epi), want)
+    assert torch.equal(gnn.propagate_msg(g, gnn.COPY_XJ, X, epi={}), gnn.propagate_fused(g, X))
+    w = torch.ones(g.E, device="cuda")
+    assert gnn.propagate_msg_backward(g, gnn.E_MUL_XJ, X, Xj=X, e_csrT=w, e_width=None, want_de=True)["de"].shape == (g.E, 1)
+    assert len(gnn.merge_edge_lists([[i, i, np.float64(0), 0]])) == 3
+
+
+def test_arguments_that_python_would_refuse(gnn, small):
+    import torch
+    g, X = small
+    i = torch.zeros(3, dtype=torch.int32, device="cuda")
+    two = torch.zeros(2, device="cuda")
+    for error, call in ((ValueError, lambda: gnn.merge_edge_lists([(i, i, 0, 0, 0)])), ((TypeError, ValueError), lambda: gnn.merge_edge_lists([(i, i, 0)])),
+                        (RuntimeError, lambda: gnn.linear_bias_act(X, torch.ones((16, 8), device="cuda"), relu=two)),
+                        (TypeError, lambda: gnn.propagate_msg(g, gnn.COPY_XJ, X, epi=dict(self_coef=None))),
+                        ((AttributeError, TypeError), lambda: gnn.propagate_fused(g, X, ws=False)), (KeyError, lambda: gnn.propagate_fused(g, X, None, "sums")),
+                        (TypeError, lambda: gnn.degree(g, transposed=None)), (TypeError, lambda: gnn.gather(i.long(), X)),
+                        (TypeError, lambda: gnn.propagate_fused(g, X, torch.ones(g.E, dtype=torch.float64, device="cuda"))),
+                        (AssertionError, lambda: gnn.propagate_fused(g, X.t()))):
+        with pytest.raises(error):
+            call()
