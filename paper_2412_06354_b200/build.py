@@ -48,7 +48,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
                 if r.returncode != 0:
                     raise RuntimeError("nvcc failed: " + " ".join(r.args))
     if jobs or not os.path.exists(LIB):
-        subprocess.check_call([NVCC, "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-o", LIB, *objs])
+        subprocess.check_call([NVCC, "-gencode", "arch=compute_100a,code=sm_100a", "-shared", "-Xlinker=-soname,libgnn_b200.so", "-o", LIB, *objs])
     build_binding(force)
     from . import synth
     synth.build(force)

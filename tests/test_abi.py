@@ -57,3 +57,16 @@ def test_binding_rejects_wrong_index_dtype():
         gnn._pf32(torch.zeros(3, dtype=torch.float64), "w_csr")
     assert gnn._pi(None, torch.int32, "argmax") is None
     assert gnn._pi(torch.zeros(3, dtype=torch.int32), torch.int32, "src") is not None
+
+
+def test_a_library_loaded_from_elsewhere_serves_the_compiled_calls_too(tmp_path):
+    """load(path) takes the library that the extension is linked against by name: one copy in the process, the one asked for."""
+    import shutil
+    import subprocess
+    import sys
+    other = tmp_path / "libgnn_b200.so"
+    shutil.copy(gnn.LIB_PATH, other)
+    code = ("import sys; sys.path.insert(0, %r)\nfrom paper_2412_06354_b200 import gnn\ngnn.load(%r)\n"
+            "print({l.split()[-1] for l in open('/proc/self/maps') if 'libgnn_b200' in l})" % (ROOT, str(other)))
+    out = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, check=True).stdout
+    assert out.strip() == str({str(other)})
