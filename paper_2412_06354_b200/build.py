@@ -22,6 +22,7 @@ FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-lineinfo", "-std
 
 
 BINDING = os.path.join(HERE, "_binding.so")
+BINDING_KEY = os.path.join(OBJ, "binding.key")  # what the extension was built against
 
 
 def _newest(paths):
@@ -57,11 +58,14 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 def build_binding(force: bool = False) -> str:
     """The CPython extension (host code only) that gnn.py calls; linked against libgnn_b200.so beside it and torch."""
-    src = os.path.join(CSRC, "binding.cpp")
-    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= _newest([src, os.path.join(ROOT, "include", "gnn.h")]):
-        return BINDING
     import sysconfig
     import torch
+    src = os.path.join(CSRC, "binding.cpp")
+    # the extension uses torch's C++ interface, which another version or Python need not share
+    key = " ".join(map(str, (torch.__version__, int(torch._C._GLIBCXX_USE_CXX11_ABI), sysconfig.get_config_var("SOABI"))))
+    built = open(BINDING_KEY).read() if os.path.exists(BINDING_KEY) else None
+    if not force and built == key and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= _newest([src, os.path.join(ROOT, "include", "gnn.h")]):
+        return BINDING
     tdir = os.path.dirname(torch.__file__)
     inc = [os.path.join(ROOT, "include"), os.path.join(tdir, "include"), os.path.join(tdir, "include", "torch", "csrc", "api", "include"),
            sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(NVCC)), "include")]
@@ -69,6 +73,9 @@ def build_binding(force: bool = False) -> str:
                            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", src, "-o", BINDING,
                            "-L" + HERE, "-l:libgnn_b200.so", "-Wl,-rpath,$ORIGIN", "-L" + os.path.join(tdir, "lib"),
                            "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python"])
+    os.makedirs(OBJ, exist_ok=True)
+    with open(BINDING_KEY, "w") as f:
+        f.write(key)
     return BINDING
 
 

@@ -70,3 +70,20 @@ def test_a_library_loaded_from_elsewhere_serves_the_compiled_calls_too(tmp_path)
             "print({l.split()[-1] for l in open('/proc/self/maps') if 'libgnn_b200' in l})" % (ROOT, str(other)))
     out = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, check=True).stdout
     assert out.strip() == str({str(other)})
+
+
+def test_extension_is_rebuilt_for_another_torch(monkeypatch, tmp_path):
+    import torch
+    build.build_binding()
+    compiled = []
+    monkeypatch.setattr(build.subprocess, "check_call", lambda cmd, **kw: compiled.append(cmd))
+    build.build_binding()
+    assert not compiled
+    stamp = tmp_path / "binding.key"
+    stamp.write_text(open(build.BINDING_KEY).read())
+    monkeypatch.setattr(build, "BINDING_KEY", str(stamp))
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    build.build_binding()
+    assert len(compiled) == 1
+    build.build_binding()
+    assert len(compiled) == 1  # and then it is up to date
