@@ -47,9 +47,14 @@ static inline int grid_for(int64_t n, int threads) {
 
 #ifdef __CUDACC__
 // ---------------------------------------------------------------- launches
-// Launch whose blocks may be set up while the kernel before it in the stream drains.  The kernel's first statement is
-// pdl_wait(): nothing of it touches global memory before all earlier work of the stream is complete and visible, so the
-// order of the stream is kept; what overlaps is the launch latency (about 1 us of a 3-5 us kernel on a small graph).
+// Launch whose blocks may be set up while the kernel before it in the stream drains (and, as every kernel lets its successor
+// come up before it waits itself, while the one before that does).  The kernel's first statement is pdl_wait(): nothing of it
+// touches global memory before all earlier work of the stream is complete and visible, so the order of the stream is kept;
+// what overlaps is the launch latency (about 1 us of a 3-5 us kernel on a small graph).
+// What griddepcontrol.wait makes visible are ordinary (coherent) loads.  Such a kernel is resident while what it reads is being
+// written, so that the condition of the non-coherent path, data that is read-only as long as the kernel lives, does not hold:
+// no ld.global.nc and no __ldg in it, and no __restrict__ on a pointer to const, from which the compiler would make them.
+// (Outputs may be __restrict__: then loads can move ahead of stores.)  tests/test_overlapped_launches.py looks at the sources.
 template <class... Params, class... Args>
 static inline void launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
     cudaLaunchConfig_t cfg = {};
@@ -90,24 +95,39 @@ __device__ __forceinline__ uint64_t policy_evict_first() {
 }
 __device__ __forceinline__ uint4 ld_hint16(const void* p, uint64_t pol) {
     uint4 v;
-    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v4.u32 {%0,%1,%2,%3}, [%4], %5;"
                  : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
                  : "l"(p), "l"(pol));
     return v;
 }
 __device__ __forceinline__ int ld_hint_i32(const int* p, uint64_t pol) {
     int v;
-    asm volatile("ld.global.nc.L1::no_allocate.L2::cache_hint.s32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.s32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));
     return v;
 }
 __device__ __forceinline__ int ld_stream_i32(const int* p) {
     int v;
-    asm volatile("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(v) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.s32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
 __device__ __forceinline__ float ld_stream_f32(const float* p) {
     float v;
-    asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    asm volatile("ld.global.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+// coherent loads whose place among the other loads and stores in flight is kept
+__device__ __forceinline__ uint4 ld_16(const void* p) {
+    uint4 v;
+    asm volatile("ld.global.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ int4 ld_int4(const int4* p) {
+    const uint4 v = ld_16(p);
+    return make_int4((int)v.x, (int)v.y, (int)v.z, (int)v.w);
+}
+__device__ __forceinline__ float ld_f32(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
     return v;
 }
 __device__ __forceinline__ void st_stream16(void* p, uint4 v) {

@@ -406,7 +406,7 @@ struct CudaSlots {
 static FlagSlots<CudaSlots> g_slots;
 
 // ------------------------------------------------------------------ degrees / GCN coefficients
-__global__ void degree_count_kernel(int32_t N, const int64_t* __restrict__ rowptr,
+__global__ void degree_count_kernel(int32_t N, const int64_t* rowptr,
                                     int32_t* __restrict__ deg) {
     pdl_wait();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -417,8 +417,8 @@ __global__ void degree_count_kernel(int32_t N, const int64_t* __restrict__ rowpt
 // of 10^5 positions walked by a warp alone takes milliseconds).  Fixed orders.  170k rows of nine positions on average:
 // 31 us with a warp per row, 14 us.
 constexpr int DEG_LONG = 512;
-__global__ void __launch_bounds__(256) degree_weighted_kernel(int32_t N, const int64_t* __restrict__ rowptr,
-                                                             const float* __restrict__ w, float* __restrict__ deg) {
+__global__ void __launch_bounds__(256) degree_weighted_kernel(int32_t N, const int64_t* rowptr,
+                                                             const float* w, float* __restrict__ deg) {
     __shared__ int todo[32], ntodo;
     __shared__ float sums[8];
     pdl_wait();
@@ -461,7 +461,7 @@ __global__ void __launch_bounds__(256) degree_weighted_kernel(int32_t N, const i
     }
 }
 
-__global__ void degree_unit_kernel(int32_t N, const int64_t* __restrict__ rowptr,
+__global__ void degree_unit_kernel(int32_t N, const int64_t* rowptr,
                                    float* __restrict__ deg) {
     pdl_wait();
     int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -549,8 +549,8 @@ __global__ void __launch_bounds__(256) gcn_coef_kernel(const __grid_constant__ C
 }
 
 template <typename T>
-__global__ void permute_rows_kernel(int64_t E, int width, const int32_t* __restrict__ perm,
-                                    const T* __restrict__ in, T* __restrict__ out) {
+__global__ void permute_rows_kernel(int64_t E, int width, const int32_t* perm,
+                                    const T* in, T* __restrict__ out) {
     pdl_wait();
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -562,8 +562,8 @@ __global__ void permute_rows_kernel(int64_t E, int width, const int32_t* __restr
     }
 }
 
-__global__ void add_self_loops_kernel(int32_t N, int64_t E, const int32_t* __restrict__ src,
-                                      const int32_t* __restrict__ dst, int32_t* __restrict__ so,
+__global__ void add_self_loops_kernel(int32_t N, int64_t E, const int32_t* src,
+                                      const int32_t* dst, int32_t* __restrict__ so,
                                       int32_t* __restrict__ dout) {
     pdl_wait();
     int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;

@@ -97,7 +97,7 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
         }
         q = lo;
     }
-    auto own = [&](int qq) { return __ldg(reinterpret_cast<const uint4*>(Dl + (size_t)(uint32_t)max(S.row[qq], 0) * row_bytes)); };
+    auto own = [&](int qq) { return ld_16(Dl + (size_t)(uint32_t)max(S.row[qq], 0) * row_bytes); };
     float d[EPC], sc = 1.0f;
     uint4 own_next = make_uint4(0u, 0u, 0u, 0u);
     if (a < b) {

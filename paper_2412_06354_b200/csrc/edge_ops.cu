@@ -15,7 +15,7 @@ __device__ __forceinline__ int row_of_position(const int64_t* rowptr, int N, int
 // so from one step to the next a thread's position moves on by blockDim / chunks-per-position and its row by a step or
 // two.  A full search per 16-byte chunk made the calls below run at a sixth of the memory rate; now there is one full
 // search per thread, and another only where more than eight rows (a run of empty ones) are skipped at once.
-__device__ __forceinline__ int advance_row(const int64_t* __restrict__ rowptr, int N, int row, int64_t p) {
+__device__ __forceinline__ int advance_row(const int64_t* rowptr, int N, int row, int64_t p) {
     if (row < 0) return row_of_position(rowptr, N, p);
 #pragma unroll 1
     for (int k = 0; k < 8; ++k) {
@@ -59,7 +59,7 @@ struct PairTile {
 static dim3 pair_grid(int64_t total) { return dim3((unsigned)ceil_div(total, (int64_t)EO_U * 256)); }
 
 // out[k, chunk] = X[idx[k], chunk]
-__global__ void __launch_bounds__(256) gather_rows_kernel(const int32_t* __restrict__ idx, int64_t E, const uint4* __restrict__ X,
+__global__ void __launch_bounds__(256) gather_rows_kernel(const int32_t* idx, int64_t E, const uint4* X,
                                                           int nvec, uint32_t magic, uint4* __restrict__ out) {
     pdl_wait();
     const PairTile tile(E * nvec, nvec, magic);
@@ -85,8 +85,8 @@ __global__ void __launch_bounds__(256) gather_rows_kernel(const int32_t* __restr
 
 // m[p, f] = e[p, g(f)] * X[col[p], f]   (e == nullptr: plain copy of the source row)
 template <typename T>
-__global__ void __launch_bounds__(256) apply_edges_mul_kernel(const int32_t* __restrict__ col, int64_t E, const uint4* __restrict__ X,
-                                                              int nvec, uint32_t magic, const float* __restrict__ e, int ew, int feats_per_e,
+__global__ void __launch_bounds__(256) apply_edges_mul_kernel(const int32_t* col, int64_t E, const uint4* X,
+                                                              int nvec, uint32_t magic, const float* e, int ew, int feats_per_e,
                                                               uint4* __restrict__ m) {
     pdl_wait();
     constexpr int EPC = Chunk<T>::N;
@@ -126,8 +126,8 @@ __global__ void __launch_bounds__(256) apply_edges_mul_kernel(const int32_t* __r
 }
 
 // s[p, h] = LeakyReLU_slope(al[col[p], h] + ar[row(p), h]), fp32
-__global__ void gat_logit_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int N,
-                                 int64_t E, int H, const float* __restrict__ al, const float* __restrict__ ar,
+__global__ void gat_logit_kernel(const int64_t* rowptr, const int32_t* col, int N,
+                                 int64_t E, int H, const float* al, const float* ar,
                                  float slope, float* __restrict__ s) {
     pdl_wait();
     int64_t t0, t1;
@@ -149,8 +149,8 @@ __global__ void gat_logit_kernel(const int64_t* __restrict__ rowptr, const int32
 // winners per position and chunk (the L1 path was busy 77 % of the time), 86 us now; writing them takes 54 us.
 constexpr int AB_SUB = 128;  // most positions per warp
 template <typename T>
-__global__ void __launch_bounds__(256) aggregate_backward_kernel(const int64_t* __restrict__ rowptr, int N, int64_t E, int op, int sub, int lpr, bool wide,
-                                                                 const uint4* __restrict__ dOut, const int32_t* __restrict__ argmax,
+__global__ void __launch_bounds__(256) aggregate_backward_kernel(const int64_t* rowptr, int N, int64_t E, int op, int sub, int lpr, bool wide,
+                                                                 const uint4* dOut, const int32_t* argmax,
                                                                  int nvec, uint4* __restrict__ dm) {
     constexpr int EPC = Chunk<T>::N;
     __shared__ int s_rows[8][AB_SUB + 1];
@@ -184,13 +184,13 @@ __global__ void __launch_bounds__(256) aggregate_backward_kernel(const int64_t* 
                 return;
             }
             const size_t from = (size_t)row[q] * nvec + ci;
-            R.v = __ldg(dOut + from);
+            R.v = ld_16(dOut + from);
             if (op == GNN_MEAN) R.deg = (float)(rowptr[row[q] + 1] - rowptr[row[q]]);
             if (route) {
 #pragma unroll
                 for (int j = 0; j < EPC / 4; ++j) {
                     const int32_t* w = argmax + from * EPC + 4 * j;  // wide: 16-byte aligned
-                    if (wide) R.win[j] = __ldg(reinterpret_cast<const uint4*>(w));
+                    if (wide) R.win[j] = ld_16(w);
                     else R.win[j] = make_uint4(w[0], w[1], w[2], w[3]);
                 }
             }
@@ -253,7 +253,7 @@ static gnn_status check_rows(const char* who, int F, gnn_dtype dtype, int* nvec)
 }
 
 // graph_ptr[g] = first node whose graph id is >= g; flag set if ids are unsorted or out of range
-__global__ void graph_ptr_kernel(const int32_t* __restrict__ gid, int32_t N, int32_t G,
+__global__ void graph_ptr_kernel(const int32_t* gid, int32_t N, int32_t G,
                                  int64_t* __restrict__ gptr, int* __restrict__ flag) {
     pdl_wait();
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -274,7 +274,7 @@ __global__ void graph_ptr_kernel(const int32_t* __restrict__ gid, int32_t N, int
 
 // out = alpha*a + beta*b, element-wise in fp32 (self terms of layers: W1*x_i + W2*agg, (1+eps)*x_i + sum)
 template <typename T>
-__global__ void axpby_kernel(float alpha, const uint4* __restrict__ a, float beta, const uint4* __restrict__ b,
+__global__ void axpby_kernel(float alpha, const uint4* a, float beta, const uint4* b,
                              int64_t nvec, uint4* __restrict__ out) {
     pdl_wait();
     constexpr int EPC = Chunk<T>::N;

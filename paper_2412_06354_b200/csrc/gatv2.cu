@@ -181,7 +181,7 @@ __global__ void __launch_bounds__(256) v2_colsum_partial_kernel(const float* __r
     }
 }
 // out[f] = sum of the nb partials of column f: 32 walkers per column, four loads in flight each, added in walker order
-__global__ void __launch_bounds__(1024) v2_colsum_final_kernel(const float* __restrict__ bsum, int nb, int F, float* __restrict__ out) {
+__global__ void __launch_bounds__(1024) v2_colsum_final_kernel(const float* bsum, int nb, int F, float* __restrict__ out) {
     pdl_wait();
     __shared__ float sums[32][33];
     const int col = threadIdx.x & 31, w = threadIdx.x >> 5, f = blockIdx.x * 32 + col;

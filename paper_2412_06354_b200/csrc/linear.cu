@@ -94,7 +94,7 @@ gemm_simt_kernel(const TA* __restrict__ A, int64_t sam, int64_t sak, const TB* _
 // (4.7 us for the 148 partials of a 128 x 128 result: 9.7 MB from L2).
 template <typename TC>
 __global__ void __launch_bounds__(256)
-slab_sum_kernel(const float* __restrict__ part, int slabs, int64_t n, TC* __restrict__ out, int cols, int rows_out, int cols_out, int ld, int c0) {
+slab_sum_kernel(const float* part, int slabs, int64_t n, TC* __restrict__ out, int cols, int rows_out, int cols_out, int ld, int c0) {
     __shared__ float gsum[8][32];
     pdl_wait();
     const int e = threadIdx.x & 31, g = threadIdx.x >> 5;
@@ -126,7 +126,7 @@ slab_sum_kernel(const float* __restrict__ part, int slabs, int64_t n, TC* __rest
 // column in a row of dst is zero and never read (the tensor maps know the real width).
 template <typename TE, int PER>
 __global__ void __launch_bounds__(256)
-pad_rows_kernel(const TE* __restrict__ src, int64_t rows, int cols, TE* __restrict__ dst, int chunks) {
+pad_rows_kernel(const TE* src, int64_t rows, int cols, TE* __restrict__ dst, int chunks) {
     pdl_wait();
     const int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x;
     if (i >= rows * chunks) return;

@@ -54,7 +54,7 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
 // the bias of the CTA's output columns in shared memory, zeros past the last, for the epilogue warps (256 threads from `first`)
 __device__ __forceinline__ void stage_bias(float* to, const float* bias, int have, int first) {
     const int c = (int)threadIdx.x - first;
-    to[c] = bias && c < have ? __ldg(bias + c) : 0.f;
+    to[c] = bias && c < have ? bias[c] : 0.f;
     asm volatile("bar.sync 1, 256;" ::: "memory");
 }
 // 16 columns of a row: + bias, max(., 0)
@@ -516,11 +516,11 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
                 off[u] = P.b_transposed ? (uint32_t)(r >> 3) * b_sbo + (uint32_t)c * 128 + (uint32_t)(r & 7) * 16
                                         : (uint32_t)c * b_sbo + (uint32_t)(r >> 3) * 128 + (uint32_t)(r & 7) * 16;
                 if (P.ldw % 4 == 0 && r < have_rows && c * 8 + 8 <= have_cols) {
-                    const float4 lo = __ldg(reinterpret_cast<const float4*>(srcf)), hi = __ldg(reinterpret_cast<const float4*>(srcf) + 1);
+                    const float4 lo = reinterpret_cast<const float4*>(srcf)[0], hi = reinterpret_cast<const float4*>(srcf)[1];
                     x[u][0] = lo.x; x[u][1] = lo.y; x[u][2] = lo.z; x[u][3] = lo.w; x[u][4] = hi.x; x[u][5] = hi.y; x[u][6] = hi.z; x[u][7] = hi.w;
                 } else {
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) x[u][j] = (r < have_rows && c * 8 + j < have_cols) ? __ldg(srcf + j) : 0.f;
+                    for (int j = 0; j < 8; ++j) x[u][j] = (r < have_rows && c * 8 + j < have_cols) ? srcf[j] : 0.f;
                 }
             }
 #pragma unroll

@@ -12,8 +12,8 @@ namespace gnn {
 // ------------------------------------------------------------------ element-wise kernels
 // out[i, chunk] = c(i) * D[i, chunk], c(i) = row length (times_degree) or [row length > 0]
 template <typename T>
-__global__ void row_scale_kernel(const int64_t* __restrict__ rowptr, int32_t N, int nvec, int times_degree,
-                                 const uint4* __restrict__ D, uint4* __restrict__ out) {
+__global__ void row_scale_kernel(const int64_t* rowptr, int32_t N, int nvec, int times_degree,
+                                 const uint4* D, uint4* __restrict__ out) {
     pdl_wait();
     constexpr int EPC = Chunk<T>::N;
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -32,9 +32,9 @@ __global__ void row_scale_kernel(const int64_t* __restrict__ rowptr, int32_t N, 
 
 // de[p, f] = scale(i) * X[col[p], f] * D[i, f] for p in row i: the gradient of element-wise edge factors
 template <typename T>
-__global__ void edge_factor_grad_kernel(const int64_t* __restrict__ rowptr, const int32_t* __restrict__ col, int32_t N,
-                                        int64_t E, int nvec, int mean, const uint4* __restrict__ X,
-                                        const uint4* __restrict__ D, float* __restrict__ de) {
+__global__ void edge_factor_grad_kernel(const int64_t* rowptr, const int32_t* col, int32_t N,
+                                        int64_t E, int nvec, int mean, const uint4* X,
+                                        const uint4* D, float* __restrict__ de) {
     pdl_wait();
     constexpr int EPC = Chunk<T>::N;
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
@@ -58,7 +58,7 @@ __global__ void edge_factor_grad_kernel(const int64_t* __restrict__ rowptr, cons
 // combines its threads by a shuffle / shared-memory tree, and a second launch adds the block results
 constexpr int DOT_THREADS = 256, DOT_MAX_BLOCKS = 1184;
 template <typename T>
-__global__ void __launch_bounds__(DOT_THREADS) dot_partial_kernel(const uint4* __restrict__ a, const uint4* __restrict__ b,
+__global__ void __launch_bounds__(DOT_THREADS) dot_partial_kernel(const uint4* a, const uint4* b,
                                                                   int64_t nvec, float* __restrict__ partial) {
     pdl_wait();
     constexpr int EPC = Chunk<T>::N;
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(DOT_THREADS) dot_partial_kernel(const uint4* _
     }
 }
 // the partials' sum in a fixed order: a lane takes every 32nd, the lanes are added by an xor tree
-__global__ void dot_final_kernel(const float* __restrict__ partial, int nb, float* __restrict__ out) {
+__global__ void dot_final_kernel(const float* partial, int nb, float* __restrict__ out) {
     pdl_wait();
     float s = 0.f;
 #pragma unroll 4
@@ -99,7 +99,7 @@ __global__ void dot_final_kernel(const float* __restrict__ partial, int nb, floa
 // range of rows; its threads form row groups of nvec threads (one 16-byte chunk each).
 constexpr int EB_THREADS = 256, EB_MAX_BLOCKS = 592;
 template <typename T>
-__global__ void __launch_bounds__(EB_THREADS) epilogue_backward_kernel(const uint4* __restrict__ Y, const uint4* __restrict__ dY,
+__global__ void __launch_bounds__(EB_THREADS) epilogue_backward_kernel(const uint4* Y, const uint4* dY,
                                                                       int32_t N, int nvec, int relu, uint4* __restrict__ dZ,
                                                                       float* __restrict__ partial, int rows_per_block) {
     pdl_wait();
@@ -147,7 +147,7 @@ __global__ void __launch_bounds__(EB_THREADS) epilogue_backward_kernel(const uin
 // out[f] = sum of the nb partials of column f: 8 walkers per column take every eighth partial, four loads in flight each, and
 // are added in walker order (one thread per column walking them all took 14 us for 400 partials)
 constexpr int CS_WALKERS = 8;
-__global__ void __launch_bounds__(32 * CS_WALKERS) column_sum_final_kernel(const float* __restrict__ partial, int nb, int F, float* __restrict__ out) {
+__global__ void __launch_bounds__(32 * CS_WALKERS) column_sum_final_kernel(const float* partial, int nb, int F, float* __restrict__ out) {
     pdl_wait();
     __shared__ float sums[CS_WALKERS][32];
     const int col = threadIdx.x & 31, w = threadIdx.x >> 5, f = blockIdx.x * 32 + col;
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(32 * CS_WALKERS) column_sum_final_kernel(const
 }
 
 // merged edge list of one segment: ids shifted by the segment's offsets
-__global__ void merge_segment_kernel(const int32_t* __restrict__ src, const int32_t* __restrict__ dst, int64_t E,
+__global__ void merge_segment_kernel(const int32_t* src, const int32_t* dst, int64_t E,
                                      int32_t so, int32_t dof, int32_t seg, int32_t* __restrict__ src_out,
                                      int32_t* __restrict__ dst_out, int32_t* __restrict__ seg_out) {
     pdl_wait();
@@ -180,8 +180,8 @@ __global__ void merge_segment_kernel(const int32_t* __restrict__ src, const int3
 
 // coef[p] = w[p] / max(1, number of positions of p's row in p's segment) for mean segments, else w[p].
 // Inside a row the segments are contiguous and ascending, so the count comes from two binary searches.
-__global__ void segment_coef_kernel(const int64_t* __restrict__ rowptr, int32_t N, int64_t E, const int32_t* __restrict__ seg,
-                                    const float* __restrict__ w, const int32_t* __restrict__ seg_is_mean, int S,
+__global__ void segment_coef_kernel(const int64_t* rowptr, int32_t N, int64_t E, const int32_t* seg,
+                                    const float* w, const int32_t* seg_is_mean, int S,
                                     float* __restrict__ coef, int* __restrict__ flag) {
     pdl_wait();
     int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;

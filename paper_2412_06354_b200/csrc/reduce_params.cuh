@@ -82,7 +82,7 @@ __device__ __forceinline__ void add2(float& a0, float& a1, float x0, float x1) {
 // Smallest row r in [lo, N) with rowptr[r + 1] > v, or N: the first row at or after lo that has a
 // position beyond v.  Warp-cooperative (every lane must call it with the same arguments): a look at the
 // next 32 rows, then a 32-way search.
-__device__ __forceinline__ int first_row_ending_after(const int64_t* __restrict__ rowptr, int lo, int N, int64_t v, int lane) {
+__device__ __forceinline__ int first_row_ending_after(const int64_t* rowptr, int lo, int N, int64_t v, int lane) {
     {  // the common case, one coalesced load: the row is among the next 32
         const int r = lo + lane;
         const unsigned m = __ballot_sync(0xffffffffu, r >= N || rowptr[r + 1] > v);
@@ -105,7 +105,7 @@ __device__ __forceinline__ int first_row_ending_after(const int64_t* __restrict_
 
 // Position holding `pos`: the last row r with rowptr[r] <= pos (0 <= pos < E), or row 0 if there is none.  Warp-cooperative.  The
 // first look is at 32 rows spaced 64 apart around the row that even degrees would give, then 32-way steps, then 64 rows at once.
-__device__ __forceinline__ int row_of_position(const int64_t* __restrict__ rowptr, int N, int64_t E, int64_t pos, int lane) {
+__device__ __forceinline__ int row_of_position(const int64_t* rowptr, int N, int64_t E, int64_t pos, int lane) {
     int lo = 0, hi = N;  // rowptr[lo] <= pos < rowptr[hi]
     if (N > 1024) {
         const int guess = (int)((double)pos * ((double)N / (double)E));
@@ -132,7 +132,7 @@ __device__ __forceinline__ int row_of_position(const int64_t* __restrict__ rowpt
 // row that began before), start[count] = the last one's end, or n + 1 if it goes on.  Positions before the first row or after the
 // last (row pointers of a caller that leave some uncovered, as nodes outside graph_ptr) are staged as a row of id -1, whose
 // sums the callers drop.  Returns the count, at most n.  Warp-cooperative.
-__device__ __forceinline__ int stage_rows(const int64_t* __restrict__ rowptr, int N, int64_t E, int cs, int n, int lane, int* row, uint16_t* start,
+__device__ __forceinline__ int stage_rows(const int64_t* rowptr, int N, int64_t E, int cs, int n, int lane, int* row, uint16_t* start,
                                           bool& began_before) {
     const int r0 = row_of_position(rowptr, N, E, cs, lane);
     int m = 1;

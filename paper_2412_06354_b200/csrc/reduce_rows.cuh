@@ -59,7 +59,7 @@ __device__ __forceinline__ void finish_row(const PropParams& P, int row, int64_t
                 c = (P.self_mode == GNN_SELF_TIMES_DEGREE) ? c * (float)d : (d > 0 ? c : 0.f);
             }
             float x[EPC];
-            Chunk<T>::unpack(__ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(P.self_X) + (size_t)row * P.self_ld + (size_t)ci * 16)), x);
+            Chunk<T>::unpack(*reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(P.self_X) + (size_t)row * P.self_ld + (size_t)ci * 16), x);
 #pragma unroll
             for (int j = 0; j < EPC; ++j) v[j] = fmaf(c, x[j], v[j]);
         }
@@ -139,7 +139,7 @@ struct RowReducer {
             const int t = HEAD ? __shfl_sync(0xffffffffu, e.t, j + u, LPR) : 0;
             if (u < n) {
                 buf[u] = ld_hint16(Xl + (size_t)(uint32_t)c * P.x_ld, pol_keep);
-                if (HEAD) hw[HEAD ? u : 0][0] = __ldg(wh_l + (size_t)(uint32_t)t * P.H);
+                if (HEAD) hw[HEAD ? u : 0][0] = ld_f32(wh_l + (size_t)(uint32_t)t * P.H);
                 if (EF) {
                     const float4* q = reinterpret_cast<const float4*>(P.ef + (size_t)(pos + u) * P.ef_ld + (size_t)ci * EPC);
 #pragma unroll
@@ -152,7 +152,7 @@ struct RowReducer {
                 if (ROUTE) {
                     const int4* q = reinterpret_cast<const int4*>(P.route_arg + (size_t)(uint32_t)c * P.arg_ld + (size_t)ci * EPC);
 #pragma unroll
-                    for (int k = 0; k < EPC / 4; ++k) win[ROUTE ? u : 0][ROUTE ? k : 0] = __ldg(q + k);
+                    for (int k = 0; k < EPC / 4; ++k) win[ROUTE ? u : 0][ROUTE ? k : 0] = ld_int4(q + k);
                 }
             }
         }
@@ -457,7 +457,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     // MODE_V2: this row's own features, the next row's on their way, and the share of da (all rows of the group together)
     float xs[V2 ? EPC : 1], da[DA ? EPC : 1];
     uint4 own_next = make_uint4(0u, 0u, 0u, 0u);
-    auto own = [&](int qq) { return __ldg(reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(P.v2_self) + (size_t)max(S.row[qq], 0) * P.x_ld) + ci); };
+    auto own = [&](int qq) { return ld_16(reinterpret_cast<const uint4*>(reinterpret_cast<const char*>(P.v2_self) + (size_t)max(S.row[qq], 0) * P.x_ld) + ci); };
     if (V2) {
         if (a < b) {
             Chunk<T>::unpack(own(q), xs);
@@ -507,7 +507,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
             ends |= ((unsigned)cc >> 31) << u;
             cc &= 0x7fffffff;
             B.x[u] = ld_hint16(Xl + (size_t)(uint32_t)cc * P.x_ld, pol_keep);
-            if (HEAD) B.hw[HEAD ? u : 0][0] = __ldg(wh_l + (size_t)(uint32_t)ts[u] * P.H);
+            if (HEAD) B.hw[HEAD ? u : 0][0] = ld_f32(wh_l + (size_t)(uint32_t)ts[u] * P.H);
             if (EF) {
                 const float4* f = reinterpret_cast<const float4*>(P.ef + (size_t)(cs + i + u) * P.ef_ld + (size_t)ci * EPC);
 #pragma unroll
@@ -520,7 +520,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
             if (ROUTE) {
                 const int4* f = reinterpret_cast<const int4*>(P.route_arg + (size_t)(uint32_t)cc * P.arg_ld + (size_t)ci * EPC);
 #pragma unroll
-                for (int k = 0; k < EPC / 4; ++k) B.win[ROUTE ? u : 0][ROUTE ? k : 0] = __ldg(f + k);
+                for (int k = 0; k < EPC / 4; ++k) B.win[ROUTE ? u : 0][ROUTE ? k : 0] = ld_int4(f + k);
             }
         }
         return ends;
@@ -606,7 +606,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
             const bool end = cc < 0;
             cc &= 0x7fffffff;
             R.x[0] = ld_hint16(Xl + (size_t)(uint32_t)cc * P.x_ld, pol_keep);
-            if (HEAD) R.hw[0][0] = __ldg(wh_l + (size_t)(uint32_t)St[HEAD ? i : 0] * P.H);
+            if (HEAD) R.hw[0][0] = ld_f32(wh_l + (size_t)(uint32_t)St[HEAD ? i : 0] * P.H);
             if (EF) {
 #pragma unroll
                 for (int k = 0; k < MW; ++k) R.hw[0][k] = P.ef[(size_t)(cs + i) * P.ef_ld + (size_t)ci * EPC + k];
@@ -614,7 +614,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
             if (ROUTE) {
 #pragma unroll
                 for (int k = 0; k < EPC / 4; ++k)
-                    R.win[0][ROUTE ? k : 0] = __ldg(reinterpret_cast<const int4*>(P.route_arg + (size_t)(uint32_t)cc * P.arg_ld + (size_t)ci * EPC) + k);
+                    R.win[0][ROUTE ? k : 0] = ld_int4(reinterpret_cast<const int4*>(P.route_arg + (size_t)(uint32_t)cc * P.arg_ld + (size_t)ci * EPC) + k);
             }
             use(R, 0, i, HAS_W ? Sw[HAS_W ? i : 0] : 1.0f, ROUTE ? St[ROUTE ? i : 0] : 0);
             if (end) flush();
