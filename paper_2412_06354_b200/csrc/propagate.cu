@@ -62,7 +62,9 @@ static int warp_positions(int32_t N, int64_t E, int row_bytes, bool stream) {
     if (E >= (int64_t)4 * 1024 * 1024) return 256;
     if (E >= 512 * 1024) return E > 64 * (int64_t)N || E >= 2500 * 1000 || (row_bytes <= 128 && E >= 1000 * 1000) ? 256 : 128;
     if (!stream) return 64;
-    return E >= 256 * 1024 ? 128 : E >= 128 * 1024 || row_bytes <= 64 ? 64 : 32;
+    // rows over 512 bytes run in slabs: the last one's eight lane groups, if it has 64 bytes or less, need 64 positions to pipeline
+    const int narrowest = row_bytes > 512 && row_bytes % 512 != 0 ? row_bytes % 512 : row_bytes;
+    return E >= 256 * 1024 ? 128 : E >= 128 * 1024 || narrowest <= 64 ? 64 : 32;
 }
 
 // Room for a partial row per 64 to 256 positions.  The streaming kernel needs an eighth of that; the size is what callers

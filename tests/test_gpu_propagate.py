@@ -577,6 +577,21 @@ def test_rows_cut_at_every_kind_of_boundary(gnn, e, dtype, F):
 
 # Sort digits of 10 bits (ids at 2^10 and 2^20), tiles of 2048 edges, rows over 512 positions for the degrees, edge counts
 # that are no multiple of a vector
+# Rows a little over 512 bytes on small graphs: the last column slab has one to four 16-byte chunks and eight lane groups, whose
+# runs have to be whole pipeline steps
+@pytest.mark.parametrize("e,dtype,F", [(9000, "f32", 132), (20_001, "f32", 272), (131_071, "bf16", 264), (4097, "bf16", 544)])
+def test_narrow_last_slab_on_small_graphs(gnn, e, dtype, F):
+    n, src, dst = ragged_graph(e, n=600, e=e, hub=e // 9, empty_from=590)
+    g, X, w = build_graph(gnn, n, src, dst), feats((n, F), dtype, 77), synth.uniform_f32((e,), 0.0, 1.0, 78)
+    eid = g.eid[:e].cpu().numpy()
+    for op in ("sum", "mean"):
+        o, S, _ = oracle.propagate(op, n, src, dst, X, w)
+        assert_close(to_host64(gnn.propagate_fused(g, to_dev(X), to_dev(w[eid]), op)), o, S, dtype, op)
+    o, _, a = oracle.propagate("max", n, src, dst, X)
+    out, arg = gnn.propagate_fused(g, to_dev(X), None, "max")
+    assert np.array_equal(bits(out), f64_to_dtype_bits(o, dtype))
+
+
 @pytest.mark.parametrize("n,e", [(1023, 2047), (1024, 2048), (1025, 2049), (1 << 20, 4097), ((1 << 20) + 1, 6143), (3, 5001)])
 def test_setup_at_digit_and_tile_boundaries(gnn, n, e):
     rng = np.random.default_rng(n + e)
