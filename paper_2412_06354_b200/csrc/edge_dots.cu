@@ -313,7 +313,7 @@ static gnn_status run_edges(const char* who, const gnn_csr* g, const void* X, co
     GNN_REQUIRE(H == 1 || (lph <= 32 && (lph & (lph - 1)) == 0), GNN_ERR_UNSUPPORTED,
                 "%s: a head must span a power-of-two number (<= 32) of 16-byte chunks (C=%d)", who, C);
     GNN_REQUIRE(aligned16(X) && aligned16(D), GNN_ERR_INVALID_ARG, "%s: feature matrices must be 16-byte aligned", who);
-    GNN_REQUIRE(g->E < ((int64_t)1 << 31) - 4096, GNN_ERR_UNSUPPORTED, "%s: positions must fit 32 bits (E < 2^31)", who);
+    GNN_REQUIRE(g->E < ((int64_t)1 << 31), GNN_ERR_UNSUPPORTED, "%s: positions must fit 32 bits (E < 2^31)", who);
     if (g->E == 0) return GNN_OK;
     EdgeParams P = {};
     P.rowptr = g->rowptr; P.col = g->col; P.X = X; P.D = D; P.a = a; P.out = out;

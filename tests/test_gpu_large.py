@@ -120,3 +120,22 @@ def test_edge_weight_gradient_full_size(big):
     bw = oracle.propagate_backward("sum", n, src, dst, X, np.ones(len(src), np.float32), R, want_dX=False, want_dw=True)
     eid = g.eid.cpu().numpy()
     assert_close(to_host64(dW), bw["dw"][eid], bw["Sdw"][eid], "f32", "edge-weight gradient, all edges")
+
+
+def test_edge_values_up_to_the_last_index():
+    """Dot products of 2^31 - 2 edges, the most that 32-bit positions hold: one row, so that every value is known."""
+    import torch
+    from paper_2412_06354_b200 import gnn
+    gnn.load()
+    E = 2**31 - 2
+    if torch.cuda.mem_get_info()[0] < 40 << 30:
+        pytest.skip("needs 18 GB of device memory")
+    rowptr, col = torch.tensor([0, E], dtype=torch.int64, device="cuda"), torch.zeros(E, dtype=torch.int32, device="cuda")
+    X, D = torch.tensor([[1.0, 2.0, 3.0, 4.0]], device="cuda"), torch.tensor([[5.0, 6.0, 7.0, 8.0]], device="cuda")
+    s = torch.zeros(E, device="cuda")
+    c = gnn.CsrStruct(1, E, rowptr.data_ptr(), col.data_ptr(), None, None, None, None, None)
+    gnn._check(gnn.load().gnn_edge_dot(c, X.data_ptr(), D.data_ptr(), 1, 4, gnn.F32, s.data_ptr(), torch.cuda.current_stream().cuda_stream))
+    assert float(s.min()) == 70.0 and float(s.max()) == 70.0
+    s.zero_()
+    gnn._check(gnn.load().gnn_gatv2_logits(c, X.data_ptr(), D.data_ptr(), X.data_ptr(), 1, 4, gnn.F32, 0.2, s.data_ptr(), torch.cuda.current_stream().cuda_stream))
+    assert float(s.min()) == 100.0 and float(s.max()) == 100.0
