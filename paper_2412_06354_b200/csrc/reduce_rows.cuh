@@ -37,7 +37,7 @@ __device__ __forceinline__ void finish_row(const PropParams& P, int row, int64_t
 #pragma unroll
         for (int j = 0; j < EPC; ++j) v[j] *= f;
     }
-    if (MODE == MODE_V2) {
+    if (MODE == MODE_V2 && len > 0) {  // (a row without positions stays zero, whatever a holds)
 #pragma unroll
         for (int j = 0; j < EPC; ++j) v[j] *= P.epi_a[ci * EPC + j];
     }
@@ -728,7 +728,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
             for (int k = wib + 1; k < RR_WARPS && s_head[k] != HEAD_NONE; ++k) {
                 join(true, all[k].head + li * EPC, all[k].head_a + (ARG ? li * EPC : 0));
                 if (s_head[k] == HEAD_CLOSED) {
-                    if (row >= 0) finish_row<T, MODE, EPI>(P, row, P.mean ? P.rowptr[row + 1] - P.rowptr[row] : 0, ci, carry, carg);
+                    if (row >= 0) finish_row<T, MODE, EPI>(P, row, P.mean ? P.rowptr[row + 1] - P.rowptr[row] : 1, ci, carry, carg);
                     else write_partial(0, carry, carg);
                     return;
                 }

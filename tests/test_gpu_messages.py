@@ -267,6 +267,18 @@ def test_gatv2_backward_hub_rows_of_both_orientations(gnn, dtype, H, C):
     assert all(np.array_equal(bits(x), bits(y)) for x, y in zip((dXl, dXr, da), again)), "not bit-reproducible"
 
 
+@pytest.mark.parametrize("a0", [float("inf"), float("nan")])
+def test_gatv2_gradient_of_nodes_without_edges_is_zero(gnn, a0):
+    """... also where the attention vector is not finite: there are no terms to multiply."""
+    import torch
+    n, src, dst = 40, np.arange(20, dtype=np.int32), np.arange(20, 40, dtype=np.int32)
+    g = build_graph(gnn, n, src, dst)
+    X, a, ds = torch.ones((n, 64), device="cuda"), torch.full((4, 16), a0, device="cuda"), torch.ones((g.E, 4), device="cuda")
+    dXl, dXr, _ = gnn.gatv2_logits_backward(g, X, X, a, ds, 4)
+    assert torch.count_nonzero(dXr[:20]) == 0 and torch.count_nonzero(dXl[20:]) == 0
+    assert not torch.isfinite(dXr[20:]).any() and not torch.isfinite(dXl[:20]).any()
+
+
 @pytest.mark.parametrize("dtype,H,C", [("f32", 4, 16), ("bf16", 8, 32)])
 def test_gatv2_backward_without_workspace(gnn, dtype, H, C):
     """A call without da may come without a workspace: rows are then walked one by one (and hubs by a block)."""
