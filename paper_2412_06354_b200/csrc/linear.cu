@@ -9,7 +9,7 @@
 // K and M: sizes are rounded up with zeros from the copy engine.  The copy engine wants rows that start on 16 bytes;
 // matrices whose rows do not (K or M odd, say) are first copied to padded rows in the workspace, one pass at L2 or HBM
 // speed.  Such shapes took the FFMA kernel before (170000 x 100 x 47 fp32, forward and backward: 1410 -> 121 us).
-// linear_tc.cu (single-buffered) takes over if the tensor-map encoder is not available; everything else runs the
+// Everything else, a driver without the tensor-map encoder and calls that lack the room or the alignment included, runs the
 // shared-memory tiled FFMA kernel below with fp32 accumulation.  All sums have a fixed order.
 #include "common.cuh"
 
@@ -151,9 +151,6 @@ static void launch_simt(const TA* A, int64_t sam, int64_t sak, const TB* B, int6
 static int dw_slab_rows(int64_t N) { return N <= 148 * 128 ? 128 : 4096; }
 static int dw_slabs(int64_t N) { return (int)(N > 0 ? ceil_div(N, dw_slab_rows(N)) : 1); }
 
-bool linear_tc_supported(int64_t N, int K, int M, gnn_dtype dtype);
-gnn_status linear_tc_forward(const void* X, const void* W, int64_t N, int K, int M, int w_transposed, gnn_dtype dtype,
-                             void* Y, int* d_flag, cudaStream_t st);
 bool linear_tma_supported(int64_t N, int Kc, int Mo, int b_transposed, gnn_dtype dtype);
 gnn_status linear_tma_forward(const void* X, int ldx, const void* W, int ldw, int64_t N, int Kc, int Mo, int b_transposed, void* Y, int* d_flag, int reset,
                               cudaStream_t st, const float* bias, int relu);
@@ -166,10 +163,6 @@ gnn_status linear_tma_dw(const void* X, int ldx, const void* dY, int ldd, int64_
 bool linear_tma_f32_dw_supported(int64_t N, int K, int M, int Mo, gnn_dtype dtype);
 int linear_tma_f32_dw_partials(int64_t N);
 gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, int Mo, float* part, int* d_flag, int reset, cudaStream_t st);
-bool linear_tc_dw_supported(int64_t N, int K, int M, gnn_dtype dtype);
-int linear_tc_dw_partials(int64_t N);
-gnn_status linear_tc_dw(const void* X, const void* dY, int64_t N, int K, int M, gnn_dtype dtype, float* part, int* d_flag,
-                        cudaStream_t st);
 
 static int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
@@ -259,9 +252,6 @@ gnn_status gnn_linear_bias_act(const void* X, const void* W, int32_t N, int K, i
         }
     }
     if (cudaMemsetAsync(ws, 0, sizeof(int), st) != cudaSuccess) GNN_FAIL(GNN_ERR_CUDA, "%s: memset failed (is ws a device pointer?)", who);
-    // the single-buffered tensor-core kernel has no epilogue: with a bias or relu the FFMA kernel, whose epilogue applies
-    // them before the single rounding
-    if (!bias && !relu && linear_tc_supported(N, K, M, dtype)) return linear_tc_forward(X, W, N, K, M, 0, dtype, Y, (int*)ws, st);
     if (dtype == GNN_F32) {
         launch_simt<float, float, float>((const float*)X, K, 1, (const float*)W, M, 1, (float*)Y, N, M, K, K, 1, 0, st, bias, relu);
     } else {
@@ -318,9 +308,6 @@ gnn_status gnn_linear_backward(const void* X, const void* W, const void* dY, int
             }
             if (rc != GNN_OK) return rc;
             reset = 0;
-        } else if (linear_tc_supported(N, M, K, dtype)) {
-            gnn_status rc = linear_tc_forward(dY, W, N, M, K, 1, dtype, dX, status, st);
-            if (rc != GNN_OK) return rc;
         } else if (dtype == GNN_F32) {
             launch_simt<float, float, float>((const float*)dY, M, 1, (const float*)W, 1, M, (float*)dX, N, K, M, M, 1, 0, st);
         } else {
@@ -351,13 +338,9 @@ gnn_status gnn_linear_backward(const void* X, const void* W, const void* dY, int
             }
             return GNN_OK;
         }
-        int slabs = dw_slabs(N);
+        const int slabs = dw_slabs(N);
         const int64_t km = (int64_t)K * M;
-        if (N > 0 && linear_tc_dw_supported(N, K, M, dtype)) {
-            slabs = linear_tc_dw_partials(N);
-            gnn_status rc = linear_tc_dw(X, dY, N, K, M, dtype, part, status, st);
-            if (rc != GNN_OK) return rc;
-        } else if (N == 0) {
+        if (N == 0) {
             if (cudaMemsetAsync(part, 0, (size_t)km * 4, st) != cudaSuccess) GNN_FAIL(GNN_ERR_CUDA, "%s: memset failed", who);
         } else if (dtype == GNN_F32) {
             launch_simt<float, float, float>((const float*)X, 1, K, (const float*)dY, M, 1, part, K, M, N, dw_slab_rows(N), slabs, km, st);

@@ -8,15 +8,8 @@ namespace gnn {
 
 constexpr int TC_ROWS = 128;                  // rows of X per tile = MMA M
 constexpr uint32_t TC_WAIT_LIMIT = 1u << 20;  // polls of one barrier phase before a kernel gives up
-constexpr size_t TC_SMEM_LIMIT = 200 * 1024;  // dynamic shared memory the single-buffered kernels ask for
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// 16-byte asynchronous copy global -> shared, bypassing registers; src_bytes = 0 writes zeros
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // shared-memory matrix descriptor: start address, leading/stride byte offsets (all >> 4), swizzle mode
 // (0 = none, 2 = 128-byte swizzle)
@@ -121,7 +114,7 @@ __device__ __forceinline__ void tmem_st4(uint32_t taddr, uint4 v) {
 __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // raise a kernel's dynamic shared memory limit, once per (device, kernel slot)
-inline gnn_status allow_big_smem(const char* who, const void* kernel, int which, size_t bytes = TC_SMEM_LIMIT) {
+inline gnn_status allow_big_smem(const char* who, const void* kernel, int which, size_t bytes) {
     static std::atomic<unsigned char> done[64][24];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = -1;
