@@ -301,8 +301,9 @@ gnn_status gnn_edge_dot_backward(const gnn_csr* g, const void* Xj, const void* X
  * e_width = H).  Rows of H*C elements up to 512 bytes; with H > 1 a head must span a power-of-two number of
  * 16-byte chunks.  The E x F tensor is never formed.
  * Backward for ds_csr float [E,H]: dXl, dXr [N,H,C] of dtype and da float [H,C] (da needs dXr and the
- * workspace; each may be NULL); the derivative of LeakyReLU at 0 is slope.  Rows are walked by a warp, rows over
- * 256 positions by a block, in a fixed order.  ws: gnn_gatv2_logits_backward_workspace(N, H, C) bytes. */
+ * workspace; each may be NULL); the derivative of LeakyReLU at 0 is slope.  Every order of additions is
+ * fixed.  ws: gnn_gatv2_logits_backward_workspace(N, H, C) bytes; without it, and where a graph has so many edges
+ * per node that the partial rows do not fit it, a warp walks a row (over 256 positions a block), several times slower. */
 gnn_status gnn_gatv2_logits(const gnn_csr* g, const void* Xl, const void* Xr, const float* a, int H, int C,
                             gnn_dtype dtype, float slope, float* s_csr, gnn_stream stream);
 size_t gnn_gatv2_logits_backward_workspace(int32_t N, int H, int C);
@@ -418,7 +419,7 @@ gnn_status gnn_edge_softmax_backward(const gnn_csr* g, const void* alpha_EH, con
  * head must span a power-of-two number (1..32) of 16-byte chunks (C = 4, 8, 16, ... for float,
  * 8, 16, 32, ... for bf16); other shapes return GNN_ERR_UNSUPPORTED from the forward and the
  * backward call alike.  The E x F message tensor is never formed.
- * The first gnn_gat_fused / _backward call on a device creates two helper streams and three events (no device
+ * The first gnn_gat_fused / _backward call on a device creates three helper streams and three events (no device
  * memory) on which row classes of the attention kernels run side by side; they are forked from and joined back
  * into `stream`, so the call keeps its place in the stream's order.  Make that first call outside a stream capture.
  * ws: gnn_gat_fused_workspace(N, E, H, C, backward) bytes. */
@@ -465,7 +466,8 @@ gnn_status gnn_reduce_nodes_backward(const int64_t* graph_ptr, int32_t G, int32_
  * W [K,M], Y [N,M], all row-major and of dtype, 16-byte aligned.  With K up to 512 and M up
  * to 1024 the products run on the tensor cores with fp32 accumulation: bf16 directly, fp32 by an exact
  * three-term bf16 split of every value, which keeps fp32 accuracy (weights that do not fit shared memory
- * three times, e.g. 256x256, run as one launch per block of output columns).  Rows that do not start on 16 bytes
+ * three times, e.g. 256x256, are divided among the blocks of the launch by output columns; a value that is not
+ * finite gives NaN in the results it enters).  Rows that do not start on 16 bytes
  * (K or M not a multiple of 16 bytes worth of elements) are first copied to padded rows in the workspace.  A
  * call given less than gnn_linear_workspace bytes (say, sized for a wider layer without such rows; the least are
  * 256 bytes forward, 512 + 4 K M max(148, ceil(N / 4096)) backward) then uses an fp32 FFMA kernel, several times

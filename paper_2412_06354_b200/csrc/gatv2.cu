@@ -9,7 +9,7 @@
 // ds * a * LeakyReLU'(z) needing both rows again; da sums ds * LeakyReLU(z) over all positions.  Both are the segmented
 // reduction of reduce_rows.cuh with the own row's chunk in registers; da falls out of the first as one partial per block.
 // Its scratch (partial rows) has to fit the caller's workspace, whose size knows N only, and a call without da may come
-// without a workspace: then (below, mean degrees of several hundred) a warp walks a row, rows over 256 positions get a
+// without a workspace: then (a mean degree above some 85 where a warp's share is 32 positions, up to 680 where it is 256) a warp walks a row, rows over 256 positions get a
 // block whose warps take contiguous shares that are added in warp order, and da is the column sum of per-row partials.
 // Every order is fixed: results are bit-reproducible.
 // 100k nodes / 1.6 M edges with hubs, 4 heads x 32 fp32: 1010 us by row and block, 265 us as segmented reductions.

@@ -8,7 +8,7 @@
 // 512 and up to 1024 output columns (dW: 512 x 256, or as much as fits tensor memory at a time), whatever the divisors of
 // K and M: sizes are rounded up with zeros from the copy engine.  The copy engine wants rows that start on 16 bytes;
 // matrices whose rows do not (K or M odd, say) are first copied to padded rows in the workspace, one pass at L2 or HBM
-// speed.  Such shapes took the FFMA kernel before (170000 x 100 x 47 fp32, forward and backward: 1410 -> 121 us).
+// speed.  Such shapes took the FFMA kernel before (170000 x 100 x 47 fp32, forward and backward: 1405 -> 121 us).
 // Everything else, a driver without the tensor-map encoder and calls that lack the room or the alignment included, runs the
 // shared-memory tiled FFMA kernel below with fp32 accumulation.  All sums have a fixed order.
 #include "common.cuh"

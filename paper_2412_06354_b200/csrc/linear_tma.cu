@@ -14,7 +14,7 @@
 //   warps 2..9  epilogue: wait for a tile's accumulator, read it back (tcgen05.ld), round to bf16,
 //            write 32 rows x 64 columns at a time into a swizzled staging block that one bulk tensor
 //            store sends to Y (rows past N are clipped by the copy engine), and hand the accumulator back.
-// The contraction is short (Kc <= 256), so the kernel is bound by reading X and writing Y; the ring
+// The contraction is short (Kc <= 512), so the kernel is bound by reading X and writing Y; the ring
 // keeps 64-100 KB of loads in flight per SM.
 //
 // Every wait has an iteration limit: on expiry the role raises a status word and leaves its loop, the
@@ -924,7 +924,7 @@ static bool make_map_f32_blocks(CUtensorMap* m, const void* ptr, int64_t rows, i
 //               that stays in tensor memory for the whole kernel;
 //   at the end the first eight converter warps write the accumulator as this CTA's fp32 partial [K,M]; the caller sums the
 //   partials in CTA order (fixed order: deterministic).
-// K a multiple of 32 up to 128 features (the MMA has 128 rows; those past K are zeros), M a multiple of 32 up to 128.
+// K a multiple of 32 up to 512 features (blocks of the MMA's 128 rows; those past K are zeros), M a multiple of 32 up to 256.
 // Every wait is bounded.
 // Two groups on slots of 32 rows, on slots of 16 four where four buffers and slots fit.  170k x 128 x 128: 50 us with 8 warps
 // on one slot after the other, 47 us with 16, 58 us in four groups on slots of 16 rows, 42 us so; reading X and dY takes 27 us.

@@ -59,7 +59,6 @@ static ReduceWs carve(void* ws, int64_t pieces, int F, bool with_arg) {
 //  - Small graphs are bound by the longest chain of loads of a warp, so their shares shrink with them (80k edges with hubs,
 //    512-byte rows: 15.8 us at 64, 11.8 us at 32; 64-byte rows have eight groups per warp and gain nothing below 64).
 static int warp_positions(int32_t N, int64_t E, int row_bytes, bool stream) {
-    if (E >= (int64_t)4 * 1024 * 1024) return 256;
     if (E >= 512 * 1024) return E > 64 * (int64_t)N || E >= 2500 * 1000 || (row_bytes <= 128 && E >= 1000 * 1000) ? 256 : 128;
     if (!stream) return 64;
     // rows over 512 bytes run in slabs: the last one's eight lane groups, if it has 64 bytes or less, need 64 positions to pipeline
@@ -67,8 +66,9 @@ static int warp_positions(int32_t N, int64_t E, int row_bytes, bool stream) {
     return E >= 256 * 1024 ? 128 : E >= 128 * 1024 || narrowest <= 64 ? 64 : 32;
 }
 
-// Room for a partial row per 64 to 256 positions.  The streaming kernel needs an eighth of that; the size is what callers
-// have been told since the first version, and what decides which problems the built-in scratch takes.
+// Room for a partial row per 64, 128 or 1024 positions.  The streaming kernel, whose pieces are 256 to 2048 positions, needs a
+// sixteenth to a quarter of that below 4 Mi edges and half above; the size is what callers have been told since the first
+// version, and what decides which problems the built-in scratch takes.
 size_t chunked_workspace(int64_t E, int F, bool with_arg) {
     if (E <= 0) return carve(nullptr, 1, F, with_arg).bytes;
     const int per = E >= (int64_t)4 * 1024 * 1024 ? 1024 : E >= 512 * 1024 ? 128 : 64;
