@@ -33,6 +33,7 @@ METRIC = "propagate fwd+bwd edges*feat/s"
 UNIT = "edges*feat/s"
 ALL_CASES = [(F, dt) for dt in ("bf16", "f32") for F in (32, 64, 128, 256, 512)]
 FMAX = 512
+LAUNCHES_PER_PASS = 2  # of a sum over one column slab: the reduction, and the rows cut between its blocks
 
 # DRAM bytes (read + write, GB) of one gnn_propagate_fused / _backward call (all its reduction and
 # fix-up launches: wide rows run as 512-byte column slabs), taken with the hardware counters
@@ -40,56 +41,56 @@ FMAX = 512
 # N = 600,000, E = 30,750,000, a quarter of the workload) so that the capture stays small.  The line reports
 # these numbers times TRAFFIC_SCALE (the ratio of the edges*features processed).  That is a LOWER bound of the
 # full-size traffic: the reduced feature matrix is four times smaller against the same L2, so a larger share of
-# its gathers hits (a full-size capture of an earlier build of the same loop gave 79.6 GB where this gives 32.8).
+# its gathers hits.
 # The numbers belong to the kernel sources whose digest is TRAFFIC_KERNEL_SHA256; with other sources the line
 # reports traffic = null.
 TRAFFIC_SOURCE = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --clock-control none -k regex:rows_kernel over one step of "
                   "`bench.py --graph-scale 20` (N=600000, E=30.75M), scaled by 4.0 = ratio of edges*features; lower bound of the "
-                  "full-size traffic (better L2 reuse on the reduced matrix); summary under profiles/")
+                  "full-size traffic (better L2 reuse on the reduced matrix); profiles/dram_bytes_of_the_sweep_reduced_graph.md")
 TRAFFIC_SCALE = 4.0
 TRAFFIC_KERNEL_FILES = ("propagate.cu", "propagate.cuh", "reduce_params.cuh", "reduce_rows.cuh", "common.cuh")
-TRAFFIC_KERNEL_SHA256 = "62facf4d2c659f955d3468cd3144d3ed4b685ffbeb12d73cf41affba107fcf9c"
+TRAFFIC_KERNEL_SHA256 = "5d69e557b823263b90bb7e11d40498844044dfb1e9657da586e83fb64c52592a"
 TRAFFIC_GB_REDUCED = {
-    "32:bf16:copy_xj:fwd": 0.192,
-    "32:bf16:copy_xj:bwd": 0.19,
-    "32:bf16:e_mul_xj:fwd": 0.315,
-    "32:bf16:e_mul_xj:bwd": 0.315,
-    "64:bf16:copy_xj:fwd": 0.269,
-    "64:bf16:copy_xj:bwd": 0.27,
-    "64:bf16:e_mul_xj:fwd": 0.395,
-    "64:bf16:e_mul_xj:bwd": 0.395,
-    "128:bf16:copy_xj:fwd": 0.61,
-    "128:bf16:copy_xj:bwd": 0.61,
-    "128:bf16:e_mul_xj:fwd": 0.737,
-    "128:bf16:e_mul_xj:bwd": 0.737,
-    "256:bf16:copy_xj:fwd": 2.004,
-    "256:bf16:copy_xj:bwd": 2.004,
-    "256:bf16:e_mul_xj:fwd": 2.133,
-    "256:bf16:e_mul_xj:bwd": 2.133,
-    "512:bf16:copy_xj:fwd": 4.018,
-    "512:bf16:copy_xj:bwd": 4.021,
-    "512:bf16:e_mul_xj:fwd": 4.277,
-    "512:bf16:e_mul_xj:bwd": 4.281,
-    "32:f32:copy_xj:fwd": 0.257,
-    "32:f32:copy_xj:bwd": 0.258,
-    "32:f32:e_mul_xj:fwd": 0.381,
-    "32:f32:e_mul_xj:bwd": 0.382,
-    "64:f32:copy_xj:fwd": 0.579,
-    "64:f32:copy_xj:bwd": 0.58,
-    "64:f32:e_mul_xj:fwd": 0.706,
-    "64:f32:e_mul_xj:bwd": 0.706,
-    "128:f32:copy_xj:fwd": 1.918,
-    "128:f32:copy_xj:bwd": 1.917,
-    "128:f32:e_mul_xj:fwd": 2.047,
-    "128:f32:e_mul_xj:bwd": 2.044,
-    "256:f32:copy_xj:fwd": 3.848,
-    "256:f32:copy_xj:bwd": 3.843,
-    "256:f32:e_mul_xj:fwd": 4.107,
-    "256:f32:e_mul_xj:bwd": 4.103,
-    "512:f32:copy_xj:fwd": 7.685,
-    "512:f32:copy_xj:bwd": 7.68,
-    "512:f32:e_mul_xj:fwd": 8.199,
-    "512:f32:e_mul_xj:bwd": 8.198,
+    "32:bf16:copy_xj:fwd": 0.209,
+    "32:bf16:copy_xj:bwd": 0.209,
+    "32:bf16:e_mul_xj:fwd": 0.35,
+    "32:bf16:e_mul_xj:bwd": 0.349,
+    "64:bf16:copy_xj:fwd": 0.294,
+    "64:bf16:copy_xj:bwd": 0.294,
+    "64:bf16:e_mul_xj:fwd": 0.444,
+    "64:bf16:e_mul_xj:bwd": 0.445,
+    "128:bf16:copy_xj:fwd": 0.644,
+    "128:bf16:copy_xj:bwd": 0.645,
+    "128:bf16:e_mul_xj:fwd": 0.821,
+    "128:bf16:e_mul_xj:bwd": 0.822,
+    "256:bf16:copy_xj:fwd": 2.042,
+    "256:bf16:copy_xj:bwd": 2.041,
+    "256:bf16:e_mul_xj:fwd": 2.265,
+    "256:bf16:e_mul_xj:bwd": 2.264,
+    "512:bf16:copy_xj:fwd": 4.085,
+    "512:bf16:copy_xj:bwd": 4.086,
+    "512:bf16:e_mul_xj:fwd": 4.532,
+    "512:bf16:e_mul_xj:bwd": 4.529,
+    "32:f32:copy_xj:fwd": 0.287,
+    "32:f32:copy_xj:bwd": 0.287,
+    "32:f32:e_mul_xj:fwd": 0.436,
+    "32:f32:e_mul_xj:bwd": 0.438,
+    "64:f32:copy_xj:fwd": 0.628,
+    "64:f32:copy_xj:bwd": 0.629,
+    "64:f32:e_mul_xj:fwd": 0.802,
+    "64:f32:e_mul_xj:bwd": 0.803,
+    "128:f32:copy_xj:fwd": 1.992,
+    "128:f32:copy_xj:bwd": 1.991,
+    "128:f32:e_mul_xj:fwd": 2.177,
+    "128:f32:e_mul_xj:bwd": 2.175,
+    "256:f32:copy_xj:fwd": 3.994,
+    "256:f32:copy_xj:bwd": 3.993,
+    "256:f32:e_mul_xj:fwd": 4.363,
+    "256:f32:e_mul_xj:bwd": 4.359,
+    "512:f32:copy_xj:fwd": 7.982,
+    "512:f32:copy_xj:bwd": 7.986,
+    "512:f32:e_mul_xj:fwd": 8.719,
+    "512:f32:e_mul_xj:bwd": 8.721,
 }
 TRAFFIC_GB = {k: v * TRAFFIC_SCALE for k, v in TRAFFIC_GB_REDUCED.items()}
 
@@ -457,7 +458,7 @@ def main():
                 "traffic_source": (TRAFFIC_SOURCE + "; kernel sources sha256 " + TRAFFIC_KERNEL_SHA256[:16]) if traffic is not None else
                                   "null: the kernel sources differ from the ones the counters were taken with, or this is not the full-size relabelled workload",
                 "peak_source": peak_src, "bytes_model": "compulsory bytes per call: 4E(+4E weights)+8N+2*N*F*s = %d" % comp,
-                "ms_per_call": dom["fwd_ms"], "launches_per_call": launches_per_pass(E) * nslab,
+                "ms_per_call": dom["fwd_ms"], "launches_per_call": LAUNCHES_PER_PASS * nslab,
                 "dram_traffic_GBs": None if traffic is None else traffic * 1e3 / dom["fwd_ms"],
                 "dram_traffic_frac_of_peak": None if traffic is None else traffic * 1e3 / dom["fwd_ms"] / peak,
                 "l2_side_model_GBs": gather_bytes(N, E, dom["F"], sdom, wdom) / dom["fwd_ms"] / 1e6,
@@ -475,7 +476,7 @@ def main():
             "config": {"workload": ("VARIANT with the generator's natural vertex ids of: " if args.natural_ids else "") + WORKLOAD_NAME if shrink == 0 else f"REDUCED graph (R-MAT scale {args.graph_scale}) of: " + WORKLOAD_NAME, "N": N, "E": E, "cases": [f"{F}:{dt}" for F, dt in cases],
                        "l2": "inputs larger than L2: every launch streams >= 0.5 GB of indices and a feature matrix of 154 MB to 4.9 GB",
                        "parallelism": "replicas only" if world > 1 else "single GPU"},
-            "clocks": clocks, "gpu_launches": args.steps * sum(2 * launches_per_pass(E) * max(1, F * (2 if dt == "bf16" else 4) // 512) for F, dt, _, _ in plan), "roofline": roofline, "per_case": per_case}
+            "clocks": clocks, "gpu_launches": args.steps * sum(2 * LAUNCHES_PER_PASS * max(1, F * (2 if dt == "bf16" else 4) // 512) for F, dt, _, _ in plan), "roofline": roofline, "per_case": per_case}
 
     # ---- end to end through the host-buffer entry points
     if not args.no_e2e and hasattr(gnn, "propagate_fused_host"):
@@ -497,11 +498,6 @@ def main():
         print(json.dumps(line), flush=True)
     if world > 1:
         dist.destroy_process_group()
-
-
-def launches_per_pass(E):
-    """Kernels one column-slab pass of a sum launches: the reduction and the fix-up of rows cut between its blocks."""
-    return 2
 
 
 def run_e2e(args, torch, gnn, g, plan, hX, hR, w_csr, w_csrT, ws, N, E, fmax, dev, world, barrier):
