@@ -91,7 +91,7 @@ def test_graph_setup_and_propagate_stay_inside_their_buffers(guarded, n, e, hub)
 
 
 def test_row_walking_kernel_with_narrow_rows_stays_inside_its_buffers(guarded):
-    """8.4 M edges: narrow rows on the row-walking kernel (1024 positions per warp)."""
+    """8.4 M edges: narrow rows with 256 positions per warp (the most)."""
     gnn, gt = guarded
     n, e = 50_000, 8_400_000
     src, dst = graph(n, e, 1, hub=400_000)

@@ -135,10 +135,8 @@ def test_gat_attention_workload_full_size(gnn):
 
 @pytest.mark.parametrize("E", [8_400_000, 17_000_000])
 def test_gat_more_than_8mi_edges_uses_the_row_walking_kernels(gnn, E):
-    """8.4 M edges: above the size where the per-head gather, its transposed form (with the permuted
-    coefficients) and the per-head dot products switch from the position-first kernels to the row-walking ones.
-    17 M edges: more than 16384 chunks, so the hub rows (cut into more than 64 chunks) are finished by the
-    block-per-row fix-up, here with the per-head multipliers and the rank-1 row epilogue of the backward pass."""
+    """8.4 M edges: the per-head gather, its transposed form and the per-head dot products with the most positions
+    per warp.  17 M edges: hub rows are cut into more than 64 pieces and finished by the block-per-row fix-up, here with the per-head multipliers and the rank-1 row epilogue of the backward pass."""
     n, H, C = 200_000, 4, 8
     src, dst = synth.rmat(18, n, E, 4321, symmetric=False)
     Wx = synth.normal_f32((n, H * C), 4322)

@@ -46,8 +46,8 @@ def test_csr_bit_exact_full_size(big):
 
 @pytest.mark.parametrize("dtype,F", [("bf16", 128), ("f32", 32), ("f32", 512), ("bf16", 512), ("f32", 256), ("bf16", 64), ("bf16", 256)])
 def test_propagate_sampled_rows_full_size(big, dtype, F):
-    """Every launch shape the benchmark times at this size: narrow and 512-byte rows on the row-walking kernel,
-    and the column-slab passes (two for 1024-byte rows: bf16 F=512, f32 F=256; four for f32 F=512)."""
+    """Every launch shape the benchmark times at this size: narrow and 512-byte rows, and the
+    column-slab passes (two for 1024-byte rows: bf16 F=512, f32 F=256; four for f32 F=512)."""
     import torch
     gnn, wl, g = big
     n, src, dst, w, seed = wl["N"], wl["src"], wl["dst"], wl["w"], wl["seed"]
@@ -80,8 +80,7 @@ def test_propagate_sampled_rows_full_size(big, dtype, F):
 
 
 def test_mean_max_and_backward_of_max_full_size(big):
-    """The row-walking kernel's other modes at a size where it (not the position-first kernel) runs:
-    mean on sampled rows, max with winner positions on every row (bit-exact), routing backward on sampled rows."""
+    """The other modes at full size: mean on sampled rows, max with winner positions on every row (bit-exact), routing backward on sampled rows."""
     import torch
     from util import bits, f64_to_dtype_bits
     gnn, wl, g = big

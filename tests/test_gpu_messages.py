@@ -31,7 +31,7 @@ def absval(a):
     return (a & np.uint16(0x7FFF)) if a.dtype == np.uint16 else np.abs(a)
 
 
-# rows up to 512 bytes take the position-first kernel on these graphs, wider rows the row-walking one
+# rows of one column slab and of several
 SUB_SHAPES = [("f32", 64), ("f32", 256), ("bf16", 32), ("bf16", 128), ("bf16", 1024)]
 
 
@@ -98,8 +98,7 @@ def test_edge_factors_per_head_and_per_feature(gnn, dtype, F, H, width, op):
 
 
 def test_edge_factors_on_the_row_walking_kernel_for_narrow_rows(gnn):
-    """Narrow rows reach the row-walking kernel only on graphs of 8 Mi edges and more: per-feature and per-head
-    factors there, sampled against the checker on the rows of a node subset."""
+    """Narrow rows on a graph of more than 8 Mi edges: per-feature and per-head factors there, sampled against the checker on the rows of a node subset."""
     n, e = 60_000, 8_500_000
     rng = np.random.default_rng(77)
     src = rng.integers(0, n, e).astype(np.int32)
@@ -117,7 +116,7 @@ def test_edge_factors_on_the_row_walking_kernel_for_narrow_rows(gnn):
             ev = synth.uniform_f32((e, ew), -1.0, 1.0, 14 + ew)
             out = gnn.propagate_msg(g, gnn.E_MUL_XJ, to_dev(X), e_csr=to_dev(ev[eid]), op="sum")
             o, S, _ = oracle.propagate_msg(oracle.E_MUL_XJ, "sum", n, src[keep], dst[keep], X, e=ev[keep])
-            assert_close(to_host64(out)[rows], o[rows], S[rows], "bf16", f"width {ew} on the row-walking kernel")
+            assert_close(to_host64(out)[rows], o[rows], S[rows], "bf16", f"width {ew} on a large graph")
     finally:
         oracle.set_threads(1)
 

@@ -266,8 +266,8 @@ def test_propagate_max_min_bit_exact(gnn, dtype, F, op):
 @pytest.mark.parametrize("op", ["max", "min"])
 def test_propagate_weighted_max_min(gnn, dtype, F, op):
     """e_mul_xj with max/min: the message w*x is rounded once to fp32 and compared in fp32 (the checker does
-    the same), so values and winners are bit-exact; signed weights, both kernels (rows up to 512 bytes take the
-    position-first kernel here, wider rows the row-walking one); then the routing backward with the weights."""
+    the same), so values and winners are bit-exact; signed weights, rows of one column slab and of
+    several; then the routing backward with the weights."""
     n, src, dst = ragged_graph(50 + F)
     g = build_graph(gnn, n, src, dst)
     ref = host_csr(n, src, dst)
@@ -472,8 +472,8 @@ def test_chunk_regimes_with_empty_rows_everywhere(gnn, e, dtype, F):
 @pytest.mark.parametrize("dtype,F", [("bf16", 64), ("f32", 16), ("bf16", 512)])
 def test_long_runs_of_rows_without_edges(gnn, dtype, F):
     """A bipartite-like graph: 200000 nodes of which only 2000 in the middle receive edges, with one more
-    run of 40000 empty rows between two of them.  Both the short-row kernel (F*s <= 512 bytes) and the
-    row-walking kernel (wider rows) must jump over the runs and still zero every empty row."""
+    run of 40000 empty rows between two of them.  Rows of one column slab and of several: the
+    row lookup must jump over the runs and every empty row still be zeroed."""
     n, e = 200_000, 50_000
     rng = np.random.default_rng(F)
     dst = rng.integers(90_000, 92_000, e).astype(np.int32)
@@ -505,8 +505,7 @@ def test_long_runs_of_rows_without_edges(gnn, dtype, F):
 
 @pytest.mark.parametrize("dtype,F", [("bf16", 32), ("f32", 64), ("f32", 128), ("bf16", 128)])
 def test_low_mean_degree_above_8mi_edges_takes_positions_first(gnn, dtype, F):
-    """Graphs of 8 Mi edges and more whose mean degree is a handful run sums on one-slab chunks (positions first)
-    instead of the row walk: forward sum, mean and the backward of the mean, on sampled rows, with a hub cut by
+    """Graphs of 8 Mi edges and more whose mean degree is a handful run positions first: forward sum, mean and the backward of the mean, on sampled rows, with a hub cut by
     hundreds of chunks, rows without edges and a ragged last chunk."""
     import torch
     n, e = 2_300_000, 8_600_037
