@@ -475,7 +475,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
                 S.head[lane * EPC + j] = acc[j];
                 if (ARG) S.head_a[ARG ? lane * EPC + j : 0] = arg[ARG ? j : 0];
             }
-        } else if (col_lane && S.row[q] >= 0) {
+        } else if (col_lane) {
             finish_row<T, MODE, EPI>(P, S.row[q], S.start[q + 1] - S.start[q], ci, acc, arg);
         }
         clear();
@@ -670,7 +670,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
                 if (before) {
                     head_state = HEAD_CLOSED;
                     leave(S.head, S.head_a, carry, carg);
-                } else if (lane < LPR && col_lane && S.row[hq] >= 0) {
+                } else if (lane < LPR && col_lane) {
                     finish_row<T, MODE, EPI>(P, S.row[hq], S.start[hq + 1] - S.start[hq], ci, carry, carg);
                 }
                 have = before = false;
