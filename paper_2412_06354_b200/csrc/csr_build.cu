@@ -569,7 +569,10 @@ __global__ void add_self_loops_kernel(int32_t N, int64_t E, const int32_t* src,
     int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (; k < E + N; k += stride) {
-        if (k < E) { so[k] = src[k]; dout[k] = dst[k]; }
+        if (k < E) {
+            const int32_t s = src[k], d = dst[k];
+            so[k] = s; dout[k] = d;
+        }
         else { so[k] = (int32_t)(k - E); dout[k] = (int32_t)(k - E); }
     }
 }

@@ -176,16 +176,10 @@ __global__ void __launch_bounds__(256) aggregate_backward_kernel(const int64_t* 
     struct Row { uint4 v, win[EPC / 4]; float deg; };
     for (int ci = lane % lpr; ci < nvec; ci += lpr) {
         auto load = [&](int q, Row& R) {
-            if (row[q] < 0) {  // positions of no row: zero
-                R.v = make_uint4(0u, 0u, 0u, 0u);
-                R.deg = 1.f;
-#pragma unroll
-                for (int j = 0; j < EPC / 4; ++j) R.win[j] = make_uint4(~0u, ~0u, ~0u, ~0u);
-                return;
-            }
-            const size_t from = (size_t)row[q] * nvec + ci;
+            const int r = max(row[q], 0);
+            const size_t from = (size_t)r * nvec + ci;
             R.v = ld_16(dOut + from);
-            if (op == GNN_MEAN) R.deg = (float)(rowptr[row[q] + 1] - rowptr[row[q]]);
+            if (op == GNN_MEAN) R.deg = (float)(rowptr[r + 1] - rowptr[r]);
             if (route) {
 #pragma unroll
                 for (int j = 0; j < EPC / 4; ++j) {
@@ -208,6 +202,7 @@ __global__ void __launch_bounds__(256) aggregate_backward_kernel(const int64_t* 
                 for (int j = 0; j < EPC; ++j) x[j] = x[j] / R.deg;
                 R.v = Chunk<T>::pack(x);
             }
+            if (row[q] < 0) R.v = make_uint4(0u, 0u, 0u, 0u);  // positions of no row (not where they are loaded: it would wait)
             for (; p < e; ++p) {
                 uint4 v = R.v;
                 if (route) {  // zero where another position won

@@ -114,19 +114,30 @@ __global__ void __launch_bounds__(EB_THREADS) epilogue_backward_kernel(const uin
 #pragma unroll
     for (int j = 0; j < EPC; ++j) acc[j] = 0.f;
     if (active) {
-#pragma unroll 4
-        for (int64_t r = r0 + grp; r < r1; r += groups) {
-            float d[EPC];
-            Chunk<T>::unpack(dY[(size_t)r * nvec + ci], d);
-            if (relu) {
-                float y[EPC];
-                Chunk<T>::unpack(Y[(size_t)r * nvec + ci], y);
+        constexpr int U = 4;  // rows whose loads are in flight together
+        for (int64_t r = r0 + grp; r < r1; r += U * groups) {
+            uint4 dr[U], yr[U];
 #pragma unroll
-                for (int j = 0; j < EPC; ++j) d[j] = y[j] > 0.f ? d[j] : 0.f;
+            for (int u = 0; u < U; ++u)
+                if (r + u * groups < r1) {
+                    dr[u] = dY[(size_t)(r + u * groups) * nvec + ci];
+                    if (relu) yr[u] = Y[(size_t)(r + u * groups) * nvec + ci];
+                }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                if (r + u * groups >= r1) break;
+                float d[EPC];
+                Chunk<T>::unpack(dr[u], d);
+                if (relu) {
+                    float y[EPC];
+                    Chunk<T>::unpack(yr[u], y);
+#pragma unroll
+                    for (int j = 0; j < EPC; ++j) d[j] = y[j] > 0.f ? d[j] : 0.f;
+                }
+                if (dZ) dZ[(size_t)(r + u * groups) * nvec + ci] = Chunk<T>::pack(d);
+#pragma unroll
+                for (int j = 0; j < EPC; ++j) acc[j] += d[j];
             }
-            if (dZ) dZ[(size_t)r * nvec + ci] = Chunk<T>::pack(d);
-#pragma unroll
-            for (int j = 0; j < EPC; ++j) acc[j] += d[j];
         }
     }
     if (!partial) return;
