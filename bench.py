@@ -49,31 +49,31 @@ TRAFFIC_SOURCE = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --cl
                   "full-size traffic (better L2 reuse on the reduced matrix); profiles/dram_bytes_of_the_sweep_reduced_graph.md")
 TRAFFIC_SCALE = 4.0
 TRAFFIC_KERNEL_FILES = ("propagate.cu", "propagate.cuh", "reduce_params.cuh", "reduce_rows.cuh", "common.cuh")
-TRAFFIC_KERNEL_SHA256 = "5d69e557b823263b90bb7e11d40498844044dfb1e9657da586e83fb64c52592a"
+TRAFFIC_KERNEL_SHA256 = "e9d423fe4f03d42e050e45b1e7f22d5688c799216b726aef0f97073d0a97eea1"
 TRAFFIC_GB_REDUCED = {
     "32:bf16:copy_xj:fwd": 0.209,
     "32:bf16:copy_xj:bwd": 0.209,
     "32:bf16:e_mul_xj:fwd": 0.35,
-    "32:bf16:e_mul_xj:bwd": 0.349,
+    "32:bf16:e_mul_xj:bwd": 0.35,
     "64:bf16:copy_xj:fwd": 0.294,
     "64:bf16:copy_xj:bwd": 0.294,
     "64:bf16:e_mul_xj:fwd": 0.444,
-    "64:bf16:e_mul_xj:bwd": 0.445,
+    "64:bf16:e_mul_xj:bwd": 0.446,
     "128:bf16:copy_xj:fwd": 0.644,
     "128:bf16:copy_xj:bwd": 0.645,
-    "128:bf16:e_mul_xj:fwd": 0.821,
-    "128:bf16:e_mul_xj:bwd": 0.822,
-    "256:bf16:copy_xj:fwd": 2.042,
-    "256:bf16:copy_xj:bwd": 2.041,
+    "128:bf16:e_mul_xj:fwd": 0.82,
+    "128:bf16:e_mul_xj:bwd": 0.823,
+    "256:bf16:copy_xj:fwd": 2.043,
+    "256:bf16:copy_xj:bwd": 2.04,
     "256:bf16:e_mul_xj:fwd": 2.265,
-    "256:bf16:e_mul_xj:bwd": 2.264,
-    "512:bf16:copy_xj:fwd": 4.085,
+    "256:bf16:e_mul_xj:bwd": 2.263,
+    "512:bf16:copy_xj:fwd": 4.087,
     "512:bf16:copy_xj:bwd": 4.086,
-    "512:bf16:e_mul_xj:fwd": 4.532,
-    "512:bf16:e_mul_xj:bwd": 4.529,
+    "512:bf16:e_mul_xj:fwd": 4.533,
+    "512:bf16:e_mul_xj:bwd": 4.528,
     "32:f32:copy_xj:fwd": 0.287,
-    "32:f32:copy_xj:bwd": 0.287,
-    "32:f32:e_mul_xj:fwd": 0.436,
+    "32:f32:copy_xj:bwd": 0.288,
+    "32:f32:e_mul_xj:fwd": 0.437,
     "32:f32:e_mul_xj:bwd": 0.438,
     "64:f32:copy_xj:fwd": 0.628,
     "64:f32:copy_xj:bwd": 0.629,
@@ -83,14 +83,14 @@ TRAFFIC_GB_REDUCED = {
     "128:f32:copy_xj:bwd": 1.991,
     "128:f32:e_mul_xj:fwd": 2.177,
     "128:f32:e_mul_xj:bwd": 2.175,
-    "256:f32:copy_xj:fwd": 3.994,
-    "256:f32:copy_xj:bwd": 3.993,
+    "256:f32:copy_xj:fwd": 3.992,
+    "256:f32:copy_xj:bwd": 3.992,
     "256:f32:e_mul_xj:fwd": 4.363,
     "256:f32:e_mul_xj:bwd": 4.359,
-    "512:f32:copy_xj:fwd": 7.982,
-    "512:f32:copy_xj:bwd": 7.986,
+    "512:f32:copy_xj:fwd": 7.979,
+    "512:f32:copy_xj:bwd": 7.984,
     "512:f32:e_mul_xj:fwd": 8.719,
-    "512:f32:e_mul_xj:bwd": 8.721,
+    "512:f32:e_mul_xj:bwd": 8.723,
 }
 TRAFFIC_GB = {k: v * TRAFFIC_SCALE for k, v in TRAFFIC_GB_REDUCED.items()}
 
