@@ -25,20 +25,21 @@ enum { EDGE_DOT = 0, EDGE_DOT_MEAN = 1, EDGE_GATV2 = 2 };
 // ------------------------------------------------------------------ rows of up to 512 bytes
 // Positions first, as in the segmented reduction: a warp stages the gathered rows' indices of its share of positions and
 // the rows they lie in; each of its lane groups streams a run of them with four to eight gathers in flight (two register
-// buffers, each refilled as soon as it is used).  The row's own chunk stays in registers while the row lasts (its end is
-// marked in the sign bit of the staged index), the next row's is fetched meanwhile.  The lanes' shares of four positions
+// buffers, each refilled as soon as it is used).  The row's own chunk stays in registers while the row lasts (row ends
+// are bits; a batch of positions without one has nothing to test), the next row's is fetched meanwhile.  The lanes' shares of four positions
 // are folded together: two levels halve the values a lane carries, the rest reduce the one left (32 lanes: 6 shuffles per
 // four positions instead of 20).
 // Bound by instruction issue for narrow rows and by the gathers (L2 -> SM) for rows of 512 bytes.  Before (4 positions per
 // batch, one batch after the other, 8-byte entries, the row's chunk loaded when it changes) -> now:
-//   100k nodes / 1.6 M edges, 512-byte rows, 8 heads bf16 150 -> 116 us; 123 M edges, 128-byte bf16 rows 2.86 -> 2.49 ms;
-//   GATv2 logits of 100k nodes / 1.6 M edges, 512-byte fp32 rows (a gather per index load, four at a time) 358 -> 119 us.
+//   100k nodes / 1.6 M edges, 512-byte rows, 8 heads bf16 150 -> 105 us; 123 M edges, 128-byte bf16 rows 2.86 -> 2.4 ms;
+//   GATv2 logits of 100k nodes / 1.6 M edges, 512-byte fp32 rows (a gather per index load, four at a time) 358 -> 113 us.
 constexpr int ED_SUB = 256;  // most positions per warp
 constexpr int ED_H = 4;      // positions per register buffer
 
 template <bool MEAN>
 struct EdgeStage {
-    alignas(16) int col[ED_SUB + 32];  // gathered row; sign bit: last position of a row; four words further for every lane group before it
+    alignas(16) int col[ED_SUB + 32];  // gathered row; four words further for every lane group before it
+    uint32_t ends[ED_SUB / 32];        // a bit per position: the last one of its row
     int row[ED_SUB + 1];       // [q] the q-th row with positions in the warp's share
     uint16_t start[ED_SUB + 2];
     float inv[MEAN ? ED_SUB + 1 : 1];  // [q] 1 / length of that row
@@ -61,6 +62,7 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
     // skewed as in the segmented reduction: the groups' runs are in different banks, and four entries are one load
     const int L = P.sub / NG, lsh = 31 - __clz(L);
     auto sk = [&](int i) { return i + ((i >> lsh) << 2); };
+    if (lane < ED_SUB / 32) S.ends[lane] = 0u;
     for (int i = lane; i < n; i += 32)
         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(S.col + sk(i))), "l"(P.col + cs + i) : "memory");
     bool began_before;
@@ -69,7 +71,7 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
     __syncwarp();
     for (int q = lane; q < m; q += 32) {
         const int e = S.start[q + 1];
-        if (e <= n) S.col[sk(e - 1)] |= (int)0x80000000;
+        if (e <= n) atomicOr(S.ends + ((e - 1) >> 5), 1u << ((e - 1) & 31));
         if (MEAN) {
             const int r = max(S.row[q], 0);
             S.inv[MEAN ? q : 0] = 1.0f / (float)(P.rowptr[r + 1] - P.rowptr[r]);
@@ -113,22 +115,15 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
     };
     for (int i = n + lane; i < P.sub; i += 32) S.col[sk(i)] = 0;  // the last warp: positions past the end gather row 0
     __syncwarp();
-    auto issue = [&](uint4* x, int i) -> unsigned {
-        unsigned ends = 0;
+    auto issue = [&](uint4* x, int i) {
         const int4 c4 = V2 ? make_int4(Sc[i], Sc[i + 1], Sc[i + 2], Sc[i + 3]) : *reinterpret_cast<const int4*>(Sc + i);
         const int ccs[H] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
-        for (int u = 0; u < H; ++u) {
-            const int cc = ccs[u];
-            ends |= ((unsigned)cc >> 31) << u;
-            x[u] = ld_hint16(Xl + (size_t)(uint32_t)(cc & 0x7fffffff) * row_bytes, pol_keep);
-        }
-        return ends;
+        for (int u = 0; u < H; ++u) x[u] = ld_hint16(Xl + (size_t)(uint32_t)ccs[u] * row_bytes, pol_keep);
     };
     auto use = [&](const uint4* xr, unsigned ends, int i) {
         float dot[H], scale[MEAN ? H : 1];
-#pragma unroll
-        for (int u = 0; u < H; ++u) {
+        auto one = [&](int u) {
             float x[EPC], t = 0.f, t1 = 0.f;
             Chunk<T>::unpack(xr[u], x);
 #pragma unroll
@@ -143,9 +138,18 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
             }
             dot[u] = col_lane ? t + t1 : 0.f;
             if (MEAN) scale[MEAN ? u : 0] = sc;
-            if (ends >> u & 1u) next_row();
+        };
+        if (V2 || __any_sync(0xffffffffu, ends != 0)) {  // (GATv2: two copies of the loop spill)
+#pragma unroll
+            for (int u = 0; u < H; ++u) {
+                one(u);
+                if (ends >> u & 1u) next_row();
+            }
+            __syncwarp();
+        } else {  // most positions of a skewed graph lie in long rows: nothing to test
+#pragma unroll
+            for (int u = 0; u < H; ++u) one(u);
         }
-        __syncwarp();
         if (span >= 4) {
             const int h1 = span >> 1, h2 = span >> 2;
             const bool up1 = (li & h1) != 0, up2 = (li & h2) != 0;
@@ -170,14 +174,16 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
     };
     // same trip count in every group (the shuffles are warp-wide); L is a multiple of 2 H
     uint4 A[H], B[H];
-    unsigned ea = issue(A, a), eb = issue(B, a + H);
+    issue(A, a);
+    issue(B, a + H);
 #pragma unroll 1
     for (int i = a; i < a + L; i += 2 * H) {
         const bool more = i + 2 * H < a + L;
-        use(A, ea, i);
-        if (more) ea = issue(A, i + 2 * H);
-        use(B, eb, i + H);
-        if (more) eb = issue(B, i + 3 * H);
+        const unsigned ends = S.ends[i >> 5] >> (i & 31);
+        use(A, ends & ((1u << H) - 1u), i);
+        if (more) issue(A, i + 2 * H);
+        use(B, (ends >> H) & ((1u << H) - 1u), i + H);
+        if (more) issue(B, i + 3 * H);
     }
 }
 

@@ -29,7 +29,8 @@ extern template void launch_reduce_others<__nv_bfloat16>(const PropParams&, int,
 template <typename T>
 static void launch_mode(const PropParams& P, int mode, bool stream, cudaStream_t st) {
     if (mode == MODE_SUM && (P.w || P.gscale_rowptr)) mode = MODE_WSUM;
-    if (mode == MODE_SUM || mode == MODE_WSUM || mode == MODE_HEADSUM) launch_reduce_sums<T>(P, mode, stream, st);
+    if (mode == MODE_HEADSUM && (P.gscale_rowptr || P.epi_l)) mode = P.epi_l ? MODE_HEADRANK : MODE_HEADSUM_W;
+    if (mode == MODE_SUM || mode == MODE_WSUM || mode == MODE_HEADSUM || mode == MODE_HEADSUM_W || mode == MODE_HEADRANK) launch_reduce_sums<T>(P, mode, stream, st);
     else launch_reduce_others<T>(P, mode, stream, st);
 }
 
@@ -66,6 +67,11 @@ static int warp_positions(int32_t N, int64_t E, int row_bytes, bool stream) {
     return E >= 256 * 1024 ? 128 : E >= 128 * 1024 || narrowest <= 64 ? 64 : 32;
 }
 
+// Mean row length from which the reduction looks whether a batch of positions holds a row end at all before it tests each
+// (lane groups side by side; a warp-wide row always does).  123 M edges, 51 per row, 128-byte rows: 1.96 -> 1.87 ms; 1.36 M edges, 8
+// per row, 256-byte rows, where hardly a batch is without one: 2 % slower.
+constexpr int VOTE_DEGREE = 24;
+
 // Room for a partial row per 64, 128 or 1024 positions.  The streaming kernel, whose pieces are 256 to 2048 positions, needs a
 // sixteenth to a quarter of that below 4 Mi edges and half above; the size is what callers have been told since the first
 // version, and what decides which problems the built-in scratch takes.
@@ -98,6 +104,7 @@ gnn_status run_gatv2_rows(const char* who, int32_t N, int64_t E, const int64_t* 
     const ReduceWs w = carve(ws, P.npieces, F, false);
     P.tail_row = w.tail_row; P.part_val = w.part_val;
     P.wh = ds; P.wh_index = ds_index; P.H = H; P.fph = F / H; P.epi_a = a;
+    P.vote = E > VOTE_DEGREE * (int64_t)N;
     P.v2_self = Xself; P.slope = slope; P.da_part = da_part;
     if (dtype == GNN_F32) launch_gatv2_rows<float>(P, st);
     else launch_gatv2_rows<__nv_bfloat16>(P, st);
@@ -126,6 +133,7 @@ gnn_status run_chunked(const char* who, int mode, int32_t N, int64_t E, const in
     P.rowptr = rowptr; P.col = col; P.w = w; P.argmax = argmax;
     P.gscale_rowptr = gscale_rowptr; P.route_arg = route_arg; P.route_pos = route_pos;
     P.N = N; P.E = E; P.mean = mean; P.arg_ld = F;
+    P.vote = E > VOTE_DEGREE * (int64_t)N;
     P.v2_self = nullptr; P.slope = 0.f; P.da_part = nullptr;
     P.wh = nullptr; P.wh_index = nullptr; P.H = 1; P.fph = F; P.epi_l = P.epi_r = P.epi_a = P.epi_b = nullptr;
     if (hx) {

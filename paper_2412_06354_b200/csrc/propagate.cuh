@@ -4,7 +4,7 @@
 
 namespace gnn {
 
-enum { MODE_SUM = 0, MODE_MAX = 1, MODE_MIN = 2, MODE_ROUTE = 3, MODE_HEADSUM = 4, MODE_EFSUM = 5, MODE_WSUM = 6, MODE_V2 = 7 };
+enum { MODE_SUM = 0, MODE_MAX = 1, MODE_MIN = 2, MODE_ROUTE = 3, MODE_HEADSUM = 4, MODE_EFSUM = 5, MODE_WSUM = 6, MODE_V2 = 7, MODE_HEADSUM_W = 8, MODE_HEADRANK = 9 };
 
 // MODE_HEADSUM extras: multipliers per (position, head) and an optional rank-1 row epilogue
 //   out[r,f] += epi_l[r,h(f)] * epi_a[f] + epi_r[r,h(f)] * epi_b[f]

@@ -28,8 +28,14 @@ __device__ __forceinline__ bool beats(float cv, int32_t ca, float v, int32_t a) 
 
 // Everything between the reduced values of a row and its stored 16-byte column ci (of the slab): division of the mean,
 // rank-1 epilogue of the per-head mode and row epilogue (only with EPI), rounding, winners.
-template <typename T, int MODE, bool EPI>
-__device__ __forceinline__ void finish_row(const PropParams& P, int row, int64_t len, int ci, float* v, const int32_t* a) {
+// r1 (READY): the rank-1 epilogue's factors, which the caller has at hand; loaded here, where the row ends, they are waited for
+// once per row.
+struct RankOne {
+    float l, r;          // this row's and head's
+    const float *a, *b;  // this column's, in shared memory
+};
+template <typename T, int MODE, bool EPI, bool READY = false>
+__device__ __forceinline__ void finish_row(const PropParams& P, int row, int64_t len, int ci, float* v, const int32_t* a, const RankOne& r1 = RankOne()) {
     constexpr int EPC = Chunk<T>::N;
     constexpr bool ARG = MODE == MODE_MAX || MODE == MODE_MIN;
     if (P.mean) {
@@ -41,7 +47,16 @@ __device__ __forceinline__ void finish_row(const PropParams& P, int row, int64_t
 #pragma unroll
         for (int j = 0; j < EPC; ++j) v[j] *= P.epi_a[ci * EPC + j];
     }
-    if (EPI && MODE == MODE_HEADSUM && P.epi_l) {
+    if (READY) {
+#pragma unroll
+        for (int j = 0; j < EPC; j += 4) {
+            const float4 x = *reinterpret_cast<const float4*>(r1.a + j), y = *reinterpret_cast<const float4*>(r1.b + j);
+            v[j] += r1.l * x.x + r1.r * y.x;
+            v[j + 1] += r1.l * x.y + r1.r * y.y;
+            v[j + 2] += r1.l * x.z + r1.r * y.z;
+            v[j + 3] += r1.l * x.w + r1.r * y.w;
+        }
+    } else if (MODE == MODE_HEADRANK) {
         const int f0 = (P.vec0 + ci) * EPC, h = f0 / P.fph;  // a 16-byte chunk lies inside one head
         const float el = P.epi_l[(size_t)row * P.H + h], er = P.epi_r[(size_t)row * P.H + h];
 #pragma unroll
@@ -84,8 +99,9 @@ __device__ __forceinline__ void finish_row(const PropParams& P, int row, int64_t
 template <typename T, int LPR, int MODE>
 struct RowReducer {
     static constexpr int EPC = Chunk<T>::N, NG = 32 / LPR;
-    static constexpr bool ARG = MODE == MODE_MAX || MODE == MODE_MIN, EF = MODE == MODE_EFSUM, HEAD = MODE == MODE_HEADSUM, ROUTE = MODE == MODE_ROUTE;
-    static constexpr bool PLAIN = MODE == MODE_SUM;  // no multiplier at all (MODE_WSUM: one per position)
+    static constexpr bool ARG = MODE == MODE_MAX || MODE == MODE_MIN, EF = MODE == MODE_EFSUM, ROUTE = MODE == MODE_ROUTE;
+    static constexpr bool HEAD = MODE == MODE_HEADSUM || MODE == MODE_HEADSUM_W || MODE == MODE_HEADRANK;
+    static constexpr bool PLAIN = MODE == MODE_SUM || MODE == MODE_HEADSUM || MODE == MODE_HEADRANK;  // no multiplier per position (MODE_WSUM, MODE_HEADSUM_W: one)
     static constexpr int U = 4;  // gathers in flight per lane
     static constexpr int MW = EF ? EPC : 1;
 
@@ -184,12 +200,11 @@ struct RowReducer {
 #pragma unroll
                     for (int k = 0; k < EPC; k += 2)
                         fma2(acc[k], acc[k + 1], x[k], x[k + 1], hw[EF ? u : 0][EF ? k : 0] * w, hw[EF ? u : 0][EF ? k + 1 : 0] * w);
-                } else if (PLAIN) {
+                } else if (PLAIN && !HEAD) {
 #pragma unroll
                     for (int k = 0; k < EPC; k += 2) add2(acc[k], acc[k + 1], x[k], x[k + 1]);
                 } else {
-                    // w = 1 in the per-head mode unless the gathered rows are rescaled (backward of the mean)
-                    const float m = HEAD ? hw[HEAD ? u : 0][0] * w : w;
+                    const float h = hw[HEAD ? u : 0][0], m = !HEAD ? w : PLAIN ? h : h * w;
 #pragma unroll
                     for (int k = 0; k < EPC; k += 2) fma2(acc[k], acc[k + 1], x[k], x[k + 1], m, m);
                 }
@@ -305,7 +320,7 @@ reduce_rows_kernel(const __grid_constant__ PropParams P, int long_blocks) {
 // ------------------------------------------------------------------ positions first
 // One warp per run of P.sub consecutive positions, a block per piece of RR_WARPS such runs.  The gathers do not depend on the rows: every lane group streams
 // sub/NG of them with four to eight gathers always in flight (two register buffers of H, each refilled as soon
-// as it has been added), and a row's end, marked in the sign bit of the staged index of its last position, only makes the
+// as it has been added), and a row's end, a bit per position, only makes the
 // accumulator go out.  Rows cut between lane groups are stitched inside the warp, rows cut between warps inside the block
 // (through shared memory, by the warp in which they begin), both in position order; rows cut by the piece leave the
 // partials that the second kernel adds (a piece per warp: that kernel took 313 us of 4.9 ms on 123 M edges).  Rows without edges are written by a scan that is spread over all warps.
@@ -315,17 +330,20 @@ reduce_rows_kernel(const __grid_constant__ PropParams P, int long_blocks) {
 // warps per SM), buffers refilled in turn instead of one batch after the other, an epilogue-free row end: fp32 sums over
 // 512-byte rows 113 -> 75 us, bf16 256-byte 74 -> 60 us, 64-byte 54 -> 32 us, max fp32 157 -> 117 us; on 123 M edges the
 // 128-byte rows of a weighted sum 2.45 -> 2.26 ms, max over 256-byte rows 8.1 -> 6.6 ms.
+// Row ends as bits beside the indices instead of in their sign: no index to mask, and a batch without an end has nothing to
+// test: 123 M edges, 128-byte bf16 rows 1.96 -> 1.87 ms, sums over 512 fp32 features 37.9 -> 35.4 ms a forward and backward pass.
 constexpr int RS_SUB = 256;  // most positions per warp
 constexpr int RS_SKEW = 32;
 
 template <int EPC, bool HAS_W, bool HAS_T, bool ARG>
 struct alignas(16) StreamStage {
     // per position; four words further for every lane group before the position's (see sk)
-    int col[RS_SUB + RS_SKEW];                         // gathered row; sign bit: last position of a row
+    int col[RS_SUB + RS_SKEW];                         // gathered row
     alignas(16) float w[HAS_W ? RS_SUB + RS_SKEW : 1]; // multiplier
     alignas(16) int t[HAS_T ? RS_SUB + RS_SKEW : 1];   // ROUTE: forward position; HEAD: row of the multiplier matrix
     int row[RS_SUB + 1];                   // [q] the q-th row with positions in the warp's share
     uint16_t start[RS_SUB + 2];            // [q] its first position in the warp's share; [count]: end of the last, or n + 1 if it is cut
+    uint32_t ends[RS_SUB / 32];            // a bit per position: the last one of its row
     float head[32 * EPC];                  // per lane: sum of a group's (then the warp's) first row, which began before it
     int32_t head_a[ARG ? 32 * EPC : 1];
     // the warp's last row, if it goes on past the warp: over col and w, which are done with by then
@@ -335,20 +353,21 @@ struct alignas(16) StreamStage {
 // what a warp leaves to the block: its first row began in an earlier warp and ends here (CLOSED) or does not (THROUGH)
 enum { HEAD_NONE = 0, HEAD_CLOSED = 1, HEAD_THROUGH = 2 };
 
-template <int MODE>
+template <typename T, int MODE, bool EPI>
 __host__ __device__ constexpr int rs_min_blocks() {
-    return (MODE == MODE_SUM || MODE == MODE_WSUM) ? 4 : 3;
+    return (MODE == MODE_SUM || MODE == MODE_WSUM) ? 4 : MODE == MODE_V2 && EPI && sizeof(T) == 2 ? 2 : 3;  // (three: 170 bytes of spills)
 }
 
 template <typename T, int LPR, int MODE, bool EPI>
-__global__ void __launch_bounds__(RR_WARPS * 32, (rs_min_blocks<MODE>()))
+__global__ void __launch_bounds__(RR_WARPS * 32, (rs_min_blocks<T, MODE, EPI>()))
 stream_rows_kernel(const __grid_constant__ PropParams P) {
     constexpr int EPC = Chunk<T>::N, NG = 32 / LPR;
-    constexpr bool ARG = MODE == MODE_MAX || MODE == MODE_MIN, EF = MODE == MODE_EFSUM, HEAD = MODE == MODE_HEADSUM || MODE == MODE_V2, ROUTE = MODE == MODE_ROUTE;
+    constexpr bool ARG = MODE == MODE_MAX || MODE == MODE_MIN, EF = MODE == MODE_EFSUM, ROUTE = MODE == MODE_ROUTE;
+    constexpr bool RANK1 = MODE == MODE_HEADRANK, HEAD = MODE == MODE_HEADSUM || MODE == MODE_HEADSUM_W || RANK1 || MODE == MODE_V2;
     constexpr bool PLAIN = MODE == MODE_SUM, V2 = MODE == MODE_V2, DA = V2 && EPI;
     constexpr int H = (ROUTE || EF) ? 2 : 4;  // positions per register buffer
     constexpr int MW = EF ? EPC : 1;
-    constexpr bool HAS_W = !PLAIN && !V2;  // a multiplier per position
+    constexpr bool HAS_W = !PLAIN && !V2 && MODE != MODE_HEADSUM && !RANK1;  // a multiplier per position
     using Stage = StreamStage<EPC, HAS_W, ROUTE || HEAD, ARG>;
     static_assert(32 * EPC <= RS_SUB, "a row's sums fit over the staged indices");
     extern __shared__ __align__(16) unsigned char rs_smem[];
@@ -367,6 +386,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     // words of skew per group keep the runs apart and on 16 bytes, so that a register buffer's entries are one load.
     const int L = P.sub / NG, lsh = 31 - __clz(L);
     auto sk = [&](int i) { return i + ((i >> lsh) << 2); };
+    if (lane < RS_SUB / 32) S.ends[lane] = 0u;
     {  // ---- indices and multipliers, asynchronously while the rows are looked up
         auto copy = [&](void* dst, const void* src) {
             asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
@@ -403,12 +423,14 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     }
     for (int q = lane; q < m; q += 32) {
         const int e = S.start[q + 1];
-        if (e <= n) S.col[sk(e - 1)] |= (int)0x80000000;
+        if (e <= n) atomicOr(S.ends + ((e - 1) >> 5), 1u << ((e - 1) & 31));
     }
     __syncwarp();
 
     // ---- this group's run
     const int a = g * L, b = min(a + L, n);
+    const bool vote = P.vote && n == P.sub;  // (every group has a run of the same length)
+    auto ends_at = [&](int i) { return (S.ends[i >> 5] >> (i & 31) & 1u) != 0; };
     const int* const Sc = S.col + 4 * g;
     const float* const Sw = S.w + (HAS_W ? 4 * g : 0);
     const int* const St = S.t + (ROUTE || HEAD ? 4 * g : 0);
@@ -452,6 +474,22 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
         }
         q = lo;
     }
+    // the rank-1 epilogue: the attention vectors from shared memory, the row's two factors loaded when it begins
+    float* const ab = reinterpret_cast<float*>(rs_smem + RR_WARPS * sizeof(Stage));  // [2][F]
+    RankOne r1 = {0.f, 0.f, ab + ci * EPC, ab + P.F + ci * EPC};
+    auto row_factors = [&](int qq) {
+        const size_t k = (size_t)max(S.row[qq], 0) * P.H + ((P.vec0 + ci) * EPC) / P.fph;
+        r1.l = ld_f32(P.epi_l + k);
+        r1.r = ld_f32(P.epi_r + k);
+    };
+    if (RANK1) {
+        if (a < b) row_factors(q);
+        for (int f = threadIdx.x; f < P.F; f += RR_WARPS * 32) {
+            ab[f] = P.epi_a[P.vec0 * EPC + f];
+            ab[P.F + f] = P.epi_b[P.vec0 * EPC + f];
+        }
+        __syncthreads();
+    }
     bool open = a < b && (S.start[q] < a || (a == 0 && began_before));  // the run's first row began before the run
     int head_q = -1;
     // MODE_V2: this row's own features, the next row's on their way, and the share of da (all rows of the group together)
@@ -476,10 +514,11 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
                 if (ARG) S.head_a[ARG ? lane * EPC + j : 0] = arg[ARG ? j : 0];
             }
         } else if (col_lane) {
-            finish_row<T, MODE, EPI>(P, S.row[q], S.start[q + 1] - S.start[q], ci, acc, arg);
+            finish_row<T, MODE, EPI, RANK1>(P, S.row[q], S.start[q + 1] - S.start[q], ci, acc, arg, r1);
         }
         clear();
         ++q;
+        if (RANK1 && q < m) row_factors(q);
         if (V2) {
             Chunk<T>::unpack(own_next, xs);
             if (q + 1 < m) own_next = own(q + 1);
@@ -490,9 +529,8 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
         float hw[(HEAD || EF) ? H : 1][MW];
         int4 win[ROUTE ? H : 1][ROUTE ? EPC / 4 : 1];
     };
-    // the gathers of positions i .. i + H - 1; a bit per row end
-    auto issue = [&](Buf& B, int i) -> unsigned {
-        unsigned ends = 0;
+    // the gathers of positions i .. i + H - 1
+    auto issue = [&](Buf& B, int i) {
         alignas(16) int ccs[H], ts[H];
         if (ONE_BY_ONE) {
 #pragma unroll
@@ -503,9 +541,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
         if (HEAD) words(ts, St + (HEAD ? i : 0));
 #pragma unroll
         for (int u = 0; u < H; ++u) {
-            int cc = ccs[u];
-            ends |= ((unsigned)cc >> 31) << u;
-            cc &= 0x7fffffff;
+            const int cc = ccs[u];
             B.x[u] = ld_hint16(Xl + (size_t)(uint32_t)cc * P.x_ld, pol_keep);
             if (HEAD) B.hw[HEAD ? u : 0][0] = ld_f32(wh_l + (size_t)(uint32_t)ts[u] * P.H);
             if (EF) {
@@ -523,7 +559,6 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
                 for (int k = 0; k < EPC / 4; ++k) B.win[ROUTE ? u : 0][ROUTE ? k : 0] = ld_int4(f + k);
             }
         }
-        return ends;
     };
     auto use = [&](const Buf& B, int u, int i, float w, int t) {  // entry u of the buffer, position i of the piece
         float x[EPC];
@@ -564,8 +599,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
                 if (DA) da[DA ? k : 0] = fmaf(d, z, da[DA ? k : 0]);
             }
         } else {
-            // w = 1 in the per-head mode unless the gathered rows are rescaled (backward of the mean)
-            const float f = HEAD ? B.hw[HEAD ? u : 0][0] * w : w;
+            const float h = B.hw[HEAD ? u : 0][0], f = !HEAD ? w : HAS_W ? h * w : h;
 #pragma unroll
             for (int k = 0; k < EPC; k += 2) fma2(acc[k], acc[k + 1], x[k], x[k + 1], f, f);
         }
@@ -575,6 +609,12 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
         alignas(16) int ts[H];
         if (HAS_W && !ONE_BY_ONE) words(reinterpret_cast<int*>(ws), Sw + (HAS_W ? i : 0));
         if (ROUTE) words(ts, St + (ROUTE ? i : 0));
+        // most positions of a skewed graph lie in long rows: without a row end in any group there is nothing to test
+        if (NG == 1 ? ends == 0 : vote && !__any_sync(0xffffffffu, ends != 0)) {
+#pragma unroll
+            for (int u = 0; u < H; ++u) use(B, u, i + u, !HAS_W ? 1.0f : ONE_BY_ONE ? Sw[HAS_W ? i + u : 0] : ws[u], ROUTE ? ts[u] : 0);
+            return;
+        }
 #pragma unroll
         for (int u = 0; u < H; ++u) {
             use(B, u, i + u, !HAS_W ? 1.0f : ONE_BY_ONE ? Sw[HAS_W ? i + u : 0] : ws[u], ROUTE ? ts[u] : 0);
@@ -585,26 +625,25 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
         Buf A, B;
         // L is a multiple of 2 H: only the last piece of the graph has a remainder
         int i = a;
-        unsigned ea = 0, eb = 0;
         if (i + 2 * H <= b) {
-            ea = issue(A, i);
-            eb = issue(B, i + H);
+            issue(A, i);
+            issue(B, i + H);
         }
 #pragma unroll 1
         for (; i + 2 * H <= b; i += 2 * H) {
             const bool more = i + 4 * H <= b;
-            use_all(A, ea, i);
-            if (more) ea = issue(A, i + 2 * H);
-            use_all(B, eb, i + H);
-            if (more) eb = issue(B, i + 3 * H);
+            const unsigned ends = S.ends[i >> 5] >> (i & 31);  // a run starts at a multiple of 2 H
+            use_all(A, ends & ((1u << H) - 1u), i);
+            if (more) issue(A, i + 2 * H);
+            use_all(B, (ends >> H) & ((1u << H) - 1u), i + H);
+            if (more) issue(B, i + 3 * H);
         }
 #pragma unroll 1
         for (; i < b; ++i) {
             // one at a time: entry 0 of a buffer whose other entries repeat it
             Buf R;
-            int cc = Sc[i];
-            const bool end = cc < 0;
-            cc &= 0x7fffffff;
+            const int cc = Sc[i];
+            const bool end = ends_at(i);
             R.x[0] = ld_hint16(Xl + (size_t)(uint32_t)cc * P.x_ld, pol_keep);
             if (HEAD) R.hw[0][0] = ld_f32(wh_l + (size_t)(uint32_t)St[HEAD ? i : 0] * P.H);
             if (EF) {
@@ -621,7 +660,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
         }
     }
     // ---- what the groups leave: a closed head (parked), and the sum of a row that goes on past the group (in acc)
-    const bool rest = a < b && Sc[b - 1] >= 0;
+    const bool rest = a < b && !ends_at(b - 1);
     int head_state = HEAD_NONE, tail_row = -1;
     __syncwarp();
     // the warp's first or last row, as far as it lies here, for the block (lanes below LPR)
@@ -948,9 +987,11 @@ fixup_rows_kernel(const __grid_constant__ PropParams P, int nsimple) {
 template <typename T, int MODE, bool EPI, int L>
 static void launch_width(const PropParams& P, bool stream, cudaStream_t st) {
     if (stream) {
-        constexpr size_t smem = RR_WARPS * sizeof(StreamStage<Chunk<T>::N, MODE != MODE_SUM && MODE != MODE_V2,
-                                                             MODE == MODE_ROUTE || MODE == MODE_HEADSUM || MODE == MODE_V2, MODE == MODE_MAX || MODE == MODE_MIN>);
-        static_assert(smem <= 48 * 1024, "staging fits the default shared memory");
+        constexpr bool rank1 = MODE == MODE_HEADRANK, head = MODE == MODE_HEADSUM || MODE == MODE_HEADSUM_W || MODE == MODE_V2 || rank1;
+        constexpr size_t stages = RR_WARPS * sizeof(StreamStage<Chunk<T>::N, MODE != MODE_SUM && MODE != MODE_V2 && MODE != MODE_HEADSUM && !rank1,
+                                                               MODE == MODE_ROUTE || head, MODE == MODE_MAX || MODE == MODE_MIN>);
+        static_assert(stages + (rank1 ? 2 * 256 * sizeof(float) : 0) <= 48 * 1024, "staging fits the default shared memory");
+        const size_t smem = stages + (rank1 ? 2 * P.F * sizeof(float) : 0);
         launch_overlapped(stream_rows_kernel<T, L, MODE, EPI>, dim3((unsigned)P.npieces), dim3(RR_WARPS * 32), smem, st, P);
     } else if constexpr (MODE != MODE_V2) {
         const int long_blocks = P.E > RR_SHORT ? (int)ceil_div(P.npieces, RR_WARPS) : 0;
@@ -961,8 +1002,9 @@ static void launch_width(const PropParams& P, bool stream, cudaStream_t st) {
 
 template <typename T, int MODE>
 static void launch_reduce(const PropParams& P, bool stream, cudaStream_t st) {
-    const bool epi = MODE == MODE_V2 ? P.da_part != nullptr : P.has_epi || P.epi_l;
-#define GNN_WIDTH(L) epi ? launch_width<T, MODE, true, L>(P, stream, st) : launch_width<T, MODE, false, L>(P, stream, st)
+    constexpr bool EPI = MODE != MODE_HEADRANK;  // (the rank-1 epilogue comes alone)
+    const bool epi = MODE == MODE_V2 ? P.da_part != nullptr : P.has_epi;
+#define GNN_WIDTH(L) epi && EPI ? launch_width<T, MODE, EPI, L>(P, stream, st) : launch_width<T, MODE, false, L>(P, stream, st)
     if (P.nvec <= 4) GNN_WIDTH(4);
     else if (P.nvec <= 8) GNN_WIDTH(8);
     else if (P.nvec <= 16) GNN_WIDTH(16);
@@ -980,7 +1022,9 @@ template <typename T>
 void launch_reduce_sums(const PropParams& P, int mode, bool stream, cudaStream_t st) {
     if (mode == MODE_SUM) launch_reduce<T, MODE_SUM>(P, stream, st);
     else if (mode == MODE_WSUM) launch_reduce<T, MODE_WSUM>(P, stream, st);
-    else launch_reduce<T, MODE_HEADSUM>(P, stream, st);
+    else if (mode == MODE_HEADSUM) launch_reduce<T, MODE_HEADSUM>(P, stream, st);
+    else if (mode == MODE_HEADRANK) launch_reduce<T, MODE_HEADRANK>(P, stream, st);
+    else launch_reduce<T, MODE_HEADSUM_W>(P, stream, st);
 }
 
 template <typename T>
