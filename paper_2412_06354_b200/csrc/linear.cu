@@ -90,35 +90,52 @@ gemm_simt_kernel(const TA* __restrict__ A, int64_t sam, int64_t sak, const TB* _
 }
 
 // out[i] = sum over slabs of part[s][i] in a fixed order: eight contiguous groups of slabs, each summed in ascending order
-// by one thread with eight loads in flight, then added in ascending group order.  32 elements x 8 groups per block
-// (4.7 us for the 148 partials of a 128 x 128 result: 9.7 MB from L2).
-template <typename TC>
-__global__ void __launch_bounds__(256)
+// by one thread with eight loads in flight, then added in ascending group order.  64 elements x 8 groups per block, four
+// elements to a load (V = 4); 32 x 8, one by one, where their number is no multiple of four.  Bound by instruction issue with
+// single loads (61 % issued).
+template <typename TC, int V>
+__global__ void __launch_bounds__(V == 4 ? 128 : 256)
 slab_sum_kernel(const float* part, int slabs, int64_t n, TC* __restrict__ out, int cols, int rows_out, int cols_out, int ld, int c0) {
-    __shared__ float gsum[8][32];
+    constexpr int L = V == 4 ? 16 : 32, E = L * V;
+    __shared__ float gsum[8][E];
     pdl_wait();
-    const int e = threadIdx.x & 31, g = threadIdx.x >> 5;
-    const int64_t i = blockIdx.x * (int64_t)32 + e;
+    const int e = (threadIdx.x % L) * V, g = threadIdx.x / L;
+    const int64_t i = blockIdx.x * (int64_t)E + e;
     const int per = (slabs + 7) / 8, z0 = g * per, z1 = min(slabs, z0 + per);
-    float s = 0.f;
+    float s[V];
+#pragma unroll
+    for (int j = 0; j < V; ++j) s[j] = 0.f;
     if (i < n) {
         for (int z = z0; z < z1; z += 8) {
-            float v[8];
+            float v[8][V];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = z + u < z1 ? part[(size_t)(z + u) * n + i] : 0.f;
+            for (int u = 0; u < 8; ++u) {
+                const float* const p = part + (size_t)(z + u) * n + i;
+                if constexpr (V == 4) {
+                    const float4 q = z + u < z1 ? *reinterpret_cast<const float4*>(p) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    v[u][0] = q.x; v[u][1] = q.y; v[u][2] = q.z; v[u][3] = q.w;
+                } else {
+                    v[u][0] = z + u < z1 ? *p : 0.f;
+                }
+            }
 #pragma unroll
-            for (int u = 0; u < 8; ++u) s += v[u];
+            for (int u = 0; u < 8; ++u)
+#pragma unroll
+                for (int j = 0; j < V; ++j) s[j] += v[u][j];
         }
     }
-    gsum[g][e] = s;
+#pragma unroll
+    for (int j = 0; j < V; ++j) gsum[g][e + j] = s[j];
     __syncthreads();
     // the partials are [rows, cols], of which [rows_out, cols_out] exist; the result may be a block of columns (c0 ..) of a
     // matrix with rows ld apart
-    if (g == 0 && i < n) {
-        const int r = (int)(i / cols), c = (int)(i % cols);
+    const int64_t k = blockIdx.x * (int64_t)E + threadIdx.x;
+    if (threadIdx.x < E && k < n) {
+        const int r = (int)(k / cols), c = (int)(k % cols);
+        float t = gsum[0][threadIdx.x];
 #pragma unroll
-        for (int k = 1; k < 8; ++k) s += gsum[k][e];
-        if (r < rows_out && c < cols_out) out[(int64_t)r * ld + c0 + c] = from_f32<TC>(s);
+        for (int q = 1; q < 8; ++q) t += gsum[q][threadIdx.x];
+        if (r < rows_out && c < cols_out) out[(int64_t)r * ld + c0 + c] = from_f32<TC>(t);
     }
 }
 
@@ -159,10 +176,10 @@ gnn_status linear_tma_f32_forward(const void* X, int ldx, const void* W, int64_t
                                   cudaStream_t st, const float* bias, int relu);
 bool linear_tma_dw_supported(int64_t N, int K, int M, gnn_dtype dtype);
 int linear_tma_dw_partials(int64_t N);
-gnn_status linear_tma_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, float* part, int* d_flag, int reset, cudaStream_t st);
+gnn_status linear_tma_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, float* part, int* d_flag, int reset, int beside, cudaStream_t st);
 bool linear_tma_f32_dw_supported(int64_t N, int K, int M, int Mo, gnn_dtype dtype);
 int linear_tma_f32_dw_partials(int64_t N);
-gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, int Mo, float* part, int* d_flag, int reset, cudaStream_t st);
+gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, int Mo, float* part, int* d_flag, int reset, int beside, cudaStream_t st);
 
 static int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
@@ -320,17 +337,24 @@ gnn_status gnn_linear_backward(const void* X, const void* W, const void* dY, int
         float* part = (float*)(w8 + lw.part);
         auto sum = [&](int slabs, int rows, int cols, int cols_out, int c0) {
             const int64_t n = (int64_t)rows * cols;
-            const dim3 grid((unsigned)ceil_div(n, 32));
-            if (dtype == GNN_F32) launch_overlapped(slab_sum_kernel<float>, grid, dim3(256), 0, st, part, slabs, n, (float*)dW, cols, K, cols_out, M, c0);
-            else launch_overlapped(slab_sum_kernel<__nv_bfloat16>, grid, dim3(256), 0, st, part, slabs, n, (__nv_bfloat16*)dW, cols, K, cols_out, M, c0);
+            auto run = [&](auto kernel, auto* to, int elements, int threads) {
+                launch_overlapped(kernel, dim3((unsigned)ceil_div(n, (int64_t)elements)), dim3(threads), 0, st, part, slabs, n, to, cols, K, cols_out, M, c0);
+            };
+            const bool four = n % 4 == 0 && aligned16(part);
+            if (dtype == GNN_F32) four ? run(slab_sum_kernel<float, 4>, (float*)dW, 64, 128) : run(slab_sum_kernel<float, 1>, (float*)dW, 32, 256);
+            else four ? run(slab_sum_kernel<__nv_bfloat16, 4>, (__nv_bfloat16*)dW, 64, 128) : run(slab_sum_kernel<__nv_bfloat16, 1>, (__nv_bfloat16*)dW, 32, 256);
         };
         if (block) {
             const void* Xp = with_padded_rows(X, N, K, s, w8 + lw.x, st);
             for (int c0 = 0; c0 < M; c0 += block) {
                 const int mc = M - c0 < block ? M - c0 : block;
                 const void* dYb = (const char*)dYp + (size_t)c0 * s;
-                gnn_status rc = dtype == GNN_F32 ? linear_tma_f32_dw(Xp, padded(K, s), dYb, ldd, N, K, mc, M, part, status, reset, st)
-                                                 : linear_tma_dw(Xp, padded(K, s), dYb, ldd, N, K, mc, part, status, reset, st);
+                // The products of dX let the next kernel come up only after their own wait, when everything before them is done and
+                // visible.  Those of dW that follow directly read nothing that dX's write (X and dY, through the copy engine, out of
+                // L2): they start where SMs are free, and wait for dX's end before their own, so that the stream's order is kept.
+                const int beside = dx_tma && Xp == X && c0 == 0;
+                gnn_status rc = dtype == GNN_F32 ? linear_tma_f32_dw(Xp, padded(K, s), dYb, ldd, N, K, mc, M, part, status, reset, beside, st)
+                                                 : linear_tma_dw(Xp, padded(K, s), dYb, ldd, N, K, mc, part, status, reset, beside, st);
                 if (rc != GNN_OK) return rc;
                 reset = 0;
                 sum(dtype == GNN_F32 ? linear_tma_f32_dw_partials(N) : linear_tma_dw_partials(N), round_up(K, 32), round_up(mc, dtype == GNN_F32 ? 32 : 16), mc, c0);
