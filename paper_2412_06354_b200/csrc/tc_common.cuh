@@ -115,7 +115,7 @@ __device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.
 
 // raise a kernel's dynamic shared memory limit, once per (device, kernel slot)
 inline gnn_status allow_big_smem(const char* who, const void* kernel, int which, size_t bytes) {
-    static std::atomic<unsigned char> done[64][24];
+    static std::atomic<unsigned char> done[64][48];
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) dev = -1;
     if (dev >= 0 && done[dev][which].load()) return GNN_OK;
