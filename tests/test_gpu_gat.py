@@ -91,6 +91,50 @@ def test_gat_one_and_two_heads_with_source_hubs(gnn, H, C):
     run_case(gnn, n, src, dst, Wx, a_s, a_d, H, C, "f32", f"gat source hubs H={H}")
 
 
+# The row kernels of four and eight heads take chunks of positions: 512 and 256 on small graphs, 2048 and 1024 from 800 and 400 Ki edges on.
+# Rows that fill a chunk, end one before or one past its end, lie over several chunks, empty rows at the seams, a last chunk of a few.
+@pytest.mark.parametrize("H,chunk,edges", [(4, 512, 9_001), (8, 256, 4_611), (8, 256, 256), (8, 1024, 420_003), (4, 2048, 830_011)])
+def test_gat_and_softmax_rows_at_chunk_ends(gnn, H, chunk, edges):
+    rng = np.random.default_rng(edges)
+    degree = [chunk, 0, chunk - 1, 1, chunk + 1, chunk - 2, 1, 3 * chunk, 0, 0, 5, 2 * chunk - 5] if edges > chunk else []
+    while sum(degree) < edges:
+        degree += [min(int(d), edges - sum(degree)) for d in rng.integers(0, 40, 1 if edges - sum(degree) < 4000 else 100)]
+    n = len(degree)
+    order = rng.permutation(edges)
+    dst = np.repeat(np.arange(n, dtype=np.int32), degree)[order]
+    src = rng.integers(0, n, edges).astype(np.int32)
+    C = 8
+    Wx = synth.normal((n, H * C), "f32", 910 + H, 1)
+    a_s = synth.uniform_f32((H, C), -0.8, 0.8, 911, 1)
+    a_d = synth.uniform_f32((H, C), -0.8, 0.8, 912, 1)
+    g, _ = run_case(gnn, n, src, dst, Wx, a_s, a_d, H, C, "f32", f"gat H={H}, chunks of {chunk}")
+    eid = g.eid[:g.E].cpu().numpy()
+    for dtype in ("f32", "bf16"):
+        logits, R = synth.normal((edges, H), dtype, 913, 1), synth.normal((edges, H), dtype, 914, 1)
+        alpha, top, total = gnn.edge_softmax(g, to_dev(logits[eid]), want_stats=True)
+        ao = oracle.edge_softmax(n, dst, logits)
+        assert_close(to_host64(alpha), ao[eid], ao[eid], dtype, "alpha")
+        x = synth.to_f64(logits)
+        most = np.full((n, H), -np.inf)
+        np.maximum.at(most, dst, x)
+        sums = np.zeros((n, H))
+        np.add.at(sums, dst, np.exp(x - most[dst]))
+        most[np.array(degree) == 0] = 0.0  # what a row without edges has
+        assert np.array_equal(to_host64(top), most)
+        assert_close(to_host64(total), sums, sums, "f32", "sums of the rows")
+        a_host = np.empty((edges, H))
+        a_host[eid] = to_host64(alpha)
+        ds = gnn.edge_softmax_backward(g, alpha, to_dev(R[eid]))
+        dso, S = oracle.edge_softmax_backward(n, dst, a_host, R)
+        assert_close(to_host64(ds), dso[eid], S[eid], dtype, "dlogits")
+        # written over their own input (no chunks then): within the same bounds
+        own, upstream = to_dev(logits[eid]).clone(), to_dev(R[eid]).clone()
+        gnn._check(gnn.load().gnn_edge_softmax(gnn.C.byref(g.c), gnn._p(own), H, gnn._dtype(own), gnn._p(own), None, None, gnn._stream()))
+        assert_close(to_host64(own), ao[eid], ao[eid], dtype, "alpha over the logits")
+        gnn._check(gnn.load().gnn_edge_softmax_backward(gnn.C.byref(g.c), gnn._p(alpha), gnn._p(upstream), H, gnn._dtype(own), gnn._p(upstream), gnn._stream()))
+        assert_close(to_host64(upstream), dso[eid], S[eid], dtype, "dlogits over dalpha")
+
+
 def test_gat_zero_attention_is_mean_aggregation(gnn):
     n, src, dst = ragged_graph(95)
     H, C = 4, 16
