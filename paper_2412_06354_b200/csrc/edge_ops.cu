@@ -267,7 +267,8 @@ __global__ void graph_ptr_kernel(const int32_t* gid, int32_t N, int32_t G,
     }
 }
 
-// out = alpha*a + beta*b, element-wise in fp32 (self terms of layers: W1*x_i + W2*agg, (1+eps)*x_i + sum)
+// out = alpha*a + beta*b, element-wise in fp32 (self terms of layers: W1*x_i + W2*agg, (1+eps)*x_i + sum).  From the end: a and b
+// were usually written just before, in ascending order, and L2 holds their ends; what reads `out` next begins with the part written last.
 template <typename T>
 __global__ void axpby_kernel(float alpha, const uint4* a, float beta, const uint4* b,
                              int64_t nvec, uint4* __restrict__ out) {
@@ -275,7 +276,7 @@ __global__ void axpby_kernel(float alpha, const uint4* a, float beta, const uint
     constexpr int EPC = Chunk<T>::N;
     int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (; t < nvec; t += stride) {
+    for (t = nvec - 1 - t; t >= 0; t -= stride) {
         float x[EPC], y[EPC];
         Chunk<T>::unpack(a[t], x);
         Chunk<T>::unpack(b[t], y);
@@ -314,8 +315,12 @@ gnn_status gnn_gather_backward(const gnn_csr* g, int by_src, const void* dOut_EF
     const int64_t* rp = by_src ? g->rowptrT : g->rowptr;
     const int32_t* rows = by_src ? g->eidT : g->eid;  // COO row of dOut for each position
     GNN_REQUIRE(rp && (g->E == 0 || rows), GNN_ERR_INVALID_ARG, "%s: incomplete gnn_csr", who);
+    // The edge tensor is usually larger than L2 and has just been written in ascending order: its end is what L2 still holds.
+    RowExtra rx = {};
+    rx.agg_c = 1.0f;
+    rx.descending = 1;
     return run_chunked(who, MODE_SUM, g->N, g->E, rp, rows, nullptr, dOut_EF, dX, nullptr, nullptr,
-                       nullptr, nullptr, 0, F, dtype, ws, ws_bytes, as_stream(stream));
+                       nullptr, nullptr, 0, F, dtype, ws, ws_bytes, as_stream(stream), nullptr, &rx);
 }
 
 gnn_status gnn_apply_edges(const gnn_csr* g, gnn_msg msg, const void* X_or_al, const void* ar,

@@ -146,7 +146,7 @@ gnn_status run_chunked(const char* who, int mode, int32_t N, int64_t E, const in
     }
     P.x_ld = P.out_ld = P.self_ld = (uint32_t)nvec * 16;
     P.ef = nullptr; P.ef_ld = 0; P.has_epi = 0; P.agg_c = 1.0f; P.self_c = 0.f; P.self_mode = GNN_SELF_ALWAYS; P.relu = 0;
-    P.self_X = nullptr; P.self_rowptr = rowptr; P.bias = nullptr;
+    P.self_X = nullptr; P.self_rowptr = rowptr; P.bias = nullptr; P.descending = 0;
     if (rx) {
         GNN_REQUIRE(mode == MODE_EFSUM ? (rx->ef != nullptr || E == 0) : rx->ef == nullptr, GNN_ERR_INVALID_ARG,
                     "%s: per-feature multipliers and mode disagree", who);
@@ -158,6 +158,7 @@ gnn_status run_chunked(const char* who, int mode, int32_t N, int64_t E, const in
         P.agg_c = rx->agg_c; P.self_c = rx->self_c; P.self_mode = rx->self_mode;
         if (rx->self_rowptr) P.self_rowptr = rx->self_rowptr;
         P.relu = rx->relu;
+        P.descending = rx->descending;
         P.has_epi = (rx->agg_c != 1.0f || rx->self_X || rx->bias || rx->relu) ? 1 : 0;
     } else {
         GNN_REQUIRE(mode != MODE_EFSUM, GNN_ERR_INVALID_ARG, "%s: per-feature mode without multipliers", who);

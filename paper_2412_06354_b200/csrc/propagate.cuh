@@ -29,6 +29,7 @@ struct RowExtra {
     const int64_t* self_rowptr;
     const float* bias;  // [F] or nullptr
     int relu;
+    int descending = 0;  // positions from the last to the first: the gathered matrix was just written in ascending order
 };
 
 // lanes per row (4..32) and 16-byte vectors per lane (1, 2, 4) for rows of nvec 16-byte chunks

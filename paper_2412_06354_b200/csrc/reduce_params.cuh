@@ -44,6 +44,7 @@ struct PropParams {
     //   v = agg_c * v + self_c * c(r) * self_X[r,f] + bias[f], then max(v, 0) if relu
     // c(r) = 1 (GNN_SELF_ALWAYS), the length of row r in self_rowptr (GNN_SELF_TIMES_DEGREE), or 1 if that
     // length is positive else 0 (GNN_SELF_IF_NONEMPTY)
+    int descending;  // pieces from the last to the first
     int vote;  // rows are long enough on average that whole batches without a row end are common
     int has_epi;
     float agg_c, self_c;

@@ -373,7 +373,8 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     extern __shared__ __align__(16) unsigned char rs_smem[];
     pdl_wait();
     const int lane = threadIdx.x & 31, g = lane / LPR, li = lane % LPR;
-    const int wib = threadIdx.x >> 5, c = (int)blockIdx.x * RR_WARPS + wib;
+    const int piece = P.descending ? (int)(gridDim.x - 1 - blockIdx.x) : (int)blockIdx.x;
+    const int wib = threadIdx.x >> 5, c = piece * RR_WARPS + wib;
     __shared__ int s_head[RR_WARPS], s_tail_row[RR_WARPS];
     Stage& S = reinterpret_cast<Stage*>(rs_smem)[wib];
     const int cs = (int)min((int64_t)c * P.sub, P.E);
@@ -457,7 +458,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
     };
     auto write_partial = [&](int which, const float* v, const int32_t* va) {
         if (lane >= LPR || !col_lane) return;
-        const size_t off = ((size_t)blockIdx.x * 2 + which) * P.F + (size_t)ci * EPC;
+        const size_t off = ((size_t)piece * 2 + which) * P.F + (size_t)ci * EPC;
 #pragma unroll
         for (int j = 0; j < EPC; j += 4) {
             *reinterpret_cast<float4*>(P.part_val + off + j) = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
@@ -799,7 +800,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
             float v = 0.f;
 #pragma unroll
             for (int k = 0; k < RR_WARPS; ++k) v += sums[k * LPR * EPC + f];
-            P.da_part[(size_t)blockIdx.x * P.F + f] = v;
+            P.da_part[(size_t)piece * P.F + f] = v;
         }
     }
     if (threadIdx.x == 0) {  // the row that begins in the block and reaches past it
@@ -808,7 +809,7 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
             if (s_head[k] != HEAD_THROUGH) t = -1;
             if (s_tail_row[k] >= 0) t = s_tail_row[k];
         }
-        P.tail_row[blockIdx.x] = t;
+        P.tail_row[piece] = t;
     }
 }
 
