@@ -6,7 +6,7 @@
 //   out[i,h,:] = sum_p alpha[p,h] * Wx[col[p],h,:]
 // The E x F message tensor is never formed: the weighted sum runs in the chunked gather kernel
 // with one multiplier per (edge, head).  Scores and coefficients are fp32.
-#include "propagate.cuh"
+#include "reduce_params.cuh"
 
 namespace gnn {
 
@@ -29,14 +29,15 @@ __global__ void gat_scores_kernel(const T* __restrict__ Wx, const float* __restr
     ar[t] = sr;
 }
 
-// Rows of at most 32 16-byte chunks whose heads span a power-of-two number of chunks: LPR lanes
-// cover a node's row with one coalesced 16-byte load each (32/LPR nodes per warp), keep their slice
-// of both attention vectors in registers, and the lanes of a head add up by xor-shuffles (fixed tree).
+// Rows of at most 32 16-byte chunks whose heads span a power-of-two number of chunks: LPR lanes cover a node's row with one
+// coalesced 16-byte load each (32/LPR nodes per warp), four rows in flight, and keep their slice of both attention vectors in
+// registers.  The lanes of a head add up by xor-shuffles (fixed tree); from the first step on even lanes carry the sum of a_src and
+// odd ones that of a_dst, so that a row takes one shuffle per step and one store.  Bound by instruction issue.
 template <typename T, int LPR>
 __global__ void __launch_bounds__(256)
-gat_scores_rows_kernel(const T* __restrict__ Wx, const float* __restrict__ a_src, const float* __restrict__ a_dst,
-                       int N, int H, int nvec, int lph, float* __restrict__ al, float* __restrict__ ar) {
+gat_scores_rows_kernel(const T* Wx, const float* a_src, const float* a_dst, int N, int H, int nvec, int lph, float* __restrict__ al, float* __restrict__ ar) {
     constexpr int EPC = Chunk<T>::N, NG = 32 / LPR;
+    pdl_wait();
     const int lane = threadIdx.x & 31, g = lane / LPR, li = lane % LPR;
     const bool on = li < nvec;
     float as[EPC], ad[EPC];
@@ -45,29 +46,39 @@ gat_scores_rows_kernel(const T* __restrict__ Wx, const float* __restrict__ a_src
         as[j] = on ? a_src[li * EPC + j] : 0.f;
         ad[j] = on ? a_dst[li * EPC + j] : 0.f;
     }
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5, nwarps = (gridDim.x * (int64_t)blockDim.x) >> 5;
+    const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), nwarps = (int)((gridDim.x * blockDim.x) >> 5);
     constexpr int U = 4;  // rows in flight per lane group
-    for (int64_t n0 = warp * NG * U; n0 < N; n0 += nwarps * NG * U) {
+    const int h = li / lph, in_head = li % lph;
+    const bool odd = (li & 1) != 0, split = lph > 1;
+    float* const to = (split && odd ? ar : al) + h;
+    const bool writes = on && (split ? in_head < 2 : true);
+    const char* const base = reinterpret_cast<const char*>(Wx) + (size_t)(on ? li : 0) * 16;
+    const size_t row_bytes = (size_t)nvec * 16;
+    for (int64_t n0 = (int64_t)warp * (NG * U) + g; n0 < N + g; n0 += (int64_t)nwarps * (NG * U)) {  // the same number of turns in every group
         uint4 raw[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int64_t n = n0 + u * NG + g;
-            raw[u] = n < N && on ? __ldg(reinterpret_cast<const uint4*>(Wx) + (size_t)n * nvec + li) : make_uint4(0u, 0u, 0u, 0u);
+            const int64_t n = n0 + u * NG;
+            raw[u] = n < N && on ? ld_16(base + (size_t)n * row_bytes) : make_uint4(0u, 0u, 0u, 0u);
         }
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int64_t n = n0 + u * NG + g;
-            float x[EPC], sl = 0.f, sr = 0.f;
+            const int64_t n = n0 + u * NG;
+            float x[EPC], l0 = 0.f, l1 = 0.f, r0 = 0.f, r1 = 0.f;
             Chunk<T>::unpack(raw[u], x);
 #pragma unroll
-            for (int j = 0; j < EPC; ++j) { sl = fmaf(as[j], x[j], sl); sr = fmaf(ad[j], x[j], sr); }
-            for (int o = lph >> 1; o > 0; o >>= 1) {
-                sl += __shfl_xor_sync(0xffffffffu, sl, o);
-                sr += __shfl_xor_sync(0xffffffffu, sr, o);
+            for (int j = 0; j < EPC; j += 2) {
+                fma2(l0, l1, x[j], x[j + 1], as[j], as[j + 1]);
+                fma2(r0, r1, x[j], x[j + 1], ad[j], ad[j + 1]);
             }
-            if (n < N && on && (li % lph) == 0) {
-                al[(size_t)n * H + li / lph] = sl;
-                ar[(size_t)n * H + li / lph] = sr;
+            const float sl = l0 + l1, sr = r0 + r1;
+            if (split) {
+                float v = (odd ? sr : sl) + __shfl_xor_sync(0xffffffffu, odd ? sl : sr, 1);
+                for (int o = 2; o < lph; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                if (n < N && writes) to[(size_t)n * H] = v;
+            } else if (n < N && writes) {
+                al[(size_t)n * H + h] = sl;
+                ar[(size_t)n * H + h] = sr;
             }
         }
     }
@@ -335,7 +346,7 @@ gnn_status gnn_gat_fused(const gnn_csr* g, const void* Wx, const float* a_src, c
     int lpr = 0, vpl = 0;
     if (((size_t)C * s_el) % 16 == 0 && (lph & (lph - 1)) == 0 && pick_shape(nvec, &lpr, &vpl) && vpl == 1) {
         const int grid = grid_for(ceil_div(g->N, 4 * (32 / lpr)) * 32, 256);
-#define GNN_GS(T, L) gat_scores_rows_kernel<T, L><<<grid, 256, 0, st>>>((const T*)Wx, a_src, a_dst, g->N, H, nvec, lph, al, ar)
+#define GNN_GS(T, L) launch_overlapped(gat_scores_rows_kernel<T, L>, dim3(grid), dim3(256), 0, st, (const T*)Wx, a_src, a_dst, g->N, H, nvec, lph, al, ar)
         if (dtype == GNN_F32) { if (lpr == 4) GNN_GS(float, 4); else if (lpr == 8) GNN_GS(float, 8); else if (lpr == 16) GNN_GS(float, 16); else GNN_GS(float, 32); }
         else { if (lpr == 4) GNN_GS(__nv_bfloat16, 4); else if (lpr == 8) GNN_GS(__nv_bfloat16, 8); else if (lpr == 16) GNN_GS(__nv_bfloat16, 16); else GNN_GS(__nv_bfloat16, 32); }
 #undef GNN_GS
