@@ -935,6 +935,9 @@ static bool make_map_f32_blocks(CUtensorMap* m, const void* ptr, int64_t rows, i
 // Every wait is bounded.
 // Two groups on slots of 32 rows, on slots of 16 four where four buffers and slots fit.  170k x 128 x 128: 50 us with 8 warps
 // on one slot after the other, 47 us with 16, 58 us in four groups on slots of 16 rows, 42 us so; reading X and dY takes 27 us.
+// Then the bound was shared memory's bandwidth (copies, conversion and both operands of every MMA: 80 % of a slot's time), so X's
+// levels go to tensor memory (A_TMEM), transposed on the way: a feature per lane.  Where the accumulators leave no columns for two
+// operand buffers (K of 256 by M over 208, for one) A stays in shared memory.
 // Exact form (K or M no multiple of 32): the accumulator truncates at every MMA, 1.8e-8 of the result each and one way, so that
 // a CTA's hundreds of rows in one sum cost 7.8e-6 norm-wise at 170k rows and 2.3e-5 at 500k, where the FFMA kernel that these
 // sizes took before has 1.1e-6.  There the five small products go to an accumulator of corrections, and after every FD_FLUSH
@@ -961,7 +964,7 @@ struct TmaF32DwParams {
     int beside; // runs beside the kernel before it in the stream, of whose results it reads none
 };
 
-template <int FD_ROWS, bool EXACT>
+template <int FD_ROWS, bool EXACT, bool A_TMEM>
 __global__ void __launch_bounds__(FD_THREADS + (EXACT ? 32 * FD_FLUSH_WARPS : 0), 1)
 linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constant__ CUtensorMap mapD, const TmaF32DwParams P) {
     extern __shared__ unsigned char smem_raw[];
@@ -975,8 +978,10 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
     constexpr uint32_t FD_SBO = (uint32_t)(FD_ROWS / 8) * 128u;   // next chunk of 8 features / columns in an operand level
     const int xboxes = K / 32, dboxes = M / 32;
     const uint32_t slot_bytes = (uint32_t)(xboxes + dboxes) * FD_BOX_BYTES;
-    // the A operand always has whole blocks of the MMA's 128 feature rows; with K < 128 the rows past K stay zero
-    const uint32_t a_level = (uint32_t)halves * 128u * FD_ROWS * 2, b_level = (uint32_t)M * FD_ROWS * 2;
+    // the A operand always has whole blocks of the MMA's 128 feature rows; with K < 128 the rows past K stay zero (in tensor memory:
+    // whatever they are, they only reach accumulator rows that nobody reads)
+    const uint32_t a_level = A_TMEM ? 0u : (uint32_t)halves * 128u * FD_ROWS * 2, b_level = (uint32_t)M * FD_ROWS * 2;
+    constexpr uint32_t A_COLS = FD_ROWS / 2;  // tensor memory columns of one level of 128 features
     const uint32_t op_bytes = 3u * (a_level + b_level);
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t ring0 = base, op0 = ring0 + (uint32_t)S * slot_bytes;
@@ -1002,7 +1007,7 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
         tmem_alloc(smem_u32(&tmem_base_slot), (uint32_t)P.tmem_cols);
         pdl_let_next();
     }
-    if (K % 128 != 0) {  // the converters never write the feature rows past K: zero the buffers' A levels once
+    if (!A_TMEM && K % 128 != 0) {  // the converters never write the feature rows past K: zero the buffers' A levels once
         for (int o = 0; o < (int)G; ++o)
             for (uint32_t off = (uint32_t)tid * 16u; off < 3u * a_level; off += blockDim.x * 16u)
                 st_shared16(op0 + (uint32_t)o * op_bytes + off, make_uint4(0u, 0u, 0u, 0u));
@@ -1015,6 +1020,7 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
     if (P.reset && blockIdx.x == 0 && tid == 0) *P.status = 0;
     const uint32_t tmem_base = tmem_base_slot;
     const int64_t nslots = (P.N + FD_ROWS - 1) / FD_ROWS;
+    const uint32_t a_tmem = tmem_base + (EXACT ? mains + 1u : 1u) * acc_cols;  // A_TMEM: operand buffers, [group][128 features][level]
     bool failed = false;
 
     if (warp == 0) {
@@ -1043,7 +1049,7 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
         if (lane == 0) {
-            const uint32_t idesc = make_idesc(M, 1) | (1u << 15);  // A and B both MN-major
+            const uint32_t idesc = make_idesc(M, 1, A_TMEM ? 0 : 1);  // B MN-major, A too where it lies in shared memory
             uint32_t it = 0, acc = tmem_base, fresh = 1, v = 0;  // fresh: the main sum begins with this slot; v: how many began before
             for (int64_t t = blockIdx.x; t < nslots; t += gridDim.x, ++it) {
                 const uint32_t o = it % G;
@@ -1055,6 +1061,7 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
                 tc_fence_after();
                 const uint32_t abuf = op0 + o * op_bytes, bbuf = abuf + 3u * a_level;
                 const uint64_t adesc = make_smem_desc(abuf, 128, FD_SBO), bdesc = make_smem_desc(bbuf, 128, FD_SBO);
+                const uint32_t at = a_tmem + o * (uint32_t)halves * 3u * A_COLS;
                 for (int h = 0; h < halves; ++h) {  // features [128h, 128h + 128): chunks 16h.., accumulator columns h*M..
 #pragma unroll
                     for (int kk = 0; kk < FD_ROWS / 16; ++kk)
@@ -1065,8 +1072,10 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
                                 if (q < 5) to = tmem_base + mains * acc_cols;
                                 else more = (!fresh || kk > 0) ? 1u : 0u;
                             }
-                            mma_bf16_ss(to + (uint32_t)h * (uint32_t)M, adesc + (uint64_t)(pair_a(q) * (a_level / 16) + (uint32_t)h * FD_SBO + (uint32_t)kk * 16u),
-                                        bdesc + (uint64_t)(pair_b(q) * (b_level / 16) + (uint32_t)kk * 16u), idesc, more);
+                            const uint64_t bd = bdesc + (uint64_t)(pair_b(q) * (b_level / 16) + (uint32_t)kk * 16u);
+                            if (A_TMEM) mma_bf16_ts(to + (uint32_t)h * (uint32_t)M, at + ((uint32_t)h * 3u + pair_a(q)) * A_COLS + (uint32_t)kk * 8u, bd, idesc, more);
+                            else
+                                mma_bf16_ss(to + (uint32_t)h * (uint32_t)M, adesc + (uint64_t)(pair_a(q) * (a_level / 16) + (uint32_t)h * FD_SBO + (uint32_t)kk * 16u), bd, idesc, more);
                         }
                 }
                 mma_commit(o_empty((int)o));
@@ -1134,8 +1143,29 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
             tc_fence_after();
             const uint32_t src0 = ring0 + (uint32_t)s * slot_bytes;
             const uint32_t abuf = op0 + o * op_bytes, bbuf = abuf + 3u * a_level;
+            if (A_TMEM) {  // a feature per lane, eight rows at a time; a warp reaches the 32 lanes of tensor memory of its number modulo 4
+                const int quarter = warp & 3;
+                const uint32_t at = a_tmem + o * (uint32_t)halves * 3u * A_COLS + ((uint32_t)(quarter * 32) << 16);
+                for (int h = 0; h < halves; ++h) {
+                    const int box = 4 * h + quarter;
+                    if (box >= xboxes) break;
+                    const uint32_t src = src0 + (uint32_t)box * FD_BOX_BYTES + (uint32_t)(lane & 3) * 4u;
+                    for (int rg = ((warp - 2) % GW) >> 2; rg < BU; rg += GW >> 2) {
+                        float x[8];
+#pragma unroll
+                        for (int j = 0; j < 8; ++j)
+                            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(x[j]) : "r"(src + (uint32_t)rg * 1024u + (uint32_t)j * 128u + (uint32_t)(((lane >> 2) ^ j) << 4)) : "memory");
+                        uint4 lv[3];
+                        split8(x, lv);
+#pragma unroll
+                        for (int l = 0; l < 3; ++l) tmem_st4(at + (uint32_t)(h * 3 + l) * A_COLS + (uint32_t)rg * 4u, lv[l]);
+                    }
+                }
+                tmem_st_wait();
+                tc_fence_before();
+            }
 #pragma unroll 2
-            for (int u = (warp - 2) % GW; u < units; u += GW) {
+            for (int u = (warp - 2) % GW + (A_TMEM ? xboxes * BU : 0); u < units; u += GW) {
                 const int box = u / BU, rg = u % BU;
                 const uint32_t rows8 = src0 + (uint32_t)box * FD_BOX_BYTES + (uint32_t)rg * 1024u;
                 const uint4 c0 = ld_shared16(rows8 + from0), c1 = ld_shared16(rows8 + from1);
@@ -1212,17 +1242,21 @@ gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, in
     if (!(P.x_whole ? make_map_f32_blocks : make_map_f32_ld)(&mapX, X, N, Kr, ldx, R) || !(P.d_whole ? make_map_f32_blocks : make_map_f32_ld)(&mapD, dY, N, Mr, ldd, R))
         GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
     P.part = part; P.N = N; P.K = K; P.M = M; P.status = d_flag; P.reset = reset; P.beside = beside;
-    const size_t slot = (size_t)(K / 32 + M / 32) * R * 128, op = 3 * ((size_t)ka * R * 2 + (size_t)M * R * 2);
-    P.groups = R == 16 && 1024 + FD_MAX_GROUPS * (op + slot) <= TM_SMEM_MAX ? FD_MAX_GROUPS : 2;
+    const bool exact = fd_exact(Kr, Mo);
+    const int acc_cols = M * (ka / 128);
+    P.mains = exact && 3 * acc_cols <= 512 ? 2 : 1;
+    const int acc_all = (exact ? P.mains + 1 : 1) * acc_cols;
+    // X's levels in tensor memory where two buffers of them fit beside the accumulators
+    const bool a_tmem = acc_all + 2 * (ka / 128) * 3 * (R / 2) <= 512;
+    const size_t slot = (size_t)(K / 32 + M / 32) * R * 128, op = 3 * ((a_tmem ? 0 : (size_t)ka * R * 2) + (size_t)M * R * 2);
+    auto columns = [&](int groups) { return acc_all + (a_tmem ? groups * (ka / 128) * 3 * (R / 2) : 0); };
+    P.groups = R == 16 && 1024 + FD_MAX_GROUPS * (op + slot) <= TM_SMEM_MAX && columns(FD_MAX_GROUPS) <= 512 ? FD_MAX_GROUPS : 2;
     const size_t ops = (size_t)P.groups * op;
     int stages = (int)((TM_SMEM_MAX - 1024 - ops) / slot);
     if (stages > FD_MAX_STAGES) stages = FD_MAX_STAGES;
     P.stages = stages / P.groups * P.groups;
-    const bool exact = fd_exact(Kr, Mo);
-    const int acc_cols = M * (ka / 128);
-    P.mains = exact && 3 * acc_cols <= 512 ? 2 : 1;
     int cols = 32;
-    while (cols < (exact ? P.mains + 1 : 1) * acc_cols) cols <<= 1;
+    while (cols < columns(P.groups)) cols <<= 1;
     P.tmem_cols = cols;
     auto launch = [&](auto kernel, int which, int threads) {
         gnn_status rc = allow_big_smem(who, (const void*)kernel, which, TM_SMEM_MAX);
@@ -1232,8 +1266,12 @@ gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, in
         return GNN_OK;
     };
     constexpr int more = FD_THREADS + 32 * FD_FLUSH_WARPS;
-    if (exact) return R == 32 ? launch(linear_tma_f32_dw_kernel<32, true>, 18, more) : launch(linear_tma_f32_dw_kernel<16, true>, 19, more);
-    return R == 32 ? launch(linear_tma_f32_dw_kernel<32, false>, 12, FD_THREADS) : launch(linear_tma_f32_dw_kernel<16, false>, 15, FD_THREADS);
+    if (a_tmem) {
+        if (exact) return R == 32 ? launch(linear_tma_f32_dw_kernel<32, true, true>, 44, more) : launch(linear_tma_f32_dw_kernel<16, true, true>, 45, more);
+        return R == 32 ? launch(linear_tma_f32_dw_kernel<32, false, true>, 46, FD_THREADS) : launch(linear_tma_f32_dw_kernel<16, false, true>, 47, FD_THREADS);
+    }
+    if (exact) return R == 32 ? launch(linear_tma_f32_dw_kernel<32, true, false>, 18, more) : launch(linear_tma_f32_dw_kernel<16, true, false>, 19, more);
+    return R == 32 ? launch(linear_tma_f32_dw_kernel<32, false, false>, 12, FD_THREADS) : launch(linear_tma_f32_dw_kernel<16, false, false>, 15, FD_THREADS);
 }
 
 static size_t tf_fixed_bytes(int Kc, int Mo) {
