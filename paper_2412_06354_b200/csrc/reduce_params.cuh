@@ -105,11 +105,10 @@ __device__ __forceinline__ int first_row_ending_after(const int64_t* rowptr, int
     return lo;
 }
 
-// Rows [lo, hi), at most 64, one of which is the last row r with rowptr[r] <= pos (0 <= pos < E), or row 0 if there is none.
-// Warp-cooperative.  The first look is at 32 rows spaced 64 apart around the row that even degrees would give, then 32-way steps.
-__device__ __forceinline__ void narrow_rows(const int64_t* rowptr, int N, int64_t E, int64_t pos, int lane, int& lo, int& hi) {
-    lo = 0;
-    hi = N;  // rowptr[lo] <= pos < rowptr[hi]
+// Position holding `pos`: the last row r with rowptr[r] <= pos (0 <= pos < E), or row 0 if there is none.  Warp-cooperative.  The
+// first look is at 32 rows spaced 64 apart around the row that even degrees would give, then 32-way steps, then 64 rows at once.
+__device__ __forceinline__ int row_of_position(const int64_t* rowptr, int N, int64_t E, int64_t pos, int lane) {
+    int lo = 0, hi = N;  // rowptr[lo] <= pos < rowptr[hi]
     if (N > 1024) {
         const int guess = (int)((double)pos * ((double)N / (double)E));
         const int idx = guess + (lane - 16) * 64;
@@ -126,12 +125,6 @@ __device__ __forceinline__ void narrow_rows(const int64_t* rowptr, int N, int64_
         lo = lo + max(c - 1, 0) * step;
         hi = min(lo + step, hi);
     }
-}
-
-// The row that holds pos (see narrow_rows).
-__device__ __forceinline__ int row_of_position(const int64_t* rowptr, int N, int64_t E, int64_t pos, int lane) {
-    int lo, hi;
-    narrow_rows(rowptr, N, E, pos, lane, lo, hi);
     const int a = lo + 1 + lane, b = a + 32;
     const bool la = a < hi && rowptr[a] <= pos, lb = b < hi && rowptr[b] <= pos;
     return lo + __popc(__ballot_sync(0xffffffffu, la)) + __popc(__ballot_sync(0xffffffffu, lb));
@@ -142,30 +135,25 @@ __device__ __forceinline__ int row_of_position(const int64_t* rowptr, int N, int
 // last (row pointers of a caller that leave some uncovered, as nodes outside graph_ptr) are staged as a row of id -1 that counts
 // as begun before, if it is the first, and never ends, if it is the last: no caller finishes it, and none needs to look (a look
 // at every row end cost 1 to 3 % of the segmented reduction).  Returns the count, at most n.  Warp-cooperative.
-// The 64 row pointers of the search's last step serve the scan that follows it: a warp whose rows lie among them has waited for
-// two loads, one after the other (six before; every warp of the reductions starts with this).
 __device__ __forceinline__ int stage_rows(const int64_t* rowptr, int N, int64_t E, int cs, int n, int lane, int* row, uint16_t* start,
                                           bool& began_before) {
-    int lo, hi;
-    narrow_rows(rowptr, N, E, cs, lane, lo, hi);
-    constexpr int64_t NONE = (int64_t)1 << 62;
-    const int ra = lo + 1 + lane, rb32 = ra + 32;
-    const int64_t v0 = rowptr[lo], va = ra <= N ? rowptr[ra] : NONE, vb = rb32 <= N ? rowptr[rb32] : NONE;
-    const int before = __popc(__ballot_sync(0xffffffffu, ra < hi && va <= cs)) + __popc(__ballot_sync(0xffffffffu, rb32 < hi && vb <= cs));  // < 64
-    const int r0 = lo + before;
-    auto pointer = [&](int k) {  // rowptr[lo + 1 + k]
-        const int64_t x = __shfl_sync(0xffffffffu, va, k & 31), y = __shfl_sync(0xffffffffu, vb, k & 31);
-        return k < 32 ? x : y;
-    };
-    const int64_t sk = pointer(before > 0 ? before - 1 : 0), s0 = before > 0 ? sk : v0, e0 = pointer(before);
+    const int r0 = row_of_position(rowptr, N, E, cs, lane);
     int m = 1;
+    const int64_t s0 = rowptr[r0], e0 = rowptr[r0 + 1];
     const bool none = s0 > cs || e0 <= cs;  // the first position is in no row
     int64_t last_end = none ? (int64_t)cs + n + 1 : e0;
     began_before = none || s0 < cs;
     if (lane == 0) { row[0] = none ? -1 : r0; start[0] = 0; }
-    // rows [s, e) that begin in [cs, cs + n), ascending over the lanes; false when one of them does not: the scan is over
-    auto take = [&](int r, int64_t s, int64_t e, bool skip) {
-        const bool in = !skip && r < N && s < (int64_t)cs + n, live = in && e > s;
+    for (int rb = s0 > cs ? r0 : r0 + 1; rb < N;) {
+        const int r = rb + lane;
+        int64_t s = 0, e = 0;
+        bool in = false;
+        if (r < N) {
+            s = rowptr[r];
+            in = s < cs + n;
+            if (in) e = rowptr[r + 1];
+        }
+        const bool live = in && e > s;
         const unsigned lm = __ballot_sync(0xffffffffu, live);
         if (live) {
             const int q = m + __popc(lm & ((1u << lane) - 1u));
@@ -174,19 +162,8 @@ __device__ __forceinline__ int stage_rows(const int64_t* rowptr, int N, int64_t 
         }
         m += __popc(lm);
         if (lm) last_end = __shfl_sync(0xffffffffu, e, 31 - __clz(lm));
-        return __all_sync(0xffffffffu, skip || in) != 0;
-    };
-    int rb = s0 > cs ? r0 : N;
-    if (s0 <= cs) {
-        const int64_t na = __shfl_down_sync(0xffffffffu, va, 1), first_b = __shfl_sync(0xffffffffu, vb, 0), nb = __shfl_down_sync(0xffffffffu, vb, 1);
-        if (take(ra, va, lane == 31 ? first_b : na, ra <= r0) && take(rb32, vb, nb, rb32 <= r0 || lane == 31)) rb = lo + 64;  // r0 < lo + 64
-    }
-    while (rb < N) {
-        const int r = rb + lane;
-        const int64_t s = r < N ? rowptr[r] : NONE, e = r < N ? rowptr[r + 1] : NONE;
-        const int had = m;
-        if (!take(r, s, e, false)) break;
-        if (m == had) rb = first_row_ending_after(rowptr, rb + 32, N, __shfl_sync(0xffffffffu, s, 0), lane);  // over a run of empty rows
+        if (!__all_sync(0xffffffffu, in)) break;
+        if (lm == 0) rb = first_row_ending_after(rowptr, rb + 32, N, __shfl_sync(0xffffffffu, s, 0), lane);  // over a run of empty rows
         else rb += 32;
     }
     if (last_end < (int64_t)cs + n) {  // no row holds the rest
