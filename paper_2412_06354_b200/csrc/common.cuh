@@ -73,11 +73,10 @@ static inline void launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 
 // ---------------------------------------------------------------- device helpers
 // every thread of a kernel started by launch_overlapped, before its first access to global memory
 __device__ __forceinline__ void pdl_wait_exclusive() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// The next kernel of the stream may be set up from here on, once every block of this one is here.  Kernels that allocate tensor
-// memory say so only when they have it: a block of the next one that took it first would wait for this kernel, and this for it.
-__device__ __forceinline__ void pdl_let_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// ... and in kernels that leave room on an SM (the persistent dense kernels take all of its shared memory): the next kernel
+// of the stream may be set up from here on.
 __device__ __forceinline__ void pdl_wait() {
-    pdl_let_next();
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     pdl_wait_exclusive();
 }
 

@@ -176,10 +176,10 @@ gnn_status linear_tma_f32_forward(const void* X, int ldx, const void* W, int64_t
                                   cudaStream_t st, const float* bias, int relu);
 bool linear_tma_dw_supported(int64_t N, int K, int M, gnn_dtype dtype);
 int linear_tma_dw_partials(int64_t N);
-gnn_status linear_tma_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, float* part, int* d_flag, int reset, int beside, cudaStream_t st);
+gnn_status linear_tma_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, float* part, int* d_flag, int reset, cudaStream_t st);
 bool linear_tma_f32_dw_supported(int64_t N, int K, int M, int Mo, gnn_dtype dtype);
 int linear_tma_f32_dw_partials(int64_t N);
-gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, int Mo, float* part, int* d_flag, int reset, int beside, cudaStream_t st);
+gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, int Mo, float* part, int* d_flag, int reset, cudaStream_t st);
 
 static int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
@@ -349,12 +349,8 @@ gnn_status gnn_linear_backward(const void* X, const void* W, const void* dY, int
             for (int c0 = 0; c0 < M; c0 += block) {
                 const int mc = M - c0 < block ? M - c0 : block;
                 const void* dYb = (const char*)dYp + (size_t)c0 * s;
-                // The products of dX let the next kernel come up only after their own wait, when everything before them is done and
-                // visible.  Those of dW that follow directly read nothing that dX's write (X and dY, through the copy engine, out of
-                // L2): they start where SMs are free, and wait for dX's end before their own, so that the stream's order is kept.
-                const int beside = dx_tma && Xp == X && c0 == 0;
-                gnn_status rc = dtype == GNN_F32 ? linear_tma_f32_dw(Xp, padded(K, s), dYb, ldd, N, K, mc, M, part, status, reset, beside, st)
-                                                 : linear_tma_dw(Xp, padded(K, s), dYb, ldd, N, K, mc, part, status, reset, beside, st);
+                gnn_status rc = dtype == GNN_F32 ? linear_tma_f32_dw(Xp, padded(K, s), dYb, ldd, N, K, mc, M, part, status, reset, st)
+                                                 : linear_tma_dw(Xp, padded(K, s), dYb, ldd, N, K, mc, part, status, reset, st);
                 if (rc != GNN_OK) return rc;
                 reset = 0;
                 sum(dtype == GNN_F32 ? linear_tma_f32_dw_partials(N) : linear_tma_dw_partials(N), round_up(K, 32), round_up(mc, dtype == GNN_F32 ? 32 : 16), mc, c0);

@@ -126,7 +126,6 @@ linear_tma_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_constan
     __syncthreads();
     tc_fence_after();
     pdl_wait_exclusive();
-    if (warp == 1) pdl_let_next();  // after the wait: see dW in gnn_linear_backward
     if (P.reset && blockIdx.x == 0 && tid == 0) *P.status = 0;
     const uint32_t tmem_base = tmem_base_slot;
     const int64_t ntiles = (P.N + TC_ROWS - 1) / TC_ROWS;
@@ -484,7 +483,6 @@ linear_tma_f32_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_con
     }
     if (warp == 1) tmem_alloc(smem_u32(&tmem_base_slot), (uint32_t)P.tmem_cols);
     pdl_wait_exclusive();
-    if (warp == 1) pdl_let_next();  // after the wait: see dW in gnn_linear_backward
     if (P.reset && blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) *P.status = 0;
     const int64_t ntiles = (P.N + TC_ROWS - 1) / TC_ROWS;
     const uint64_t stream = policy_evict_first();
@@ -723,7 +721,6 @@ struct TmaDwParams {
     int tmem_cols;
     int* status;
     int reset;  // first launch of a call: set the status word to 0
-    int beside; // runs beside the kernel before it in the stream, of whose results it reads none
 };
 
 __global__ void __launch_bounds__(TM_THREADS, 1)
@@ -751,14 +748,11 @@ linear_tma_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_cons
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapD)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapP)) : "memory");
     }
-    if (warp == 1) {
-        tmem_alloc(smem_u32(&tmem_base_slot), (uint32_t)P.tmem_cols);
-        pdl_let_next();
-    }
+    if (warp == 1) tmem_alloc(smem_u32(&tmem_base_slot), (uint32_t)P.tmem_cols);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (!P.beside) pdl_wait_exclusive();
+    pdl_wait_exclusive();
     if (P.reset && blockIdx.x == 0 && tid == 0) *P.status = 0;
     const uint32_t tmem_base = tmem_base_slot;
     const int64_t nchunks = (P.N + DW_ROWS - 1) / DW_ROWS;  // gridDim.x <= nchunks: every CTA has work
@@ -846,7 +840,6 @@ linear_tma_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_cons
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_base, (uint32_t)P.tmem_cols);
-    if (P.beside) pdl_wait_exclusive();  // this kernel ends after the one beside it
 }
 
 // K and M: any (inside, rounded up to 32 and 16 with zeros from the copy engine; that is the shape of the partials)
@@ -865,7 +858,7 @@ int linear_tma_dw_partials(int64_t N) {
 bool make_map_f32(CUtensorMap* m, const void* ptr, int64_t rows, int cols, int box_rows);
 
 // writes linear_tma_dw_partials(N) fp32 partials [up32(K), up16(M)] to part; X and dY: rows ldx and ldd elements apart
-gnn_status linear_tma_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, float* part, int* d_flag, int reset, int beside, cudaStream_t st) {
+gnn_status linear_tma_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int K, int M, float* part, int* d_flag, int reset, cudaStream_t st) {
     const char* who = "gnn_linear_backward (pipelined tensor-core dW)";
     GNN_REQUIRE(aligned16(X) && aligned16(dY) && aligned16(part), GNN_ERR_INVALID_ARG, "%s: matrices must be 16-byte aligned", who);
     const int K32 = up32(K), M16 = up16(M);
@@ -874,7 +867,7 @@ gnn_status linear_tma_dw(const void* X, int ldx, const void* dY, int ldd, int64_
         !make_map_f32(&mapP, part, (int64_t)linear_tma_dw_partials(N) * K32, M16, 32))
         GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
     TmaDwParams P;
-    P.part = part; P.N = N; P.K = K32; P.M = M16; P.status = d_flag; P.reset = reset; P.beside = beside;
+    P.part = part; P.N = N; P.K = K32; P.M = M16; P.status = d_flag; P.reset = reset;
     const size_t slot = (size_t)(2 * ((K32 + 127) / 128) + (M16 + 63) / 64) * DW_BOX_BYTES;
     int stages = (int)((TM_SMEM_MAX - 1024) / slot);
     P.stages = stages > TM_MAX_STAGES ? TM_MAX_STAGES : stages;
@@ -961,7 +954,6 @@ struct TmaF32DwParams {
     int tmem_cols;
     int* status;
     int reset;  // first launch of a call: set the status word to 0
-    int beside; // runs beside the kernel before it in the stream, of whose results it reads none
 };
 
 template <int FD_ROWS, bool EXACT, bool A_TMEM>
@@ -1003,10 +995,7 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapX)) : "memory");
         asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mapD)) : "memory");
     }
-    if (warp == 1) {
-        tmem_alloc(smem_u32(&tmem_base_slot), (uint32_t)P.tmem_cols);
-        pdl_let_next();
-    }
+    if (warp == 1) tmem_alloc(smem_u32(&tmem_base_slot), (uint32_t)P.tmem_cols);
     if (!A_TMEM && K % 128 != 0) {  // the converters never write the feature rows past K: zero the buffers' A levels once
         for (int o = 0; o < (int)G; ++o)
             for (uint32_t off = (uint32_t)tid * 16u; off < 3u * a_level; off += blockDim.x * 16u)
@@ -1016,7 +1005,7 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (!P.beside) pdl_wait_exclusive();
+    pdl_wait_exclusive();
     if (P.reset && blockIdx.x == 0 && tid == 0) *P.status = 0;
     const uint32_t tmem_base = tmem_base_slot;
     const int64_t nslots = (P.N + FD_ROWS - 1) / FD_ROWS;
@@ -1208,7 +1197,6 @@ linear_tma_f32_dw_kernel(const __grid_constant__ CUtensorMap mapX, const __grid_
     tc_fence_before();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_base, (uint32_t)P.tmem_cols);
-    if (P.beside) pdl_wait_exclusive();  // this kernel ends after the one beside it
 }
 
 // The exact form where the whole product (K features, Mo columns, of which a launch may take a block of M) is no multiple of 32
@@ -1231,7 +1219,7 @@ int linear_tma_f32_dw_partials(int64_t N) {
 
 // writes linear_tma_f32_dw_partials(N) fp32 partials [up32(K), up32(M)] to part; X and dY: rows ldx and ldd elements apart
 // (a block of Mr of the Mo columns of dY)
-gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int Kr, int Mr, int Mo, float* part, int* d_flag, int reset, int beside, cudaStream_t st) {
+gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, int64_t N, int Kr, int Mr, int Mo, float* part, int* d_flag, int reset, cudaStream_t st) {
     const char* who = "gnn_linear_backward (pipelined fp32 tensor-core dW)";
     GNN_REQUIRE(aligned16(X) && aligned16(dY) && aligned16(part), GNN_ERR_INVALID_ARG, "%s: matrices must be 16-byte aligned", who);
     const int K = up32(Kr), M = up32(Mr);
@@ -1241,7 +1229,7 @@ gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, in
     P.x_whole = Kr % 32 == 0; P.d_whole = Mr % 32 == 0;
     if (!(P.x_whole ? make_map_f32_blocks : make_map_f32_ld)(&mapX, X, N, Kr, ldx, R) || !(P.d_whole ? make_map_f32_blocks : make_map_f32_ld)(&mapD, dY, N, Mr, ldd, R))
         GNN_FAIL(GNN_ERR_CUDA, "%s: tensor map encoding failed", who);
-    P.part = part; P.N = N; P.K = K; P.M = M; P.status = d_flag; P.reset = reset; P.beside = beside;
+    P.part = part; P.N = N; P.K = K; P.M = M; P.status = d_flag; P.reset = reset;
     const bool exact = fd_exact(Kr, Mo);
     const int acc_cols = M * (ka / 128);
     P.mains = exact && 3 * acc_cols <= 512 ? 2 : 1;
@@ -1250,7 +1238,7 @@ gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, in
     const bool a_tmem = acc_all + 2 * (ka / 128) * 3 * (R / 2) <= 512;
     const size_t slot = (size_t)(K / 32 + M / 32) * R * 128, op = 3 * ((a_tmem ? 0 : (size_t)ka * R * 2) + (size_t)M * R * 2);
     auto columns = [&](int groups) { return acc_all + (a_tmem ? groups * (ka / 128) * 3 * (R / 2) : 0); };
-    P.groups = R == 16 && 1024 + FD_MAX_GROUPS * (op + slot) <= TM_SMEM_MAX && columns(FD_MAX_GROUPS) <= 512 ? FD_MAX_GROUPS : 2;
+    P.groups = (R == 16 || a_tmem) && 1024 + FD_MAX_GROUPS * (op + slot) <= TM_SMEM_MAX && columns(FD_MAX_GROUPS) <= 512 ? FD_MAX_GROUPS : 2;
     const size_t ops = (size_t)P.groups * op;
     int stages = (int)((TM_SMEM_MAX - 1024 - ops) / slot);
     if (stages > FD_MAX_STAGES) stages = FD_MAX_STAGES;
