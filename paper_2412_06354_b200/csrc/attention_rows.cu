@@ -57,6 +57,78 @@ __device__ __forceinline__ float4 ld_float4(const float* p) {
     return make_float4(__uint_as_float(u.x), __uint_as_float(u.y), __uint_as_float(u.z), __uint_as_float(u.w));
 }
 
+// stage_rows for these kernels, which latency bounds: the 64 row pointers of the search's last step serve the scan behind it, so that a
+// warp whose rows lie among them waits for two loads, one after the other, instead of six.  (In the reductions, which issue bounds,
+// its instructions cost more than the waits: 123 M edges of 128-byte rows 6.13 -> 6.22 ms, 170k bf16 sums over 256-byte rows 271 -> 290 us.)
+__device__ __forceinline__ int stage_rows_early(const int64_t* rowptr, int N, int64_t E, int cs, int n, int lane, int* row, uint16_t* start,
+                                                bool& began_before) {
+    int lo = 0, hi = N;  // the row that holds cs is one of [lo, hi): row_of_position up to its last step
+    if (N > 1024) {
+        const int guess = (int)((double)cs * ((double)N / (double)E));
+        const int idx = guess + (lane - 16) * 64;
+        const bool le = idx <= 0 || (idx < N && rowptr[idx] <= cs);
+        const int c = __popc(__ballot_sync(0xffffffffu, le));
+        if (c > 0) lo = max(lo, guess + (c - 1 - 16) * 64);
+        if (c < 32) hi = min(hi, guess + (c - 16) * 64);
+    }
+    while (hi - lo > 64) {
+        const int step = (hi - lo + 31) / 32;
+        const int idx = lo + lane * step;
+        const bool le = idx < hi && rowptr[idx] <= cs;
+        const int c = __popc(__ballot_sync(0xffffffffu, le));
+        lo = lo + max(c - 1, 0) * step;
+        hi = min(lo + step, hi);
+    }
+    constexpr int64_t NONE = (int64_t)1 << 62;
+    const int ra = lo + 1 + lane, rb32 = ra + 32;
+    const int64_t v0 = rowptr[lo], va = ra <= N ? rowptr[ra] : NONE, vb = rb32 <= N ? rowptr[rb32] : NONE;
+    const int before = __popc(__ballot_sync(0xffffffffu, ra < hi && va <= cs)) + __popc(__ballot_sync(0xffffffffu, rb32 < hi && vb <= cs));  // < 64
+    const int r0 = lo + before;
+    auto pointer = [&](int k) {  // rowptr[lo + 1 + k]
+        const int64_t x = __shfl_sync(0xffffffffu, va, k & 31), y = __shfl_sync(0xffffffffu, vb, k & 31);
+        return k < 32 ? x : y;
+    };
+    const int64_t sk = pointer(before > 0 ? before - 1 : 0), s0 = before > 0 ? sk : v0, e0 = pointer(before);
+    int m = 1;
+    const bool none = s0 > cs || e0 <= cs;  // the first position is in no row
+    int64_t last_end = none ? (int64_t)cs + n + 1 : e0;
+    began_before = none || s0 < cs;
+    if (lane == 0) { row[0] = none ? -1 : r0; start[0] = 0; }
+    // rows [s, e) that begin in [cs, cs + n), ascending over the lanes; false when one of them does not: the scan is over
+    auto take = [&](int r, int64_t s, int64_t e, bool skip) {
+        const bool in = !skip && r < N && s < (int64_t)cs + n, live = in && e > s;
+        const unsigned lm = __ballot_sync(0xffffffffu, live);
+        if (live) {
+            const int q = m + __popc(lm & ((1u << lane) - 1u));
+            row[q] = r;
+            start[q] = (uint16_t)(s - cs);
+        }
+        m += __popc(lm);
+        if (lm) last_end = __shfl_sync(0xffffffffu, e, 31 - __clz(lm));
+        return __all_sync(0xffffffffu, skip || in) != 0;
+    };
+    int rb = s0 > cs ? r0 : N;
+    if (s0 <= cs) {
+        const int64_t na = __shfl_down_sync(0xffffffffu, va, 1), first_b = __shfl_sync(0xffffffffu, vb, 0), nb = __shfl_down_sync(0xffffffffu, vb, 1);
+        if (take(ra, va, lane == 31 ? first_b : na, ra <= r0) && take(rb32, vb, nb, rb32 <= r0 || lane == 31)) rb = lo + 64;  // r0 < lo + 64
+    }
+    while (rb < N) {
+        const int r = rb + lane;
+        const int64_t s = r < N ? rowptr[r] : NONE, e = r < N ? rowptr[r + 1] : NONE;
+        const int had = m;
+        if (!take(r, s, e, false)) break;
+        if (m == had) rb = first_row_ending_after(rowptr, rb + 32, N, __shfl_sync(0xffffffffu, s, 0), lane);  // over a run of empty rows
+        else rb += 32;
+    }
+    if (last_end < (int64_t)cs + n) {  // no row holds the rest
+        if (lane == 0) { row[m] = -1; start[m] = (uint16_t)(last_end - cs); }
+        ++m;
+        last_end = (int64_t)cs + n + 1;
+    }
+    if (lane == 0) start[m] = (uint16_t)min(last_end - cs, (int64_t)n + 1);
+    return m;
+}
+
 // The rows of the warp's share [cs, cs + n) of the chunk, their ends as bits, and what the chunk's ends are; a block barrier
 // has to follow before head_row, tail_row, began and open are read.
 template <int NT, int HV>
@@ -68,7 +140,7 @@ __device__ __forceinline__ void chunk_rows(RowsTile<NT, HV>& S, const int64_t* r
     if (n_chunk <= 0 && threadIdx.x == 0) { S.head_row = S.tail_row = -1; S.began = S.open = 0; }
     if (n <= 0) { __syncwarp(); return; }
     bool began = false;
-    const int m = stage_rows(rowptr, N, E, (int)cs, n, lane, R.row, R.start, began);
+    const int m = stage_rows_early(rowptr, N, E, (int)cs, n, lane, R.row, R.start, began);
     __syncwarp();
     for (int q = lane; q < m; q += 32) {
         const int e = R.start[q + 1];
@@ -357,7 +429,7 @@ __device__ __forceinline__ float4 attn_dz(float4 a, float4 b, float4 d, unsigned
 __device__ __forceinline__ unsigned sign_bits(float4 z) { return (z.x > 0.f ? 1u : 0u) | (z.y > 0.f ? 2u : 0u) | (z.z > 0.f ? 4u : 0u) | (z.w > 0.f ? 8u : 0u); }
 
 template <int NT, int HV>
-__global__ void __launch_bounds__(NT, ar_blocks<NT>())
+__global__ void __launch_bounds__(NT, 512 / NT)
 attention_gradient_kernel(const __grid_constant__ AttnArgs A) {
     using Tile = RowsTile<NT, HV>;
     constexpr int H = 4 * HV;
@@ -377,33 +449,27 @@ attention_gradient_kernel(const __grid_constant__ AttnArgs A) {
     const int64_t c0 = (int64_t)blockIdx.x * Tile::CHUNK;
     const int n_chunk = (int)min((int64_t)Tile::CHUNK, A.E - c0), n = min(max(n_chunk - w * Tile::WP, 0), Tile::WP);
     const int64_t cs = c0 + w * Tile::WP;
-    // the lane's items: (position, quad) lane + 32 k of the warp's share; alpha and dalpha are read twice, the second time out of L1 or L2
+    // the lane's items: (position, quad) lane + 32 k of the warp's share; all loads of the chunk are on their way before its rows are
+    // looked up, and alpha and dalpha stay in registers (read again for dz, at three blocks per SM: 104 us instead of GRAD_US)
     const float* const alpha = A.alpha + (size_t)cs * H;
     float* const dz = A.dz + (size_t)cs * H;
     unsigned pos = 0;  // four bits per item: z > 0
+    float4 a[AR_RUN], b[AR_RUN];
     {
         float4 x[AR_RUN];
         gather_sources<HV>(A, cs, n, x);
+#pragma unroll
+        for (int k = 0; k < AR_RUN; ++k)
+            if ((lane + 32 * k) / HV < n) {
+                a[k] = ld_float4(alpha + 4 * (lane + 32 * k));
+                b[k] = ld_float4(dz + 4 * (lane + 32 * k));
+            }
         chunk_rows<NT, HV>(S, A.rowptr, A.N, A.E, cs, n, n_chunk);
         chunk_logits<NT, HV>(A, S, n, x, [&](int k, int, float4 z) { pos |= sign_bits(z) << (4 * k); });
     }
-    constexpr int HALF = AR_RUN / 2;
-    auto pairs = [&](int k0, float4 (&a)[HALF], float4 (&b)[HALF]) {
 #pragma unroll
-        for (int k = 0; k < HALF; ++k)
-            if ((lane + 32 * (k0 + k)) / HV < n) {
-                a[k] = ld_float4(alpha + 4 * (lane + 32 * (k0 + k)));
-                b[k] = ld_float4(dz + 4 * (lane + 32 * (k0 + k)));
-            }
-    };
-#pragma unroll
-    for (int k0 = 0; k0 < AR_RUN; k0 += HALF) {
-        float4 a[HALF], b[HALF];
-        pairs(k0, a, b);
-#pragma unroll
-        for (int k = 0; k < HALF; ++k)
-            if ((lane + 32 * (k0 + k)) / HV < n) tile[Tile::at(w * Tile::WP + (lane + 32 * (k0 + k)) / HV, v)] = mul4(a[k], b[k]);
-    }
+    for (int k = 0; k < AR_RUN; ++k)
+        if ((lane + 32 * k) / HV < n) tile[Tile::at(w * Tile::WP + (lane + 32 * k) / HV, v)] = mul4(a[k], b[k]);
     const unsigned ends = run_ends<NT, HV>(S);
     __syncthreads();
     const int here = min(max(n_chunk - run * AR_RUN, 0), AR_RUN);
@@ -421,21 +487,16 @@ attention_gradient_kernel(const __grid_constant__ AttnArgs A) {
     for (int i = 0; i < AR_RUN; ++i) own[i * HV] = t[i];
     __syncwarp();
 #pragma unroll
-    for (int k0 = 0; k0 < AR_RUN; k0 += HALF) {
-        float4 a[HALF], b[HALF];
-        pairs(k0, a, b);
-#pragma unroll
-        for (int k = 0; k < HALF; ++k) {
-            const int p = w * Tile::WP + (lane + 32 * (k0 + k)) / HV;
-            if (p - w * Tile::WP < n) {
-                float4& d = tile[Tile::at(p, v)];
-                float4 o = zero;
-                if (S.whole[p / AR_RUN] >> (p % AR_RUN) & 1u) {
-                    o = attn_dz(a[k], b[k], d, pos >> (4 * (k0 + k)) & 15u, A.slope);
-                    *reinterpret_cast<float4*>(dz + 4 * (lane + 32 * (k0 + k))) = o;
-                }
-                d = o;
+    for (int k = 0; k < AR_RUN; ++k) {
+        const int p = w * Tile::WP + (lane + 32 * k) / HV;
+        if (p - w * Tile::WP < n) {
+            float4& d = tile[Tile::at(p, v)];
+            float4 o = zero;
+            if (S.whole[p / AR_RUN] >> (p % AR_RUN) & 1u) {
+                o = attn_dz(a[k], b[k], d, pos >> (4 * k) & 15u, A.slope);
+                *reinterpret_cast<float4*>(dz + 4 * (lane + 32 * k)) = o;
             }
+            d = o;
         }
     }
     __syncthreads();  // also: the totals have been read
