@@ -41,6 +41,11 @@ struct RowsTile {
 
 template <bool MAX> __device__ __forceinline__ float comb(float x, float y) { return MAX ? fmaxf(x, y) : x + y; }
 template <bool MAX> __device__ __forceinline__ float4 comb4(float4 x, float4 y) {
+    if (!MAX) {  // two packed additions
+        add2(x.x, x.y, y.x, y.y);
+        add2(x.z, x.w, y.z, y.w);
+        return x;
+    }
     return make_float4(comb<MAX>(x.x, y.x), comb<MAX>(x.y, y.y), comb<MAX>(x.z, y.z), comb<MAX>(x.w, y.w));
 }
 __device__ __forceinline__ float4 shfl4(float4 v, int from) {
@@ -194,10 +199,13 @@ __device__ __forceinline__ void row_totals(RowsTile<NT, HV>& S, float4 (&p)[AR_R
     if (lane == 31) S.warp_closed[w] = f;
     if (lane == 0) {
         unsigned bits = any;
-        if (HV > 1) {  // one bit per run
-            bits = 0;
-#pragma unroll
-            for (int k = 0; k < Tile::RPW; ++k) bits |= (any >> (k * HV) & 1u) << k;
+        static_assert(HV <= 2, "one or two lanes per run");
+        if (HV == 2) {  // one bit per run: the even bits, together
+            bits &= 0x55555555u;
+            bits = (bits | bits >> 1) & 0x33333333u;
+            bits = (bits | bits >> 2) & 0x0f0f0f0fu;
+            bits = (bits | bits >> 4) & 0x00ff00ffu;
+            bits = (bits | bits >> 8) & 0x0000ffffu;
         }
         if (Tile::RPW == 32) S.has_end[w] = bits;
         else reinterpret_cast<uint16_t*>(S.has_end)[w] = (uint16_t)bits;
@@ -214,10 +222,11 @@ __device__ __forceinline__ void row_totals(RowsTile<NT, HV>& S, float4 (&p)[AR_R
     const bool gl = __shfl_sync(0xffffffffu, (int)f, left) != 0;
     const float4 cin = lane < HV ? before : gl ? y : comb4<MAX>(before, y);
     const int fe = __ffs(ends) - 1;
-    float4 first = none;
+    float4 first = p[AR_RUN - 1];
 #pragma unroll
-    for (int i = 0; i < AR_RUN; ++i)
-        if (i == fe) first = comb4<MAX>(cin, p[i]);
+    for (int i = AR_RUN - 2; i >= 0; --i)
+        if (ends >> i & 1u) first = p[i];
+    first = comb4<MAX>(cin, first);
     const float4 ones = make_float4(1.f, 1.f, 1.f, 1.f);
     if (ends != 0) {
         bool earlier = false;  // a row ends in the chunk before this run
@@ -439,13 +448,6 @@ attention_gradient_kernel(const __grid_constant__ AttnArgs A) {
     pdl_wait();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, v = lane % HV, run = w * Tile::RPW + lane / HV;
     const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
-    {  // rows without edges: the blocks share them
-        const int64_t per = ((int64_t)A.N + gridDim.x - 1) / gridDim.x, r0 = per * blockIdx.x, r1 = min(r0 + per, (int64_t)A.N);
-        for (int64_t r = r0 + threadIdx.x; r < r1; r += NT)
-            if (A.rowptr[r + 1] == A.rowptr[r])
-#pragma unroll
-                for (int q = 0; q < HV; ++q) *reinterpret_cast<float4*>(A.dar + (size_t)r * H + 4 * q) = zero;
-    }
     const int64_t c0 = (int64_t)blockIdx.x * Tile::CHUNK;
     const int n_chunk = (int)min((int64_t)Tile::CHUNK, A.E - c0), n = min(max(n_chunk - w * Tile::WP, 0), Tile::WP);
     const int64_t cs = c0 + w * Tile::WP;
@@ -515,6 +517,13 @@ attention_gradient_kernel(const __grid_constant__ AttnArgs A) {
     if (threadIdx.x == 0 && n_chunk > 0) {
         A.parts.head_row[blockIdx.x] = S.head_row;
         A.parts.tail_row[blockIdx.x] = S.tail_row;
+    }
+    {  // rows without edges: the blocks share them
+        const int64_t per = ((int64_t)A.N + gridDim.x - 1) / gridDim.x, r0 = per * blockIdx.x, r1 = min(r0 + per, (int64_t)A.N);
+        for (int64_t r = r0 + threadIdx.x; r < r1; r += NT)
+            if (A.rowptr[r + 1] == A.rowptr[r])
+#pragma unroll
+                for (int q = 0; q < HV; ++q) *reinterpret_cast<float4*>(A.dar + (size_t)r * H + 4 * q) = zero;
     }
 }
 

@@ -548,6 +548,22 @@ __global__ void __launch_bounds__(256) gcn_coef_kernel(const __grid_constant__ C
     }
 }
 
+// rows of one element: four index -> element chains in flight per thread
+template <typename T>
+__global__ void __launch_bounds__(256) permute_elements_kernel(int64_t E, const int32_t* perm, const T* in, T* __restrict__ out) {
+    pdl_wait();
+    const int64_t t0 = blockIdx.x * (int64_t)1024 + threadIdx.x;
+    int32_t p[4];
+    T v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) p[u] = t0 + u * 256 < E ? perm[t0 + u * 256] : 0;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = in[p[u]];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (t0 + u * 256 < E) out[t0 + u * 256] = v[u];
+}
+
 template <typename T>
 __global__ void permute_rows_kernel(int64_t E, int width, const int32_t* perm,
                                     const T* in, T* __restrict__ out) {
@@ -575,6 +591,14 @@ __global__ void add_self_loops_kernel(int32_t N, int64_t E, const int32_t* src,
         }
         else { so[k] = (int32_t)(k - E); dout[k] = (int32_t)(k - E); }
     }
+}
+
+void launch_gather_rows(const int32_t* idx, int64_t E, const void* X, int nvec, void* out, cudaStream_t st);  // edge_ops.cu
+
+template <typename T>
+static void launch_permute(int64_t E, int width, const int32_t* perm, const void* in, void* out, cudaStream_t st) {
+    if (width == 1) launch_overlapped(permute_elements_kernel<T>, dim3((unsigned)ceil_div(E, 1024)), dim3(256), 0, st, E, perm, (const T*)in, (T*)out);
+    else launch_overlapped(permute_rows_kernel<T>, dim3((unsigned)grid_for(E * width, 256)), dim3(256), 0, st, E, width, perm, (const T*)in, (T*)out);
 }
 
 }  // namespace gnn
@@ -743,7 +767,7 @@ gnn_status gnn_gcn_norm(const gnn_csr* g, const float* w_csr, float* deg_out, fl
         A.w = w_csr; A.deg = deg_out; A.N = g->N; A.E = g->E;
         launch_overlapped(gcn_coef_kernel, dim3((unsigned)ceil_div(g->E, 256 * 8), both ? 2 : 1), dim3(256), 0, st, A);
         if (coef_csrT && !both)
-            launch_overlapped(permute_rows_kernel<uint32_t>, dim3((unsigned)grid_for(g->E, 256)), dim3(256), 0, st, g->E, 1, g->t2f, (const uint32_t*)coef_csr, (uint32_t*)coef_csrT);
+            launch_permute<uint32_t>(g->E, 1, g->t2f, coef_csr, coef_csrT, st);
     }
     GNN_CHECK_LAUNCH("gnn_gcn_norm");
     return GNN_OK;
@@ -755,12 +779,19 @@ gnn_status gnn_permute_edge_data(const int32_t* perm, int64_t E, int width, int 
     if (E == 0) return GNN_OK;
     GNN_REQUIRE(perm && in && out && in != out, GNN_ERR_INVALID_ARG, "gnn_permute_edge_data: null or aliased argument");
     cudaStream_t st = as_stream(stream);
-    int grid = grid_for(E * width, 256);
+    const int64_t row = (int64_t)width * elem_bytes;
+    const bool known = elem_bytes == 1 || elem_bytes == 2 || elem_bytes == 4 || elem_bytes == 8;
+    // whole 16-byte chunks to a thread: 1.6 M rows of four floats 26 -> PERMUTE_US us (an element per thread, a division each)
+    if (known && row % 16 == 0 && row <= 4096 && aligned16(in) && aligned16(out)) {
+        launch_gather_rows(perm, E, in, (int)(row / 16), out, st);
+        GNN_CHECK_LAUNCH("gnn_permute_edge_data");
+        return GNN_OK;
+    }
     switch (elem_bytes) {
-        case 1: launch_overlapped(permute_rows_kernel<uint8_t>, dim3((unsigned)(grid)), dim3(256), 0, st, E, width, perm, (const uint8_t*)in, (uint8_t*)out); break;
-        case 2: launch_overlapped(permute_rows_kernel<uint16_t>, dim3((unsigned)(grid)), dim3(256), 0, st, E, width, perm, (const uint16_t*)in, (uint16_t*)out); break;
-        case 4: launch_overlapped(permute_rows_kernel<uint32_t>, dim3((unsigned)(grid)), dim3(256), 0, st, E, width, perm, (const uint32_t*)in, (uint32_t*)out); break;
-        case 8: launch_overlapped(permute_rows_kernel<uint64_t>, dim3((unsigned)(grid)), dim3(256), 0, st, E, width, perm, (const uint64_t*)in, (uint64_t*)out); break;
+        case 1: launch_permute<uint8_t>(E, width, perm, in, out, st); break;
+        case 2: launch_permute<uint16_t>(E, width, perm, in, out, st); break;
+        case 4: launch_permute<uint32_t>(E, width, perm, in, out, st); break;
+        case 8: launch_permute<uint64_t>(E, width, perm, in, out, st); break;
         default: GNN_FAIL(GNN_ERR_UNSUPPORTED, "gnn_permute_edge_data: elem_bytes must be 1, 2, 4 or 8");
     }
     GNN_CHECK_LAUNCH("gnn_permute_edge_data");

@@ -286,6 +286,11 @@ __global__ void axpby_kernel(float alpha, const uint4* a, float beta, const uint
     }
 }
 
+// out[k, :] = X[idx[k], :], rows of nvec 16-byte chunks
+void launch_gather_rows(const int32_t* idx, int64_t E, const void* X, int nvec, void* out, cudaStream_t st) {
+    launch_overlapped(gather_rows_kernel, pair_grid(E * nvec), dim3(256), 0, st, idx, E, (const uint4*)X, nvec, pair_magic(nvec), (uint4*)out);
+}
+
 }  // namespace gnn
 
 using namespace gnn;
@@ -302,7 +307,7 @@ gnn_status gnn_gather(const int32_t* idx, int64_t E, const void* X, int32_t N, i
     if (E == 0) return GNN_OK;
     GNN_REQUIRE(idx && X && out && aligned16(X) && aligned16(out), GNN_ERR_INVALID_ARG,
                 "%s: null or misaligned argument", who);
-    launch_overlapped(gather_rows_kernel, pair_grid(E * nvec), dim3(256), 0, as_stream(stream), idx, E, (const uint4*)X, nvec, pair_magic(nvec), (uint4*)out);
+    launch_gather_rows(idx, E, X, nvec, out, as_stream(stream));
     GNN_CHECK_LAUNCH(who);
     return GNN_OK;
 }
