@@ -311,7 +311,6 @@ static gnn_status gat_check(const char* who, const gnn_csr* g, int H, int C, gnn
 }
 
 gnn_status gat_alpha(const gnn_csr* g, const float* al, const float* ar, float slope, int H, float* alpha, cudaStream_t st);
-void launch_gather_rows(const int32_t* idx, int64_t E, const void* X, int nvec, void* out, cudaStream_t st);
 bool attention_rows_fit(int64_t E, int H, const void* ws, size_t ws_bytes);
 gnn_status attention_rows(const char* who, const gnn_csr* g, const float* al, const float* ar, float slope, int H, float* alpha, float* dz, float* dar,
                           void* ws, cudaStream_t st);
@@ -431,15 +430,7 @@ gnn_status gnn_gat_fused_backward(const gnn_csr* g, const void* Wx, const float*
         GNN_FAIL(GNN_ERR_CUDA, "%s: launch failed", who);
     }
     // dWx[j,h,:] = sum_q alpha[t2f[q],h]*dOut[colT[q],h,:] + dal[j,h]*a_src[h,:] + dar[j,h]*a_dst[h,:]
-    // Rows of whole 16-byte chunks: the coefficients are brought into the transposed order first (dz is done with), so that the
-    // gather reads them in order, not a 32-byte sector somewhere per position (1.6 M edges, 8 heads x 32 bf16: 148 us).
     HeadExtra hx = {alpha_csr, g->t2f, H, w.dal, w.dar, a_src, a_dst};
-    if (H % 4 == 0 && g->E > 0 && aligned16(alpha_csr)) {
-        launch_gather_rows(g->t2f, g->E, alpha_csr, H / 4, w.dz, st);
-        GNN_CHECK_LAUNCH(who);
-        hx.wh = w.dz;
-        hx.wh_index = nullptr;
-    }
     rc = run_chunked(who, MODE_HEADSUM, g->N, g->E, g->rowptrT, g->colT, nullptr, dOut, dWx, nullptr, nullptr,
                      nullptr, nullptr, 0, F, dtype, w.chunk_ws, w.chunk_bytes, st, &hx);
     side_join(st, side);  // the call's work is complete in the caller's stream only once the side branch is
