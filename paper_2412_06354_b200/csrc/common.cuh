@@ -100,6 +100,14 @@ __device__ __forceinline__ uint4 ld_hint16(const void* p, uint64_t pol) {
                  : "l"(p), "l"(pol));
     return v;
 }
+// VB 16-byte chunks, by one load: 16 or 32 bytes, aligned to their size
+template <int VB> struct Vec16 { uint4 v[VB]; };
+__device__ __forceinline__ void ld_hint(Vec16<1>& x, const void* p, uint64_t pol) { x.v[0] = ld_hint16(p, pol); }
+__device__ __forceinline__ void ld_hint(Vec16<2>& x, const void* p, uint64_t pol) {
+    asm volatile("ld.global.L1::no_allocate.L2::cache_hint.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8], %9;"
+                 : "=r"(x.v[0].x), "=r"(x.v[0].y), "=r"(x.v[0].z), "=r"(x.v[0].w), "=r"(x.v[1].x), "=r"(x.v[1].y), "=r"(x.v[1].z), "=r"(x.v[1].w)
+                 : "l"(p), "l"(pol));
+}
 __device__ __forceinline__ int ld_hint_i32(const int* p, uint64_t pol) {
     int v;
     asm volatile("ld.global.L1::no_allocate.L2::cache_hint.s32 %0, [%1], %2;" : "=r"(v) : "l"(p), "l"(pol));

@@ -45,10 +45,17 @@ struct EdgeStage {
     float inv[MEAN ? ED_SUB + 1 : 1];  // [q] 1 / length of that row
 };
 
-template <typename T, int LPR, int KIND>
-__global__ void __launch_bounds__(RR_WARPS * 32, sizeof(T) == 4 ? 4 : 3)
+// VB: 16-byte chunks per lane.  With two, half as many lanes cover a row, and what is done per position and lane (index, address,
+// load, fold, row end) is done half as often.
+template <typename T, int LPR, int KIND, int VB>
+__global__ void __launch_bounds__(RR_WARPS * 32, VB == 2 ? 2 : sizeof(T) == 4 ? 4 : 3)
 edge_rows_kernel(const __grid_constant__ EdgeParams P) {
-    constexpr int EPC = Chunk<T>::N, NG = 32 / LPR, H = ED_H;
+    constexpr int EPL = Chunk<T>::N, EPC = VB * EPL, NG = 32 / LPR, H = ED_H;
+    using Raw = Vec16<VB>;
+    auto unpack = [](const Raw& r, float* f) {
+#pragma unroll
+        for (int k = 0; k < VB; ++k) Chunk<T>::unpack(r.v[k], f + k * EPL);
+    };
     constexpr bool MEAN = KIND == EDGE_DOT_MEAN, V2 = KIND == EDGE_GATV2;
     __shared__ EdgeStage<MEAN> s_all[RR_WARPS];
     pdl_wait();
@@ -57,7 +64,7 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
     EdgeStage<MEAN>& S = s_all[threadIdx.x >> 5];
     if ((int64_t)c * P.sub >= P.E) return;
     const int cs = c * P.sub, n = (int)min((int64_t)P.sub, P.E - cs);
-    const bool col_lane = li < P.nvec;
+    const bool col_lane = li * VB < P.nvec;
     const int ci = col_lane ? li : 0;
     // skewed as in the segmented reduction: the groups' runs are in different banks, and four entries are one load
     const int L = P.sub / NG, lsh = 31 - __clz(L);
@@ -83,10 +90,10 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
     const int* const Sc = S.col + 4 * g;
     const uint64_t pol_keep = policy_evict_last();
     const uint32_t row_bytes = (uint32_t)P.nvec * 16;
-    const char* const Xl = reinterpret_cast<const char*>(P.X) + (size_t)ci * 16;
-    const char* const Dl = reinterpret_cast<const char*>(P.D) + (size_t)ci * 16;
-    const int span = P.lph == 0 ? LPR : P.lph;  // lanes per result: the whole row, or one head
-    const int head = P.lph == 0 ? 0 : li / P.lph, wstride = P.lph == 0 ? 1 : P.H;
+    const char* const Xl = reinterpret_cast<const char*>(P.X) + (size_t)ci * (16 * VB);
+    const char* const Dl = reinterpret_cast<const char*>(P.D) + (size_t)ci * (16 * VB);
+    const int span = P.lph == 0 ? LPR : P.lph / VB;  // lanes per result: the whole row, or one head
+    const int head = P.lph == 0 ? 0 : li / span, wstride = P.lph == 0 ? 1 : P.H;
     float av[V2 ? EPC : 1];
 #pragma unroll
     for (int j = 0; j < (V2 ? EPC : 1); ++j) av[j] = V2 ? P.a[ci * EPC + j] : 0.f;
@@ -99,33 +106,39 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
         }
         q = lo;
     }
-    auto own = [&](int qq) { return ld_16(Dl + (size_t)(uint32_t)max(S.row[qq], 0) * row_bytes); };
+    auto own = [&](int qq) {
+        Raw r;
+        const char* const p = Dl + (size_t)(uint32_t)max(S.row[qq], 0) * row_bytes;
+#pragma unroll
+        for (int k = 0; k < VB; ++k) r.v[k] = ld_16(p + 16 * k);
+        return r;
+    };
     float d[EPC], sc = 1.0f;
-    uint4 own_next = make_uint4(0u, 0u, 0u, 0u);
+    Raw own_next = {};
     if (a < b) {
-        Chunk<T>::unpack(own(q), d);
+        unpack(own(q), d);
         if (MEAN) sc = S.inv[MEAN ? q : 0];
         if (q + 1 < m) own_next = own(q + 1);
     }
     auto next_row = [&]() {
         ++q;
-        Chunk<T>::unpack(own_next, d);
+        unpack(own_next, d);
         if (MEAN && q < m) sc = S.inv[MEAN ? q : 0];
         if (q + 1 < m) own_next = own(q + 1);
     };
     for (int i = n + lane; i < P.sub; i += 32) S.col[sk(i)] = 0;  // the last warp: positions past the end gather row 0
     __syncwarp();
-    auto issue = [&](uint4* x, int i) {
+    auto issue = [&](Raw* x, int i) {
         const int4 c4 = V2 ? make_int4(Sc[i], Sc[i + 1], Sc[i + 2], Sc[i + 3]) : *reinterpret_cast<const int4*>(Sc + i);
         const int ccs[H] = {c4.x, c4.y, c4.z, c4.w};
 #pragma unroll
-        for (int u = 0; u < H; ++u) x[u] = ld_hint16(Xl + (size_t)(uint32_t)ccs[u] * row_bytes, pol_keep);
+        for (int u = 0; u < H; ++u) ld_hint(x[u], Xl + (size_t)(uint32_t)ccs[u] * row_bytes, pol_keep);
     };
-    auto use = [&](const uint4* xr, unsigned ends, int i) {
+    auto use = [&](const Raw* xr, unsigned ends, int i) {
         float dot[H], scale[MEAN ? H : 1];
         auto one = [&](int u) {
             float x[EPC], t = 0.f, t1 = 0.f;
-            Chunk<T>::unpack(xr[u], x);
+            unpack(xr[u], x);
 #pragma unroll
             for (int j = 0; j < EPC; j += 2) {
                 if (V2) {  // single FMAs: packed ones measured 126 us instead of 119 (register pairs)
@@ -173,7 +186,7 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
         }
     };
     // same trip count in every group (the shuffles are warp-wide); L is a multiple of 2 H
-    uint4 A[H], B[H];
+    Raw A[H], B[H];
     issue(A, a);
     issue(B, a + H);
 #pragma unroll 1
@@ -299,14 +312,22 @@ static void launch_edge_rows(EdgeParams& P, int kind, cudaStream_t st) {
     // positions per warp: fewer on small graphs, so that all SMs have warps
     P.sub = P.E >= 2500 * 1000 ? 256 : P.E >= 512 * 1024 ? 128 : 64;
     const dim3 grid((unsigned)ceil_div(P.E, (int64_t)P.sub * RR_WARPS)), block(RR_WARPS * 32);
-#define GNN_EDGE(L)                                                                                             \
-    kind == EDGE_DOT ? launch_overlapped(edge_rows_kernel<T, L, EDGE_DOT>, grid, block, 0, st, P)               \
-    : kind == EDGE_DOT_MEAN ? launch_overlapped(edge_rows_kernel<T, L, EDGE_DOT_MEAN>, grid, block, 0, st, P)   \
-                            : launch_overlapped(edge_rows_kernel<T, L, EDGE_GATV2>, grid, block, 0, st, P)
-    if (P.nvec <= 4) GNN_EDGE(4);
-    else if (P.nvec <= 8) GNN_EDGE(8);
-    else if (P.nvec <= 16) GNN_EDGE(16);
-    else GNN_EDGE(32);
+#define GNN_EDGE(L, VB)                                                                                             \
+    kind == EDGE_DOT ? launch_overlapped(edge_rows_kernel<T, L, EDGE_DOT, VB>, grid, block, 0, st, P)               \
+    : kind == EDGE_DOT_MEAN ? launch_overlapped(edge_rows_kernel<T, L, EDGE_DOT_MEAN, VB>, grid, block, 0, st, P)   \
+                            : launch_overlapped(edge_rows_kernel<T, L, EDGE_GATV2, VB>, grid, block, 0, st, P)
+    // GATv2 logits of fp32 rows over 256 bytes: 32 bytes to a lane, where rows, heads and matrices are whole multiples of that (1.6 M edges
+    // of 512 bytes: 113 -> 100 us).  Not the plain dots, which have less to do per value (600 k edges: 53 -> 57 us), nor bf16, whose
+    // sixteen values a lane leave no room for a second buffer's worth of loads (512 bytes, eight heads: 105 -> 154 us).
+    if constexpr (sizeof(T) == 4)
+        if (kind == EDGE_GATV2 && P.nvec > 16 && P.nvec % 2 == 0 && P.lph % 2 == 0 && ((reinterpret_cast<uintptr_t>(P.X) | reinterpret_cast<uintptr_t>(P.D)) & 31) == 0) {
+            launch_overlapped(edge_rows_kernel<T, 16, EDGE_GATV2, 2>, grid, block, 0, st, P);
+            return;
+        }
+    if (P.nvec <= 4) GNN_EDGE(4, 1);
+    else if (P.nvec <= 8) GNN_EDGE(8, 1);
+    else if (P.nvec <= 16) GNN_EDGE(16, 1);
+    else GNN_EDGE(32, 1);
 #undef GNN_EDGE
 }
 

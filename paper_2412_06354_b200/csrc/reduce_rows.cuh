@@ -751,28 +751,6 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
             const int r = rb + lane;
             unsigned em = __ballot_sync(0xffffffffu, r < e1 && P.rowptr[r + 1] == P.rowptr[r]);
             em &= (NG == 8 ? 0x01010101u : NG == 4 ? 0x11111111u : NG == 2 ? 0x55555555u : 0xffffffffu) << g;  // group g takes every NG-th
-            if (RANK1) {  // the factors of four rows on their way together: one by one, a load's latency per row at the end of every warp
-                while (em) {
-                    int rows[4];
-                    RankOne f[4];
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        rows[u] = em ? rb + __ffs(em) - 1 : -1;
-                        em &= em - 1;  // (0 stays 0)
-                        f[u] = r1;
-                        if (rows[u] >= 0) {
-                            const size_t k = (size_t)rows[u] * P.H + ((P.vec0 + ci) * EPC) / P.fph;
-                            f[u].l = ld_f32(P.epi_l + k);
-                            f[u].r = ld_f32(P.epi_r + k);
-                        }
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        clear();
-                        if (rows[u] >= 0 && col_lane) finish_row<T, MODE, EPI, RANK1>(P, rows[u], 0, ci, acc, arg, f[u]);
-                    }
-                }
-            }
             while (em) {
                 const int bit = __ffs(em) - 1;
                 em &= em - 1;
