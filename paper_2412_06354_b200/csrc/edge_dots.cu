@@ -318,9 +318,10 @@ static void launch_edge_rows(EdgeParams& P, int kind, cudaStream_t st) {
                             : launch_overlapped(edge_rows_kernel<T, L, EDGE_GATV2, VB>, grid, block, 0, st, P)
     // GATv2 logits of fp32 rows over 256 bytes: 32 bytes to a lane, where rows, heads and matrices are whole multiples of that (1.6 M edges
     // of 512 bytes: 113 -> 100 us).  Not the plain dots, which have less to do per value (600 k edges: 53 -> 57 us), nor bf16, whose
-    // sixteen values a lane leave no room for a second buffer's worth of loads (512 bytes, eight heads: 105 -> 154 us).
+    // sixteen values a lane leave no room for a second buffer's worth of loads (512 bytes, eight heads: 105 -> 154 us), nor heads of fewer
+    // than four such lanes, whose sums cannot be folded together (3 M edges, eight heads of 64 bytes: 188 -> 247 us).
     if constexpr (sizeof(T) == 4)
-        if (kind == EDGE_GATV2 && P.nvec > 16 && P.nvec % 2 == 0 && P.lph % 2 == 0 && ((reinterpret_cast<uintptr_t>(P.X) | reinterpret_cast<uintptr_t>(P.D)) & 31) == 0) {
+        if (kind == EDGE_GATV2 && P.nvec > 16 && P.nvec % 2 == 0 && (P.lph == 0 || P.lph >= 8) && ((reinterpret_cast<uintptr_t>(P.X) | reinterpret_cast<uintptr_t>(P.D)) & 31) == 0) {
             launch_overlapped(edge_rows_kernel<T, 16, EDGE_GATV2, 2>, grid, block, 0, st, P);
             return;
         }
