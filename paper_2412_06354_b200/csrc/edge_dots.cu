@@ -32,6 +32,7 @@ enum { EDGE_DOT = 0, EDGE_DOT_MEAN = 1, EDGE_GATV2 = 2 };
 // Bound by instruction issue for narrow rows and by the gathers (L2 -> SM) for rows of 512 bytes.  Before (4 positions per
 // batch, one batch after the other, 8-byte entries, the row's chunk loaded when it changes) -> now:
 //   100k nodes / 1.6 M edges, 512-byte rows, 8 heads bf16 150 -> 105 us; 123 M edges, 128-byte bf16 rows 2.86 -> 2.4 ms;
+//   bf16 dots by multiply-adds that take bf16 (nothing unpacked, the same bits): 105 -> 96 us and 2.33 -> 2.10 ms there;
 //   GATv2 logits of 100k nodes / 1.6 M edges, 512-byte fp32 rows (a gather per index load, four at a time) 358 -> 113 us.
 constexpr int ED_SUB = 256;  // most positions per warp
 constexpr int ED_H = 4;      // positions per register buffer
@@ -113,16 +114,21 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
         for (int k = 0; k < VB; ++k) r.v[k] = ld_16(p + 16 * k);
         return r;
     };
-    float d[EPC], sc = 1.0f;
-    Raw own_next = {};
+    constexpr bool MIXED = sizeof(T) == 2 && !V2;  // dots of bf16 need no unpacked values
+    float d[MIXED ? 1 : EPC], sc = 1.0f;
+    Raw dr = {}, own_next = {};
+    auto take = [&](const Raw& r) {
+        if constexpr (MIXED) dr = r;
+        else unpack(r, d);
+    };
     if (a < b) {
-        unpack(own(q), d);
+        take(own(q));
         if (MEAN) sc = S.inv[MEAN ? q : 0];
         if (q + 1 < m) own_next = own(q + 1);
     }
     auto next_row = [&]() {
         ++q;
-        unpack(own_next, d);
+        take(own_next);
         if (MEAN && q < m) sc = S.inv[MEAN ? q : 0];
         if (q + 1 < m) own_next = own(q + 1);
     };
@@ -138,9 +144,19 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
         float dot[H], scale[MEAN ? H : 1];
         auto one = [&](int u) {
             float x[EPC], t = 0.f, t1 = 0.f;
-            unpack(xr[u], x);
+            if constexpr (MIXED) {
 #pragma unroll
-            for (int j = 0; j < EPC; j += 2) {
+                for (int k = 0; k < VB; ++k) {
+                    fma_bf16(t, t1, xr[u].v[k].x, dr.v[k].x);
+                    fma_bf16(t, t1, xr[u].v[k].y, dr.v[k].y);
+                    fma_bf16(t, t1, xr[u].v[k].z, dr.v[k].z);
+                    fma_bf16(t, t1, xr[u].v[k].w, dr.v[k].w);
+                }
+            } else {
+                unpack(xr[u], x);
+            }
+#pragma unroll
+            for (int j = 0; j < (MIXED ? 0 : EPC); j += 2) {
                 if (V2) {  // single FMAs: packed ones measured 126 us instead of 119 (register pairs)
                     const float z = x[j] + d[j], z1 = x[j + 1] + d[j + 1];
                     t = fmaf(av[V2 ? j : 0], z > 0.f ? z : P.slope * z, t);

@@ -81,6 +81,18 @@ __device__ __forceinline__ void add2(float& a0, float& a1, float x0, float x1) {
         : "f"(x0), "f"(x1));
 }
 
+// t0 += x.lo * d.lo, t1 += x.hi * d.hi for pairs of bf16: the fused multiply-adds of the unpacked values, without unpacking
+__device__ __forceinline__ void fma_bf16(float& t0, float& t1, uint32_t x, uint32_t d) {
+    asm("{\n\t.reg .b16 xl, xh, dl, dh;\n\tmov.b32 {xl, xh}, %2;\n\tmov.b32 {dl, dh}, %3;\n\t"
+        "fma.rn.f32.bf16 %0, xl, dl, %0;\n\tfma.rn.f32.bf16 %1, xh, dh, %1;\n\t}"
+        : "+f"(t0), "+f"(t1)
+        : "r"(x), "r"(d));
+}
+// t0 += x.lo, t1 += x.hi
+__device__ __forceinline__ void add_bf16(float& t0, float& t1, uint32_t x) {
+    asm("{\n\t.reg .b16 xl, xh;\n\tmov.b32 {xl, xh}, %2;\n\tadd.rn.f32.bf16 %0, xl, %0;\n\tadd.rn.f32.bf16 %1, xh, %1;\n\t}" : "+f"(t0), "+f"(t1) : "r"(x));
+}
+
 // Smallest row r in [lo, N) with rowptr[r + 1] > v, or N: the first row at or after lo that has a
 // position beyond v.  Warp-cooperative (every lane must call it with the same arguments): a look at the
 // next 32 rows, then a 32-way search.

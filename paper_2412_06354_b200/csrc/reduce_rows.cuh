@@ -332,6 +332,7 @@ reduce_rows_kernel(const __grid_constant__ PropParams P, int long_blocks) {
 // 128-byte rows of a weighted sum 2.45 -> 2.26 ms, max over 256-byte rows 8.1 -> 6.6 ms.
 // Row ends as bits beside the indices instead of in their sign: no index to mask, and a batch without an end has nothing to
 // test: 123 M edges, 128-byte bf16 rows 1.96 -> 1.87 ms, sums over 512 fp32 features 37.9 -> 35.4 ms a forward and backward pass.
+// Plain bf16 sums by additions that take bf16 (nothing unpacked, the same bits): 1.36 M edges, 256-byte rows 63.7 -> 60.9 us.
 constexpr int RS_SUB = 256;  // most positions per warp
 constexpr int RS_SKEW = 32;
 
@@ -562,6 +563,13 @@ stream_rows_kernel(const __grid_constant__ PropParams P) {
         }
     };
     auto use = [&](const Buf& B, int u, int i, float w, int t) {  // entry u of the buffer, position i of the piece
+        if constexpr (PLAIN && sizeof(T) == 2) {
+            add_bf16(acc[0], acc[1], B.x[u].x);
+            add_bf16(acc[2], acc[3], B.x[u].y);
+            add_bf16(acc[4], acc[5], B.x[u].z);
+            add_bf16(acc[6], acc[7], B.x[u].w);
+            return;
+        }
         float x[EPC];
         Chunk<T>::unpack(B.x[u], x);
         if (ARG) {
