@@ -32,7 +32,8 @@ enum { EDGE_DOT = 0, EDGE_DOT_MEAN = 1, EDGE_GATV2 = 2 };
 // Bound by instruction issue for narrow rows and by the gathers (L2 -> SM) for rows of 512 bytes.  Before (4 positions per
 // batch, one batch after the other, 8-byte entries, the row's chunk loaded when it changes) -> now:
 //   100k nodes / 1.6 M edges, 512-byte rows, 8 heads bf16 150 -> 105 us; 123 M edges, 128-byte bf16 rows 2.86 -> 2.4 ms;
-//   bf16 dots by multiply-adds that take bf16 (nothing unpacked, the same bits): 105 -> 96 us and 2.33 -> 2.10 ms there;
+//   bf16 dots by multiply-adds that take bf16 (nothing unpacked, the same bits): 105 -> 96 us and 2.33 -> 2.10 ms there, and with
+//   the registers that frees four blocks per SM for rows up to 256 bytes, 1.96 ms (512 bytes: 96 -> 98 us, three it stays); bf16 logits 81 -> 77 us;
 //   GATv2 logits of 100k nodes / 1.6 M edges, 512-byte fp32 rows (a gather per index load, four at a time) 358 -> 113 us.
 constexpr int ED_SUB = 256;  // most positions per warp
 constexpr int ED_H = 4;      // positions per register buffer
@@ -49,7 +50,7 @@ struct EdgeStage {
 // VB: 16-byte chunks per lane.  With two, half as many lanes cover a row, and what is done per position and lane (index, address,
 // load, fold, row end) is done half as often.
 template <typename T, int LPR, int KIND, int VB>
-__global__ void __launch_bounds__(RR_WARPS * 32, VB == 2 ? 2 : sizeof(T) == 4 ? 4 : 3)
+__global__ void __launch_bounds__(RR_WARPS * 32, VB == 2 ? 2 : sizeof(T) == 4 || (KIND == EDGE_DOT && LPR <= 16) ? 4 : 3)
 edge_rows_kernel(const __grid_constant__ EdgeParams P) {
     constexpr int EPL = Chunk<T>::N, EPC = VB * EPL, NG = 32 / LPR, H = ED_H;
     using Raw = Vec16<VB>;
@@ -152,13 +153,23 @@ edge_rows_kernel(const __grid_constant__ EdgeParams P) {
                     fma_bf16(t, t1, xr[u].v[k].z, dr.v[k].z);
                     fma_bf16(t, t1, xr[u].v[k].w, dr.v[k].w);
                 }
+            } else if constexpr (V2 && sizeof(T) == 2) {  // x + d, of which only the sum is used
+#pragma unroll
+                for (int j = 0; j < EPC; ++j) x[j] = d[j];
+#pragma unroll
+                for (int k = 0; k < VB; ++k) {
+                    add_bf16(x[8 * k], x[8 * k + 1], xr[u].v[k].x);
+                    add_bf16(x[8 * k + 2], x[8 * k + 3], xr[u].v[k].y);
+                    add_bf16(x[8 * k + 4], x[8 * k + 5], xr[u].v[k].z);
+                    add_bf16(x[8 * k + 6], x[8 * k + 7], xr[u].v[k].w);
+                }
             } else {
                 unpack(xr[u], x);
             }
 #pragma unroll
             for (int j = 0; j < (MIXED ? 0 : EPC); j += 2) {
                 if (V2) {  // single FMAs: packed ones measured 126 us instead of 119 (register pairs)
-                    const float z = x[j] + d[j], z1 = x[j + 1] + d[j + 1];
+                    const float z = sizeof(T) == 2 ? x[j] : x[j] + d[j], z1 = sizeof(T) == 2 ? x[j + 1] : x[j + 1] + d[j + 1];
                     t = fmaf(av[V2 ? j : 0], z > 0.f ? z : P.slope * z, t);
                     t = fmaf(av[V2 ? j + 1 : 0], z1 > 0.f ? z1 : P.slope * z1, t);
                 } else {
