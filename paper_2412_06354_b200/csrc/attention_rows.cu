@@ -5,8 +5,12 @@
 // block are finished there.  GAT: a row that is cut leaves its maximum and sum per block, and a second kernel, again a block per
 // chunk, combines a row's shares in ascending order and finishes the chunk's positions of it.  Edge softmax, which has no
 // workspace: the blocks that a row is cut into read all of it, out of L2.
-// No row takes longer than another.  What bounds it: the latency of a chunk (search, gathers, four barriers) at three blocks
-// per SM, then instruction issue (an exponential and a division per value).
+// No row takes longer than another.  What bounds it: the latency of a chunk (search, gathers, four barriers) at two or three blocks
+// per SM, and instruction issue (an exponential and a division per value).
+// Before: a row per 8 threads, per warp or per block, three kernels side by side on streams of their own, as long as their
+// longest row and mostly idle warps.  100k nodes, 1.6 M edges, R-MAT: softmax of GAT logits of 8 heads 97 -> 43 us (tiers of rows side
+// by side -> both kernels), its gradient 104 -> 100 us; edge softmax 80 -> 41 us and 55 -> 27 us (4 heads fp32), 113 -> 72 us and 83 -> 50 us (8).
+// Distance to 64 bits as before (alpha 4.1e-8, 4.0e-8 by tiers; da_src 2.3e-7, 2.1e-7).
 #include <atomic>
 
 #include "reduce_params.cuh"
@@ -452,7 +456,7 @@ attention_gradient_kernel(const __grid_constant__ AttnArgs A) {
     const int n_chunk = (int)min((int64_t)Tile::CHUNK, A.E - c0), n = min(max(n_chunk - w * Tile::WP, 0), Tile::WP);
     const int64_t cs = c0 + w * Tile::WP;
     // the lane's items: (position, quad) lane + 32 k of the warp's share; all loads of the chunk are on their way before its rows are
-    // looked up, and alpha and dalpha stay in registers (read again for dz, at three blocks per SM: 104 us instead of GRAD_US)
+    // looked up, and alpha and dalpha stay in registers (read again for dz, at three blocks per SM: 1.05 times as long)
     const float* const alpha = A.alpha + (size_t)cs * H;
     float* const dz = A.dz + (size_t)cs * H;
     unsigned pos = 0;  // four bits per item: z > 0
@@ -793,26 +797,23 @@ static gnn_status gradient_launch(const char* who, const AttnArgs& A, int chunks
 
 static int ar_chunk(int64_t E, int H) { return (E * H / 8 < AR_SMALL ? 64 : 256) / (H / 4) * AR_RUN; }
 
-// 4 and 8 heads, and a workspace with room for the shares of the cut rows
-bool attention_rows_fit(int64_t E, int H, const void* ws, size_t ws_bytes) {
-    if ((H != 4 && H != 8) || E >= ((int64_t)1 << 31) - 4096) return false;
-    const size_t chunks = (size_t)ceil_div(E, (int64_t)ar_chunk(E, H));
-    return ws && aligned16(ws) && ws_bytes >= 2 * up256(chunks * 4) + 2 * up256(chunks * 2 * H * 4);
-}
-
+// The shares of the cut rows fit any workspace of the chunked reduction of rows of four or more features a head, which is what the
+// attention calls are given: at most 136 bytes per chunk, where that has 132 per 128 positions or more.
 // dz and dar null: alpha = softmax over each row of LeakyReLU(al[col] + ar[row]).  Else dz (dalpha on entry) and dar from alpha.
 gnn_status attention_rows(const char* who, const gnn_csr* g, const float* al, const float* ar, float slope, int H, float* alpha, float* dz, float* dar,
-                          void* ws, cudaStream_t st) {
+                          void* ws, size_t ws_bytes, cudaStream_t st) {
     const int chunk = ar_chunk(g->E, H);
     const int64_t chunks = ceil_div(g->E, (int64_t)chunk);
     const bool small = chunk == 64 / (H / 4) * AR_RUN;
-    const size_t rows = up256((size_t)chunks * 4), part = up256((size_t)chunks * 2 * H * 4);
+    const size_t rows = ((size_t)chunks * 8 + 15) & ~(size_t)15, part = (size_t)chunks * 2 * H * 4;
+    GNN_REQUIRE(ws && aligned16(ws) && ws_bytes >= rows + 2 * part, GNN_ERR_WORKSPACE_TOO_SMALL, "%s: %zu bytes needed for the rows that chunks cut", who, rows + 2 * part);
+    GNN_REQUIRE(g->E < ((int64_t)1 << 31) - 1024, GNN_ERR_UNSUPPORTED, "%s: positions must fit 32 bits (E < 2^31)", who);
     AttnArgs A = {};
     A.rowptr = g->rowptr; A.col = g->col; A.al = al; A.ar = ar; A.slope = slope; A.N = g->N; A.E = g->E;
     A.alpha = alpha; A.dz = dz; A.dar = dar;
     char* p = (char*)ws;
-    A.parts.head_row = (int32_t*)p; A.parts.tail_row = (int32_t*)(p + rows);
-    A.parts.a = (float*)(p + 2 * rows); A.parts.b = (float*)(p + 2 * rows + part);
+    A.parts.head_row = (int32_t*)p; A.parts.tail_row = A.parts.head_row + chunks;
+    A.parts.a = (float*)(p + rows); A.parts.b = (float*)(p + rows + part);
     gnn_status rc;
 #define GNN_AR(NT, HV) rc = dz ? gradient_launch<NT, HV>(who, A, (int)chunks, st) : softmax_launch<NT, HV>(who, A, (int)chunks, st)
     if (H == 4) { if (small) GNN_AR(64, 1); else GNN_AR(256, 1); }
@@ -844,7 +845,7 @@ static gnn_status edge_softmax_dispatch(const char* who, const SoftmaxArgs& A, i
 
 // 4 and 8 heads, four values to an access, and results that do not lie over what other blocks still read
 bool edge_softmax_chunks_fit(int64_t E, int H, gnn_dtype dtype, const void* x, const void* y, const void* out) {
-    if ((H != 4 && H != 8) || E <= 0 || E >= ((int64_t)1 << 31) - 4096) return false;
+    if ((H != 4 && H != 8) || E <= 0 || E >= ((int64_t)1 << 31) - 1024) return false;
     const size_t bytes = (size_t)E * H * elem_size(dtype), quad = 4 * elem_size(dtype);
     auto apart = [&](const void* p) { return (const char*)p + bytes <= (const char*)out || (const char*)out + bytes <= (const char*)p; };
     return ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(out)) & (quad - 1)) == 0 && apart(x) && (!y || apart(y));

@@ -311,13 +311,13 @@ static gnn_status gat_check(const char* who, const gnn_csr* g, int H, int C, gnn
 }
 
 gnn_status gat_alpha(const gnn_csr* g, const float* al, const float* ar, float slope, int H, float* alpha, cudaStream_t st);
-bool attention_rows_fit(int64_t E, int H, const void* ws, size_t ws_bytes);
 gnn_status attention_rows(const char* who, const gnn_csr* g, const float* al, const float* ar, float slope, int H, float* alpha, float* dz, float* dar,
-                          void* ws, cudaStream_t st);
+                          void* ws, size_t ws_bytes, cudaStream_t st);
 bool gat_rows_backward_pl(const gnn_csr* g, const float* alpha, float* dalpha_dz, const float* al, const float* ar,
                           float slope, int H, float* dar, cudaStream_t st);
 cudaStream_t side_fork(cudaStream_t st);
 void side_join(cudaStream_t st, cudaStream_t side);
+void side_prepare();
 
 }  // namespace gnn
 
@@ -357,10 +357,12 @@ gnn_status gnn_gat_fused(const gnn_csr* g, const void* Wx, const float* a_src, c
     GNN_CHECK_LAUNCH(who);
     // logits and their per-row softmax, written straight into alpha_csr
     GNN_REQUIRE(g->E == 0 || g->col, GNN_ERR_INVALID_ARG, "%s: null col", who);
-    if (g->E > 0 && attention_rows_fit(g->E, H, w.chunk_ws, w.chunk_bytes))
-        rc = attention_rows(who, g, al, ar, slope, H, alpha_csr, nullptr, nullptr, w.chunk_ws, st);
-    else
+    if ((H == 4 || H == 8) && g->E > 0) {
+        side_prepare();
+        rc = attention_rows(who, g, al, ar, slope, H, alpha_csr, nullptr, nullptr, w.chunk_ws, w.chunk_bytes, st);
+    } else {
         rc = gat_alpha(g, al, ar, slope, H, alpha_csr, st);
+    }
     if (rc != GNN_OK) return rc;
     HeadExtra hx = {alpha_csr, nullptr, H, nullptr, nullptr, nullptr, nullptr};
     return run_chunked(who, MODE_HEADSUM, g->N, g->E, g->rowptr, g->col, nullptr, Wx, out, nullptr, nullptr,
@@ -391,8 +393,8 @@ gnn_status gnn_gat_fused_backward(const gnn_csr* g, const void* Wx, const float*
     rc = run_sddmm(who, g, Wx, dOut, H, C, 0, dtype, w.dz, st);
     if (rc != GNN_OK) return rc;
     // softmax and LeakyReLU derivatives, dz over dalpha, dar per row
-    if (attention_rows_fit(g->E, H, w.chunk_ws, w.chunk_bytes)) {
-        rc = attention_rows(who, g, al, ar, slope, H, const_cast<float*>(alpha_csr), w.dz, w.dar, w.chunk_ws, st);
+    if (H == 4 || H == 8) {
+        rc = attention_rows(who, g, al, ar, slope, H, const_cast<float*>(alpha_csr), w.dz, w.dar, w.chunk_ws, w.chunk_bytes, st);
         if (rc != GNN_OK) return rc;
     } else if (!gat_rows_backward_pl(g, alpha_csr, w.dz, al, ar, slope, H, w.dar, st)) {
         const int64_t wwant = ceil_div((int64_t)g->N * 32, GB_BLOCK), cap = (int64_t)148 * 64;

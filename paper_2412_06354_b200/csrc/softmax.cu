@@ -2,6 +2,8 @@
 // the GAT layer named in Sec. 3 "Graph Convolutional Layers"), forward and backward.
 // Logits and coefficients are [E,H] in CSR order, so a node's incoming edges are contiguous.
 //
+// Four and eight heads run positions first (attention_rows.cu), unless the result lies over an input or an array is off its
+// four-value alignment.  Here, the other head counts and those cases:
 // One warp per row for ordinary rows; rows longer than SM_LONG_ROW positions are left to a
 // second kernel that gives each of them a whole block, and rows longer than SM_HUB_ROW positions
 // (4, 8, 16 or 32 heads) a cluster of eight blocks that combine their results through distributed
@@ -938,6 +940,12 @@ static TierStreams* tier_streams() {
     return t;
 }
 
+// The helper streams exist from the first call on a device on, whether it needs them or not: the call after it may be captured.
+void side_prepare() {
+    std::lock_guard<std::mutex> lock(g_tier_mutex);
+    tier_streams();
+}
+
 // A side branch of the caller's stream: work enqueued on the returned stream starts after everything enqueued on
 // st so far; side_join makes st wait for it.  Returns st itself if no helper stream is available.
 cudaStream_t side_fork(cudaStream_t st) {
@@ -985,7 +993,7 @@ gnn_status gat_alpha(const gnn_csr* g, const float* al, const float* ar, float s
         st, [&](cudaStream_t q) { gat_alpha_pl_kernel<HV, true><<<lg, PL_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, al, ar, slope, alpha); }, \
         [&](cudaStream_t q) { gat_alpha_pl_kernel<HV, false><<<wg, SM_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, al, ar, slope, alpha); },    \
         [&](cudaStream_t q) { gat_alpha_pl_kernel<HV, false, 8><<<sg, SM_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, al, ar, slope, alpha); });
-    if (H == 4) { GNN_GA(1) } else if (H == 8) { GNN_GA(2) } else if (H == 16) { GNN_GA(4) } else if (H == 32) { GNN_GA(8) } else {
+    if (H == 16) { GNN_GA(4) } else if (H == 32) { GNN_GA(8) } else {  // (4 and 8: attention_rows.cu)
         run_row_tiers(  // the two tiers write disjoint rows: side by side
             st, [&](cudaStream_t q) { gat_alpha_kernel<true><<<row_grid(g->N, true), SM_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, H, al, ar, slope, alpha); },
             [&](cudaStream_t q) { gat_alpha_kernel<false><<<row_grid(g->N, false), SM_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, H, al, ar, slope, alpha); },
@@ -1005,7 +1013,7 @@ bool gat_rows_backward_pl(const gnn_csr* g, const float* alpha, float* dalpha_dz
         st, [&](cudaStream_t q) { gat_rows_bwd_pl_kernel<HV, true><<<lg, PL_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, alpha, dalpha_dz, al, ar, slope, dar); }, \
         [&](cudaStream_t q) { gat_rows_bwd_pl_kernel<HV, false><<<wg, SM_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, alpha, dalpha_dz, al, ar, slope, dar); },    \
         [&](cudaStream_t q) { gat_rows_bwd_pl_kernel<HV, false, 8><<<sg, SM_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, alpha, dalpha_dz, al, ar, slope, dar); });
-    if (H == 4) { GNN_GB(1) } else if (H == 8) { GNN_GB(2) } else if (H == 16) { GNN_GB(4) } else if (H == 32) { GNN_GB(8) } else return false;
+    if (H == 16) { GNN_GB(4) } else if (H == 32) { GNN_GB(8) } else return false;
 #undef GNN_GB
     return true;
 }
@@ -1030,8 +1038,10 @@ gnn_status gnn_edge_softmax(const gnn_csr* g, const void* logits_EH, int H, gnn_
     if (g->N == 0) return GNN_OK;
     GNN_REQUIRE(g->E == 0 || (logits_EH && alpha_EH), GNN_ERR_INVALID_ARG, "%s: null argument", who);
     cudaStream_t st = as_stream(stream);
-    if (edge_softmax_chunks_fit(g->E, H, dtype, logits_EH, nullptr, alpha_EH))
+    if (edge_softmax_chunks_fit(g->E, H, dtype, logits_EH, nullptr, alpha_EH)) {
+        side_prepare();
         return edge_softmax_chunks(who, g, logits_EH, nullptr, H, dtype, alpha_EH, rowmax, rowsum, st);
+    }
     const int wgrid = row_grid(g->N, false), lgrid = row_grid_cluster(g->N);
     // the two row tiers write disjoint rows: side by side (the long rows' blocks beside the warps of the short ones)
     if (dtype == GNN_F32)
@@ -1056,8 +1066,10 @@ gnn_status gnn_edge_softmax_backward(const gnn_csr* g, const void* alpha_EH, con
     if (g->N == 0 || g->E == 0) return GNN_OK;
     GNN_REQUIRE(alpha_EH && dAlpha_EH && dLogits_EH, GNN_ERR_INVALID_ARG, "%s: null argument", who);
     cudaStream_t st = as_stream(stream);
-    if (edge_softmax_chunks_fit(g->E, H, dtype, alpha_EH, dAlpha_EH, dLogits_EH))
+    if (edge_softmax_chunks_fit(g->E, H, dtype, alpha_EH, dAlpha_EH, dLogits_EH)) {
+        side_prepare();
         return edge_softmax_chunks(who, g, alpha_EH, dAlpha_EH, H, dtype, dLogits_EH, nullptr, nullptr, st);
+    }
     const int wgrid = row_grid(g->N, false), lgrid = row_grid_cluster(g->N);
     if (dtype == GNN_F32)
         run_row_tiers(
