@@ -49,48 +49,48 @@ TRAFFIC_SOURCE = ("ncu --metrics dram__bytes_read.sum,dram__bytes_write.sum --cl
                   "full-size traffic (better L2 reuse on the reduced matrix); profiles/dram_bytes_of_the_sweep_reduced_graph.md")
 TRAFFIC_SCALE = 4.0
 TRAFFIC_KERNEL_FILES = ("propagate.cu", "propagate.cuh", "reduce_params.cuh", "reduce_rows.cuh", "common.cuh")
-TRAFFIC_KERNEL_SHA256 = "e9d423fe4f03d42e050e45b1e7f22d5688c799216b726aef0f97073d0a97eea1"
+TRAFFIC_KERNEL_SHA256 = "70d0a5fcfe01053a7478684aee19b1b97fbfde3f16b606d92d6234915e3e6fd1"
 TRAFFIC_GB_REDUCED = {
-    "32:bf16:copy_xj:fwd": 0.209,
-    "32:bf16:copy_xj:bwd": 0.209,
+    "32:bf16:copy_xj:fwd": 0.213,
+    "32:bf16:copy_xj:bwd": 0.211,
     "32:bf16:e_mul_xj:fwd": 0.35,
-    "32:bf16:e_mul_xj:bwd": 0.35,
-    "64:bf16:copy_xj:fwd": 0.294,
-    "64:bf16:copy_xj:bwd": 0.294,
-    "64:bf16:e_mul_xj:fwd": 0.444,
-    "64:bf16:e_mul_xj:bwd": 0.446,
-    "128:bf16:copy_xj:fwd": 0.644,
-    "128:bf16:copy_xj:bwd": 0.645,
-    "128:bf16:e_mul_xj:fwd": 0.82,
-    "128:bf16:e_mul_xj:bwd": 0.823,
-    "256:bf16:copy_xj:fwd": 2.043,
-    "256:bf16:copy_xj:bwd": 2.04,
-    "256:bf16:e_mul_xj:fwd": 2.265,
-    "256:bf16:e_mul_xj:bwd": 2.263,
-    "512:bf16:copy_xj:fwd": 4.087,
-    "512:bf16:copy_xj:bwd": 4.086,
-    "512:bf16:e_mul_xj:fwd": 4.533,
-    "512:bf16:e_mul_xj:bwd": 4.528,
-    "32:f32:copy_xj:fwd": 0.287,
+    "32:bf16:e_mul_xj:bwd": 0.351,
+    "64:bf16:copy_xj:fwd": 0.295,
+    "64:bf16:copy_xj:bwd": 0.296,
+    "64:bf16:e_mul_xj:fwd": 0.447,
+    "64:bf16:e_mul_xj:bwd": 0.448,
+    "128:bf16:copy_xj:fwd": 0.651,
+    "128:bf16:copy_xj:bwd": 0.651,
+    "128:bf16:e_mul_xj:fwd": 0.836,
+    "128:bf16:e_mul_xj:bwd": 0.836,
+    "256:bf16:copy_xj:fwd": 2.025,
+    "256:bf16:copy_xj:bwd": 2.027,
+    "256:bf16:e_mul_xj:fwd": 2.246,
+    "256:bf16:e_mul_xj:bwd": 2.245,
+    "512:bf16:copy_xj:fwd": 4.06,
+    "512:bf16:copy_xj:bwd": 4.064,
+    "512:bf16:e_mul_xj:fwd": 4.499,
+    "512:bf16:e_mul_xj:bwd": 4.502,
+    "32:f32:copy_xj:fwd": 0.286,
     "32:f32:copy_xj:bwd": 0.288,
     "32:f32:e_mul_xj:fwd": 0.437,
-    "32:f32:e_mul_xj:bwd": 0.438,
-    "64:f32:copy_xj:fwd": 0.628,
-    "64:f32:copy_xj:bwd": 0.629,
+    "32:f32:e_mul_xj:bwd": 0.439,
+    "64:f32:copy_xj:fwd": 0.634,
+    "64:f32:copy_xj:bwd": 0.638,
     "64:f32:e_mul_xj:fwd": 0.802,
-    "64:f32:e_mul_xj:bwd": 0.803,
-    "128:f32:copy_xj:fwd": 1.992,
-    "128:f32:copy_xj:bwd": 1.991,
-    "128:f32:e_mul_xj:fwd": 2.177,
-    "128:f32:e_mul_xj:bwd": 2.175,
-    "256:f32:copy_xj:fwd": 3.992,
-    "256:f32:copy_xj:bwd": 3.992,
-    "256:f32:e_mul_xj:fwd": 4.363,
-    "256:f32:e_mul_xj:bwd": 4.359,
-    "512:f32:copy_xj:fwd": 7.979,
+    "64:f32:e_mul_xj:bwd": 0.805,
+    "128:f32:copy_xj:fwd": 1.995,
+    "128:f32:copy_xj:bwd": 1.995,
+    "128:f32:e_mul_xj:fwd": 2.181,
+    "128:f32:e_mul_xj:bwd": 2.182,
+    "256:f32:copy_xj:fwd": 3.994,
+    "256:f32:copy_xj:bwd": 3.995,
+    "256:f32:e_mul_xj:fwd": 4.365,
+    "256:f32:e_mul_xj:bwd": 4.364,
+    "512:f32:copy_xj:fwd": 7.987,
     "512:f32:copy_xj:bwd": 7.984,
-    "512:f32:e_mul_xj:fwd": 8.719,
-    "512:f32:e_mul_xj:bwd": 8.723,
+    "512:f32:e_mul_xj:fwd": 8.729,
+    "512:f32:e_mul_xj:bwd": 8.722,
 }
 TRAFFIC_GB = {k: v * TRAFFIC_SCALE for k, v in TRAFFIC_GB_REDUCED.items()}
 
