@@ -319,3 +319,34 @@ def test_edge_tensor_tiles(gnn, e, dtype, F):
     off.copy_(to_dev(arg))
     for a in (to_dev(arg), off):
         assert np.array_equal(to_host64(gnn.aggregate_backward(g, to_dev(R), "max", argmax=a)), want)
+
+
+# Rows of whole 16-byte chunks, single elements (four to a thread) and other widths; perm of one block less, exactly and more
+@pytest.mark.parametrize("e", [1, 1023, 1024, 1025, 70_001])
+@pytest.mark.parametrize("width,dtype", [(1, "int32"), (1, "uint8"), (3, "float32"), (4, "float32"), (8, "float32"), (8, "bfloat16"), (2, "float64"), (16, "uint8")])
+def test_permuted_edge_data(gnn, e, width, dtype):
+    import torch
+    perm = torch.randperm(e, device="cuda").to(torch.int32)
+    data = torch.randint(0, 200, (e + 1, width) if width > 1 else (e + 1,), device="cuda").to(getattr(torch, dtype))[1:]  # (off 16 bytes where a row is less)
+    out = gnn.permute_edge_data(perm, data)
+    assert torch.equal(out, data[perm.long()])
+
+
+# fp32 rows over 256 bytes take 32 bytes per lane where matrices lie on 32 bytes, 16 otherwise: one warp's share of positions less, exactly and more
+@pytest.mark.parametrize("e", [1, 63, 64, 65, 513, 6001])
+@pytest.mark.parametrize("H,C", [(1, 128), (4, 32), (2, 64), (1, 72), (8, 16)])
+def test_gatv2_logits_lane_widths(gnn, e, H, C):
+    import torch
+    rng = np.random.default_rng(e)
+    n, F = 97, H * C
+    src, dst = rng.integers(0, n, e).astype(np.int32), np.sort(rng.integers(0, n, e).astype(np.int32))
+    g = build_graph(gnn, n, src, dst)
+    eid = host_csr(n, src, dst)["eid"]
+    Xl, Xr, a = feats((n, F), "f32", 70), feats((n, F), "f32", 71), feats((H, C), "f32", 72)
+    z = synth.to_f64(Xl)[src] + synth.to_f64(Xr)[dst]
+    terms = (np.where(z > 0, z, 0.2 * z) * synth.to_f64(a).reshape(1, F)).reshape(e, H, C)
+    for off in (0, 4):  # elements before the matrix
+        room = torch.zeros(n * F + off, device="cuda")
+        room[off:] = to_dev(Xl).reshape(-1)
+        got = gnn.gatv2_logits(g, room[off:].view(n, F), to_dev(Xr), to_dev(a), H, 0.2)
+        assert_close(to_host64(got).reshape(e, H), terms.sum(-1)[eid], np.abs(terms).sum(-1)[eid], "f32", f"logits, offset {off}")
