@@ -12,6 +12,7 @@
 // by side -> both kernels), its gradient 104 -> 100 us; edge softmax 80 -> 41 us and 55 -> 27 us (4 heads fp32), 113 -> 72 us and 83 -> 50 us (8).
 // Distance to 64 bits as before (alpha 4.1e-8, 4.0e-8 by tiers; da_src 2.3e-7, 2.1e-7).
 #include <atomic>
+#include <cfloat>
 
 #include "reduce_params.cuh"
 #include "tc_common.cuh"
@@ -373,8 +374,11 @@ attention_softmax_kernel(const __grid_constant__ AttnArgs A) {
     const int here = min(max(n_chunk - run * AR_RUN, 0), AR_RUN);  // positions of this run
     float4 t[AR_RUN];  // (the values stay in the tile: with them in registers too an SM holds two blocks)
     float4* const own = tile + Tile::at(run * AR_RUN, v);  // positions HV apart
+    // The maximum of nothing but -inf counts as the lowest finite value: the exponentials are 0 then, not NaN, and so is the share that a
+    // row has in a chunk where all its logits are -inf.  A row of nothing else comes to 0 / 0.
+    const float4 lowest = make_float4(-FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX);
 #pragma unroll
-    for (int i = 0; i < AR_RUN; ++i) t[i] = i < here ? own[i * HV] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    for (int i = 0; i < AR_RUN; ++i) t[i] = i < here ? comb4<true>(lowest, own[i * HV]) : lowest;
     const bool cut_head = S.head_row >= 0;
     // the open row's share is the chunk's tail where the row begins here, else its head
     float* const head = A.parts.a + (size_t)blockIdx.x * 2 * H;

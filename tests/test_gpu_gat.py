@@ -17,7 +17,8 @@ def gnn():
     return g
 
 
-def run_case(gnn, n, src, dst, Wx, a_s, a_d, H, C, dtype, what):
+def run_case(gnn, n, src, dst, Wx, a_s, a_d, H, C, dtype, what, masked=()):
+    """masked: nodes whose scores al are below the range of fp32"""
     F = H * C
     g = build_graph(gnn, n, src, dst)
     eid = g.eid[:g.E].cpu().numpy() if g.E else np.zeros(0, np.int64)
@@ -26,7 +27,9 @@ def run_case(gnn, n, src, dst, Wx, a_s, a_d, H, C, dtype, what):
     x64 = synth.to_f64(Wx).reshape(n, H, C)
     Sal = np.einsum("nhc,hc->nh", np.abs(x64), np.abs(a_s.astype(np.float64)))
     Sar = np.einsum("nhc,hc->nh", np.abs(x64), np.abs(a_d.astype(np.float64)))
-    assert_close(to_host64(fwd["al"]), ref["al"], Sal, "f32", what + " al")
+    seen = np.setdiff1d(np.arange(n), masked)
+    assert_close(to_host64(fwd["al"])[seen], ref["al"][seen], Sal[seen], "f32", what + " al")
+    assert np.all(to_host64(fwd["al"])[np.asarray(masked, int)] == -np.inf)
     assert_close(to_host64(fwd["ar"]), ref["ar"], Sar, "f32", what + " ar")
     if g.E:
         # a coefficient moves by about (error of its logit) * alpha; the logit is a two-dot-product sum
@@ -133,6 +136,41 @@ def test_gat_and_softmax_rows_at_chunk_ends(gnn, H, chunk, edges):
         assert_close(to_host64(own), ao[eid], ao[eid], dtype, "alpha over the logits")
         gnn._check(gnn.load().gnn_edge_softmax_backward(gnn.C.byref(g.c), gnn._p(alpha), gnn._p(upstream), H, gnn._dtype(own), gnn._p(upstream), gnn._stream()))
         assert_close(to_host64(upstream), dso[eid], S[eid], dtype, "dlogits over dalpha")
+
+
+# Logits of -inf (scores that overflow) take no part in their rows, wherever the chunks cut them: a single position past a chunk's end, a
+# chunk's whole share in the middle or at the beginning of a row, scattered ones.
+@pytest.mark.parametrize("H,chunk,edges", [(4, 512, 9_001), (8, 256, 6_611), (8, 1024, 420_003), (4, 2048, 830_011)])
+def test_gat_scores_of_minus_infinity(gnn, H, chunk, edges):
+    rng = np.random.default_rng(edges)
+    degree = [chunk + 1, 3 * chunk, 2 * chunk]
+    while sum(degree) < edges:
+        degree.append(min(int(rng.integers(1, 3000)), edges - sum(degree)))
+    n, C = max(len(degree), 500), 8
+    dst = np.repeat(np.arange(len(degree), dtype=np.int32), degree)  # positions in the order of the edge list
+    hidden = np.arange(n - 5, n)
+    src = rng.integers(0, n - 5, edges).astype(np.int32)
+    away = rng.random(edges) < 0.05
+    away[np.cumsum(degree) - 1] = False  # no row of nothing else
+    away[chunk] = True
+    away[2 * chunk:3 * chunk] = True
+    away[4 * chunk + 1:5 * chunk] = True
+    src[away] = rng.choice(hidden, away.sum())
+    Wx = synth.normal((n, H * C), "f32", 920 + H, 1).reshape(n, H, C)
+    Wx[:, :, 0] = 0.0
+    Wx[hidden, :, 0] = -1e37
+    a_s = synth.uniform_f32((H, C), -0.8, 0.8, 921, 1)
+    a_d = synth.uniform_f32((H, C), -0.8, 0.8, 922, 1)
+    a_s[:, 0], a_d[:, 0] = 100.0, 0.0
+    Wx = Wx.reshape(n, H * C)
+    _, fwd = run_case(gnn, n, src, dst, Wx, a_s, a_d, H, C, "f32", f"gat H={H}, chunks of {chunk}, scores of -inf", masked=hidden)
+    # rows of nothing but -inf, cut and whole, are NaN; the others are what they were
+    rows = np.array([1, 3, 5])
+    src[np.isin(dst, rows)] = hidden[0]
+    alpha = to_host64(gnn.gat_fused(build_graph(gnn, n, src, dst), to_dev(Wx), to_dev(a_s), to_dev(a_d), H)["alpha"])
+    assert np.isnan(alpha[np.isin(dst, rows)]).all()
+    others = ~np.isin(dst, rows)
+    assert np.array_equal(alpha[others], to_host64(fwd["alpha"])[others])
 
 
 def test_gat_zero_attention_is_mean_aggregation(gnn):
