@@ -5,7 +5,8 @@
 // block are finished there.  GAT: a row that is cut leaves its maximum and sum per block, and a second kernel, again a block per
 // chunk, combines a row's shares in ascending order and finishes the chunk's positions of it.  Edge softmax, which has no
 // workspace: the blocks that a row is cut into read all of it, out of L2.
-// No row takes longer than another.  What bounds it: the latency of a chunk (search, gathers, four barriers) at two or three blocks
+// Rows of more than AR_SPAN chunks are left to clusters (softmax.cu), which read them once per pass: the blocks together would read a row of k chunks
+// k times (8 heads fp32, a row of 330 k positions among 1.9 M 632 -> 200 us, of 2.4 M 20 -> 1.8 ms).  What bounds it: the latency of a chunk (search, gathers, four barriers) at two or three blocks
 // per SM, and instruction issue (an exponential and a division per value).
 // Before: a row per 8 threads, per warp or per block, three kernels side by side on streams of their own, as long as their
 // longest row and mostly idle warps.  100k nodes, 1.6 M edges, R-MAT: softmax of GAT logits of 8 heads 97 -> 43 us (tiers of rows side
@@ -611,6 +612,7 @@ struct SoftmaxArgs {
     float *rowmax, *rowsum;  // [N,H] or nullptr
     int32_t N;
     int64_t E;
+    int64_t over;  // rows of more positions are left to others
 };
 
 // v over the threads of a quad: lanes, then warps in order
@@ -628,7 +630,9 @@ __device__ __forceinline__ float4 block_quads(RowsTile<NT, HV>& S, float4 v) {
     return v;
 }
 __device__ __forceinline__ void put_stats(float* to, size_t at, float4 v) {  // (any alignment)
-    if (to) { to[at] = v.x; to[at + 1] = v.y; to[at + 2] = v.z; to[at + 3] = v.w; }
+    if (!to) return;
+    if ((reinterpret_cast<uintptr_t>(to) & 15) == 0) *reinterpret_cast<float4*>(to + at) = v;
+    else { to[at] = v.x; to[at + 1] = v.y; to[at + 2] = v.z; to[at + 3] = v.w; }
 }
 __device__ __forceinline__ float4 softmax_grad(float4 a, float4 b, float4 d) {
     return make_float4(a.x * (b.x - d.x), a.y * (b.y - d.y), a.z * (b.z - d.z), a.w * (b.w - d.w));
@@ -741,6 +745,7 @@ edge_softmax_chunk_kernel(const __grid_constant__ SoftmaxArgs A) {
         const int r = slot ? tail_row : head_row;  // the same in every thread
         if (r < 0) continue;
         const int64_t rs = A.rowptr[r], re = A.rowptr[r + 1], t0 = rs * HV + threadIdx.x, t1 = re * HV;  // NT, rs * HV: multiples of HV
+        if (re - rs > A.over) continue;
         float4 m = least, s = zero;
         if (BACKWARD) {
 #pragma unroll 4
@@ -774,6 +779,9 @@ edge_softmax_chunk_kernel(const __grid_constant__ SoftmaxArgs A) {
 constexpr int AR_SLOT = 20;  // of allow_big_smem: 24 of them
 // Chunks of 256 threads are 1024 (8 heads) or 2048 (4 heads) positions; small graphs take a quarter, so that all SMs have work.
 constexpr int64_t AR_SMALL = 400 * 1024;  // edges * heads / 8
+// Edge softmax: rows of up to so many chunks' positions are read by every block that they reach, longer ones by a cluster (1.6 M edges, R-MAT, 8
+// heads fp32, of 2, 4, 8 and 16 chunks: 80, 78, 75 and 74 us; 300 k edges: 46, 31, 25 and 24 us; 160 k: 24, 24, 20 and 27 us).
+constexpr int AR_SPAN = 8;
 
 template <int NT, int HV>
 static gnn_status softmax_launch(const char* who, const AttnArgs& A, int chunks, cudaStream_t st) {
@@ -855,10 +863,14 @@ bool edge_softmax_chunks_fit(int64_t E, int H, gnn_dtype dtype, const void* x, c
     return ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(out)) & (quad - 1)) == 0 && apart(x) && (!y || apart(y));
 }
 
+// Up to 8 Ki edges without the clusters, whose launch beside this one is 2 us of 9 there; a single row of 8000 positions of 8 heads takes 29 us (one block
+// for all of it: 37 us).
+int64_t edge_softmax_chunk_rows(int64_t E, int H) { return E <= 8192 ? E : (int64_t)AR_SPAN * ar_chunk(E, H); }
+
 // y null: out = softmax of x over each row; else out = x * (y - sum over the row of x * y)
 gnn_status edge_softmax_chunks(const char* who, const gnn_csr* g, const void* x, const void* y, int H, gnn_dtype dtype, void* out, float* rowmax, float* rowsum,
                                cudaStream_t st) {
-    const SoftmaxArgs A = {g->rowptr, x, y, out, rowmax, rowsum, g->N, g->E};
+    const SoftmaxArgs A = {g->rowptr, x, y, out, rowmax, rowsum, g->N, g->E, edge_softmax_chunk_rows(g->E, H)};
     if (dtype == GNN_F32) return y ? edge_softmax_dispatch<float, true>(who, A, H, st) : edge_softmax_dispatch<float, false>(who, A, H, st);
     return y ? edge_softmax_dispatch<__nv_bfloat16, true>(who, A, H, st) : edge_softmax_dispatch<__nv_bfloat16, false>(who, A, H, st);
 }

@@ -9,9 +9,10 @@
 // (4, 8, 16 or 32 heads) a cluster of eight blocks that combine their results through distributed
 // shared memory.  Reductions use fixed shuffle / shared memory trees and a fixed block order, so
 // results are bit-reproducible.  All arithmetic is fp32.
+#include <algorithm>
 #include <mutex>
 
-#include "common.cuh"
+#include "reduce_params.cuh"
 #include <cooperative_groups.h>
 
 namespace cg = cooperative_groups;
@@ -389,7 +390,7 @@ __device__ __forceinline__ void hub_share(int64_t nch, int rank, int64_t* first,
 
 template <typename T>
 __device__ __forceinline__ void softmax_row_vec4_cluster(const T* __restrict__ s, T* __restrict__ alpha, int64_t a, int64_t b, int H, int row,
-                                                         float* rowmax, float* rowsum, float* red, HubRows& hub, cg::cluster_group& cluster) {
+                                                         float* rowmax, float* rowsum, float* red, float (&res)[2][32], cg::cluster_group& cluster) {
     const size_t lo = (size_t)a * H;
     int64_t first, last;
     hub_share(((b - a) * H) >> 2, (int)cluster.block_rank(), &first, &last);
@@ -398,12 +399,12 @@ __device__ __forceinline__ void softmax_row_vec4_cluster(const T* __restrict__ s
 #pragma unroll
         for (int j = 0; j < 4; ++j) m[j] = fmaxf(m[j], v[j]);
     }, first);
-    reduce_heads4_cluster<MaxOp>(m, H, red, hub.res[0], cluster);
+    reduce_heads4_cluster<MaxOp>(m, H, red, res[0], cluster);
     for_chunks4(s, lo, last, [&](int64_t, float* v) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) z[j] += expf(v[j] - m[j]);
     }, first);
-    reduce_heads4_cluster<SumOp>(z, H, red, hub.res[1], cluster);
+    reduce_heads4_cluster<SumOp>(z, H, red, res[1], cluster);
     for_chunks4(s, lo, last, [&](int64_t c, float* v) {
 #pragma unroll
         for (int j = 0; j < 4; ++j) v[j] = expf(v[j] - m[j]) / z[j];
@@ -551,7 +552,7 @@ edge_softmax_long_kernel(const int64_t* __restrict__ rowptr, int N, const T* __r
             else if (head_pow2(H)) softmax_row_pow2<T, SM_BLOCK>(s, alpha, a, b, H, row, rowmax, rowsum, red);
             else softmax_row_any<T, SM_BLOCK>(s, alpha, a, b, H, row, rowmax, rowsum, red);
         },
-        [&](int row, int64_t a, int64_t b, int) { softmax_row_vec4_cluster<T>(s, alpha, a, b, H, row, rowmax, rowsum, red, hub, cluster); });
+        [&](int row, int64_t a, int64_t b, int) { softmax_row_vec4_cluster<T>(s, alpha, a, b, H, row, rowmax, rowsum, red, hub.res, cluster); });
 }
 
 template <typename T>
@@ -572,6 +573,57 @@ edge_softmax_backward_long_kernel(const int64_t* __restrict__ rowptr, int N, con
         },
         // one result buffer per parity of the hub's place in the list: it is written again two barriers later
         [&](int, int64_t a, int64_t b, int i) { softmax_bwd_row_vec4_cluster<T>(alpha, dalpha, ds, a, b, H, red, hub.res[i & 1], cluster); });
+}
+
+// The rows of more than `over` positions, which the chunk kernels (attention_rows.cu) leave: a cluster each, as above.  Such a row holds a
+// multiple of `over`; the first one that it holds names it.  The warps of a block look up the rows at eight multiples at a time (every block of
+// a cluster for itself, with the same outcome), neighbouring multiples in different clusters.
+template <class HubBody>
+__device__ __forceinline__ void for_each_row_over(const int64_t* rowptr, int N, int64_t E, int64_t over, cg::cluster_group& cluster, HubBody hub_body) {
+    __shared__ int rows[SM_BLOCK / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t clusters = gridDim.x / SM_CLUSTER, me = blockIdx.x / SM_CLUSTER;
+    int count = 0;
+    for (int64_t k0 = me; k0 * over < E; k0 += clusters * (SM_BLOCK / 32)) {
+        const int64_t pos = (k0 + clusters * w) * over;
+        int found = -1;
+        if (pos < E) {
+            const int r = row_of_position(rowptr, N, E, pos, lane);
+            const int64_t a = rowptr[r], b = rowptr[r + 1];
+            if (a <= pos && pos < b && b - a > over && pos - a < over) found = r;
+        }
+        __syncthreads();  // every thread is done with the rows before
+        if (lane == 0) rows[w] = found;
+        __syncthreads();
+        for (int q = 0; q < SM_BLOCK / 32; ++q) {
+            const int row = rows[q];  // the same in every block of the cluster
+            if (row >= 0) hub_body(row, rowptr[row], rowptr[row + 1], count++);
+        }
+    }
+    cluster.sync();  // nobody reads a result buffer of a block that is gone
+}
+
+template <typename T>
+__global__ void __cluster_dims__(SM_CLUSTER, 1, 1) __launch_bounds__(SM_BLOCK, SM_LONG_MINB)
+edge_softmax_over_kernel(const int64_t* __restrict__ rowptr, int N, int64_t E, int64_t over, const T* __restrict__ s, int H,
+                         T* __restrict__ alpha, float* __restrict__ rowmax, float* __restrict__ rowsum) {
+    __shared__ float red[SM_BLOCK], res[2][32];
+    cg::cluster_group cluster = cg::this_cluster();
+    for_each_row_over(rowptr, N, E, over, cluster, [&](int row, int64_t a, int64_t b, int) {
+        softmax_row_vec4_cluster<T>(s, alpha, a, b, H, row, rowmax, rowsum, red, res, cluster);
+    });
+}
+
+template <typename T>
+__global__ void __cluster_dims__(SM_CLUSTER, 1, 1) __launch_bounds__(SM_BLOCK)
+edge_softmax_backward_over_kernel(const int64_t* __restrict__ rowptr, int N, int64_t E, int64_t over, const T* __restrict__ alpha,
+                                  const T* __restrict__ dalpha, int H, T* __restrict__ ds) {
+    __shared__ float red[SM_BLOCK], res[2][32];
+    cg::cluster_group cluster = cg::this_cluster();
+    // one result buffer per parity of the row's place: it is written again two barriers later
+    for_each_row_over(rowptr, N, E, over, cluster, [&](int, int64_t a, int64_t b, int i) {
+        softmax_bwd_row_vec4_cluster<T>(alpha, dalpha, ds, a, b, H, red, res[i & 1], cluster);
+    });
 }
 
 template <typename T, bool LONG>
@@ -985,6 +1037,23 @@ static void run_row_tiers(cudaStream_t st, Long run_long, Warp run_warp, Sub run
     cudaStreamWaitEvent(st, t->join[1], 0);
 }
 
+// main_work on the caller's stream and side_work beside it, forked from it and joined back
+template <class Side, class Main>
+static void run_beside(cudaStream_t st, Side side_work, Main main_work) {
+    std::lock_guard<std::mutex> lock(g_tier_mutex);
+    TierStreams* t = tier_streams();
+    if (!t || cudaEventRecord(t->fork, st) != cudaSuccess || cudaStreamWaitEvent(t->first, t->fork, 0) != cudaSuccess) {
+        (void)cudaGetLastError();
+        side_work(st);
+        main_work(st);
+        return;
+    }
+    side_work(t->first);
+    main_work(st);
+    cudaEventRecord(t->join[0], t->first);
+    cudaStreamWaitEvent(st, t->join[0], 0);
+}
+
 gnn_status gat_alpha(const gnn_csr* g, const float* al, const float* ar, float slope, int H, float* alpha, cudaStream_t st) {
     if (g->N == 0 || g->E == 0) return GNN_OK;
     const int wg = row_grid_pl(g->N, false), lg = row_grid_pl(g->N, true), sg = row_grid_sub(g->N);
@@ -1021,9 +1090,37 @@ bool gat_rows_backward_pl(const gnn_csr* g, const float* alpha, float* dalpha_dz
 }  // namespace gnn
 
 namespace gnn {
-bool edge_softmax_chunks_fit(int64_t E, int H, gnn_dtype dtype, const void* x, const void* y, const void* out);  // attention_rows.cu
+// attention_rows.cu
+bool edge_softmax_chunks_fit(int64_t E, int H, gnn_dtype dtype, const void* x, const void* y, const void* out);
+int64_t edge_softmax_chunk_rows(int64_t E, int H);  // the longest row that it takes
 gnn_status edge_softmax_chunks(const char* who, const gnn_csr* g, const void* x, const void* y, int H, gnn_dtype dtype, void* out, float* rowmax, float* rowsum,
                                cudaStream_t st);
+
+// Rows by chunks, and beside them the rows that are longer than that takes, if the graph has positions enough for one.
+static gnn_status softmax_by_chunks(const char* who, const gnn_csr* g, const void* x, const void* y, int H, gnn_dtype dtype, void* out, float* rowmax,
+                                    float* rowsum, cudaStream_t st) {
+    const int64_t over = edge_softmax_chunk_rows(g->E, H);
+    if (g->E <= over) {
+        side_prepare();
+        return edge_softmax_chunks(who, g, x, y, H, dtype, out, rowmax, rowsum, st);
+    }
+    gnn_status rc = GNN_OK;
+    const int grid = SM_CLUSTER * (int)std::min<int64_t>(ceil_div(g->E, over * (SM_BLOCK / 32)), 148);
+    run_beside(
+        st,
+        [&](cudaStream_t q) {
+#define GNN_OVER(T)                                                                                                                                      \
+    y ? edge_softmax_backward_over_kernel<T><<<grid, SM_BLOCK, 0, q>>>(g->rowptr, g->N, g->E, over, (const T*)x, (const T*)y, H, (T*)out)                 \
+      : edge_softmax_over_kernel<T><<<grid, SM_BLOCK, 0, q>>>(g->rowptr, g->N, g->E, over, (const T*)x, H, (T*)out, rowmax, rowsum)
+            if (dtype == GNN_F32) GNN_OVER(float);
+            else GNN_OVER(__nv_bfloat16);
+#undef GNN_OVER
+        },
+        [&](cudaStream_t q) { rc = edge_softmax_chunks(who, g, x, y, H, dtype, out, rowmax, rowsum, q); });
+    if (rc != GNN_OK) return rc;
+    GNN_CHECK_LAUNCH(who);
+    return GNN_OK;
+}
 }  // namespace gnn
 
 using namespace gnn;
@@ -1038,10 +1135,8 @@ gnn_status gnn_edge_softmax(const gnn_csr* g, const void* logits_EH, int H, gnn_
     if (g->N == 0) return GNN_OK;
     GNN_REQUIRE(g->E == 0 || (logits_EH && alpha_EH), GNN_ERR_INVALID_ARG, "%s: null argument", who);
     cudaStream_t st = as_stream(stream);
-    if (edge_softmax_chunks_fit(g->E, H, dtype, logits_EH, nullptr, alpha_EH)) {
-        side_prepare();
-        return edge_softmax_chunks(who, g, logits_EH, nullptr, H, dtype, alpha_EH, rowmax, rowsum, st);
-    }
+    if (edge_softmax_chunks_fit(g->E, H, dtype, logits_EH, nullptr, alpha_EH))
+        return softmax_by_chunks(who, g, logits_EH, nullptr, H, dtype, alpha_EH, rowmax, rowsum, st);
     const int wgrid = row_grid(g->N, false), lgrid = row_grid_cluster(g->N);
     // the two row tiers write disjoint rows: side by side (the long rows' blocks beside the warps of the short ones)
     if (dtype == GNN_F32)
@@ -1066,10 +1161,8 @@ gnn_status gnn_edge_softmax_backward(const gnn_csr* g, const void* alpha_EH, con
     if (g->N == 0 || g->E == 0) return GNN_OK;
     GNN_REQUIRE(alpha_EH && dAlpha_EH && dLogits_EH, GNN_ERR_INVALID_ARG, "%s: null argument", who);
     cudaStream_t st = as_stream(stream);
-    if (edge_softmax_chunks_fit(g->E, H, dtype, alpha_EH, dAlpha_EH, dLogits_EH)) {
-        side_prepare();
-        return edge_softmax_chunks(who, g, alpha_EH, dAlpha_EH, H, dtype, dLogits_EH, nullptr, nullptr, st);
-    }
+    if (edge_softmax_chunks_fit(g->E, H, dtype, alpha_EH, dAlpha_EH, dLogits_EH))
+        return softmax_by_chunks(who, g, alpha_EH, dAlpha_EH, H, dtype, dLogits_EH, nullptr, nullptr, st);
     const int wgrid = row_grid(g->N, false), lgrid = row_grid_cluster(g->N);
     if (dtype == GNN_F32)
         run_row_tiers(

@@ -173,6 +173,53 @@ def test_edge_softmax_rows_of_tens_of_thousands_of_positions(gnn, dtype, H):
     assert np.array_equal(bits(gnn.edge_softmax_backward(g, alpha, to_dev(R[eid]))), bits(ds))
 
 
+# One row beside short ones: as long as the chunk kernels take, one position more, and over many blocks' chunks.  Up to 8192 edges they take any row.
+@pytest.mark.parametrize("H,longest,e", [(8, 2048, 20_000), (8, 2049, 20_000), (4, 4096, 30_000), (4, 4097, 30_000), (8, 8000, 8192), (4, 8193, 8193), (8, 8192, 430_000), (8, 8193, 430_000), (4, 120_000, 900_000)])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_edge_softmax_one_long_row(gnn, dtype, H, longest, e):
+    rng = np.random.default_rng(longest + H)
+    n = e // 7
+    dst = np.sort(np.concatenate([np.full(longest, n // 2), rng.integers(0, n, e - longest)])).astype(np.int32)
+    src = rng.integers(0, n, e).astype(np.int32)
+    keep = (dst == n // 2).nonzero()[0][longest:]  # (exactly `longest` positions)
+    dst[keep] = n // 2 + 1
+    g = build_graph(gnn, n, src, dst)  # sorted by target: positions are in the order of the list
+    s, R = feats((e, H), dtype, 940 + H), feats((e, H), dtype, 941 + H)
+    alpha, top, total = gnn.edge_softmax(g, to_dev(s), want_stats=True)
+    ao = oracle.edge_softmax(n, dst, s)
+    assert_close(to_host64(alpha), ao, ao, dtype, "alpha")
+    x = synth.to_f64(s)
+    most, sums = np.full((n, H), -np.inf), np.zeros((n, H))
+    np.maximum.at(most, dst, x)
+    np.add.at(sums, dst, np.exp(x - most[dst]))
+    most[np.isinf(most)] = 0.0
+    assert np.array_equal(to_host64(top), most)
+    assert_close(to_host64(total), sums, sums, "f32", "sums of the rows")
+    dso, S = oracle.edge_softmax_backward(n, dst, to_host64(alpha), R)
+    assert_close(to_host64(gnn.edge_softmax_backward(g, alpha, to_dev(R))), dso, S, dtype, "dlogits")
+
+
+def test_edge_softmax_time_of_a_very_long_row(gnn):
+    """A row of 2.4 M positions (a readout node) is read a fixed number of times: 21 times as long as rows of 8 when measured, 240 times with every
+    block that it reaches reading all of it."""
+    import torch
+    e, H = 2_400_000, 8
+    times = []
+    for dst in (torch.arange(e, device="cuda") // 8, torch.zeros(e, device="cuda")):
+        g = gnn.coo_to_csr(e // 8, torch.randint(e // 8, (e,), device="cuda", dtype=torch.int32), dst.to(torch.int32))
+        s, R = torch.randn(e, H, device="cuda"), torch.randn(e, H, device="cuda")
+        for f in (lambda: gnn.edge_softmax(g, s), lambda: gnn.edge_softmax_backward(g, s, R)):
+            f()
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            for _ in range(5):
+                f()
+            b.record()
+            torch.cuda.synchronize()
+            times.append(a.elapsed_time(b))
+    assert times[2] < 80 * times[0] and times[3] < 80 * times[1], times
+
+
 def test_edge_softmax_degenerate(gnn):
     import torch
     # one edge -> 1; equal logits -> 1/deg; huge logits do not overflow
