@@ -1091,7 +1091,7 @@ bool gat_rows_backward_pl(const gnn_csr* g, const float* alpha, float* dalpha_dz
 
 namespace gnn {
 // attention_rows.cu
-bool edge_softmax_chunks_fit(int64_t E, int H, gnn_dtype dtype, const void* x, const void* y, const void* out);
+bool edge_softmax_chunks_fit(int32_t N, int64_t E, int H, gnn_dtype dtype, const void* x, const void* y, const void* out);
 int64_t edge_softmax_chunk_rows(int64_t E, int H);  // the longest row that it takes
 gnn_status edge_softmax_chunks(const char* who, const gnn_csr* g, const void* x, const void* y, int H, gnn_dtype dtype, void* out, float* rowmax, float* rowsum,
                                cudaStream_t st);
@@ -1135,7 +1135,7 @@ gnn_status gnn_edge_softmax(const gnn_csr* g, const void* logits_EH, int H, gnn_
     if (g->N == 0) return GNN_OK;
     GNN_REQUIRE(g->E == 0 || (logits_EH && alpha_EH), GNN_ERR_INVALID_ARG, "%s: null argument", who);
     cudaStream_t st = as_stream(stream);
-    if (edge_softmax_chunks_fit(g->E, H, dtype, logits_EH, nullptr, alpha_EH))
+    if (edge_softmax_chunks_fit(g->N, g->E, H, dtype, logits_EH, nullptr, alpha_EH))
         return softmax_by_chunks(who, g, logits_EH, nullptr, H, dtype, alpha_EH, rowmax, rowsum, st);
     const int wgrid = row_grid(g->N, false), lgrid = row_grid_cluster(g->N);
     // the two row tiers write disjoint rows: side by side (the long rows' blocks beside the warps of the short ones)
@@ -1161,7 +1161,7 @@ gnn_status gnn_edge_softmax_backward(const gnn_csr* g, const void* alpha_EH, con
     if (g->N == 0 || g->E == 0) return GNN_OK;
     GNN_REQUIRE(alpha_EH && dAlpha_EH && dLogits_EH, GNN_ERR_INVALID_ARG, "%s: null argument", who);
     cudaStream_t st = as_stream(stream);
-    if (edge_softmax_chunks_fit(g->E, H, dtype, alpha_EH, dAlpha_EH, dLogits_EH))
+    if (edge_softmax_chunks_fit(g->N, g->E, H, dtype, alpha_EH, dAlpha_EH, dLogits_EH))
         return softmax_by_chunks(who, g, alpha_EH, dAlpha_EH, H, dtype, dLogits_EH, nullptr, nullptr, st);
     const int wgrid = row_grid(g->N, false), lgrid = row_grid_cluster(g->N);
     if (dtype == GNN_F32)

@@ -220,6 +220,35 @@ def test_edge_softmax_time_of_a_very_long_row(gnn):
     assert times[2] < 80 * times[0] and times[3] < 80 * times[1], times
 
 
+@pytest.mark.parametrize("H,n,dtype", [(8, 50_000, "f32"), (8, 50_000, "bf16"), (4, 14_000, "f32")])
+def test_edge_softmax_of_many_long_rows(gnn, H, n, dtype):
+    """Rows that are long on average take a warp, a block or a cluster each, and no more time than over their own input, which always does."""
+    import torch
+    e = 2_100_000
+    rng = np.random.default_rng(n)
+    dst = np.sort(rng.integers(0, n, e)).astype(np.int32)
+    dst[400_000:409_000], dst[500_000:500_700] = dst[400_000], dst[500_000]
+    g = build_graph(gnn, n, rng.integers(0, n, e).astype(np.int32), dst)
+    s, R = feats((e, H), dtype, 950 + H), feats((e, H), dtype, 951 + H)
+    S, up = to_dev(s), to_dev(R)
+    alpha = gnn.edge_softmax(g, S)
+    ao = oracle.edge_softmax(n, dst, s)
+    assert_close(to_host64(alpha), ao, ao, dtype, "alpha")
+    dso, terms = oracle.edge_softmax_backward(n, dst, to_host64(alpha), R)
+    assert_close(to_host64(gnn.edge_softmax_backward(g, alpha, up)), dso, terms, dtype, "dlogits")
+    own, times = S.clone(), []
+    for f in (lambda: gnn.edge_softmax(g, S), lambda: gnn._check(gnn.load().gnn_edge_softmax(gnn.C.byref(g.c), gnn._p(own), H, gnn._dtype(own), gnn._p(own), None, None, gnn._stream()))):
+        f()
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(20):
+            f()
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b))
+    assert times[0] < 1.2 * times[1], times  # (by chunks: 1.4 to 1.7 times as long)
+
+
 def test_edge_softmax_degenerate(gnn):
     import torch
     # one edge -> 1; equal logits -> 1/deg; huge logits do not overflow
