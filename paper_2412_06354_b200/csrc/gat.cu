@@ -311,6 +311,7 @@ static gnn_status gat_check(const char* who, const gnn_csr* g, int H, int C, gnn
 }
 
 gnn_status gat_alpha(const gnn_csr* g, const float* al, const float* ar, float slope, int H, float* alpha, cudaStream_t st);
+bool attention_by_chunks(int32_t N, int64_t E, int H);  // attention_rows.cu
 gnn_status attention_rows(const char* who, const gnn_csr* g, const float* al, const float* ar, float slope, int H, float* alpha, float* dz, float* dar,
                           void* ws, size_t ws_bytes, cudaStream_t st);
 bool gat_rows_backward_pl(const gnn_csr* g, const float* alpha, float* dalpha_dz, const float* al, const float* ar,
@@ -357,7 +358,7 @@ gnn_status gnn_gat_fused(const gnn_csr* g, const void* Wx, const float* a_src, c
     GNN_CHECK_LAUNCH(who);
     // logits and their per-row softmax, written straight into alpha_csr
     GNN_REQUIRE(g->E == 0 || g->col, GNN_ERR_INVALID_ARG, "%s: null col", who);
-    if ((H == 4 || H == 8) && g->E > 0) {
+    if (attention_by_chunks(g->N, g->E, H)) {
         side_prepare();
         rc = attention_rows(who, g, al, ar, slope, H, alpha_csr, nullptr, nullptr, w.chunk_ws, w.chunk_bytes, st);
     } else {
@@ -393,7 +394,7 @@ gnn_status gnn_gat_fused_backward(const gnn_csr* g, const void* Wx, const float*
     rc = run_sddmm(who, g, Wx, dOut, H, C, 0, dtype, w.dz, st);
     if (rc != GNN_OK) return rc;
     // softmax and LeakyReLU derivatives, dz over dalpha, dar per row
-    if (H == 4 || H == 8) {
+    if (attention_by_chunks(g->N, g->E, H)) {
         rc = attention_rows(who, g, al, ar, slope, H, const_cast<float*>(alpha_csr), w.dz, w.dar, w.chunk_ws, w.chunk_bytes, st);
         if (rc != GNN_OK) return rc;
     } else if (!gat_rows_backward_pl(g, alpha_csr, w.dz, al, ar, slope, H, w.dar, st)) {

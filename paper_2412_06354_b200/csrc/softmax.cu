@@ -2,8 +2,8 @@
 // the GAT layer named in Sec. 3 "Graph Convolutional Layers"), forward and backward.
 // Logits and coefficients are [E,H] in CSR order, so a node's incoming edges are contiguous.
 //
-// Four and eight heads run positions first (attention_rows.cu), unless the result lies over an input or an array is off its
-// four-value alignment.  Here, the other head counts and those cases:
+// Four and eight heads run positions first (attention_rows.cu) on most graphs; the rules stand there.  Here, the other head counts, and of those two
+// what chunks of positions do not suit: mostly empty rows, rows long on average, a softmax over its own input or off its four-value alignment.
 // One warp per row for ordinary rows; rows longer than SM_LONG_ROW positions are left to a
 // second kernel that gives each of them a whole block, and rows longer than SM_HUB_ROW positions
 // (4, 8, 16 or 32 heads) a cluster of eight blocks that combine their results through distributed
@@ -1062,7 +1062,7 @@ gnn_status gat_alpha(const gnn_csr* g, const float* al, const float* ar, float s
         st, [&](cudaStream_t q) { gat_alpha_pl_kernel<HV, true><<<lg, PL_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, al, ar, slope, alpha); }, \
         [&](cudaStream_t q) { gat_alpha_pl_kernel<HV, false><<<wg, SM_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, al, ar, slope, alpha); },    \
         [&](cudaStream_t q) { gat_alpha_pl_kernel<HV, false, 8><<<sg, SM_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, al, ar, slope, alpha); });
-    if (H == 16) { GNN_GA(4) } else if (H == 32) { GNN_GA(8) } else {  // (4 and 8: attention_rows.cu)
+    if (H == 4) { GNN_GA(1) } else if (H == 8) { GNN_GA(2) } else if (H == 16) { GNN_GA(4) } else if (H == 32) { GNN_GA(8) } else {
         run_row_tiers(  // the two tiers write disjoint rows: side by side
             st, [&](cudaStream_t q) { gat_alpha_kernel<true><<<row_grid(g->N, true), SM_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, H, al, ar, slope, alpha); },
             [&](cudaStream_t q) { gat_alpha_kernel<false><<<row_grid(g->N, false), SM_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, H, al, ar, slope, alpha); },
@@ -1082,7 +1082,7 @@ bool gat_rows_backward_pl(const gnn_csr* g, const float* alpha, float* dalpha_dz
         st, [&](cudaStream_t q) { gat_rows_bwd_pl_kernel<HV, true><<<lg, PL_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, alpha, dalpha_dz, al, ar, slope, dar); }, \
         [&](cudaStream_t q) { gat_rows_bwd_pl_kernel<HV, false><<<wg, SM_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, alpha, dalpha_dz, al, ar, slope, dar); },    \
         [&](cudaStream_t q) { gat_rows_bwd_pl_kernel<HV, false, 8><<<sg, SM_BLOCK, 0, q>>>(g->rowptr, g->col, g->N, alpha, dalpha_dz, al, ar, slope, dar); });
-    if (H == 16) { GNN_GB(4) } else if (H == 32) { GNN_GB(8) } else return false;
+    if (H == 4) { GNN_GB(1) } else if (H == 8) { GNN_GB(2) } else if (H == 16) { GNN_GB(4) } else if (H == 32) { GNN_GB(8) } else return false;
 #undef GNN_GB
     return true;
 }

@@ -173,6 +173,48 @@ def test_gat_scores_of_minus_infinity(gnn, H, chunk, edges):
     assert np.array_equal(alpha[others], to_host64(fwd["alpha"])[others])
 
 
+# Few edges on many nodes: rows one by one below 150 k / heads edges on more nodes than edges, chunks from there on
+@pytest.mark.parametrize("H,n,edges", [(4, 9_000, 8_999), (4, 9_000, 9_000), (8, 60_000, 1_000), (8, 18_760, 18_750), (8, 18_760, 18_749), (4, 40_000, 37_500), (4, 40_000, 37_499)])
+def test_gat_mostly_empty_rows(gnn, H, n, edges):
+    rng = np.random.default_rng(n + edges)
+    src, dst = rng.integers(0, n, edges).astype(np.int32), rng.integers(0, n, edges).astype(np.int32)
+    C = 8
+    Wx = synth.normal((n, H * C), "f32", 930 + H, 1)
+    a_s, a_d = synth.uniform_f32((H, C), -0.8, 0.8, 931, 1), synth.uniform_f32((H, C), -0.8, 0.8, 932, 1)
+    g, _ = run_case(gnn, n, src, dst, Wx, a_s, a_d, H, C, "f32", f"gat H={H}, {edges} edges on {n} nodes")
+    eid = g.eid[:g.E].cpu().numpy()
+    logits = synth.normal((edges, H), "f32", 933, 1)
+    alpha, top, total = gnn.edge_softmax(g, to_dev(logits[eid]), want_stats=True)
+    ao = oracle.edge_softmax(n, dst, logits)
+    assert_close(to_host64(alpha), ao[eid], ao[eid], "f32", "alpha")
+    most, sums = np.full((n, H), -np.inf), np.zeros((n, H))
+    np.maximum.at(most, dst, synth.to_f64(logits))
+    np.add.at(sums, dst, np.exp(synth.to_f64(logits) - most[dst]))
+    most[np.isinf(most)] = 0.0
+    assert np.array_equal(to_host64(top), most)
+    assert_close(to_host64(total), sums, sums, "f32", "sums of the rows")
+
+
+def test_softmax_time_of_a_thousand_edges_on_two_million_nodes(gnn):
+    """No longer than three times what 16 heads, twice the values, take (by chunks: 15 times as long as these)."""
+    import torch
+    n, e, C = 2_000_000, 1_000, 4
+    src, dst = (torch.randint(n, (e,), device="cuda", dtype=torch.int32) for _ in range(2))
+    g = gnn.coo_to_csr(n, src, dst)
+    times = []
+    for H in (4, 8, 16):
+        s = torch.randn(e, H, device="cuda")
+        gnn.edge_softmax(g, s, want_stats=True)
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(5):
+            gnn.edge_softmax(g, s, want_stats=True)
+        b.record()
+        torch.cuda.synchronize()
+        times.append(a.elapsed_time(b))
+    assert max(times[:2]) < 3 * times[2], times
+
+
 def test_gat_zero_attention_is_mean_aggregation(gnn):
     n, src, dst = ragged_graph(95)
     H, C = 4, 16
