@@ -861,6 +861,16 @@ static gnn_status edge_softmax_dispatch(const char* who, const SoftmaxArgs& A, i
 static bool mostly_empty(int32_t N, int64_t E, int H) { return N > E && E * H < 150 * 1000; }
 bool attention_by_chunks(int32_t N, int64_t E, int H) { return (H == 4 || H == 8) && E > 0 && !mostly_empty(N, E, H); }
 
+// The GAT gradient by chunks is a chain of three kernels; on small graphs the three that take rows by length, side by side, are done sooner, and where
+// rows are long and many they read faster.  The call by rows / by chunks, us.  R-MAT, graphs replayed, 4 heads: 8 k edges 36 / 45, 40 k 40 / 52 (calls in
+// a row 53 / 56), 160 k 52 / 60 with rows up to 4820, 53 / 63, 320 k 74 / 76; 8 heads: 8 k 44 / 54, 160 k 67 / 69.  The line lies as low as it does for graphs
+// with one row of all edges: 4 heads, 32 k 62 / 54, 64 k 103 / 64; 8 heads, 16 k 74 / 58, 32 k 118 / 65.  Long rows, 8 heads: 24 M edges of mean
+// length 64 3290 / 3690, 48 M, 32 7440 / 8110, 24 M of even length 64 3300 / 3780.
+bool attention_gradient_by_chunks(int32_t N, int64_t E, int H) {
+    const double mean = (double)E / (N > 0 ? N : 1);
+    return attention_by_chunks(N, E, H) && E * H / 8 >= 24 * 1024 && E * mean * mean < (H == 8 ? 1.5e10 : 9e10);
+}
+
 // Long rows on average: the edge softmax by chunks keeps 32 to 47 us per million edges of 8 heads whatever the rows' lengths, a warp or block
 // per row falls to 18 there.  Rows by length / by chunks, us, R-MAT if not said otherwise.  8 heads, forward: 12 M edges of mean length 16 548 / 533,
 // 32 488 / 546; 24 M, 8 1282 / 1040, 16 1017 / 1070; 3 M of even length 32 75 / 102; gradient: 12 M, 32 382 / 356, 24 M, 16 769 / 701, 32 635 / 703.

@@ -312,6 +312,7 @@ static gnn_status gat_check(const char* who, const gnn_csr* g, int H, int C, gnn
 
 gnn_status gat_alpha(const gnn_csr* g, const float* al, const float* ar, float slope, int H, float* alpha, cudaStream_t st);
 bool attention_by_chunks(int32_t N, int64_t E, int H);  // attention_rows.cu
+bool attention_gradient_by_chunks(int32_t N, int64_t E, int H);
 gnn_status attention_rows(const char* who, const gnn_csr* g, const float* al, const float* ar, float slope, int H, float* alpha, float* dz, float* dar,
                           void* ws, size_t ws_bytes, cudaStream_t st);
 bool gat_rows_backward_pl(const gnn_csr* g, const float* alpha, float* dalpha_dz, const float* al, const float* ar,
@@ -394,7 +395,7 @@ gnn_status gnn_gat_fused_backward(const gnn_csr* g, const void* Wx, const float*
     rc = run_sddmm(who, g, Wx, dOut, H, C, 0, dtype, w.dz, st);
     if (rc != GNN_OK) return rc;
     // softmax and LeakyReLU derivatives, dz over dalpha, dar per row
-    if (attention_by_chunks(g->N, g->E, H)) {
+    if (attention_gradient_by_chunks(g->N, g->E, H)) {
         rc = attention_rows(who, g, al, ar, slope, H, const_cast<float*>(alpha_csr), w.dz, w.dar, w.chunk_ws, w.chunk_bytes, st);
         if (rc != GNN_OK) return rc;
     } else if (!gat_rows_backward_pl(g, alpha_csr, w.dz, al, ar, slope, H, w.dar, st)) {

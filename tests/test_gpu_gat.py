@@ -95,8 +95,8 @@ def test_gat_one_and_two_heads_with_source_hubs(gnn, H, C):
 
 
 # The row kernels of four and eight heads take chunks of positions: 512 and 256 on small graphs, 2048 and 1024 from 800 and 400 Ki edges on.
-# Rows that fill a chunk, end one before or one past its end, lie over several chunks, empty rows at the seams, a last chunk of a few.
-@pytest.mark.parametrize("H,chunk,edges", [(4, 512, 9_001), (8, 256, 4_611), (8, 256, 256), (8, 1024, 420_003), (4, 2048, 830_011)])
+# The gradient takes rows by length below 48 Ki and 24 Ki edges.  Rows that fill a chunk, end one before or one past its end, lie over several chunks, empty rows at the seams, a last chunk of a few.
+@pytest.mark.parametrize("H,chunk,edges", [(4, 512, 9_001), (8, 256, 4_611), (8, 256, 256), (4, 512, 49_151), (4, 512, 49_152), (8, 256, 24_576), (8, 1024, 420_003), (4, 2048, 830_011)])
 def test_gat_and_softmax_rows_at_chunk_ends(gnn, H, chunk, edges):
     rng = np.random.default_rng(edges)
     degree = [chunk, 0, chunk - 1, 1, chunk + 1, chunk - 2, 1, 3 * chunk, 0, 0, 5, 2 * chunk - 5] if edges > chunk else []
@@ -140,7 +140,7 @@ def test_gat_and_softmax_rows_at_chunk_ends(gnn, H, chunk, edges):
 
 # Logits of -inf (scores that overflow) take no part in their rows, wherever the chunks cut them: a single position past a chunk's end, a
 # chunk's whole share in the middle or at the beginning of a row, scattered ones.
-@pytest.mark.parametrize("H,chunk,edges", [(4, 512, 9_001), (8, 256, 6_611), (8, 1024, 420_003), (4, 2048, 830_011)])
+@pytest.mark.parametrize("H,chunk,edges", [(4, 512, 9_001), (8, 256, 6_611), (4, 512, 50_003), (8, 256, 25_001), (8, 1024, 420_003), (4, 2048, 830_011)])
 def test_gat_scores_of_minus_infinity(gnn, H, chunk, edges):
     rng = np.random.default_rng(edges)
     degree = [chunk + 1, 3 * chunk, 2 * chunk]
@@ -193,6 +193,20 @@ def test_gat_mostly_empty_rows(gnn, H, n, edges):
     most[np.isinf(most)] = 0.0
     assert np.array_equal(to_host64(top), most)
     assert_close(to_host64(total), sums, sums, "f32", "sums of the rows")
+
+
+def test_gat_gradient_of_many_long_rows(gnn):
+    """3.1 M edges, rows of 70 on average: by length"""
+    n, e, H, C = 43_000, 3_100_000, 8, 8
+    rng = np.random.default_rng(n)
+    src, dst = rng.integers(0, n, e).astype(np.int32), rng.integers(0, n, e).astype(np.int32)
+    Wx = synth.normal((n, H * C), "f32", 934, 1)
+    a_s, a_d = synth.uniform_f32((H, C), -0.8, 0.8, 935, 1), synth.uniform_f32((H, C), -0.8, 0.8, 936, 1)
+    oracle.set_threads(8)
+    try:
+        run_case(gnn, n, src, dst, Wx, a_s, a_d, H, C, "f32", "gat, long rows")
+    finally:
+        oracle.set_threads(1)
 
 
 def test_softmax_time_of_a_thousand_edges_on_two_million_nodes(gnn):
