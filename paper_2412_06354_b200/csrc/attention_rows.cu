@@ -414,6 +414,66 @@ __device__ __forceinline__ void for_shares(const AttnParts& P, int c0, int c1, B
     }
 }
 
+// A row in more than AR_MANY chunks has its shares combined once, before the kernels that finish its positions, which else do it in every block
+// (a row of k chunks: k * k shares of 64 bytes and more).  The result lies where the shares of the second chunk's other end would: the row
+// goes through all of that chunk.  A block per 32 chunks, for the rows that begin in them.  8 heads fp32, one row of 20 M positions: GAT 19.6 -> 2.6 ms, its
+// gradient 13.2 -> 8.3 ms, of 2.4 M 1160 -> 890 us and 2325 -> 2260 us; 3 us of 222 on 3 M edges without such a row.
+constexpr int AR_MANY = 2048;
+__device__ __forceinline__ size_t combined_at(int c0, int H) { return ((size_t)(c0 + 1) * 2 + 1) * H; }
+
+template <int CHUNK, int HV, bool GRADIENT>
+__global__ void __launch_bounds__(256)
+attention_combine_kernel(const __grid_constant__ AttnArgs A, int chunks) {
+    constexpr int H = 4 * HV, W = 8;
+    __shared__ float4 part[W][HV];
+    pdl_wait();
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, v = lane % HV;
+    auto over_block = [&](float4 x, auto op) {
+#pragma unroll
+        for (int o = 16; o >= HV; o >>= 1) x = op(x, shfl_xor4(x, o));
+        __syncthreads();
+        if (lane < HV) part[w][lane] = x;
+        __syncthreads();
+        x = part[0][v];
+#pragma unroll
+        for (int k = 1; k < W; ++k) x = op(x, part[k][v]);
+        return x;
+    };
+    const auto most = [](float4 x, float4 y) { return comb4<true>(x, y); };
+    const auto sum = [](float4 x, float4 y) { return comb4<false>(x, y); };
+    int last = 0;  // lane k < 32: the last chunk of the row that begins in the block's k-th chunk, if it reaches far enough
+    {
+        const int c = (int)blockIdx.x * 32 + lane, r = c < chunks ? A.parts.tail_row[c] : -1;
+        if (r >= 0) {
+            const int c1 = (int)((A.rowptr[r + 1] - 1) / CHUNK);
+            last = c1 - c >= AR_MANY ? c1 : 0;
+        }
+    }
+    for (unsigned mask = __ballot_sync(0xffffffffu, last > 0); mask; mask &= mask - 1) {  // the same in every warp
+        const int k0 = __ffs(mask) - 1, c0 = (int)blockIdx.x * 32 + k0, c1 = __shfl_sync(0xffffffffu, last, k0);
+        auto share = [&](const float* p, int k) { return ld_float4(p + ((size_t)k * 2 + (k == c0 ? 1 : 0)) * H + 4 * v); };
+        const int first = c0 + (int)threadIdx.x / HV, step = 256 / HV;
+        float4 m = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY), s = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (GRADIENT) {
+#pragma unroll 8
+            for (int k = first; k <= c1; k += step) s = sum(s, share(A.parts.a, k));
+            s = over_block(s, sum);
+            if (threadIdx.x < HV) *reinterpret_cast<float4*>(A.parts.a + combined_at(c0, H) + 4 * v) = s;
+        } else {
+#pragma unroll 8
+            for (int k = first; k <= c1; k += step) m = most(m, share(A.parts.a, k));
+            m = over_block(m, most);
+#pragma unroll 4
+            for (int k = first; k <= c1; k += step) s = sum(s, mul4(share(A.parts.b, k), exp_of(share(A.parts.a, k), m)));
+            s = over_block(s, sum);
+            if (threadIdx.x < HV) {
+                *reinterpret_cast<float4*>(A.parts.a + combined_at(c0, H) + 4 * v) = m;
+                *reinterpret_cast<float4*>(A.parts.b + combined_at(c0, H) + 4 * v) = s;
+            }
+        }
+    }
+}
+
 // Second kernel of the softmax: a block per (chunk, end of it), for the row that it cuts.
 template <int NT, int HV>
 __global__ void __launch_bounds__(NT)
@@ -426,12 +486,17 @@ attention_softmax_cut_kernel(const __grid_constant__ AttnArgs A) {
     const int64_t rs = A.rowptr[r], re = A.rowptr[r + 1];
     const int c0 = (int)(rs / CHUNK), c1 = (int)((re - 1) / CHUNK);
     float4 m = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY), s = make_float4(0.f, 0.f, 0.f, 0.f);
-    for_shares<HV>(A.parts, c0, c1, [&](const float* a, const float*) { m = comb4<true>(m, ld_float4(a)); });
+    if (c1 - c0 >= AR_MANY) {
+        m = ld_float4(A.parts.a + combined_at(c0, H) + 4 * v);
+        s = ld_float4(A.parts.b + combined_at(c0, H) + 4 * v);
+    } else {
+        for_shares<HV>(A.parts, c0, c1, [&](const float* a, const float*) { m = comb4<true>(m, ld_float4(a)); });
 #pragma unroll
-    for (int o = 16; o >= HV; o >>= 1) m = comb4<true>(m, shfl_xor4(m, o));
-    for_shares<HV>(A.parts, c0, c1, [&](const float* a, const float* b) { s = comb4<false>(s, mul4(ld_float4(b), exp_of(ld_float4(a), m))); });
+        for (int o = 16; o >= HV; o >>= 1) m = comb4<true>(m, shfl_xor4(m, o));
+        for_shares<HV>(A.parts, c0, c1, [&](const float* a, const float* b) { s = comb4<false>(s, mul4(ld_float4(b), exp_of(ld_float4(a), m))); });
 #pragma unroll
-    for (int o = 16; o >= HV; o >>= 1) s = comb4<false>(s, shfl_xor4(s, o));
+        for (int o = 16; o >= HV; o >>= 1) s = comb4<false>(s, shfl_xor4(s, o));
+    }
     const float4 f = over(exp_of(ld_float4(A.parts.a + ((size_t)c * 2 + slot) * H + 4 * v), m), s);
     const int64_t p0 = max(rs, (int64_t)c * CHUNK), p1 = min(re, (int64_t)(c + 1) * CHUNK);
     float4* const al = reinterpret_cast<float4*>(A.alpha);
@@ -549,9 +614,13 @@ attention_gradient_cut_kernel(const __grid_constant__ AttnArgs A) {
     const int64_t rs = A.rowptr[r], re = A.rowptr[r + 1];
     const int c0 = (int)(rs / CHUNK), c1 = (int)((re - 1) / CHUNK);
     float4 d = make_float4(0.f, 0.f, 0.f, 0.f), s = d;
-    for_shares<HV>(A.parts, c0, c1, [&](const float* a, const float*) { d = comb4<false>(d, ld_float4(a)); });
+    if (c1 - c0 >= AR_MANY) {
+        d = ld_float4(A.parts.a + combined_at(c0, H) + 4 * v);
+    } else {
+        for_shares<HV>(A.parts, c0, c1, [&](const float* a, const float*) { d = comb4<false>(d, ld_float4(a)); });
 #pragma unroll
-    for (int o = 16; o >= HV; o >>= 1) d = comb4<false>(d, shfl_xor4(d, o));
+        for (int o = 16; o >= HV; o >>= 1) d = comb4<false>(d, shfl_xor4(d, o));
+    }
     const float4 arv = ld_float4(A.ar + (size_t)r * H + 4 * v);
     const int64_t p0 = max(rs, (int64_t)c * CHUNK), p1 = min(re, (int64_t)(c + 1) * CHUNK);
 #pragma unroll 4
@@ -790,6 +859,8 @@ static gnn_status softmax_launch(const char* who, const AttnArgs& A, int chunks,
     const gnn_status rc = allow_big_smem(who, (const void*)attention_softmax_kernel<NT, HV>, AR_SLOT + (NT == 256) * 2 + HV - 1, smem);
     if (rc != GNN_OK) return rc;
     launch_overlapped(attention_softmax_kernel<NT, HV>, dim3(chunks), dim3(NT), smem, st, A);
+    if constexpr (NT == 256)  // (small graphs have at most 1600 chunks)
+        if (chunks > AR_MANY) launch_overlapped(attention_combine_kernel<Tile::CHUNK, HV, false>, dim3((unsigned)ceil_div(chunks, 32)), dim3(256), 0, st, A, chunks);
     launch_overlapped(attention_softmax_cut_kernel<NT, HV>, dim3(chunks, 2), dim3(NT), 0, st, A);
     return GNN_OK;
 }
@@ -802,6 +873,8 @@ static gnn_status gradient_launch(const char* who, const AttnArgs& A, int chunks
     if (rc != GNN_OK) return rc;
     launch_overlapped(attention_gradient_kernel<NT, HV>, dim3(chunks > 0 ? chunks : 1), dim3(NT), smem, st, A);
     if (chunks == 0) return GNN_OK;
+    if constexpr (NT == 256)  // (small graphs have at most 1600 chunks)
+        if (chunks > AR_MANY) launch_overlapped(attention_combine_kernel<Tile::CHUNK, HV, true>, dim3((unsigned)ceil_div(chunks, 32)), dim3(256), 0, st, A, chunks);
     launch_overlapped(attention_gradient_cut_kernel<NT, HV>, dim3(chunks, 2), dim3(NT), 0, st, A);
     launch_overlapped(attention_gradient_sums_kernel<NT, HV>, dim3((unsigned)ceil_div(chunks, 8)), dim3(256), 0, st, A, chunks);
     return GNN_OK;

@@ -195,6 +195,23 @@ def test_gat_mostly_empty_rows(gnn, H, n, edges):
     assert_close(to_host64(total), sums, sums, "f32", "sums of the rows")
 
 
+# A row over so many chunks that its shares are combined by a kernel of their own: in one chunk less (2048 of them), exactly and more
+@pytest.mark.parametrize("H,positions", [(8, 2047 * 1024 + 5), (8, 2048 * 1024 + 5), (8, 2_300_000), (4, 2048 * 2048 + 5)])
+def test_gat_row_of_millions(gnn, H, positions):
+    n, C, before = 250_000, 8 if H == 4 else 4, 1_000
+    rng = np.random.default_rng(positions)
+    others = rng.integers(0, n, 400_000)
+    dst = np.sort(np.concatenate([np.full(before, 0), np.full(positions, 1), others[others > 1]])).astype(np.int32)  # the row begins inside the first chunk
+    src = rng.integers(0, n, len(dst)).astype(np.int32)
+    Wx = synth.normal((n, H * C), "f32", 937, 1)
+    a_s, a_d = synth.uniform_f32((H, C), -0.8, 0.8, 938, 1), synth.uniform_f32((H, C), -0.8, 0.8, 939, 1)
+    oracle.set_threads(8)
+    try:
+        run_case(gnn, n, src, dst, Wx, a_s, a_d, H, C, "f32", f"gat H={H}, a row of {positions}")
+    finally:
+        oracle.set_threads(1)
+
+
 def test_gat_gradient_of_many_long_rows(gnn):
     """3.1 M edges, rows of 70 on average: by length"""
     n, e, H, C = 43_000, 3_100_000, 8, 8
