@@ -929,8 +929,10 @@ static bool make_map_f32_blocks(CUtensorMap* m, const void* ptr, int64_t rows, i
 // Two groups on slots of 32 rows, on slots of 16 four where four buffers and slots fit.  170k x 128 x 128: 50 us with 8 warps
 // on one slot after the other, 47 us with 16, 58 us in four groups on slots of 16 rows, 42 us so; reading X and dY takes 27 us.
 // Then the bound was shared memory's bandwidth (copies, conversion and both operands of every MMA: 80 % of a slot's time), so X's
-// levels go to tensor memory (A_TMEM), transposed on the way: a feature per lane.  Where the accumulators leave no columns for two
-// operand buffers (K of 256 by M over 208, for one) A stays in shared memory.
+// levels go to tensor memory (A_TMEM), transposed on the way: a feature per lane, which leaves room for four groups on slots of 32 rows.  On slots
+// of 16 rows, which had four groups before, that gives little and often loses, by the features that do not fill their four warps and by narrow results:
+// A in shared / in tensor memory, 120k rows, K x M of 96 x 64 1.02, 128 x 128 1.04, 160 x 160 1.04, 256 x 128 1.03, 128 x 256 1.04, but 64 x 256 0.95,
+// 160 x 192 0.91, 256 x 64 0.97, exact ones 187 x 59 0.96, 91 x 219 0.98; 170k x 200 x 47 92 and 98 us, x 100 x 200 100 and 105 us.
 // Exact form (K or M no multiple of 32): the accumulator truncates at every MMA, 1.8e-8 of the result each and one way, so that
 // a CTA's hundreds of rows in one sum cost 7.8e-6 norm-wise at 170k rows and 2.3e-5 at 500k, where the FFMA kernel that these
 // sizes took before has 1.1e-6.  There the five small products go to an accumulator of corrections, and after every FD_FLUSH
@@ -1234,8 +1236,8 @@ gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, in
     const int acc_cols = M * (ka / 128);
     P.mains = exact && 3 * acc_cols <= 512 ? 2 : 1;
     const int acc_all = (exact ? P.mains + 1 : 1) * acc_cols;
-    // X's levels in tensor memory where two buffers of them fit beside the accumulators
-    const bool a_tmem = acc_all + 2 * (ka / 128) * 3 * (R / 2) <= 512;
+    // X's levels in tensor memory (see above), where two buffers of them fit beside the accumulators (R = 32: always, 480 columns at most)
+    const bool a_tmem = acc_all + 2 * (ka / 128) * 3 * (R / 2) <= 512 && (R == 32 || (!exact && (K > 128 ? M >= 128 && M <= 160 : K >= 96 && M == 256)));
     const size_t slot = (size_t)(K / 32 + M / 32) * R * 128, op = 3 * ((a_tmem ? 0 : (size_t)ka * R * 2) + (size_t)M * R * 2);
     auto columns = [&](int groups) { return acc_all + (a_tmem ? groups * (ka / 128) * 3 * (R / 2) : 0); };
     P.groups = (R == 16 || a_tmem) && 1024 + FD_MAX_GROUPS * (op + slot) <= TM_SMEM_MAX && columns(FD_MAX_GROUPS) <= 512 ? FD_MAX_GROUPS : 2;
@@ -1254,12 +1256,9 @@ gnn_status linear_tma_f32_dw(const void* X, int ldx, const void* dY, int ldd, in
         return GNN_OK;
     };
     constexpr int more = FD_THREADS + 32 * FD_FLUSH_WARPS;
-    if (a_tmem) {
-        if (exact) return R == 32 ? launch(linear_tma_f32_dw_kernel<32, true, true>, 44, more) : launch(linear_tma_f32_dw_kernel<16, true, true>, 45, more);
-        return R == 32 ? launch(linear_tma_f32_dw_kernel<32, false, true>, 46, FD_THREADS) : launch(linear_tma_f32_dw_kernel<16, false, true>, 47, FD_THREADS);
-    }
-    if (exact) return R == 32 ? launch(linear_tma_f32_dw_kernel<32, true, false>, 18, more) : launch(linear_tma_f32_dw_kernel<16, true, false>, 19, more);
-    return R == 32 ? launch(linear_tma_f32_dw_kernel<32, false, false>, 12, FD_THREADS) : launch(linear_tma_f32_dw_kernel<16, false, false>, 15, FD_THREADS);
+    if (R == 32) return exact ? launch(linear_tma_f32_dw_kernel<32, true, true>, 44, more) : launch(linear_tma_f32_dw_kernel<32, false, true>, 46, FD_THREADS);
+    if (a_tmem) return launch(linear_tma_f32_dw_kernel<16, false, true>, 47, FD_THREADS);
+    return exact ? launch(linear_tma_f32_dw_kernel<16, true, false>, 19, more) : launch(linear_tma_f32_dw_kernel<16, false, false>, 15, FD_THREADS);
 }
 
 static size_t tf_fixed_bytes(int Kc, int Mo) {

@@ -195,6 +195,19 @@ def test_linear_ragged_fp32_is_as_exact_as_plain_fp32(gnn, n, K, M):
         oracle.set_threads(1)
 
 
+# dW of fp32 has X's levels in tensor memory up to 128 x 128, for some wider products too, in shared memory for the others: both sides of each line
+@pytest.mark.parametrize("K,M", [(128, 128), (129, 128), (128, 129), (160, 128), (160, 96), (160, 160), (160, 192), (256, 160), (256, 128), (256, 127), (96, 256), (64, 256), (128, 224)])
+def test_linear_dw_operand_places(gnn, K, M):
+    import torch
+    n = 9_700
+    X, W, D = (torch.randn(s, device="cuda") for s in ((n, K), (K, M), (n, M)))
+    dW = gnn.linear_backward(X, W, D, want_dX=False)[1]
+    want, terms = X.double().T @ D.double(), X.double().abs().T @ D.double().abs()
+    assert bool(((dW.double() - want).abs() <= 1e-5 * terms).all())
+    assert float((dW.double() - want).norm() / want.norm()) < 4e-6  # as plain fp32 sums of 9700 terms
+    assert torch.equal(dW, gnn.linear_backward(X, W, D, want_dX=False)[1])
+
+
 def test_linear_large_rows_tensor_core(gnn):
     """N = 100000 rows, 256 -> 256 bf16 (the attention workload's transform): many tiles per CTA."""
     import torch
