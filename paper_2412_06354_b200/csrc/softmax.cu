@@ -10,6 +10,7 @@
 // shared memory.  Reductions use fixed shuffle / shared memory trees and a fixed block order, so
 // results are bit-reproducible.  All arithmetic is fp32.
 #include <algorithm>
+#include <atomic>
 #include <mutex>
 
 #include "reduce_params.cuh"
@@ -994,8 +995,12 @@ static TierStreams* tier_streams() {
 
 // The helper streams exist from the first call on a device on, whether it needs them or not: the call after it may be captured.
 void side_prepare() {
+    static std::atomic<bool> tried[64];
+    int dev = -1;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || tried[dev].load(std::memory_order_acquire)) return;
     std::lock_guard<std::mutex> lock(g_tier_mutex);
     tier_streams();
+    tried[dev].store(true, std::memory_order_release);
 }
 
 // A side branch of the caller's stream: work enqueued on the returned stream starts after everything enqueued on

@@ -305,3 +305,36 @@ def test_gat_more_than_8mi_edges_uses_the_row_walking_kernels(gnn, E):
             assert int(np.diff(g.rowptr.cpu().numpy()).max()) > 65 * 1024 and int(np.diff(g.rowptrT.cpu().numpy()).max()) > 65 * 1024
     finally:
         oracle.set_threads(1)
+
+
+def test_attention_calls_under_capture_after_a_first_call_that_forks_nothing():
+    """The first call of a process, a forward pass by chunks, needs no helper streams; the calls captured after it fork onto them."""
+    import subprocess
+    import sys
+    code = """
+import torch
+from paper_2412_06354_b200 import gnn
+n, e, H, C = 5000, 60000, 8, 8
+dst = torch.randint(n, (e,), device="cuda", dtype=torch.int32)
+dst[:9000] = 7
+g = gnn.coo_to_csr(n, torch.randint(n, (e,), device="cuda", dtype=torch.int32), dst)
+Wx, a1, a2, R = torch.randn(n, H * C, device="cuda"), torch.randn(H, C, device="cuda"), torch.randn(H, C, device="cuda"), torch.randn(n, H * C, device="cuda")
+s, up = torch.randn(e, H, device="cuda"), torch.randn(e, H, device="cuda")
+fwd = gnn.gat_fused(g, Wx, a1, a2, H)
+def calls():
+    alpha = gnn.edge_softmax(g, s)
+    b = gnn.gat_fused_backward(g, Wx, a1, a2, fwd, R, H)
+    f = gnn.gat_fused(g, Wx, a1, a2, H)
+    return [alpha, gnn.edge_softmax_backward(g, alpha, up), b["dWx"], b["da_src"], b["da_dst"], f["out"], f["alpha"]]
+torch.cuda.synchronize()
+graph = torch.cuda.CUDAGraph()
+with torch.cuda.graph(graph):
+    got = calls()
+graph.replay()
+want = calls()
+torch.cuda.synchronize()
+assert all(torch.equal(x, y) for x, y in zip(got, want))
+print("same")
+"""
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "same" in r.stdout, r.stderr[-2000:]
