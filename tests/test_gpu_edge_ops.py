@@ -132,8 +132,9 @@ def test_edge_softmax_forward_backward(gnn, dtype, H):
 @pytest.mark.parametrize("dtype", ["f32", "bf16"])
 @pytest.mark.parametrize("H", [1, 4, 8, 32])
 def test_edge_softmax_rows_of_tens_of_thousands_of_positions(gnn, dtype, H):
-    """Three rows above 8192 positions (shared by a cluster of blocks when H is 4, 8, 16 or 32), two of them in one
-    scan window, one a single position above the threshold; a band of rows of 513 ... 3000 positions (a block each)."""
+    """Three rows above 8192 positions (a cluster of blocks each when H is 4, 8 or 32; with 4 and 8 found at multiples of 4096 and 2048 positions,
+    else two of them in one scan window and one a single position above the threshold); a band of rows of 513 ... 3000 positions (a block each, 4 and 8
+    heads in chunks up to 4096 and 2048).  Over its own input the softmax goes by row length with every head count."""
     rng = np.random.default_rng(31 + H)
     n, e = 3000, 120000
     src = rng.integers(0, n, e).astype(np.int32)
@@ -171,6 +172,11 @@ def test_edge_softmax_rows_of_tens_of_thousands_of_positions(gnn, dtype, H):
     again = gnn.edge_softmax(g, to_dev(s[eid]))
     assert np.array_equal(bits(again), bits(alpha))
     assert np.array_equal(bits(gnn.edge_softmax_backward(g, alpha, to_dev(R[eid]))), bits(ds))
+    own, upstream = to_dev(s[eid]), to_dev(R[eid])
+    gnn._check(gnn.load().gnn_edge_softmax(gnn.C.byref(g.c), gnn._p(own), H, gnn._dtype(own), gnn._p(own), None, None, gnn._stream()))
+    assert_close(to_host64(own), ao[eid], ao[eid], dtype, "alpha over the logits")
+    gnn._check(gnn.load().gnn_edge_softmax_backward(gnn.C.byref(g.c), gnn._p(alpha), gnn._p(upstream), H, gnn._dtype(own), gnn._p(upstream), gnn._stream()))
+    assert_close(to_host64(upstream), dso[eid], S[eid], dtype, "dlogits over dalpha")
 
 
 # One row beside short ones: as long as the chunk kernels take, one position more, and over many blocks' chunks.  Up to 8192 edges they take any row.
