@@ -6,8 +6,9 @@
 // chunk, combines a row's shares in ascending order and finishes the chunk's positions of it.  Edge softmax, which has no
 // workspace: the blocks that a row is cut into read all of it, out of L2.
 // Rows of more than AR_SPAN chunks are left to clusters (softmax.cu), which read them once per pass: the blocks together would read a row of k chunks
-// k times (8 heads fp32, a row of 330 k positions among 1.9 M 632 -> 200 us, of 2.4 M 20 -> 1.8 ms).  What bounds it: the latency of a chunk (search, gathers, four barriers) at two or three blocks
-// per SM, and instruction issue (an exponential and a division per value).
+// k times (8 heads fp32, a row of 330 k positions among 1.9 M edges 632 -> 200 us, of 2.4 M among 7.2 M 20 -> 1.8 ms).
+// What bounds it: the latency of a chunk (search, gathers, four to six barriers) at two or three blocks per SM, and instruction issue (an exponential and
+// a division per value).
 // Before: a row per 8 threads, per warp or per block, three kernels side by side on streams of their own, as long as their
 // longest row and mostly idle warps.  100k nodes, 1.6 M edges, R-MAT: softmax of GAT logits of 8 heads 97 -> 43 us (tiers of rows side
 // by side -> both kernels), its gradient 104 -> 100 us; edge softmax 80 -> 41 us and 55 -> 27 us (4 heads fp32), 113 -> 72 us and 83 -> 50 us (8).
@@ -526,7 +527,7 @@ attention_gradient_kernel(const __grid_constant__ AttnArgs A) {
     const int n_chunk = (int)min((int64_t)Tile::CHUNK, A.E - c0), n = min(max(n_chunk - w * Tile::WP, 0), Tile::WP);
     const int64_t cs = c0 + w * Tile::WP;
     // the lane's items: (position, quad) lane + 32 k of the warp's share; all loads of the chunk are on their way before its rows are
-    // looked up, and alpha and dalpha stay in registers (read again for dz, at three blocks per SM: 1.05 times as long)
+    // looked up, and alpha and dalpha stay in registers but for 52 to 60 bytes (read again for dz, at three blocks per SM: 1.05 times as long)
     const float* const alpha = A.alpha + (size_t)cs * H;
     float* const dz = A.dz + (size_t)cs * H;
     unsigned pos = 0;  // four bits per item: z > 0
@@ -846,7 +847,10 @@ edge_softmax_chunk_kernel(const __grid_constant__ SoftmaxArgs A) {
 
 // ------------------------------------------------------------------ launches
 constexpr int AR_SLOT = 20;  // of allow_big_smem: 24 of them
-// Chunks of 256 threads are 1024 (8 heads) or 2048 (4 heads) positions; small graphs take a quarter, so that all SMs have work.
+// Chunks of 256 threads are 1024 (8 heads) or 2048 (4 heads) positions; small graphs take a quarter, so that all SMs have work.  A quarter / whole, us, R-MAT
+// of mean length 12, graphs replayed, edges * heads / 8 of 100, 200, 300, 400 and 600 Ki: edge softmax of 8 heads 14.5 / 15.8, 19.6 / 20.2, 21.6 / 21.8,
+// 26.9 / 22.9, 37.9 / 34.0, of 4 heads 17.3 / 13.8, 20.9 / 19.5, 22.1 / 22.1, 27.5 / 22.4, 39.6 / 32.4; GAT of 8 heads 28.0 / 29.0, 35.8 / 35.9, 42.4 / 41.4,
+// 42.3 / 41.8, 60.2 / 61.6, its gradient within 2 % throughout.
 constexpr int64_t AR_SMALL = 400 * 1024;  // edges * heads / 8
 // Edge softmax: rows of up to so many chunks' positions are read by every block that they reach, longer ones by a cluster (1.6 M edges, R-MAT, 8
 // heads fp32, of 2, 4, 8 and 16 chunks: 80, 78, 75 and 74 us; 300 k edges: 46, 31, 25 and 24 us; 160 k: 24, 24, 20 and 27 us).
@@ -882,8 +886,9 @@ static gnn_status gradient_launch(const char* who, const AttnArgs& A, int chunks
 
 static int ar_chunk(int64_t E, int H) { return (E * H / 8 < AR_SMALL ? 64 : 256) / (H / 4) * AR_RUN; }
 
-// The shares of the cut rows fit any workspace of the chunked reduction of rows of four or more features a head, which is what the
-// attention calls are given: at most 136 bytes per chunk, where that has 132 per 128 positions or more.
+// The shares of the cut rows fit the workspace of the chunked reduction, which the attention calls are given and whose smallest room is a partial row per 1024
+// positions: a head has four features or more, so 4 heads need 72 bytes per 512 or 2048 positions of at least 132 per 1024, 8 heads 136 per 256 or 1024 of at
+// least 260 per 1024.
 // dz and dar null: alpha = softmax over each row of LeakyReLU(al[col] + ar[row]).  Else dz (dalpha on entry) and dar from alpha.
 gnn_status attention_rows(const char* who, const gnn_csr* g, const float* al, const float* ar, float slope, int H, float* alpha, float* dz, float* dar,
                           void* ws, size_t ws_bytes, cudaStream_t st) {

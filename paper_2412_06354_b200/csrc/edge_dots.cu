@@ -33,7 +33,7 @@ enum { EDGE_DOT = 0, EDGE_DOT_MEAN = 1, EDGE_GATV2 = 2 };
 // batch, one batch after the other, 8-byte entries, the row's chunk loaded when it changes) -> now:
 //   100k nodes / 1.6 M edges, 512-byte rows, 8 heads bf16 150 -> 105 us; 123 M edges, 128-byte bf16 rows 2.86 -> 2.4 ms;
 //   bf16 dots by multiply-adds that take bf16 (nothing unpacked, the same bits): 105 -> 96 us and 2.33 -> 2.10 ms there, and with
-//   the registers that frees four blocks per SM for rows up to 256 bytes, 1.96 ms (512 bytes: 96 -> 98 us, three it stays); bf16 logits 81 -> 77 us;
+//   the registers that frees four blocks per SM for rows up to 256 bytes, 1.96 ms with 12 bytes of spills (512 bytes: 96 -> 98 us, three it stays); bf16 logits 81 -> 77 us;
 //   GATv2 logits of 100k nodes / 1.6 M edges, 512-byte fp32 rows (a gather per index load, four at a time) 358 -> 113 us.
 constexpr int ED_SUB = 256;  // most positions per warp
 constexpr int ED_H = 4;      // positions per register buffer

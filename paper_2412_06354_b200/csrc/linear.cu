@@ -340,7 +340,8 @@ gnn_status gnn_linear_backward(const void* X, const void* W, const void* dY, int
             auto run = [&](auto kernel, auto* to, int elements, int threads) {
                 launch_overlapped(kernel, dim3((unsigned)ceil_div(n, (int64_t)elements)), dim3(threads), 0, st, part, slabs, n, to, cols, K, cols_out, M, c0);
             };
-            // (148 partials of 16 Ki elements: 4.9 us one by one, 7.2 us by four, in too few blocks; of 64 Ki: 10.6 and 7.7 us)
+            // (148 partials of 16 Ki elements: 4.9 us one by one, 7.2 us by four, in too few blocks; of 64 Ki: 10.6 and 7.7 us.  With the product before
+            // it, 170k rows bf16, one by one / by four: 16 Ki 22.6 / 24.7, 25 Ki 28.9 / 30.9, 36 Ki 34.5 / 35.1, 42 Ki 37.0 / 37.0, 49 Ki 39.3 / 38.9, 64 Ki 46.5 / 45.1)
             const bool four = n >= 48 * 1024 && n % 4 == 0 && aligned16(part);
             if (dtype == GNN_F32) four ? run(slab_sum_kernel<float, 4>, (float*)dW, 64, 128) : run(slab_sum_kernel<float, 1>, (float*)dW, 32, 256);
             else four ? run(slab_sum_kernel<__nv_bfloat16, 4>, (__nv_bfloat16*)dW, 64, 128) : run(slab_sum_kernel<__nv_bfloat16, 1>, (__nv_bfloat16*)dW, 32, 256);
